@@ -107,11 +107,11 @@ CVLC_HD inline uint64_t row_tiles_total(const Partition& P) { return P.total / k
 CVLC_HD inline uint64_t seg_first_tile(uint64_t p0, uint32_t seg) { return p0 / kTileUnits + seg; }
 
 // plan workspace:
-//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2] | uint32 leader[n]
+//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2]
 //   | uint32 seg_count[S] | uint64 seg_prefix[S] | uint32 seg_rows[S] | uint32 row_max[64 * tiles]
 //   | uint32 row_list[64 * tiles] | uint32 seg_hist[S][4096]          (S = max_segments, tiles = row_tiles_total)
 // tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths;
-// leader[c] = the first client of the batch with c's key (it runs the length tuning, the others copy its result).
+// the first of them runs the length tuning and writes the result to all.
 struct PlanWsHeader {
   int32_t status;   // byte 0
   uint32_t n;       // clients of the batch the workspace was filled for
@@ -123,8 +123,7 @@ constexpr uint32_t kPlanWsMagic = 0x53454743u;
 constexpr size_t kPlanWsHist = 256;
 CVLC_HD constexpr size_t plan_off_flags(uint32_t n) { return kPlanWsHist + (size_t)n * CVLC_HIST_BINS * 8; }
 CVLC_HD constexpr size_t plan_off_keys(uint32_t n) { return align256(plan_off_flags(n) + (size_t)n * 4); }
-CVLC_HD constexpr size_t plan_off_leader(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
-CVLC_HD constexpr size_t plan_off_seg_count(uint32_t n) { return align256(plan_off_leader(n) + (size_t)n * 4); }
+CVLC_HD constexpr size_t plan_off_seg_count(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
 CVLC_HD constexpr size_t plan_off_seg_prefix(uint32_t n, uint32_t S) { return align256(plan_off_seg_count(n) + (size_t)S * 4); }
 CVLC_HD constexpr size_t plan_off_seg_rows(uint32_t n, uint32_t S) { return align256(plan_off_seg_prefix(n, S) + (size_t)S * 8); }
 CVLC_HD constexpr size_t plan_off_row_max(uint32_t n, uint32_t S) { return align256(plan_off_seg_rows(n, S) + (size_t)S * 4); }
@@ -207,7 +206,7 @@ CVLC_HD constexpr size_t dec_ws_bytes(uint32_t n) { return align256(dec_off_meta
 // ---- launch accounting and optional per-kernel timing ------------------------------
 
 enum KernelId {
-  kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKPlanFinish, kKEncodeInit, kKSelect, kKSelectLookback, kKSortHist, kKSortScan,
+  kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKSortHist, kKSortScan,
   kKSortPass, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
   kKPlanLiteral, kKEcAccumulate, kKPackUnframed, kKDecodeUnframed, kNumKernelIds
 };

@@ -197,15 +197,14 @@ __device__ __forceinline__ double energy_E(uint64_t Z, double beta, double D) {
 }
 
 // ===================================================================================
-// K2  planner: per client a fit kernel (one CTA of 1024 threads), a tuning kernel and a small copy kernel
+// K2  planner: per client a fit kernel (one CTA of 1024 threads) and a tuning kernel
 // ===================================================================================
 
 constexpr int kPlanThreads = 1024;  // the fit kernel: one thread per four histogram bins
-// The tuning kernel evaluates up to kPlanItems (evaluation, length) items per round with kTuneThreads threads (an item
-// is a chain of about 175 dependent FP64 operations) and leaves most of its SM to the kernels that run next to it:
-// measured on the 100-client benchmark, 256 threads take 0.84 ms instead of 0.62 ms with 512 or 1024, all of it hidden
-// behind selection and ranking, and slow those down the least.
-constexpr int kTuneThreads = 256;
+// The tuning kernel decides most atomic operations with one warp per operation or per trial split (see tune_fast below):
+// 16 warps are as many operations as a sweep over neighbouring lengths usually has, and a 17-way search.
+constexpr int kTuneThreads = 512;
+constexpr int kTuneWarps = kTuneThreads / 32;
 constexpr int kPlanItems = 1024;
 constexpr int kPairSlots = (496 + kTuneThreads - 1) / kTuneThreads;  // pairs of a sweep a thread looks at
 constexpr unsigned kFull = 0xFFFFFFFFu;
@@ -559,6 +558,98 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
   }
 }
 
+
+// ---- atomic operations decided without the series arithmetic -----------------------------------
+// An atomic operation on the lengths i > j looks for the first split t with F(t + 1) <= F(t), F evaluated in the
+// series arithmetic.  Over the reals F(t) = sum_l h_l E(W_l(t)) with h_l = g_l - g_(l-1) >= 0 over the candidate
+// lengths (Eq. (5) summed by parts: a length without packets adds nothing), W_l linear in t and E concave, so the
+// differences F(t + 1) - F(t) fall with t.  A difference whose size exceeds `guard` has the same sign in the series
+// arithmetic, and by concavity so has every difference on the far side of it: two differences around the answer, each
+// beyond the guard, settle the whole bisection, and with it the comparison of the new split with the current one.
+// The guard covers the rounding of both sides.  E(W) = (p - 1) / D with p = (W + 1)^beta <= max(1, D + 1): a power is
+// within about 5e-15 of its value in either arithmetic (log2 of up to 31 rounded to 1.8e-15 twice, the polynomial's
+// roundings), the weights h_l add up to at most 1, the ordered sum of 32 terms adds 4e-15, twice: below
+// 3e-14 (1 + 1 / |D|); the guard is 7 times that.  Differences around an optimum are 1e-11 and more for the usual
+// budgets; an operation that meets a smaller one is left to the series arithmetic (steep power laws: most are).
+// Measured on one ResNet-18-sized client (15 moves, 22 + 13 rounds of checks, 27 of trial splits): the
+// kernel takes 53 us, 632 us with every difference in the series arithmetic; 11 instead of 45 us on a client of 100,000
+// coordinates.  What is left is instruction latency: about 60 steps of some 200 instructions and a barrier each.
+constexpr double kTuneGuard = 0x1p-42;
+// Nearly every sign already shows in fp32, where the terms of a difference are worked out as
+// h / D a^beta ((1 + x)^beta - 1), x = step / a, without cancellation inside a term.  A term is good to 3e-6 of itself
+// (for |beta| <= 1; the argument of a^beta is split so that its rounding stays below 1e-7, see fast_power; the growth
+// factor where its logarithm leaves the series: 2.5e-6), the sum to 5e-7 of its largest term: a sum beyond
+// kTuneRel (1 + |beta|) of the terms' sizes has a certain sign, and the rest is looked at in fp64.
+constexpr float kTuneRel = 0x1p-17f;
+
+struct FastShared {  // one code and one pair per warp, in two buffers: a single barrier per step
+  int code[2][kTuneWarps];
+  int pair[2][kTuneWarps];
+};
+// every warp keeps a copy of the current counts, one candidate length per lane
+struct FastLane {
+  double h;         // weight of E(W) in F (0 beyond the last length)
+  float hD, u;      // h / D, h / D a^beta
+  uint32_t a;       // W + 1, W = ranks covered down to this lane's length
+  uint32_t n, cap;  // packets and records per packet of this lane's length
+};
+struct FastConst {
+  double beta, inv_D, guard;
+  float fbeta, frel, fguard;
+};
+
+__device__ __forceinline__ float fast_lg2(float v) {
+  float r;
+  asm("lg2.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float fast_ex2(float v) {
+  float r;
+  asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+// a^beta, beta a multiple of 1/128 below 8 in size: beta times the exponent of a is exact, its whole part goes to the
+// result's exponent, and only a number below 5 is rounded before the exponential
+__device__ __forceinline__ float fast_power(uint32_t a, float beta) {
+  const float af = (float)a;
+  const uint32_t bits = __float_as_uint(af) - 0x3F3504F3u;        // mantissa into [sqrt(1/2), sqrt(2))
+  const float e = (float)((int)bits >> 23);
+  const float m = __uint_as_float((bits & 0x007FFFFFu) + 0x3F3504F3u);
+  const float be = beta * e, whole = rintf(be);
+  const float r = fast_ex2((be - whole) + beta * fast_lg2(m));
+  const float w = fmaxf(whole, -100.0f);                           // below 2^-100: nothing next to the guard
+  return r * __uint_as_float((uint32_t)((int)w + 127) << 23);
+}
+// (b1 / b0)^beta - 1, step = b1 - b0
+__device__ __forceinline__ float fast_growth(uint32_t from, uint32_t to, int step, float beta) {
+  const float b0 = (float)from, b1 = (float)to;
+  const float s = __fdividef((float)step, b0 + b1), q = s * s;     // ln(b1 / b0) = 2 atanh(s)
+  const float series = 2.0f * s * fmaf(q, fmaf(q, fmaf(q, 1.0f / 7, 1.0f / 5), 1.0f / 3), 1.0f);
+  const float ln = fabsf(s) <= 0.1f ? series : 0.693147181f * fast_lg2(__fdividef(b1, b0));
+  const float z = beta * ln;
+  const float e = z * fmaf(z, fmaf(z, fmaf(z, fmaf(z, fmaf(z, 1.0f / 720, 1.0f / 120), 1.0f / 24), 1.0f / 6), 0.5f), 1.0f);
+  return fabsf(z) < 0.25f ? e : fast_ex2(1.44269504f * z) - 1.0f;
+}
+// the terms' sum and the sum of their sizes, to 2^-21 of the largest term (fixed point relative to it)
+__device__ __forceinline__ void fast_sum(float term, float& sum, float& size) {
+  const uint32_t top = __reduce_max_sync(kFull, __float_as_uint(term) & 0x7F800000u);  // exponent field of the largest term
+  const uint32_t e = top >> 23;
+  const bool in_range = e > 32u && e < 220u;
+  const float up = in_range ? __uint_as_float((127u + 25u + 127u - e) << 23) : 0.0f;   // 2^(25 - exponent)
+  const float down = in_range ? __uint_as_float((e - 25u) << 23) : 0.0f;
+  const int v = __float2int_rn(term * up);                                             // below 2^26: no sum leaves 32 bits
+  sum = (float)__reduce_add_sync(kFull, v) * down;
+  size = (float)__reduce_add_sync(kFull, (uint32_t)(v < 0 ? -v : v)) * down;
+}
+
+// sign of F(t + 1) - F(t) from fp64 powers; 0: too close to tell
+__device__ __noinline__ int fast_sign64(double h, double at, double step, double beta, double inv_D, double guard) {
+  double diff = h * (exp2(beta * log2(at + step)) - exp2(beta * log2(at)));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) diff += __shfl_xor_sync(kFull, diff, off);
+  diff *= inv_D;
+  return diff > guard ? 1 : (diff < -guard ? -1 : 0);
+}
 // K2b  code-length tuning, one CTA per client; only the first client of every tuning key does the work
 template <int CAP>
 __global__ void __launch_bounds__(kTuneThreads, 1)
@@ -566,41 +657,33 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
   extern __shared__ unsigned char smem_raw[];
   __shared__ PlanShared S;
   __shared__ PlanTab T;
+  __shared__ FastShared FS;
   __shared__ uint32_t s_leader;
+  __shared__ uint32_t s_ny[CVLC_MAX_CODE_BITS + 1];
+  __shared__ double s_single[CVLC_MAX_CODE_BITS];
   const uint32_t c = blockIdx.x;
-  cvlc_plan_t* __restrict__ plan = batch.c[c].plan;
-  uint32_t* leader = reinterpret_cast<uint32_t*>(ws + plan_off_leader(batch.n));
   const unsigned long long* keys = reinterpret_cast<const unsigned long long*>(ws + plan_off_keys(batch.n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   const unsigned long long key0 = keys[2 * (size_t)c], key1 = keys[2 * (size_t)c + 1];
+  if (key1 == 0ull) return;  // no key: the fit refused this client's histogram
   if (tid == 0) s_leader = c;
   __syncthreads();
-  if (key1 == 0ull) {  // no key: the fit refused this client's histogram
-    if (tid == 0) leader[c] = 0xFFFFFFFFu;
-    return;
-  }
   for (uint32_t i = tid; i < c; i += kTuneThreads)
     if (keys[2 * (size_t)i] == key0 && keys[2 * (size_t)i + 1] == key1) atomicMin(&s_leader, i);
   __syncthreads();
-  if (tid == 0) leader[c] = s_leader;
-  if (s_leader != c) return;  // an earlier client of the batch tunes for this key; k_plan_finish copies its result
+  if (s_leader != c) return;  // an earlier client of the batch tunes for this key and writes the result to all that share it
 
+  // side by side: the table of lengths, the powers of the single-length plans (lane = length - 1), the power of d
+  const double beta = __dadd_rn(__dmul_rn(2.0, __longlong_as_double((long long)key0)), 1.0);
   if (warp == 0) build_plan_tab(T, shape, batch.c[c].scale_B, lane);
-  if (tid == 0) {
-    const double aq = __longlong_as_double((long long)key0);
-    const double beta = __dadd_rn(__dmul_rn(2.0, aq), 1.0);
-    S.alpha_q = aq;
-    S.beta = beta;
-    S.D = __dsub_rn(series_powr((double)shape.d, beta), 1.0);
-  }
-  if (tid < 32) S.n[tid] = 0;
+  if (warp == 1) s_single[lane] = series_powr((double)((uint64_t)shape.R * shape.cap[lane + 1] + 1), beta);
+  if (tid == 64) S.D = __dsub_rn(series_powr((double)shape.d, beta), 1.0);
+  if (warp == 3) S.n[lane] = 0;
   __syncthreads();
-  const double beta = S.beta, D = S.D;
+  const double D = S.D;
   const int nY = (int)T.nY;
   const uint32_t my_cap = (lane < nY) ? T.capY[lane] : 0u;
-  double* ptX = reinterpret_cast<double*>(smem_raw);  // the solver's scratch
-
 
   // ---- objective bookkeeping -----------------------------------------------------------
   // F(n) = 1 - gamma of Eq. (5) is a running sum over the used lengths, longest first:
@@ -611,7 +694,7 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
   // above i untouched, so a trial split only needs E for the used lengths at or below i and
   // continues the running sum from Q.Fpre[i + 1]: the same operations in the same order as a
   // full evaluation, on a fraction of the lanes.
-  PlanSolver& Q = *reinterpret_cast<PlanSolver*>(ptX);  // the fit points are no longer needed
+  PlanSolver& Q = *reinterpret_cast<PlanSolver*>(smem_raw);
 
   auto refresh_state = [&]() {  // all threads; ends with a barrier
     if (warp == 0) {
@@ -622,24 +705,28 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
         const uint64_t o = __shfl_down_sync(kFull, W, off);
         if (lane + off < 32) W += o;
       }
-      Q.Ecur[lane] = (my_n > 0) ? energy_E(W, beta, D) : 0.0;
-      Q.Wc[lane] = W;
+      const double E = (my_n > 0) ? energy_E(W, beta, D) : 0.0;
       const unsigned used = __ballot_sync(kFull, my_n > 0);
-      if (lane == 0) Q.used = used;
-      __syncwarp();
+      // the terms side by side, their sum in the order of the lengths
+      const unsigned above = lane < 31 ? used & (kFull << (lane + 1)) : 0u;
+      const double Eup = __shfl_sync(kFull, E, above ? __ffs(above) - 1 : 0);
+      const double Eprev = above ? Eup : 0.0;
+      const double term = (my_n > 0) ? __dmul_rn(T.gY[lane], __dsub_rn(E, Eprev)) : 0.0;
+      double F = 0.0, Fmine = 0.0;
+      for (unsigned rest = used; rest;) {
+        const int l = 31 - __clz(rest);
+        rest ^= 1u << l;
+        F = __dadd_rn(F, __shfl_sync(kFull, term, l));
+        if (lane <= l) Fmine = F;
+      }
+      Q.Ecur[lane] = E;
+      Q.Wc[lane] = W;
+      Q.Fpre[lane] = Fmine;
+      Q.Eab[lane] = (my_n > 0) ? E : Eprev;
       if (lane == 0) {
-        double F = 0.0, Eprev = 0.0;
+        Q.used = used;
         Q.Fpre[32] = 0.0;
         Q.Eab[32] = 0.0;
-        for (int l = 31; l >= 0; --l) {
-          if (l < nY && S.n[l] > 0) {
-            const double Ec = Q.Ecur[l];
-            F = __dadd_rn(F, __dmul_rn(T.gY[l], __dsub_rn(Ec, Eprev)));
-            Eprev = Ec;
-          }
-          Q.Fpre[l] = F;
-          Q.Eab[l] = Eprev;
-        }
       }
     }
     __syncthreads();
@@ -653,8 +740,8 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
     // ---- equal packets: best admissible single-length plan, ties to the longer code ----
     if (tid < nY) {
       const uint64_t W = (uint64_t)T.R * T.capY[tid];
-      // one term: F = 0 + g * (E - 0)
-      S.Fv[tid] = (W > T.d) ? -CUDART_INF : __dmul_rn(T.gY[tid], energy_E(W, beta, D));
+      // one term: F = 0 + g * (E - 0), E = (power - 1) / D
+      S.Fv[tid] = (W > T.d) ? -CUDART_INF : __dmul_rn(T.gY[tid], __ddiv_rn(__dsub_rn(s_single[T.Y[tid] - 1], 1.0), D));
     }
     __syncthreads();
     if (tid == 0) {
@@ -671,7 +758,6 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
       S.n[best < 0 ? 0 : best] = T.R;  // the host has checked that a plan is admissible
     }
     __syncthreads();
-    refresh_state();
 
     // ---- atomic operations (Section IV-C) on pairs of lengths until nothing moves ----
     // An atomic operation bisects the split of X = n_i + n_j packets between the lengths i > j
@@ -694,6 +780,167 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
         j = i - 1;
       }
     };
+    // ---- the operations that the concavity of F settles (see FastLane above) -----------------
+    const bool fast = (uint64_t)T.R * T.capY[0] <= T.d;  // no trial can send more than d coordinates (F = -infinity)
+    FastConst fc;
+    fc.beta = beta;
+    fc.inv_D = 1.0 / D;
+    fc.guard = kTuneGuard * (1.0 + fabs(fc.inv_D));
+    fc.fbeta = (float)beta;
+    fc.frel = kTuneRel * (1.0f + fabsf(fc.fbeta));
+    fc.fguard = (float)fc.guard * 1.0001f;
+    FastLane fl;
+    fl.cap = my_cap;
+    fl.h = (lane < nY) ? T.gY[lane] - (lane ? T.gY[lane - 1] : 0.0) : 0.0;
+    fl.hD = (float)(fl.h * fc.inv_D);
+    bool stale = true;  // the bookkeeping of the series arithmetic is behind the counts
+    int buf = 0;
+    auto load_counts = [&]() {  // the counts of S.n into every warp's copy
+      fl.n = S.n[lane];
+      uint32_t W = fl.n * my_cap;  // at most d in all
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_down_sync(kFull, W, off);
+        if (lane + off < 32) W += o;
+      }
+      fl.a = W + 1u;
+      fl.u = fl.hD * fast_power(fl.a, fc.fbeta);
+    };
+    // ranks that this lane's cover W gains for every packet moved from length j to length i > j
+    auto cover_step = [&](int i, int j) -> int {
+      const int ci = (int)__shfl_sync(kFull, fl.cap, i), cj = (int)__shfl_sync(kFull, fl.cap, j);
+      return lane > i ? 0 : (lane > j ? ci : ci - cj);
+    };
+    // One step of every warp's search: all warps learn all codes.  Returns this lane's (lane < kTuneWarps) code.
+    auto exchange = [&](int code, int pair) -> int {
+      if (lane == 0) {
+        FS.code[buf][warp] = code;
+        FS.pair[buf][warp] = pair;
+      }
+      __syncthreads();
+      const int got = lane < kTuneWarps ? FS.code[buf][lane] : 0;
+      buf ^= 1;
+      return got;
+    };
+    // Walks the sweep from the cursor (ci, cj) on; ends with ci = 0 behind its last operation, or with the cursor on an
+    // operation that only the series arithmetic can decide.
+    auto fast_sweep = [&](int phase, int& ci, int& cj, int& moved) {
+      while (ci >= 1) {
+        // operations left in every row i = lane: pairs (i, j) that share packets, rows and columns descending
+        const unsigned used = __ballot_sync(kFull, fl.n > 0);
+        const int jmax = (lane == ci) ? cj : lane - 1;
+        const unsigned below = (jmax >= 0) ? used & (kFull >> (31 - jmax)) : 0u;
+        int cnt = 0;
+        if (lane <= ci && jmax >= 0) {
+          if (phase == 0) cnt = (fl.n > 0 || ((used >> jmax) & 1u)) ? 1 : 0;
+          else cnt = (fl.n > 0) ? jmax + 1 : __popc(below);
+        }
+        int first = 0;  // operations in the rows above
+        if (phase == 0) {
+          first = __popc(__ballot_sync(kFull, cnt != 0) & ~(kFull >> (31 - lane)));
+        } else {
+          first = cnt;
+#pragma unroll
+          for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_down_sync(kFull, first, off);
+            if (lane + off < 32) first += o;
+          }
+          first -= cnt;
+        }
+        const int total = __shfl_sync(kFull, first + cnt, 0);
+        int code = 0, i = 0, j = 0;
+        for (int base = 0; base < total && code == 0; base += kTuneWarps) {
+          // ---- one operation per warp: does the current split stay?
+          const int q = base + warp;
+          int mine = 0;
+          if (q < total) {
+            i = __ffs(__ballot_sync(kFull, q >= first && q < first + cnt)) - 1;
+            const int o = q - __shfl_sync(kFull, first, i);
+            const int top = __shfl_sync(kFull, jmax, i);
+            const uint32_t ni = __shfl_sync(kFull, fl.n, i);
+            if (phase == 0 || ni > 0) {
+              j = top - o;
+            } else {  // the o-th used length below, from the longest on
+              const unsigned m = __shfl_sync(kFull, below, i);
+              j = __ffs(__ballot_sync(kFull, ((m >> lane) & 1u) && __popc(m & ~(kFull >> (31 - lane))) == o)) - 1;
+            }
+            const uint32_t nj = __shfl_sync(kFull, fl.n, j);
+            const int step = cover_step(i, j);
+            // forward from the current split, and forward to it from one packet less (a side without packets: no trial)
+            const uint32_t ahead = nj > 0 ? fl.a + (uint32_t)step : fl.a, back = ni > 0 ? fl.a - (uint32_t)step : fl.a;
+            float u, d, u_size, d_size;
+            fast_sum(fl.u * fast_growth(fl.a, ahead, nj > 0 ? step : 0, fc.fbeta), u, u_size);
+            fast_sum(-fl.u * fast_growth(fl.a, back, ni > 0 ? -step : 0, fc.fbeta), d, d_size);
+            int su = fabsf(u) > fc.frel * u_size + fc.fguard ? (u > 0.0f ? 1 : -1) : 0;
+            int sd = fabsf(d) > fc.frel * d_size + fc.fguard ? (d > 0.0f ? 1 : -1) : 0;
+            if (nj == 0) su = -1;
+            if (ni == 0) sd = 1;
+            if (su == 0) su = fast_sign64(fl.h, (double)fl.a, (double)step, fc.beta, fc.inv_D, fc.guard);
+            if (sd == 0) sd = fast_sign64(fl.h, (double)back, (double)step, fc.beta, fc.inv_D, fc.guard);
+            mine = (su < 0 && sd > 0) ? 0 : (su > 0) ? 1 : (sd < 0) ? 2 : 3;
+          }
+          const int parity = buf;
+          const int got = exchange(mine, (i << 8) | j);
+          const unsigned hit = __ballot_sync(kFull, got != 0);
+          if (hit) {  // the first operation of the sweep that moves, or may
+            const int w = __ffs(hit) - 1;
+            code = __shfl_sync(kFull, got, w);
+            i = FS.pair[parity][w] >> 8;
+            j = FS.pair[parity][w] & 0xFF;
+          }
+        }
+        if (code == 0) {
+          ci = 0;
+          return;
+        }
+        ci = i;
+        cj = j;
+        if (code == 3) return;
+        // ---- where to: one trial split per warp, first at distances 1, 2, 4, ..., then evenly spread over the bracket
+        const uint32_t ni = __shfl_sync(kFull, fl.n, i), nj = __shfl_sync(kFull, fl.n, j);
+        const int step = cover_step(i, j);
+        uint32_t lo = (code == 1) ? ni + 1 : 0u, hi = (code == 1) ? ni + nj : ni - 1;  // the answer lies in [lo, hi]
+        bool spread = false;
+        while (lo < hi) {
+          const uint32_t span = hi - lo;
+          uint32_t t = hi;  // hi: no trial
+          if (!spread && span > (uint32_t)kTuneWarps) {
+            const uint32_t away = 1u << warp;
+            if (away <= span) t = (code == 1) ? lo + away - 1 : hi - away;
+          } else if (span <= (uint32_t)kTuneWarps) {
+            if ((uint32_t)warp < span) t = lo + warp;
+          } else {
+            t = lo + (uint32_t)(((uint64_t)span * (warp + 1)) / (kTuneWarps + 1));
+          }
+          int mine = -1;
+          if (t < hi) {
+            const uint32_t at = fl.a + (t - ni) * (uint32_t)step;
+            float sum, size;
+            fast_sum(fl.hD * fast_power(at, fc.fbeta) * fast_growth(at, at + (uint32_t)step, step, fc.fbeta), sum, size);
+            mine = fabsf(sum) > fc.frel * size + fc.fguard ? (sum > 0.0f ? 1 : -1) : 0;
+            if (mine == 0) mine = fast_sign64(fl.h, (double)at, (double)step, fc.beta, fc.inv_D, fc.guard);
+          }
+          const int parity = buf;
+          const int got = exchange(mine, (int)t);
+          const int got_t = lane < kTuneWarps ? FS.pair[parity][lane] : (int)hi;
+          if (__any_sync(kFull, lane < kTuneWarps && got == 0)) return;  // too close to tell
+          // F still rises at the trials below the answer and no longer at those from it on
+          const uint32_t rises = __reduce_max_sync(kFull, (lane < kTuneWarps && got > 0) ? (uint32_t)got_t + 1 : lo);
+          const uint32_t falls = __reduce_min_sync(kFull, (lane < kTuneWarps && got < 0) ? (uint32_t)got_t : hi);
+          lo = rises;
+          hi = falls < hi ? falls : hi;
+          spread = true;
+        }
+        if (lane == i) fl.n = lo;
+        if (lane == j) fl.n = ni + nj - lo;
+        fl.a += (lo - ni) * (uint32_t)step;
+        fl.u = fl.hD * fast_power(fl.a, fc.fbeta);
+        stale = true;
+        moved = 1;
+        next_pair(phase, ci, cj);
+      }
+    };
+    if (fast) load_counts();
     for (int round = 0; round < 64; ++round) {
       int movedB = 0;
       for (int phase = 0; phase < 2; ++phase) {  // 0: neighbouring lengths until quiet; 1: every pair once
@@ -702,6 +949,16 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
           int moved = 0;
           int ci = nY - 1, cj = nY - 2;  // cursor of the sweep
           while (ci >= 1) {
+            if (fast) {
+              fast_sweep(phase, ci, cj, moved);
+              if (ci < 1) break;
+              if (stale && warp == 0) S.n[lane] = fl.n;
+            }
+            if (stale) {
+              __syncthreads();
+              refresh_state();
+              stale = false;
+            }
             // ---- collect a batch: thread t looks at the t-th pair of the sweep from the cursor on (at most
             // 31 + 465 pairs).  The batch is the first pairs, in sweep order, that share packets (X > 0), up to
             // kMaxBatchOps of them and as long as two evaluations of each fit the block: a prefix of the flagged
@@ -1003,6 +1260,7 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
             if (Q.moved) {
               moved = 1;
               refresh_state();
+              if (fast) load_counts();
             } else {
               __syncthreads();
             }
@@ -1013,40 +1271,36 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
       }
       if (!movedB) break;
     }
-  }
-
-  // ---- outputs ---------------------------------------------------------------------
-  if (tid == 0) {
-    unsigned long long k = 0;
-    double Qmax = 0.0;
-    for (int i = 0; i < nY; ++i) {
-      k += (unsigned long long)S.n[i] * T.capY[i];
-      if (S.n[i] > 0 && T.QY[i] > Qmax) Qmax = T.QY[i];
+    if (stale) {
+      if (fast && warp == 0) S.n[lane] = fl.n;
+      __syncthreads();
+      refresh_state();
     }
-    plan->k = k;
-    plan->gamma = __dsub_rn(1.0, Q.Fpre[0]);
-    plan->B_next = __dadd_rn(1.0, Qmax);
-    for (int i = 0; i < nY; ++i) plan->n_y[T.Y[i]] = S.n[i];
   }
-}
 
-// K2c  the clients that share a tuning key take the lengths of the client that tuned for it
-template <int CAP>
-__global__ void __launch_bounds__(256)
-k_plan_finish(const __grid_constant__ BatchDesc<CAP> batch, const unsigned char* ws) {
-  const uint32_t c = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (c >= batch.n) return;
-  const uint32_t l = reinterpret_cast<const uint32_t*>(ws + plan_off_leader(batch.n))[c];
-  if (l == 0xFFFFFFFFu || l == c || l >= batch.n) return;
-  cvlc_plan_t* dst = batch.c[c].plan;
-  const cvlc_plan_t* src = batch.c[l].plan;
-  dst->n_y[lane] = src->n_y[lane];
-  if (lane == 0) {
-    dst->n_y[CVLC_MAX_CODE_BITS] = src->n_y[CVLC_MAX_CODE_BITS];
-    dst->k = src->k;
-    dst->gamma = src->gamma;
-    dst->B_next = src->B_next;
+  // ---- outputs, to this client and to the later ones that share its tuning key -------------------
+  if (tid <= CVLC_MAX_CODE_BITS) s_ny[tid] = 0;
+  __syncthreads();
+  if (tid < nY) s_ny[T.Y[tid]] = S.n[tid];
+  unsigned long long k = (lane < nY) ? (unsigned long long)S.n[lane] * my_cap : 0ull;
+  double Qmax = (lane < nY && S.n[lane] > 0) ? T.QY[lane] : 0.0;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    k += __shfl_xor_sync(kFull, k, off);
+    const double o = __shfl_xor_sync(kFull, Qmax, off);
+    if (o > Qmax) Qmax = o;
+  }
+  __syncthreads();
+  for (uint32_t i = c + warp; i < batch.n; i += kTuneWarps) {
+    if (keys[2 * (size_t)i] != key0 || keys[2 * (size_t)i + 1] != key1) continue;
+    cvlc_plan_t* __restrict__ dst = batch.c[i].plan;
+    dst->n_y[lane] = s_ny[lane];
+    if (lane == 0) {
+      dst->n_y[CVLC_MAX_CODE_BITS] = s_ny[CVLC_MAX_CODE_BITS];
+      dst->k = k;
+      dst->gamma = __dsub_rn(1.0, Q.Fpre[0]);
+      dst->B_next = __dadd_rn(1.0, Qmax);
+    }
   }
 }
 
@@ -1133,10 +1387,6 @@ static cudaError_t launch_plan_back_t(const ClientDesc* clients, uint32_t n, con
     LaunchScope ls(kKPlanTune, st);
     k_plan_tune<CAP><<<n, kTuneThreads, kTuneSmem, st>>>(batch, shape, w);
   }
-  {
-    LaunchScope ls(kKPlanFinish, st);
-    k_plan_finish<CAP><<<(n + 7) / 8, 256, 0, st>>>(batch, w);
-  }
   return cudaGetLastError();
 }
 
@@ -1199,7 +1449,7 @@ static cudaError_t launch_plan_from_hist_t(const ClientDesc* clients, uint32_t n
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   const Partition part = make_partition(shape.d, n);
   {
-    // status word, header, tuning keys and leaders start at zero: the header stays unmarked, so an encode call
+    // status word, header and tuning keys start at zero: the header stays unmarked, so an encode call
     // cannot take this workspace for one that holds segment tables
     LaunchScope ls(kKZeroWords, st);
     k_zero_words<<<1, 64, 0, st>>>(reinterpret_cast<uint32_t*>(w), kPlanWsHist / 4);
