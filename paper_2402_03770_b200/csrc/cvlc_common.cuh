@@ -94,10 +94,9 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
 }
 
 // Rows: the float4 units of a segment are also grouped into rows of 16 units (64 coordinates, half of a warp-wide
-// load).  The histogram kernel leaves the largest magnitude key of every row; once the selection threshold is known
-// the planner lists, per segment and in ascending order, the rows that hold a candidate (a key at or above the
-// threshold).  The selection kernel works through that list 128 rows (one tile of its staging buffers) at a time:
-// rows without candidates are neither read nor looked at.  Both tables are indexed by row; row r of the segment that
+// load).  The histogram kernel leaves the largest magnitude key of every row; the selection kernel lists, per segment and
+// in ascending order, the rows that hold a candidate (a key at or above the threshold) and works through that list 128
+// rows (one tile of its staging buffers) at a time: rows without candidates are not read.  Both tables are indexed by row; row r of the segment that
 // starts at position p0 of the concatenated array sits at 128 * (p0 / 2048 + segment id) + r, so that the index
 // ranges of different segments do not overlap.
 constexpr int kRowUnits = 16;
@@ -108,8 +107,8 @@ CVLC_HD inline uint64_t seg_first_tile(uint64_t p0, uint32_t seg) { return p0 / 
 
 // plan workspace:
 //   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2]
-//   | uint32 seg_count[S] | uint64 seg_prefix[S] | uint32 seg_rows[S] | uint32 row_max[64 * tiles]
-//   | uint32 row_list[64 * tiles] | uint32 seg_hist[S][4096]          (S = max_segments, tiles = row_tiles_total)
+//   | uint32 seg_count[S] | uint64 seg_prefix[S] | uint32 row_max[128 * tiles] | uint32 seg_hist[S][4096]
+//   (S = max_segments, tiles = row_tiles_total)
 // tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths;
 // the first of them runs the length tuning and writes the result to all.
 struct PlanWsHeader {
@@ -125,13 +124,9 @@ CVLC_HD constexpr size_t plan_off_flags(uint32_t n) { return kPlanWsHist + (size
 CVLC_HD constexpr size_t plan_off_keys(uint32_t n) { return align256(plan_off_flags(n) + (size_t)n * 4); }
 CVLC_HD constexpr size_t plan_off_seg_count(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
 CVLC_HD constexpr size_t plan_off_seg_prefix(uint32_t n, uint32_t S) { return align256(plan_off_seg_count(n) + (size_t)S * 4); }
-CVLC_HD constexpr size_t plan_off_seg_rows(uint32_t n, uint32_t S) { return align256(plan_off_seg_prefix(n, S) + (size_t)S * 8); }
-CVLC_HD constexpr size_t plan_off_row_max(uint32_t n, uint32_t S) { return align256(plan_off_seg_rows(n, S) + (size_t)S * 4); }
-CVLC_HD constexpr size_t plan_off_row_list(uint32_t n, uint32_t S, uint64_t tiles) {
-  return align256(plan_off_row_max(n, S) + (size_t)tiles * kTileRows * 4);
-}
+CVLC_HD constexpr size_t plan_off_row_max(uint32_t n, uint32_t S) { return align256(plan_off_seg_prefix(n, S) + (size_t)S * 8); }
 CVLC_HD constexpr size_t plan_off_seg_hist(uint32_t n, uint32_t S, uint64_t tiles) {
-  return align256(plan_off_row_list(n, S, tiles) + (size_t)tiles * kTileRows * 4);
+  return align256(plan_off_row_max(n, S) + (size_t)tiles * kTileRows * 4);
 }
 CVLC_HD constexpr size_t plan_ws_bytes(uint32_t n, uint32_t S, uint64_t tiles) {
   return align256(plan_off_seg_hist(n, S, tiles) + (size_t)S * CVLC_HIST_BINS * 4);
@@ -170,6 +165,7 @@ struct EncLayout {
   size_t off_ghist;              // uint64[n][4][512] digit histograms
   size_t off_gbase;              // uint64[n][4][512] their exclusive scans
   size_t off_select_state;       // uint64[n][select_tiles]
+  size_t off_row_list;           // uint32[128 * row_tiles_total]: rows that hold candidates
   size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]
   size_t off_buf_a, off_buf_b;   // uint64[n][capacity]
   size_t total;
@@ -187,7 +183,8 @@ static inline EncLayout enc_layout(uint64_t d, uint32_t n, uint64_t capacity) {
   L.off_ghist = align256(L.off_pass_mask + (size_t)n * 4);
   L.off_gbase = align256(L.off_ghist + (size_t)n * kSortPasses * kDigits * 8);
   L.off_select_state = align256(L.off_gbase + (size_t)n * kSortPasses * kDigits * 8);
-  L.off_sort_state = align256(L.off_select_state + (size_t)n * L.select_tiles * 8);
+  L.off_row_list = align256(L.off_select_state + (size_t)n * L.select_tiles * 8);
+  L.off_sort_state = align256(L.off_row_list + (size_t)row_tiles_total(make_partition(d, n)) * kTileRows * 4);
   L.off_buf_a = align256(L.off_sort_state + (size_t)kSortPasses * n * L.sort_tiles_max * kDigits * 8);
   L.off_buf_b = align256(L.off_buf_a + (size_t)n * capacity * 8);
   L.total = align256(L.off_buf_b + (size_t)n * capacity * 8);

@@ -64,7 +64,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     unsigned long long* a = reinterpret_cast<unsigned long long*>(ws + L.off_n_selected);
     for (size_t i = gtid; i < n; i += gstride) a[i] = 0ull;
     unsigned long long* b = reinterpret_cast<unsigned long long*>(ws + L.off_ghist);
-    const size_t nb = (L.off_sort_state - L.off_ghist) / 8;  // digit histograms, their scans, selection tile states
+    const size_t nb = (L.off_row_list - L.off_ghist) / 8;  // digit histograms, their scans, selection tile states
     for (size_t i = gtid; i < nb; i += gstride) b[i] = 0ull;
   }
   // look-back states of the digit passes that will run (the fourth only if some client's keys span more than 2^27)
@@ -329,9 +329,8 @@ k_select(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_
   const uint32_t S = part.max_segments;
   const uint32_t* seg_count = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_seg_count(batch.n));
   const unsigned long long* seg_prefix = reinterpret_cast<const unsigned long long*>(plan_ws + plan_off_seg_prefix(batch.n, S));
-  // per segment, the rows of 32 units that hold a candidate, in ascending order (from the planner)
-  const uint32_t* row_list = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_row_list(batch.n, S, row_tiles_total(part)));
-  const uint32_t* seg_rows = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_seg_rows(batch.n, S));
+  const uint32_t* row_max = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_row_max(batch.n, S));
+  uint32_t* row_list = reinterpret_cast<uint32_t*>(ws + L.off_row_list);
   unsigned long long* n_selected = reinterpret_cast<unsigned long long*>(ws + L.off_n_selected);
   const uint64_t nvec = d >> 2;
   const uint64_t units = part.units;
@@ -377,13 +376,60 @@ k_select(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_
     // order is kept).
     constexpr uint32_t kRowsPerWarp = 32 * kSelVec / kRowUnits;
     const uint32_t n_vec32 = (uint32_t)n_vec;  // a segment is at most one chunk: far below 2^32 units
-    const uint32_t n_listed = seg_rows[seg];
+    uint32_t* list = row_list + seg_first_tile(pos, seg) * kTileRows;
+    // ---- the rows that hold a candidate, in ascending order.  Every thread looks at 16 consecutive rows at a time (four
+    // 128-bit loads in flight), one block scan gives their places: a chunk's rows are usually one such step, about 3 us of
+    // the 90 us a chunk takes.  On 10 clients of 1e8 coordinates the list adds 20 us to this kernel; one planner block
+    // per client listing the rows took 215 us more than the planner takes without it.
+    uint32_t n_listed = 0;
+    {
+      constexpr uint32_t kRowsPerThread = 16;
+      const uint32_t n_rows = (n_vec32 + kRowUnits - 1) / kRowUnits;
+      const uint4* __restrict__ rm = reinterpret_cast<const uint4*>(row_max + seg_first_tile(pos, seg) * kTileRows);
+      for (uint32_t r0 = 0; r0 < n_rows; r0 += kSelThreads * kRowsPerThread) {
+        const uint32_t mine = r0 + (uint32_t)tid * kRowsPerThread;
+        uint4 q4[kRowsPerThread / 4];
+#pragma unroll
+        for (uint32_t v = 0; v < kRowsPerThread / 4; ++v) q4[v] = (mine + 4 * v < n_rows) ? __ldg(rm + mine / 4 + v) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t m = 0;
+#pragma unroll
+        for (uint32_t v = 0; v < kRowsPerThread / 4; ++v)
+          m |= ((q4[v].x >= thresh ? 1u : 0u) | (q4[v].y >= thresh ? 2u : 0u) | (q4[v].z >= thresh ? 4u : 0u) | (q4[v].w >= thresh ? 8u : 0u)) << (4 * v);
+        const uint32_t left = (mine < n_rows) ? n_rows - mine : 0u;
+        if (left < kRowsPerThread) m &= (1u << left) - 1u;
+        const uint32_t cnt = __popc(m);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const uint32_t o = __shfl_up_sync(kFull, incl, off);
+          if (lane >= off) incl += o;
+        }
+        if (lane == 31) s_warp_incl[parity][warp] = incl;
+        __syncthreads();
+        const uint32_t wt = (lane < kSelThreads / 32) ? s_warp_incl[parity][lane] : 0u;
+        uint32_t wincl = wt;
+#pragma unroll
+        for (int off = 1; off < kSelThreads / 32; off <<= 1) {
+          const uint32_t o = __shfl_up_sync(kFull, wincl, off);
+          if (lane >= off) wincl += o;
+        }
+        const uint32_t tot = __shfl_sync(kFull, wincl, kSelThreads / 32 - 1);
+        uint32_t o = n_listed + __shfl_sync(kFull, wincl - wt, warp) + incl - cnt;
+        parity ^= 1;
+        while (m) {
+          const uint32_t b = (uint32_t)__ffs(m) - 1u;
+          m &= m - 1u;
+          list[o++] = mine + b;
+        }
+        n_listed += tot;
+      }
+      __syncthreads();  // the list is complete
+    }
     const uint32_t n_tiles = (n_listed + kTileRows - 1) / kTileRows;
-    const uint32_t* __restrict__ list = row_list + seg_first_tile(pos, seg) * kTileRows;
     constexpr uint32_t kNoRow = 0xFFFFFFFFu;
     auto row_at = [&](uint32_t t, uint32_t slot) -> uint32_t {  // the row in slot `slot` of this warp's part of tile t
       const uint32_t idx = t * (uint32_t)kTileRows + (uint32_t)warp * kRowsPerWarp + slot;
-      return (idx < n_listed) ? __ldg(list + idx) : kNoRow;
+      return (idx < n_listed) ? list[idx] : kNoRow;  // written by this block: not for the read-only path
     };
 
     // A warp stages exactly the 128 units (512 coordinates) its own lanes will read: four copies of 32 float4s each,
