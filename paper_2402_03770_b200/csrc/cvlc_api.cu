@@ -420,7 +420,7 @@ int cvlc_encode_unframed_batch(const float* const* x_dev, const cvlc_params* par
   if (S.R > 0x7FFFFFFFu || n > 65535) return CVLC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (launch_encode(desc, n, S, cap, plan_ws_dev, enc_ws_dev, st, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
-  return launch_pack_unframed(desc, n, S, cap, stream_capacity, enc_ws_dev, uf_ws_dev,
+  return launch_pack_unframed(n, S, cap, stream_capacity, enc_ws_dev, uf_ws_dev,
                               reinterpret_cast<unsigned long long*>(stream_bytes_dev), st) == cudaSuccess
              ? CVLC_OK
              : CVLC_ERR_CUDA;
@@ -505,14 +505,14 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   Senc.fixed_y = 0;
   if (launch_plan_front(desc, n, S, plan_ws_dev, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
-    if (launch_plan_back(desc, n, S, plan_ws_dev, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
+    if (launch_plan_back(n, S, plan_ws_dev, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
   // the length tuning reads the histograms' fit only; selection and ranking do not need its result
   cudaEvent_t fork, join;
   if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;
-  if (launch_plan_back(desc, n, S, plan_ws_dev, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_plan_back(n, S, plan_ws_dev, side_st, false) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(join, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
   return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
 }

@@ -11,15 +11,25 @@ constexpr int kDecodeThreads = 256;
 constexpr uint32_t kDecStageWords = 512;  // packets up to 2 KB are staged in shared memory
 constexpr uint64_t kDecodeWindow = 24ull << 20;  // coordinates of the accumulator filled per decode launch (96 MB: inside the L2)
 
+// thread `first` of `stride` writes its share of d zeros
+__device__ __forceinline__ void zero_fill(float* __restrict__ out, uint64_t d, uint64_t first, uint64_t stride) {
+  const uint64_t nvec = d >> 2;
+  float4* ov = reinterpret_cast<float4*>(out);
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (uint64_t v = first; v < nvec; v += stride) ov[v] = z;
+  if (first < (d & 3)) out[(nvec << 2) + first] = 0.f;
+}
+
 struct StreamHead {
   uint32_t magic, ver_q_s, d_lo, d_hi, R, packet_bits, header_bits, client_id, seed_lo, seed_hi, round, zero, B_lo, B_hi, k_lo, k_hi;
 };
 
-// K7a  validate the global headers, derive per-client coefficients and the packet prefix
+// K7a  validate the global headers, derive per-client coefficients and the packet prefix (block 0); meanwhile the other
+// blocks write the zeros of the accumulator's first zero_d coordinates, which depend on nothing
 __global__ void __launch_bounds__(kPrepThreads)
 k_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* __restrict__ stream_bytes,
                  const float* __restrict__ weights, uint32_t n, double weight_total, uint64_t d, uint32_t s,
-                 unsigned char* ws) {
+                 unsigned char* ws, float* __restrict__ zero_out, uint64_t zero_d) {
   __shared__ double s_part[kPrepThreads / 32];
   __shared__ uint32_t s_cnt[kPrepThreads / 32];
   __shared__ double s_W;
@@ -30,6 +40,11 @@ k_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* __r
   uint32_t* prefix = reinterpret_cast<uint32_t*>(ws + dec_off_prefix(n));
   uint32_t* meta = reinterpret_cast<uint32_t*>(ws + dec_off_meta(n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_enter();
+  if (blockIdx.x > 0) {
+    zero_fill(zero_out, zero_d, (uint64_t)(blockIdx.x - 1) * kPrepThreads + tid, (uint64_t)(gridDim.x - 1) * kPrepThreads);
+    return;
+  }
   if (tid == 0) {
     *status = 0;
     s_carry = 0;
@@ -109,11 +124,8 @@ k_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* __r
 // K7b  out = 0 (when not accumulating): 4 bytes written per coordinate
 __global__ void __launch_bounds__(256)
 k_fill_zero(float* __restrict__ out, uint64_t d) {
-  const uint64_t nvec = d >> 2;
-  float4* ov = reinterpret_cast<float4*>(out);
-  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (uint64_t v = (uint64_t)blockIdx.x * 256 + threadIdx.x; v < nvec; v += (uint64_t)gridDim.x * 256) ov[v] = z;
-  if (blockIdx.x == 0 && threadIdx.x < (d & 3)) out[(nvec << 2) + threadIdx.x] = 0.f;
+  pdl_enter();
+  zero_fill(out, d, (uint64_t)blockIdx.x * 256 + threadIdx.x, (uint64_t)gridDim.x * 256);
 }
 
 // A stream word is read once per window pass and should not push the accumulator's window out of the L2.
@@ -131,6 +143,7 @@ __device__ __forceinline__ uint32_t ld_stream(const uint32_t* p, uint64_t pol) {
 // asks for n floats into the L2, one request per 128-byte line
 __global__ void __launch_bounds__(256)
 k_prefetch_l2(const float* __restrict__ p, uint64_t n) {
+  pdl_enter();
   const uint64_t lines = (n * 4 + 127) / 128;
   const char* base = reinterpret_cast<const char*>(p);
   for (uint64_t l = (uint64_t)blockIdx.x * 256 + threadIdx.x; l < lines; l += (uint64_t)gridDim.x * 256)
@@ -179,6 +192,7 @@ k_decode(const uint8_t* const* __restrict__ streams, uint32_t n, uint64_t d, uin
   // coalesced, independent loads; the records are then cut out of shared memory (larger packets: out of global)
   __shared__ uint32_t s_pkt[kDecodeThreads / 32][kDecStageWords + 1];  // one word of slack: the narrow path reads word wi + 1
   uint32_t* sp = s_pkt[threadIdx.x >> 5];
+  pdl_enter();
   int32_t* status = reinterpret_cast<int32_t*>(ws + kDecWsStatus);
   const float* coef = reinterpret_cast<const float*>(ws + kDecWsCoef);
   const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + dec_off_prefix(n));
@@ -288,25 +302,28 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
                           uint32_t n, double weight_total, uint64_t d, uint32_t s, float* out, int accumulate,
                           void* ws, cudaStream_t st) {
   unsigned char* w = static_cast<unsigned char*>(ws);
-  { LaunchScope ls(kKDecodePrepare, st); k_decode_prepare<<<1, kPrepThreads, 0, st>>>(streams, stream_bytes, weights, n, weight_total, d, s, w); }
   // Windows of equal size (a multiple of 1024 coordinates), none above kDecodeWindow.  Each window is brought
   // into the L2 right before its decode launch, by the zero fill or, when accumulating, by a prefetch: a
   // reduction that misses the L2 is a DRAM read-modify-write.
   const uint64_t n_win = (d + kDecodeWindow - 1) / kDecodeWindow;
   const uint64_t win = (((d + n_win - 1) / n_win) + 1023) & ~(uint64_t)1023;
+  auto fill_grid = [](uint64_t coords, uint64_t threads, uint64_t most) -> unsigned {
+    const uint64_t want = (coords / 4 + threads - 1) / threads;
+    return (unsigned)(want < most ? (want ? want : 1) : most);
+  };
+  const uint64_t first = win < d ? win : d;
+  const uint64_t zero_d = accumulate ? 0 : first;
+  launch_kernel(kKDecodePrepare, k_decode_prepare, 1 + (accumulate ? 0 : fill_grid(first, kPrepThreads, 2 * kNumSM)), kPrepThreads, 0, st, true,
+                streams, stream_bytes, weights, n, weight_total, d, s, w, out, zero_d);
   for (uint64_t lo = 0; lo < d; lo += win) {
     const uint64_t hi = lo + win < d ? lo + win : d;
-    const uint64_t want = ((hi - lo) / 4 + 255) / 256;
-    const int grid = (int)(want < (uint64_t)(8 * kNumSM) ? (want ? want : 1) : 8 * kNumSM);
+    const unsigned grid = fill_grid(hi - lo, 256, 8 * kNumSM);
     if (!accumulate) {
-      LaunchScope ls(kKFillZero, st);
-      k_fill_zero<<<grid, 256, 0, st>>>(out + lo, hi - lo);
+      if (lo > 0) launch_kernel(kKFillZero, k_fill_zero, grid, 256, 0, st, true, out + lo, hi - lo);
     } else if (n_win > 1) {
-      LaunchScope ls(kKPrefetchL2, st);
-      k_prefetch_l2<<<grid, 256, 0, st>>>(out + lo, hi - lo);
+      launch_kernel(kKPrefetchL2, k_prefetch_l2, grid, 256, 0, st, true, out + lo, hi - lo);
     }
-    LaunchScope ls(kKDecode, st);
-    k_decode<<<8 * kNumSM, kDecodeThreads, ((size_t)n + 1) * 4, st>>>(streams, n, d, s, out, w, lo, hi);
+    launch_kernel(kKDecode, k_decode, 8 * kNumSM, kDecodeThreads, ((size_t)n + 1) * 4, st, true, streams, n, d, s, out, w, lo, hi);
   }
   return cudaGetLastError();
 }
@@ -314,14 +331,14 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
 cudaError_t launch_fill_zero(float* out, uint64_t d, cudaStream_t st) {
   const uint64_t want = (d / 4 + 255) / 256;
   const int grid = (int)(want < (uint64_t)(8 * kNumSM) ? (want ? want : 1) : 8 * kNumSM);
-  LaunchScope ls(kKFillZero, st);
-  k_fill_zero<<<grid, 256, 0, st>>>(out, d);
+  launch_kernel(kKFillZero, k_fill_zero, grid, 256, 0, st, true, out, d);
   return cudaGetLastError();
 }
 
 // K8  model <- model - aggregate (Section III, step 3); nothing is touched after a decode error
 __global__ void __launch_bounds__(256)
 k_apply(float* __restrict__ model, const float* __restrict__ agg, uint64_t d, const unsigned char* dec_ws) {
+  pdl_enter();
   if (*reinterpret_cast<const int32_t*>(dec_ws + kDecWsStatus) != 0) return;
   const uint64_t nvec = d >> 2;
   float4* mv = reinterpret_cast<float4*>(model);
@@ -345,8 +362,7 @@ cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void*
   const uint64_t nvec = d >> 2;
   const uint64_t want = (nvec + 255) / 256;
   const int grid = (int)(want < (uint64_t)(8 * kNumSM) ? (want ? want : 1) : 8 * kNumSM);
-  LaunchScope ls(kKApply, st);
-  k_apply<<<grid, 256, 0, st>>>(model, agg, d, static_cast<const unsigned char*>(dec_ws));
+  launch_kernel(kKApply, k_apply, grid, 256, 0, st, true, model, agg, d, static_cast<const unsigned char*>(dec_ws));
   return cudaGetLastError();
 }
 
@@ -366,6 +382,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 
 // copies the status word of the scratch to the caller's word (device code names the array directly)
 __global__ void k_noalloc_publish_status(int32_t* status_out) {
+  pdl_enter();
   *status_out = *reinterpret_cast<const int32_t*>(g_noalloc_scratch + kDecWsStatus);
 }
 
@@ -412,10 +429,7 @@ extern "C" int cvlc_decode_aggregate_noalloc(const uint8_t* const* streams_dev, 
   if (launch_decode(streams_dev, stream_bytes_dev, weights_dev, n_clients, weight_total, d, s, out_dev,
                     accumulate ? 1 : 0, scratch, st) != cudaSuccess)
     return CVLC_ERR_CUDA;
-  {
-    LaunchScope ls(kKNoallocStatus, st);
-    k_noalloc_publish_status<<<1, 1, 0, st>>>(status_dev);
-  }
+  launch_kernel(kKNoallocStatus, k_noalloc_publish_status, 1, 1, 0, st, true, status_dev);
   return cudaGetLastError() == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
 }
 

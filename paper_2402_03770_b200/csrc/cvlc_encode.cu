@@ -3,6 +3,8 @@
 // by |x|, the per-packet centroid distribution (PQ: minimum and maximum; QSGD: l2-norm),
 // stochastic quantization with Philox4x32-10 (PQ or QSGD) and bit packing of
 // (position ID, centroid ID) pairs into fixed-size packets (Fig. 2).
+#include <string.h>
+
 #include "cvlc_common.cuh"
 #include "cvlc_lookback.cuh"
 #include "cvlc_quant.cuh"
@@ -38,6 +40,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
   __shared__ int s_bad, s_pass3;
   __shared__ uint32_t s_tiles[CVLC_MAX_BATCH];  // sort tiles of every client
   const uint32_t n = batch.n;
+  pdl_enter();
   if (threadIdx.x == 0) {
     s_total = 0;
     s_bad = 0;
@@ -79,7 +82,9 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
 
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   uint32_t* prefix = reinterpret_cast<uint32_t*>(ws + L.off_sort_prefix);
+  ClientDesc* desc = reinterpret_cast<ClientDesc*>(ws + L.off_desc);
   for (uint32_t c = threadIdx.x; c < n; c += blockDim.x) {
+    desc[c] = batch.c[c];
     // Only what selection and ranking use is checked here (the code lengths may still be on their way on
     // another stream); the packing kernel checks the lengths.
     const cvlc_plan_t* plan = batch.c[c].plan;
@@ -126,13 +131,13 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
 // predecessor of a tile is running or done; the look-back reads 512 predecessors per step.
 // Used when the plan's workspace (and with it the per-segment counts) is not available.
 
-template <int CAP>
 __global__ void __launch_bounds__(kSelectThreads)
-k_select_lookback(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
   __shared__ uint32_t s_tile;
   __shared__ unsigned long long s_warp_incl[kSelectThreads / 32];
   __shared__ unsigned long long s_look_sum[kSelectThreads / 32];
   __shared__ uint32_t s_look_flag[kSelectThreads / 32];
+  pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -314,15 +319,14 @@ constexpr uint32_t kSelTileVec = kSelThreads * kSelVec;  // 2048 float4 = 8192 c
 static_assert(kSelTileVec * 16 == kSelStageBytes, "stage size");
 __device__ __forceinline__ uint32_t sel_slot(uint32_t g) { return g ^ ((g >> 3) & (uint32_t)(kSelVec - 1)); }
 
-template <int CAP>
 __global__ void __launch_bounds__(kSelThreads, 2)
-k_select(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_constant__ Partition part,
+k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
          const unsigned char* __restrict__ plan_ws, unsigned char* ws, const __grid_constant__ EncLayout L) {
   extern __shared__ float4 s_stage[];  // [kSelStages][2048 float4]
   __shared__ uint32_t s_warp_incl[2][kSelThreads / 32];
   __shared__ uint32_t s_dhist[kSortPasses * kDigits];  // digit histograms of the segment's candidates (for the ranking passes)
   for (int i = threadIdx.x; i < kSortPasses * kDigits; i += kSelThreads) s_dhist[i] = 0;
-  __syncthreads();
+  pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -585,10 +589,10 @@ k_select(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_
 // The clients' candidate arrays are concatenated in units of sort tiles (kSortTile pairs) and cut
 // into equal contiguous chunks, one per block; a block that crosses a client boundary merges
 // its shared histograms into that client's and starts afresh.
-template <int CAP>
 __global__ void __launch_bounds__(256)
-k_sort_hist(const __grid_constant__ BatchDesc<CAP> batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_sort_hist(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
   __shared__ uint32_t sh[kSortPasses * kDigits];
+  pdl_enter();
   const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + L.off_sort_prefix);
@@ -629,10 +633,10 @@ k_sort_hist(const __grid_constant__ BatchDesc<CAP> batch, unsigned char* ws, con
 }
 
 // per client: exclusive scans of the four digit histograms and the mask of constant digits
-template <int CAP>
 __global__ void __launch_bounds__(kDigits)
-k_sort_scan(const __grid_constant__ BatchDesc<CAP> batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_sort_scan(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
   __shared__ unsigned long long s_scan[kDigits / 32];
+  pdl_enter();
   const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const uint32_t c = blockIdx.x;
@@ -854,9 +858,8 @@ __device__ __forceinline__ void sort_tile(SortShared& sh, unsigned long long* __
   }
 }
 
-template <int CAP>
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks)
-k_sort_pass(int pass, const __grid_constant__ BatchDesc<CAP> batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_sort_pass(int pass, const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
   static_assert(kSortThreads * 2 >= kDigits && kSortTile <= 0xFFFF, "two digit values per owning thread; 16-bit slots");
   extern __shared__ __align__(16) unsigned char s_raw[];
   SortShared& sh = *reinterpret_cast<SortShared*>(s_raw);
@@ -865,6 +868,7 @@ k_sort_pass(int pass, const __grid_constant__ BatchDesc<CAP> batch, unsigned cha
   uint32_t* s_ncand = s_prefix + (batch.n + 1);  // [n] candidates of the client
   uint32_t* s_keytop = s_ncand + batch.n;        // [n] top of its key range
   uint32_t* s_mask = s_keytop + batch.n;         // [n] its constant digits
+  pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x;
@@ -960,6 +964,7 @@ __global__ void __launch_bounds__(kPackThreads)
 k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape, unsigned char* ws,
        const __grid_constant__ EncLayout L, uint32_t warp_bytes, int write_residual) {
   extern __shared__ __align__(16) unsigned char s_pack[];  // per warp: packet words; QSGD: then cap(1) squares
+  pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1172,87 +1177,83 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
 // ===================================================================================
 
 template <int CAP>
-static cudaError_t launch_encode_t(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                                   const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack,
-                                   int write_residual) {
+static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, const Partition& part,
+                          const unsigned char* plan_ws, unsigned char* w, cudaStream_t st) {
+  BatchDesc<CAP> batch;
+  batch.n = n;
+  batch.pad = 0;
+  memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
+  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, true, w, batch, shape, L, plan_ws, part);
+}
+
+template <int CAP>
+static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, unsigned char* w, size_t warp_bytes,
+                                 int write_residual, cudaStream_t st, bool overlap) {
+  const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
+  auto kernel = qsgd ? k_pack<CAP, true> : k_pack<CAP, false>;
+  if (warp_bytes * kPackWarps > 48 * 1024) {  // large packets only
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e != cudaSuccess) return e;
+  }
+  BatchDesc<CAP> batch;
+  batch.n = n;
+  batch.pad = 0;
+  memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
+  const unsigned grid = (shape.R + kPackWarps * kPackGroup - 1) / (kPackWarps * kPackGroup);
+  launch_kernel(kKPack, kernel, dim3(grid, n), kPackThreads, warp_bytes * kPackWarps, st, overlap, batch, shape, w, L, (uint32_t)warp_bytes, write_residual);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
+                          const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack, int write_residual) {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_pack<CAP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSelStages * kSelStageBytes));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_pack<CAP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_select<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSelStages * kSelStageBytes));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_sort_pass<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
+    e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  BatchDesc<CAP> batch;
-  batch.n = n;
-  batch.pad = 0;
-  for (uint32_t i = 0; i < n; ++i) batch.c[i] = clients[i];
   const EncLayout L = enc_layout(shape.d, n, capacity);
   unsigned char* w = static_cast<unsigned char*>(ws);
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
   // packet words; QSGD: and the squares of a packet's values
   const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
-  const size_t pack_smem = pack_warp * kPackWarps;
-  const unsigned pack_grid = (shape.R + kPackWarps * kPackGroup - 1) / (kPackWarps * kPackGroup);
 
   const Partition part = make_partition(shape.d, n);
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
-  {
-    LaunchScope ls(kKEncodeInit, st);
-    k_encode_init<CAP><<<2 * kNumSM, 256, 0, st>>>(w, batch, shape, L, pws, part);
-  }
+  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, part, pws, w, st);
+  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, part, pws, w, st);
+  else launch_init_t<kLargeBatch>(clients, n, shape, L, part, pws, w, st);
+  const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (pws) {
-    LaunchScope ls(kKSelect, st);
-    k_select<CAP><<<part.grid, kSelThreads, kSelStages * kSelStageBytes, st>>>(batch, shape.d, part, pws, w, L);
+    launch_kernel(kKSelect, k_select, part.grid, kSelThreads, kSelStages * kSelStageBytes, st, true, batch, shape.d, part, pws, w, L);
   } else {
     const uint64_t want = L.select_tiles * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(4 * kNumSM) ? want : 4 * kNumSM);
-    LaunchScope ls(kKSelectLookback, st);
-    k_select_lookback<CAP><<<grid, kSelectThreads, 0, st>>>(batch, shape.d, w, L);
+    launch_kernel(kKSelectLookback, k_select_lookback, grid, kSelectThreads, 0, st, true, batch, shape.d, w, L);
   }
   {
     const uint64_t want = L.sort_tiles_max * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(kSortMinBlocks * kNumSM) ? want : kSortMinBlocks * kNumSM);
-    if (!pws) {  // the selection with known offsets has counted the digits already
-      LaunchScope ls(kKSortHist, st);
-      k_sort_hist<CAP><<<grid, 256, 0, st>>>(batch, w, L);
-    }
-    {
-      LaunchScope ls(kKSortScan, st);
-      k_sort_scan<CAP><<<n, kDigits, 0, st>>>(batch, w, L);
-    }
-    for (int pass = 0; pass < kSortPasses; ++pass) {
-      LaunchScope ls(kKSortPass, st);
-      k_sort_pass<CAP><<<grid, kSortThreads, sort_smem_bytes(n), st>>>(pass, batch, w, L);
-    }
+    if (!pws)  // the selection with known offsets has counted the digits already
+      launch_kernel(kKSortHist, k_sort_hist, grid, 256, 0, st, true, batch, w, L);
+    launch_kernel(kKSortScan, k_sort_scan, n, kDigits, 0, st, true, batch, w, L);
+    for (int pass = 0; pass < kSortPasses; ++pass)
+      launch_kernel(kKSortPass, k_sort_pass, grid, kSortThreads, sort_smem_bytes(n), st, true, pass, batch, w, L);
   }
   if (wait_before_pack) {
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);
     if (ew != cudaSuccess) return ew;
   }
   if (write_residual == kPackNone) return cudaGetLastError();  // the caller writes the ranked records in a format of its own
-  {
-    LaunchScope ls(kKPack, st);
-    if (qsgd)
-      k_pack<CAP, true><<<dim3(pack_grid, n), kPackThreads, pack_smem, st>>>(batch, shape, w, L, (uint32_t)pack_warp, write_residual);
-    else
-      k_pack<CAP, false><<<dim3(pack_grid, n), kPackThreads, pack_smem, st>>>(batch, shape, w, L, (uint32_t)pack_warp, write_residual);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack, int write_residual) {
-  if (n <= (uint32_t)kSmallBatch)
-    return launch_encode_t<kSmallBatch>(clients, n, shape, capacity, plan_ws, ws, st, wait_before_pack, write_residual);
-  return launch_encode_t<kLargeBatch>(clients, n, shape, capacity, plan_ws, ws, st, wait_before_pack, write_residual);
+  const bool overlap = wait_before_pack == nullptr;
+  if (n <= (uint32_t)kSmallBatch) return launch_pack_t<kSmallBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+  if (n <= (uint32_t)kMediumBatch) return launch_pack_t<kMediumBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+  return launch_pack_t<kLargeBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
 }
 
 // memory <- memory + update in fp32, for every client of a batch (the first step of a round with error compensation)
@@ -1260,13 +1261,16 @@ struct EcPair {
   float* memory;
   const float* update;
 };
+template <int CAP>
 struct EcBatch {
   uint32_t n, pad;
-  EcPair c[CVLC_MAX_BATCH];
+  EcPair c[CAP];
 };
 
+template <int CAP>
 __global__ void __launch_bounds__(256)
-k_ec_accumulate(const __grid_constant__ EcBatch batch, uint64_t d) {
+k_ec_accumulate(const __grid_constant__ EcBatch<CAP> batch, uint64_t d) {
+  pdl_enter();
   const uint64_t nvec = d >> 2;
   const uint64_t per_client = nvec + 1;  // float4 units and one unit for the ragged tail
   const uint64_t total = per_client * batch.n;
@@ -1289,8 +1293,9 @@ k_ec_accumulate(const __grid_constant__ EcBatch batch, uint64_t d) {
   }
 }
 
-cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st) {
-  EcBatch batch;
+template <int CAP>
+static void launch_ec_t(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st) {
+  EcBatch<CAP> batch;
   batch.n = n;
   batch.pad = 0;
   for (uint32_t i = 0; i < n; ++i) {
@@ -1299,7 +1304,12 @@ cudaError_t launch_ec_accumulate(float* const* memory, const float* const* updat
   }
   const uint64_t want = (((d >> 2) + 1) * n + 255) / 256;
   const unsigned grid = (unsigned)(want < (uint64_t)(8 * kNumSM) ? want : 8 * kNumSM);
-  { LaunchScope ls(kKEcAccumulate, st); k_ec_accumulate<<<grid, 256, 0, st>>>(batch, d); }
+  launch_kernel(kKEcAccumulate, k_ec_accumulate<CAP>, grid, 256, 0, st, true, batch, d);
+}
+
+cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st) {
+  if (n <= (uint32_t)kMediumBatch) launch_ec_t<kMediumBatch>(memory, update, n, d, st);
+  else launch_ec_t<kLargeBatch>(memory, update, n, d, st);
   return cudaGetLastError();
 }
 

@@ -5,6 +5,8 @@
 // The planner's floating point is IEEE binary64 with every multiply and add
 // rounded separately (the *_rn intrinsics keep the compiler from contracting
 // them), in a fixed order, so that its decisions do not depend on the machine.
+#include <string.h>
+
 #include "cvlc_common.cuh"
 
 namespace cvlc {
@@ -33,12 +35,12 @@ __device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
   return m01 > m23 ? m01 : m23;
 }
 
-template <int CAP>
 __global__ void __launch_bounds__(kHistThreads, 2)
-k_hist(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_constant__ Partition part,
+k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
        unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint32_t* __restrict__ seg_hist_all,
        uint32_t* __restrict__ row_max_all) {
   extern __shared__ uint32_t sh_hist[];  // [kHistSub][4096]
+  pdl_enter();
   for (int i = threadIdx.x; i < kHistSub * CVLC_HIST_BINS; i += kHistThreads) sh_hist[i] = 0;
   __syncthreads();
   uint32_t* my = sh_hist + ((threadIdx.x >> 5) & (kHistSub - 1)) * CVLC_HIST_BINS;
@@ -129,8 +131,15 @@ k_hist(const __grid_constant__ BatchDesc<CAP> batch, uint64_t d, const __grid_co
   }
 }
 
-__global__ void k_zero_words(uint32_t* p, size_t n_words) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += (size_t)gridDim.x * blockDim.x) p[i] = 0;
+// zeroes two ranges of the workspace and leaves the clients' descriptors in it
+template <int CAP>
+__global__ void __launch_bounds__(256)
+k_zero_words(const __grid_constant__ BatchDesc<CAP> batch, ClientDesc* desc, uint4* p, size_t n16, uint4* q, size_t m16) {
+  pdl_enter();
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = first; i < batch.n; i += stride) desc[i] = batch.c[i];
+  for (size_t i = first; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = first; i < m16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ===================================================================================
@@ -313,10 +322,9 @@ __device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, d
 // lengths are tuned, but it never exceeds k_sel = R * cap(shortest candidate length) (every packet at the shortest
 // code; with a fixed length, exactly R * cap(y)), so the selection keeps every coordinate down to the bin that holds
 // rank min(k_sel, d): a superset of the top k whose first k ranks are the top k.
-template <int CAP>
 __global__ void __launch_bounds__(kPlanThreads, 1)
 k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __restrict__ nonfinite_all,
-           const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape,
+           const Batch batch, const __grid_constant__ Shape shape,
            const __grid_constant__ Partition part, unsigned char* ws, int have_segments) {
   extern __shared__ unsigned char smem_raw[];
   unsigned long long* Nsuf = reinterpret_cast<unsigned long long*>(smem_raw);  // [4096] survival counts
@@ -327,6 +335,7 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
   __shared__ uint32_t s_thresh_bin, s_top_bin;
   __shared__ unsigned long long s_seg_warp[kPlanThreads / 32];
   int32_t* ws_status = reinterpret_cast<int32_t*>(ws);
+  pdl_enter();
 
   // blockIdx.x = client
   const unsigned long long* __restrict__ hist = hist_all + (size_t)blockIdx.x * CVLC_HIST_BINS;
@@ -646,9 +655,8 @@ __device__ __noinline__ int fast_sign64(double h, double at, double step, double
   return diff > guard ? 1 : (diff < -guard ? -1 : 0);
 }
 // K2b  code-length tuning, one CTA per client; only the first client of every tuning key does the work
-template <int CAP>
 __global__ void __launch_bounds__(kTuneThreads, 1)
-k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape, unsigned char* ws) {
+k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ PlanShared S;
   __shared__ PlanTab T;
@@ -659,6 +667,7 @@ k_plan_tune(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant_
   const uint32_t c = blockIdx.x;
   const unsigned long long* keys = reinterpret_cast<const unsigned long long*>(ws + plan_off_keys(batch.n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_enter();
 
   const unsigned long long key0 = keys[2 * (size_t)c], key1 = keys[2 * (size_t)c + 1];
   if (key1 == 0ull) return;  // no key: the fit refused this client's histogram
@@ -1307,39 +1316,49 @@ constexpr size_t kFitSmem = 3 * 4096 * 8 + 4096 * 2;  // survival counts, the fi
 static_assert((kNumSM * 2 * kChunksPerBlock + 1) * 4 <= 4096 * 8, "a client's segment counts fit the fit points' place");
 constexpr size_t kTuneSmem = (sizeof(PlanSolver) + 255) & ~(size_t)255;
 
-template <int CAP>
 static cudaError_t plan_attributes() {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_hist<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSub * CVLC_HIST_BINS * 4);
+    e = cudaFuncSetAttribute(k_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSub * CVLC_HIST_BINS * 4);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_plan_fit<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFitSmem);
+    e = cudaFuncSetAttribute(k_plan_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFitSmem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_plan_tune<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTuneSmem);
+    e = cudaFuncSetAttribute(k_plan_tune, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTuneSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
   return cudaSuccess;
 }
 
+// the start of a planning call: the descriptors into the workspace, `bytes` from its start and `more` from `at` on zeroed
+// (multiples of 256 bytes)
 template <int CAP>
-static void fill_batch(BatchDesc<CAP>& batch, const ClientDesc* clients, uint32_t n) {
+static void launch_zero_t(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t off_desc, size_t bytes, size_t at, size_t more, cudaStream_t st) {
+  BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
-  for (uint32_t i = 0; i < n; ++i) batch.c[i] = clients[i];
+  memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
+  const size_t want = (bytes + more) / 16 / 256 + 1;
+  const unsigned grid = (unsigned)(want < (size_t)(4 * kNumSM) ? want : 4 * kNumSM);
+  launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, true, batch, reinterpret_cast<ClientDesc*>(w + off_desc),
+                reinterpret_cast<uint4*>(w), bytes / 16, reinterpret_cast<uint4*>(w + at), more / 16);
+}
+static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, const Partition& part, size_t bytes, size_t at, size_t more, cudaStream_t st) {
+  const size_t off_desc = plan_off_desc(n, part.max_segments);
+  if (n <= (uint32_t)kSmallBatch) launch_zero_t<kSmallBatch>(clients, n, w, off_desc, bytes, at, more, st);
+  else if (n <= (uint32_t)kMediumBatch) launch_zero_t<kMediumBatch>(clients, n, w, off_desc, bytes, at, more, st);
+  else launch_zero_t<kLargeBatch>(clients, n, w, off_desc, bytes, at, more, st);
+  return Batch{reinterpret_cast<const ClientDesc*>(w + off_desc), n};
 }
 
 // histogram of every client, then (unless only the histograms are wanted) fit, threshold and segment tables
-template <int CAP>
-static cudaError_t launch_plan_front_t(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
-                                       unsigned long long* hist_out, cudaStream_t st) {
-  cudaError_t e = plan_attributes<CAP>();
+static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
+                              unsigned long long* hist_out, cudaStream_t st) {
+  cudaError_t e = plan_attributes();
   if (e != cudaSuccess) return e;
-  BatchDesc<CAP> batch;
-  fill_batch(batch, clients, n);
   unsigned char* w = static_cast<unsigned char*>(ws);
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(w + kPlanWsHist);
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
@@ -1347,17 +1366,11 @@ static cudaError_t launch_plan_front_t(const ClientDesc* clients, uint32_t n, co
   const uint64_t row_tiles = row_tiles_total(part);
   uint32_t* seg_hist = reinterpret_cast<uint32_t*>(w + plan_off_seg_hist(n, part.max_segments, row_tiles));
   uint32_t* row_max = reinterpret_cast<uint32_t*>(w + plan_off_row_max(n, part.max_segments));
-  {
-    // header, histograms, flags, tuning keys and segment tables start at zero; the per-segment histograms and the
-    // rows' maxima are written in full by the histogram kernel
-    LaunchScope ls(kKZeroWords, st);
-    k_zero_words<<<2 * kNumSM, 1024, 0, st>>>(reinterpret_cast<uint32_t*>(w), plan_off_row_max(n, part.max_segments) / 4);
-  }
-  {
-    // two resident blocks per SM share the concatenated updates evenly
-    LaunchScope ls(kKHist, st);
-    k_hist<CAP><<<part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st>>>(batch, shape.d, part, hist, flags, seg_hist, row_max);
-  }
+  // header, histograms, flags and tuning keys start at zero; the segment tables, the per-segment histograms and the
+  // rows' maxima are written in full by the kernels that follow
+  const Batch batch = launch_zero(clients, n, w, part, plan_off_seg_count(n), 0, 0, st);
+  // two resident blocks per SM share the concatenated updates evenly
+  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape.d, part, hist, flags, seg_hist, row_max);
   if (hist_out) {
     // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
     // header stays unmarked, so an encode call cannot take it for one that holds a plan's segment tables.
@@ -1365,47 +1378,34 @@ static cudaError_t launch_plan_front_t(const ClientDesc* clients, uint32_t n, co
     if (e2 != cudaSuccess) return e2;
     return cudaMemcpyAsync(hist_out, hist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
   }
-  {
-    LaunchScope ls(kKPlanFit, st);
-    k_plan_fit<CAP><<<n, kPlanThreads, kFitSmem, st>>>(hist, flags, batch, shape, part, w, 1);
-  }
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, part, w, 1);
   return cudaGetLastError();
 }
 
-template <int CAP>
-static cudaError_t launch_plan_back_t(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  cudaError_t e = plan_attributes<CAP>();
-  if (e != cudaSuccess) return e;
-  BatchDesc<CAP> batch;
-  fill_batch(batch, clients, n);
+static cudaError_t plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap) {
   unsigned char* w = static_cast<unsigned char*>(ws);
-  {
-    LaunchScope ls(kKPlanTune, st);
-    k_plan_tune<CAP><<<n, kTuneThreads, kTuneSmem, st>>>(batch, shape, w);
-  }
+  const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n, make_partition(shape.d, n).max_segments)), n};
+  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w);
   return cudaGetLastError();
 }
 
 cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  if (n <= (uint32_t)kSmallBatch) return launch_plan_front_t<kSmallBatch>(clients, n, shape, ws, nullptr, st);
-  return launch_plan_front_t<kLargeBatch>(clients, n, shape, ws, nullptr, st);
+  return plan_front(clients, n, shape, ws, nullptr, st);
 }
 
-cudaError_t launch_plan_back(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  if (n <= (uint32_t)kSmallBatch) return launch_plan_back_t<kSmallBatch>(clients, n, shape, ws, st);
-  return launch_plan_back_t<kLargeBatch>(clients, n, shape, ws, st);
+cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap) {
+  return plan_back(n, shape, ws, st, overlap);
 }
 
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  const cudaError_t e = launch_plan_front(clients, n, shape, ws, st);
+  const cudaError_t e = plan_front(clients, n, shape, ws, nullptr, st);
   if (e != cudaSuccess) return e;
-  return launch_plan_back(clients, n, shape, ws, st);
+  return plan_back(n, shape, ws, st, true);
 }
 
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st) {
-  if (n <= (uint32_t)kSmallBatch) return launch_plan_front_t<kSmallBatch>(clients, n, shape, ws, hist_out, st);
-  return launch_plan_front_t<kLargeBatch>(clients, n, shape, ws, hist_out, st);
+  return plan_front(clients, n, shape, ws, hist_out, st);
 }
 
 // Checks histograms that come from outside: flag bit 0 = a value of exponent 255 (Inf, NaN),
@@ -1414,6 +1414,7 @@ __global__ void __launch_bounds__(256)
 k_hist_check(const unsigned long long* __restrict__ hist_all, uint64_t d, uint32_t* __restrict__ flags) {
   __shared__ unsigned long long s_sum[8];
   __shared__ uint32_t s_nonfinite;
+  pdl_enter();
   const unsigned long long* hist = hist_all + (size_t)blockIdx.x * CVLC_HIST_BINS;
   if (threadIdx.x == 0) s_nonfinite = 0;
   __syncthreads();
@@ -1434,43 +1435,21 @@ k_hist_check(const unsigned long long* __restrict__ hist_all, uint64_t d, uint32
   }
 }
 
-template <int CAP>
-static cudaError_t launch_plan_from_hist_t(const ClientDesc* clients, uint32_t n, const Shape& shape,
-                                           const unsigned long long* hist, void* ws, cudaStream_t st) {
-  cudaError_t e = plan_attributes<CAP>();
+cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const Shape& shape,
+                                  const unsigned long long* hist, void* ws, cudaStream_t st) {
+  const cudaError_t e = plan_attributes();
   if (e != cudaSuccess) return e;
-  BatchDesc<CAP> batch;
-  fill_batch(batch, clients, n);
   unsigned char* w = static_cast<unsigned char*>(ws);
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   const Partition part = make_partition(shape.d, n);
-  {
-    // status word, header and tuning keys start at zero: the header stays unmarked, so an encode call
-    // cannot take this workspace for one that holds segment tables
-    LaunchScope ls(kKZeroWords, st);
-    k_zero_words<<<1, 64, 0, st>>>(reinterpret_cast<uint32_t*>(w), kPlanWsHist / 4);
-  }
-  {
-    LaunchScope ls(kKZeroWords, st);
-    k_zero_words<<<8, 256, 0, st>>>(reinterpret_cast<uint32_t*>(w + plan_off_keys(n)), (plan_off_seg_count(n) - plan_off_keys(n)) / 4);
-  }
-  {
-    LaunchScope ls(kKHistCheck, st);
-    k_hist_check<<<n, 256, 0, st>>>(hist, shape.d, flags);
-  }
-  {
-    LaunchScope ls(kKPlanFit, st);
-    k_plan_fit<CAP><<<n, kPlanThreads, kFitSmem, st>>>(hist, flags, batch, shape, part, w, 0);
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_plan_back_t<CAP>(clients, n, shape, ws, st);
-}
-
-cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const Shape& shape,
-                                  const unsigned long long* hist, void* ws, cudaStream_t st) {
-  if (n <= (uint32_t)kSmallBatch) return launch_plan_from_hist_t<kSmallBatch>(clients, n, shape, hist, ws, st);
-  return launch_plan_from_hist_t<kLargeBatch>(clients, n, shape, hist, ws, st);
+  // status word, header and tuning keys start at zero: the header stays unmarked, so an encode call cannot take this
+  // workspace for one that holds segment tables
+  const Batch batch = launch_zero(clients, n, w, part, kPlanWsHist, plan_off_keys(n), plan_off_seg_count(n) - plan_off_keys(n), st);
+  launch_kernel(kKHistCheck, k_hist_check, n, 256, 0, st, true, hist, shape.d, flags);
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, part, w, 0);
+  const cudaError_t e2 = cudaGetLastError();
+  if (e2 != cudaSuccess) return e2;
+  return plan_back(n, shape, ws, st, true);
 }
 
 // ===================================================================================

@@ -30,9 +30,9 @@ constexpr int kUfWarps = kUfThreads / 32;
 
 // every byte of the output buffers starts at zero: block boundaries share words (they are OR-ed in) and the
 // stream ends with zero padding
-template <int CAP>
 __global__ void __launch_bounds__(256)
-k_uf_clear(const __grid_constant__ BatchDesc<CAP> batch, size_t words16, unsigned char* uf_ws, size_t ws_words) {
+k_uf_clear(const Batch batch, size_t words16, unsigned char* uf_ws, size_t ws_words) {
+  pdl_enter();
   const size_t gtid = (size_t)blockIdx.x * 256 + threadIdx.x, gstride = (size_t)gridDim.x * 256;
   const size_t total = words16 * batch.n;
   for (size_t i = gtid; i < total; i += gstride) {
@@ -65,20 +65,21 @@ __device__ __forceinline__ void or_ones(uint32_t* img, uint32_t pos, uint32_t co
 
 // One warp writes one block.  Blocks are handed out by a per-client ticket, so every earlier block of the client is
 // being written or done when a warp looks back for its bit offset.
-template <int CAP, bool QSGD>
+template <bool QSGD>
 __global__ void __launch_bounds__(kUfThreads)
-k_pack_unframed(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape, unsigned char* enc_ws,
+k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned char* enc_ws,
                 const __grid_constant__ EncLayout L, unsigned char* uf_ws, uint32_t n_pad, uint32_t img_words,
                 uint32_t warp_bytes, unsigned long long* __restrict__ sizes_out) {
   extern __shared__ __align__(16) unsigned char s_uf[];
   __shared__ int s_err;
+  pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(enc_ws);
   if (threadIdx.x == 0) s_err = *reinterpret_cast<const volatile int32_t*>(&hdr->status);
   __syncthreads();
   if (s_err != 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t c = blockIdx.y;
-  const ClientDesc& cd = batch.c[c];
+  const ClientDesc cd = batch.c[c];
   const cvlc_plan_t* __restrict__ plan = cd.plan;
   const uint32_t R = shape.R;
   unsigned char* s_mine = s_uf + (size_t)warp * warp_bytes;
@@ -329,26 +330,22 @@ k_pack_unframed(const __grid_constant__ BatchDesc<CAP> batch, const __grid_const
   }
 }
 
-template <int CAP>
-static cudaError_t launch_pack_unframed_t(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                                          size_t stream_capacity, void* enc_ws, void* uf_ws, unsigned long long* sizes_out,
-                                          cudaStream_t st) {
+cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capacity,
+                                 size_t stream_capacity, void* enc_ws, void* uf_ws, unsigned long long* sizes_out, cudaStream_t st) {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_pack_unframed<CAP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_pack_unframed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_pack_unframed<CAP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_pack_unframed<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  BatchDesc<CAP> batch;
-  batch.n = n;
-  batch.pad = 0;
-  for (uint32_t i = 0; i < n; ++i) batch.c[i] = clients[i];
   const EncLayout L = enc_layout(shape.d, n, capacity);
+  // the encoder has left the descriptors in its workspace
+  const Batch batch{reinterpret_cast<const ClientDesc*>(static_cast<unsigned char*>(enc_ws) + L.off_desc), n};
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
   // the largest block: cap of the shortest admissible length
   const uint32_t y_lo = qsgd ? 2u : 1u;
@@ -363,31 +360,12 @@ static cudaError_t launch_pack_unframed_t(const ClientDesc* clients, uint32_t n,
   }
   const uint32_t img_words = (uint32_t)((bits + 31) / 32);
   const size_t warp_bytes = (size_t)n_pad * 8 + ((((size_t)img_words + 2) * 4 + 15) & ~(size_t)15) + (qsgd ? (size_t)P_max * 8 : 0);
-  {
-    LaunchScope ls(kKZeroWords, st);
-    k_uf_clear<CAP><<<4 * kNumSM, 256, 0, st>>>(batch, stream_capacity / 16, static_cast<unsigned char*>(uf_ws),
-                                                 uf_ws_bytes(n, shape.R) / 4);
-  }
-  {
-    LaunchScope ls(kKPackUnframed, st);
-    const unsigned grid = (shape.R + kUfWarps - 1) / kUfWarps;
-    if (qsgd)
-      k_pack_unframed<CAP, true><<<dim3(grid, n), kUfThreads, warp_bytes * kUfWarps, st>>>(
-          batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), n_pad, img_words,
-          (uint32_t)warp_bytes, sizes_out);
-    else
-      k_pack_unframed<CAP, false><<<dim3(grid, n), kUfThreads, warp_bytes * kUfWarps, st>>>(
-          batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), n_pad, img_words,
-          (uint32_t)warp_bytes, sizes_out);
-  }
+  launch_kernel(kKZeroWords, k_uf_clear, 4 * kNumSM, 256, 0, st, true, batch, stream_capacity / 16, static_cast<unsigned char*>(uf_ws),
+                uf_ws_bytes(n, shape.R) / 4);
+  const unsigned grid = (shape.R + kUfWarps - 1) / kUfWarps;
+  launch_kernel(kKPackUnframed, qsgd ? k_pack_unframed<true> : k_pack_unframed<false>, dim3(grid, n), kUfThreads, warp_bytes * kUfWarps, st, true,
+                batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), n_pad, img_words, (uint32_t)warp_bytes, sizes_out);
   return cudaGetLastError();
-}
-
-cudaError_t launch_pack_unframed(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                                 size_t stream_capacity, void* enc_ws, void* uf_ws, unsigned long long* sizes_out, cudaStream_t st) {
-  if (n <= (uint32_t)kSmallBatch)
-    return launch_pack_unframed_t<kSmallBatch>(clients, n, shape, capacity, stream_capacity, enc_ws, uf_ws, sizes_out, st);
-  return launch_pack_unframed_t<kLargeBatch>(clients, n, shape, capacity, stream_capacity, enc_ws, uf_ws, sizes_out, st);
 }
 
 // ===================================================================================
@@ -408,6 +386,7 @@ k_uf_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* 
   float* coef = reinterpret_cast<float*>(ws + kDecWsCoef);
   uint32_t* prefix = reinterpret_cast<uint32_t*>(ws + dec_off_prefix(n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_enter();
   if (tid == 0) {
     *status = 0;
     s_carry = 0;
@@ -505,6 +484,7 @@ __global__ void __launch_bounds__(kUfDecThreads)
 k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64_t d, float* __restrict__ out, unsigned char* ws) {
   extern __shared__ uint32_t s_dec[];  // [n + 1] block prefix, then per warp kUfMaxRecords positions and codes
   __shared__ int s_err;
+  pdl_enter();
   int32_t* status = reinterpret_cast<int32_t*>(ws + kDecWsStatus);
   const float* coef = reinterpret_cast<const float*>(ws + kDecWsCoef);
   const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + dec_off_prefix(n));
@@ -629,19 +609,13 @@ cudaError_t launch_decode_unframed(const uint8_t* const* streams, const uint64_t
     attr_done[dev] = true;
   }
   unsigned char* w = static_cast<unsigned char*>(ws);
-  {
-    LaunchScope ls(kKDecodePrepare, st);
-    k_uf_decode_prepare<<<1, kUfPrepThreads, 0, st>>>(streams, stream_bytes, weights, n, weight_total, d, s, w);
-  }
+  launch_kernel(kKDecodePrepare, k_uf_decode_prepare, 1, kUfPrepThreads, 0, st, true, streams, stream_bytes, weights, n, weight_total, d, s, w);
   if (!accumulate) {
     e = launch_fill_zero(out, d, st);
     if (e != cudaSuccess) return e;
   }
-  {
-    LaunchScope ls(kKDecodeUnframed, st);
-    const size_t smem = ((size_t)n + 1) * 4 + (size_t)(kUfDecThreads / 32) * 2 * kUfMaxRecords * 4;
-    k_decode_unframed<<<4 * kNumSM, kUfDecThreads, smem, st>>>(streams, n, d, out, w);
-  }
+  const size_t smem = ((size_t)n + 1) * 4 + (size_t)(kUfDecThreads / 32) * 2 * kUfMaxRecords * 4;
+  launch_kernel(kKDecodeUnframed, k_decode_unframed, 4 * kNumSM, kUfDecThreads, smem, st, true, streams, n, d, out, w);
   return cudaGetLastError();
 }
 
