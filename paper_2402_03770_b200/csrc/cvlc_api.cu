@@ -6,6 +6,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <mutex>
+
 #include "cvlc_common.cuh"
 
 using namespace cvlc;
@@ -70,7 +72,7 @@ double coeff_g(double Q, double B) {
 
 // Checks one client's parameters and fills the shape shared by a batch.  The per-length
 // coefficients are rebuilt on the device from scale_B with the same IEEE operations; the host
-// evaluates them here only to reject parameters for which no length is usable.
+// evaluates one here only to reject parameters for which no length is usable.
 int build_shape(const cvlc_params* p, uint32_t fixed_y, Shape* S) {
   Derived D;
   const int rc = derive(p, &D);
@@ -91,10 +93,8 @@ int build_shape(const cvlc_params* p, uint32_t fixed_y, Shape* S) {
     if ((uint64_t)D.R * D.cap[fixed_y] > p->d) return CVLC_ERR_BUDGET_TOO_LARGE;
     return CVLC_OK;
   }
-  bool usable = false;
-  for (uint32_t y = 1; y <= p->max_code_bits; ++y)
-    if (coeff_g(quant_Q(p->quantizer, D.cap[y], y), p->scale_B) > 0.0) usable = true;
-  if (!usable) return CVLC_ERR_SCALE_TOO_SMALL;
+  // the coefficients grow with the length: if any is usable, the longest is
+  if (!(coeff_g(quant_Q(p->quantizer, D.cap[p->max_code_bits], p->max_code_bits), p->scale_B) > 0.0)) return CVLC_ERR_SCALE_TOO_SMALL;
   // an admissible single-length plan must exist: the longest code sends the fewest coordinates
   if ((uint64_t)D.R * D.cap[p->max_code_bits] > p->d) return CVLC_ERR_BUDGET_TOO_LARGE;
   return CVLC_OK;
@@ -103,6 +103,21 @@ int build_shape(const cvlc_params* p, uint32_t fixed_y, Shape* S) {
 bool same_shape(const cvlc_params& a, const cvlc_params& b) {
   return a.d == b.d && a.budget_bits / a.packet_bits == b.budget_bits / b.packet_bits && a.packet_bits == b.packet_bits &&
          a.header_bits == b.header_bits && a.quantizer == b.quantizer && a.max_code_bits == b.max_code_bits;
+}
+
+// The shape of a batch from its first client, the other clients' parameters checked against it.  A client with the first
+// one's shape differs in what depends on scale_B alone: the coefficients grow with the length (Q falls with it and every
+// rounding is monotone), so the longest length tells whether any is usable.
+int batch_shape(const cvlc_params* params, uint32_t i, uint32_t fixed_y, Shape* S) {
+  if (i == 0) return build_shape(&params[0], fixed_y, S);
+  const cvlc_params& p = params[i];
+  if (!params_ok(&p) || !same_shape(params[0], p)) {
+    Shape other;
+    const int rc = build_shape(&p, fixed_y, &other);
+    return rc != CVLC_OK ? rc : CVLC_ERR_INVALID_ARG;
+  }
+  if (fixed_y) return CVLC_OK;
+  return coeff_g(quant_Q(p.quantizer, S->cap[p.max_code_bits], p.max_code_bits), p.scale_B) > 0.0 ? CVLC_OK : CVLC_ERR_SCALE_TOO_SMALL;
 }
 
 bool aligned(const void* p, size_t a) { return p && (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -186,10 +201,8 @@ int cvlc_plan_batch(const float* const* x_dev, const cvlc_params* params, uint32
   Shape S;
   ClientDesc desc[CVLC_MAX_BATCH];
   for (uint32_t i = 0; i < n; ++i) {
-    Shape Si;
-    const int rc = build_shape(&params[i], fixed_y, i == 0 ? &S : &Si);
+    const int rc = batch_shape(params, i, fixed_y, &S);
     if (rc != CVLC_OK) return rc;
-    if (i && !same_shape(params[0], params[i])) return CVLC_ERR_INVALID_ARG;
     if (!aligned(x_dev[i], 16)) return CVLC_ERR_INVALID_ARG;
     desc[i].x = x_dev[i];
     desc[i].plan = plans_dev + i;
@@ -232,10 +245,8 @@ int cvlc_plan_from_histogram_batch(const uint64_t* hist_dev, const cvlc_params* 
   Shape S;
   ClientDesc desc[CVLC_MAX_BATCH];
   for (uint32_t i = 0; i < n; ++i) {
-    Shape Si;
-    const int rc = build_shape(&params[i], 0, i == 0 ? &S : &Si);
+    const int rc = batch_shape(params, i, 0, &S);
     if (rc != CVLC_OK) return rc;
-    if (i && !same_shape(params[0], params[i])) return CVLC_ERR_INVALID_ARG;
     memset(&desc[i], 0, sizeof desc[i]);
     desc[i].plan = plans_dev + i;
     desc[i].seed = params[i].seed;
@@ -297,12 +308,15 @@ static int encode_batch(const float* const* x_dev, const cvlc_params* params, ui
                         uint64_t max_candidates, void* ws_dev, size_t ws_bytes, void* cuda_stream, int write_residual) {
   if (!x_dev || !params || !streams_dev || n == 0 || n > CVLC_MAX_BATCH) return CVLC_ERR_INVALID_ARG;
   Shape S;
+  Derived D;
   ClientDesc desc[CVLC_MAX_BATCH];
   for (uint32_t i = 0; i < n; ++i) {
-    Derived D;
-    const int rc = derive(&params[i], &D);
-    if (rc != CVLC_OK) return rc;
-    if (i && !same_shape(params[0], params[i])) return CVLC_ERR_INVALID_ARG;
+    if (i == 0 || !params_ok(&params[i]) || !same_shape(params[0], params[i])) {
+      Derived Di;
+      const int rc = derive(&params[i], i == 0 ? &D : &Di);
+      if (rc != CVLC_OK) return rc;
+      if (i) return CVLC_ERR_INVALID_ARG;
+    }
     if (!aligned(x_dev[i], 16) || !aligned(streams_dev[i], 16)) return CVLC_ERR_INVALID_ARG;
     if (i == 0) {
       memset(&S, 0, sizeof S);
@@ -383,13 +397,16 @@ int cvlc_encode_unframed_batch(const float* const* x_dev, const cvlc_params* par
                                void* uf_ws_dev, size_t uf_ws_bytes_given, void* cuda_stream) {
   if (!x_dev || !params || !streams_dev || n == 0 || n > CVLC_MAX_BATCH) return CVLC_ERR_INVALID_ARG;
   Shape S;
+  Derived D;
   ClientDesc desc[CVLC_MAX_BATCH];
   size_t need_capacity = 0;
   for (uint32_t i = 0; i < n; ++i) {
-    Derived D;
-    const int rc = derive(&params[i], &D);
-    if (rc != CVLC_OK) return rc;
-    if (i && !same_shape(params[0], params[i])) return CVLC_ERR_INVALID_ARG;
+    if (i == 0 || !params_ok(&params[i]) || !same_shape(params[0], params[i])) {
+      Derived Di;
+      const int rc = derive(&params[i], i == 0 ? &D : &Di);
+      if (rc != CVLC_OK) return rc;
+      if (i) return CVLC_ERR_INVALID_ARG;
+    }
     if (!aligned(x_dev[i], 16) || !aligned(streams_dev[i], 16)) return CVLC_ERR_INVALID_ARG;
     if (i == 0) {
       if (!unframed_fits(D, &params[0], &need_capacity)) return CVLC_ERR_INVALID_ARG;  // blocks of more than 2048 records
@@ -479,10 +496,8 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   Shape S;
   ClientDesc desc[CVLC_MAX_BATCH];
   for (uint32_t i = 0; i < n; ++i) {
-    Shape Si;
-    const int rc = build_shape(&params[i], fixed_y, i == 0 ? &S : &Si);
+    const int rc = batch_shape(params, i, fixed_y, &S);
     if (rc != CVLC_OK) return rc;
-    if (i && !same_shape(params[0], params[i])) return CVLC_ERR_INVALID_ARG;
     if (!aligned(x_dev[i], 16) || !aligned(streams_dev[i], 16)) return CVLC_ERR_INVALID_ARG;
     desc[i].x = x_dev[i];
     desc[i].plan = plans_dev + i;
@@ -508,7 +523,10 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
     if (launch_plan_back(n, S, plan_ws_dev, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
-  // the length tuning reads the histograms' fit only; selection and ranking do not need its result
+  // the length tuning reads the histograms' fit only; selection and ranking do not need its result.  The lock keeps two
+  // threads from recording the device's events between each other's record and wait.
+  static std::mutex order;
+  std::lock_guard<std::mutex> hold(order);
   cudaEvent_t fork, join;
   if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;
