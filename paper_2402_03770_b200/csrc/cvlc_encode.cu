@@ -1052,7 +1052,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
 
     if constexpr (QSGD) {
       // ---- QSGD: |x| against the packet's l2-norm; code = sign bit above a level of s_q = 2^(y-1) - 1 steps ----
-      double* sqv = reinterpret_cast<double*>(s_mine + (((size_t)n_words * 4 + 15) & ~(size_t)15));
+      double* sqv = reinterpret_cast<double*>(s_mine + (((size_t)n_words * 4 + 8 + 15) & ~(size_t)15));
       for (uint32_t j = lane; j < P; j += 32) {
         const double a = (double)__uint_as_float((uint32_t)(seg[j] >> 32));
         sqv[j] = __dmul_rn(a, a);  // exact: 24 x 24 bits
@@ -1068,6 +1068,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
       const double sqd = (double)sq;
       const double dn = (double)norm;
       const double scale = (norm > 0.0f) ? __ddiv_rn(sqd, dn) : 0.0;
+      const float fscale = fast_scale(scale, y - 1);
       for (uint32_t j = lane; j < P; j += 32) {
         const unsigned long long pair = seg[j];
         const uint32_t key = (uint32_t)(pair >> 32);
@@ -1075,9 +1076,8 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
         const uint32_t sign = key ? (((uint32_t)pair >> 31) & 1u) : 0u;  // -0 is stored as +0
         uint32_t level = 0;
         if (norm > 0.0f) {
-          const double a = (double)__uint_as_float(key);
-          const double u = __dmul_rn((double)philox_coord(rk, cd.client_id, cd.round, pid), 1.0 / 4294967296.0);
-          level = qsgd_quantize_level(a, dn, sqd, sq, scale, u);
+          const uint32_t word = philox_coord(rk, cd.client_id, cd.round, pid);
+          if (!fast_round(__uint_as_float(key), fscale, (float)sqd, word, level)) level = qsgd_quantize_slow(__uint_as_float(key), norm, sq, word);
         }
         const uint32_t code = (sign << (y - 1)) | level;
         put(j, (unsigned long long)pid | ((unsigned long long)code << s));
@@ -1112,17 +1112,43 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
       const double dlo = (double)lo;
       const double den = __dsub_rn((double)hi, dlo);
       const double scale = (hi != lo) ? __ddiv_rn(Lc, den) : 0.0;
+      const float fscale = fast_scale(scale, y);
       const double cstep = (hi != lo) ? __ddiv_rn(den, Lc) : 0.0;  // distance of two centroids
-      for (uint32_t j = lane; j < P; j += 32) {
+      const bool plain = !residual && hi != lo;
+      if (plain) {
+        // the usual case, without a branch but for the rounding fp32 cannot tell; the next record is requested ahead
+        const float fL = (float)Lc;
+        unsigned long long next = (uint32_t)lane < P ? seg[lane] : 0ull;
+        uint32_t bitpos = H + (uint32_t)lane * wd;
+        for (uint32_t j = lane; j < P; j += 32, bitpos += 32 * wd) {
+          const unsigned long long pair = next;
+          if (j + 32 < P) next = seg[j + 32];
+          const uint32_t key = (uint32_t)(pair >> 32), pid = (uint32_t)pair & 0x7FFFFFFFu;
+          const float v = __uint_as_float(key | ((uint32_t)pair & 0x80000000u));
+          const uint32_t word = philox_coord(rk, cd.client_id, cd.round, pid);
+          uint32_t code;
+          if (!fast_round(__fsub_rn(v, lo), fscale, fL, word, code)) code = pq_quantize_slow(v, lo, hi, y, word);
+          const uint32_t r0 = pid | (code << s), sh = bitpos & 31u;
+          uint32_t* w = words + (bitpos >> 5);
+          atomicOr(w, r0 << sh);
+          if (narrow) {
+            atomicOr(w + 1, __funnelshift_l(r0, 0u, sh));  // zero behind the packet's last word
+          } else {
+            const uint32_t r1 = __funnelshift_l(code, 0u, s);
+            atomicOr(w + 1, __funnelshift_l(r0, r1, sh));
+            atomicOr(w + 2, __funnelshift_l(r1, 0u, sh));
+          }
+        }
+      }
+      for (uint32_t j = plain ? P : lane; j < P; j += 32) {
         const unsigned long long pair = seg[j];
         const uint32_t key = (uint32_t)(pair >> 32);
         const uint32_t pid = (uint32_t)pair & 0x7FFFFFFFu;
         const uint32_t b = key ? (key | ((uint32_t)pair & 0x80000000u)) : 0u;
         uint32_t code = 0;
         if (hi != lo) {
-          const double num = __dsub_rn((double)__uint_as_float(b), dlo);
-          const double u = __dmul_rn((double)philox_coord(rk, cd.client_id, cd.round, pid), 1.0 / 4294967296.0);
-          code = pq_quantize(num, den, Lc, scale, u);
+          const uint32_t word = philox_coord(rk, cd.client_id, cd.round, pid);
+          if (!fast_round(__fsub_rn(__uint_as_float(b), lo), fscale, (float)Lc, word, code)) code = pq_quantize_slow(__uint_as_float(b), lo, hi, y, word);
         }
         put(j, (unsigned long long)pid | ((unsigned long long)code << s));
         if (residual) {
@@ -1220,8 +1246,8 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const EncLayout L = enc_layout(shape.d, n, capacity);
   unsigned char* w = static_cast<unsigned char*>(ws);
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
-  // packet words; QSGD: and the squares of a packet's values
-  const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
+  // packet words and two more; QSGD: and the squares of a packet's values
+  const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
 
   const Partition part = make_partition(shape.d, n);
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
