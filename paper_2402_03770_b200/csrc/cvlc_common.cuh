@@ -66,95 +66,79 @@ struct Shape {
 
 // ---- workspace layouts (byte offsets; every region 256-byte aligned) ----------
 
-// The histogram and the selection kernel stream the clients' updates as one concatenated
-// array of units (a unit = one float4; every client ends with one ragged-tail unit) cut into
-// equal contiguous chunks, several per thread block (the histogram takes them round-robin, the
-// selection by ticket, because its cost per chunk depends on how many candidates it holds).
-// A segment is the part of one client inside one chunk; with chunk q and client c both
-// non-decreasing along the array, q + c numbers the segments uniquely.
+// The float4 units of an update are grouped into rows of kRowUnits (64 coordinates, half of a warp-wide load).  The histogram
+// kernel streams the clients' rows as one concatenated array cut into equal contiguous chunks and leaves the largest magnitude
+// key of every row; the selection reads only the rows that hold a candidate (a key at or above the threshold).  The ragged
+// tail of an update (d % 4 coordinates) goes with its last row.
 constexpr int kStreamThreads = 512;
-constexpr int kChunksPerBlock = 8;
+constexpr int kRowUnits = 16;
 struct Partition {
-  uint64_t units;         // per client: d / 4 float4 units + 1 tail unit
-  uint64_t total;         // units * n
-  uint64_t chunk;         // units per chunk
+  uint64_t rows;      // per client
+  uint64_t total;     // rows * n
+  uint64_t chunk;     // rows per chunk of the histogram kernel
   uint32_t n_chunks;
-  uint32_t grid;          // blocks
-  uint32_t max_segments;  // n_chunks + n
-  uint32_t pad;
+  uint32_t grid;      // its blocks
 };
 CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   Partition P;
-  P.units = (d >> 2) + 1;
-  P.total = P.units * n;
-  uint64_t grid = (P.total + 4 * kStreamThreads - 1) / (4 * kStreamThreads);
+  P.rows = ((d >> 2) + kRowUnits - 1) / kRowUnits;
+  if (P.rows == 0) P.rows = 1;
+  P.total = P.rows * n;
+  uint64_t grid = (P.total + 63) / 64;
   if (grid > (uint64_t)(2 * kNumSM)) grid = 2 * kNumSM;
-  if (grid == 0) grid = 1;
   P.grid = (uint32_t)grid;
-  // chunks of at least 16 tiles of 2048 units, at most kChunksPerBlock per block
-  uint64_t n_chunks = P.total / (16 * 4 * kStreamThreads);
-  if (n_chunks > grid * kChunksPerBlock) n_chunks = grid * kChunksPerBlock;
-  if (n_chunks < grid) n_chunks = grid;
+  // two chunks per block where that leaves each 64 KB and more: every chunk ends with a merge into a client's histogram
+  const uint64_t n_chunks = P.total / (2 * grid) >= 256 ? 2 * grid : grid;
   P.chunk = (P.total + n_chunks - 1) / n_chunks;
   P.n_chunks = (uint32_t)((P.total + P.chunk - 1) / P.chunk);
-  P.max_segments = P.n_chunks + n;
-  P.pad = 0;
   return P;
 }
 
-// Rows: the float4 units of a segment are also grouped into rows of 16 units (64 coordinates, half of a warp-wide
-// load).  The histogram kernel leaves the largest magnitude key of every row; the selection kernel lists, per segment and
-// in ascending order, the rows that hold a candidate (a key at or above the threshold) and works through that list 128
-// rows (one tile of its staging buffers) at a time: rows without candidates are not read.  Both tables are indexed by row; row r of the segment that
-// starts at position p0 of the concatenated array sits at 128 * (p0 / 2048 + segment id) + r, so that the index
-// ranges of different segments do not overlap.
-constexpr int kRowUnits = 16;
-constexpr int kTileUnits = 2048;                    // 2048 float4 = 8192 coordinates: a tile of the selection kernel
-constexpr int kTileRows = kTileUnits / kRowUnits;   // 128
-CVLC_HD inline uint64_t row_tiles_total(const Partition& P) { return P.total / kTileUnits + P.max_segments + 1; }
-CVLC_HD inline uint64_t seg_first_tile(uint64_t p0, uint32_t seg) { return p0 / kTileUnits + seg; }
-
 // plan workspace:
-//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2]
-//   | uint32 seg_count[S] | uint64 seg_prefix[S] | ClientDesc[n] | uint32 row_max[128 * tiles] | uint32 seg_hist[S][4096]
-//   (S = max_segments, tiles = row_tiles_total)
+//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2] | ClientDesc[n]
+//   | uint32 bin_start[n][4096] | uint32 max_bin[n] | uint32 row_max[n][rows]
+// bin_start: candidates of the client in the bins above this one; max_bin: candidates in its fullest bin.
 // tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths;
 // the first of them runs the length tuning and writes the result to all.
 struct PlanWsHeader {
   int32_t status;   // byte 0
   uint32_t n;       // clients of the batch the workspace was filled for
   uint64_t d;
-  uint32_t n_chunks;
-  uint32_t magic;   // set when the segment tables are valid
+  uint32_t pad;
+  uint32_t magic;   // set when the bins' tables and the rows' maxima are valid
 };
 constexpr uint32_t kPlanWsMagic = 0x53454743u;
 constexpr size_t kPlanWsHist = 256;
 CVLC_HD constexpr size_t plan_off_flags(uint32_t n) { return kPlanWsHist + (size_t)n * CVLC_HIST_BINS * 8; }
 CVLC_HD constexpr size_t plan_off_keys(uint32_t n) { return align256(plan_off_flags(n) + (size_t)n * 4); }
-CVLC_HD constexpr size_t plan_off_seg_count(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
-CVLC_HD constexpr size_t plan_off_seg_prefix(uint32_t n, uint32_t S) { return align256(plan_off_seg_count(n) + (size_t)S * 4); }
-CVLC_HD constexpr size_t plan_off_desc(uint32_t n, uint32_t S) { return align256(plan_off_seg_prefix(n, S) + (size_t)S * 8); }
-CVLC_HD constexpr size_t plan_off_row_max(uint32_t n, uint32_t S) { return align256(plan_off_desc(n, S) + (size_t)n * sizeof(ClientDesc)); }
-CVLC_HD constexpr size_t plan_off_seg_hist(uint32_t n, uint32_t S, uint64_t tiles) {
-  return align256(plan_off_row_max(n, S) + (size_t)tiles * kTileRows * 4);
-}
-CVLC_HD constexpr size_t plan_ws_bytes(uint32_t n, uint32_t S, uint64_t tiles) {
-  return align256(plan_off_seg_hist(n, S, tiles) + (size_t)S * CVLC_HIST_BINS * 4);
-}
-CVLC_HD inline size_t plan_ws_bytes(const Partition& P, uint32_t n) { return plan_ws_bytes(n, P.max_segments, row_tiles_total(P)); }
+CVLC_HD constexpr size_t plan_off_desc(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
+CVLC_HD constexpr size_t plan_off_bin_start(uint32_t n) { return align256(plan_off_desc(n) + (size_t)n * sizeof(ClientDesc)); }
+CVLC_HD constexpr size_t plan_off_max_bin(uint32_t n) { return align256(plan_off_bin_start(n) + (size_t)n * CVLC_HIST_BINS * 4); }
+CVLC_HD constexpr size_t plan_off_row_max(uint32_t n) { return align256(plan_off_max_bin(n) + (size_t)n * 4); }
+CVLC_HD inline size_t plan_ws_bytes(const Partition& P, uint32_t n) { return align256(plan_off_row_max(n) + (size_t)P.total * 4); }
 
-// encode workspace header (first 256 bytes), zeroed at the start of a call
+// encode workspace header (first 256 bytes), written at the start of a call
 struct EncHeader {
   int32_t status;           // byte 0
-  uint32_t select_ticket;   // tile tickets of the selection kernel
-  uint32_t sort_ticket[4];  // tile tickets of the four digit passes
+  uint32_t lsd;             // kRankPartition, kRankDigits or kRankAllDigits
+  uint32_t select_ticket;   // tile tickets of the look-back selection
+  uint32_t split_ticket, rank_ticket;  // tile tickets of the partition and of the final ranking
+  uint32_t split_tiles;     // largest per-client tile count among the clients that need the partition
+  uint32_t window;          // candidates per tile of the final ranking
+  uint32_t rank_tiles;      // largest per-client tile count of the final ranking
+  uint32_t sort_ticket;     // work items of the digit passes
+  uint32_t sort_done[8];    // finished items of their phases
   uint32_t total_sort_tiles;
   uint32_t max_sort_tiles;  // largest per-client tile count of this batch
 };
 
+// How a batch is ranked: by partition into buckets; by digit passes over candidates selected in index order; or by digit passes
+// with the selection done over again in that order, because a bucket turned out too large for the partition.
+constexpr uint32_t kRankPartition = 0, kRankDigits = 1, kRankAllDigits = 2;
+
 constexpr int kSelectThreads = 512;
-constexpr int kSelectVecPerThread = 4;                                 // float4 loads per thread per tile
-constexpr int kSelectTile = kSelectThreads * kSelectVecPerThread * 4;  // 8192 coordinates
+constexpr int kSelectVecPerThread = 4;  // float4 loads per thread per tile of the look-back selection
+CVLC_HD constexpr uint64_t select_tiles_of(uint64_t d, int threads) { return (d + threads * kSelectVecPerThread * 4 - 1) / (threads * kSelectVecPerThread * 4); }
 
 constexpr int kSortThreads = 256;
 constexpr int kSortItemsPerThread = 20;  // 128 registers per thread hold a tile without spilling: two blocks per SM
@@ -164,19 +148,70 @@ constexpr int kSortPasses = 4;                                 // digits of 9,9,
 constexpr int kDigitBits = 9;
 constexpr int kDigits = 1 << kDigitBits;                       // 512 digit values
 
+// Ranking by partition.  The sort key of a candidate is inv = keytop - key, keytop the largest key of the client's top bin,
+// so that histogram bins (and groups of them) are ranges of inv whose counts the planner knows: the selection writes every
+// candidate straight into its coarse bucket, in any order.  A bucket that a block can hold is then ranked in shared memory
+// by (inv, index); where coarse buckets are larger, a partition by the next bits of inv comes in between, with the
+// sub-buckets' counts taken by the selection.
+constexpr uint32_t kRankCoarse = 256;      // coarse buckets of a client
+constexpr uint32_t kRankSubs = 8192;       // sub-buckets of a client
+constexpr uint32_t kRankItems = 8192;      // candidates a block of the final ranking holds
+constexpr uint32_t kRankBucket = 4096;     // largest coarse bucket that is ranked without a partition
+constexpr uint32_t kRankWindow = 4096;     // candidates of a tile of the final ranking
+constexpr uint32_t kRankSplitTile = 4096;  // candidates of a tile of the partition
+constexpr uint32_t kRankLargest = 65536;   // a larger bucket (equal keys) sends the batch to the digit passes
+struct ClientRank {
+  uint32_t n;          // candidates
+  uint32_t keytop;     // largest key of the top bin
+  uint32_t group;      // a coarse bucket holds 2^group histogram bins
+  uint32_t n_coarse;
+  uint32_t sub_bits;   // a coarse bucket holds 2^sub_bits sub-buckets
+  uint32_t split;      // 1: coarse buckets are partitioned into sub-buckets
+  uint32_t top_bin, pad;
+};
+// The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates.  As few
+// sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that a block
+// meets costs the selection a global addition).  Returns false where even the most leave more than a block holds, or where
+// zeros are candidates (more coordinates are sent than are not zero): such a batch takes the digit passes, whose cost does
+// not depend on the values.
+CVLC_HD inline bool rank_shape(uint32_t nb, uint32_t max_bin, uint32_t thresh_bin, ClientRank* r) {
+  uint32_t g = 0;
+  while (((nb - 1) >> g) + 1 > kRankCoarse) ++g;
+  r->group = g;
+  r->n_coarse = ((nb - 1) >> g) + 1;
+  const uint64_t fullest = (uint64_t)max_bin << g;
+  r->split = fullest > kRankBucket ? 1u : 0u;
+  uint32_t k = 0;
+  while ((fullest >> k) > kRankItems - kRankWindow && (r->n_coarse << (k + 1)) <= kRankSubs && k < 16) ++k;
+  r->sub_bits = k;
+  return (fullest >> k) <= kRankItems && fullest < (1u << 24) && thresh_bin != 0;
+}
+// Rows a warp of the selection takes at a time: a small batch is spread over all warps, a large one asks a client's counter (one
+// answer in about 20 ns) less often.
+constexpr int kSelThreads = 768;
+CVLC_HD inline uint32_t select_group_rows(const Partition& P) {
+  const uint64_t per_warp = P.total / ((uint64_t)kNumSM * (kSelThreads / 32));
+  return per_warp < 32 ? 8u : (per_warp < 1024 ? 32u : 128u);
+}
+
 struct EncLayout {
   uint32_t n;
   uint64_t capacity;             // candidate slots per client
-  uint64_t select_tiles;         // per client
+  uint64_t select_tiles;         // per client, of the look-back selection's smaller tiles
   uint64_t sort_tiles_max;       // per client
-  size_t off_n_selected;         // uint64[n]
+  size_t off_rank;               // ClientRank[n]
   size_t off_sort_prefix;        // uint32[n + 1]: first sort tile of every client
   size_t off_pass_mask;          // uint32[n]: digit passes that are constant for the client
   size_t off_desc;               // ClientDesc[n]
+  size_t off_group_next;         // uint32[n]: next group of rows of the client
+  size_t off_group_done;         // uint32[n]: groups whose candidates are in place
+  size_t off_bin_fill;           // uint32[n][kRankCoarse]: candidates placed in every coarse bucket
+  size_t off_sub_count;          // float[n][kRankSubs]
+  size_t off_sub_start;          // uint32[n][kRankSubs + 64]: exclusive prefix, then the client's candidates
+  size_t off_sub_pos;            // uint32[n][kRankSubs]: next free place
   size_t off_ghist;              // uint64[n][4][512] digit histograms
   size_t off_gbase;              // uint64[n][4][512] their exclusive scans
   size_t off_select_state;       // uint64[n][select_tiles]
-  size_t off_row_list;           // uint32[128 * row_tiles_total]: rows that hold candidates
   size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]
   size_t off_buf_a, off_buf_b;   // uint64[n][capacity]
   size_t total;
@@ -186,17 +221,22 @@ static inline EncLayout enc_layout(uint64_t d, uint32_t n, uint64_t capacity) {
   EncLayout L;
   L.n = n;
   L.capacity = capacity;
-  L.select_tiles = (d + kSelectTile - 1) / kSelectTile;
+  L.select_tiles = select_tiles_of(d, kSortThreads);
   L.sort_tiles_max = (capacity + kSortTile - 1) / kSortTile;
-  L.off_n_selected = 256;
-  L.off_sort_prefix = align256(L.off_n_selected + (size_t)n * 8);
+  L.off_rank = 256;
+  L.off_sort_prefix = align256(L.off_rank + (size_t)n * sizeof(ClientRank));
   L.off_pass_mask = align256(L.off_sort_prefix + ((size_t)n + 1) * 4);
   L.off_desc = align256(L.off_pass_mask + (size_t)n * 4);
-  L.off_ghist = align256(L.off_desc + (size_t)n * sizeof(ClientDesc));
+  L.off_group_next = align256(L.off_desc + (size_t)n * sizeof(ClientDesc));
+  L.off_group_done = align256(L.off_group_next + (size_t)n * 4);
+  L.off_bin_fill = align256(L.off_group_done + (size_t)n * 4);
+  L.off_sub_count = align256(L.off_bin_fill + (size_t)n * kRankCoarse * 4);
+  L.off_sub_start = align256(L.off_sub_count + (size_t)n * kRankSubs * 4);
+  L.off_sub_pos = align256(L.off_sub_start + (size_t)n * (kRankSubs + 64) * 4);
+  L.off_ghist = align256(L.off_sub_pos + (size_t)n * kRankSubs * 4);
   L.off_gbase = align256(L.off_ghist + (size_t)n * kSortPasses * kDigits * 8);
   L.off_select_state = align256(L.off_gbase + (size_t)n * kSortPasses * kDigits * 8);
-  L.off_row_list = align256(L.off_select_state + (size_t)n * L.select_tiles * 8);
-  L.off_sort_state = align256(L.off_row_list + (size_t)row_tiles_total(make_partition(d, n)) * kTileRows * 4);
+  L.off_sort_state = align256(L.off_select_state + (size_t)n * L.select_tiles * 8);
   L.off_buf_a = align256(L.off_sort_state + (size_t)kSortPasses * n * L.sort_tiles_max * kDigits * 8);
   L.off_buf_b = align256(L.off_buf_a + (size_t)n * capacity * 8);
   L.total = align256(L.off_buf_b + (size_t)n * capacity * 8);
@@ -215,8 +255,8 @@ CVLC_HD constexpr size_t dec_ws_bytes(uint32_t n) { return align256(dec_off_meta
 // ---- launch accounting and optional per-kernel timing ------------------------------
 
 enum KernelId {
-  kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKSortHist, kKSortScan,
-  kKSortPass, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
+  kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
+  kKSort, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
   kKPlanLiteral, kKEcAccumulate, kKPackUnframed, kKDecodeUnframed, kNumKernelIds
 };
 
@@ -285,6 +325,8 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
                                 unsigned long long k_lo, unsigned long long k_hi, double P_min, double P_max, double tol,
                                 cvlc_literal_plan_t* out, double* P_star, void* ws, cudaStream_t st);
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
+// ranking by partition (after the selection); returns at once on the device where the batch is ranked by digit passes
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, int index_bits, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into
@@ -375,6 +417,12 @@ __device__ __forceinline__ uint32_t philox_coord(const PhiloxRoundKeys& rk, uint
     c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk.x[i], (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ rk.y[i], (uint32_t)p0);
   }
   return c.x;
+}
+
+__device__ __forceinline__ uint32_t sort_keytop(const cvlc_plan_t* plan) { return ((plan->top_bin + 1u) << 19) - 1u; }
+// candidates of a client in the coarse buckets before bucket i (bins from the top down)
+__device__ __forceinline__ uint32_t coarse_start(const ClientRank& r, const uint32_t* bin_start, uint32_t i) {
+  return i < r.n_coarse ? bin_start[r.top_bin - (i << r.group)] : r.n;
 }
 
 __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {

@@ -35,9 +35,10 @@ __device__ __forceinline__ uint32_t sort_tiles_of(unsigned long long n_candidate
 template <int CAP>
 __global__ void __launch_bounds__(256)
 k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape,
-              const __grid_constant__ EncLayout L, const unsigned char* plan_ws, const __grid_constant__ Partition part) {
+              const __grid_constant__ EncLayout L, const unsigned char* plan_ws) {
   __shared__ unsigned long long s_total;
-  __shared__ int s_bad, s_pass3;
+  __shared__ int s_bad, s_pass3, s_lsd;
+  __shared__ uint32_t s_most, s_most_split;  // candidates of the largest client / of the largest one that needs the partition
   __shared__ uint32_t s_tiles[CVLC_MAX_BATCH];  // sort tiles of every client
   const uint32_t n = batch.n;
   pdl_enter();
@@ -45,17 +46,36 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     s_total = 0;
     s_bad = 0;
     s_pass3 = 0;
+    s_lsd = 0;
+    s_most = s_most_split = 0;
   }
+  // the plan's tables must have been made for this very batch: looked at only if the header says so
+  const PlanWsHeader* ph = reinterpret_cast<const PlanWsHeader*>(plan_ws);
+  const bool tables = ph && ph->magic == kPlanWsMagic && ph->n == n && ph->d == shape.d;
   __syncthreads();
   {
     unsigned long long t = 0;
     int pass3 = 0;
+    const uint32_t* max_bin = tables ? reinterpret_cast<const uint32_t*>(plan_ws + plan_off_max_bin(n)) : nullptr;
     for (uint32_t c = threadIdx.x; c < n; c += blockDim.x) {  // the plans are read side by side, not one after the other
       const cvlc_plan_t* plan = batch.c[c].plan;
       const uint32_t tiles = sort_tiles_of(plan->n_candidates, L.capacity);
       s_tiles[c] = tiles;
       t += tiles;
       if (plan->top_bin + 1u - plan->thresh_bin > 256u) pass3 = 1;  // see top_digit_is_zero
+      if (max_bin) {
+        ClientRank r;
+        const uint32_t top = plan->top_bin < CVLC_HIST_BINS ? plan->top_bin : CVLC_HIST_BINS - 1;
+        const uint32_t nb = plan->thresh_bin <= top ? top - plan->thresh_bin + 1 : 1;
+        if (!rank_shape(nb, max_bin[c], plan->thresh_bin, &r)) s_lsd = 1;
+        r.n = (uint32_t)(plan->n_candidates < L.capacity ? plan->n_candidates : L.capacity);
+        r.keytop = sort_keytop(plan);
+        r.top_bin = top;
+        r.pad = 0;
+        atomicMax(&s_most, r.n);
+        if (r.split) atomicMax(&s_most_split, r.n);
+        if (blockIdx.x == 0) reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;
+      }
     }
     if (t) atomicAdd(&s_total, t);
     if (pass3) atomicOr(&s_pass3, 1);
@@ -63,20 +83,22 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
   __syncthreads();
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t gstride = (size_t)gridDim.x * blockDim.x;
-  {
-    unsigned long long* a = reinterpret_cast<unsigned long long*>(ws + L.off_n_selected);
-    for (size_t i = gtid; i < n; i += gstride) a[i] = 0ull;
-    unsigned long long* b = reinterpret_cast<unsigned long long*>(ws + L.off_ghist);
-    const size_t nb = (L.off_row_list - L.off_ghist) / 8;  // digit histograms, their scans, selection tile states
-    for (size_t i = gtid; i < nb; i += gstride) b[i] = 0ull;
-  }
-  // look-back states of the digit passes that will run (the fourth only if some client's keys span more than 2^27)
-  const size_t per_pass = (size_t)s_total * kDigits;
-  const int n_passes = s_pass3 ? kSortPasses : kSortPasses - 1;
-  for (int p = 0; p < n_passes; ++p) {
-    ulonglong2* st = reinterpret_cast<ulonglong2*>(reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) +
-                                                   (size_t)p * n * L.sort_tiles_max * kDigits);
-    for (size_t i = gtid; i < per_pass / 2; i += gstride) st[i] = make_ulonglong2(0ull, 0ull);
+  auto zero = [&](size_t from, size_t to) {  // multiples of 256 bytes
+    ulonglong2* p = reinterpret_cast<ulonglong2*>(ws + from);
+    for (size_t i = gtid; i < (to - from) / 16; i += gstride) p[i] = make_ulonglong2(0ull, 0ull);
+  };
+  if (plan_ws) {
+    zero(L.off_group_next, L.off_sub_start);  // counters of the selection and the partition
+  } else {
+    zero(L.off_ghist, L.off_sort_state);  // digit histograms, their scans, selection tile states
+    // look-back states of the digit passes that will run (the fourth only if some client's keys span more than 2^27)
+    const size_t per_pass = (size_t)s_total * kDigits;
+    const int n_passes = s_pass3 ? kSortPasses : kSortPasses - 1;
+    for (int p = 0; p < n_passes; ++p) {
+      ulonglong2* st = reinterpret_cast<ulonglong2*>(reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) +
+                                                     (size_t)p * n * L.sort_tiles_max * kDigits);
+      for (size_t i = gtid; i < per_pass / 2; i += gstride) st[i] = make_ulonglong2(0ull, 0ull);
+    }
   }
   if (blockIdx.x != 0) return;
 
@@ -108,17 +130,24 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
       if (t > mx) mx = t;
     }
     prefix[n] = run;
-    if (plan_ws && !s_bad) {
-      // the segment tables must have been made for this very batch
-      const PlanWsHeader* ph = reinterpret_cast<const PlanWsHeader*>(plan_ws);
-      if (ph->magic != kPlanWsMagic || ph->n != n || ph->d != shape.d || ph->n_chunks != part.n_chunks) s_bad = CVLC_ERR_PLAN_MISMATCH;
-    }
+    if (plan_ws && !tables && !s_bad) s_bad = CVLC_ERR_PLAN_MISMATCH;
     hdr->max_sort_tiles = mx;
     hdr->status = s_bad;
-    hdr->select_ticket = 0;
-    for (int p = 0; p < kSortPasses; ++p) hdr->sort_ticket[p] = 0;
+    hdr->lsd = !plan_ws ? kRankDigits : s_lsd ? kRankAllDigits : kRankPartition;
+    hdr->select_ticket = hdr->split_ticket = hdr->rank_ticket = hdr->sort_ticket = 0;
+    for (int p = 0; p < 8; ++p) hdr->sort_done[p] = 0;
+    hdr->split_tiles = (s_most_split + kRankSplitTile - 1) / kRankSplitTile;
+    // tiles small enough that the batch gives every SM several
+    const uint64_t want = ((uint64_t)run * kSortTile + 4 * kNumSM - 1) / (4 * kNumSM);
+    uint32_t window = kRankWindow;
+    while (window > 1024 && window / 2 >= want) window >>= 1;
+    hdr->window = window;
+    hdr->rank_tiles = (s_most + window - 1) / window;
     hdr->total_sort_tiles = run;
   }
+  // ranked by partition: the result is in the first buffer (the digit passes write a mask of their own)
+  if (plan_ws)
+    for (uint32_t c = threadIdx.x; c < n; c += blockDim.x) reinterpret_cast<uint32_t*>(ws + L.off_pass_mask)[c] = (1u << kSortPasses) - 1u;
 }
 
 // ===================================================================================
@@ -129,42 +158,32 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
 // Tiles of 8192 coordinates are handed out by an atomic ticket (tile-major, clients interleaved:
 // the tiles in flight at any time are a few consecutive tiles of every client), so every
 // predecessor of a tile is running or done; the look-back reads 512 predecessors per step.
-// Used when the plan's workspace (and with it the per-segment counts) is not available.
+// Used when the plan's workspace is not available and in front of the digit passes.
 
-__global__ void __launch_bounds__(kSelectThreads)
-k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
-  __shared__ uint32_t s_tile;
-  __shared__ unsigned long long s_warp_incl[kSelectThreads / 32];
-  __shared__ unsigned long long s_look_sum[kSelectThreads / 32];
-  __shared__ uint32_t s_look_flag[kSelectThreads / 32];
-  pdl_enter();
+template <int THREADS>
+__device__ __forceinline__ void select_lookback_tile(const Batch& batch, uint64_t d, unsigned char* ws, const EncLayout& L, uint64_t gt) {
+  __shared__ unsigned long long s_warp_incl[THREADS / 32];
+  __shared__ unsigned long long s_look_sum[THREADS / 32];
+  __shared__ uint32_t s_look_flag[THREADS / 32];
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t tiles_per_client = L.select_tiles;
-  const uint64_t total_tiles = tiles_per_client * batch.n;
-  unsigned long long* n_selected = reinterpret_cast<unsigned long long*>(ws + L.off_n_selected);
-
-  while (true) {
-    if (tid == 0) s_tile = atomicAdd(&hdr->select_ticket, 1u);
-    __syncthreads();
-    const uint64_t gt = s_tile;
-    if (gt >= total_tiles) break;
+  const uint64_t tiles_per_client = select_tiles_of(d, THREADS);
+  {
     const uint64_t tile = gt / batch.n;
     const uint32_t c = (uint32_t)(gt - tile * batch.n);
     const float* __restrict__ x = batch.c[c].x;
     const cvlc_plan_t* __restrict__ plan = batch.c[c].plan;
     const float4* xv = reinterpret_cast<const float4*>(x);
     const uint32_t thresh = plan->thresh_bin << 19;
-    unsigned long long* tile_state = reinterpret_cast<unsigned long long*>(ws + L.off_select_state) + (size_t)c * tiles_per_client;
+    unsigned long long* tile_state = reinterpret_cast<unsigned long long*>(ws + L.off_select_state) + (size_t)c * L.select_tiles;
     unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
-    const uint64_t base_vec = tile * (uint64_t)(kSelectThreads * kSelectVecPerThread);
+    const uint64_t base_vec = tile * (uint64_t)(THREADS * kSelectVecPerThread);
 
     uint32_t bits[kSelectVecPerThread][4];
     uint32_t mask[kSelectVecPerThread];
 #pragma unroll
     for (int v = 0; v < kSelectVecPerThread; ++v) {
-      const uint64_t vi = base_vec + (uint64_t)v * kSelectThreads + tid;
+      const uint64_t vi = base_vec + (uint64_t)v * THREADS + tid;
       const uint64_t e0 = vi * 4;
       uint32_t valid = 0;
       if (e0 + 3 < d) {
@@ -203,7 +222,7 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
     __syncthreads();
     unsigned long long below = 0, tot = 0;
 #pragma unroll
-    for (int w = 0; w < kSelectThreads / 32; ++w) {
+    for (int w = 0; w < THREADS / 32; ++w) {
       const unsigned long long t = s_warp_incl[w];
       if (w < warp) below += t;
       tot += t;
@@ -238,7 +257,7 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
         bool found = false;
         unsigned long long add = 0;
 #pragma unroll
-        for (int w = 0; w < kSelectThreads / 32; ++w) {
+        for (int w = 0; w < THREADS / 32; ++w) {
           if (!found) {
             add += s_look_sum[w];
             found = s_look_flag[w] != 0;
@@ -247,19 +266,18 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
         run += add;
         __syncthreads();
         if (any_to || found) break;  // after a timeout the status is set and the results are void
-        base -= kSelectThreads;
+        base -= THREADS;
       }
       if (tid == 0) st_relaxed(tile_state + tile, kFlagPrefix | (run + tile_total));
     }
     if (tid == 0 && tile == tiles_per_client - 1) {
-      n_selected[c] = run + tile_total;
       if (run + tile_total != plan->n_candidates) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
     }
     unsigned long long vec_base = 0;
 #pragma unroll
     for (int v = 0; v < kSelectVecPerThread; ++v) {
       unsigned long long o = run + vec_base + ((excl >> (16 * v)) & 0xFFFF);
-      const uint64_t e0 = (base_vec + (uint64_t)v * kSelectThreads + tid) * 4;
+      const uint64_t e0 = (base_vec + (uint64_t)v * THREADS + tid) * 4;
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
         if (mask[v] & (1u << cc)) {
@@ -272,34 +290,347 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
       }
       vec_base += (tot >> (16 * v)) & 0xFFFF;
     }
-    __syncthreads();  // s_tile and the look-back scratch are reused by the next tile
+    __syncthreads();  // the look-back scratch is reused by the next tile
+  }
+}
+
+__global__ void __launch_bounds__(kSelectThreads)
+k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
+  __shared__ uint32_t s_tile;
+  pdl_enter();
+  EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
+  if (block_sees_error(&hdr->status)) return;
+  const uint64_t total_tiles = select_tiles_of(d, kSelectThreads) * batch.n;
+  while (true) {
+    if (threadIdx.x == 0) s_tile = atomicAdd(&hdr->select_ticket, 1u);
+    __syncthreads();
+    const uint64_t gt = s_tile;
+    if (gt >= total_tiles) break;
+    __syncthreads();  // everyone has read the ticket
+    select_lookback_tile<kSelectThreads>(batch, d, ws, L, gt);
   }
 }
 
 // ===================================================================================
-// K3' threshold selection with offsets known in advance (no exchange between blocks)
+// K3' threshold selection into the buckets of the ranking (no order inside a bucket)
 // ===================================================================================
-// Same chunking of the concatenated updates as the histogram kernel: block b streams its chunk
-// once with 128-bit loads, one tile (8192 coordinates) ahead of the compaction.  The number of
-// candidates in every earlier segment of the client is known from the per-segment histograms
-// (seg_prefix, written by the planner), so the output position of a candidate is
-// seg_prefix + its rank inside the block's segment: a block-level scan per tile and nothing else.
+// Groups of rows, every client with a counter of its own; a block keeps to one client while that has groups left, so that its
+// counts of the client's sub-buckets go out once.  Its warps work on their own: they take groups (the first one without asking)
+// and read the rows that hold a candidate (the histogram pass left the rows' maxima), eight at a time with the next eight on
+// their way in registers.  A step goes through shared memory so that every lane gets 16 consecutive coordinates: their flags are
+// then one word, and a lane's loop runs over its candidates only, which it appends to the warp's buffer.  When that is full the
+// warp counts its candidates per coarse bucket, reserves room in every bucket with one global addition and puts the candidates
+// there; they are also counted per sub-bucket where the client needs the partition.  The block that completes a client turns
+// those counts into offsets.  (One buffer per block, emptied by all its warps together, left them waiting for one another: 860 us
+// instead of SELECT_FIGURES.)
 
-constexpr int kSelStages = 3;  // tiles in flight per block (cp.async groups)
-constexpr size_t kSelStageBytes = (size_t)kSelectThreads * kSelectVecPerThread * 16;  // 32 KB
+constexpr uint32_t kSelBuffer = 512;    // candidates in a warp's buffer: all of a step at least
+constexpr int kSelVec = 4;              // 128-bit loads per lane and step: eight rows
+constexpr uint32_t kSelRows = 2 * kSelVec;
+constexpr uint32_t kSelQueue = 64;      // rows a warp has found (ring)
+struct SelWarp {
+  unsigned long long items[kSelBuffer];
+  float4 stage[kSelVec * 32];
+  uint32_t cnt[kRankCoarse];            // counts, then next places (zero between)
+  uint32_t queue[kSelQueue];
+};
+constexpr size_t kSelSmem = (kSelThreads / 32) * sizeof(SelWarp) + ((size_t)kRankCoarse + kRankSubs) * 4;
+static_assert(kRowUnits == 16 && kSelRows - 1 + 32 <= kSelQueue, "two rows per warp-wide load; the ring holds a group and a rest");
+static_assert(kSelVec * 128 <= kSelBuffer && kSelSmem <= 227 * 1024, "shared memory");
 
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gmem_src) : "memory");
+// red.add of four fp32 counts at once: counts stay below 2^24 in this mode (see rank_shape), where they are exact
+__device__ __forceinline__ void add_counts4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t e) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"((float)a), "f"((float)b), "f"((float)c), "f"((float)e) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+
+__global__ void __launch_bounds__(kSelThreads, 1)
+k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, const unsigned char* __restrict__ plan_ws, unsigned char* ws,
+         const __grid_constant__ EncLayout L) {
+  extern __shared__ __align__(16) unsigned char s_sel[];
+  SelWarp& sw = reinterpret_cast<SelWarp*>(s_sel)[threadIdx.x >> 5];
+  uint32_t* s_start = reinterpret_cast<uint32_t*>(s_sel + (kSelThreads / 32) * sizeof(SelWarp));  // [kRankCoarse] starts of the client's buckets
+  uint32_t* s_sub = s_start + kRankCoarse;                                                        // [kRankSubs] candidates per sub-bucket
+  __shared__ uint32_t s_client, s_taken, s_scan[kSelThreads / 32];
+  pdl_enter();
+  EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
+  if (block_sees_error(&hdr->status)) return;
+  if (hdr->lsd != kRankPartition) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n = batch.n;
+  const uint32_t rows = (uint32_t)part.rows, group_rows = select_group_rows(part), groups = (rows + group_rows - 1) / group_rows;
+  const uint32_t nvec = (uint32_t)(d >> 2);
+  uint32_t* group_next = reinterpret_cast<uint32_t*>(ws + L.off_group_next);
+  uint32_t* group_done = reinterpret_cast<uint32_t*>(ws + L.off_group_done);
+  for (uint32_t i = tid; i < kRankSubs; i += kSelThreads) s_sub[i] = 0;
+  for (uint32_t i = lane; i < kRankCoarse; i += 32) sw.cnt[i] = 0;
+  if (tid == 0) s_taken = 0;
+  // Block b starts with client b n / grid; the first groups of a client go to the warps of the blocks that start with it, the rest
+  // by its counter.
+  const uint32_t home = (uint32_t)(((uint64_t)blockIdx.x * n) / gridDim.x);
+  auto first_block = [&](uint32_t c) -> uint32_t { return (uint32_t)(((uint64_t)c * gridDim.x + n - 1) / n); };
+  auto given = [&](uint32_t c) -> uint32_t { return (first_block(c + 1) - first_block(c)) * (kSelThreads / 32); };
+
+  // the first client from `from` on that has groups left (n: none), found by all threads together
+  auto find_client = [&](uint32_t from) -> uint32_t {
+    if (tid == 0) s_client = 0xFFFFFFFFu;
+    __syncthreads();
+    for (uint32_t i = tid; i < n; i += kSelThreads) {
+      const uint32_t c = from + i < n ? from + i : from + i - n;
+      if (__ldcg(group_next + c) + given(c) < groups) {
+        atomicMin(&s_client, i);
+        break;
+      }
+    }
+    __syncthreads();
+    const uint32_t i = s_client;
+    __syncthreads();
+    return i == 0xFFFFFFFFu ? n : (from + i < n ? from + i : from + i - n);
+  };
+
+  for (uint32_t c = home, visit = 0;; ++visit) {
+    if (visit) c = find_client(c);
+    if (c >= n) return;
+    const ClientRank r = reinterpret_cast<const ClientRank*>(ws + L.off_rank)[c];
+    const float* __restrict__ x = batch.c[c].x;
+    const float4* __restrict__ xv = reinterpret_cast<const float4*>(x);
+    const uint32_t* __restrict__ row_max = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_row_max(n)) + (size_t)c * rows;
+    const uint32_t thresh = batch.c[c].plan->thresh_bin << 19, keytop = r.keytop;  // thresh > 0 in this mode
+    const float below_thresh = __uint_as_float(thresh - 1u);                        // key >= thresh <=> |x| > below_thresh
+    const uint32_t sh_coarse = 19 + r.group, sh_sub = sh_coarse - r.sub_bits;
+    unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
+    uint32_t* fill = reinterpret_cast<uint32_t*>(ws + L.off_bin_fill) + (size_t)c * kRankCoarse;
+    {
+      const uint32_t* __restrict__ bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS;
+      for (uint32_t i = tid; i < r.n_coarse; i += kSelThreads) s_start[i] = coarse_start(r, bin_start, i);
+    }
+    const uint32_t inv_max = keytop - thresh;
+    auto inv_of = [&](uint32_t key) -> uint32_t {  // always inside the client's buckets
+      const uint32_t inv = keytop - (key < keytop ? key : keytop);
+      return inv < inv_max ? inv : inv_max;
+    };
+    uint32_t held = 0;  // candidates in the warp's buffer
+    auto flush = [&]() {  // to their buckets
+      for (uint32_t i = lane; i < held; i += 32) {
+        const uint32_t key = (uint32_t)(sw.items[i] >> 32);
+        if (key > keytop) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);  // the update is not the plan's
+        const uint32_t inv = inv_of(key);
+        atomicAdd(sw.cnt + (inv >> sh_coarse), 1u);
+        if (r.split) atomicAdd(s_sub + (inv >> sh_sub), 1u);
+      }
+      __syncwarp();
+      for (uint32_t i0 = lane; i0 < r.n_coarse; i0 += 128) {
+        uint32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = (i0 + 32 * u < r.n_coarse) ? sw.cnt[i0 + 32 * u] : 0u;
+        uint32_t at[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) at[u] = v[u] ? atomicAdd(fill + i0 + 32 * u, v[u]) : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v[u]) sw.cnt[i0 + 32 * u] = s_start[i0 + 32 * u] + at[u];
+      }
+      __syncwarp();
+      for (uint32_t i = lane; i < held; i += 32) {
+        const unsigned long long item = sw.items[i];
+        const uint32_t p = atomicAdd(sw.cnt + (inv_of((uint32_t)(item >> 32)) >> sh_coarse), 1u);
+        if (p < r.n) out[p] = item;
+      }
+      __syncwarp();
+      for (uint32_t i = lane; i < r.n_coarse; i += 32) sw.cnt[i] = 0;
+      held = 0;
+      __syncwarp();
+    };
+
+    __syncthreads();  // the buckets' starts are there
+    // ---- the warp's groups: the maxima of the next one are on their way, and so is the number of the one after it
+    uint32_t taken = 0, group = 0, group2 = 0, maximum = 0, piece = 0;  // piece: 32 rows of the group
+    const uint32_t pieces = group_rows > 32 ? group_rows / 32 : 1;
+    const uint32_t dynamic = given(c);  // first group that goes by the counter
+    if (visit == 0) {
+      group = (blockIdx.x - first_block(c)) * (kSelThreads / 32) + warp;
+    } else {
+      if (lane == 0) group = dynamic + atomicAdd(group_next + c, 1u);
+      group = __shfl_sync(kFull, group, 0);
+    }
+    if (lane == 0) group2 = dynamic + atomicAdd(group_next + c, 1u);
+    auto maxima_of = [&](uint32_t g, uint32_t p) -> uint32_t {
+      const uint32_t row = g * group_rows + p * 32 + lane;
+      return (g < groups && (uint32_t)lane < group_rows && row < rows) ? __ldg(row_max + row) : 0u;
+    };
+    maximum = maxima_of(group, 0);
+    uint32_t* queue = sw.queue;
+    uint32_t head = 0, tail = 0;
+    float4 nf[kSelVec];
+    uint32_t next_row = 0;  // the row in which this lane's coordinates of the next step lie
+    static_assert(kSelVec == 4, "a lane's 16 coordinates are a quarter of a row");
+    auto request = [&]() -> uint32_t {  // asks for the next rows that hold a candidate; returns how many there are
+      while (tail - head < kSelRows && group < groups) {
+        const uint32_t row = group * group_rows + piece * 32 + lane, mx = maximum;
+        if (group + 1 == groups && piece == 0 && lane < (int)(d & 3)) {  // the client's ragged tail goes with its last group: straight to its buckets
+          const uint32_t b = __float_as_uint(x[(uint64_t)nvec * 4 + lane]), key = b & 0x7FFFFFFFu;
+          if (key >= thresh) {
+            if (key > keytop) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
+            const uint32_t inv = inv_of(key);
+            const uint32_t p = s_start[inv >> sh_coarse] + atomicAdd(fill + (inv >> sh_coarse), 1u);
+            if (r.split) atomicAdd(s_sub + (inv >> sh_sub), 1u);
+            if (p < r.n) out[p] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | (nvec * 4 + (uint32_t)lane));
+          }
+        }
+        if (++piece == pieces) {
+          ++taken;
+          piece = 0;
+          group = __shfl_sync(kFull, group2, 0);
+          if (lane == 0 && group < groups) group2 = dynamic + atomicAdd(group_next + c, 1u);
+        }
+        maximum = maxima_of(group, piece);
+        const unsigned m = __ballot_sync(kFull, mx >= thresh);  // mx = 0 past the last row
+        if (mx >= thresh) queue[(tail + __popc(m & ((1u << lane) - 1u))) & (kSelQueue - 1)] = row;
+        tail += __popc(m);
+        __syncwarp();
+      }
+      const uint32_t have = tail - head < kSelRows ? tail - head : kSelRows;
+#pragma unroll
+      for (int v = 0; v < kSelVec; ++v) {
+        const uint32_t slot = 2 * v + (lane >> 4);
+        const uint32_t unit = queue[(head + slot) & (kSelQueue - 1)] * kRowUnits + (lane & 15);
+        nf[v] = make_float4(0.f, 0.f, 0.f, 0.f);  // no candidate
+        if (slot < have && unit < nvec) nf[v] = __ldg(xv + unit);
+      }
+      next_row = queue[(head + (lane >> 2)) & (kSelQueue - 1)];
+      head += have;
+      __syncwarp();
+      return have;
+    };
+    // Staging layout: float4 g of a step (in memory order) sits in slot g ^ ((g >> 3) & 3): the stores of a warp (consecutive g) and
+    // its loads (lane l reads 4 l .. 4 l + 3) are then both free of bank conflicts.
+    float4* stage = sw.stage;
+    const uint32_t ct = ((uint32_t)lane >> 1) & 3u;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(stage) + 16 * lane;
+    uint32_t pending = request();
+    uint32_t m = 0, first = 0;  // flags of this lane's coordinates, lowest index in bit 15; index of the first one
+    auto advance = [&]() -> bool {
+      if (pending == 0) return false;
+      __syncwarp();  // the step before has been read
+#pragma unroll
+      for (int v = 0; v < kSelVec; ++v) {
+        const uint32_t g = (uint32_t)(v * 32 + lane);
+        stage[g ^ ((g >> 3) & 3u)] = nf[v];
+      }
+      first = next_row * (4 * kRowUnits) + (lane & 3) * 16;
+      pending = request();
+      __syncwarp();
+      m = 0;
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) {  // the difference of two distinct floats never rounds to zero: its sign is the flag
+        const float4 f = stage[4 * lane + (j ^ ct)];
+        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.x))), m, 1);
+        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.y))), m, 1);
+        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.z))), m, 1);
+        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.w))), m, 1);
+      }
+      return true;
+    };
+    while (advance()) {
+      const uint32_t cnt = __popc(m);
+      uint32_t incl = cnt;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_up_sync(kFull, incl, off);
+        if (lane >= off) incl += o;
+      }
+      const uint32_t total = __shfl_sync(kFull, incl, 31);
+      if (held + total > kSelBuffer) flush();
+      unsigned long long* o = sw.items + held + incl - cnt;
+      while (m) {
+        const int hb = 31 - __clz(m);  // highest flag = lowest index first
+        m ^= 1u << hb;
+        const uint32_t c16 = 15u - (uint32_t)hb;
+        const uint32_t b = words[c16 ^ (ct << 2)];
+        *o++ = ((unsigned long long)(b & 0x7FFFFFFFu) << 32) | (unsigned long long)((b & 0x80000000u) | (first + c16));
+      }
+      held += total;
+    }
+    __syncwarp();
+    if (held) flush();
+    if (lane == 0 && taken) atomicAdd(&s_taken, taken);
+    __syncthreads();
+    const uint32_t block_taken = s_taken;
+    __syncthreads();
+    if (block_taken == 0) continue;
+    if (tid == 0) s_taken = 0;
+    if (r.split) {
+      float* count = reinterpret_cast<float*>(ws + L.off_sub_count) + (size_t)c * kRankSubs;
+      const uint32_t n_sub4 = ((r.n_coarse << r.sub_bits) + 3) / 4;
+      uint4* sub4 = reinterpret_cast<uint4*>(s_sub);
+      for (uint32_t i = tid; i < n_sub4; i += kSelThreads) {
+        const uint4 v = sub4[i];
+        if (v.x | v.y | v.z | v.w) {
+          add_counts4(count + 4 * i, v.x, v.y, v.z, v.w);
+          sub4[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_client = atomicAdd(group_done + c, block_taken) + block_taken;
+    __syncthreads();
+    if (s_client == groups) {
+      __threadfence();
+      // the update must be the one the plan was made from
+      for (uint32_t i = tid; i < r.n_coarse; i += kSelThreads) {
+        const uint32_t end = i + 1 < r.n_coarse ? s_start[i + 1] : r.n;
+        if (__ldcg(fill + i) != end - s_start[i]) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
+      }
+      if (r.split) {
+        const uint32_t n_sub = r.n_coarse << r.sub_bits;
+        const float* count = reinterpret_cast<const float*>(ws + L.off_sub_count) + (size_t)c * kRankSubs;
+        uint32_t* start = reinterpret_cast<uint32_t*>(ws + L.off_sub_start) + (size_t)c * (kRankSubs + 64);
+        uint32_t* next = reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs;
+        constexpr uint32_t kMine = 8;
+        uint32_t carry = 0, largest = 0;
+        for (uint32_t base = 0; base < n_sub; base += kSelThreads * kMine) {
+          const uint32_t i0 = base + (uint32_t)tid * kMine;
+          uint32_t v[kMine], sum = 0;
+#pragma unroll
+          for (uint32_t e = 0; e < kMine; ++e) v[e] = (i0 + e < n_sub) ? (uint32_t)__ldcg(count + i0 + e) : 0u;
+#pragma unroll
+          for (uint32_t e = 0; e < kMine; ++e) {
+            sum += v[e];
+            largest = v[e] > largest ? v[e] : largest;
+          }
+          uint32_t incl = sum;
+#pragma unroll
+          for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t o = __shfl_up_sync(kFull, incl, off);
+            if (lane >= off) incl += o;
+          }
+          if (lane == 31) s_scan[warp] = incl;
+          __syncthreads();
+          uint32_t run = carry + incl - sum, all = 0;
+          for (int w = 0; w < kSelThreads / 32; ++w) {
+            const uint32_t t = s_scan[w];
+            if (w < warp) run += t;
+            all += t;
+          }
+#pragma unroll
+          for (uint32_t e = 0; e < kMine; ++e) {
+            if (i0 + e < n_sub) {
+              start[i0 + e] = run;
+              next[i0 + e] = run;
+            }
+            run += v[e];
+          }
+          carry += all;
+          __syncthreads();
+        }
+        if (tid == 0) start[n_sub] = carry;
+        if (largest > kRankLargest) hdr->lsd = kRankAllDigits;
+      }
+    }
+    __syncthreads();
+  }
 }
 
-// sort key digits (see the ranking kernels below); the selection kernel already counts them
-__device__ __forceinline__ uint32_t sort_keytop(const cvlc_plan_t* plan) { return ((plan->top_bin + 1u) << 19) - 1u; }
 // With at most 256 histogram bins between the threshold and the top, keytop - key stays below 2^27 for every
 // candidate: the fourth digit is zero throughout and neither counted nor ranked.
 __device__ __forceinline__ bool top_digit_is_zero(const cvlc_plan_t* plan) { return plan->top_bin + 1u - plan->thresh_bin <= 256u; }
@@ -310,359 +641,19 @@ __device__ __forceinline__ uint32_t sort_digit(unsigned long long pair, int pass
   return (inv >> (kDigitBits * pass)) & (kDigits - 1);
 }
 
-// Staging layout: float4 unit g of a tile (g = 0 .. 2047, in memory order) sits in slot
-// g ^ ((g >> 3) & 3).  The copies of a warp (consecutive g) and the reads of a warp (thread t
-// reads its own four consecutive units 4t .. 4t+3) are then both free of bank conflicts.
-constexpr int kSelThreads = 512;                      // threads of the selection kernel
-constexpr int kSelVec = 4;                            // float4 units (16 coordinates) per thread and tile
-constexpr uint32_t kSelTileVec = kSelThreads * kSelVec;  // 2048 float4 = 8192 coordinates = 32 KB
-static_assert(kSelTileVec * 16 == kSelStageBytes, "stage size");
-__device__ __forceinline__ uint32_t sel_slot(uint32_t g) { return g ^ ((g >> 3) & (uint32_t)(kSelVec - 1)); }
-
-__global__ void __launch_bounds__(kSelThreads, 2)
-k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
-         const unsigned char* __restrict__ plan_ws, unsigned char* ws, const __grid_constant__ EncLayout L) {
-  extern __shared__ float4 s_stage[];  // [kSelStages][2048 float4]
-  __shared__ uint32_t s_warp_incl[2][kSelThreads / 32];
-  __shared__ uint32_t s_dhist[kSortPasses * kDigits];  // digit histograms of the segment's candidates (for the ranking passes)
-  for (int i = threadIdx.x; i < kSortPasses * kDigits; i += kSelThreads) s_dhist[i] = 0;
-  pdl_enter();
-  EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t S = part.max_segments;
-  const uint32_t* seg_count = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_seg_count(batch.n));
-  const unsigned long long* seg_prefix = reinterpret_cast<const unsigned long long*>(plan_ws + plan_off_seg_prefix(batch.n, S));
-  const uint32_t* row_max = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_row_max(batch.n, S));
-  uint32_t* row_list = reinterpret_cast<uint32_t*>(ws + L.off_row_list);
-  unsigned long long* n_selected = reinterpret_cast<unsigned long long*>(ws + L.off_n_selected);
-  const uint64_t nvec = d >> 2;
-  const uint64_t units = part.units;
-  constexpr uint32_t kTileVec = kSelTileVec;
-  static_assert(kSelTileVec == kTileUnits && kSelVec == 4 && kRowUnits % kSelVec == 0 && 32 % kRowUnits == 0,
-                "a warp stages whole rows of a tile, a thread's four units lie in one row");
-  int parity = 0;
-  __shared__ uint32_t s_chunk;
-
-  while (true) {
-  // chunks by ticket: a chunk full of candidates costs several times one without
-  if (tid == 0) s_chunk = atomicAdd(&hdr->select_ticket, 1u);
-  __syncthreads();
-  const uint32_t q = s_chunk;
-  if (q >= part.n_chunks) break;
-  uint64_t pos = (uint64_t)q * part.chunk;
-  const uint64_t end = (pos + part.chunk < part.total) ? pos + part.chunk : part.total;
-
-  while (pos < end) {
-    const uint32_t c = (uint32_t)(pos / units);
-    const uint64_t seg_end = ((c + 1) * units < end) ? (c + 1) * units : end;
-    const uint64_t u0 = pos - c * units, u1 = seg_end - c * units;  // units [u0, u1) of client c
-    const bool with_tail = (u1 == units);                            // the segment ends with the client's tail unit
-    const uint64_t v_end = with_tail ? nvec : u1;                    // float4 units [u0, v_end)
-    const float* __restrict__ x = batch.c[c].x;
-    const float4* __restrict__ xseg = reinterpret_cast<const float4*>(x) + u0;
-    const cvlc_plan_t* __restrict__ plan = batch.c[c].plan;
-    const uint32_t thresh = plan->thresh_bin << 19;
-    // finite inputs: key >= thresh <=> |x| > the float just below thresh <=> (that float) - |x| is negative.  The
-    // difference of two distinct floats never rounds to zero, so its sign bit is the candidate flag: one
-    // subtraction and one funnel shift per coordinate.  thresh == 0: every coordinate is a candidate.
-    const float below_thresh_f = __uint_as_float(thresh ? thresh - 1u : 0u);
-    const uint32_t cap32 = (uint32_t)L.capacity;  // <= d <= 2^31
-    const uint32_t keytop = sort_keytop(plan);
-    const bool count_top = !top_digit_is_zero(plan);
-    const uint32_t seg = q + c;
-    unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
-    unsigned long long run = seg_prefix[seg];
-    const unsigned long long run0 = run;
-    const uint64_t n_vec = (v_end > u0) ? v_end - u0 : 0;        // float4 units of the segment
-    // The segment's rows with candidates, a tile (kTileRows of them) at a time: tile t of the staging buffers holds the
-    // rows kTileRows t .. of the list, warp w the next kRowsPerWarp of them (ascending rows in ascending lanes: index
-    // order is kept).
-    constexpr uint32_t kRowsPerWarp = 32 * kSelVec / kRowUnits;
-    const uint32_t n_vec32 = (uint32_t)n_vec;  // a segment is at most one chunk: far below 2^32 units
-    uint32_t* list = row_list + seg_first_tile(pos, seg) * kTileRows;
-    // ---- the rows that hold a candidate, in ascending order.  Every thread looks at 16 consecutive rows at a time (four
-    // 128-bit loads in flight), one block scan gives their places: a chunk's rows are usually one such step, about 3 us of
-    // the 90 us a chunk takes.  On 10 clients of 1e8 coordinates the list adds 20 us to this kernel; one planner block
-    // per client listing the rows took 215 us more than the planner takes without it.
-    uint32_t n_listed = 0;
-    {
-      constexpr uint32_t kRowsPerThread = 16;
-      const uint32_t n_rows = (n_vec32 + kRowUnits - 1) / kRowUnits;
-      const uint4* __restrict__ rm = reinterpret_cast<const uint4*>(row_max + seg_first_tile(pos, seg) * kTileRows);
-      for (uint32_t r0 = 0; r0 < n_rows; r0 += kSelThreads * kRowsPerThread) {
-        const uint32_t mine = r0 + (uint32_t)tid * kRowsPerThread;
-        uint4 q4[kRowsPerThread / 4];
-#pragma unroll
-        for (uint32_t v = 0; v < kRowsPerThread / 4; ++v) q4[v] = (mine + 4 * v < n_rows) ? __ldg(rm + mine / 4 + v) : make_uint4(0u, 0u, 0u, 0u);
-        uint32_t m = 0;
-#pragma unroll
-        for (uint32_t v = 0; v < kRowsPerThread / 4; ++v)
-          m |= ((q4[v].x >= thresh ? 1u : 0u) | (q4[v].y >= thresh ? 2u : 0u) | (q4[v].z >= thresh ? 4u : 0u) | (q4[v].w >= thresh ? 8u : 0u)) << (4 * v);
-        const uint32_t left = (mine < n_rows) ? n_rows - mine : 0u;
-        if (left < kRowsPerThread) m &= (1u << left) - 1u;
-        const uint32_t cnt = __popc(m);
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const uint32_t o = __shfl_up_sync(kFull, incl, off);
-          if (lane >= off) incl += o;
-        }
-        if (lane == 31) s_warp_incl[parity][warp] = incl;
-        __syncthreads();
-        const uint32_t wt = (lane < kSelThreads / 32) ? s_warp_incl[parity][lane] : 0u;
-        uint32_t wincl = wt;
-#pragma unroll
-        for (int off = 1; off < kSelThreads / 32; off <<= 1) {
-          const uint32_t o = __shfl_up_sync(kFull, wincl, off);
-          if (lane >= off) wincl += o;
-        }
-        const uint32_t tot = __shfl_sync(kFull, wincl, kSelThreads / 32 - 1);
-        uint32_t o = n_listed + __shfl_sync(kFull, wincl - wt, warp) + incl - cnt;
-        parity ^= 1;
-        while (m) {
-          const uint32_t b = (uint32_t)__ffs(m) - 1u;
-          m &= m - 1u;
-          list[o++] = mine + b;
-        }
-        n_listed += tot;
-      }
-      __syncthreads();  // the list is complete
-    }
-    const uint32_t n_tiles = (n_listed + kTileRows - 1) / kTileRows;
-    constexpr uint32_t kNoRow = 0xFFFFFFFFu;
-    auto row_at = [&](uint32_t t, uint32_t slot) -> uint32_t {  // the row in slot `slot` of this warp's part of tile t
-      const uint32_t idx = t * (uint32_t)kTileRows + (uint32_t)warp * kRowsPerWarp + slot;
-      return (idx < n_listed) ? list[idx] : kNoRow;  // written by this block: not for the read-only path
-    };
-
-    // A warp stages exactly the 128 units (512 coordinates) its own lanes will read: four copies of 32 float4s each,
-    // 32 / kRowUnits rows per copy.  Waiting for a tile and reusing a staging slot are then a matter between the lanes of one
-    // warp, and the block meets only once per tile, for the scan.
-    struct CopyRows { uint32_t r[kSelVec]; };
-    auto copy_rows_of = [&](uint32_t t) -> CopyRows {  // the rows this lane copies from in tile t, one per copy
-      CopyRows cr;
-#pragma unroll
-      for (int v = 0; v < kSelVec; ++v) cr.r[v] = row_at(t, ((uint32_t)v * 32u + (uint32_t)lane) / kRowUnits);
-      return cr;
-    };
-    uint32_t istage = 0;
-    auto issue = [&](const CopyRows& cr) {
-      float4* dst = s_stage + (size_t)istage * kTileVec;
-#pragma unroll
-      for (int v = 0; v < kSelVec; ++v) {
-        const uint32_t g = (uint32_t)(warp * (32 * kSelVec) + v * 32 + lane);
-        const uint32_t unit = cr.r[v] * (uint32_t)kRowUnits + (uint32_t)lane % kRowUnits;
-        if (cr.r[v] != kNoRow && unit < n_vec32) cp_async16(dst + sel_slot(g), xseg + unit);
-      }
-      istage = (istage + 1 == kSelStages) ? 0u : istage + 1;
-      cp_async_commit();  // one group per tile slot, empty past the end, keeps the group count uniform
-    };
-
-    static_assert(kSelStages == 3, "row indices are carried two tiles (copies) and one tile (own row) ahead");
-    issue(copy_rows_of(0));
-    issue(copy_rows_of(1));
-    CopyRows ahead = copy_rows_of(2);                 // for the copies of tile t + 2
-    const uint32_t my_slot = (uint32_t)lane * kSelVec / kRowUnits;  // the slot of the row this thread's four units lie in
-    uint32_t mine = row_at(0, my_slot);                              // the row this thread reads in tile t
-    uint32_t mine_next = row_at(1, my_slot);
-    uint32_t stage = 0;
-    for (uint32_t t = 0; t < n_tiles; ++t) {
-      const CopyRows ahead2 = copy_rows_of(t + 3);    // asked for one tile before they are needed
-      const uint32_t mine_next2 = row_at(t + 2, my_slot);
-      cp_async_wait<kSelStages - 2>();  // this lane's copies of tile t have landed
-      __syncwarp();                     // ... and the other lanes'; and the warp is done with its part of tile t - 1,
-      issue(ahead);                     // whose staging slot the next copies overwrite
-      ahead = ahead2;
-      const uint32_t my_row = mine;
-      mine = mine_next;
-      mine_next = mine_next2;
-      const float4* src = s_stage + (size_t)stage * kTileVec;
-      stage = (stage + 1 == kSelStages) ? 0u : stage + 1;
-      // this thread's 16 consecutive coordinates: four units of the row that it reads with its neighbours
-      uint32_t m = 0;
-      const uint32_t g0 = (uint32_t)kSelVec * tid;
-      const uint32_t ct = ((uint32_t)tid >> 1) & (uint32_t)(kSelVec - 1);
-      const uint32_t unit0 = my_row * (uint32_t)kRowUnits + ((uint32_t)lane * kSelVec) % kRowUnits;  // first unit of the thread, in the segment
-      const uint32_t left = (my_row != kNoRow && unit0 < n_vec32) ? ((n_vec32 - unit0 < (uint32_t)kSelVec) ? n_vec32 - unit0 : (uint32_t)kSelVec) : 0u;
-#pragma unroll
-      for (int j = 0; j < kSelVec; ++j) {
-        if ((uint32_t)j < left) {
-          // units 4 tid + j sit in slots 4 tid + (j ^ ct): the swizzle only touches the two low bits
-          const float4 f = src[g0 + ((uint32_t)j ^ ct)];
-          m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh_f, fabsf(f.x))), m, 1);
-          m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh_f, fabsf(f.y))), m, 1);
-          m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh_f, fabsf(f.z))), m, 1);
-          m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh_f, fabsf(f.w))), m, 1);
-        } else {
-          m <<= 4;
-        }
-      }
-      if (thresh == 0u) m = (left >= (uint32_t)kSelVec) ? 0xFFFFu : (0xFFFFu << (4 * (kSelVec - left))) & 0xFFFFu;
-      // coordinate c of the thread (0 .. 15, ascending index) is bit 15 - c of m
-      const uint32_t cnt = __popc(m);
-      // block scan of the per-thread counts: inside the warp, then over the warp totals
-      uint32_t incl = cnt;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t o = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += o;
-      }
-      if (lane == 31) s_warp_incl[parity][warp] = incl;
-      __syncthreads();
-      const uint32_t wt = (lane < kSelThreads / 32) ? s_warp_incl[parity][lane] : 0u;
-      uint32_t wincl = wt;
-#pragma unroll
-      for (int off = 1; off < kSelThreads / 32; off <<= 1) {
-        const uint32_t o = __shfl_up_sync(kFull, wincl, off);
-        if (lane >= off) wincl += o;
-      }
-      const uint32_t tot = __shfl_sync(kFull, wincl, kSelThreads / 32 - 1);
-      const uint32_t below = __shfl_sync(kFull, wincl - wt, warp);
-      parity ^= 1;
-      // emit this thread's candidates (few): values are re-read from the staging buffer
-      uint32_t o = (uint32_t)run + below + incl - cnt;  // positions inside a client's buffer fit 32 bits
-      const uint32_t* srcw16 = reinterpret_cast<const uint32_t*>(src) + 16 * tid;  // this thread's 16 staged words
-      const uint32_t cx = ct << 2;
-      const uint32_t e32 = (uint32_t)((u0 + unit0) * 4);  // index of the thread's first coordinate (< 2^31)
-      while (m) {
-        const int hb = 31 - __clz(m);  // highest flag = lowest index first
-        m ^= 1u << hb;
-        const uint32_t c16 = 15u - (uint32_t)hb;
-        const uint32_t b = srcw16[c16 ^ cx];
-        const uint32_t key = b & 0x7FFFFFFFu;
-        if (o < cap32) out[o] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | (e32 + c16));
-        const uint32_t inv = keytop - (key < keytop ? key : keytop);
-#pragma unroll
-        for (int p = 0; p < kSortPasses - 1; ++p) atomicAdd(&s_dhist[p * kDigits + ((inv >> (kDigitBits * p)) & (kDigits - 1))], 1u);
-        if (count_top) atomicAdd(&s_dhist[(kSortPasses - 1) * kDigits + (inv >> (kDigitBits * (kSortPasses - 1)))], 1u);
-        ++o;
-      }
-      run += tot;
-    }
-    cp_async_wait<0>();
-    if (with_tail && tid == 0) {
-      // the client's ragged tail (d % 4 scalars) follows every float4 unit: one thread appends it
-      for (uint64_t e = nvec * 4; e < d; ++e) {
-        const uint32_t b = __float_as_uint(x[e]);
-        if ((b & 0x7FFFFFFFu) >= thresh) {
-          const unsigned long long pair = ((unsigned long long)(b & 0x7FFFFFFFu) << 32) | (unsigned long long)(b & 0x80000000u) | (unsigned long long)e;
-          if (run < L.capacity) out[run] = pair;
-          for (int p = 0; p < kSortPasses; ++p)
-            if (p < kSortPasses - 1 || count_top) atomicAdd(&s_dhist[p * kDigits + sort_digit(pair, p, keytop)], 1u);
-          ++run;
-        }
-      }
-    }
-    if (tid == 0) {
-      // the update must be the one the plan was made from
-      if (run - run0 != seg_count[seg]) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
-      if (with_tail) n_selected[c] = run;
-    }
-    __syncthreads();  // the staging buffers (and the ticket word) are reused by the next segment
-    {
-      // the segment's digit counts join the client's
-      unsigned long long* ghist = reinterpret_cast<unsigned long long*>(ws + L.off_ghist) + (size_t)c * kSortPasses * kDigits;
-      for (int i = tid; i < kSortPasses * kDigits; i += kSelThreads) {
-        const uint32_t v = s_dhist[i];
-        s_dhist[i] = 0;
-        if (v) atomicAdd(ghist + i, (unsigned long long)v);
-      }
-      __syncthreads();
-    }
-    pos = seg_end;
-  }
-  }
-}
-
 // ===================================================================================
 // K4  stable LSD radix ranking of the candidates, |x| descending (ties keep ascending index)
 // ===================================================================================
 // Sort key = keytop - key, keytop = the largest key of the client's highest non-empty histogram
 // bin, so the key only spans the bins between the threshold and the top: 19 + log2(#bins) bits.
-// Digits of 9, 9, 9, 4 bits.  One histogram kernel for all four digits and all clients, a small
-// scan kernel, then one single-pass kernel per digit (tiles handed out by ticket, tile-major with
-// the clients interleaved; decoupled look-back per digit value).  A pass whose digit is the same
-// for every candidate of a client (normally the fourth) is skipped for that client; which buffer
-// holds its data after pass q follows from the mask of skipped passes.
-
-// The clients' candidate arrays are concatenated in units of sort tiles (kSortTile pairs) and cut
-// into equal contiguous chunks, one per block; a block that crosses a client boundary merges
-// its shared histograms into that client's and starts afresh.
-__global__ void __launch_bounds__(256)
-k_sort_hist(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
-  __shared__ uint32_t sh[kSortPasses * kDigits];
-  pdl_enter();
-  const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
-  const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + L.off_sort_prefix);
-  unsigned long long* ghist_all = reinterpret_cast<unsigned long long*>(ws + L.off_ghist);
-  for (int i = threadIdx.x; i < kSortPasses * kDigits; i += 256) sh[i] = 0;
-  __syncthreads();
-  const uint32_t total_tiles = prefix[batch.n];
-  const uint32_t chunk = (total_tiles + gridDim.x - 1) / gridDim.x;
-  uint32_t t = blockIdx.x * chunk;
-  const uint32_t t_end = (t + chunk < total_tiles) ? t + chunk : total_tiles;
-  uint32_t c = 0;
-  while (t < t_end) {
-    while (prefix[c + 1] <= t) ++c;  // client of tile t (clients without tiles are passed over)
-    const uint32_t seg_end = prefix[c + 1] < t_end ? prefix[c + 1] : t_end;
-    const unsigned long long n = batch.c[c].plan->n_candidates;
-    const uint32_t keytop = sort_keytop(batch.c[c].plan);
-    const int n_count = top_digit_is_zero(batch.c[c].plan) ? kSortPasses - 1 : kSortPasses;
-    const unsigned long long* __restrict__ in = reinterpret_cast<const unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
-    const unsigned long long i0 = (unsigned long long)(t - prefix[c]) * kSortTile;
-    unsigned long long i1 = (unsigned long long)(seg_end - prefix[c]) * kSortTile;
-    if (i1 > n) i1 = n;
-    for (unsigned long long i = i0 + threadIdx.x; i < i1; i += 256) {
-      const unsigned long long pair = in[i];
-#pragma unroll
-      for (int p = 0; p < kSortPasses; ++p)
-        if (p < n_count) atomicAdd(&sh[p * kDigits + sort_digit(pair, p, keytop)], 1u);
-    }
-    __syncthreads();
-    unsigned long long* ghist = ghist_all + (size_t)c * kSortPasses * kDigits;
-    for (int i = threadIdx.x; i < kSortPasses * kDigits; i += 256) {
-      const uint32_t v = sh[i];
-      sh[i] = 0;
-      if (v) atomicAdd(ghist + i, (unsigned long long)v);
-    }
-    __syncthreads();
-    t = seg_end;
-  }
-}
-
-// per client: exclusive scans of the four digit histograms and the mask of constant digits
-__global__ void __launch_bounds__(kDigits)
-k_sort_scan(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
-  __shared__ unsigned long long s_scan[kDigits / 32];
-  pdl_enter();
-  const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
-  const uint32_t c = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const unsigned long long n = batch.c[c].plan->n_candidates;
-  const unsigned long long* ghist = reinterpret_cast<const unsigned long long*>(ws + L.off_ghist) + (size_t)c * kSortPasses * kDigits;
-  unsigned long long* gbase = reinterpret_cast<unsigned long long*>(ws + L.off_gbase) + (size_t)c * kSortPasses * kDigits;
-  uint32_t mask = top_digit_is_zero(batch.c[c].plan) ? 1u << (kSortPasses - 1) : 0u;  // not counted: known to be constant
-  for (int p = 0; p < kSortPasses; ++p) {
-    const unsigned long long cnt = ghist[p * kDigits + tid];
-    if (__syncthreads_or(cnt == n)) mask |= 1u << p;
-    unsigned long long incl = cnt;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned long long o = __shfl_up_sync(kFull, incl, off);
-      if (lane >= off) incl += o;
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    unsigned long long below = 0;
-    for (int w = 0; w < warp; ++w) below += s_scan[w];
-    gbase[p * kDigits + tid] = below + incl - cnt;
-    __syncthreads();
-  }
-  if (tid == 0) reinterpret_cast<uint32_t*>(ws + L.off_pass_mask)[c] = mask;
-}
+// Digits of 9, 9, 9, 4 bits, in one kernel of eight phases: the counters cleared and the candidates
+// selected in index order (unless that has been done), histograms of all four digits, their scans, and
+// per digit a single pass over tiles (tile-major with the clients interleaved; decoupled
+// look-back per digit value).  All phases draw from one ticket counter, and an item waits until the
+// phase before its own is complete: the items it waits for have lower tickets, so blocks that are
+// running hold them.  A pass whose digit is the same for every candidate of a client (normally the
+// fourth) is skipped for that client; which buffer holds its data after pass q follows from the
+// mask of skipped passes.  Used where the ranking by partition is not (see rank_shape).
 
 // two adjacent look-back words in one 128-bit access (each 64-bit half is its own atomic access)
 __device__ __forceinline__ void ld_relaxed2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
@@ -704,13 +695,13 @@ __device__ __forceinline__ void sort_tile(SortShared& sh, unsigned long long* __
   {
     const unsigned long long* __restrict__ p = src + (size_t)tile * kSortTile + wbase;
 #pragma unroll
-    for (int i = 0; i < IT; ++i) item[i] = (FULL || wbase + i * 32 < count) ? p[i * 32] : ~0ull;
+    for (int i = 0; i < IT; ++i) item[i] = (FULL || wbase + i * 32 < count) ? __ldcg(p + i * 32) : ~0ull;  // written in this kernel: L2
   }
   if (tid == 0) sh.next = next;  // waits for the ticket counter's answer, behind the item requests
   // the look-back needs the digit values' first positions in dst: requested early, used late
   unsigned long long gb0 = 0, gb1 = 0;
   if (tid < kDigits / 2) {
-    const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gbase + 2 * tid);
+    const ulonglong2 g = __ldcg(reinterpret_cast<const ulonglong2*>(gbase + 2 * tid));
     gb0 = g.x;
     gb1 = g.y;
   }
@@ -858,9 +849,12 @@ __device__ __forceinline__ void sort_tile(SortShared& sh, unsigned long long* __
   }
 }
 
+constexpr uint32_t kSortHistTiles = 8;   // tiles of a histogram item
+constexpr size_t kSortClear = 1 << 16;   // bytes of a clearing item
+
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks)
-k_sort_pass(int pass, const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
-  static_assert(kSortThreads * 2 >= kDigits && kSortTile <= 0xFFFF, "two digit values per owning thread; 16-bit slots");
+k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
+  static_assert(kSortThreads * 2 == kDigits && kSortTile <= 0xFFFF, "two digit values per thread; 16-bit slots");
   extern __shared__ __align__(16) unsigned char s_raw[];
   SortShared& sh = *reinterpret_cast<SortShared*>(s_raw);
   unsigned long long* s_items = reinterpret_cast<unsigned long long*>(s_raw + kSortSharedBytes);  // [kSortTile] the tile's items in digit order
@@ -870,78 +864,178 @@ k_sort_pass(int pass, const Batch batch, unsigned char* ws, const __grid_constan
   uint32_t* s_mask = s_keytop + batch.n;         // [n] its constant digits
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
-  const int tid = threadIdx.x;
-  const uint32_t n_clients = batch.n;
+  if (block_sees_error(&hdr->status) || hdr->lsd == kRankPartition) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n = batch.n;
   {
     const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + L.off_sort_prefix);
-    const uint32_t* pass_mask = reinterpret_cast<const uint32_t*>(ws + L.off_pass_mask);
-    for (uint32_t i = tid; i <= n_clients; i += kSortThreads) s_prefix[i] = prefix[i];
-    for (uint32_t i = tid; i < n_clients; i += kSortThreads) {
+    for (uint32_t i = tid; i <= n; i += kSortThreads) s_prefix[i] = prefix[i];
+    for (uint32_t i = tid; i < n; i += kSortThreads) {
       const cvlc_plan_t* plan = batch.c[i].plan;
       s_ncand[i] = (uint32_t)plan->n_candidates;  // <= capacity < 2^32: checked by k_encode_init
       s_keytop[i] = sort_keytop(plan);
-      s_mask[i] = pass_mask[i];
     }
   }
   for (int i = tid; i < (kSortThreads / 32) * kDigits; i += kSortThreads) (&sh.mm[0][0])[i] = 0u;
-  if (tid == 0) sh.tile = atomicAdd(&hdr->sort_ticket[pass], 1u);
+  if (tid == 0) sh.tile = atomicAdd(&hdr->sort_ticket, 1u);
   __syncthreads();
-  const uint32_t total_tickets = hdr->max_sort_tiles * n_clients;
-  unsigned long long* state_all =
-      reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) + (size_t)pass * n_clients * L.sort_tiles_max * kDigits;
+  // first items of the phases: 0 clearing, 1 selection, 2 histograms, 3 scans, 4 .. 7 digit passes
+  const bool all = hdr->lsd == kRankAllDigits;
+  const size_t clear_bytes = L.off_buf_a - L.off_ghist;
+  const uint32_t n_pass = hdr->max_sort_tiles * n;
+  uint32_t first_item[9];
+  first_item[0] = 0;
+  first_item[1] = all ? (uint32_t)((clear_bytes + kSortClear - 1) / kSortClear) : 0u;
+  first_item[2] = first_item[1] + (all ? (uint32_t)(select_tiles_of(d, kSortThreads) * n) : 0u);
+  first_item[3] = first_item[2] + (hdr->max_sort_tiles + kSortHistTiles - 1) / kSortHistTiles * n;
+  first_item[4] = first_item[3] + n;
+#pragma unroll
+  for (int p = 5; p < 9; ++p) first_item[p] = first_item[p - 1] + n_pass;
+  unsigned long long* ghist_all = reinterpret_cast<unsigned long long*>(ws + L.off_ghist);
+  unsigned long long* gbase_all = reinterpret_cast<unsigned long long*>(ws + L.off_gbase);
+  uint32_t* pass_mask = reinterpret_cast<uint32_t*>(ws + L.off_pass_mask);
   uint4* s_wc4 = reinterpret_cast<uint4*>(&sh.wc[0][0]);
-  const int shift = kDigitBits * pass;
+  int phase = all ? 0 : 2;
 
   while (true) {
     const uint32_t gt = sh.tile;
-    if (gt >= total_tickets) break;
-    s_wc4[2 * tid] = make_uint4(0u, 0u, 0u, 0u);
-    s_wc4[2 * tid + 1] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();  // everyone has read the ticket; the counters are clear
-    // the next ticket is fetched while this tile is worked on
+    if (gt >= first_item[8]) break;
+    __syncthreads();  // everyone has read the ticket
+    // the next ticket is fetched while this item is worked on
     uint32_t next = 0;
-    if (tid == 0) next = atomicAdd(&hdr->sort_ticket[pass], 1u);
-    // tile-major tickets with the clients interleaved: the tiles in flight are a few consecutive
-    // tiles of every client, which keeps every look-back short
-    const uint32_t tile = gt / n_clients;
-    const uint32_t c = gt - tile * n_clients;
-    const uint32_t mask = s_mask[c];
-    auto source = [&](uint32_t cc, uint32_t m) -> unsigned long long* {  // buffer holding client cc's items before this pass
-      const int flips = __popc(~m & ((1u << pass) - 1u));
-      return reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_b : L.off_buf_a)) + (size_t)cc * L.capacity;
-    };
-    if (tile < s_prefix[c + 1] - s_prefix[c] && !(mask & (1u << pass))) {  // else: no such tile, or a constant digit
-      const uint32_t n32 = s_ncand[c];
-      const uint32_t keytop = s_keytop[c];
-      const int flips = __popc(~mask & ((1u << pass) - 1u));
-      const unsigned long long* src = source(c, mask);
-      unsigned long long* dst =
-          reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_a : L.off_buf_b)) + (size_t)c * L.capacity;
-      unsigned long long* state = state_all + (size_t)s_prefix[c] * kDigits;
-      const unsigned long long* gbase = reinterpret_cast<const unsigned long long*>(ws + L.off_gbase) +
-                                        (size_t)c * kSortPasses * kDigits + (size_t)pass * kDigits;
-      const uint32_t tile_first = tile * (uint32_t)kSortTile;
-      const uint32_t count = (n32 - tile_first < (uint32_t)kSortTile) ? n32 - tile_first : (uint32_t)kSortTile;
-      // the next tile's items are asked into L2 while this one is ranked and written
-      auto prefetch_next = [&](uint32_t nt) {
-        if (nt >= total_tickets) return;
-        const uint32_t t2 = nt / n_clients, c2 = nt - t2 * n_clients;
-        for (uint32_t l = tid; l < (uint32_t)(kSortTile / 16); l += kSortThreads) {  // 128-byte lines of 16 items
-          const uint32_t line = t2 * (uint32_t)(kSortTile / 16) + l;
-          if (line * 16u < s_ncand[c2]) {
-            const unsigned long long* p = source(c2, s_mask[c2]) + (size_t)line * 16;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    if (tid == 0) next = atomicAdd(&hdr->sort_ticket, 1u);
+    int my_phase = 0;
+    uint32_t want = 0, first = 0;  // items of the phase before; first item of this one
+#pragma unroll
+    for (int p = 1; p < 8; ++p) {
+      if (gt >= first_item[p]) {
+        my_phase = p;
+        want = first_item[p] - first_item[p - 1];
+        first = first_item[p];
+      }
+    }
+    if (my_phase != phase) {
+      if (tid == 0) {
+        int polls = 0;
+        while (*reinterpret_cast<volatile uint32_t*>(&hdr->sort_done[my_phase - 1]) < want) {
+          if (++polls > kMaxPolls) {
+            set_status(&hdr->status, CVLC_ERR_DEVICE_TIMEOUT);
+            break;
           }
+          __nanosleep(polls > 64 ? 256 : 32);
         }
+        __threadfence();
+      }
+      __syncthreads();
+      if (phase < 4 && my_phase >= 4)
+        for (uint32_t i = tid; i < n; i += kSortThreads) s_mask[i] = __ldcg(pass_mask + i);
+      phase = my_phase;
+      __syncthreads();
+    }
+    if (phase == 0) {
+      ulonglong2* p = reinterpret_cast<ulonglong2*>(ws + L.off_ghist + (size_t)gt * kSortClear);
+      const size_t left = clear_bytes - (size_t)gt * kSortClear, m = (left < kSortClear ? left : kSortClear) / 16;
+      for (size_t i = tid; i < m; i += kSortThreads) p[i] = make_ulonglong2(0ull, 0ull);
+    } else if (phase == 1) {
+      select_lookback_tile<kSortThreads>(batch, d, ws, L, gt - first);
+    } else if (phase == 2) {
+      // digit counts of up to kSortHistTiles tiles of a client
+      uint32_t* cnt = reinterpret_cast<uint32_t*>(s_items);
+      const uint32_t g = (gt - first) / n, c = (gt - first) - g * n;
+      const uint64_t i0 = (uint64_t)g * kSortHistTiles * kSortTile, i1 = i0 + (uint64_t)kSortHistTiles * kSortTile;
+      const uint32_t hi = (uint64_t)s_ncand[c] < i1 ? s_ncand[c] : (uint32_t)i1;
+      if (i0 < s_ncand[c]) {
+        for (int i = tid; i < kSortPasses * kDigits; i += kSortThreads) cnt[i] = 0;
+        __syncthreads();
+        const uint32_t keytop = s_keytop[c];
+        const int n_count = top_digit_is_zero(batch.c[c].plan) ? kSortPasses - 1 : kSortPasses;
+        const unsigned long long* in = reinterpret_cast<const unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
+        for (uint32_t i = (uint32_t)i0 + tid; i < hi; i += kSortThreads) {
+          const unsigned long long pair = __ldcg(in + i);
+#pragma unroll
+          for (int p = 0; p < kSortPasses; ++p)
+            if (p < n_count) atomicAdd(&cnt[p * kDigits + sort_digit(pair, p, keytop)], 1u);
+        }
+        __syncthreads();
+        unsigned long long* ghist = ghist_all + (size_t)c * kSortPasses * kDigits;
+        for (int i = tid; i < kSortPasses * kDigits; i += kSortThreads)
+          if (cnt[i]) atomicAdd(ghist + i, (unsigned long long)cnt[i]);
+      }
+    } else if (phase == 3) {
+      // one client's exclusive scans of the digit histograms and the mask of its constant digits
+      const uint32_t c = gt - first;
+      const unsigned long long have = s_ncand[c];
+      unsigned long long* s_scan = s_items;
+      uint32_t mask = top_digit_is_zero(batch.c[c].plan) ? 1u << (kSortPasses - 1) : 0u;  // not counted: known to be constant
+      for (int p = 0; p < kSortPasses; ++p) {
+        const size_t at = ((size_t)c * kSortPasses + p) * kDigits + 2 * tid;
+        const unsigned long long a = __ldcg(ghist_all + at), b = __ldcg(ghist_all + at + 1);
+        if (__syncthreads_or(a == have || b == have)) mask |= 1u << p;
+        unsigned long long incl = a + b;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const unsigned long long o = __shfl_up_sync(kFull, incl, off);
+          if (lane >= off) incl += o;
+        }
+        if (lane == 31) s_scan[warp] = incl;
+        __syncthreads();
+        unsigned long long below = incl - a - b;
+        for (int w = 0; w < warp; ++w) below += s_scan[w];
+        gbase_all[at] = below;
+        gbase_all[at + 1] = below + a;
+        __syncthreads();
+      }
+      if (tid == 0) pass_mask[c] = mask;
+    } else {
+      // tile-major tickets with the clients interleaved: the tiles in flight are a few consecutive
+      // tiles of every client, which keeps every look-back short
+      const int pass = phase - 4;
+      const uint32_t t = gt - first;
+      const uint32_t tile = t / n, c = t - tile * n;
+      const uint32_t mask = s_mask[c];
+      auto source = [&](uint32_t cc) -> unsigned long long* {  // buffer holding client cc's items before this pass
+        const int flips = __popc(~s_mask[cc] & ((1u << pass) - 1u));
+        return reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_b : L.off_buf_a)) + (size_t)cc * L.capacity;
       };
-      if (count == (uint32_t)kSortTile)
-        sort_tile<true>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, shift, &hdr->status, next, prefetch_next);
-      else
-        sort_tile<false>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, shift, &hdr->status, next, prefetch_next);
+      s_wc4[2 * tid] = make_uint4(0u, 0u, 0u, 0u);
+      s_wc4[2 * tid + 1] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();  // the counters are clear
+      if (tile < s_prefix[c + 1] - s_prefix[c] && !(mask & (1u << pass))) {  // else: no such tile, or a constant digit
+        const uint32_t n32 = s_ncand[c];
+        const uint32_t keytop = s_keytop[c];
+        const int flips = __popc(~mask & ((1u << pass) - 1u));
+        const unsigned long long* src = source(c);
+        unsigned long long* dst =
+            reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_a : L.off_buf_b)) + (size_t)c * L.capacity;
+        unsigned long long* state = reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) +
+                                    ((size_t)pass * n * L.sort_tiles_max + s_prefix[c]) * kDigits;
+        const unsigned long long* gbase = gbase_all + ((size_t)c * kSortPasses + pass) * kDigits;
+        const uint32_t tile_first = tile * (uint32_t)kSortTile;
+        const uint32_t count = (n32 - tile_first < (uint32_t)kSortTile) ? n32 - tile_first : (uint32_t)kSortTile;
+        // the next tile's items are asked into L2 while this one is ranked and written
+        auto prefetch_next = [&](uint32_t nt) {
+          if (nt < first || nt - first >= n_pass) return;
+          const uint32_t t2 = (nt - first) / n, c2 = (nt - first) - t2 * n;
+          for (uint32_t l = tid; l < (uint32_t)(kSortTile / 16); l += kSortThreads) {  // 128-byte lines of 16 items
+            const uint32_t line = t2 * (uint32_t)(kSortTile / 16) + l;
+            if (line * 16u < s_ncand[c2]) {
+              const unsigned long long* p = source(c2) + (size_t)line * 16;
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+            }
+          }
+        };
+        if (count == (uint32_t)kSortTile)
+          sort_tile<true>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
+        else
+          sort_tile<false>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
+      }
     }
     if (tid == 0) sh.tile = next;
     __syncthreads();
+    if (tid == 0) {  // behind the barrier: the item's writes are done
+      __threadfence();
+      atomicAdd(&hdr->sort_done[phase], 1u);
+    }
   }
 }
 
@@ -1203,13 +1297,13 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
 // ===================================================================================
 
 template <int CAP>
-static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, const Partition& part,
-                          const unsigned char* plan_ws, unsigned char* w, cudaStream_t st) {
+static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, const unsigned char* plan_ws,
+                          unsigned char* w, cudaStream_t st) {
   BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
-  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, true, w, batch, shape, L, plan_ws, part);
+  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, true, w, batch, shape, L, plan_ws);
 }
 
 template <int CAP>
@@ -1237,9 +1331,9 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSelStages * kSelStageBytes));
+    e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
+    e = cudaFuncSetAttribute(k_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -1251,25 +1345,25 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
 
   const Partition part = make_partition(shape.d, n);
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
-  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, part, pws, w, st);
-  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, part, pws, w, st);
-  else launch_init_t<kLargeBatch>(clients, n, shape, L, part, pws, w, st);
+  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st);
+  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st);
+  else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st);
   const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (pws) {
-    launch_kernel(kKSelect, k_select, part.grid, kSelThreads, kSelStages * kSelStageBytes, st, true, batch, shape.d, part, pws, w, L);
+    const uint64_t want = (part.rows + select_group_rows(part) - 1) / select_group_rows(part) * n;
+    const unsigned grid = (unsigned)(want < (uint64_t)kNumSM ? want : kNumSM);
+    launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, pws, w, L);
+    e = launch_rank(batch, L, pws, w, (int)shape.s, st);
+    if (e != cudaSuccess) return e;
   } else {
-    const uint64_t want = L.select_tiles * n;
+    const uint64_t want = select_tiles_of(shape.d, kSelectThreads) * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(4 * kNumSM) ? want : 4 * kNumSM);
     launch_kernel(kKSelectLookback, k_select_lookback, grid, kSelectThreads, 0, st, true, batch, shape.d, w, L);
   }
   {
     const uint64_t want = L.sort_tiles_max * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(kSortMinBlocks * kNumSM) ? want : kSortMinBlocks * kNumSM);
-    if (!pws)  // the selection with known offsets has counted the digits already
-      launch_kernel(kKSortHist, k_sort_hist, grid, 256, 0, st, true, batch, w, L);
-    launch_kernel(kKSortScan, k_sort_scan, n, kDigits, 0, st, true, batch, w, L);
-    for (int pass = 0; pass < kSortPasses; ++pass)
-      launch_kernel(kKSortPass, k_sort_pass, grid, kSortThreads, sort_smem_bytes(n), st, true, pass, batch, w, L);
+    launch_kernel(kKSort, k_sort, grid, kSortThreads, sort_smem_bytes(n), st, true, batch, shape.d, w, L);
   }
   if (wait_before_pack) {
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);

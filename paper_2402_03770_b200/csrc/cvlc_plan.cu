@@ -18,9 +18,8 @@ namespace cvlc {
 constexpr int kHistThreads = kStreamThreads;
 constexpr int kHistSub = 4;  // shared sub-histograms per block (64 KB)
 
-// The clients' updates are treated as one concatenated array of units (a unit = one float4,
-// plus one ragged-tail unit per client) that is cut into equal contiguous chunks, one per
-// block, so the load is even whatever the number of clients; a block that crosses a client
+// The clients' rows form one concatenated array that is cut into equal contiguous chunks, one or two
+// per block, so the load is even whatever the number of clients; a block that crosses a client
 // boundary merges its shared histogram into that client's global one and starts afresh.
 
 // counts the four magnitude keys of a float4; returns the largest of them
@@ -37,8 +36,7 @@ __device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
 
 __global__ void __launch_bounds__(kHistThreads, 2)
 k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
-       unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint32_t* __restrict__ seg_hist_all,
-       uint32_t* __restrict__ row_max_all) {
+       unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint32_t* __restrict__ row_max_all) {
   extern __shared__ uint32_t sh_hist[];  // [kHistSub][4096]
   pdl_enter();
   for (int i = threadIdx.x; i < kHistSub * CVLC_HIST_BINS; i += kHistThreads) sh_hist[i] = 0;
@@ -47,21 +45,20 @@ k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
   const int lane = threadIdx.x & 31;
 
   const uint64_t nvec = d >> 2;
-  const uint64_t units = part.units;  // per client: nvec float4 units and one tail unit
   for (uint32_t q = blockIdx.x; q < part.n_chunks; q += gridDim.x) {
   uint64_t pos = (uint64_t)q * part.chunk;
   const uint64_t end = (pos + part.chunk < part.total) ? pos + part.chunk : part.total;
 
   while (pos < end) {
-    const uint64_t c = pos / units;
-    const uint64_t seg_end = ((c + 1) * units < end) ? (c + 1) * units : end;
-    const uint64_t u0 = pos - c * units, u1 = seg_end - c * units;
+    const uint64_t c = pos / part.rows;
+    const uint64_t seg_end = ((c + 1) * part.rows < end) ? (c + 1) * part.rows : end;
+    const uint64_t u0 = (pos - c * part.rows) * kRowUnits, u1 = (seg_end - c * part.rows) * kRowUnits;  // units of the client
     const float* __restrict__ x = batch.c[c].x;
     const float4* xv = reinterpret_cast<const float4*>(x);
     const uint64_t v1 = (u1 < nvec) ? u1 : nvec;  // float4 units of this segment: [u0, v1)
-    // largest key of every row (kRowUnits consecutive units from u0 on: a warp-wide load covers 32 / kRowUnits rows);
-    // one whole-warp reduction per row of a load, each seeing that row's keys only
-    uint32_t* __restrict__ row_max = row_max_all + seg_first_tile(pos, (uint32_t)(q + c)) * kTileRows;
+    // largest key of every row (a warp-wide load covers 32 / kRowUnits of them); one whole-warp reduction per row of a load,
+    // each seeing that row's keys only
+    uint32_t* __restrict__ row_max = row_max_all + c * part.rows;
     static_assert(32 % kRowUnits == 0, "a warp-wide load covers whole rows");
     constexpr int kRowsPerLoad = 32 / kRowUnits;
     const int my_group = lane / kRowUnits;
@@ -94,27 +91,24 @@ k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
       for (int u = 0; u < 4; ++u) {
         const uint32_t m = row_maxima(hist_add4(my, a[u]));
         top = m > top ? m : top;
-        if (lane % kRowUnits == 0) row_max[(v - u0 + u * kHistThreads) / kRowUnits] = m;
+        if (lane % kRowUnits == 0) row_max[(v + u * kHistThreads) / kRowUnits] = m;
       }
     }
     for (; v - lane < v1; v += kHistThreads) {  // rows that may end inside the warp
       const bool on = v < v1;
       const uint32_t m = row_maxima(on ? hist_add4(my, __ldg(xv + v)) : 0u);
       top = m > top ? m : top;
-      if (lane % kRowUnits == 0 && on) row_max[(v - u0) / kRowUnits] = m;
+      if (lane % kRowUnits == 0 && on) row_max[v / kRowUnits] = m;
     }
     // ragged tail of the client (d not a multiple of 4)
-    if (u1 == units && threadIdx.x < (d & 3)) {
+    if (seg_end == (c + 1) * part.rows && threadIdx.x < (d & 3)) {
       const uint32_t k0 = __float_as_uint(x[(nvec << 2) + threadIdx.x]) & 0x7FFFFFFFu;
       top = k0 > top ? k0 : top;
       atomicAdd(my + (k0 >> 19), 1u);
     }
     if (top >= 0x7F800000u) atomicOr(nonfinite_all + c, 1u);  // a key of exponent 255: Inf or NaN
     __syncthreads();
-    // merge into the client's histogram and keep this segment's own counts (segment = chunk + client):
-    // the selection kernel derives its output offsets from them
     unsigned long long* __restrict__ hist = hist_all + (size_t)c * CVLC_HIST_BINS;
-    uint32_t* __restrict__ seg_hist = seg_hist_all + ((size_t)q + c) * CVLC_HIST_BINS;
     for (int b = threadIdx.x; b < CVLC_HIST_BINS; b += kHistThreads) {
       uint32_t cnt = 0;
 #pragma unroll
@@ -122,7 +116,6 @@ k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
         cnt += sh_hist[sub * CVLC_HIST_BINS + b];
         sh_hist[sub * CVLC_HIST_BINS + b] = 0;
       }
-      seg_hist[b] = cnt;
       if (cnt) atomicAdd(hist + b, (unsigned long long)cnt);
     }
     __syncthreads();
@@ -325,15 +318,14 @@ __device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, d
 __global__ void __launch_bounds__(kPlanThreads, 1)
 k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __restrict__ nonfinite_all,
            const Batch batch, const __grid_constant__ Shape shape,
-           const __grid_constant__ Partition part, unsigned char* ws, int have_segments) {
+           unsigned char* ws, int have_rows) {
   extern __shared__ unsigned char smem_raw[];
   unsigned long long* Nsuf = reinterpret_cast<unsigned long long*>(smem_raw);  // [4096] survival counts
   double* ptX = reinterpret_cast<double*>(smem_raw + 4096 * 8);                // fit points, ascending bin
   double* ptY = ptX + 4096;
   __shared__ PlanShared S;
   __shared__ PlanTab T;
-  __shared__ uint32_t s_thresh_bin, s_top_bin;
-  __shared__ unsigned long long s_seg_warp[kPlanThreads / 32];
+  __shared__ uint32_t s_thresh_bin, s_top_bin, s_fullest;
   int32_t* ws_status = reinterpret_cast<int32_t*>(ws);
   pdl_enter();
 
@@ -353,6 +345,7 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
   }
 
   if (warp == 0) build_plan_tab(T, shape, batch.c[blockIdx.x].scale_B, lane);
+  if (tid == 0) s_fullest = 0;
   __syncthreads();
 
   // ---- survival counts N_j = #{bin >= j} ------------------------------------------
@@ -499,63 +492,27 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
   }
   __syncthreads();
 
-  // candidates per segment of this client (segment = part of the client inside one block's chunk of
-  // the histogram / selection kernels) and their exclusive prefix: the selection kernel's offsets.
-  // A plan made from a histogram alone has no segments; its workspace header stays unmarked.
-
-  if (have_segments) {
-    const uint32_t c = blockIdx.x;
-    const uint32_t S = part.max_segments;
-    uint32_t* seg_count = reinterpret_cast<uint32_t*>(ws + plan_off_seg_count(batch.n));
-    unsigned long long* seg_prefix = reinterpret_cast<unsigned long long*>(ws + plan_off_seg_prefix(batch.n, S));
-    const uint64_t row_tiles = row_tiles_total(part);
-    const uint32_t* seg_hist = reinterpret_cast<const uint32_t*>(ws + plan_off_seg_hist(batch.n, S, row_tiles));
-    const uint64_t first = (uint64_t)c * part.units, last = first + part.units - 1;
-    const uint32_t b0 = (uint32_t)(first / part.chunk), b1 = (uint32_t)(last / part.chunk);
-    const uint32_t jt = s_thresh_bin, jtop = s_top_bin;  // nothing above the client's highest non-empty bin
-    uint32_t* s_count = reinterpret_cast<uint32_t*>(ptX);  // the fit points are no longer needed; at most n_chunks + 1 segments
-    for (uint32_t b = b0 + warp; b <= b1; b += kPlanThreads / 32) {
-      const uint32_t* hsrc = seg_hist + ((size_t)b + c) * CVLC_HIST_BINS;
-      uint32_t sum = 0;
-      for (uint32_t j = jt + lane; j <= jtop; j += 32) sum += hsrc[j];
-      sum = __reduce_add_sync(kFull, sum);
-      if (lane == 0) s_count[b - b0] = sum;
-    }
-    __syncthreads();
-    // exclusive prefix over the client's segments, a block scan of kPlanThreads of them at a time (this, the row lists and
-    // the fit's sums moved off one thread: 58 -> 14 us for one client of 1.1e7 coordinates)
-    unsigned long long carry = 0;
-    for (uint32_t base = 0; base <= b1 - b0; base += kPlanThreads) {
-      const uint32_t b = base + tid;
-      const unsigned long long cnt = (b <= b1 - b0) ? s_count[b] : 0u;
-      unsigned long long incl = cnt;
+  // where every candidate bin starts among the client's candidates (from the top bin down) and the fullest of them: the
+  // selection's and the ranking's buckets.  A plan made from a histogram alone has no rows; its workspace header stays unmarked.
+  if (have_rows) {
+    uint32_t* bin_start = reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(batch.n)) + (size_t)blockIdx.x * CVLC_HIST_BINS;
+    uint32_t fullest = 0;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long o = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += o;
-      }
-      if (lane == 31) s_seg_warp[warp] = incl;
-      __syncthreads();
-      unsigned long long below = carry, all = carry;
-#pragma unroll 8
-      for (int w = 0; w < kPlanThreads / 32; ++w) {
-        const unsigned long long t = s_seg_warp[w];
-        if (w < warp) below += t;
-        all += t;
-      }
-      if (b <= b1 - b0) {
-        seg_count[b0 + b + c] = (uint32_t)cnt;
-        seg_prefix[b0 + b + c] = below + incl - cnt;
-      }
-      carry = all;
-      __syncthreads();
+    for (int i = 0; i < 4; ++i) {
+      const int j = 4 * tid + i;
+      if (j < (int)s_thresh_bin || j > (int)s_top_bin) continue;
+      bin_start[j] = (j == CVLC_HIST_BINS - 1) ? 0u : (uint32_t)Nsuf[j + 1];
+      if ((uint32_t)h[i] > fullest) fullest = (uint32_t)h[i];
     }
+    fullest = __reduce_max_sync(kFull, fullest);
+    if (lane == 0 && fullest) atomicMax(&s_fullest, fullest);
+    __syncthreads();
     if (tid == 0) {
-      if (c == 0) {
+      reinterpret_cast<uint32_t*>(ws + plan_off_max_bin(batch.n))[blockIdx.x] = s_fullest;
+      if (blockIdx.x == 0) {
         PlanWsHeader* hdr = reinterpret_cast<PlanWsHeader*>(ws);
         hdr->n = batch.n;
         hdr->d = shape.d;
-        hdr->n_chunks = part.n_chunks;
         hdr->magic = kPlanWsMagic;
       }
     }
@@ -1313,7 +1270,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // ===================================================================================
 
 constexpr size_t kFitSmem = 3 * 4096 * 8 + 4096 * 2;  // survival counts, the fit points and their bins
-static_assert((kNumSM * 2 * kChunksPerBlock + 1) * 4 <= 4096 * 8, "a client's segment counts fit the fit points' place");
+
 constexpr size_t kTuneSmem = (sizeof(PlanSolver) + 255) & ~(size_t)255;
 
 static cudaError_t plan_attributes() {
@@ -1346,15 +1303,15 @@ static void launch_zero_t(const ClientDesc* clients, uint32_t n, unsigned char* 
   launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, true, batch, reinterpret_cast<ClientDesc*>(w + off_desc),
                 reinterpret_cast<uint4*>(w), bytes / 16, reinterpret_cast<uint4*>(w + at), more / 16);
 }
-static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, const Partition& part, size_t bytes, size_t at, size_t more, cudaStream_t st) {
-  const size_t off_desc = plan_off_desc(n, part.max_segments);
+static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t bytes, size_t at, size_t more, cudaStream_t st) {
+  const size_t off_desc = plan_off_desc(n);
   if (n <= (uint32_t)kSmallBatch) launch_zero_t<kSmallBatch>(clients, n, w, off_desc, bytes, at, more, st);
   else if (n <= (uint32_t)kMediumBatch) launch_zero_t<kMediumBatch>(clients, n, w, off_desc, bytes, at, more, st);
   else launch_zero_t<kLargeBatch>(clients, n, w, off_desc, bytes, at, more, st);
   return Batch{reinterpret_cast<const ClientDesc*>(w + off_desc), n};
 }
 
-// histogram of every client, then (unless only the histograms are wanted) fit, threshold and segment tables
+// histogram of every client, then (unless only the histograms are wanted) fit, threshold and the bins' tables
 static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                               unsigned long long* hist_out, cudaStream_t st) {
   cudaError_t e = plan_attributes();
@@ -1363,28 +1320,25 @@ static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(w + kPlanWsHist);
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   const Partition part = make_partition(shape.d, n);
-  const uint64_t row_tiles = row_tiles_total(part);
-  uint32_t* seg_hist = reinterpret_cast<uint32_t*>(w + plan_off_seg_hist(n, part.max_segments, row_tiles));
-  uint32_t* row_max = reinterpret_cast<uint32_t*>(w + plan_off_row_max(n, part.max_segments));
-  // header, histograms, flags and tuning keys start at zero; the segment tables, the per-segment histograms and the
-  // rows' maxima are written in full by the kernels that follow
-  const Batch batch = launch_zero(clients, n, w, part, plan_off_seg_count(n), 0, 0, st);
+  uint32_t* row_max = reinterpret_cast<uint32_t*>(w + plan_off_row_max(n));
+  // header, histograms, flags and tuning keys start at zero; the rest is written in full by the kernels that follow
+  const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), 0, 0, st);
   // two resident blocks per SM share the concatenated updates evenly
-  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape.d, part, hist, flags, seg_hist, row_max);
+  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape.d, part, hist, flags, row_max);
   if (hist_out) {
     // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
-    // header stays unmarked, so an encode call cannot take it for one that holds a plan's segment tables.
+    // header stays unmarked, so an encode call cannot take it for one that holds a plan's tables.
     const cudaError_t e2 = cudaGetLastError();
     if (e2 != cudaSuccess) return e2;
     return cudaMemcpyAsync(hist_out, hist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
   }
-  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, part, w, 1);
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 1);
   return cudaGetLastError();
 }
 
 static cudaError_t plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap) {
   unsigned char* w = static_cast<unsigned char*>(ws);
-  const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n, make_partition(shape.d, n).max_segments)), n};
+  const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
   launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w);
   return cudaGetLastError();
 }
@@ -1441,12 +1395,11 @@ cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const S
   if (e != cudaSuccess) return e;
   unsigned char* w = static_cast<unsigned char*>(ws);
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
-  const Partition part = make_partition(shape.d, n);
   // status word, header and tuning keys start at zero: the header stays unmarked, so an encode call cannot take this
-  // workspace for one that holds segment tables
-  const Batch batch = launch_zero(clients, n, w, part, kPlanWsHist, plan_off_keys(n), plan_off_seg_count(n) - plan_off_keys(n), st);
+  // workspace for one that holds the rows' maxima
+  const Batch batch = launch_zero(clients, n, w, kPlanWsHist, plan_off_keys(n), plan_off_desc(n) - plan_off_keys(n), st);
   launch_kernel(kKHistCheck, k_hist_check, n, 256, 0, st, true, hist, shape.d, flags);
-  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, part, w, 0);
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 0);
   const cudaError_t e2 = cudaGetLastError();
   if (e2 != cudaSuccess) return e2;
   return plan_back(n, shape, ws, st, true);

@@ -1,0 +1,54 @@
+"""GPU parity of the ranking on value distributions at the edges of its buckets: buckets that need the partition, ties of all
+sizes up to and beyond what a block holds, buckets that send the batch to the digit passes, zeros among the candidates, mixed
+batches; plan and stream against the oracle, with the plan's workspace (partition) and without it (digit passes)."""
+import numpy as np
+import pytest
+
+from gpu_util import assert_plan_equal, gpu_params, oracle_plan_encode, params_dict
+
+pytestmark = pytest.mark.gpu
+
+
+def values(kind, d, rng):
+    if kind == "narrow":                                    # every candidate in two or three bins: large coarse buckets
+        return rng.choice([-1.0, 1.0], d) * (1.0 + 0.06 * rng.random(d))
+    x = rng.laplace(0, 1e-3, d)
+    if kind.startswith("ties"):                             # one value many times, in the middle of the candidates
+        n = int(kind[4:])
+        x[rng.choice(d, n, replace=False)] = np.quantile(np.abs(x), 0.97) * rng.choice([-1.0, 1.0], n)
+    elif kind == "grid":
+        x = np.round(x * 4096.0) / 4096.0
+    elif kind == "near_ties":                               # neighbouring floats
+        n = d // 20
+        x[rng.choice(d, n, replace=False)] = np.float32(0.01) + np.arange(n) % 37 * np.float32(2.0 ** -30)
+    elif kind == "wide":
+        x = rng.standard_normal(d) * 10.0 ** rng.uniform(-30, 30, d)
+    elif kind == "sparse":                                  # fewer values than are sent
+        x[rng.random(d) < 0.97] = 0.0
+    return x
+
+
+@pytest.mark.parametrize("kind", ["laplace", "narrow", "ties900", "ties5000", "ties20000", "ties100000", "grid", "near_ties", "wide", "sparse"])
+@pytest.mark.parametrize("d,bits", [(2_000_003, 3.0), (70_001, 2.0)])
+def test_ranking_matches_the_oracle(kind, d, bits):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    assert torch.cuda.is_available()
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(d + len(kind))
+    if kind.startswith("ties") and int(kind[4:]) > d // 4:
+        kind = f"ties{d // 4}"
+    xs = [values(kind, d, rng).astype(np.float32), values("laplace", d, rng).astype(np.float32)]
+    pds = [params_dict(d, int(bits * d), seed=5 + c, client_id=c) for c in range(2)]
+    params = [gpu_params(pd) for pd in pds]
+    refs = [oracle_plan_encode(x, pd) for x, pd in zip(xs, pds)]
+    dxs = [torch.from_numpy(x).to(dev) for x in xs]
+    enc = B.BatchEncoder(params, dev)
+    for use_plan_ws in (True, False):
+        for o in enc.outs:
+            o.fill_(0x3C)
+        outs = enc.run(dxs, use_plan_ws=use_plan_ws)
+        assert enc.status() == 0
+        for c, (fields, stream) in enumerate(refs):
+            assert_plan_equal(enc.read_plan(c), fields)
+            assert (outs[c].cpu().numpy() == stream).all(), (c, use_plan_ws)
