@@ -66,14 +66,15 @@ struct Shape {
 
 // ---- workspace layouts (byte offsets; every region 256-byte aligned) ----------
 
-// The float4 units of an update are grouped into rows of kRowUnits (64 coordinates, half of a warp-wide load).  The histogram
-// kernel streams the clients' rows as one concatenated array cut into equal contiguous chunks and leaves the largest magnitude
-// key of every row; the selection reads only the rows that hold a candidate (a key at or above the threshold).  The ragged
-// tail of an update (d % 4 coordinates) goes with its last row.
+// The float4 units of an update are grouped into rows of kRowUnits (16 coordinates, 64 bytes: what a DRAM access moves).  The
+// histogram kernel streams the clients' rows as one concatenated array cut into equal contiguous chunks and leaves the bin of
+// every row's largest key; the selection reads only the rows that hold a candidate (a bin at or above the threshold's).  With
+// rows of 64 coordinates most of a spread-out update was read again (83 % at 3 % candidates, now 42 %).  The ragged tail of an
+// update (d % 4 coordinates) goes with its last row.
 constexpr int kStreamThreads = 512;
-constexpr int kRowUnits = 16;
+constexpr int kRowUnits = 4;
 struct Partition {
-  uint64_t rows;      // per client
+  uint64_t rows;      // per client, rounded up to a multiple of 16 (the last ones may be empty)
   uint64_t total;     // rows * n
   uint64_t chunk;     // rows per chunk of the histogram kernel
   uint32_t n_chunks;
@@ -81,22 +82,22 @@ struct Partition {
 };
 CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   Partition P;
-  P.rows = ((d >> 2) + kRowUnits - 1) / kRowUnits;
-  if (P.rows == 0) P.rows = 1;
+  P.rows = (((d >> 2) + kRowUnits - 1) / kRowUnits + 15) & ~(uint64_t)15;
+  if (P.rows == 0) P.rows = 16;
   P.total = P.rows * n;
-  uint64_t grid = (P.total + 63) / 64;
+  uint64_t grid = (P.total + 255) / 256;
   if (grid > (uint64_t)(2 * kNumSM)) grid = 2 * kNumSM;
   P.grid = (uint32_t)grid;
   // two chunks per block where that leaves each 64 KB and more: every chunk ends with a merge into a client's histogram
-  const uint64_t n_chunks = P.total / (2 * grid) >= 256 ? 2 * grid : grid;
-  P.chunk = (P.total + n_chunks - 1) / n_chunks;
+  const uint64_t n_chunks = P.total / (2 * grid) >= 1024 ? 2 * grid : grid;
+  P.chunk = ((P.total + n_chunks - 1) / n_chunks + 15) & ~(uint64_t)15;
   P.n_chunks = (uint32_t)((P.total + P.chunk - 1) / P.chunk);
   return P;
 }
 
 // plan workspace:
 //   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2] | ClientDesc[n]
-//   | uint32 bin_start[n][4096] | uint32 max_bin[n] | uint32 row_max[n][rows]
+//   | uint32 bin_start[n][4096] | uint32 max_bin[n] | uint16 row_max[n][rows]
 // bin_start: candidates of the client in the bins above this one; max_bin: candidates in its fullest bin.
 // tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths;
 // the first of them runs the length tuning and writes the result to all.
@@ -115,7 +116,7 @@ CVLC_HD constexpr size_t plan_off_desc(uint32_t n) { return align256(plan_off_ke
 CVLC_HD constexpr size_t plan_off_bin_start(uint32_t n) { return align256(plan_off_desc(n) + (size_t)n * sizeof(ClientDesc)); }
 CVLC_HD constexpr size_t plan_off_max_bin(uint32_t n) { return align256(plan_off_bin_start(n) + (size_t)n * CVLC_HIST_BINS * 4); }
 CVLC_HD constexpr size_t plan_off_row_max(uint32_t n) { return align256(plan_off_max_bin(n) + (size_t)n * 4); }
-CVLC_HD inline size_t plan_ws_bytes(const Partition& P, uint32_t n) { return align256(plan_off_row_max(n) + (size_t)P.total * 4); }
+CVLC_HD inline size_t plan_ws_bytes(const Partition& P, uint32_t n) { return align256(plan_off_row_max(n) + (size_t)P.total * 2); }
 
 // encode workspace header (first 256 bytes), written at the start of a call
 struct EncHeader {
@@ -186,12 +187,32 @@ CVLC_HD inline bool rank_shape(uint32_t nb, uint32_t max_bin, uint32_t thresh_bi
   r->sub_bits = k;
   return (fullest >> k) <= kRankItems && fullest < (1u << 24) && thresh_bin != 0;
 }
-// Rows a warp of the selection takes at a time: a small batch is spread over all warps, a large one asks a client's counter (one
-// answer in about 20 ns) less often.
-constexpr int kSelThreads = 768;
-CVLC_HD inline uint32_t select_group_rows(const Partition& P) {
+// Groups of rows that the warps of the selection take one at a time by a client's counter: three quarters of a client in large
+// groups, three quarters of the rest in groups a quarter as large, the last ones small, so that a block's warps finish about
+// together.  A counter answers about every 20 ns, so the fewer clients share the rows the larger are the groups (10 clients of
+// 100 M coordinates: 486 us with large groups of 4 pieces, 228 us with 25); with many clients small ones share out the dense
+// layers better (100 of 11.2 M: 880 us with 24 pieces, 674 us with 4).  A large group is at most an eighth of a warp's share of
+// the batch; a small batch is spread over all warps.
+constexpr int kSelThreads = 608;
+constexpr uint32_t kSelPiece = 128;  // rows whose maxima a warp loads at once (64 bits per lane)
+struct SelectGroups {
+  uint32_t pieces[2], count[2];  // large and middle groups: pieces in one, how many
+  uint32_t small, groups;        // rows of a small group; all groups
+};
+CVLC_HD inline SelectGroups select_groups(const Partition& P, uint32_t n) {
   const uint64_t per_warp = P.total / ((uint64_t)kNumSM * (kSelThreads / 32));
-  return per_warp < 32 ? 8u : (per_warp < 1024 ? 32u : 128u);
+  SelectGroups G;
+  const uint32_t want = 256 / n < 4 ? 4u : (256 / n > 32 ? 32u : 256 / n);
+  uint64_t pieces = per_warp / (8 * kSelPiece), left = P.rows;
+  if (pieces > want) pieces = want;
+  for (int l = 0; l < 2; ++l, pieces /= 4) {
+    G.pieces[l] = (uint32_t)pieces;
+    G.count[l] = pieces > 1 ? (uint32_t)(left * 3 / 4 / (pieces * kSelPiece)) : 0u;
+    left -= G.count[l] * pieces * kSelPiece;
+  }
+  G.small = per_warp < kSelPiece ? 32u : kSelPiece;
+  G.groups = G.count[0] + G.count[1] + (uint32_t)((left + G.small - 1) / G.small);
+  return G;
 }
 
 struct EncLayout {
@@ -302,8 +323,8 @@ __device__ __forceinline__ void pdl_enter() {
 
 // ---- launchers (one per translation unit) ---------------------------------------
 
-// Planning is launched in two parts.  The front (histogram, exponent fit, selection threshold, per-segment candidate
-// counts) is all the selection and ranking kernels need; the back (length tuning, copied to the clients that share a
+// Planning is launched in two parts.  The front (histogram, rows' maxima, exponent fit, selection threshold, the bins'
+// starts) is all the selection and ranking kernels need; the back (length tuning, copied to the clients that share a
 // tuning key) is only needed by the packing kernel, so it may run on another stream next to selection and ranking.
 cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
 // overlap: nothing but the planning front precedes it on the stream (no wait for an event)
@@ -326,7 +347,7 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
                                 cvlc_literal_plan_t* out, double* P_star, void* ws, cudaStream_t st);
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
 // ranking by partition (after the selection); returns at once on the device where the batch is ranked by digit passes
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, int index_bits, cudaStream_t st);
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into

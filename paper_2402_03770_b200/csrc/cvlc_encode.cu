@@ -316,27 +316,41 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
 // ===================================================================================
 // Groups of rows, every client with a counter of its own; a block keeps to one client while that has groups left, so that its
 // counts of the client's sub-buckets go out once.  Its warps work on their own: they take groups (the first one without asking)
-// and read the rows that hold a candidate (the histogram pass left the rows' maxima), eight at a time with the next eight on
-// their way in registers.  A step goes through shared memory so that every lane gets 16 consecutive coordinates: their flags are
-// then one word, and a lane's loop runs over its candidates only, which it appends to the warp's buffer.  When that is full the
-// warp counts its candidates per coarse bucket, reserves room in every bucket with one global addition and puts the candidates
-// there; they are also counted per sub-bucket where the client needs the partition.  The block that completes a client turns
-// those counts into offsets.  (One buffer per block, emptied by all its warps together, left them waiting for one another: 860 us
-// instead of SELECT_FIGURES.)
+// and read the rows that hold a candidate (the histogram pass left the rows' maxima), 32 at a time, while the next 32 are copied
+// to shared memory.  There every lane finds its row of 16 coordinates: their flags are one word.  In a step with few candidates
+// a lane's loop runs over its own, in one with many every coordinate is stored or not; either way they are appended to the warp's
+// buffer.  When that is full the warp counts its candidates per coarse bucket, reserves room in every bucket with one global
+// addition and puts the candidates there; they are also counted per sub-bucket where the client needs the partition.  The block
+// that completes a client turns those counts into offsets.
+// Bound by instruction issue (0.55 per scheduler and cycle).  100 clients of 11.2 M coordinates, 7 % candidates: 680 us; 50 of
+// 23.5 M, 3.5 %: 587; 10 of 100 M, 1 %: 229.  The copies go past the L1 (cp.async.cg): with loads into registers the warps were
+// bound by the L1 lines that shared memory leaves for loads in flight (832, 943 and 377 us), and more warps made it worse; asking
+// the L2 for 64 bytes instead of the 128 that it fetches by default takes 344 instead of 512 MB from DRAM for 8 of the second.
+// (One buffer per block, emptied by all its warps together, left them waiting for one another: 860 us for the first.)
 
 constexpr uint32_t kSelBuffer = 512;    // candidates in a warp's buffer: all of a step at least
-constexpr int kSelVec = 4;              // 128-bit loads per lane and step: eight rows
-constexpr uint32_t kSelRows = 2 * kSelVec;
-constexpr uint32_t kSelQueue = 64;      // rows a warp has found (ring)
+constexpr int kSelVec = 4;              // 128-bit loads per lane and step
+constexpr uint32_t kSelRows = 32;       // rows of a step
+constexpr uint32_t kSelDense = 96;      // a step with this many candidates takes each coordinate in turn, one with fewer only its candidates
+constexpr int kSelStages = 2;           // steps in shared memory: the current one and those on their way
+constexpr uint32_t kSelQueue = 256;     // rows a warp has found (ring)
 struct SelWarp {
   unsigned long long items[kSelBuffer];
-  float4 stage[kSelVec * 32];
+  float4 stage[kSelStages][kSelVec * 32];
   uint32_t cnt[kRankCoarse];            // counts, then next places (zero between)
   uint32_t queue[kSelQueue];
 };
 constexpr size_t kSelSmem = (kSelThreads / 32) * sizeof(SelWarp) + ((size_t)kRankCoarse + kRankSubs) * 4;
-static_assert(kRowUnits == 16 && kSelRows - 1 + 32 <= kSelQueue, "two rows per warp-wide load; the ring holds a group and a rest");
+static_assert(kRowUnits == kSelVec && kSelRows - 1 + kSelPiece <= kSelQueue, "a row per lane and step; the ring holds a piece and a rest");
 static_assert(kSelVec * 128 <= kSelBuffer && kSelSmem <= 227 * 1024, "shared memory");
+
+// inclusive sums over the lanes
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t v) {
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1)
+    asm volatile("{.reg .pred p; .reg .b32 o; shfl.sync.up.b32 o|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, o;}" : "+r"(v) : "r"(off));
+  return v;
+}
 
 // red.add of four fp32 counts at once: counts stay below 2^24 in this mode (see rank_shape), where they are exact
 __device__ __forceinline__ void add_counts4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t e) {
@@ -357,7 +371,9 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   if (hdr->lsd != kRankPartition) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = batch.n;
-  const uint32_t rows = (uint32_t)part.rows, group_rows = select_group_rows(part), groups = (rows + group_rows - 1) / group_rows;
+  const uint32_t rows = (uint32_t)part.rows, held_rows = ((uint32_t)(d >> 2) + kRowUnits - 1) / kRowUnits;  // with coordinates
+  const SelectGroups sg = select_groups(part, n);
+  const uint32_t groups = sg.groups;
   const uint32_t nvec = (uint32_t)(d >> 2);
   uint32_t* group_next = reinterpret_cast<uint32_t*>(ws + L.off_group_next);
   uint32_t* group_done = reinterpret_cast<uint32_t*>(ws + L.off_group_done);
@@ -393,8 +409,8 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     const ClientRank r = reinterpret_cast<const ClientRank*>(ws + L.off_rank)[c];
     const float* __restrict__ x = batch.c[c].x;
     const float4* __restrict__ xv = reinterpret_cast<const float4*>(x);
-    const uint32_t* __restrict__ row_max = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_row_max(n)) + (size_t)c * rows;
-    const uint32_t thresh = batch.c[c].plan->thresh_bin << 19, keytop = r.keytop;  // thresh > 0 in this mode
+    const uint16_t* __restrict__ row_max = reinterpret_cast<const uint16_t*>(plan_ws + plan_off_row_max(n)) + (size_t)c * rows;
+    const uint32_t thresh_bin = batch.c[c].plan->thresh_bin, thresh = thresh_bin << 19, keytop = r.keytop;  // thresh > 0 in this mode
     const float below_thresh = __uint_as_float(thresh - 1u);                        // key >= thresh <=> |x| > below_thresh
     const uint32_t sh_coarse = 19 + r.group, sh_sub = sh_coarse - r.sub_bits;
     unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
@@ -403,20 +419,25 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
       const uint32_t* __restrict__ bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS;
       for (uint32_t i = tid; i < r.n_coarse; i += kSelThreads) s_start[i] = coarse_start(r, bin_start, i);
     }
-    const uint32_t inv_max = keytop - thresh;
-    auto inv_of = [&](uint32_t key) -> uint32_t {  // always inside the client's buckets
-      const uint32_t inv = keytop - (key < keytop ? key : keytop);
-      return inv < inv_max ? inv : inv_max;
-    };
+    auto inv_of = [&](uint32_t key) -> uint32_t { return keytop - (key < keytop ? key : keytop); };  // key >= thresh: inside the buckets
     uint32_t held = 0;  // candidates in the warp's buffer
     auto flush = [&]() {  // to their buckets
-      for (uint32_t i = lane; i < held; i += 32) {
-        const uint32_t key = (uint32_t)(sw.items[i] >> 32);
-        if (key > keytop) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);  // the update is not the plan's
-        const uint32_t inv = inv_of(key);
-        atomicAdd(sw.cnt + (inv >> sh_coarse), 1u);
-        if (r.split) atomicAdd(s_sub + (inv >> sh_sub), 1u);
+      bool above = false;
+      for (uint32_t i = lane; i < held; i += 128) {  // four at a time: their loads, then their additions
+        uint32_t key[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) key[u] = i + 32 * u < held ? (uint32_t)(sw.items[i + 32 * u] >> 32) : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (i + 32 * u < held) {
+            above |= key[u] > keytop;
+            const uint32_t inv = inv_of(key[u]);
+            atomicAdd(sw.cnt + (inv >> sh_coarse), 1u);
+            if (r.split) atomicAdd(s_sub + (inv >> sh_sub), 1u);
+          }
+        }
       }
+      if (above) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);  // the update is not the plan's
       __syncwarp();
       for (uint32_t i0 = lane; i0 < r.n_coarse; i0 += 128) {
         uint32_t v[4];
@@ -430,10 +451,17 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
           if (v[u]) sw.cnt[i0 + 32 * u] = s_start[i0 + 32 * u] + at[u];
       }
       __syncwarp();
-      for (uint32_t i = lane; i < held; i += 32) {
-        const unsigned long long item = sw.items[i];
-        const uint32_t p = atomicAdd(sw.cnt + (inv_of((uint32_t)(item >> 32)) >> sh_coarse), 1u);
-        if (p < r.n) out[p] = item;
+      for (uint32_t i = lane; i < held; i += 128) {
+        unsigned long long item[4];
+        uint32_t p[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) item[u] = i + 32 * u < held ? sw.items[i + 32 * u] : 0ull;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          p[u] = i + 32 * u < held ? atomicAdd(sw.cnt + (inv_of((uint32_t)(item[u] >> 32)) >> sh_coarse), 1u) : 0xFFFFFFFFu;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (p[u] < r.n) out[p[u]] = item[u];
       }
       __syncwarp();
       for (uint32_t i = lane; i < r.n_coarse; i += 32) sw.cnt[i] = 0;
@@ -442,9 +470,9 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     };
 
     __syncthreads();  // the buckets' starts are there
-    // ---- the warp's groups: the maxima of the next one are on their way, and so is the number of the one after it
-    uint32_t taken = 0, group = 0, group2 = 0, maximum = 0, piece = 0;  // piece: 32 rows of the group
-    const uint32_t pieces = group_rows > 32 ? group_rows / 32 : 1;
+    // ---- the warp's groups, piece after piece: the maxima of the next two pieces are on their way, and so is the number of the
+    // group after the last one asked for
+    uint32_t taken = 0, group = 0, group2 = 0, piece = 0;
     const uint32_t dynamic = given(c);  // first group that goes by the counter
     if (visit == 0) {
       group = (blockIdx.x - first_block(c)) * (kSelThreads / 32) + warp;
@@ -453,20 +481,50 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
       group = __shfl_sync(kFull, group, 0);
     }
     if (lane == 0) group2 = dynamic + atomicAdd(group_next + c, 1u);
-    auto maxima_of = [&](uint32_t g, uint32_t p) -> uint32_t {
-      const uint32_t row = g * group_rows + p * 32 + lane;
-      return (g < groups && (uint32_t)lane < group_rows && row < rows) ? __ldg(row_max + row) : 0u;
+    struct Piece {
+      uint32_t row, end;  // [row, end): none left where row = end
+      uint2 maxima;       // lane l: rows row + 4 l .. row + 4 l + 3
     };
-    maximum = maxima_of(group, 0);
+    auto next_piece = [&]() -> Piece {
+      Piece p{0u, 0u, make_uint2(0u, 0u)};
+      if (group >= groups) return p;
+      uint32_t pieces = 1;
+      if (group < sg.count[0]) {
+        pieces = sg.pieces[0];
+        p.row = (group * pieces + piece) * kSelPiece;
+      } else if (group < sg.count[0] + sg.count[1]) {
+        pieces = sg.pieces[1];
+        p.row = (sg.count[0] * sg.pieces[0] + (group - sg.count[0]) * pieces + piece) * kSelPiece;
+      } else {
+        p.row = (sg.count[0] * sg.pieces[0] + sg.count[1] * sg.pieces[1]) * kSelPiece + (group - sg.count[0] - sg.count[1]) * sg.small;
+      }
+      p.end = p.row + (group < sg.count[0] + sg.count[1] ? kSelPiece : sg.small);
+      ++piece;
+      if (p.row + 4 * (uint32_t)lane < (p.end < rows ? p.end : rows)) p.maxima = __ldg(reinterpret_cast<const uint2*>(row_max + p.row) + lane);
+      if (piece == pieces) {
+        ++taken;
+        piece = 0;
+        group = __shfl_sync(kFull, group2, 0);
+        if (lane == 0 && group < groups) group2 = dynamic + atomicAdd(group_next + c, 1u);
+      }
+      return p;
+    };
+    Piece now = next_piece(), then = next_piece();
     uint32_t* queue = sw.queue;
     uint32_t head = 0, tail = 0;
-    float4 nf[kSelVec];
-    uint32_t next_row = 0;  // the row in which this lane's coordinates of the next step lie
-    static_assert(kSelVec == 4, "a lane's 16 coordinates are a quarter of a row");
-    auto request = [&]() -> uint32_t {  // asks for the next rows that hold a candidate; returns how many there are
-      while (tail - head < kSelRows && group < groups) {
-        const uint32_t row = group * group_rows + piece * 32 + lane, mx = maximum;
-        if (group + 1 == groups && piece == 0 && lane < (int)(d & 3)) {  // the client's ragged tail goes with its last group: straight to its buckets
+    uint32_t slot = 0;                         // stage that the next step goes to
+    bool ragged = false;                       // the last row has been listed
+    uint32_t step_row[kSelStages], step_rows[kSelStages];  // per step, the oldest first: this lane's row; rows
+    static_assert(kSelVec == 4, "a lane's 16 coordinates are a row");
+    // Staging layout: float4 g of a step (in memory order) sits in slot g ^ ((g >> 3) & 3): what a warp's copies write (consecutive g)
+    // and its loads (lane l reads 4 l .. 4 l + 3) are then both free of bank conflicts.
+    const uint32_t stage0 = (uint32_t)__cvta_generic_to_shared(sw.stage[0]);
+    auto request = [&](uint32_t& my_row) -> uint32_t {  // asks for the next rows that hold a candidate; returns how many there are
+      while (tail - head < kSelRows && now.row < now.end) {
+        const Piece p = now;
+        now = then;
+        then = next_piece();
+        if (p.end >= rows && lane < (int)(d & 3)) {  // the client's ragged tail goes with its last piece: straight to its buckets
           const uint32_t b = __float_as_uint(x[(uint64_t)nvec * 4 + lane]), key = b & 0x7FFFFFFFu;
           if (key >= thresh) {
             if (key > keytop) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
@@ -476,77 +534,96 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
             if (p < r.n) out[p] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | (nvec * 4 + (uint32_t)lane));
           }
         }
-        if (++piece == pieces) {
-          ++taken;
-          piece = 0;
-          group = __shfl_sync(kFull, group2, 0);
-          if (lane == 0 && group < groups) group2 = dynamic + atomicAdd(group_next + c, 1u);
+        // bins are 12 bits: the top bit of a half survives the subtraction where the row's bin reaches the threshold's
+        uint32_t h01 = (p.maxima.x | 0x80008000u) - thresh_bin * 0x10001u, h23 = (p.maxima.y | 0x80008000u) - thresh_bin * 0x10001u;
+        const uint32_t row = p.row + 4 * (uint32_t)lane;
+        if (p.end - p.row < kSelPiece || p.end >= held_rows) {  // not every lane has rows
+          const uint32_t end = p.end < held_rows ? p.end : held_rows;
+          h01 &= (row < end ? 0x8000u : 0u) | (row + 1 < end ? 0x80000000u : 0u);
+          h23 &= (row + 2 < end ? 0x8000u : 0u) | (row + 3 < end ? 0x80000000u : 0u);
+          ragged |= p.end >= held_rows;
         }
-        maximum = maxima_of(group, piece);
-        const unsigned m = __ballot_sync(kFull, mx >= thresh);  // mx = 0 past the last row
-        if (mx >= thresh) queue[(tail + __popc(m & ((1u << lane) - 1u))) & (kSelQueue - 1)] = row;
-        tail += __popc(m);
+        if (!__any_sync(kFull, ((h01 | h23) & 0x80008000u) != 0)) continue;
+        auto list = [&](bool hit, uint32_t which) {
+          const unsigned hits = __ballot_sync(kFull, hit);
+          if (hit) queue[(tail + __popc(hits & ((1u << lane) - 1u))) & (kSelQueue - 1)] = which;
+          tail += __popc(hits);
+        };
+        list(h01 & 0x8000u, row);
+        list(h01 & 0x80000000u, row + 1);
+        list(h23 & 0x8000u, row + 2);
+        list(h23 & 0x80000000u, row + 3);
         __syncwarp();
       }
       const uint32_t have = tail - head < kSelRows ? tail - head : kSelRows;
+      my_row = queue[(head + lane) & (kSelQueue - 1)];
+      const bool whole = have == kSelRows && !ragged;
 #pragma unroll
-      for (int v = 0; v < kSelVec; ++v) {
-        const uint32_t slot = 2 * v + (lane >> 4);
-        const uint32_t unit = queue[(head + slot) & (kSelQueue - 1)] * kRowUnits + (lane & 15);
-        nf[v] = make_float4(0.f, 0.f, 0.f, 0.f);  // no candidate
-        if (slot < have && unit < nvec) nf[v] = __ldg(xv + unit);
+      for (int v = 0; v < kSelVec; ++v) {  // four neighbouring lanes fetch a row
+        const uint32_t i = 8 * v + (lane >> 2), g = v * 32 + lane;
+        const uint32_t unit = __shfl_sync(kFull, my_row, i) * kRowUnits + (lane & 3);
+        const uint32_t to = stage0 + (slot * (kSelVec * 32) + (g ^ ((g >> 3) & 3u))) * 16;
+        if (whole) {
+          asm volatile("cp.async.cg.shared.global.L2::64B [%0], [%1], 16;" ::"r"(to), "l"(xv + unit) : "memory");
+        } else {
+          const bool on = i < have && unit < nvec;  // else zeros: no candidates
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(xv + (on ? unit : 0u)), "r"(on ? 16 : 0) : "memory");
+        }
       }
-      next_row = queue[(head + (lane >> 2)) & (kSelQueue - 1)];
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      slot = slot + 1 == kSelStages ? 0 : slot + 1;
       head += have;
       __syncwarp();
       return have;
     };
-    // Staging layout: float4 g of a step (in memory order) sits in slot g ^ ((g >> 3) & 3): the stores of a warp (consecutive g) and
-    // its loads (lane l reads 4 l .. 4 l + 3) are then both free of bank conflicts.
-    float4* stage = sw.stage;
     const uint32_t ct = ((uint32_t)lane >> 1) & 3u;
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(stage) + 16 * lane;
-    uint32_t pending = request();
-    uint32_t m = 0, first = 0;  // flags of this lane's coordinates, lowest index in bit 15; index of the first one
-    auto advance = [&]() -> bool {
-      if (pending == 0) return false;
+    const uint32_t word_of = 15u ^ (ct << 2);
+    uint32_t cur = 0;  // stage of the current step
+#pragma unroll
+    for (int i = 0; i + 1 < kSelStages; ++i) step_rows[i] = request(step_row[i]);
+    while (step_rows[0]) {
       __syncwarp();  // the step before has been read
-#pragma unroll
-      for (int v = 0; v < kSelVec; ++v) {
-        const uint32_t g = (uint32_t)(v * 32 + lane);
-        stage[g ^ ((g >> 3) & 3u)] = nf[v];
-      }
-      first = next_row * (4 * kRowUnits) + (lane & 3) * 16;
-      pending = request();
+      step_rows[kSelStages - 1] = request(step_row[kSelStages - 1]);
+      asm volatile("cp.async.wait_group %0;" ::"n"(kSelStages - 1) : "memory");
       __syncwarp();
-      m = 0;
+      const float4* stage = sw.stage[cur];
+      const uint32_t* words = reinterpret_cast<const uint32_t*>(stage) + 16 * lane;
+      cur = cur + 1 == kSelStages ? 0 : cur + 1;
+      const uint32_t first = step_row[0] * (4 * kRowUnits);
+      uint32_t m = 0;  // flags of this lane's coordinates, lowest index in bit 15
+      uint32_t bits[16];
 #pragma unroll
-      for (uint32_t j = 0; j < 4; ++j) {  // the difference of two distinct floats never rounds to zero: its sign is the flag
+      for (uint32_t j = 0; j < 4; ++j) {
         const float4 f = stage[4 * lane + (j ^ ct)];
-        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.x))), m, 1);
-        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.y))), m, 1);
-        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.z))), m, 1);
-        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(f.w))), m, 1);
+        bits[4 * j] = __float_as_uint(f.x);
+        bits[4 * j + 1] = __float_as_uint(f.y);
+        bits[4 * j + 2] = __float_as_uint(f.z);
+        bits[4 * j + 3] = __float_as_uint(f.w);
       }
-      return true;
-    };
-    while (advance()) {
-      const uint32_t cnt = __popc(m);
-      uint32_t incl = cnt;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t o = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += o;
+      for (int j = 0; j < 16; ++j)  // the difference of two distinct floats never rounds to zero: its sign is the flag
+        m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(__uint_as_float(bits[j])))), m, 1);
+#pragma unroll
+      for (int i = 0; i + 1 < kSelStages; ++i) {
+        step_row[i] = step_row[i + 1];
+        step_rows[i] = step_rows[i + 1];
       }
+      const uint32_t cnt = __popc(m);
+      const uint32_t incl = warp_inclusive(cnt);
       const uint32_t total = __shfl_sync(kFull, incl, 31);
       if (held + total > kSelBuffer) flush();
       unsigned long long* o = sw.items + held + incl - cnt;
-      while (m) {
-        const int hb = 31 - __clz(m);  // highest flag = lowest index first
-        m ^= 1u << hb;
-        const uint32_t c16 = 15u - (uint32_t)hb;
-        const uint32_t b = words[c16 ^ (ct << 2)];
-        *o++ = ((unsigned long long)(b & 0x7FFFFFFFu) << 32) | (unsigned long long)((b & 0x80000000u) | (first + c16));
+      if (total >= kSelDense) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (m & (1u << (15 - j))) *o++ = ((unsigned long long)(bits[j] & 0x7FFFFFFFu) << 32) | (unsigned long long)((bits[j] & 0x80000000u) | (first + j));
+      } else {
+        while (m) {
+          const int hb = 31 - __clz(m);  // highest flag = lowest index first
+          m ^= 1u << hb;
+          const uint32_t b = words[hb ^ word_of];
+          *o++ = ((unsigned long long)(b & 0x7FFFFFFFu) << 32) | (unsigned long long)((b & 0x80000000u) | (first + 15 - hb));
+        }
       }
       held += total;
     }
@@ -1350,10 +1427,10 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st);
   const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (pws) {
-    const uint64_t want = (part.rows + select_group_rows(part) - 1) / select_group_rows(part) * n;
+    const uint64_t want = (uint64_t)select_groups(part, n).groups * n;
     const unsigned grid = (unsigned)(want < (uint64_t)kNumSM ? want : kNumSM);
     launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, pws, w, L);
-    e = launch_rank(batch, L, pws, w, (int)shape.s, st);
+    e = launch_rank(batch, L, pws, w, st);
     if (e != cudaSuccess) return e;
   } else {
     const uint64_t want = select_tiles_of(shape.d, kSelectThreads) * n;

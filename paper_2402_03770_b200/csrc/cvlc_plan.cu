@@ -36,7 +36,7 @@ __device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
 
 __global__ void __launch_bounds__(kHistThreads, 2)
 k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
-       unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint32_t* __restrict__ row_max_all) {
+       unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint16_t* __restrict__ row_max_all) {
   extern __shared__ uint32_t sh_hist[];  // [kHistSub][4096]
   pdl_enter();
   for (int i = threadIdx.x; i < kHistSub * CVLC_HIST_BINS; i += kHistThreads) sh_hist[i] = 0;
@@ -56,30 +56,8 @@ k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
     const float* __restrict__ x = batch.c[c].x;
     const float4* xv = reinterpret_cast<const float4*>(x);
     const uint64_t v1 = (u1 < nvec) ? u1 : nvec;  // float4 units of this segment: [u0, v1)
-    // largest key of every row (a warp-wide load covers 32 / kRowUnits of them); one whole-warp reduction per row of a load,
-    // each seeing that row's keys only
-    uint32_t* __restrict__ row_max = row_max_all + c * part.rows;
-    static_assert(32 % kRowUnits == 0, "a warp-wide load covers whole rows");
-    constexpr int kRowsPerLoad = 32 / kRowUnits;
-    const int my_group = lane / kRowUnits;
-    auto row_maxima = [&](uint32_t mk) -> uint32_t {  // the largest key among the lanes of this lane's row
-      if constexpr (kRowsPerLoad <= 2) {  // few rows per load: one whole-warp reduction per row, each seeing that row's keys only
-        uint32_t mine = 0;
-#pragma unroll
-        for (int g = 0; g < kRowsPerLoad; ++g) {
-          const uint32_t mg = __reduce_max_sync(0xFFFFFFFFu, my_group == g ? mk : 0u);
-          if (my_group == g) mine = mg;
-        }
-        return mine;
-      } else {  // more rows per load: a butterfly inside the row's lanes
-#pragma unroll
-        for (int off = 1; off < kRowUnits; off <<= 1) {
-          const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, mk, off);
-          mk = o > mk ? o : mk;
-        }
-        return mk;
-      }
-    };
+    uint16_t* __restrict__ row_max = row_max_all + c * part.rows;
+    static_assert(kRowUnits == 4, "a row is held by four neighbouring lanes");
     uint32_t top = 0;
     uint64_t v = u0 + threadIdx.x;
     // four independent 128-bit loads in flight per thread; the loop condition is the same for the lanes of a warp
@@ -87,18 +65,27 @@ k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
       float4 a[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) a[u] = __ldg(xv + v + u * kHistThreads);
+      uint32_t m[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const uint32_t m = row_maxima(hist_add4(my, a[u]));
-        top = m > top ? m : top;
-        if (lane % kRowUnits == 0) row_max[(v + u * kHistThreads) / kRowUnits] = m;
+        m[u] = hist_add4(my, a[u]);
+        top = m[u] > top ? m[u] : top;
       }
+      // The rows' maxima of the four loads, two bins to a word: the first exchange leaves an even lane with loads 0 and 1, an odd
+      // lane with 2 and 3, the second completes the rows; each lane then stores one of its row's four.
+      const uint32_t w01 = m[0] >> 19 | (m[1] >> 3 & 0xFFFF0000u), w23 = m[2] >> 19 | (m[3] >> 3 & 0xFFFF0000u);
+      uint32_t w = __vmaxu2(lane & 1 ? w23 : w01, __shfl_xor_sync(0xFFFFFFFFu, lane & 1 ? w01 : w23, 1));
+      w = __vmaxu2(w, __shfl_xor_sync(0xFFFFFFFFu, w, 2));
+      const uint32_t load = ((lane & 1) << 1) | (lane >> 1 & 1);
+      row_max[(v + load * kHistThreads) / kRowUnits] = (uint16_t)(lane & 2 ? w >> 16 : w);
     }
     for (; v - lane < v1; v += kHistThreads) {  // rows that may end inside the warp
       const bool on = v < v1;
-      const uint32_t m = row_maxima(on ? hist_add4(my, __ldg(xv + v)) : 0u);
+      uint32_t m = on ? hist_add4(my, __ldg(xv + v)) : 0u;
       top = m > top ? m : top;
-      if (lane % kRowUnits == 0 && on) row_max[v / kRowUnits] = m;
+      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+      if (lane % kRowUnits == 0 && on) row_max[v / kRowUnits] = (uint16_t)(m >> 19);
     }
     // ragged tail of the client (d not a multiple of 4)
     if (seg_end == (c + 1) * part.rows && threadIdx.x < (d & 3)) {
@@ -310,7 +297,7 @@ __device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, d
   }
 }
 
-// K2a  per client: survival counts, exponent fit, the threshold bin of the selection and the candidates per segment.
+// K2a  per client: survival counts, exponent fit, the threshold bin of the selection and where each bin's candidates start.
 // Everything here depends on the histogram alone.  The number of transmitted coordinates k is not known before the
 // lengths are tuned, but it never exceeds k_sel = R * cap(shortest candidate length) (every packet at the shortest
 // code; with a fixed length, exactly R * cap(y)), so the selection keeps every coordinate down to the bin that holds
@@ -1320,7 +1307,7 @@ static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(w + kPlanWsHist);
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   const Partition part = make_partition(shape.d, n);
-  uint32_t* row_max = reinterpret_cast<uint32_t*>(w + plan_off_row_max(n));
+  uint16_t* row_max = reinterpret_cast<uint16_t*>(w + plan_off_row_max(n));
   // header, histograms, flags and tuning keys start at zero; the rest is written in full by the kernels that follow
   const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), 0, 0, st);
   // two resident blocks per SM share the concatenated updates evenly

@@ -121,24 +121,19 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
 // ===================================================================================
 
 struct RankShared {
-  u64 items[kRankItems + 2];  // inv << 32 | index << shift | sign: all distinct, ordered like the ranks
+  u64 items[kRankItems + 2];  // values (see to_value): all distinct, ordered like the ranks
   uint32_t zero[4];           // cell[-1] = 0: where the first cell starts
   uint32_t cell[kCells];      // counts, then starts, then (after placing) ends of the cells
 };
 
-// A candidate as a value to rank: inv in the high word; in the low word the index, moved up to the top bit so that equal keys
-// spread over the whole word, above the sign.
-struct ValueFormat {
-  uint32_t keytop;
-  int shift;  // 32 - bits of an index, at least 1
-};
-__device__ __forceinline__ u64 to_value(u64 item, const ValueFormat& f) {
+// A candidate as a value to rank: the key's complement in the high word, index << 1 | sign in the low word.
+__device__ __forceinline__ u64 to_value(u64 item) {
   const uint32_t lo = (uint32_t)item;
-  return ((u64)inv_of(item, f.keytop) << 32) | (u64)((lo << f.shift) | lo >> 31);
+  return ((u64)~(uint32_t)(item >> 32) << 32) | (u64)__funnelshift_l(lo, lo, 1);
 }
-__device__ __forceinline__ u64 to_item(u64 value, const ValueFormat& f) {
+__device__ __forceinline__ u64 to_item(u64 value) {
   const uint32_t lo = (uint32_t)value;
-  return ((u64)(f.keytop - (uint32_t)(value >> 32)) << 32) | (u64)(lo >> f.shift | lo << 31);
+  return ((u64)~(uint32_t)(value >> 32) << 32) | (u64)__funnelshift_r(lo, lo, 1);
 }
 
 // exclusive scan of the cells in place by the whole block; returns the total
@@ -218,9 +213,9 @@ __device__ __forceinline__ void bitonic_sort(u64* items, uint32_t n, uint32_t t0
 }
 
 // by the whole block: sorts items[0 .. n) and writes them out
-__device__ __noinline__ void rank_by_block(u64* items, uint32_t n, u64* __restrict__ out, ValueFormat fmt) {
+__device__ __noinline__ void rank_by_block(u64* items, uint32_t n, u64* __restrict__ out) {
   bitonic_sort(items, n, threadIdx.x, kRankThreads, [] { __syncthreads(); });
-  for (uint32_t i = threadIdx.x; i < n; i += kRankThreads) out[i] = to_item(items[i], fmt);
+  for (uint32_t i = threadIdx.x; i < n; i += kRankThreads) out[i] = to_item(items[i]);
   __syncthreads();
 }
 
@@ -232,7 +227,7 @@ struct Cut {
   u64 value;
   uint32_t below;
 };
-__device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t x, ValueFormat fmt) {
+__device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t x) {
   __shared__ uint32_t s_cell, s_below, s_count;
   const int tid = threadIdx.x;
   Cut cut{lo, 0};
@@ -243,7 +238,7 @@ __device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src,
     if (tid == 0) s_cell = s_below = s_count = 0;
     __syncthreads();
     for (uint32_t i = tid; i < m; i += kRankThreads) {
-      const u64 v = to_value(src[i], fmt);
+      const u64 v = to_value(src[i]);
       if (v >= lo && v < hi) atomicAdd(&s.cell[(uint32_t)((v - lo) >> sh)], 1u);
     }
     __syncthreads();
@@ -272,15 +267,15 @@ __device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src,
 
 // Ranks a .. b (about) of a bucket that a block cannot hold, m values in [lo, hi): equal or nearly equal keys.  src and out differ.
 __device__ __noinline__ void rank_part(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t a, uint32_t b,
-                                       u64* __restrict__ out, ValueFormat fmt) {
+                                       u64* __restrict__ out) {
   __shared__ uint32_t s_n;
   const int tid = threadIdx.x;
-  const Cut from = a == 0 ? Cut{lo, 0} : cut_near(s, src, m, lo, hi, a, fmt);
-  const Cut to = b >= m ? Cut{hi, m} : cut_near(s, src, m, lo, hi, b, fmt);
+  const Cut from = a == 0 ? Cut{lo, 0} : cut_near(s, src, m, lo, hi, a);
+  const Cut to = b >= m ? Cut{hi, m} : cut_near(s, src, m, lo, hi, b);
   if (tid == 0) s_n = 0;
   __syncthreads();
   for (uint32_t i = tid; i < m; i += kRankThreads) {
-    const u64 v = to_value(src[i], fmt);
+    const u64 v = to_value(src[i]);
     if (v >= from.value && v < to.value) {
       const uint32_t p = atomicAdd(&s_n, 1u);
       if (p < kRankItems) s.items[p] = v;
@@ -289,12 +284,12 @@ __device__ __noinline__ void rank_part(RankShared& s, const u64* __restrict__ sr
   __syncthreads();
   const uint32_t got = s_n < kRankItems ? s_n : kRankItems;  // at most a window and kCutRest
   __syncthreads();
-  rank_by_block(s.items, got, out + from.below, fmt);
+  rank_by_block(s.items, got, out + from.below);
 }
 
 // Cells of equal or nearly equal keys (a layer's clipped outliers, values on a grid), first item | items << 16: every warp sorts
 // some of them, the block the largest.
-__device__ __noinline__ void rank_big_cells(RankShared& s, const uint32_t* big, uint32_t n_big, u64* __restrict__ out, ValueFormat fmt) {
+__device__ __noinline__ void rank_big_cells(RankShared& s, const uint32_t* big, uint32_t n_big, u64* __restrict__ out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool any_huge = false;
   for (uint32_t g = 0; g < n_big; ++g) any_huge |= (big[g] >> 16) > kWarpCell;
@@ -302,18 +297,18 @@ __device__ __noinline__ void rank_big_cells(RankShared& s, const uint32_t* big, 
     const uint32_t b0 = big[g] & 0xFFFFu, n = big[g] >> 16;
     if (n > kWarpCell) continue;
     bitonic_sort(s.items + b0, n, lane, 32, [] { __syncwarp(); });
-    for (uint32_t i = lane; i < n; i += 32) out[b0 + i] = to_item(s.items[b0 + i], fmt);
+    for (uint32_t i = lane; i < n; i += 32) out[b0 + i] = to_item(s.items[b0 + i]);
   }
   __syncthreads();
   if (any_huge)
     for (uint32_t g = 0; g < n_big; ++g)
-      if ((big[g] >> 16) > kWarpCell) rank_by_block(s.items + (big[g] & 0xFFFFu), big[g] >> 16, out + (big[g] & 0xFFFFu), fmt);
+      if ((big[g] >> 16) > kWarpCell) rank_by_block(s.items + (big[g] & 0xFFFFu), big[g] >> 16, out + (big[g] & 0xFFFFu));
 }
 
 // Ranks m <= kRankItems items whose inv lies in [base, base + span]: spread over kCells equal ranges of inv, about one item per
 // cell, then compared with the others of their cell.  `meanwhile` is run once all threads have passed a barrier.
 template <class Meanwhile>
-__device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, const ValueFormat& fmt,
+__device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
                                              Meanwhile&& meanwhile) {
   __shared__ uint32_t s_n_big, s_big[kRankItems / kCompareAll];  // cells beyond kCompareAll
   const int tid = threadIdx.x;
@@ -330,7 +325,7 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
   }
   __syncthreads();
   const int csh = span < kCells ? 0 : 32 - __clz(span) - (int)kCellBits;  // span >> csh below kCells
-  const uint32_t top = fmt.keytop - base;
+  const uint32_t top = keytop - base;
   auto cell_of_key = [&](uint32_t key) -> uint32_t {
     const uint32_t k = (top - key) >> csh;
     return k < kCells ? k : kCells - 1;
@@ -341,7 +336,7 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
   for (uint32_t i = tid + kHold * kRankThreads; i < m; i += kRankThreads) atomicAdd(&s.cell[cell_of_key((uint32_t)(src[i] >> 32))], 1u);
   __syncthreads();
   scan_cells(s.cell);
-  auto put = [&](u64 item) { s.items[atomicAdd(&s.cell[cell_of_key((uint32_t)(item >> 32))], 1u)] = to_value(item, fmt); };
+  auto put = [&](u64 item) { s.items[atomicAdd(&s.cell[cell_of_key((uint32_t)(item >> 32))], 1u)] = to_value(item); };
 #pragma unroll
   for (int u = 0; u < kHold; ++u)
     if ((uint32_t)tid + u * kRankThreads < m) put(it[u]);
@@ -350,7 +345,7 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
   meanwhile();
   for (uint32_t p = tid; p < m; p += kRankThreads) {
     const u64 v = s.items[p];
-    uint32_t k = ((uint32_t)(v >> 32) - base) >> csh;
+    uint32_t k = ((uint32_t)(v >> 32) - ~top) >> csh;
     k = k < kCells ? k : kCells - 1;
     const uint32_t e1 = s.cell[k], e0 = (&s.cell[k])[-1];  // the places have advanced to the cells' ends
     uint32_t rank = p;
@@ -366,17 +361,17 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
         rank += (a < v ? 1u : 0u) + ((q + 1 < e1 && b < v) ? 1u : 0u);
       }
     }
-    out[rank] = to_item(v, fmt);
+    out[rank] = to_item(v);
   }
   __syncthreads();
-  if (s_n_big) rank_big_cells(s, s_big, s_n_big, out, fmt);
+  if (s_n_big) rank_big_cells(s, s_big, s_n_big, out);
 }
 
 // Tile t of a client: the buckets (sub-buckets after a partition) that start in [t window, (t + 1) window), at most the window
 // plus one bucket; of a bucket that a block cannot hold the ranks that lie in the window, whether it starts there or before.
-// RANK_FIGURES
+// 79 M candidates of 100 clients: 755 us, 1.7 TB/s of candidates in and out; bound by issue and by the barriers of a tile.
 __global__ void __launch_bounds__(kRankThreads, 2)
-k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, int index_bits) {
+k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   RankShared& s = *reinterpret_cast<RankShared*>(s_raw);
   // per slot: ticket; first bucket at or behind the window's start and end; where those start; where the bucket before the first starts
@@ -425,7 +420,6 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
     if (tid == 0) s_ticket[slot ^ 1u] = atomicAdd(&hdr->rank_ticket, 1u);
     const uint32_t tile = t / n, c = t - tile * n;
     const ClientRank r = rank[c];
-    const ValueFormat fmt{r.keytop, 32 - index_bits};
     const uint32_t sh = 19 + r.group - (r.split ? r.sub_bits : 0u);
     bool searched = false;
     auto next_search = [&]() {  // behind a barrier that follows the ticket
@@ -436,10 +430,11 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
     const u64* from = reinterpret_cast<const u64*>(ws + (r.split ? L.off_buf_b : L.off_buf_a)) + (size_t)c * L.capacity;
     u64* into = reinterpret_cast<u64*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
     auto part_of = [&](uint32_t bucket, uint32_t first, uint32_t end) {  // the window's part of a large bucket
-      const u64 lo = ((u64)bucket << sh) << 32, hi = ((u64)(bucket + 1) << sh) << 32;
+      const u64 lo = ((u64)~r.keytop + ((u64)bucket << sh)) << 32, end_high = (u64)~r.keytop + ((u64)(bucket + 1) << sh);
+      const u64 hi = end_high >> 32 ? ~0ull : end_high << 32;  // the last bucket may reach below key 0
       const uint32_t a = x0 > first ? (uint32_t)(x0 - first) : 0u;
       const uint32_t b = x1 < end ? (uint32_t)(x1 - first) : end - first;
-      rank_part(s, from + first, end - first, lo, hi, a, b, into + first, fmt);
+      rank_part(s, from + first, end - first, lo, hi, a, b, into + first);
     };
     uint32_t b_lo = s_bucket[slot][0], at = s_start[slot][0];
     const uint32_t b_end = s_bucket[slot][1], at_end = s_start[slot][1];
@@ -454,18 +449,20 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
       if (to - at > kRankItems) {
         if (r.split) part_of(b_lo, at, to);
       } else if (to > at) {
-        rank_buckets(s, from + at, to - at, b_lo << sh, (uint32_t)(((u64)b_hi << sh) - ((u64)b_lo << sh) - 1), into + at, fmt, next_search);
+        rank_buckets(s, from + at, to - at, b_lo << sh, (uint32_t)(((u64)b_hi << sh) - ((u64)b_lo << sh) - 1), into + at, r.keytop, next_search);
       }
       b_lo = b_hi;
       at = to;
     }
-    __syncthreads();
-    next_search();
+    if (!searched) {
+      __syncthreads();
+      next_search();
+    }
     __syncthreads();
   }
 }
 
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, int index_bits, cudaStream_t st) {
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, cudaStream_t st) {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -479,8 +476,7 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
   launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * kNumSM), kRankThreads, kRankSubs * 4, st, true,
                 batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
-  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * kNumSM), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start,
-                index_bits);
+  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * kNumSM), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start);
   return cudaGetLastError();
 }
 

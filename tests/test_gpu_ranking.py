@@ -52,3 +52,25 @@ def test_ranking_matches_the_oracle(kind, d, bits):
         for c, (fields, stream) in enumerate(refs):
             assert_plan_equal(enc.read_plan(c), fields)
             assert (outs[c].cpu().numpy() == stream).all(), (c, use_plan_ws)
+
+
+@pytest.mark.parametrize("d", [40_960, 40_961, 40_975, 40_976, 43_007, 43_011])   # multiples of a row and of a warp's piece, and next to them
+@pytest.mark.parametrize("bits", [0.5, 4.0])
+def test_selection_at_the_edges_of_rows(d, bits):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(d)
+    x = rng.laplace(0, 1e-3, d)
+    x[d // 2:] *= np.where(rng.random(d - d // 2) < 0.02, 100.0, 0.01)      # a few candidates per step, then whole rows of them
+    x[d // 4:d // 4 + 3000] = 0.2 + 0.001 * rng.standard_normal(3000)
+    x[-1] = -0.9                                                            # the last coordinate of the last row
+    xs = [x.astype(np.float32), np.ascontiguousarray(x[::-1]).astype(np.float32)]
+    pds = [params_dict(d, int(bits * d), seed=9 + c, client_id=c) for c in range(2)]
+    refs = [oracle_plan_encode(v, pd) for v, pd in zip(xs, pds)]
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    outs = enc.run([torch.from_numpy(v).to(dev) for v in xs], use_plan_ws=True)
+    assert enc.status() == 0
+    for c, (fields, stream) in enumerate(refs):
+        assert_plan_equal(enc.read_plan(c), fields)
+        assert (outs[c].cpu().numpy() == stream).all(), c
