@@ -64,6 +64,8 @@ struct Shape {
   uint32_t cap[CVLC_MAX_CODE_BITS + 1];  // records per packet per code length
 };
 
+constexpr unsigned kFull = 0xFFFFFFFFu;  // all lanes of a warp
+
 // ---- workspace layouts (byte offsets; every region 256-byte aligned) ----------
 
 // The float4 units of an update are grouped into rows of kRowUnits (16 coordinates, 64 bytes: what a DRAM access moves).  The
@@ -127,6 +129,7 @@ struct EncHeader {
   uint32_t split_tiles;     // largest per-client tile count among the clients that need the partition
   uint32_t window;          // candidates per tile of the final ranking
   uint32_t rank_tiles;      // largest per-client tile count of the final ranking
+  uint32_t list_n[2], list_next[2];  // entries of the ranking's lists (of cells for a warp and for a block) and of them taken
   uint32_t sort_ticket;     // work items of the digit passes
   uint32_t sort_done[8];    // finished items of their phases
   uint32_t total_sort_tiles;
@@ -233,7 +236,7 @@ struct EncLayout {
   size_t off_ghist;              // uint64[n][4][512] digit histograms
   size_t off_gbase;              // uint64[n][4][512] their exclusive scans
   size_t off_select_state;       // uint64[n][select_tiles]
-  size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]
+  size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]; ranked by partition: the ranking's lists, a half each
   size_t off_buf_a, off_buf_b;   // uint64[n][capacity]
   size_t total;
 };

@@ -7,7 +7,6 @@
 
 namespace cvlc {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kPrepThreads = 1024;
 constexpr int kDecodeThreads = 256;
 constexpr uint32_t kDecStageWords = 512;  // packets up to 2 KB are staged in shared memory

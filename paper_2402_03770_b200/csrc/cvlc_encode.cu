@@ -8,10 +8,10 @@
 #include "cvlc_common.cuh"
 #include "cvlc_lookback.cuh"
 #include "cvlc_quant.cuh"
+#include "cvlc_rank.cuh"
 
 namespace cvlc {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 // Whether an earlier kernel of the call has reported an error.  Other blocks may set the word while this kernel
 // runs, so one thread reads it and the whole block takes the same branch.
 __device__ __forceinline__ bool block_sees_error(const int32_t* status) {
@@ -135,6 +135,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     hdr->status = s_bad;
     hdr->lsd = !plan_ws ? kRankDigits : s_lsd ? kRankAllDigits : kRankPartition;
     hdr->select_ticket = hdr->split_ticket = hdr->rank_ticket = hdr->sort_ticket = 0;
+    hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
     for (int p = 0; p < 8; ++p) hdr->sort_done[p] = 0;
     hdr->split_tiles = (s_most_split + kRankSplitTile - 1) / kRankSplitTile;
     // tiles small enough that the batch gives every SM several
@@ -730,7 +731,8 @@ __device__ __forceinline__ uint32_t sort_digit(unsigned long long pair, int pass
 // phase before its own is complete: the items it waits for have lower tickets, so blocks that are
 // running hold them.  A pass whose digit is the same for every candidate of a client (normally the
 // fourth) is skipped for that client; which buffer holds its data after pass q follows from the
-// mask of skipped passes.  Used where the ranking by partition is not (see rank_shape).
+// mask of skipped passes.  Used where the ranking by partition is not (see rank_shape); otherwise the kernel works off what that
+// has left over (see rank_lists).
 
 // two adjacent look-back words in one 128-bit access (each 64-bit half is its own atomic access)
 __device__ __forceinline__ void ld_relaxed2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
@@ -751,7 +753,10 @@ struct SortShared {
 };
 
 constexpr size_t kSortSharedBytes = (sizeof(SortShared) + 15) & ~(size_t)15;
-constexpr size_t sort_smem_bytes(uint32_t n) { return kSortSharedBytes + (size_t)kSortTile * 8 + (4 * (size_t)n + 1) * 4; }
+constexpr size_t sort_smem_bytes(uint32_t n) {
+  const size_t passes = kSortSharedBytes + (size_t)kSortTile * 8 + (4 * (size_t)n + 1) * 4;
+  return passes > sizeof(RankShared) ? passes : sizeof(RankShared);
+}
 
 // One tile of one digit pass.  FULL: the tile holds kSortTile items (no bounds checks in the item loops).
 // Thread t < 256 owns the digit values 2t and 2t + 1 in the counting, scan and look-back steps.
@@ -930,7 +935,7 @@ constexpr uint32_t kSortHistTiles = 8;   // tiles of a histogram item
 constexpr size_t kSortClear = 1 << 16;   // bytes of a clearing item
 
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks)
-k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start) {
   static_assert(kSortThreads * 2 == kDigits && kSortTile <= 0xFFFF, "two digit values per thread; 16-bit slots");
   extern __shared__ __align__(16) unsigned char s_raw[];
   SortShared& sh = *reinterpret_cast<SortShared*>(s_raw);
@@ -941,7 +946,11 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
   uint32_t* s_mask = s_keytop + batch.n;         // [n] its constant digits
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status) || hdr->lsd == kRankPartition) return;
+  if (block_sees_error(&hdr->status)) return;
+  if (hdr->lsd == kRankPartition) {  // only what the ranking has left over
+    if (hdr->list_n[0] | hdr->list_n[1]) rank_lists<kSortThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, rank_args(ws, L, bin_start, hdr, batch.n));
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = batch.n;
   {
@@ -1440,7 +1449,8 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   {
     const uint64_t want = L.sort_tiles_max * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(kSortMinBlocks * kNumSM) ? want : kSortMinBlocks * kNumSM);
-    launch_kernel(kKSort, k_sort, grid, kSortThreads, sort_smem_bytes(n), st, true, batch, shape.d, w, L);
+    launch_kernel(kKSort, k_sort, grid, kSortThreads, sort_smem_bytes(n), st, true, batch, shape.d, w, L,
+                  pws ? reinterpret_cast<const uint32_t*>(pws + plan_off_bin_start(n)) : nullptr);
   }
   if (wait_before_pack) {
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);

@@ -196,7 +196,6 @@ constexpr int kTuneThreads = 512;
 constexpr int kTuneWarps = kTuneThreads / 32;
 constexpr int kPlanItems = 1024;
 constexpr int kPairSlots = (496 + kTuneThreads - 1) / kTuneThreads;  // pairs of a sweep a thread looks at
-constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // scratch of the length-tuning loop (the tuning kernel's dynamic shared memory)
 constexpr int kMaxBatchOps = 32;  // atomic operations evaluated together

@@ -24,7 +24,6 @@
 
 namespace cvlc {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kUfThreads = 128;
 constexpr int kUfWarps = kUfThreads / 32;
 constexpr uint32_t kUfCellBits = 9, kUfCells = 1u << kUfCellBits;  // position ranges a block's records are sorted by

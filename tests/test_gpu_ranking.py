@@ -74,3 +74,26 @@ def test_selection_at_the_edges_of_rows(d, bits):
     for c, (fields, stream) in enumerate(refs):
         assert_plan_equal(enc.read_plan(c), fields)
         assert (outs[c].cpu().numpy() == stream).all(), c
+
+
+@pytest.mark.parametrize("n", [48, 49, 50, 256, 257, 290, 4000, 8191, 8193, 12000])   # limits of comparing, of a warp's cell, of a tile
+@pytest.mark.parametrize("crowded", [False, True])                                    # indices next to one another
+def test_equal_keys_among_others(n, crowded):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    d = 500_009
+    rng = np.random.default_rng(n)
+    x = rng.laplace(0, 1e-3, d).astype(np.float32)
+    tie = np.quantile(np.abs(x), 0.95).astype(np.float32)
+    where = np.arange(n) + 1234 if crowded else rng.choice(d, n, replace=False)
+    x[where] = tie * rng.choice(np.float32([-1, 1]), n)
+    near = rng.choice(d, 20, replace=False)                                           # neighbours of the repeated value
+    x[near] = (np.full(20, tie).view(np.int32) + np.arange(-10, 10, dtype=np.int32)).view(np.float32)
+    pd = params_dict(d, 3 * d, seed=3, client_id=0)
+    fields, stream = oracle_plan_encode(x, pd)
+    enc = B.BatchEncoder([gpu_params(pd)], dev)
+    outs = enc.run([torch.from_numpy(x).to(dev)], use_plan_ws=True)
+    assert enc.status() == 0
+    assert_plan_equal(enc.read_plan(0), fields)
+    assert (outs[0].cpu().numpy() == stream).all()
