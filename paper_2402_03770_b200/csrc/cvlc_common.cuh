@@ -350,7 +350,7 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
                                 cvlc_literal_plan_t* out, double* P_star, void* ws, cudaStream_t st);
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
 // ranking by partition (after the selection); returns at once on the device where the batch is ranked by digit passes
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, cudaStream_t st);
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into

@@ -382,10 +382,17 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   for (uint32_t i = lane; i < kRankCoarse; i += 32) sw.cnt[i] = 0;
   if (tid == 0) s_taken = 0;
   // Block b starts with client b n / grid; the first groups of a client go to the warps of the blocks that start with it, the rest
-  // by its counter.
+  // by its counter.  A small batch would wait for that: there the warps have three quarters of the groups without asking (with few
+  // clients, whose blocks are as good as equally many, all).
   const uint32_t home = (uint32_t)(((uint64_t)blockIdx.x * n) / gridDim.x);
   auto first_block = [&](uint32_t c) -> uint32_t { return (uint32_t)(((uint64_t)c * gridDim.x + n - 1) / n); };
-  auto given = [&](uint32_t c) -> uint32_t { return (first_block(c + 1) - first_block(c)) * (kSelThreads / 32); };
+  auto warps_of = [&](uint32_t c) -> uint32_t { return (first_block(c + 1) - first_block(c)) * (kSelThreads / 32); };
+  auto rounds_of = [&](uint32_t warps) -> uint32_t {
+    if (sg.count[0] + sg.count[1] || warps == 0) return 1;
+    const uint32_t most = n <= 8 ? (groups + warps - 1) / warps : groups / 4 * 3 / warps;
+    return most > 1 ? most : 1;
+  };
+  auto given = [&](uint32_t c) -> uint32_t { return warps_of(c) * rounds_of(warps_of(c)); };
 
   // the first client from `from` on that has groups left (n: none), found by all threads together
   auto find_client = [&](uint32_t from) -> uint32_t {
@@ -474,14 +481,16 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     // ---- the warp's groups, piece after piece: the maxima of the next two pieces are on their way, and so is the number of the
     // group after the last one asked for
     uint32_t taken = 0, group = 0, group2 = 0, piece = 0;
-    const uint32_t dynamic = given(c);  // first group that goes by the counter
+    const uint32_t warps = warps_of(c), dynamic = given(c);  // first group that goes by the counter
+    uint32_t rounds = 0;                                     // groups to come without asking
     if (visit == 0) {
-      group = (blockIdx.x - first_block(c)) * (kSelThreads / 32) + warp;
+      group = warp * (warps / (kSelThreads / 32)) + (blockIdx.x - first_block(c));  // a dense layer goes to all blocks
+      rounds = rounds_of(warps) - 1;
     } else {
       if (lane == 0) group = dynamic + atomicAdd(group_next + c, 1u);
       group = __shfl_sync(kFull, group, 0);
     }
-    if (lane == 0) group2 = dynamic + atomicAdd(group_next + c, 1u);
+    if (lane == 0 && rounds == 0) group2 = dynamic + atomicAdd(group_next + c, 1u);
     struct Piece {
       uint32_t row, end;  // [row, end): none left where row = end
       uint2 maxima;       // lane l: rows row + 4 l .. row + 4 l + 3
@@ -505,8 +514,9 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
       if (piece == pieces) {
         ++taken;
         piece = 0;
-        group = __shfl_sync(kFull, group2, 0);
-        if (lane == 0 && group < groups) group2 = dynamic + atomicAdd(group_next + c, 1u);
+        group = rounds ? group + warps : __shfl_sync(kFull, group2, 0);
+        if (rounds) --rounds;
+        if (lane == 0 && rounds == 0 && group < groups) group2 = dynamic + atomicAdd(group_next + c, 1u);
       }
       return p;
     };
@@ -1410,6 +1420,12 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
   return cudaGetLastError();
 }
 
+// While the length tuning runs on another stream, one block per client, selection and ranking leave it its SMs: their blocks fill an
+// SM, those behind a tuning block start when that ends (after 25 to 80 us, 67 us into a selection of 120), and the kernel ends with
+// them.  Not for long selections, where blocks that start late still find work, nor for so many clients that too few SMs are left.
+constexpr uint32_t kTuneRoom = 24;
+constexpr uint64_t kTuneRoomRows = 8 << 20;
+
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack, int write_residual) {
   static bool attr_done[64] = {};
@@ -1430,6 +1446,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
 
   const Partition part = make_partition(shape.d, n);
+  const unsigned sms = wait_before_pack && n <= kTuneRoom && part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
   if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st);
   else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st);
@@ -1437,9 +1454,9 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (pws) {
     const uint64_t want = (uint64_t)select_groups(part, n).groups * n;
-    const unsigned grid = (unsigned)(want < (uint64_t)kNumSM ? want : kNumSM);
+    const unsigned grid = (unsigned)(want < (uint64_t)sms ? want : sms);
     launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, pws, w, L);
-    e = launch_rank(batch, L, pws, w, st);
+    e = launch_rank(batch, L, pws, w, sms, st);
     if (e != cudaSuccess) return e;
   } else {
     const uint64_t want = select_tiles_of(shape.d, kSelectThreads) * n;
@@ -1448,7 +1465,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   }
   {
     const uint64_t want = L.sort_tiles_max * n;
-    const unsigned grid = (unsigned)(want < (uint64_t)(kSortMinBlocks * kNumSM) ? want : kSortMinBlocks * kNumSM);
+    const unsigned most = kSortMinBlocks * sms, grid = (unsigned)(want < (uint64_t)most ? want : most);
     launch_kernel(kKSort, k_sort, grid, kSortThreads, sort_smem_bytes(n), st, true, batch, shape.d, w, L,
                   pws ? reinterpret_cast<const uint32_t*>(pws + plan_off_bin_start(n)) : nullptr);
   }

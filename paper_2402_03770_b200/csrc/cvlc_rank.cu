@@ -162,7 +162,7 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   }
 }
 
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, cudaStream_t st) {
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -173,10 +173,10 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
     attr_done[dev] = true;
   }
   auto blocks = [](uint64_t tiles, uint64_t most) -> unsigned { return (unsigned)(tiles < most ? tiles : most); };
-  launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * kNumSM), kRankThreads, kRankSubs * 4, st, true,
+  launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * sms), kRankThreads, kRankSubs * 4, st, true,
                 batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
-  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * kNumSM), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start);
+  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start);
   return cudaGetLastError();
 }
 
