@@ -39,10 +39,11 @@ FALLBACK_HBM_GBS = 6650.0
 # proportion to the clients); scaled to the clients of a launch, None for any other configuration, for fewer than
 # 32 clients per launch, and for a kernel that has changed since its capture.
 NCU_TRAFFIC_BYTES_PER_CLIENT = {
-    "k_hist": (1434.27e6 + 58.85e6) / 32,          # the update once, plus row maxima and per-segment histograms
-    "k_select": (477.15e6 + 164.51e6) / 32,        # the rows that hold candidates (a third of the update), plus the candidates
-    "k_sort_pass": (209.78e6 + 174.11e6 + 208.96e6 + 173.35e6 + 206.46e6 + 173.98e6 + 0.08e6) / 32 / 4,  # mean of a step's four launches
-    "k_pack": (177.98e6 + 54.22e6) / 32,
+    "k_hist": (1433.83e6 + 44.89e6) / 32,          # the update once, plus the rows' maxima
+    "k_select": (402.58e6 + 172.90e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
+    "k_rank_split": (203.49e6 + 155.95e6) / 32,
+    "k_rank": (203.13e6 + 158.17e6) / 32,
+    "k_pack": (177.98e6 + 55.82e6) / 32,
 }
 NOMINAL_HBM_GBS = 8000.0
 
@@ -406,17 +407,13 @@ def run_ours(args):
     n_groups = len(groups)
     sum_cand = float(sum(p.n_candidates for p in plans))
     sum_k = float(sum(p.k for p in plans))
-    # digit passes that move a client's candidates: its sort key keytop - key has 19 bits below the histogram bins plus
-    # the bits of the bin range between the threshold and the top bin; 9 bits per pass
-    def moving_passes(p):
-        bits = 19 + int(np.ceil(np.log2(max(1, p.top_bin + 1 - p.thresh_bin))))
-        return min(4, (bits + 8) // 9)
-    sort_bytes = float(sum(16.0 * p.n_candidates * moving_passes(p) for p in plans))
+    # the partition moves the candidates of clients with a bucket of more than 4096 (here: on average)
+    split_bytes = float(sum(16.0 * p.n_candidates for p in plans if p.n_candidates > 4096 * min(256, p.top_bin + 1 - p.thresh_bin)))
     alg_bytes_per_step = {   # algorithmic bytes all launches of one step move
         "k_hist": 4.0 * d * n_clients,
         "k_select": 4.0 * d * n_clients + 8.0 * sum_cand,
-        "k_sort_hist": 8.0 * sum_cand,
-        "k_sort_pass": sort_bytes,
+        "k_rank_split": split_bytes,
+        "k_rank": 16.0 * sum_cand,
         "k_pack": 8.0 * sum_k + float(n_clients) * stream_bytes,
         "k_decode": float(n_clients) * stream_bytes + 4.0 * d,
         "k_fill_zero": 4.0 * d,
@@ -457,9 +454,9 @@ def run_ours(args):
     # whole-step minimum bytes (read every update once, write every stream; read the streams, write the aggregate)
     step_min_bytes = n_clients * (4.0 * d + stream_bytes) + n_clients * stream_bytes + 4.0 * d
     step_frac = step_min_bytes / (ms_per_step * 1e-3) / 1e9 / peak
-    # the same with every pass counted at its own minimum (histogram read, selection read + candidates, three
-    # ranking passes, pack, decode): what this multi-pass design has to move
-    pass_bytes = sum(alg_bytes_per_step[k] for k in ("k_hist", "k_select", "k_sort_pass", "k_pack", "k_decode"))
+    # the same with every pass counted at its own minimum (histogram read, selection read + candidates, partition,
+    # ranking, pack, decode): what this multi-pass design has to move
+    pass_bytes = sum(alg_bytes_per_step[k] for k in ("k_hist", "k_select", "k_rank_split", "k_rank", "k_pack", "k_decode"))
     pass_frac = pass_bytes / (ms_per_step * 1e-3) / 1e9 / peak
     pass_frac_nominal = pass_bytes / (ms_per_step * 1e-3) / 1e9 / NOMINAL_HBM_GBS
 
@@ -490,8 +487,8 @@ def run_ours(args):
         "phase_ms_per_step": {
             "plan": sum(kernels[k]["ms_per_step"] for k in ("k_zero_words", "k_hist", "k_plan_fit", "k_plan_tune")
                         if k in kernels),
-            "encode": sum(kernels[k]["ms_per_step"] for k in ("k_encode_init", "k_select", "k_select_lookback", "k_sort_hist",
-                                                                "k_sort_scan", "k_sort_pass", "k_pack") if k in kernels),
+            "encode": sum(kernels[k]["ms_per_step"] for k in ("k_encode_init", "k_select", "k_select_lookback", "k_rank_split",
+                                                                "k_rank", "k_sort", "k_pack") if k in kernels),
             "decode_aggregate": sum(kernels[k]["ms_per_step"] for k in ("k_decode_prepare", "k_fill_zero", "k_decode")
                                     if k in kernels)},
         "step_min_bytes_frac_of_nominal_8TBps": step_min_bytes / (ms_per_step * 1e-3) / 8e12,
