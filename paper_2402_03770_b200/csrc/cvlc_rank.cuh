@@ -40,10 +40,10 @@ __device__ __forceinline__ void for_items(const u64* src, uint32_t n, F&& f) {
 }
 
 // exclusive scan of the cells in place by the whole block; returns the total
-template <int THREADS>
+template <int THREADS, uint32_t CELLS = kCells>
 __device__ __forceinline__ uint32_t scan_cells(uint32_t* cell) {
   __shared__ uint32_t s_warp[THREADS / 32];
-  constexpr int kVec = kCells / THREADS / 4;
+  constexpr int kVec = CELLS / THREADS / 4;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint4* mine = reinterpret_cast<uint4*>(cell) + kVec * tid;
   uint4 a[kVec];
@@ -174,7 +174,7 @@ __device__ __forceinline__ void rank_other(Others& o, uint32_t i, uint32_t key, 
 
 // Ranks items[0 .. n), n <= kRankItems, and writes them out; by the whole block.  False, and nothing done, if too many keys differ or
 // a range has too many items.
-template <int THREADS>
+template <int THREADS, uint32_t BITS>
 __device__ __noinline__ bool rank_equal(RankShared& s, u64* items, uint32_t n, u64* __restrict__ out) {
   __shared__ uint32_t s_least, s_most, s_no;
   __shared__ Others s_others;
@@ -187,10 +187,11 @@ __device__ __noinline__ bool rank_equal(RankShared& s, u64* items, uint32_t n, u
   }
   {
     uint4* cells = reinterpret_cast<uint4*>(s.zero);
-    for (uint32_t i = tid; i < kCells / 4 + 1; i += THREADS) cells[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t i = tid; i < (1u << BITS) / 4 + 1; i += THREADS) cells[i] = make_uint4(0u, 0u, 0u, 0u);
   }
   __syncthreads();
   uint32_t least = 0xFFFFFFFFu, most = 0;
+#pragma unroll 4
   for (uint32_t p = tid; p < n; p += THREADS) {
     const uint2 v = it[p];
     if (v.y != key || v.x == kAside) {
@@ -209,12 +210,17 @@ __device__ __noinline__ bool rank_equal(RankShared& s, u64* items, uint32_t n, u
   __syncthreads();
   least = s_least;
   const uint32_t span = s_most > least ? s_most - least : 0u;
-  const int sh = span < kCells ? 0 : 32 - __clz(span) - (int)kCellBits;
+  const int sh = span < (1u << BITS) ? 0 : 32 - __clz(span) - (int)BITS;
   if (!s_no) {
-    for (uint32_t p = tid; p < n; p += THREADS) {
-      const uint32_t x = it[p].x;
-      if (x != kAside && atomicAdd(&s.cell[(x - least) >> sh], 1u) >= kCompareAll) s_no = 1;
+    bool crowded = false;
+    for (uint32_t p0 = tid; p0 < n; p0 += 4 * THREADS) {
+      uint32_t x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = p0 + u * THREADS < n ? it[p0 + u * THREADS].x : kAside;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) crowded |= x[u] != kAside && atomicAdd(&s.cell[(x[u] - least) >> sh], 1u) >= kCompareAll;
     }
+    if (crowded) s_no = 1;
   }
   __syncthreads();
   if (s_no) {
@@ -222,12 +228,18 @@ __device__ __noinline__ bool rank_equal(RankShared& s, u64* items, uint32_t n, u
     __syncthreads();
     return false;
   }
-  scan_cells<THREADS>(s.cell);
+  scan_cells<THREADS, 1u << BITS>(s.cell);
   const uint32_t equal = n - s_others.n;
   rank_other(s_others, tid, key, equal, out);
-  for (uint32_t p = tid; p < n; p += THREADS) {
-    const uint32_t x = it[p].x;
-    if (x != kAside) it[atomicAdd(&s.cell[(x - least) >> sh], 1u)].y = x;
+  for (uint32_t p0 = tid; p0 < n; p0 += 4 * THREADS) {
+    uint32_t x[4], to[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = p0 + u * THREADS < n ? it[p0 + u * THREADS].x : kAside;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) to[u] = x[u] != kAside ? atomicAdd(&s.cell[(x[u] - least) >> sh], 1u) : 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (x[u] != kAside) it[to[u]].y = x[u];
   }
   __syncthreads();
   u64* __restrict__ to = out + s_others.below;
@@ -392,7 +404,11 @@ __device__ __noinline__ void rank_cell(RankShared& s, u64* at, uint32_t n) {
       for_items<THREADS>(at, n, [&](uint32_t i, u64 item) { s.items[i] = to_value(item); });
       __syncthreads();
     }
-    if (attempt == 0 ? rank_equal<THREADS>(s, s.items, n, at) : attempt == 1 && rank_spread<THREADS>(s, at, n)) return;
+    if (attempt == 0) {
+      if (n <= kCells / 2 ? rank_equal<THREADS, kCellBits - 1>(s, s.items, n, at) : rank_equal<THREADS, kCellBits>(s, s.items, n, at)) return;
+    } else if (attempt == 1 && rank_spread<THREADS>(s, at, n)) {
+      return;
+    }
   }
   rank_by_block<THREADS>(s.items, n, at);
 }
