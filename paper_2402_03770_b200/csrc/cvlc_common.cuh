@@ -87,11 +87,15 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   P.rows = (((d >> 2) + kRowUnits - 1) / kRowUnits + 15) & ~(uint64_t)15;
   if (P.rows == 0) P.rows = 16;
   P.total = P.rows * n;
+  // Three blocks per SM finish a small batch sooner (10 clients of 5 M coordinates: 44 instead of 47 us, 20 of 1.2 M: 26 instead of
+  // 29); a large one streams faster with two (100 of 11.2 M: 709 us instead of 729).
+  const uint64_t most = P.total <= (16u << 20) ? 3 * kNumSM : 2 * kNumSM;
   uint64_t grid = (P.total + 255) / 256;
-  if (grid > (uint64_t)(2 * kNumSM)) grid = 2 * kNumSM;
+  if (grid > most) grid = most;
   P.grid = (uint32_t)grid;
-  // two chunks per block where that leaves each 64 KB and more: every chunk ends with a merge into a client's histogram
-  const uint64_t n_chunks = P.total / (2 * grid) >= 1024 ? 2 * grid : grid;
+  // two chunks per block where that leaves each a megabyte and more: every chunk ends with a merge into a client's histogram
+  // (with two of 64 KB and more 10 clients of 5 M coordinates take 53 us)
+  const uint64_t n_chunks = P.total / (2 * grid) >= 16384 ? 2 * grid : grid;
   P.chunk = ((P.total + n_chunks - 1) / n_chunks + 15) & ~(uint64_t)15;
   P.n_chunks = (uint32_t)((P.total + P.chunk - 1) / P.chunk);
   return P;

@@ -16,7 +16,7 @@ namespace cvlc {
 // ===================================================================================
 
 constexpr int kHistThreads = kStreamThreads;
-constexpr int kHistSub = 4;  // shared sub-histograms per block (64 KB)
+constexpr int kHistSub = 2;  // shared sub-histograms per block (32 KB)
 
 // The clients' rows form one concatenated array that is cut into equal contiguous chunks, one or two
 // per block, so the load is even whatever the number of clients; a block that crosses a client
@@ -34,7 +34,7 @@ __device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
   return m01 > m23 ? m01 : m23;
 }
 
-__global__ void __launch_bounds__(kHistThreads, 2)
+__global__ void __launch_bounds__(kHistThreads, 3)
 k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
        unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint16_t* __restrict__ row_max_all) {
   extern __shared__ uint32_t sh_hist[];  // [kHistSub][4096]
