@@ -26,15 +26,15 @@ __device__ __forceinline__ u64 to_item(u64 value) {
   return ((u64)~(uint32_t)(value >> 32) << 32) | (u64)__funnelshift_r(lo, lo, 1);
 }
 
-// f(i, src[i]) for the block's items, eight loads of a thread in flight
+// f(i, src[i]) for the block's items, sixteen loads of a thread in flight
 template <int THREADS, class F>
 __device__ __forceinline__ void for_items(const u64* src, uint32_t n, F&& f) {
-  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 8 * THREADS) {
-    u64 v[8];
+  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 16 * THREADS) {
+    u64 v[16];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = i0 + u * THREADS < n ? src[i0 + u * THREADS] : 0ull;
+    for (int u = 0; u < 16; ++u) v[u] = i0 + u * THREADS < n ? src[i0 + u * THREADS] : 0ull;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 16; ++u)
       if (i0 + u * THREADS < n) f(i0 + u * THREADS, v[u]);
   }
 }
@@ -413,24 +413,36 @@ __device__ __noinline__ void rank_cell(RankShared& s, u64* at, uint32_t n) {
   rank_by_block<THREADS>(s.items, n, at);
 }
 
-// A boundary near rank x of the m values of src, all in [lo, hi): a value and how many of src lie below it.  The range around the
-// rank is narrowed until at most kCutRest values are left in it; the boundary is where that range starts.  A function of the set
-// of values and x alone, so that neighbouring tiles agree on it.
+// Boundaries near ranks x[0] and x[1] of the m values of src, all in [lo, hi): a value and how many of src lie below it.  The range
+// around a rank is narrowed until at most kCutRest values are left in it; the boundary is where that range starts.  A function of the
+// set of values and the rank alone, so that neighbouring tiles agree on it.  As long as both ranks lie in one range, one pass over
+// the values serves both: of equal keys two passes find both boundaries.
 constexpr uint32_t kCutRest = kRankItems - kRankWindow;
 struct Cut {
   u64 value;
   uint32_t below;
 };
+struct CutSearch {
+  u64 lo, hi;
+  uint32_t x, below;
+  bool open;
+};
 template <int THREADS>
-__device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t x) {
-  __shared__ uint32_t s_cell, s_below, s_count;
+__device__ __noinline__ void cut_near(RankShared& s, const u64* __restrict__ src, uint32_t m, CutSearch& a, CutSearch& b) {
+  __shared__ uint32_t s_cell[2], s_below[2], s_count[2];
   const int tid = threadIdx.x;
-  Cut cut{lo, 0};
-  for (int level = 0; level < 8 && lo < hi; ++level) {  // 63 bits, 12 a level
+  for (int level = 0; level < 16 && (a.open || b.open); ++level) {  // 63 bits, 12 a level, each rank on its own at worst
+    const u64 lo = a.open ? a.lo : b.lo, hi = a.open ? a.hi : b.hi;
+    const bool for_a = a.open, for_b = b.open && b.lo == lo && b.hi == hi;
+    if (lo >= hi) {
+      if (for_a) a.open = false;
+      if (for_b) b.open = false;
+      continue;
+    }
     const u64 span = hi - lo - 1;
     const int sh = span < kCells ? 0 : 64 - __clzll((long long)span) - (int)kCellBits;  // span >> sh below kCells
     for (uint32_t i = tid; i < kCells; i += THREADS) s.cell[i] = 0;
-    if (tid == 0) s_cell = s_below = s_count = 0;
+    if (tid < 2) s_cell[tid] = s_below[tid] = s_count[tid] = 0;
     __syncthreads();
     for_items<THREADS>(src, m, [&](uint32_t, u64 item) {
       const u64 v = to_value(item);
@@ -439,35 +451,46 @@ __device__ __noinline__ Cut cut_near(RankShared& s, const u64* __restrict__ src,
     __syncthreads();
     const uint32_t total = scan_cells<THREADS>(s.cell);
     // the last cell that starts at or below the rank
-    const uint32_t at = x - cut.below;
     for (uint32_t i = tid; i < kCells; i += THREADS) {
-      const uint32_t b = s.cell[i], e = (i + 1 < kCells) ? s.cell[i + 1] : total;
-      if (b <= at && at < e) {
-        s_cell = i;
-        s_below = b;
-        s_count = e - b;
-      }
+      const uint32_t first = s.cell[i], end = (i + 1 < kCells) ? s.cell[i + 1] : total;
+      auto look = [&](const CutSearch& c, int e) {
+        const uint32_t at = c.x - c.below;
+        if (first <= at && at < end) {
+          s_cell[e] = i;
+          s_below[e] = first;
+          s_count[e] = end - first;
+        }
+      };
+      if (for_a) look(a, 0);
+      if (for_b) look(b, 1);
     }
     __syncthreads();
-    const uint32_t cell = s_cell, below = s_below, count = s_count;
+    auto narrow = [&](CutSearch& c, int e) {
+      c.lo = lo + ((u64)s_cell[e] << sh);
+      c.hi = c.lo + (1ull << sh) < hi ? c.lo + (1ull << sh) : hi;
+      c.below += s_below[e];
+      if (s_count[e] <= kCutRest || sh == 0) c.open = false;
+    };
+    if (for_a) narrow(a, 0);
+    if (for_b) narrow(b, 1);
     __syncthreads();
-    lo += (u64)cell << sh;
-    hi = lo + (1ull << sh) < hi ? lo + (1ull << sh) : hi;
-    cut.value = lo;
-    cut.below += below;
-    if (count <= kCutRest || sh == 0) break;
   }
-  return cut;
 }
 
-// Ranks a .. b (about) of a bucket that a block cannot hold, m values in [lo, hi): equal or nearly equal keys.  src and out differ.
+// Ranks a .. b (about) of a bucket that a block cannot hold, m values in [lo, hi), are collected in their place: items that begin at
+// out + below and whose values lie in [from, to).  src and out differ.
+struct RankPart {
+  u64 from, to;
+  uint32_t below, n;
+};
 template <int THREADS>
-__device__ __noinline__ void rank_part(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t a, uint32_t b,
-                                       u64* __restrict__ out) {
+__device__ __noinline__ RankPart collect_part(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t a, uint32_t b,
+                                              u64* __restrict__ out) {
   __shared__ uint32_t s_n;
   const int tid = threadIdx.x;
-  const Cut from = a == 0 ? Cut{lo, 0} : cut_near<THREADS>(s, src, m, lo, hi, a);
-  const Cut to = b >= m ? Cut{hi, m} : cut_near<THREADS>(s, src, m, lo, hi, b);
+  CutSearch at_a{lo, hi, a, 0, a != 0}, at_b{lo, hi, b, 0, b < m};
+  cut_near<THREADS>(s, src, m, at_a, at_b);
+  const Cut from{at_a.lo, at_a.below}, to = b >= m ? Cut{hi, m} : Cut{at_b.lo, at_b.below};
   if (tid == 0) s_n = 0;
   __syncthreads();
   for_items<THREADS>(src, m, [&](uint32_t, u64 item) {
@@ -480,7 +503,7 @@ __device__ __noinline__ void rank_part(RankShared& s, const u64* __restrict__ sr
   __syncthreads();
   const uint32_t got = s_n < kRankItems ? s_n : kRankItems;  // at most a window and kCutRest
   __syncthreads();
-  if (got != 0) rank_cell<THREADS>(s, out + from.below, got);
+  return RankPart{from.value, to.value, from.below, got};
 }
 
 // Ranks m <= kRankItems items whose inv lies in [base, base + span]: spread over kCells equal ranges of inv, about one item per
@@ -618,12 +641,24 @@ __device__ __noinline__ void rank_large(RankShared& s, const RankTile& T, const 
   const ClientRank r = a.rank[c];
   const u64 x0 = (u64)tile * a.window, x1 = x0 + a.window;
   const uint32_t sh = T.sh;
+  auto rank = [&](const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out) {
+    if (threadIdx.x == 0) s_n = 0;
+    rank_buckets<THREADS>(s, src, m, base, span, out, r.keytop,
+                          [&](u64* where, uint32_t items) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
+    const uint32_t n_big = s_n;
+    for (uint32_t g = 0; g < n_big; ++g) rank_cell<THREADS>(s, out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
+    __syncthreads();
+  };
   auto part_of = [&](uint32_t bucket, uint32_t first, uint32_t end) {  // the window's part of a large bucket
     const u64 lo = ((u64)~r.keytop + ((u64)bucket << sh)) << 32, end_high = (u64)~r.keytop + ((u64)(bucket + 1) << sh);
     const u64 hi = end_high >> 32 ? ~0ull : end_high << 32;  // the last bucket may reach below key 0
     const uint32_t from = x0 > first ? (uint32_t)(x0 - first) : 0u;
     const uint32_t to = x1 < end ? (uint32_t)(x1 - first) : end - first;
-    rank_part<THREADS>(s, T.from + first, end - first, lo, hi, from, to, T.into + first);
+    const RankPart p = collect_part<THREADS>(s, T.from + first, end - first, lo, hi, from, to, T.into + first);
+    if (p.n == 0) return;
+    const uint32_t base = (uint32_t)(p.from >> 32) - ~r.keytop, last = (uint32_t)((p.to - 1) >> 32) - ~r.keytop;
+    u64* at = T.into + first + p.below;
+    rank(at, p.n, base, last - base, at);
   };
   uint32_t b_lo = T.bucket[0], at = T.start[0];
   const uint32_t b_end = T.bucket[1], at_end = T.start[1];
@@ -638,12 +673,7 @@ __device__ __noinline__ void rank_large(RankShared& s, const RankTile& T, const 
     if (to - at > kRankItems) {
       if (r.split) part_of(b_lo, at, to);
     } else if (to > at) {
-      if (threadIdx.x == 0) s_n = 0;
-      rank_buckets<THREADS>(s, T.from + at, to - at, b_lo << sh, (uint32_t)(((u64)b_hi << sh) - ((u64)b_lo << sh) - 1), T.into + at, r.keytop,
-                            [&](u64* where, uint32_t m) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - (T.into + at)) | m << 16; }, [] {});
-      const uint32_t n_big = s_n;
-      for (uint32_t g = 0; g < n_big; ++g) rank_cell<THREADS>(s, T.into + at + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
-      __syncthreads();
+      rank(T.from + at, to - at, b_lo << sh, (uint32_t)(((u64)b_hi << sh) - ((u64)b_lo << sh) - 1), T.into + at);
     }
     b_lo = b_hi;
     at = to;

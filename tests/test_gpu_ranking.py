@@ -97,3 +97,20 @@ def test_equal_keys_among_others(n, crowded):
     assert enc.status() == 0
     assert_plan_equal(enc.read_plan(0), fields)
     assert (outs[0].cpu().numpy() == stream).all()
+
+
+@pytest.mark.parametrize("n", [262_000, 300_000])       # the largest bucket that is ranked window by window, and one for the digit passes
+def test_very_large_buckets(n):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    d = 2_000_003
+    rng = np.random.default_rng(n)
+    x = values(f"ties{n}", d, rng).astype(np.float32)
+    pd = params_dict(d, 6 * d, seed=4, client_id=0)
+    fields, stream = oracle_plan_encode(x, pd)
+    enc = B.BatchEncoder([gpu_params(pd)], dev)
+    outs = enc.run([torch.from_numpy(x).to(dev)], use_plan_ws=True)
+    assert enc.status() == 0
+    assert_plan_equal(enc.read_plan(0), fields)
+    assert (outs[0].cpu().numpy() == stream).all()
