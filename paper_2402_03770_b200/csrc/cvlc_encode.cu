@@ -368,8 +368,7 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   __shared__ uint32_t s_client, s_taken, s_scan[kSelThreads / 32];
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
-  if (hdr->lsd != kRankPartition) return;
+  if (rank_skips(hdr)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = batch.n;
   const uint32_t rows = (uint32_t)part.rows, held_rows = ((uint32_t)(d >> 2) + kRowUnits - 1) / kRowUnits;  // with coordinates

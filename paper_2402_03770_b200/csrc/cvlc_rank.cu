@@ -13,14 +13,6 @@ namespace cvlc {
 
 constexpr int kRankThreads = 512;
 
-// status and mode of the call, the same for all threads of a block
-__device__ __forceinline__ bool rank_skips(const EncHeader* hdr) {
-  __shared__ int s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<const volatile int32_t*>(&hdr->status) != 0 || hdr->lsd != kRankPartition;
-  __syncthreads();
-  return s_skip != 0;
-}
-
 // (no candidate lies above keytop: the selection has checked that the update is the plan's)
 __device__ __forceinline__ uint32_t inv_of(u64 item, uint32_t keytop) { return keytop - (uint32_t)(item >> 32); }
 

@@ -10,6 +10,17 @@ constexpr uint32_t kWarpCell = 256;     // one of up to this many is ranked by o
 
 typedef unsigned long long u64;
 
+// Whether the call has failed or is not ranked by partition.  While blocks of the selection start, others of the same launch may
+// write either word (an update that is not the plan's, a bucket too large for the partition), so one thread reads them and the
+// block takes one branch: warps that part here would leave the others of their block at its barriers with work not done.
+__device__ __forceinline__ bool rank_skips(const EncHeader* hdr) {
+  __shared__ int s_skip;
+  if (threadIdx.x == 0)
+    s_skip = *reinterpret_cast<const volatile int32_t*>(&hdr->status) != 0 || *reinterpret_cast<const volatile uint32_t*>(&hdr->lsd) != kRankPartition;
+  __syncthreads();
+  return s_skip != 0;
+}
+
 struct RankShared {
   u64 items[kRankItems + 2];  // values (see to_value): all distinct, ordered like the ranks
   uint32_t zero[4];           // cell[-1] = 0: where the first cell starts

@@ -114,3 +114,31 @@ def test_very_large_buckets(n):
     assert enc.status() == 0
     assert_plan_equal(enc.read_plan(0), fields)
     assert (outs[0].cpu().numpy() == stream).all()
+
+
+def test_bucket_for_the_digit_passes_found_while_blocks_still_start():
+    """The first clients' selections find a bucket that sends the batch to the digit passes, while blocks behind the length tuning's
+    (30 of them, one on an SM each) have yet to start and others are under way."""
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    d, n = 1_200_003, 30
+    rng = np.random.default_rng(30)
+    xs = [values("ties300000" if c < 2 else "laplace", d, rng).astype(np.float32) * np.float32(1 + c) for c in range(n)]
+    pds = [params_dict(d, 6 * d, seed=6 + c, client_id=c) for c in range(n)]
+    refs = {c: oracle_plan_encode(xs[c], pds[c]) for c in (0, 2, n - 1)}
+    dxs = [torch.from_numpy(x).to(dev) for x in xs]
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    side = torch.cuda.Stream(dev)
+    first = None
+    for _ in range(10):
+        for o in enc.outs:
+            o.fill_(0x3C)
+        outs = enc.compress(dxs, side_stream=side)
+        assert enc.status() == 0
+        if first is None:
+            for c, (fields, stream) in refs.items():
+                assert_plan_equal(enc.read_plan(c), fields)
+                assert (outs[c].cpu().numpy() == stream).all(), c
+            first = [o.clone() for o in outs]
+        assert all(torch.equal(a, b) for a, b in zip(first, outs))
