@@ -344,7 +344,7 @@ static int encode_batch(const float* const* x_dev, const cvlc_params* params, ui
   if (ws_bytes < enc_layout(S.d, n, cap).total) return CVLC_ERR_WORKSPACE_TOO_SMALL;
   if (!pack_fits(S)) return CVLC_ERR_INVALID_ARG;
   if (S.R > 0x7FFFFFFFu || n > 65535) return CVLC_ERR_INVALID_ARG;
-  return launch_encode(desc, n, S, cap, plan_ws_dev, ws_dev, static_cast<cudaStream_t>(cuda_stream), nullptr, write_residual) ==
+  return launch_encode(desc, n, S, cap, plan_ws_dev, ws_dev, static_cast<cudaStream_t>(cuda_stream), false, nullptr, write_residual) ==
                  cudaSuccess
              ? CVLC_OK
              : CVLC_ERR_CUDA;
@@ -436,7 +436,7 @@ int cvlc_encode_unframed_batch(const float* const* x_dev, const cvlc_params* par
   if (enc_ws_bytes < enc_layout(S.d, n, cap).total || uf_ws_bytes_given < uf_ws_bytes(n, S.R)) return CVLC_ERR_WORKSPACE_TOO_SMALL;
   if (S.R > 0x7FFFFFFFu || n > 65535) return CVLC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (launch_encode(desc, n, S, cap, plan_ws_dev, enc_ws_dev, st, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_encode(desc, n, S, cap, plan_ws_dev, enc_ws_dev, st, false, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
   return launch_pack_unframed(n, S, cap, stream_capacity, enc_ws_dev, uf_ws_dev,
                               reinterpret_cast<unsigned long long*>(stream_bytes_dev), st) == cudaSuccess
              ? CVLC_OK
@@ -521,7 +521,7 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   if (launch_plan_front(desc, n, S, plan_ws_dev, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
     if (launch_plan_back(n, S, plan_ws_dev, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
-    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
   // the length tuning reads the histograms' fit only; selection and ranking do not need its result.  The lock keeps two
   // threads from recording the device's events between each other's record and wait.
@@ -532,7 +532,7 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;
   if (launch_plan_back(n, S, plan_ws_dev, side_st, false) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(join, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
-  return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+  return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
 }
 
 int cvlc_encode(const float* x_dev, const cvlc_params* p, const cvlc_plan_t* plan_dev, const void* plan_ws_dev,

@@ -303,13 +303,15 @@ struct LaunchScope {
 };
 
 #ifdef __CUDACC__
-// Every kernel of the plan / encode / decode path is launched with programmatic stream serialization: it is set up while the
-// kernel before it drains, and pdl_enter(), the first thing every thread does, waits until that kernel is complete and its
+// Every kernel of the plan / encode / decode path but the first of a call is launched with programmatic stream serialization: it is
+// set up while the kernel before it drains, and pdl_enter(), the first thing every thread does, waits until that kernel is complete and its
 // writes are visible.  Nothing is read or written before that.  This takes about 2 us off every kernel boundary (one small
 // client, 12 kernels: 101 -> 78 us a pass; 100 ResNet-18 clients: 3.89 -> 3.87 ms).  No kernel lets its successor in before
 // its own blocks have left (griddepcontrol.launch_dependents): blocks that move in early gather on the SMs that happen to be
 // free, and the successor then runs on part of the chip (error compensation 314 -> 361 us, the large round 3.87 -> 4.00 ms).
-// A launch that a wait on another stream's event precedes is an ordinary one.
+// The attribute relaxes the order behind the kernel before it on the stream, and that must be one of ours that waits itself: the
+// first kernel of a call, and one that a wait on another stream's event precedes, are ordinary launches, behind whatever the caller
+// has put on the stream (event waits, copies, kernels that let their successors in early).
 template <class... Params, class... Args>
 inline void launch_kernel(int id, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap, Args&&... args) {
   LaunchScope ls(id, st);
@@ -363,8 +365,9 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
 // the error-compensation memory (the input buffers are written: every sent coordinate loses what the parameter
 // server rebuilds for it); kPackNone = selection and ranking only (the unframed writer follows)
 constexpr int kPackFramed = 0, kPackResidual = 1, kPackNone = 2;
+// overlap: the planning of the same call precedes it on the stream
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack, int write_residual);
+                          const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual);
 cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st);
 // unframed stream (version 2)
 constexpr uint32_t kUfMaxRecords = 2048;  // records of a block (it is sorted and assembled in one warp's shared memory)

@@ -327,7 +327,7 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
   };
   const uint64_t first = win < d ? win : d;
   const uint64_t zero_d = accumulate ? 0 : first;
-  launch_kernel(kKDecodePrepare, k_decode_prepare, 1 + (accumulate ? 0 : fill_grid(first, kPrepThreads, 2 * kNumSM)), kPrepThreads, 0, st, true,
+  launch_kernel(kKDecodePrepare, k_decode_prepare, 1 + (accumulate ? 0 : fill_grid(first, kPrepThreads, 2 * kNumSM)), kPrepThreads, 0, st, false,
                 streams, stream_bytes, weights, n, weight_total, d, s, w, out, zero_d);
   for (uint64_t lo = 0; lo < d; lo += win) {
     const uint64_t hi = lo + win < d ? lo + win : d;

@@ -1393,12 +1393,12 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
 
 template <int CAP>
 static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, const unsigned char* plan_ws,
-                          unsigned char* w, cudaStream_t st) {
+                          unsigned char* w, cudaStream_t st, bool overlap) {
   BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
-  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, true, w, batch, shape, L, plan_ws);
+  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, overlap, w, batch, shape, L, plan_ws);
 }
 
 template <int CAP>
@@ -1426,7 +1426,7 @@ constexpr uint32_t kTuneRoom = 24;
 constexpr uint64_t kTuneRoomRows = 8 << 20;
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, cudaEvent_t wait_before_pack, int write_residual) {
+                          const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual) {
   static bool attr_done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1447,9 +1447,9 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const Partition part = make_partition(shape.d, n);
   const unsigned sms = wait_before_pack && n <= kTuneRoom && part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
-  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st);
-  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st);
-  else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st);
+  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st, overlap);
+  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st, overlap);
+  else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st, overlap);
   const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (pws) {
     const uint64_t want = (uint64_t)select_groups(part, n).groups * n;
@@ -1473,10 +1473,10 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     if (ew != cudaSuccess) return ew;
   }
   if (write_residual == kPackNone) return cudaGetLastError();  // the caller writes the ranked records in a format of its own
-  const bool overlap = wait_before_pack == nullptr;
-  if (n <= (uint32_t)kSmallBatch) return launch_pack_t<kSmallBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
-  if (n <= (uint32_t)kMediumBatch) return launch_pack_t<kMediumBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
-  return launch_pack_t<kLargeBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+  const bool pack_overlap = wait_before_pack == nullptr;
+  if (n <= (uint32_t)kSmallBatch) return launch_pack_t<kSmallBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
+  if (n <= (uint32_t)kMediumBatch) return launch_pack_t<kMediumBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
+  return launch_pack_t<kLargeBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
 }
 
 // memory <- memory + update in fp32, for every client of a batch (the first step of a round with error compensation)
@@ -1527,7 +1527,7 @@ static void launch_ec_t(float* const* memory, const float* const* update, uint32
   }
   const uint64_t want = (((d >> 2) + 1) * n + 255) / 256;
   const unsigned grid = (unsigned)(want < (uint64_t)(8 * kNumSM) ? want : 8 * kNumSM);
-  launch_kernel(kKEcAccumulate, k_ec_accumulate<CAP>, grid, 256, 0, st, true, batch, d);
+  launch_kernel(kKEcAccumulate, k_ec_accumulate<CAP>, grid, 256, 0, st, false, batch, d);
 }
 
 cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st) {

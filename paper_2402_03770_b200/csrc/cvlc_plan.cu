@@ -1286,7 +1286,7 @@ static void launch_zero_t(const ClientDesc* clients, uint32_t n, unsigned char* 
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
   const size_t want = (bytes + more) / 16 / 256 + 1;
   const unsigned grid = (unsigned)(want < (size_t)(4 * kNumSM) ? want : 4 * kNumSM);
-  launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, true, batch, reinterpret_cast<ClientDesc*>(w + off_desc),
+  launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, false, batch, reinterpret_cast<ClientDesc*>(w + off_desc),
                 reinterpret_cast<uint4*>(w), bytes / 16, reinterpret_cast<uint4*>(w + at), more / 16);
 }
 static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t bytes, size_t at, size_t more, cudaStream_t st) {

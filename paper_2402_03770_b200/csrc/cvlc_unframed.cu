@@ -726,7 +726,7 @@ cudaError_t launch_decode_unframed(const uint8_t* const* streams, const uint64_t
                                    uint32_t n, double weight_total, uint64_t d, uint32_t s, float* out, int accumulate,
                                    void* ws, cudaStream_t st) {
   unsigned char* w = static_cast<unsigned char*>(ws);
-  launch_kernel(kKDecodePrepare, k_uf_decode_prepare, 1, kUfPrepThreads, 0, st, true, streams, stream_bytes, weights, n, weight_total, d, s, w);
+  launch_kernel(kKDecodePrepare, k_uf_decode_prepare, 1, kUfPrepThreads, 0, st, false, streams, stream_bytes, weights, n, weight_total, d, s, w);
   if (!accumulate) {
     const cudaError_t e = launch_fill_zero(out, d, st);
     if (e != cudaSuccess) return e;

@@ -1,0 +1,145 @@
+"""The calls among other work on the caller's streams: inputs that another stream finishes late, behind a wait on its event, and
+capture into a CUDA graph.  Streams against the oracle to the bit, aggregates within the usual tolerance."""
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_util import assert_aggregate_close, gpu_params, oracle_params, params_dict
+
+pytestmark = pytest.mark.gpu
+
+D, N = 200_003, 3
+KINDS = ["client", "compress", "separate", "ec", "decode", "unframed", "decode_unframed"]
+
+
+class Calls:
+    """Buffers of N clients.  `load` puts one of two sets of inputs in place, `run` makes the calls of a kind on the current stream,
+    `check` compares what they left with the oracle's for a set of inputs."""
+
+    def __init__(self, kind):
+        import torch
+        from paper_2402_03770_b200 import binding as B
+        self.torch, self.B, self.kind = torch, B, kind
+        self.dev = dev = torch.device("cuda:0")
+        rng = np.random.default_rng(len(kind))
+        self.pds = [params_dict(D, 2 * D, seed=11 + c, client_id=c) for c in range(N)]
+        self.params = [gpu_params(pd) for pd in self.pds]
+        self.updates = [[rng.laplace(0, 10.0 ** -(3 + s), D).astype(np.float32) for _ in range(N)] for s in range(2)]
+        self.weights = np.array([1.0, 2.5, 3.0], np.float32)
+        self.plans = [[O.plan(x, oracle_params(pd)) for x, pd in zip(xs, self.pds)] for xs in self.updates]
+        encode = O.encode_unframed if "unframed" in kind else O.encode
+        self.streams = [[encode(x, oracle_params(pd), pl) for x, pd, pl in zip(xs, self.pds, pls)]
+                        for xs, pls in zip(self.updates, self.plans)]
+        decode = O.decode_aggregate_unframed if "unframed" in kind else O.decode_aggregate
+        self.aggregates = [decode(s, self.weights, D) for s in self.streams]
+
+        self.enc = B.BatchEncoder(self.params, dev)
+        self.clients = [B.ClientEncoder(p, dev) for p in self.params]
+        self.memory = torch.zeros(N, (D + 3) // 4 * 4, device=dev)
+        self.memories = [self.memory[c, :D] for c in range(N)]
+        self.side = torch.cuda.Stream(dev)
+        size = max(B.cvlc_stream_bytes(self.params[0]), B.cvlc_unframed_stream_capacity(self.params[0]))
+        self.bytes_in = [torch.zeros(size, dtype=torch.uint8, device=dev) for _ in range(N)]
+        self.bytes_out = [torch.zeros(size, dtype=torch.uint8, device=dev) for _ in range(N)]
+        self.sizes = torch.zeros(N, dtype=torch.int64, device=dev)
+        self.uf_ws = B.alloc_bytes(B.cvlc_unframed_workspace_bytes(self.params[0], N), dev)
+        self.out = torch.zeros(D, device=dev)
+        self.agg = B.Aggregator(N, D, dev)
+        self.agg.set_clients(self.bytes_in, torch.from_numpy(self.weights))
+        self.xs = [torch.zeros(D, device=dev) for _ in range(N)]
+        # the sets as they lie on the device, to be copied into place without the host
+        if kind.startswith("decode"):
+            self.to = self.bytes_in + [self.agg.sizes]
+            self.sets = [[torch.nn.functional.pad(torch.from_numpy(s), (0, size - s.size)).to(dev) for s in streams] +
+                         [torch.tensor([s.size for s in streams], dtype=torch.int64, device=dev)] for streams in self.streams]
+        else:
+            self.to = self.xs
+            self.sets = [[torch.from_numpy(x).to(dev) for x in xs] for xs in self.updates]
+        torch.cuda.synchronize()
+
+    def load(self, which):
+        for a, b in zip(self.to, self.sets[which]):
+            a.copy_(b)
+
+    def run(self):
+        B, kind, enc = self.B, self.kind, self.enc
+        if kind == "client":
+            for c in range(N):
+                self.clients[c].run(self.xs[c])
+        elif kind == "compress":
+            enc.compress(self.xs, side_stream=self.side)
+        elif kind == "separate":
+            enc.run(self.xs)
+        elif kind == "ec":
+            self.memory.zero_()
+            B.cvlc_ec_accumulate_batch(self.memories, self.xs)
+            B.cvlc_plan_batch(self.memories, self.params, enc.plans, enc.plan_ws)
+            B.cvlc_encode_batch_ec(self.memories, self.params, enc.plans, enc.outs, enc.enc_ws, 0, plan_ws=enc.plan_ws)
+        elif kind == "decode":
+            self.agg.run(N, self.out)
+        elif kind == "unframed":
+            enc.plan(self.xs)
+            B.cvlc_encode_unframed_batch(self.xs, self.params, enc.plans, self.bytes_out, self.sizes, enc.enc_ws, self.uf_ws, 0,
+                                         plan_ws=enc.plan_ws)
+        else:
+            B.cvlc_decode_aggregate_unframed(self.agg.ptrs, self.agg.sizes, self.agg.weights, N, 0.0, D, self.out, False, self.agg.ws)
+
+    def check(self, which):
+        self.torch.cuda.synchronize()
+        if self.kind.startswith("decode"):
+            assert self.agg.status() == 0
+            assert_aggregate_close(self.out.cpu().numpy(), self.aggregates[which])
+            return
+        if self.kind == "client":
+            assert all(e.status() == 0 for e in self.clients)
+            outs = [e.out for e in self.clients]
+        else:
+            assert self.enc.status() == 0
+            outs = self.bytes_out if self.kind == "unframed" else self.enc.outs
+        for c, ref in enumerate(self.streams[which]):
+            assert (outs[c].cpu().numpy()[:ref.size] == ref).all(), c
+            if self.kind == "unframed":
+                assert int(self.sizes[c]) == ref.size
+            if self.kind == "ec":
+                assert (self.memories[c].cpu().numpy() == O.ec_residual(self.updates[which][c], ref)).all()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_inputs_behind_an_event_wait(kind):
+    """The stream holds a finished call on other inputs, then a wait for the stream that is still making the right ones."""
+    calls = Calls(kind)
+    torch = calls.torch
+    work, maker, made = torch.cuda.Stream(calls.dev), torch.cuda.Stream(calls.dev), torch.cuda.Event()
+    with torch.cuda.stream(work):
+        calls.load(0)
+        calls.run()
+    calls.check(0)
+    for which in (1, 0):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(maker):
+            torch.cuda._sleep(20_000_000)  # about 10 ms
+            calls.load(which)
+            made.record()
+        with torch.cuda.stream(work):
+            work.wait_event(made)
+            calls.run()
+        calls.check(which)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_capture_into_a_graph(kind):
+    """One capture, replayed for two sets of inputs; the length tuning's fork is captured with it."""
+    calls = Calls(kind)
+    torch = calls.torch
+    warm = torch.cuda.Stream(calls.dev)
+    with torch.cuda.stream(warm):  # attributes are set and modules loaded before the capture
+        calls.load(0)
+        calls.run()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls.run()
+    for which in (1, 0, 1):
+        calls.load(which)
+        graph.replay()
+        calls.check(which)
