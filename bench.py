@@ -488,7 +488,7 @@ def run_ours(args):
             "plan": sum(kernels[k]["ms_per_step"] for k in ("k_zero_words", "k_hist", "k_plan_fit", "k_plan_tune")
                         if k in kernels),
             "encode": sum(kernels[k]["ms_per_step"] for k in ("k_encode_init", "k_select", "k_select_lookback", "k_rank_split",
-                                                                "k_rank", "k_sort", "k_pack") if k in kernels),
+                                                                "k_rank", "k_rank_rest", "k_sort", "k_pack") if k in kernels),
             "decode_aggregate": sum(kernels[k]["ms_per_step"] for k in ("k_decode_prepare", "k_fill_zero", "k_decode")
                                     if k in kernels)},
         "step_min_bytes_frac_of_nominal_8TBps": step_min_bytes / (ms_per_step * 1e-3) / 8e12,

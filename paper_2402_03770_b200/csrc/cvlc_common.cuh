@@ -124,29 +124,36 @@ CVLC_HD constexpr size_t plan_off_max_bin(uint32_t n) { return align256(plan_off
 CVLC_HD constexpr size_t plan_off_row_max(uint32_t n) { return align256(plan_off_max_bin(n) + (size_t)n * 4); }
 CVLC_HD inline size_t plan_ws_bytes(const Partition& P, uint32_t n) { return align256(plan_off_row_max(n) + (size_t)P.total * 2); }
 
+// One round of splitting large buckets (see rank_big): counters of its lists and of what has been taken and finished
+constexpr int kBigRounds = 3;
+struct BigRound {
+  uint32_t n, pieces, slots;                        // buckets, pieces of them, their candidates in units of kBigSlot
+  uint32_t next_sample, next_count, next_place;     // taken
+  uint32_t done_sample, done_bounds, done_place;    // finished
+};
+
 // encode workspace header (first 256 bytes), written at the start of a call
 struct EncHeader {
   int32_t status;           // byte 0
-  uint32_t lsd;             // kRankPartition, kRankDigits or kRankAllDigits
+  uint32_t limit;           // ranks from here on are never sent
   uint32_t select_ticket;   // tile tickets of the look-back selection
   uint32_t split_ticket, rank_ticket;  // tile tickets of the partition and of the final ranking
   uint32_t split_tiles;     // largest per-client tile count among the clients that need the partition
   uint32_t window;          // candidates per tile of the final ranking
   uint32_t rank_tiles;      // largest per-client tile count of the final ranking
   uint32_t list_n[2], list_next[2];  // entries of the ranking's lists (of cells for a warp and for a block) and of them taken
+  BigRound big[kBigRounds];
+  uint32_t part_n, part_next;  // parts of large buckets to rank, and of them taken
   uint32_t sort_ticket;     // work items of the digit passes
   uint32_t sort_done[8];    // finished items of their phases
-  uint32_t total_sort_tiles;
   uint32_t max_sort_tiles;  // largest per-client tile count of this batch
 };
-
-// How a batch is ranked: by partition into buckets; by digit passes over candidates selected in index order; or by digit passes
-// with the selection done over again in that order, because a bucket turned out too large for the partition.
-constexpr uint32_t kRankPartition = 0, kRankDigits = 1, kRankAllDigits = 2;
+static_assert(sizeof(EncHeader) <= 256, "the header's place");
 
 constexpr int kSelectThreads = 512;
 constexpr int kSelectVecPerThread = 4;  // float4 loads per thread per tile of the look-back selection
-CVLC_HD constexpr uint64_t select_tiles_of(uint64_t d, int threads) { return (d + threads * kSelectVecPerThread * 4 - 1) / (threads * kSelectVecPerThread * 4); }
+constexpr int kSelectTile = kSelectThreads * kSelectVecPerThread * 4;  // 8192 coordinates
+CVLC_HD constexpr uint64_t select_tiles_of(uint64_t d) { return (d + kSelectTile - 1) / kSelectTile; }
 
 constexpr int kSortThreads = 256;
 constexpr int kSortItemsPerThread = 20;  // 128 registers per thread hold a tile without spilling: two blocks per SM
@@ -167,8 +174,6 @@ constexpr uint32_t kRankItems = 8192;      // candidates a block of the final ra
 constexpr uint32_t kRankBucket = 4096;     // largest coarse bucket that is ranked without a partition
 constexpr uint32_t kRankWindow = 4096;     // candidates of a tile of the final ranking
 constexpr uint32_t kRankSplitTile = 4096;  // candidates of a tile of the partition
-constexpr uint32_t kRankLargest = 1u << 18;   // a larger bucket (equal keys) sends the batch to the digit passes,
-constexpr uint32_t kRankExpected = 1u << 16;  // and so does the expectation of one larger than this
 struct ClientRank {
   uint32_t n;          // candidates
   uint32_t keytop;     // largest key of the top bin
@@ -176,15 +181,16 @@ struct ClientRank {
   uint32_t n_coarse;
   uint32_t sub_bits;   // a coarse bucket holds 2^sub_bits sub-buckets
   uint32_t split;      // 1: coarse buckets are partitioned into sub-buckets
-  uint32_t top_bin, pad;
+  uint32_t top_bin;
+  uint32_t wide;       // 1: sub-buckets are counted in whole numbers, their counts may be beyond fp32's
 };
 // The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates.  As few
 // sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that a block
-// meets costs the selection a global addition).  Returns false where even the most leave many times what a block holds, or where
-// zeros are candidates (more coordinates are sent than are not zero): such a batch takes the digit passes, whose cost does
-// not depend on the values.  (Buckets that a block cannot hold are ranked window by window; two clients of 50 M coordinates with
-// 7.5 M candidates each, every seventh layer on a grid: 1450 us a round, 3100 by digit passes.)
-CVLC_HD inline bool rank_shape(uint32_t nb, uint32_t max_bin, uint32_t thresh_bin, ClientRank* r) {
+// meets costs the selection a global addition).  No distribution is excluded: sub-buckets that a block cannot hold are split by
+// their own values (see rank_big), zeros among them where more coordinates are sent than are not zero.  (Digit passes for a batch
+// with such a client, as phases of one kernel, took it from 844 to 1110 us for one of 11.2 M coordinates, 97 % zeros, and from 1636
+// to 3100 for 10 of 5 M, 95 % zeros.)
+CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
   uint32_t g = 0;
   while (((nb - 1) >> g) + 1 > kRankCoarse) ++g;
   r->group = g;
@@ -194,7 +200,7 @@ CVLC_HD inline bool rank_shape(uint32_t nb, uint32_t max_bin, uint32_t thresh_bi
   uint32_t k = 0;
   while ((fullest >> k) > kRankItems - kRankWindow && (r->n_coarse << (k + 1)) <= kRankSubs && k < 16) ++k;
   r->sub_bits = k;
-  return (fullest >> k) <= kRankExpected && fullest < (1u << 24) && thresh_bin != 0;
+  r->wide = fullest >= (1u << 24) ? 1u : 0u;
 }
 // Groups of rows that the warps of the selection take one at a time by a client's counter: three quarters of a client in large
 // groups, three quarters of the rest in groups a quarter as large, the last ones small, so that a block's warps finish about
@@ -227,7 +233,7 @@ CVLC_HD inline SelectGroups select_groups(const Partition& P, uint32_t n) {
 struct EncLayout {
   uint32_t n;
   uint64_t capacity;             // candidate slots per client
-  uint64_t select_tiles;         // per client, of the look-back selection's smaller tiles
+  uint64_t select_tiles;         // per client, of the look-back selection
   uint64_t sort_tiles_max;       // per client
   size_t off_rank;               // ClientRank[n]
   size_t off_sort_prefix;        // uint32[n + 1]: first sort tile of every client
@@ -242,16 +248,41 @@ struct EncLayout {
   size_t off_ghist;              // uint64[n][4][512] digit histograms
   size_t off_gbase;              // uint64[n][4][512] their exclusive scans
   size_t off_select_state;       // uint64[n][select_tiles]
-  size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]; ranked by partition: the ranking's lists, a half each
+  size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]
+  // ranked by partition, in the place of the digit passes' states (see RankArgs):
+  size_t off_list[2];            // cells left over for a warp and for a block
+  size_t off_big;                // buckets that a block cannot hold, per round
+  size_t off_piece;              // pieces of them, per round
+  size_t off_splitter, off_part_count, off_part_start;  // per bucket: the values its parts begin with, what they hold, where they begin
+  size_t off_base;               // per piece and part: what earlier pieces have of the part
+  size_t off_part;               // parts to rank
   size_t off_buf_a, off_buf_b;   // uint64[n][capacity]
   size_t total;
+};
+
+// A bucket that a block cannot hold, a piece of one, and a part of one that a block can hold (see rank_big)
+constexpr uint32_t kBigPart = 3072;   // candidates of a part, about
+constexpr uint32_t kBigParts = 1024;  // most parts of a bucket in one round
+constexpr uint32_t kBigPiece = 8192;  // candidates of a piece at least
+constexpr uint32_t kBigSlot = 1024;   // candidates per entry of the tables of parts
+struct BigBucket {
+  uint64_t pos;         // where it begins among all clients' candidates
+  uint64_t from, to;    // its values lie in [from, to)
+  uint64_t last;        // larger values are never sent
+  uint32_t m, parts;
+  uint32_t counted, pad;  // pieces counted
+};
+struct BigPart {
+  uint64_t pos;
+  uint32_t n, in_b;               // in_b: it lies in the second buffer
+  uint32_t first_key, last_key;   // its keys lie between them, the larger one first
 };
 
 static inline EncLayout enc_layout(uint64_t d, uint32_t n, uint64_t capacity) {
   EncLayout L;
   L.n = n;
   L.capacity = capacity;
-  L.select_tiles = select_tiles_of(d, kSortThreads);
+  L.select_tiles = select_tiles_of(d);
   L.sort_tiles_max = (capacity + kSortTile - 1) / kSortTile;
   L.off_rank = 256;
   L.off_sort_prefix = align256(L.off_rank + (size_t)n * sizeof(ClientRank));
@@ -270,7 +301,24 @@ static inline EncLayout enc_layout(uint64_t d, uint32_t n, uint64_t capacity) {
   L.off_buf_a = align256(L.off_sort_state + (size_t)kSortPasses * n * L.sort_tiles_max * kDigits * 8);
   L.off_buf_b = align256(L.off_buf_a + (size_t)n * capacity * 8);
   L.total = align256(L.off_buf_b + (size_t)n * capacity * 8);
+  // The lists, in the place of the digit passes' states.  Cells: at most one for every 49 candidates, and one for every 257 and one
+  // per tile of at least 1024.  A large bucket has more than kRankItems candidates and at most one part for every kBigPart and one.
+  const size_t all = (size_t)n * capacity, buckets = all / kRankItems + 1;
+  L.off_list[0] = L.off_sort_state;
+  L.off_list[1] = L.off_list[0] + align256((all / 49 + 1) * 16);
+  L.off_big = L.off_list[1] + align256((all / 257 + all / 1024 + n + 1) * 16);
+  L.off_piece = L.off_big + align256(buckets * kBigRounds * sizeof(BigBucket));
+  L.off_splitter = L.off_piece + align256((all / kBigPiece + buckets) * kBigRounds * 8);
+  L.off_part_count = L.off_splitter + align256((all / kBigSlot + 1) * 8);
+  L.off_part_start = L.off_part_count + align256((all / kBigSlot + 1) * 4);
+  L.off_base = L.off_part_start + align256((all / kBigSlot + 1) * 4);
+  L.off_part = L.off_base + (all / kBigPiece + buckets) * kBigParts * 4;
   return L;
+}
+// behind the last list; never behind the states' end, off_buf_a (a state takes 16 KB for up to 5120 candidates)
+static inline size_t enc_lists_end(const EncLayout& L) {
+  const size_t all = (size_t)L.n * L.capacity;
+  return L.off_part + (all / kBigPart + all / kRankItems + 1) * kBigRounds * sizeof(BigPart);
 }
 
 // decode workspace
@@ -286,7 +334,7 @@ CVLC_HD constexpr size_t dec_ws_bytes(uint32_t n) { return align256(dec_off_meta
 
 enum KernelId {
   kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
-  kKSort, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
+  kKRankRest, kKSort, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
   kKPlanLiteral, kKEcAccumulate, kKPackUnframed, kKDecodeUnframed, kNumKernelIds
 };
 
@@ -357,7 +405,7 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
                                 unsigned long long k_lo, unsigned long long k_hi, double P_min, double P_max, double tol,
                                 cvlc_literal_plan_t* out, double* P_star, void* ws, cudaStream_t st);
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
-// ranking by partition (after the selection); returns at once on the device where the batch is ranked by digit passes
+// ranking by partition (after the selection)
 cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr

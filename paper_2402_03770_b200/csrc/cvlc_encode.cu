@@ -1,8 +1,9 @@
-// Encoding kernels (Algorithm 1, steps 15-17), batched over clients: top-k candidate
-// selection by the plan's histogram threshold, stable LSD radix ranking of the candidates
-// by |x|, the per-packet centroid distribution (PQ: minimum and maximum; QSGD: l2-norm),
-// stochastic quantization with Philox4x32-10 (PQ or QSGD) and bit packing of
-// (position ID, centroid ID) pairs into fixed-size packets (Fig. 2).
+// Encoding kernels (Algorithm 1, steps 15-17), batched over clients: top-k candidate selection by the
+// plan's histogram threshold, into the buckets of the ranking by partition (cvlc_rank.cu) or, without the
+// plan's workspace, in index order in front of a stable LSD radix ranking by |x|; the per-packet
+// centroid distribution (PQ: minimum and maximum; QSGD: l2-norm), stochastic quantization with
+// Philox4x32-10 (PQ or QSGD) and bit packing of (position ID, centroid ID) pairs into fixed-size packets
+// (Fig. 2).
 #include <string.h>
 
 #include "cvlc_common.cuh"
@@ -11,15 +12,6 @@
 #include "cvlc_rank.cuh"
 
 namespace cvlc {
-
-// Whether an earlier kernel of the call has reported an error.  Other blocks may set the word while this kernel
-// runs, so one thread reads it and the whole block takes the same branch.
-__device__ __forceinline__ bool block_sees_error(const int32_t* status) {
-  __shared__ int s_err;
-  if (threadIdx.x == 0) s_err = *reinterpret_cast<const volatile int32_t*>(status);
-  __syncthreads();
-  return s_err != 0;
-}
 
 __device__ __forceinline__ uint32_t sort_tiles_of(unsigned long long n_candidates, unsigned long long capacity) {
   const unsigned long long nc = n_candidates < capacity ? n_candidates : capacity;
@@ -37,16 +29,17 @@ __global__ void __launch_bounds__(256)
 k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape,
               const __grid_constant__ EncLayout L, const unsigned char* plan_ws) {
   __shared__ unsigned long long s_total;
-  __shared__ int s_bad, s_pass3, s_lsd;
+  __shared__ int s_bad, s_pass3;
   __shared__ uint32_t s_most, s_most_split;  // candidates of the largest client / of the largest one that needs the partition
   __shared__ uint32_t s_tiles[CVLC_MAX_BATCH];  // sort tiles of every client
   const uint32_t n = batch.n;
+  const unsigned long long most_sent = (unsigned long long)shape.R * shape.cap[1];  // no plan sends more
+  const uint32_t limit = most_sent < 0xFFFFFFFFull ? (uint32_t)most_sent : 0xFFFFFFFFu;
   pdl_enter();
   if (threadIdx.x == 0) {
     s_total = 0;
     s_bad = 0;
     s_pass3 = 0;
-    s_lsd = 0;
     s_most = s_most_split = 0;
   }
   // the plan's tables must have been made for this very batch: looked at only if the header says so
@@ -67,12 +60,11 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
         ClientRank r;
         const uint32_t top = plan->top_bin < CVLC_HIST_BINS ? plan->top_bin : CVLC_HIST_BINS - 1;
         const uint32_t nb = plan->thresh_bin <= top ? top - plan->thresh_bin + 1 : 1;
-        if (!rank_shape(nb, max_bin[c], plan->thresh_bin, &r)) s_lsd = 1;
+        rank_shape(nb, max_bin[c], &r);
         r.n = (uint32_t)(plan->n_candidates < L.capacity ? plan->n_candidates : L.capacity);
         r.keytop = sort_keytop(plan);
         r.top_bin = top;
-        r.pad = 0;
-        atomicMax(&s_most, r.n);
+        atomicMax(&s_most, r.n < limit ? r.n : limit);  // buckets from the limit on are not ranked
         if (r.split) atomicMax(&s_most_split, r.n);
         if (blockIdx.x == 0) reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;
       }
@@ -133,10 +125,13 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     if (plan_ws && !tables && !s_bad) s_bad = CVLC_ERR_PLAN_MISMATCH;
     hdr->max_sort_tiles = mx;
     hdr->status = s_bad;
-    hdr->lsd = !plan_ws ? kRankDigits : s_lsd ? kRankAllDigits : kRankPartition;
-    hdr->select_ticket = hdr->split_ticket = hdr->rank_ticket = hdr->sort_ticket = 0;
-    hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
+    hdr->limit = limit;
+    hdr->select_ticket = hdr->split_ticket = hdr->rank_ticket = 0;
+    hdr->sort_ticket = 0;
     for (int p = 0; p < 8; ++p) hdr->sort_done[p] = 0;
+    hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
+    for (int r = 0; r < kBigRounds; ++r) hdr->big[r] = BigRound{};
+    hdr->part_n = hdr->part_next = 0;
     hdr->split_tiles = (s_most_split + kRankSplitTile - 1) / kRankSplitTile;
     // tiles small enough that the batch gives every SM several
     const uint64_t want = ((uint64_t)run * kSortTile + 4 * kNumSM - 1) / (4 * kNumSM);
@@ -144,7 +139,6 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     while (window > 1024 && window / 2 >= want) window >>= 1;
     hdr->window = window;
     hdr->rank_tiles = (s_most + window - 1) / window;
-    hdr->total_sort_tiles = run;
   }
   // ranked by partition: the result is in the first buffer (the digit passes write a mask of their own)
   if (plan_ws)
@@ -159,16 +153,16 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
 // Tiles of 8192 coordinates are handed out by an atomic ticket (tile-major, clients interleaved:
 // the tiles in flight at any time are a few consecutive tiles of every client), so every
 // predecessor of a tile is running or done; the look-back reads 512 predecessors per step.
-// Used when the plan's workspace is not available and in front of the digit passes.
+// Used when the plan's workspace is not available, in front of the digit passes.
 
-template <int THREADS>
 __device__ __forceinline__ void select_lookback_tile(const Batch& batch, uint64_t d, unsigned char* ws, const EncLayout& L, uint64_t gt) {
+  constexpr int THREADS = kSelectThreads;
   __shared__ unsigned long long s_warp_incl[THREADS / 32];
   __shared__ unsigned long long s_look_sum[THREADS / 32];
   __shared__ uint32_t s_look_flag[THREADS / 32];
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t tiles_per_client = select_tiles_of(d, THREADS);
+  const uint64_t tiles_per_client = select_tiles_of(d);
   {
     const uint64_t tile = gt / batch.n;
     const uint32_t c = (uint32_t)(gt - tile * batch.n);
@@ -301,14 +295,14 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
-  const uint64_t total_tiles = select_tiles_of(d, kSelectThreads) * batch.n;
+  const uint64_t total_tiles = select_tiles_of(d) * batch.n;
   while (true) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&hdr->select_ticket, 1u);
     __syncthreads();
     const uint64_t gt = s_tile;
     if (gt >= total_tiles) break;
     __syncthreads();  // everyone has read the ticket
-    select_lookback_tile<kSelectThreads>(batch, d, ws, L, gt);
+    select_lookback_tile(batch, d, ws, L, gt);
   }
 }
 
@@ -353,9 +347,27 @@ __device__ __forceinline__ uint32_t warp_inclusive(uint32_t v) {
   return v;
 }
 
-// red.add of four fp32 counts at once: counts stay below 2^24 in this mode (see rank_shape), where they are exact
+// red.add of four fp32 counts at once: below 2^24 they are exact (see rank_shape)
 __device__ __forceinline__ void add_counts4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t e) {
   asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"((float)a), "f"((float)b), "f"((float)c), "f"((float)e) : "memory");
+}
+
+// ... and of four whole ones, kept out of the kernel's code (inlined it cost the selection 1.5 %)
+__device__ __noinline__ void add_counts4_wide(float* p, uint4 v) {
+  uint32_t* whole = reinterpret_cast<uint32_t*>(p);
+  if (v.x) atomicAdd(whole, v.x);
+  if (v.y) atomicAdd(whole + 1, v.y);
+  if (v.z) atomicAdd(whole + 2, v.z);
+  if (v.w) atomicAdd(whole + 3, v.w);
+}
+
+// a sub-bucket that a block of the ranking cannot hold
+__device__ __noinline__ void list_bucket(EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, const ClientRank& r, uint32_t sh,
+                                         uint32_t bucket, uint32_t start, uint32_t m) {
+  atomicAdd(&hdr->big[0].slots, m / kBigSlot);
+  const u64 lo = (u64)~r.keytop + ((u64)bucket << sh), end = lo + (1ull << sh);  // the last bucket may reach below key 0
+  reinterpret_cast<BigBucket*>(ws + L.off_big)[atomicAdd(&hdr->big[0].n, 1u)] =
+      BigBucket{(u64)c * L.capacity + start, lo << 32, end >> 32 ? ~0ull : end << 32, ~0ull, m, big_parts(m), 0u, 0u};
 }
 
 __global__ void __launch_bounds__(kSelThreads, 1)
@@ -368,7 +380,7 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   __shared__ uint32_t s_client, s_taken, s_scan[kSelThreads / 32];
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (rank_skips(hdr)) return;
+  if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = batch.n;
   const uint32_t rows = (uint32_t)part.rows, held_rows = ((uint32_t)(d >> 2) + kRowUnits - 1) / kRowUnits;  // with coordinates
@@ -417,8 +429,8 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     const float* __restrict__ x = batch.c[c].x;
     const float4* __restrict__ xv = reinterpret_cast<const float4*>(x);
     const uint16_t* __restrict__ row_max = reinterpret_cast<const uint16_t*>(plan_ws + plan_off_row_max(n)) + (size_t)c * rows;
-    const uint32_t thresh_bin = batch.c[c].plan->thresh_bin, thresh = thresh_bin << 19, keytop = r.keytop;  // thresh > 0 in this mode
-    const float below_thresh = __uint_as_float(thresh - 1u);                        // key >= thresh <=> |x| > below_thresh
+    const uint32_t thresh_bin = batch.c[c].plan->thresh_bin, thresh = thresh_bin << 19, keytop = r.keytop;
+    const float below_thresh = thresh ? __uint_as_float(thresh - 1u) : -1.0f;       // key >= thresh <=> |x| > below_thresh
     const uint32_t sh_coarse = 19 + r.group, sh_sub = sh_coarse - r.sub_bits;
     unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
     uint32_t* fill = reinterpret_cast<uint32_t*>(ws + L.off_bin_fill) + (size_t)c * kRankCoarse;
@@ -613,6 +625,10 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
 #pragma unroll
       for (int j = 0; j < 16; ++j)  // the difference of two distinct floats never rounds to zero: its sign is the flag
         m = __funnelshift_l(__float_as_uint(__fsub_rn(below_thresh, fabsf(__uint_as_float(bits[j])))), m, 1);
+      if (thresh == 0) {  // zeros are candidates: not those that stand for rows and coordinates there are not
+        const uint32_t there = (uint32_t)lane < step_rows[0] ? nvec - (first >> 2) : 0u;  // units of the update from this lane's row on
+        if (there < 4) m &= 0xFFFF0000u >> (4 * there);
+      }
 #pragma unroll
       for (int i = 0; i + 1 < kSelStages; ++i) {
         step_row[i] = step_row[i + 1];
@@ -652,7 +668,8 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
       for (uint32_t i = tid; i < n_sub4; i += kSelThreads) {
         const uint4 v = sub4[i];
         if (v.x | v.y | v.z | v.w) {
-          add_counts4(count + 4 * i, v.x, v.y, v.z, v.w);
+          if (r.wide) add_counts4_wide(count + 4 * i, v);
+          else add_counts4(count + 4 * i, v.x, v.y, v.z, v.w);
           sub4[i] = make_uint4(0u, 0u, 0u, 0u);
         }
       }
@@ -674,17 +691,14 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
         uint32_t* start = reinterpret_cast<uint32_t*>(ws + L.off_sub_start) + (size_t)c * (kRankSubs + 64);
         uint32_t* next = reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs;
         constexpr uint32_t kMine = 8;
-        uint32_t carry = 0, largest = 0;
+        uint32_t carry = 0;
         for (uint32_t base = 0; base < n_sub; base += kSelThreads * kMine) {
           const uint32_t i0 = base + (uint32_t)tid * kMine;
           uint32_t v[kMine], sum = 0;
 #pragma unroll
-          for (uint32_t e = 0; e < kMine; ++e) v[e] = (i0 + e < n_sub) ? (uint32_t)__ldcg(count + i0 + e) : 0u;
+          for (uint32_t e = 0; e < kMine; ++e) v[e] = (i0 + e < n_sub) ? (r.wide ? __float_as_uint(__ldcg(count + i0 + e)) : (uint32_t)__ldcg(count + i0 + e)) : 0u;
 #pragma unroll
-          for (uint32_t e = 0; e < kMine; ++e) {
-            sum += v[e];
-            largest = v[e] > largest ? v[e] : largest;
-          }
+          for (uint32_t e = 0; e < kMine; ++e) sum += v[e];
           uint32_t incl = sum;
 #pragma unroll
           for (int off = 1; off < 32; off <<= 1) {
@@ -704,6 +718,7 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
             if (i0 + e < n_sub) {
               start[i0 + e] = run;
               next[i0 + e] = run;
+              if (v[e] > kRankItems && run < hdr->limit && run + v[e] <= r.n) list_bucket(hdr, ws, L, c, r, sh_sub, i0 + e, run, v[e]);
             }
             run += v[e];
           }
@@ -711,7 +726,6 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
           __syncthreads();
         }
         if (tid == 0) start[n_sub] = carry;
-        if (largest > kRankLargest) hdr->lsd = kRankAllDigits;
       }
     }
     __syncthreads();
@@ -733,15 +747,13 @@ __device__ __forceinline__ uint32_t sort_digit(unsigned long long pair, int pass
 // ===================================================================================
 // Sort key = keytop - key, keytop = the largest key of the client's highest non-empty histogram
 // bin, so the key only spans the bins between the threshold and the top: 19 + log2(#bins) bits.
-// Digits of 9, 9, 9, 4 bits, in one kernel of eight phases: the counters cleared and the candidates
-// selected in index order (unless that has been done), histograms of all four digits, their scans, and
-// per digit a single pass over tiles (tile-major with the clients interleaved; decoupled
-// look-back per digit value).  All phases draw from one ticket counter, and an item waits until the
-// phase before its own is complete: the items it waits for have lower tickets, so blocks that are
-// running hold them.  A pass whose digit is the same for every candidate of a client (normally the
-// fourth) is skipped for that client; which buffer holds its data after pass q follows from the
-// mask of skipped passes.  Used where the ranking by partition is not (see rank_shape); otherwise the kernel works off what that
-// has left over (see rank_lists).
+// Digits of 9, 9, 9, 4 bits, in one kernel of six phases: histograms of all four digits, their scans, and
+// per digit a single pass over tiles (tile-major with the clients interleaved; decoupled look-back per digit
+// value).  All phases draw from one ticket counter, and an item waits until the phase before its own is
+// complete: the items it waits for have lower tickets, so blocks that are running hold them.  A pass whose
+// digit is the same for every candidate of a client (normally the fourth) is skipped for that client; which
+// buffer holds its data after pass q follows from the mask of skipped passes.  Used where the plan's
+// workspace is not at hand.
 
 // two adjacent look-back words in one 128-bit access (each 64-bit half is its own atomic access)
 __device__ __forceinline__ void ld_relaxed2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
@@ -762,10 +774,7 @@ struct SortShared {
 };
 
 constexpr size_t kSortSharedBytes = (sizeof(SortShared) + 15) & ~(size_t)15;
-constexpr size_t sort_smem_bytes(uint32_t n) {
-  const size_t passes = kSortSharedBytes + (size_t)kSortTile * 8 + (4 * (size_t)n + 1) * 4;
-  return passes > sizeof(RankShared) ? passes : sizeof(RankShared);
-}
+constexpr size_t sort_smem_bytes(uint32_t n) { return kSortSharedBytes + (size_t)kSortTile * 8 + (4 * (size_t)n + 1) * 4; }
 
 // One tile of one digit pass.  FULL: the tile holds kSortTile items (no bounds checks in the item loops).
 // Thread t < 256 owns the digit values 2t and 2t + 1 in the counting, scan and look-back steps.
@@ -941,10 +950,9 @@ __device__ __forceinline__ void sort_tile(SortShared& sh, unsigned long long* __
 }
 
 constexpr uint32_t kSortHistTiles = 8;   // tiles of a histogram item
-constexpr size_t kSortClear = 1 << 16;   // bytes of a clearing item
 
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks)
-k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start) {
+k_sort(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
   static_assert(kSortThreads * 2 == kDigits && kSortTile <= 0xFFFF, "two digit values per thread; 16-bit slots");
   extern __shared__ __align__(16) unsigned char s_raw[];
   SortShared& sh = *reinterpret_cast<SortShared*>(s_raw);
@@ -956,10 +964,6 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
-  if (hdr->lsd == kRankPartition) {  // only what the ranking has left over
-    if (hdr->list_n[0] | hdr->list_n[1]) rank_lists<kSortThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, rank_args(ws, L, bin_start, hdr, batch.n));
-    return;
-  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = batch.n;
   {
@@ -974,15 +978,11 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
   for (int i = tid; i < (kSortThreads / 32) * kDigits; i += kSortThreads) (&sh.mm[0][0])[i] = 0u;
   if (tid == 0) sh.tile = atomicAdd(&hdr->sort_ticket, 1u);
   __syncthreads();
-  // first items of the phases: 0 clearing, 1 selection, 2 histograms, 3 scans, 4 .. 7 digit passes
-  const bool all = hdr->lsd == kRankAllDigits;
-  const size_t clear_bytes = L.off_buf_a - L.off_ghist;
+  // first items of the phases: 2 histograms, 3 scans, 4 .. 7 digit passes
   const uint32_t n_pass = hdr->max_sort_tiles * n;
   uint32_t first_item[9];
-  first_item[0] = 0;
-  first_item[1] = all ? (uint32_t)((clear_bytes + kSortClear - 1) / kSortClear) : 0u;
-  first_item[2] = first_item[1] + (all ? (uint32_t)(select_tiles_of(d, kSortThreads) * n) : 0u);
-  first_item[3] = first_item[2] + (hdr->max_sort_tiles + kSortHistTiles - 1) / kSortHistTiles * n;
+  first_item[0] = first_item[1] = first_item[2] = 0;
+  first_item[3] = (hdr->max_sort_tiles + kSortHistTiles - 1) / kSortHistTiles * n;
   first_item[4] = first_item[3] + n;
 #pragma unroll
   for (int p = 5; p < 9; ++p) first_item[p] = first_item[p - 1] + n_pass;
@@ -990,7 +990,7 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
   unsigned long long* gbase_all = reinterpret_cast<unsigned long long*>(ws + L.off_gbase);
   uint32_t* pass_mask = reinterpret_cast<uint32_t*>(ws + L.off_pass_mask);
   uint4* s_wc4 = reinterpret_cast<uint4*>(&sh.wc[0][0]);
-  int phase = all ? 0 : 2;
+  int phase = 2;
 
   while (true) {
     const uint32_t gt = sh.tile;
@@ -999,10 +999,10 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
     // the next ticket is fetched while this item is worked on
     uint32_t next = 0;
     if (tid == 0) next = atomicAdd(&hdr->sort_ticket, 1u);
-    int my_phase = 0;
+    int my_phase = 2;
     uint32_t want = 0, first = 0;  // items of the phase before; first item of this one
 #pragma unroll
-    for (int p = 1; p < 8; ++p) {
+    for (int p = 3; p < 8; ++p) {
       if (gt >= first_item[p]) {
         my_phase = p;
         want = first_item[p] - first_item[p - 1];
@@ -1027,13 +1027,7 @@ k_sort(const Batch batch, uint64_t d, unsigned char* ws, const __grid_constant__
       phase = my_phase;
       __syncthreads();
     }
-    if (phase == 0) {
-      ulonglong2* p = reinterpret_cast<ulonglong2*>(ws + L.off_ghist + (size_t)gt * kSortClear);
-      const size_t left = clear_bytes - (size_t)gt * kSortClear, m = (left < kSortClear ? left : kSortClear) / 16;
-      for (size_t i = tid; i < m; i += kSortThreads) p[i] = make_ulonglong2(0ull, 0ull);
-    } else if (phase == 1) {
-      select_lookback_tile<kSortThreads>(batch, d, ws, L, gt - first);
-    } else if (phase == 2) {
+    if (phase == 2) {
       // digit counts of up to kSortHistTiles tiles of a client
       uint32_t* cnt = reinterpret_cast<uint32_t*>(s_items);
       const uint32_t g = (gt - first) / n, c = (gt - first) - g * n;
@@ -1199,7 +1193,8 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     const uint32_t tot_packets = __shfl_sync(kFull, cum, 31);
     const unsigned long long tot_records = __shfl_sync(kFull, zc, 31);
     const bool qsgd_one_bit = QSGD && __shfl_sync(kFull, ny, 31) != 0;  // a one-bit QSGD code holds no level
-    if (tot_packets != shape.R || tot_records != plan->k || tot_records == 0 || tot_records > plan->n_candidates || qsgd_one_bit) {
+    if (tot_packets != shape.R || tot_records != plan->k || tot_records == 0 || tot_records > plan->n_candidates ||
+        tot_records > (unsigned long long)shape.R * shape.cap[1] || qsgd_one_bit) {
       if (blockIdx.x == 0 && tid == 0) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
       return;
     }
@@ -1439,6 +1434,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     attr_done[dev] = true;
   }
   const EncLayout L = enc_layout(shape.d, n, capacity);
+  if (enc_lists_end(L) > L.off_buf_a) return cudaErrorInvalidValue;
   unsigned char* w = static_cast<unsigned char*>(ws);
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
   // packet words and two more; QSGD: and the squares of a packet's values
@@ -1458,15 +1454,12 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     e = launch_rank(batch, L, pws, w, sms, st);
     if (e != cudaSuccess) return e;
   } else {
-    const uint64_t want = select_tiles_of(shape.d, kSelectThreads) * n;
+    const uint64_t want = select_tiles_of(shape.d) * n;
     const unsigned grid = (unsigned)(want < (uint64_t)(4 * kNumSM) ? want : 4 * kNumSM);
     launch_kernel(kKSelectLookback, k_select_lookback, grid, kSelectThreads, 0, st, true, batch, shape.d, w, L);
-  }
-  {
-    const uint64_t want = L.sort_tiles_max * n;
-    const unsigned most = kSortMinBlocks * sms, grid = (unsigned)(want < (uint64_t)most ? want : most);
-    launch_kernel(kKSort, k_sort, grid, kSortThreads, sort_smem_bytes(n), st, true, batch, shape.d, w, L,
-                  pws ? reinterpret_cast<const uint32_t*>(pws + plan_off_bin_start(n)) : nullptr);
+    const uint64_t tiles = L.sort_tiles_max * n;
+    launch_kernel(kKSort, k_sort, (unsigned)(tiles < kSortMinBlocks * kNumSM ? tiles : kSortMinBlocks * kNumSM), kSortThreads, sort_smem_bytes(n), st, true,
+                  batch, w, L);
   }
   if (wait_before_pack) {
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);

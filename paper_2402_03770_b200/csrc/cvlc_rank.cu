@@ -3,7 +3,7 @@
 // The selection has left every client's candidates in coarse buckets, ranges of the sort key inv = keytop - key whose
 // starts are known, in no particular order inside a bucket.  k_rank_split moves the candidates of a client with large
 // buckets on into sub-buckets (the next bits of inv); k_rank then ranks whole buckets in shared memory by (inv, index) and
-// writes them out in order; cells of equal keys and buckets beyond a block's shared memory go on lists that the kernel after
+// writes them out in order; cells of equal keys and buckets beyond a block's shared memory are on lists that the kernel after
 // it works off.  The order is total, so the result does not depend on how the candidates arrived.  Against a
 // stable radix sort of the same keys (three passes of 9 bits) a candidate is moved once or twice instead of three times
 // and costs one counting and one placing shared-memory atomic per move instead of a stable rank among the lanes of a warp.
@@ -34,7 +34,7 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
   __shared__ uint32_t s_next;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (rank_skips(hdr)) return;
+  if (block_sees_error(&hdr->status)) return;
   const uint32_t n = batch.n, tickets = hdr->split_tiles * n;
   if (tickets == 0) return;
   const int tid = threadIdx.x;
@@ -110,8 +110,8 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
 // Tiles of buckets (RankTile), drawn by ticket; the next tile's buckets are searched for by two warps while the others compare.
 // No calls and no per-client state in registers: 62 of them and no spills (with the crowded cells ranked here, 80 bytes of
 // spills and waiting warps).  Bound by instruction issue, about 100 instructions per warp of candidates, and by a tile's barriers.
-// 79 M candidates of 100 clients: 750 -> 555 us (and 38 for what is left over); 41 M of 50, every seventh layer on a grid:
-// 784 -> 303 (and 143).  Half as many cells, or blocks of 256 threads with half the window, are within 5 %; twice the cells cost
+// 79 M candidates of 100 clients: 750 -> 555 us (and 38 for what is left over, see k_rank_rest); 41 M of 50, every seventh layer on
+// a grid: 784 -> 303 (and 143).  Half as many cells, or blocks of 256 threads with half the window, are within 5 %; twice the cells cost
 // 20 % (clearing and scanning them), keeping an item's place from the counting 10 % (the atomic then returns a value).
 __global__ void __launch_bounds__(kRankThreads, 2)
 k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all) {
@@ -121,7 +121,7 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   __shared__ RankArgs s_args;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (rank_skips(hdr)) return;
+  if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x;
   if (tid == 0) {
     s_args = rank_args(ws, L, bin_start_all, hdr, batch.n);
@@ -135,8 +135,7 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
     if (T.ticket >= s_args.tickets) return;
     if (tid == 0) s_tile[slot ^ 1u].ticket = atomicAdd(&hdr->rank_ticket, 1u);
     const uint32_t at = T.start[0], m = T.start[1] - at;
-    // (a bucket before the tile's first matters where its part in the window is the tile's)
-    const bool large = m > kRankItems || at - T.before > kRankItems;
+    const bool large = m > kRankItems;
     auto leave = [&](uint32_t list, u64 what, uint32_t items) { s_args.list[list][atomicAdd(&hdr->list_n[list], 1u)] = make_ulonglong2(what, items); };
     if (!large && m != 0) {
       const uint32_t sh = T.sh, base = T.bucket[0] << sh;
@@ -154,6 +153,19 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   }
 }
 
+// What the ranking has left over (see rank_lists)
+__global__ void __launch_bounds__(kRankThreads, 2)
+k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ RankArgs s_args;
+  pdl_enter();
+  EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
+  if (block_sees_error(&hdr->status)) return;
+  if ((hdr->list_n[0] | hdr->list_n[1] | hdr->big[0].n) == 0) return;
+  if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n);
+  rank_lists<kRankThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, s_args);
+}
+
 cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
   static bool attr_done[64] = {};
   int dev = 0;
@@ -162,6 +174,8 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
     e = cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankShared));
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_rank_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankShared));
+    if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
   auto blocks = [](uint64_t tiles, uint64_t most) -> unsigned { return (unsigned)(tiles < most ? tiles : most); };
@@ -169,6 +183,8 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
                 batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
   launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start);
+  launch_kernel(kKRankRest, k_rank_rest, blocks((L.capacity + kRankItems - 1) / kRankItems * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true,
+                batch, ws, L, bin_start);
   return cudaGetLastError();
 }
 

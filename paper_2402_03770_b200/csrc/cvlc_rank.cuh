@@ -1,6 +1,7 @@
 // Ranking of tiles of candidates in shared memory: what the ranking kernel and the kernel that works its left-overs off share.
 #pragma once
 #include "cvlc_common.cuh"
+#include "cvlc_lookback.cuh"
 
 namespace cvlc {
 
@@ -10,15 +11,14 @@ constexpr uint32_t kWarpCell = 256;     // one of up to this many is ranked by o
 
 typedef unsigned long long u64;
 
-// Whether the call has failed or is not ranked by partition.  While blocks of the selection start, others of the same launch may
-// write either word (an update that is not the plan's, a bucket too large for the partition), so one thread reads them and the
-// block takes one branch: warps that part here would leave the others of their block at its barriers with work not done.
-__device__ __forceinline__ bool rank_skips(const EncHeader* hdr) {
-  __shared__ int s_skip;
-  if (threadIdx.x == 0)
-    s_skip = *reinterpret_cast<const volatile int32_t*>(&hdr->status) != 0 || *reinterpret_cast<const volatile uint32_t*>(&hdr->lsd) != kRankPartition;
+// Whether an earlier kernel of the call has reported an error.  Other blocks may set the word while this kernel runs or blocks of
+// it start, so one thread reads it and the whole block takes the same branch: warps that part here would leave the others of their
+// block at its barriers with work not done.
+__device__ __forceinline__ bool block_sees_error(const int32_t* status) {
+  __shared__ int s_err;
+  if (threadIdx.x == 0) s_err = *reinterpret_cast<const volatile int32_t*>(status);
   __syncthreads();
-  return s_skip != 0;
+  return s_err != 0;
 }
 
 struct RankShared {
@@ -346,10 +346,10 @@ __device__ __forceinline__ bool rank_equal_by_warp(uint32_t* cell, u64* items, u
   return true;
 }
 
-// Ranks the n <= kRankItems items of a cell of many keys in their place; by the whole block.  They are spread over equal ranges of
-// (key, index) between the least and the largest of each.  False, and nothing done, if a range has too many.
+// Ranks the n <= kRankItems items of a cell of many keys and writes them out (in their place, too); by the whole block.  They are
+// spread over equal ranges of (key, index) between the least and the largest of each.  False, and nothing done, if a range has too many.
 template <int THREADS>
-__device__ __noinline__ bool rank_spread(RankShared& s, u64* at, uint32_t n) {
+__device__ __noinline__ bool rank_spread(RankShared& s, const u64* at, uint32_t n, u64* out) {
   __shared__ uint32_t s_least[2], s_most[2], s_no;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 2) {
@@ -401,120 +401,27 @@ __device__ __noinline__ bool rank_spread(RankShared& s, u64* at, uint32_t n) {
   for (uint32_t p = tid; p < n; p += THREADS) {
     const u64 v = s.items[p];
     const uint32_t k = cell_of(v);
-    at[rank_in_cell(s.items, v, (&s.cell[k])[-1], s.cell[k])] = to_item(v);
+    out[rank_in_cell(s.items, v, (&s.cell[k])[-1], s.cell[k])] = to_item(v);
   }
   __syncthreads();
   return true;
 }
 
-// Ranks n <= kRankItems items, most of them of one key or nearly equal, in their place; by the whole block
+// Ranks n <= kRankItems items, most of them of one key or nearly equal, and writes them out (in their place, too); by the whole block
 template <int THREADS>
-__device__ __noinline__ void rank_cell(RankShared& s, u64* at, uint32_t n) {
+__device__ __noinline__ void rank_cell(RankShared& s, const u64* at, uint32_t n, u64* out) {
   for (int attempt = 0; attempt < 3; ++attempt) {
     if (attempt != 1) {
       for_items<THREADS>(at, n, [&](uint32_t i, u64 item) { s.items[i] = to_value(item); });
       __syncthreads();
     }
     if (attempt == 0) {
-      if (n <= kCells / 2 ? rank_equal<THREADS, kCellBits - 1>(s, s.items, n, at) : rank_equal<THREADS, kCellBits>(s, s.items, n, at)) return;
-    } else if (attempt == 1 && rank_spread<THREADS>(s, at, n)) {
+      if (n <= kCells / 2 ? rank_equal<THREADS, kCellBits - 1>(s, s.items, n, out) : rank_equal<THREADS, kCellBits>(s, s.items, n, out)) return;
+    } else if (attempt == 1 && rank_spread<THREADS>(s, at, n, out)) {
       return;
     }
   }
-  rank_by_block<THREADS>(s.items, n, at);
-}
-
-// Boundaries near ranks x[0] and x[1] of the m values of src, all in [lo, hi): a value and how many of src lie below it.  The range
-// around a rank is narrowed until at most kCutRest values are left in it; the boundary is where that range starts.  A function of the
-// set of values and the rank alone, so that neighbouring tiles agree on it.  As long as both ranks lie in one range, one pass over
-// the values serves both: of equal keys two passes find both boundaries.
-constexpr uint32_t kCutRest = kRankItems - kRankWindow;
-struct Cut {
-  u64 value;
-  uint32_t below;
-};
-struct CutSearch {
-  u64 lo, hi;
-  uint32_t x, below;
-  bool open;
-};
-template <int THREADS>
-__device__ __noinline__ void cut_near(RankShared& s, const u64* __restrict__ src, uint32_t m, CutSearch& a, CutSearch& b) {
-  __shared__ uint32_t s_cell[2], s_below[2], s_count[2];
-  const int tid = threadIdx.x;
-  for (int level = 0; level < 16 && (a.open || b.open); ++level) {  // 63 bits, 12 a level, each rank on its own at worst
-    const u64 lo = a.open ? a.lo : b.lo, hi = a.open ? a.hi : b.hi;
-    const bool for_a = a.open, for_b = b.open && b.lo == lo && b.hi == hi;
-    if (lo >= hi) {
-      if (for_a) a.open = false;
-      if (for_b) b.open = false;
-      continue;
-    }
-    const u64 span = hi - lo - 1;
-    const int sh = span < kCells ? 0 : 64 - __clzll((long long)span) - (int)kCellBits;  // span >> sh below kCells
-    for (uint32_t i = tid; i < kCells; i += THREADS) s.cell[i] = 0;
-    if (tid < 2) s_cell[tid] = s_below[tid] = s_count[tid] = 0;
-    __syncthreads();
-    for_items<THREADS>(src, m, [&](uint32_t, u64 item) {
-      const u64 v = to_value(item);
-      if (v >= lo && v < hi) atomicAdd(&s.cell[(uint32_t)((v - lo) >> sh)], 1u);
-    });
-    __syncthreads();
-    const uint32_t total = scan_cells<THREADS>(s.cell);
-    // the last cell that starts at or below the rank
-    for (uint32_t i = tid; i < kCells; i += THREADS) {
-      const uint32_t first = s.cell[i], end = (i + 1 < kCells) ? s.cell[i + 1] : total;
-      auto look = [&](const CutSearch& c, int e) {
-        const uint32_t at = c.x - c.below;
-        if (first <= at && at < end) {
-          s_cell[e] = i;
-          s_below[e] = first;
-          s_count[e] = end - first;
-        }
-      };
-      if (for_a) look(a, 0);
-      if (for_b) look(b, 1);
-    }
-    __syncthreads();
-    auto narrow = [&](CutSearch& c, int e) {
-      c.lo = lo + ((u64)s_cell[e] << sh);
-      c.hi = c.lo + (1ull << sh) < hi ? c.lo + (1ull << sh) : hi;
-      c.below += s_below[e];
-      if (s_count[e] <= kCutRest || sh == 0) c.open = false;
-    };
-    if (for_a) narrow(a, 0);
-    if (for_b) narrow(b, 1);
-    __syncthreads();
-  }
-}
-
-// Ranks a .. b (about) of a bucket that a block cannot hold, m values in [lo, hi), are collected in their place: items that begin at
-// out + below and whose values lie in [from, to).  src and out differ.
-struct RankPart {
-  u64 from, to;
-  uint32_t below, n;
-};
-template <int THREADS>
-__device__ __noinline__ RankPart collect_part(RankShared& s, const u64* __restrict__ src, uint32_t m, u64 lo, u64 hi, uint32_t a, uint32_t b,
-                                              u64* __restrict__ out) {
-  __shared__ uint32_t s_n;
-  const int tid = threadIdx.x;
-  CutSearch at_a{lo, hi, a, 0, a != 0}, at_b{lo, hi, b, 0, b < m};
-  cut_near<THREADS>(s, src, m, at_a, at_b);
-  const Cut from{at_a.lo, at_a.below}, to = b >= m ? Cut{hi, m} : Cut{at_b.lo, at_b.below};
-  if (tid == 0) s_n = 0;
-  __syncthreads();
-  for_items<THREADS>(src, m, [&](uint32_t, u64 item) {
-    const u64 v = to_value(item);
-    if (v >= from.value && v < to.value) {
-      const uint32_t p = atomicAdd(&s_n, 1u);
-      if (p < kRankItems) out[from.below + p] = item;
-    }
-  });
-  __syncthreads();
-  const uint32_t got = s_n < kRankItems ? s_n : kRankItems;  // at most a window and kCutRest
-  __syncthreads();
-  return RankPart{from.value, to.value, from.below, got};
+  rank_by_block<THREADS>(s.items, n, out);
 }
 
 // Ranks m <= kRankItems items whose inv lies in [base, base + span]: spread over kCells equal ranges of inv, about one item per
@@ -573,12 +480,11 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
 }
 
 // A tile: the buckets (sub-buckets after a partition) of a client that start in [tile window, (tile + 1) window), at most the
-// window plus one bucket; of a bucket that a block cannot hold the ranks that lie in the window, whether it starts there or before.
+// window plus one bucket.  The last may be one that a block cannot hold: it is on the list of large buckets and ranked from there.
 // What a block needs to know of one is found by two warps and kept in shared memory.
 struct RankTile {
   uint32_t ticket;
   uint32_t bucket[2], start[2];  // first bucket at or behind the window's start and end; where those start
-  uint32_t before;               // where the bucket before the first starts
   uint32_t sh, keytop;
   const u64* from;               // the client's candidates by buckets, and in order
   u64* into;
@@ -588,9 +494,14 @@ struct RankArgs {
   const ClientRank* rank;
   const uint32_t *sub_start, *bin_start;
   u64 *buf_a, *buf_b;
-  ulonglong2* list[2];  // left over: cells for a warp; cells for a block and tiles with a bucket that a block cannot hold
-  size_t capacity;
-  uint32_t n, tickets, window;
+  ulonglong2* list[2];  // left over: cells for a warp; cells for a block and tiles of more than a block holds
+  BigBucket* big;
+  u64* piece;           // bucket of the round << 32 | piece of it
+  u64* splitter;
+  uint32_t *part_count, *part_start, *base;
+  BigPart* part;
+  size_t capacity, big_room, piece_room;  // the latter two per round
+  uint32_t n, tickets, window, limit;
 };
 __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout& L, const uint32_t* bin_start, const EncHeader* hdr, uint32_t n) {
   RankArgs a;
@@ -599,14 +510,22 @@ __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout
   a.bin_start = bin_start;
   a.buf_a = reinterpret_cast<u64*>(ws + L.off_buf_a);
   a.buf_b = reinterpret_cast<u64*>(ws + L.off_buf_b);
-  // Room: 512 entries for every 5120 candidates; at most one for every 49 of them, or one for every 257 and one per tile
-  static_assert(kSortPasses * kDigits * 8 / 2 / 16 > kSortTile / kCompareAll + 1 + kSortTile / 1024 + 1, "the lists fit");
-  a.list[0] = reinterpret_cast<ulonglong2*>(ws + L.off_sort_state);
-  a.list[1] = a.list[0] + (size_t)n * L.sort_tiles_max * (kSortPasses * kDigits * 8 / 2 / 16);
+  a.list[0] = reinterpret_cast<ulonglong2*>(ws + L.off_list[0]);
+  a.list[1] = reinterpret_cast<ulonglong2*>(ws + L.off_list[1]);
+  a.big = reinterpret_cast<BigBucket*>(ws + L.off_big);
+  a.piece = reinterpret_cast<u64*>(ws + L.off_piece);
+  a.splitter = reinterpret_cast<u64*>(ws + L.off_splitter);
+  a.part_count = reinterpret_cast<uint32_t*>(ws + L.off_part_count);
+  a.part_start = reinterpret_cast<uint32_t*>(ws + L.off_part_start);
+  a.base = reinterpret_cast<uint32_t*>(ws + L.off_base);
+  a.part = reinterpret_cast<BigPart*>(ws + L.off_part);
   a.capacity = (size_t)L.capacity;
+  a.big_room = (size_t)n * a.capacity / kRankItems + 1;
+  a.piece_room = (size_t)n * a.capacity / kBigPiece + a.big_room;
   a.n = n;
   a.tickets = hdr->rank_tiles * n;
   a.window = hdr->window;
+  a.limit = hdr->limit;
   return a;
 }
 __device__ __forceinline__ uint32_t bucket_start(const RankArgs& a, uint32_t c, const ClientRank& r, uint32_t i) {
@@ -635,7 +554,6 @@ __device__ __forceinline__ void find_tile(RankTile& T, const RankArgs& a) {
     T.bucket[warp] = lo;
     T.start[warp] = lo < n_buckets ? bucket_start(a, c, r, lo) : r.n;
     if (warp == 0) {
-      T.before = lo > 0 ? bucket_start(a, c, r, lo - 1) : 0u;
       T.sh = 19 + r.group - (r.split ? r.sub_bits : 0u);
       T.keytop = r.keytop;
       T.from = (r.split ? a.buf_b : a.buf_a) + (size_t)c * a.capacity;
@@ -644,81 +562,374 @@ __device__ __forceinline__ void find_tile(RankTile& T, const RankArgs& a) {
   }
 }
 
-// A tile with a bucket that a block cannot hold
+// ---- buckets that a block cannot hold ---------------------------------------------------------
+// Equal keys mostly: a layer's clipped values, updates that were rounded to 16 or 8 bits.  In rounds: a bucket's splitters are taken
+// from a sample of its values, its pieces counted over the parts between them, the parts' places summed up by the block that
+// counts the bucket's last piece, and the pieces placed there.  Parts that a block can hold are ranked; larger ones are the next
+// round's buckets (a bucket of more than kBigParts parts).  Values are distinct, so equal keys are split by their indices and no
+// distribution is special.  A step's items are drawn by ticket, and a block waits for the step before when no item of that is left: the
+// blocks it waits for are running.
+// A candidate is read three times and moved twice, whatever the bucket's size, and not moved where its part is never sent.  Steps in
+// this kernel, 2 blocks per SM: bound by the latencies of a piece (12 us for 8192 candidates, most of them the setting up) and of the
+// steps one behind the other (65 us for one bucket of 100,000).  The kernel's time for 4 clients of 50 M coordinates in 16 bits
+// (13.5 M candidates, buckets of 40,000): 335 us; 4 of 50 M on a grid of 24 steps per deviation: 339; one million equal keys in one
+// client of 11.2 M: 110; 10 of 5 M with 250,000 equal keys each: 115.  With every tile ranking its window of a bucket, reading all
+// of it, and digit passes over all candidates for buckets beyond 262,144: 1212, 2925, 308 and 1200.
+
+__device__ __forceinline__ uint32_t big_parts(uint32_t m) { return m / kBigPart + 1 < kBigParts ? m / kBigPart + 1 : kBigParts; }
+// where a bucket's entries in the tables of parts begin: of its own candidates' slots
+__device__ __forceinline__ u64 big_slot(u64 pos) { return (pos + kBigSlot - 1) / kBigSlot; }
+static_assert(kRankItems / kBigSlot - 1 > kRankItems / kBigPart + 1 && kBigPart > 2 * kBigSlot, "a bucket has a slot for every part");
+static_assert(kBigParts <= kRankItems / 8 && 2 * kBigParts <= kCells, "splitters and counts in shared memory, eight samples for a part");
+
+// Waits (bounded) until *done reaches `want`.  False: the wait ran out.  By the whole block.
+__device__ __forceinline__ bool block_waits(const uint32_t* done, uint32_t want, int32_t* status) {
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
+    int polls = 0;
+    s_ok = 1;
+    while (*reinterpret_cast<const volatile uint32_t*>(done) < want) {
+      if (++polls > kMaxPolls) {
+        set_status(status, CVLC_ERR_DEVICE_TIMEOUT);
+        s_ok = 0;
+        break;
+      }
+      __nanosleep(polls > 64 ? 256 : 32);
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  const bool ok = s_ok != 0;
+  __syncthreads();
+  return ok;
+}
+// counts an item of a step as finished, behind all the block's writes; by the whole block
+__device__ __forceinline__ void block_done(uint32_t* done) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(done, 1u);
+  }
+}
+// the next item of a step, the same for all threads of the block
+__device__ __forceinline__ uint32_t block_takes(uint32_t* next) {
+  __shared__ uint32_t s_item;
+  __syncthreads();
+  if (threadIdx.x == 0) s_item = atomicAdd(next, 1u);
+  __syncthreads();
+  return s_item;
+}
+// Candidates of a round's pieces: enough for some pieces a block, and the more the less the setting up of each counts
+// (20 buckets of 1.2 M: the round's counting 120 us with pieces of 8192)
+__device__ __forceinline__ uint32_t big_piece_size(const BigRound& R) {
+  const uint32_t slots = *reinterpret_cast<const volatile uint32_t*>(&R.slots);
+  uint32_t size = kBigPiece;
+  while (size < 8 * kBigPiece && slots / (2 * size / kBigSlot) >= 4 * kNumSM) size *= 2;
+  return size;
+}
+// a bucket as another block has left it
+__device__ __forceinline__ BigBucket big_bucket(const RankArgs& a, int round, uint32_t i) {
+  const volatile BigBucket* b = a.big + (size_t)round * a.big_room + i;
+  return BigBucket{b->pos, b->from, b->to, b->last, b->m, b->parts, 0u, 0u};
+}
+__device__ __forceinline__ const u64* big_source(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_a : a.buf_b) + pos; }
+__device__ __forceinline__ u64* big_target(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_b : a.buf_a) + pos; }
+
+// Ranks m <= kRankItems items in [base, base + span] of inv, with the cells of equal keys among them; by the whole block
 template <int THREADS>
-__device__ __noinline__ void rank_large(RankShared& s, const RankTile& T, const RankArgs& a) {
+__device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop) {
   __shared__ uint32_t s_n, s_big[kRankItems / kCompareAll];
-  const uint32_t tile = T.ticket / a.n, c = T.ticket - tile * a.n;
-  const ClientRank r = a.rank[c];
-  const u64 x0 = (u64)tile * a.window, x1 = x0 + a.window;
-  const uint32_t sh = T.sh;
-  auto rank = [&](const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out) {
-    if (threadIdx.x == 0) s_n = 0;
-    rank_buckets<THREADS>(s, src, m, base, span, out, r.keytop,
-                          [&](u64* where, uint32_t items) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
-    const uint32_t n_big = s_n;
-    for (uint32_t g = 0; g < n_big; ++g) rank_cell<THREADS>(s, out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
+  if (threadIdx.x == 0) s_n = 0;
+  rank_buckets<THREADS>(s, src, m, base, span, out, keytop,
+                        [&](u64* where, uint32_t items) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
+  const uint32_t n_big = s_n;
+  for (uint32_t g = 0; g < n_big; ++g) {
+    u64* at = out + (s_big[g] & 0xFFFFu);
+    rank_cell<THREADS>(s, at, s_big[g] >> 16, at);
+  }
+  __syncthreads();
+}
+
+// Ranks n <= kRankItems items whose keys lie between two, the larger one first; by the whole block
+template <int THREADS>
+__device__ __forceinline__ void rank_keys(RankShared& s, const u64* src, uint32_t n, uint32_t first_key, uint32_t last_key, u64* out) {
+  if (first_key == last_key) rank_cell<THREADS>(s, src, n, out);
+  else rank_with_cells<THREADS>(s, src, n, 0u, first_key - last_key, out, first_key);
+}
+
+// Step 1: the splitters of the round's buckets and their pieces.  A sample of 16 candidates for a part (1024 at least), one from every
+// equal stretch of the bucket at a scattered place of it, since neighbours lie there in the order of the update.  It is ranked where
+// the bucket's parts will lie (8192 of equal keys sorted in shared memory instead: 165 us).
+template <int THREADS>
+__device__ __noinline__ void big_sample(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
+  __shared__ uint32_t s_first;
+  BigRound& R = hdr->big[round];
+  const uint32_t piece_size = big_piece_size(R);
+  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.n);
+  while (true) {
+    const uint32_t i = block_takes(&R.next_sample);
+    if (i >= n) return;
+    const BigBucket b = big_bucket(a, round, i);
+    const u64* src = big_source(a, round, b.pos);
+    u64* sample = big_target(a, round, b.pos);
+    uint32_t samples = 1024;
+    while (samples < kRankItems && samples < 16 * b.parts) samples <<= 1;
+    for (uint32_t t = threadIdx.x; t < samples; t += THREADS) {
+      const uint32_t at = (uint32_t)((u64)t * b.m / samples), width = (uint32_t)((u64)(t + 1) * b.m / samples) - at;
+      sample[t] = src[at + (uint32_t)(((u64)(t * 2654435761u) * width) >> 32)];
+    }
     __syncthreads();
-  };
-  auto part_of = [&](uint32_t bucket, uint32_t first, uint32_t end) {  // the window's part of a large bucket
-    const u64 lo = ((u64)~r.keytop + ((u64)bucket << sh)) << 32, end_high = (u64)~r.keytop + ((u64)(bucket + 1) << sh);
-    const u64 hi = end_high >> 32 ? ~0ull : end_high << 32;  // the last bucket may reach below key 0
-    const uint32_t from = x0 > first ? (uint32_t)(x0 - first) : 0u;
-    const uint32_t to = x1 < end ? (uint32_t)(x1 - first) : end - first;
-    const RankPart p = collect_part<THREADS>(s, T.from + first, end - first, lo, hi, from, to, T.into + first);
-    if (p.n == 0) return;
-    const uint32_t base = (uint32_t)(p.from >> 32) - ~r.keytop, last = (uint32_t)((p.to - 1) >> 32) - ~r.keytop;
-    u64* at = T.into + first + p.below;
-    rank(at, p.n, base, last - base, at);
-  };
+    rank_keys<THREADS>(s, sample, samples, ~(uint32_t)(b.from >> 32), ~(uint32_t)((b.to - 1) >> 32), sample);
+    const u64 slot = big_slot(b.pos);
+    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
+      if (p) a.splitter[slot + p - 1] = to_value(sample[(u64)p * samples / b.parts]);
+      a.part_count[slot + p] = 0;
+    }
+    const uint32_t pieces = (b.m + piece_size - 1) / piece_size;
+    if (threadIdx.x == 0) s_first = atomicAdd(&R.pieces, pieces);
+    __syncthreads();
+    for (uint32_t p = threadIdx.x; p < pieces; p += THREADS) a.piece[(size_t)round * a.piece_room + s_first + p] = (u64)i << 32 | p;
+    block_done(&R.done_sample);
+  }
+}
+
+// What a block needs to find a value's part, the number of splitters not above it: the bucket's splitters in s.items, and, where the
+// values between the first and the last of them are cut into equal cells, how many lie in the cells before each, in s.cell behind
+// the parts' counts.  Equal keys differ by their indices, which are spread about evenly: one cell, one splitter or two.  (A search
+// among all splitters, ten steps, took 1.6 times as long.)
+constexpr uint32_t kBigCells = 2048;
+struct BigSearch {
+  u64 first, last;    // splitters (of a bucket with at least two parts)
+  int shift;          // bits of a cell
+  uint32_t steps;     // of the search among a cell's splitters
+};
+static_assert(2 * kBigParts + kBigCells <= kCells, "the cells' place");
+// ... brought into shared memory; the parts' counts are cleared
+template <int THREADS>
+__device__ __forceinline__ BigSearch big_prepare(RankShared& s, const RankArgs& a, const BigBucket& b) {
+  __shared__ uint32_t s_most;
+  const u64* splitter = a.splitter + big_slot(b.pos);
+  const uint32_t n = b.parts - 1;
+  uint32_t* cells = s.cell + 2 * kBigParts;
+  for (uint32_t p = threadIdx.x; p < n; p += THREADS) s.items[p] = __ldcg(splitter + p);
+  for (uint32_t p = threadIdx.x; p < kBigParts; p += THREADS) s.cell[p] = 0;
+  for (uint32_t p = threadIdx.x; p < kBigCells; p += THREADS) cells[p] = 0;
+  if (threadIdx.x == 0) s_most = 0;
+  __syncthreads();
+  BigSearch h;
+  h.first = s.items[0];
+  h.last = s.items[n - 1];
+  const u64 span = h.last - h.first;
+  h.shift = span < kBigCells ? 0 : 64 - __clzll((long long)span) - 11;  // span >> shift below kBigCells
+  static_assert(kBigCells == 1u << 11, "bits of a cell's number");
+  for (uint32_t p = threadIdx.x; p < n; p += THREADS) atomicMax(&s_most, atomicAdd(cells + (uint32_t)((s.items[p] - h.first) >> h.shift), 1u) + 1);
+  __syncthreads();
+  h.steps = 32 - __clz(s_most);
+  scan_cells<THREADS, kBigCells>(cells);
+  return h;
+}
+// f(part, value) for the values up to `last` of the piece of bucket b that begins at `first`
+template <int THREADS, class F>
+__device__ __forceinline__ void big_piece(const RankShared& s, const BigSearch& h, const BigBucket& b, const u64* src, uint32_t first, uint32_t size, u64 last,
+                                          F&& f) {
+  const uint32_t m = b.m - first < size ? b.m - first : size, n = b.parts - 1;
+  const uint32_t* cells = s.cell + 2 * kBigParts;
+  for (uint32_t i0 = threadIdx.x; i0 < m; i0 += 8 * THREADS) {  // eight at a time: their loads, then their searches side by side
+    u64 v[8];
+    uint32_t p[8], e[8];
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v[u] = i0 + u * THREADS < m ? to_value(src[first + i0 + u * THREADS]) : ~0ull;
+      any |= v[u] <= last;
+    }
+    if (!__any_sync(__activemask(), any)) continue;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const u64 in = v[u] < h.first ? h.first : (v[u] > h.last ? h.last : v[u]);
+      const uint32_t c = (uint32_t)((in - h.first) >> h.shift);
+      p[u] = cells[c];
+      e[u] = c + 1 < kBigCells ? cells[c + 1] : n;
+    }
+    for (uint32_t step = 0; step < h.steps; ++step) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (p[u] < e[u]) {
+          const uint32_t mid = (p[u] + e[u]) >> 1;
+          if (s.items[mid] <= v[u]) p[u] = mid + 1;
+          else e[u] = mid;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * THREADS < m && v[u] <= last) f(p[u], v[u]);
+  }
+}
+
+// Steps 2 and 3: the round's pieces counted; behind a bucket's last piece where its parts begin, and the parts to their lists
+template <int THREADS>
+__device__ __noinline__ void big_count(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
+  __shared__ uint32_t s_last;
+  BigRound& R = hdr->big[round];
+  const uint32_t piece_size = big_piece_size(R);
+  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.pieces);
+  while (true) {
+    const uint32_t t = block_takes(&R.next_count);
+    if (t >= n) return;
+    const u64 piece = __ldcg(a.piece + (size_t)round * a.piece_room + t);
+    const uint32_t i = (uint32_t)(piece >> 32);
+    const BigBucket b = big_bucket(a, round, i);
+    const u64 slot = big_slot(b.pos);
+    const BigSearch h = big_prepare<THREADS>(s, a, b);
+    big_piece<THREADS>(s, h, b, big_source(a, round, b.pos), (uint32_t)piece * piece_size, piece_size, ~0ull, [&](uint32_t p, u64) { atomicAdd(&s.cell[p], 1u); });
+    __syncthreads();
+    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS)
+      if (s.cell[p]) a.base[(size_t)t * kBigParts + p] = atomicAdd(a.part_count + slot + p, s.cell[p]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&a.big[(size_t)round * a.big_room + i].counted, 1u) + 1 == (b.m + piece_size - 1) / piece_size;
+    __syncthreads();
+    if (!s_last) continue;
+    __threadfence();
+    for (uint32_t p = threadIdx.x; p < 2 * kBigParts; p += THREADS) s.cell[p] = p < b.parts ? __ldcg(a.part_count + slot + p) : 0u;
+    __syncthreads();
+    scan_cells<THREADS, 2 * kBigParts>(s.cell);
+    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
+      const uint32_t start = s.cell[p], m = (p + 1 < b.parts ? s.cell[p + 1] : b.m) - start;
+      const bool sent = (b.pos + start) % a.capacity < a.limit;
+      a.part_start[slot + p] = start;
+      if (!sent && p && (b.pos + s.cell[p - 1]) % a.capacity < a.limit) a.big[(size_t)round * a.big_room + i].last = s.items[p - 1] - 1;
+      if (m == 0 || !sent) continue;
+      const u64 from = p ? s.items[p - 1] : b.from, to = p + 1 < b.parts ? s.items[p] : b.to;
+      if (m > kRankItems && round + 1 < kBigRounds) {
+        atomicAdd(&hdr->big[round + 1].slots, m / kBigSlot);
+        a.big[(size_t)(round + 1) * a.big_room + atomicAdd(&hdr->big[round + 1].n, 1u)] = BigBucket{b.pos + start, from, to, ~0ull, m, big_parts(m), 0u, 0u};
+      } else {
+        a.part[atomicAdd(&hdr->part_n, 1u)] = BigPart{b.pos + start, m, round & 1 ? 1u : 0u, ~(uint32_t)(from >> 32), ~(uint32_t)((to - 1) >> 32)};
+      }
+    }
+    block_done(&R.done_bounds);
+  }
+}
+
+// Step 4: the round's pieces placed, but for what is never sent
+template <int THREADS>
+__device__ __noinline__ void big_place(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
+  BigRound& R = hdr->big[round];
+  const uint32_t piece_size = big_piece_size(R);
+  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.pieces);
+  while (true) {
+    const uint32_t t = block_takes(&R.next_place);
+    if (t >= n) return;
+    const u64 piece = __ldcg(a.piece + (size_t)round * a.piece_room + t);
+    const BigBucket b = big_bucket(a, round, (uint32_t)(piece >> 32));
+    const u64 slot = big_slot(b.pos);
+    const u64* src = big_source(a, round, b.pos);
+    u64* dst = big_target(a, round, b.pos);
+    const BigSearch h = big_prepare<THREADS>(s, a, b);
+    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS)  // (of a part that the piece has nothing of the base is not read)
+      s.cell[p] = __ldcg(a.part_start + slot + p) + __ldcg(a.base + (size_t)t * kBigParts + p);
+    __syncthreads();
+    big_piece<THREADS>(s, h, b, src, (uint32_t)piece * piece_size, piece_size, b.last, [&](uint32_t p, u64 v) {
+      const uint32_t o = atomicAdd(&s.cell[p], 1u);
+      if (o < b.m) dst[o] = to_item(v);
+    });
+    block_done(&R.done_place);
+  }
+}
+
+// Step 5: the parts ranked, into the first buffer
+template <int THREADS>
+__device__ __noinline__ void big_rank(RankShared& s, EncHeader* hdr, const RankArgs& a) {
+  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&hdr->part_n);
+  while (true) {
+    const uint32_t i = block_takes(&hdr->part_next);
+    if (i >= n) return;
+    const volatile BigPart* v = a.part + i;
+    const BigPart b{v->pos, v->n, v->in_b, v->first_key, v->last_key};
+    const u64* src = (b.in_b ? a.buf_b : a.buf_a) + b.pos;
+    u64* out = a.buf_a + b.pos;
+    if (b.n > kRankItems) {  // the samples of every round have missed: sorted where it lies
+      for (uint32_t p = threadIdx.x; p < b.n; p += THREADS) out[p] = to_value(src[p]);
+      __syncthreads();
+      bitonic_sort(out, b.n, threadIdx.x, THREADS, [] { __syncthreads(); });
+      for (uint32_t p = threadIdx.x; p < b.n; p += THREADS) out[p] = to_item(out[p]);
+      __syncthreads();
+    } else {
+      rank_keys<THREADS>(s, src, b.n, b.first_key, b.last_key, out);
+    }
+  }
+}
+
+// the large buckets, from step 2 of the first round on; by the whole block
+template <int THREADS>
+__device__ __noinline__ void rank_big(RankShared& s, EncHeader* hdr, const RankArgs& a) {
+  for (int round = 0; round < kBigRounds; ++round) {
+    BigRound& R = hdr->big[round];
+    const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.n);
+    if (n == 0) break;
+    if (round) big_sample<THREADS>(s, hdr, a, round);
+    if (!block_waits(&R.done_sample, n, &hdr->status)) return;
+    big_count<THREADS>(s, hdr, a, round);
+    if (!block_waits(&R.done_bounds, n, &hdr->status)) return;
+    big_place<THREADS>(s, hdr, a, round);
+    if (!block_waits(&R.done_place, *reinterpret_cast<const volatile uint32_t*>(&R.pieces), &hdr->status)) return;
+  }
+  big_rank<THREADS>(s, hdr, a);
+}
+
+// A tile of more than a block holds: its last bucket is a step of its own, or a large one, which is ranked from its list
+template <int THREADS>
+__device__ __noinline__ void rank_full_tile(RankShared& s, const RankTile& T, const RankArgs& a) {
+  const uint32_t c = T.ticket % a.n;
+  const ClientRank r = a.rank[c];
   uint32_t b_lo = T.bucket[0], at = T.start[0];
   const uint32_t b_end = T.bucket[1], at_end = T.start[1];
-  if (x0 < r.n && r.split && b_lo > 0 && at > x0 && at - T.before > kRankItems) part_of(b_lo - 1, T.before, at);
-  // what is too large for one step ends with a large bucket: that bucket is a step of its own
   while (at < at_end) {
     uint32_t b_hi = b_end, to = at_end;
     if (at_end - at > kRankItems && b_hi - b_lo > 1) {
       --b_hi;
       to = bucket_start(a, c, r, b_hi);
     }
-    if (to - at > kRankItems) {
-      if (r.split) part_of(b_lo, at, to);
-    } else if (to > at) {
-      rank(T.from + at, to - at, b_lo << sh, (uint32_t)(((u64)b_hi << sh) - ((u64)b_lo << sh) - 1), T.into + at);
-    }
+    if (to > at && to - at <= kRankItems)
+      rank_with_cells<THREADS>(s, T.from + at, to - at, b_lo << T.sh, (uint32_t)(((u64)b_hi << T.sh) - ((u64)b_lo << T.sh) - 1), T.into + at, r.keytop);
     b_lo = b_hi;
     at = to;
   }
 }
 
 // What the ranking has left over: cells of many equal or nearly equal keys (a layer's clipped outliers, values on a grid), whose
-// items lie in any order in their place, and tiles with a bucket that a block cannot hold.  The blocks take an entry of the
-// second list at a time, then their warps one of the first.  Not among the tiles: there the calls cost registers and a block's
-// other warps waited.  By spreading the indices instead of sorting them: 50 clients of 23.5 M, every seventh layer on a grid
-// (3500 cells for a block, 1200 items each): ranking 784 us with sorting among the tiles, 500 with spreading, 303 + 143 here.
+// items lie in any order in their place, tiles of more than a block holds, and buckets of more than that.  The blocks take an entry
+// of the second list at a time, then their warps one of the first; the large buckets' splitters are looked for before that, so that
+// few blocks wait for them.  Not among the tiles: there the calls cost registers and a block's other warps waited.  By spreading the
+// indices instead of sorting them: 50 clients of 23.5 M, every seventh layer on a grid (3500 cells for a block, 1200 items each):
+// ranking 784 us with sorting among the tiles, 500 with spreading, 303 + 143 here with blocks of 256 threads (20 clients: 87 us,
+// with 512 threads 71).
 template <int THREADS>
-__device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const RankArgs a) {
-  __shared__ RankArgs s_args;
+__device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const RankArgs& a) {
   __shared__ RankTile s_tile;
   __shared__ uint32_t s_entry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_args = a;
+  __syncthreads();  // the arguments are there
+  const bool big = hdr->big[0].n != 0;  // written by the selection alone
+  if (big) big_sample<THREADS>(s, hdr, a, 0);
   while (true) {
     __syncthreads();
     if (tid == 0) s_entry = atomicAdd(&hdr->list_next[1], 1u);
     __syncthreads();
     if (s_entry >= hdr->list_n[1]) break;
-    const ulonglong2 e = s_args.list[1][s_entry];
+    const ulonglong2 e = a.list[1][s_entry];
     const uint32_t m = (uint32_t)e.y;
     if (m != 0) {
-      u64* at = s_args.buf_a + e.x;
-      rank_cell<THREADS>(s, at, m);
+      u64* at = a.buf_a + e.x;
+      rank_cell<THREADS>(s, at, m, at);
     } else {
       if (tid == 0) s_tile.ticket = (uint32_t)e.x;
       __syncthreads();
-      if (tid < 64) find_tile(s_tile, s_args);
+      if (tid < 64) find_tile(s_tile, a);
       __syncthreads();
-      rank_large<THREADS>(s, s_tile, s_args);
+      rank_full_tile<THREADS>(s, s_tile, a);
     }
   }
   __syncthreads();
@@ -728,10 +939,10 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
     uint32_t g = 0;
     if (lane == 0) g = atomicAdd(&hdr->list_next[0], 1u);
     g = __shfl_sync(kFull, g, 0);
-    if (g >= hdr->list_n[0]) return;
-    const ulonglong2 e = s_args.list[0][g];
+    if (g >= hdr->list_n[0]) break;
+    const ulonglong2 e = a.list[0][g];
     const uint32_t m = (uint32_t)e.y;
-    u64* at = s_args.buf_a + e.x;
+    u64* at = a.buf_a + e.x;
     for (uint32_t i = lane; i < m; i += 32) mine[i] = to_value(at[i]);
     __syncwarp();
     if (!rank_equal_by_warp<THREADS>(s.cell + warp * kWarpCells, mine, m, at)) {
@@ -740,6 +951,9 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
       __syncwarp();
     }
   }
+  if (!big) return;
+  __syncthreads();
+  rank_big<THREADS>(s, hdr, a);
 }
 
 }  // namespace cvlc

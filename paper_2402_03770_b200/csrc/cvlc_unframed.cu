@@ -118,7 +118,8 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     const uint32_t tot_blocks = __shfl_sync(kFull, cum, 31);
     const unsigned long long tot_records = __shfl_sync(kFull, zc, 31);
     const bool qsgd_one_bit = QSGD && __shfl_sync(kFull, ny, 31) != 0;
-    if (tot_blocks != R || tot_records != plan->k || tot_records == 0 || tot_records > plan->n_candidates || qsgd_one_bit) {
+    if (tot_blocks != R || tot_records != plan->k || tot_records == 0 || tot_records > plan->n_candidates ||
+        tot_records > (unsigned long long)shape.R * shape.cap[1] || qsgd_one_bit) {
       if (blockIdx.x == 0 && threadIdx.x == 0) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
       return;
     }

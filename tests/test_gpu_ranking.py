@@ -1,6 +1,5 @@
 """GPU parity of the ranking on value distributions at the edges of its buckets: buckets that need the partition, ties of all
-sizes up to and beyond what a block holds, buckets that send the batch to the digit passes, zeros among the candidates, mixed
-batches; plan and stream against the oracle, with the plan's workspace (partition) and without it (digit passes)."""
+sizes up to and beyond what a block holds, zeros among the candidates, mixed batches; plan and stream against the oracle, with the plan's workspace (partition) and without it (digit passes)."""
 import numpy as np
 import pytest
 
@@ -99,7 +98,7 @@ def test_equal_keys_among_others(n, crowded):
     assert (outs[0].cpu().numpy() == stream).all()
 
 
-@pytest.mark.parametrize("n", [262_000, 300_000])       # the largest bucket that is ranked window by window, and one for the digit passes
+@pytest.mark.parametrize("n", [262_000, 300_000])
 def test_very_large_buckets(n):
     import torch
     from paper_2402_03770_b200 import binding as B
@@ -116,9 +115,9 @@ def test_very_large_buckets(n):
     assert (outs[0].cpu().numpy() == stream).all()
 
 
-def test_bucket_for_the_digit_passes_found_while_blocks_still_start():
-    """The first clients' selections find a bucket that sends the batch to the digit passes, while blocks behind the length tuning's
-    (30 of them, one on an SM each) have yet to start and others are under way."""
+def test_large_bucket_found_while_blocks_still_start():
+    """The first clients' selections find a very large bucket, while blocks behind the length tuning's (30 of them, one on an SM
+    each) have yet to start and others are under way."""
     import torch
     from paper_2402_03770_b200 import binding as B
     dev = torch.device("cuda:0")
@@ -142,3 +141,89 @@ def test_bucket_for_the_digit_passes_found_while_blocks_still_start():
                 assert (outs[c].cpu().numpy() == stream).all(), c
             first = [o.clone() for o in outs]
         assert all(torch.equal(a, b) for a, b in zip(first, outs))
+
+
+def _check(xs, pds, **kw):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    refs = [oracle_plan_encode(x, pd) for x, pd in zip(xs, pds)]
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev, **kw)
+    outs = enc.run([torch.from_numpy(x).to(dev) for x in xs], use_plan_ws=True)
+    assert enc.status() == 0
+    for c, (fields, stream) in enumerate(refs):
+        assert_plan_equal(enc.read_plan(c), fields)
+        assert (outs[c].cpu().numpy() == stream).all(), c
+
+
+# Buckets beyond a block (8192): one piece and the next, a few parts, several thousand items per part; equal keys spread over the
+# update, in one stretch, in two far apart, and several keys of a bucket.
+@pytest.mark.parametrize("n", [8192, 8193, 16_385, 24_577, 99_999, 450_000])
+@pytest.mark.parametrize("where", ["spread", "stretch", "two", "keys"])
+def test_buckets_beyond_a_block(n, where):
+    d = 2_400_011
+    rng = np.random.default_rng(n)
+    x = rng.laplace(0, 1e-3, d).astype(np.float32)
+    tie = np.quantile(np.abs(x), 0.8).astype(np.float32)
+    if where == "stretch":
+        at = d // 3 + np.arange(n)
+    elif where == "two":
+        at = np.concatenate([np.arange(n // 2), d - 1 - np.arange(n - n // 2)])
+    else:
+        at = rng.choice(d, n, replace=False)
+    key = np.full(n, tie).view(np.int32) + (rng.integers(0, 5, n).astype(np.int32) if where == "keys" else np.int32(0))
+    x[at] = key.view(np.float32) * rng.choice(np.float32([-1, 1]), n)
+    other = rng.laplace(0, 1e-3, d).astype(np.float32)
+    _check([x, other], [params_dict(d, 4 * d, seed=8 + c, client_id=c) for c in range(2)])
+
+
+@pytest.mark.parametrize("kind", ["bf16", "steps", "signs"])
+def test_updates_of_few_values(kind):
+    """rounded to 16 bits, on a grid of steps, of one magnitude: every bucket is beyond a block"""
+    d = 3_000_017
+    rng = np.random.default_rng(len(kind))
+    x = rng.standard_normal(d).astype(np.float32)
+    if kind == "bf16":
+        x = (x.view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+    elif kind == "steps":
+        x = np.round(x * 8.0).astype(np.float32) / np.float32(8.0)
+    else:
+        x = np.sign(x) * np.float32(0.01)
+    _check([x], [params_dict(d, 5 * d, seed=2, client_id=1)])
+
+
+def test_bucket_of_two_rounds():
+    """more than 1024 parts that a block can hold: 9.5 M values of one magnitude"""
+    d = 9_500_003
+    rng = np.random.default_rng(95)
+    x = rng.choice(np.float32([-0.25, 0.25]), d)
+    _check([x], [params_dict(d, d // 2, seed=2, client_id=1)])
+
+
+# More coordinates are sent than are not zero: zeros of both signs are ranked behind the rest by their indices, subnormals before
+# them; the update's last row and the rows of a warp's step need not be whole.
+@pytest.mark.parametrize("d", [63, 64, 65, 1000, 40_961, 40_975, 300_003])
+@pytest.mark.parametrize("kind", ["zeros", "few", "subnormal"])
+def test_zeros_among_the_candidates(d, kind):
+    rng = np.random.default_rng(d)
+    xs = []
+    for c in range(3):
+        x = rng.laplace(0, 1e-3, d).astype(np.float32)
+        x[rng.random(d) < (1.0 if kind == "zeros" else 0.99)] = 0.0
+        if kind == "subnormal":
+            at = rng.random(d) < 0.3
+            x[at] = rng.integers(1, 1 << 19, int(at.sum())).astype(np.uint32).view(np.float32)
+        x[rng.random(d) < 0.5] *= np.float32(-1.0)
+        xs.append(x)
+    xs.append(rng.laplace(0, 1e-3, d).astype(np.float32))       # a client of the same batch without zeros
+    bits = 12000 if d > 2000 else 32 * 47
+    _check(xs, [params_dict(d, max(bits, 2 * d), packet_bits=bits, seed=3 + c, client_id=c) for c in range(4)])
+
+
+def test_counts_beyond_whole_numbers_of_fp32():
+    """17.3 M values of one magnitude in one bin: the sub-buckets are counted in whole numbers"""
+    d = 17_300_001
+    rng = np.random.default_rng(173)
+    x = rng.choice(np.float32([-0.25, 0.25]), d)
+    x[::1000] = 0.0
+    _check([x], [params_dict(d, d // 8, seed=2, client_id=1)])
