@@ -144,8 +144,7 @@ struct EncHeader {
   uint32_t list_n[2], list_next[2];  // entries of the ranking's lists (of cells for a warp and for a block) and of them taken
   BigRound big[kBigRounds];
   uint32_t part_n, part_next;  // parts of large buckets to rank, and of them taken
-  uint32_t sort_ticket;     // work items of the digit passes
-  uint32_t sort_done[8];    // finished items of their phases
+  uint32_t sort_ticket[4];  // tile tickets of the digit passes
   uint32_t max_sort_tiles;  // largest per-client tile count of this batch
 };
 static_assert(sizeof(EncHeader) <= 256, "the header's place");

@@ -127,8 +127,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     hdr->status = s_bad;
     hdr->limit = limit;
     hdr->select_ticket = hdr->split_ticket = hdr->rank_ticket = 0;
-    hdr->sort_ticket = 0;
-    for (int p = 0; p < 8; ++p) hdr->sort_done[p] = 0;
+    for (int p = 0; p < kSortPasses; ++p) hdr->sort_ticket[p] = 0;
     hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
     for (int r = 0; r < kBigRounds; ++r) hdr->big[r] = BigRound{};
     hdr->part_n = hdr->part_next = 0;
@@ -747,13 +746,14 @@ __device__ __forceinline__ uint32_t sort_digit(unsigned long long pair, int pass
 // ===================================================================================
 // Sort key = keytop - key, keytop = the largest key of the client's highest non-empty histogram
 // bin, so the key only spans the bins between the threshold and the top: 19 + log2(#bins) bits.
-// Digits of 9, 9, 9, 4 bits, in one kernel of six phases: histograms of all four digits, their scans, and
-// per digit a single pass over tiles (tile-major with the clients interleaved; decoupled look-back per digit
-// value).  All phases draw from one ticket counter, and an item waits until the phase before its own is
-// complete: the items it waits for have lower tickets, so blocks that are running hold them.  A pass whose
-// digit is the same for every candidate of a client (normally the fourth) is skipped for that client; which
-// buffer holds its data after pass q follows from the mask of skipped passes.  Used where the plan's
-// workspace is not at hand.
+// Digits of 9, 9, 9, 4 bits: one kernel counts all four for all clients, a small one scans the counts, then one
+// single-pass kernel per digit (tiles handed out by ticket, tile-major with the clients interleaved;
+// decoupled look-back per digit value).  A pass whose digit is the same for every candidate of a client
+// (normally the fourth) is skipped for that client; which buffer holds its data after pass q follows from
+// the mask of skipped passes.  Used where the plan's workspace is not at hand.
+// 100 clients of 11.2 M coordinates at 2 bits (79 M candidates): 1525 us; 24 of 3 M at 4 bits: 285; 20 of 1.2 M: 112; one of 11.2 M: 95.
+// As phases of one kernel that wait for one another 2185, 400, 165 and 117: the counting had the passes' occupancy, and a pass that
+// no client needs its tickets.
 
 // two adjacent look-back words in one 128-bit access (each 64-bit half is its own atomic access)
 __device__ __forceinline__ void ld_relaxed2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
@@ -949,10 +949,84 @@ __device__ __forceinline__ void sort_tile(SortShared& sh, unsigned long long* __
   }
 }
 
-constexpr uint32_t kSortHistTiles = 8;   // tiles of a histogram item
+// digit counts of all candidates: the clients' arrays are concatenated in units of sort tiles and cut into equal contiguous chunks,
+// one per block; a block that crosses a client boundary merges its counts into that client's and starts afresh
+__global__ void __launch_bounds__(256)
+k_sort_hist(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+  __shared__ uint32_t s_count[kSortPasses * kDigits];
+  pdl_enter();
+  const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
+  if (block_sees_error(&hdr->status)) return;
+  const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + L.off_sort_prefix);
+  for (int i = threadIdx.x; i < kSortPasses * kDigits; i += 256) s_count[i] = 0;
+  __syncthreads();
+  const uint32_t total_tiles = prefix[batch.n];
+  const uint32_t chunk = (total_tiles + gridDim.x - 1) / gridDim.x;
+  uint32_t t = blockIdx.x * chunk;
+  const uint32_t t_end = (t + chunk < total_tiles) ? t + chunk : total_tiles;
+  uint32_t c = 0;
+  while (t < t_end) {
+    while (prefix[c + 1] <= t) ++c;  // client of tile t (clients without tiles are passed over)
+    const uint32_t seg_end = prefix[c + 1] < t_end ? prefix[c + 1] : t_end;
+    const cvlc_plan_t* plan = batch.c[c].plan;
+    const uint32_t keytop = sort_keytop(plan);
+    const int n_count = top_digit_is_zero(plan) ? kSortPasses - 1 : kSortPasses;
+    const unsigned long long* __restrict__ in = reinterpret_cast<const unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
+    const unsigned long long i0 = (unsigned long long)(t - prefix[c]) * kSortTile;
+    unsigned long long i1 = (unsigned long long)(seg_end - prefix[c]) * kSortTile;
+    if (i1 > plan->n_candidates) i1 = plan->n_candidates;
+    for (unsigned long long i = i0 + threadIdx.x; i < i1; i += 256) {
+      const unsigned long long pair = in[i];
+#pragma unroll
+      for (int p = 0; p < kSortPasses; ++p)
+        if (p < n_count) atomicAdd(&s_count[p * kDigits + sort_digit(pair, p, keytop)], 1u);
+    }
+    __syncthreads();
+    unsigned long long* ghist = reinterpret_cast<unsigned long long*>(ws + L.off_ghist) + (size_t)c * kSortPasses * kDigits;
+    for (int i = threadIdx.x; i < kSortPasses * kDigits; i += 256) {
+      const uint32_t v = s_count[i];
+      s_count[i] = 0;
+      if (v) atomicAdd(ghist + i, (unsigned long long)v);
+    }
+    __syncthreads();
+    t = seg_end;
+  }
+}
+
+// per client: exclusive scans of the four digit histograms and the mask of constant digits
+__global__ void __launch_bounds__(kDigits)
+k_sort_scan(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+  __shared__ unsigned long long s_scan[kDigits / 32];
+  pdl_enter();
+  const EncHeader* hdr = reinterpret_cast<const EncHeader*>(ws);
+  if (block_sees_error(&hdr->status)) return;
+  const uint32_t c = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const cvlc_plan_t* plan = batch.c[c].plan;
+  const unsigned long long* ghist = reinterpret_cast<const unsigned long long*>(ws + L.off_ghist) + (size_t)c * kSortPasses * kDigits;
+  unsigned long long* gbase = reinterpret_cast<unsigned long long*>(ws + L.off_gbase) + (size_t)c * kSortPasses * kDigits;
+  uint32_t mask = top_digit_is_zero(plan) ? 1u << (kSortPasses - 1) : 0u;  // not counted: known to be constant
+  for (int p = 0; p < kSortPasses; ++p) {
+    const unsigned long long cnt = ghist[p * kDigits + tid];
+    if (__syncthreads_or(cnt == plan->n_candidates)) mask |= 1u << p;
+    unsigned long long incl = cnt;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned long long o = __shfl_up_sync(kFull, incl, off);
+      if (lane >= off) incl += o;
+    }
+    if (lane == 31) s_scan[warp] = incl;
+    __syncthreads();
+    unsigned long long below = 0;
+    for (int w = 0; w < warp; ++w) below += s_scan[w];
+    gbase[p * kDigits + tid] = below + incl - cnt;
+    __syncthreads();
+  }
+  if (tid == 0) reinterpret_cast<uint32_t*>(ws + L.off_pass_mask)[c] = mask;
+}
 
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks)
-k_sort(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
+k_sort_pass(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, int pass) {
   static_assert(kSortThreads * 2 == kDigits && kSortTile <= 0xFFFF, "two digit values per thread; 16-bit slots");
   extern __shared__ __align__(16) unsigned char s_raw[];
   SortShared& sh = *reinterpret_cast<SortShared*>(s_raw);
@@ -964,167 +1038,77 @@ k_sort(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const uint32_t n = batch.n;
   {
     const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + L.off_sort_prefix);
+    const uint32_t* pass_mask = reinterpret_cast<const uint32_t*>(ws + L.off_pass_mask);
     for (uint32_t i = tid; i <= n; i += kSortThreads) s_prefix[i] = prefix[i];
+    uint32_t moves = 0;  // some client's digit is not constant
     for (uint32_t i = tid; i < n; i += kSortThreads) {
       const cvlc_plan_t* plan = batch.c[i].plan;
       s_ncand[i] = (uint32_t)plan->n_candidates;  // <= capacity < 2^32: checked by k_encode_init
       s_keytop[i] = sort_keytop(plan);
+      s_mask[i] = pass_mask[i];
+      moves |= ~s_mask[i] & (1u << pass);
     }
+    if (!__syncthreads_or(moves)) return;
   }
   for (int i = tid; i < (kSortThreads / 32) * kDigits; i += kSortThreads) (&sh.mm[0][0])[i] = 0u;
-  if (tid == 0) sh.tile = atomicAdd(&hdr->sort_ticket, 1u);
+  if (tid == 0) sh.tile = atomicAdd(&hdr->sort_ticket[pass], 1u);
   __syncthreads();
-  // first items of the phases: 2 histograms, 3 scans, 4 .. 7 digit passes
-  const uint32_t n_pass = hdr->max_sort_tiles * n;
-  uint32_t first_item[9];
-  first_item[0] = first_item[1] = first_item[2] = 0;
-  first_item[3] = (hdr->max_sort_tiles + kSortHistTiles - 1) / kSortHistTiles * n;
-  first_item[4] = first_item[3] + n;
-#pragma unroll
-  for (int p = 5; p < 9; ++p) first_item[p] = first_item[p - 1] + n_pass;
-  unsigned long long* ghist_all = reinterpret_cast<unsigned long long*>(ws + L.off_ghist);
-  unsigned long long* gbase_all = reinterpret_cast<unsigned long long*>(ws + L.off_gbase);
-  uint32_t* pass_mask = reinterpret_cast<uint32_t*>(ws + L.off_pass_mask);
+  const uint32_t tickets = hdr->max_sort_tiles * n;
+  unsigned long long* state_all =
+      reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) + (size_t)pass * n * L.sort_tiles_max * kDigits;
   uint4* s_wc4 = reinterpret_cast<uint4*>(&sh.wc[0][0]);
-  int phase = 2;
 
   while (true) {
     const uint32_t gt = sh.tile;
-    if (gt >= first_item[8]) break;
-    __syncthreads();  // everyone has read the ticket
-    // the next ticket is fetched while this item is worked on
+    if (gt >= tickets) break;
+    s_wc4[2 * tid] = make_uint4(0u, 0u, 0u, 0u);
+    s_wc4[2 * tid + 1] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();  // everyone has read the ticket; the counters are clear
+    // the next ticket is fetched while this tile is worked on
     uint32_t next = 0;
-    if (tid == 0) next = atomicAdd(&hdr->sort_ticket, 1u);
-    int my_phase = 2;
-    uint32_t want = 0, first = 0;  // items of the phase before; first item of this one
-#pragma unroll
-    for (int p = 3; p < 8; ++p) {
-      if (gt >= first_item[p]) {
-        my_phase = p;
-        want = first_item[p] - first_item[p - 1];
-        first = first_item[p];
-      }
-    }
-    if (my_phase != phase) {
-      if (tid == 0) {
-        int polls = 0;
-        while (*reinterpret_cast<volatile uint32_t*>(&hdr->sort_done[my_phase - 1]) < want) {
-          if (++polls > kMaxPolls) {
-            set_status(&hdr->status, CVLC_ERR_DEVICE_TIMEOUT);
-            break;
+    if (tid == 0) next = atomicAdd(&hdr->sort_ticket[pass], 1u);
+    // tile-major tickets with the clients interleaved: the tiles in flight are a few consecutive
+    // tiles of every client, which keeps every look-back short
+    const uint32_t tile = gt / n, c = gt - tile * n;
+    const uint32_t mask = s_mask[c];
+    auto source = [&](uint32_t cc) -> unsigned long long* {  // buffer holding client cc's items before this pass
+      const int flips = __popc(~s_mask[cc] & ((1u << pass) - 1u));
+      return reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_b : L.off_buf_a)) + (size_t)cc * L.capacity;
+    };
+    if (tile < s_prefix[c + 1] - s_prefix[c] && !(mask & (1u << pass))) {  // else: no such tile, or a constant digit
+      const uint32_t n32 = s_ncand[c];
+      const uint32_t keytop = s_keytop[c];
+      const int flips = __popc(~mask & ((1u << pass) - 1u));
+      const unsigned long long* src = source(c);
+      unsigned long long* dst =
+          reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_a : L.off_buf_b)) + (size_t)c * L.capacity;
+      unsigned long long* state = state_all + (size_t)s_prefix[c] * kDigits;
+      const unsigned long long* gbase = reinterpret_cast<const unsigned long long*>(ws + L.off_gbase) + ((size_t)c * kSortPasses + pass) * kDigits;
+      const uint32_t tile_first = tile * (uint32_t)kSortTile;
+      const uint32_t count = (n32 - tile_first < (uint32_t)kSortTile) ? n32 - tile_first : (uint32_t)kSortTile;
+      // the next tile's items are asked into L2 while this one is ranked and written
+      auto prefetch_next = [&](uint32_t nt) {
+        if (nt >= tickets) return;
+        const uint32_t t2 = nt / n, c2 = nt - t2 * n;
+        for (uint32_t l = tid; l < (uint32_t)(kSortTile / 16); l += kSortThreads) {  // 128-byte lines of 16 items
+          const uint32_t line = t2 * (uint32_t)(kSortTile / 16) + l;
+          if (line * 16u < s_ncand[c2]) {
+            const unsigned long long* p = source(c2) + (size_t)line * 16;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
           }
-          __nanosleep(polls > 64 ? 256 : 32);
         }
-        __threadfence();
-      }
-      __syncthreads();
-      if (phase < 4 && my_phase >= 4)
-        for (uint32_t i = tid; i < n; i += kSortThreads) s_mask[i] = __ldcg(pass_mask + i);
-      phase = my_phase;
-      __syncthreads();
-    }
-    if (phase == 2) {
-      // digit counts of up to kSortHistTiles tiles of a client
-      uint32_t* cnt = reinterpret_cast<uint32_t*>(s_items);
-      const uint32_t g = (gt - first) / n, c = (gt - first) - g * n;
-      const uint64_t i0 = (uint64_t)g * kSortHistTiles * kSortTile, i1 = i0 + (uint64_t)kSortHistTiles * kSortTile;
-      const uint32_t hi = (uint64_t)s_ncand[c] < i1 ? s_ncand[c] : (uint32_t)i1;
-      if (i0 < s_ncand[c]) {
-        for (int i = tid; i < kSortPasses * kDigits; i += kSortThreads) cnt[i] = 0;
-        __syncthreads();
-        const uint32_t keytop = s_keytop[c];
-        const int n_count = top_digit_is_zero(batch.c[c].plan) ? kSortPasses - 1 : kSortPasses;
-        const unsigned long long* in = reinterpret_cast<const unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
-        for (uint32_t i = (uint32_t)i0 + tid; i < hi; i += kSortThreads) {
-          const unsigned long long pair = __ldcg(in + i);
-#pragma unroll
-          for (int p = 0; p < kSortPasses; ++p)
-            if (p < n_count) atomicAdd(&cnt[p * kDigits + sort_digit(pair, p, keytop)], 1u);
-        }
-        __syncthreads();
-        unsigned long long* ghist = ghist_all + (size_t)c * kSortPasses * kDigits;
-        for (int i = tid; i < kSortPasses * kDigits; i += kSortThreads)
-          if (cnt[i]) atomicAdd(ghist + i, (unsigned long long)cnt[i]);
-      }
-    } else if (phase == 3) {
-      // one client's exclusive scans of the digit histograms and the mask of its constant digits
-      const uint32_t c = gt - first;
-      const unsigned long long have = s_ncand[c];
-      unsigned long long* s_scan = s_items;
-      uint32_t mask = top_digit_is_zero(batch.c[c].plan) ? 1u << (kSortPasses - 1) : 0u;  // not counted: known to be constant
-      for (int p = 0; p < kSortPasses; ++p) {
-        const size_t at = ((size_t)c * kSortPasses + p) * kDigits + 2 * tid;
-        const unsigned long long a = __ldcg(ghist_all + at), b = __ldcg(ghist_all + at + 1);
-        if (__syncthreads_or(a == have || b == have)) mask |= 1u << p;
-        unsigned long long incl = a + b;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const unsigned long long o = __shfl_up_sync(kFull, incl, off);
-          if (lane >= off) incl += o;
-        }
-        if (lane == 31) s_scan[warp] = incl;
-        __syncthreads();
-        unsigned long long below = incl - a - b;
-        for (int w = 0; w < warp; ++w) below += s_scan[w];
-        gbase_all[at] = below;
-        gbase_all[at + 1] = below + a;
-        __syncthreads();
-      }
-      if (tid == 0) pass_mask[c] = mask;
-    } else {
-      // tile-major tickets with the clients interleaved: the tiles in flight are a few consecutive
-      // tiles of every client, which keeps every look-back short
-      const int pass = phase - 4;
-      const uint32_t t = gt - first;
-      const uint32_t tile = t / n, c = t - tile * n;
-      const uint32_t mask = s_mask[c];
-      auto source = [&](uint32_t cc) -> unsigned long long* {  // buffer holding client cc's items before this pass
-        const int flips = __popc(~s_mask[cc] & ((1u << pass) - 1u));
-        return reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_b : L.off_buf_a)) + (size_t)cc * L.capacity;
       };
-      s_wc4[2 * tid] = make_uint4(0u, 0u, 0u, 0u);
-      s_wc4[2 * tid + 1] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();  // the counters are clear
-      if (tile < s_prefix[c + 1] - s_prefix[c] && !(mask & (1u << pass))) {  // else: no such tile, or a constant digit
-        const uint32_t n32 = s_ncand[c];
-        const uint32_t keytop = s_keytop[c];
-        const int flips = __popc(~mask & ((1u << pass) - 1u));
-        const unsigned long long* src = source(c);
-        unsigned long long* dst =
-            reinterpret_cast<unsigned long long*>(ws + ((flips & 1) ? L.off_buf_a : L.off_buf_b)) + (size_t)c * L.capacity;
-        unsigned long long* state = reinterpret_cast<unsigned long long*>(ws + L.off_sort_state) +
-                                    ((size_t)pass * n * L.sort_tiles_max + s_prefix[c]) * kDigits;
-        const unsigned long long* gbase = gbase_all + ((size_t)c * kSortPasses + pass) * kDigits;
-        const uint32_t tile_first = tile * (uint32_t)kSortTile;
-        const uint32_t count = (n32 - tile_first < (uint32_t)kSortTile) ? n32 - tile_first : (uint32_t)kSortTile;
-        // the next tile's items are asked into L2 while this one is ranked and written
-        auto prefetch_next = [&](uint32_t nt) {
-          if (nt < first || nt - first >= n_pass) return;
-          const uint32_t t2 = (nt - first) / n, c2 = (nt - first) - t2 * n;
-          for (uint32_t l = tid; l < (uint32_t)(kSortTile / 16); l += kSortThreads) {  // 128-byte lines of 16 items
-            const uint32_t line = t2 * (uint32_t)(kSortTile / 16) + l;
-            if (line * 16u < s_ncand[c2]) {
-              const unsigned long long* p = source(c2) + (size_t)line * 16;
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-            }
-          }
-        };
-        if (count == (uint32_t)kSortTile)
-          sort_tile<true>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
-        else
-          sort_tile<false>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
-      }
+      if (count == (uint32_t)kSortTile)
+        sort_tile<true>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
+      else
+        sort_tile<false>(sh, s_items, src, dst, state, gbase, tile, count, n32, keytop, kDigitBits * pass, &hdr->status, next, prefetch_next);
     }
     if (tid == 0) sh.tile = next;
     __syncthreads();
-    if (tid == 0) {  // behind the barrier: the item's writes are done
-      __threadfence();
-      atomicAdd(&hdr->sort_done[phase], 1u);
-    }
   }
 }
 
@@ -1429,7 +1413,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   if (dev >= 0 && dev < 64 && !attr_done[dev]) {
     e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
+    e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -1458,8 +1442,11 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     const unsigned grid = (unsigned)(want < (uint64_t)(4 * kNumSM) ? want : 4 * kNumSM);
     launch_kernel(kKSelectLookback, k_select_lookback, grid, kSelectThreads, 0, st, true, batch, shape.d, w, L);
     const uint64_t tiles = L.sort_tiles_max * n;
-    launch_kernel(kKSort, k_sort, (unsigned)(tiles < kSortMinBlocks * kNumSM ? tiles : kSortMinBlocks * kNumSM), kSortThreads, sort_smem_bytes(n), st, true,
-                  batch, w, L);
+    auto blocks = [&](uint64_t most) -> unsigned { return (unsigned)(tiles < most ? tiles : most); };
+    launch_kernel(kKSort, k_sort_hist, blocks(8 * kNumSM), 256, 0, st, true, batch, w, L);
+    launch_kernel(kKSort, k_sort_scan, n, kDigits, 0, st, true, batch, w, L);
+    for (int pass = 0; pass < kSortPasses; ++pass)
+      launch_kernel(kKSort, k_sort_pass, blocks(kSortMinBlocks * kNumSM), kSortThreads, sort_smem_bytes(n), st, true, batch, w, L, pass);
   }
   if (wait_before_pack) {
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);
