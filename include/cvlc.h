@@ -21,8 +21,11 @@
  *    cvlc_compress_batch to order its two streams; the launch counters and, while
  *    cvlc_profile_select is active, the profiling events; the built-in scratch of
  *    cvlc_decode_aggregate_noalloc and its cached device address.  cvlc_set_device changes
- *    the calling thread's current device.  None of this is synchronised: call the library
- *    from one host thread at a time.
+ *    the calling thread's current device.
+ *  - Host threads: calls may come from several threads at once, each on buffers and workspaces of
+ *    its own; the state above is kept in order for them.  Two exceptions: cvlc_profile_select,
+ *    _reset and _read must not run next to a call of another thread, and two calls of
+ *    cvlc_decode_aggregate_noalloc on one device share its scratch, so they must not overlap on the GPU.
  *  - Host-detectable errors are returned at once.  Errors only the device can see
  *    (non-finite input, malformed stream, a wait that ran out) are written to the
  *    status word at byte 0 of the plan / workspace and read with cvlc_read_status;

@@ -2,7 +2,7 @@
 // stream-ordered kernel launches.  No device allocation, no CPU fallback.  Process-wide state is
 // limited to what include/cvlc.h lists (per-device set-up flags, two events per device for
 // cvlc_compress_batch, launch counters, the profiling events, the scratch of the allocation-free
-// decode); host calls are not thread-safe.
+// decode); calls may come from several host threads.
 #include <math.h>
 #include <string.h>
 

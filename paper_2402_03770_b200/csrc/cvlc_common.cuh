@@ -5,6 +5,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/cvlc.h"
 
 namespace cvlc {
@@ -338,16 +340,38 @@ enum KernelId {
 };
 
 // Called around every kernel launch.  Counts launches; when a kernel has been selected with
-// cvlc_profile_select, records a CUDA event pair on the launching stream around it.
-void launch_begin(int kernel_id, cudaStream_t st);
-void launch_end(int kernel_id, cudaStream_t st);
+// cvlc_profile_select, records a CUDA event pair on the launching stream around it: launch_begin
+// returns the pair's number, or -1.
+int launch_begin(int kernel_id, cudaStream_t st);
+void launch_end(int kernel_id, int pair, cudaStream_t st);
 
 struct LaunchScope {
-  int id;
+  int id, pair;
   cudaStream_t st;
-  LaunchScope(int id_, cudaStream_t st_) : id(id_), st(st_) { launch_begin(id, st); }
-  ~LaunchScope() { launch_end(id, st); }
+  LaunchScope(int id_, cudaStream_t st_) : id(id_), pair(launch_begin(id_, st_)), st(st_) {}
+  ~LaunchScope() { launch_end(id, pair, st); }
 };
+
+// Something to be done once on every device (kernel attributes), asked for by every call.  Several threads may get to it
+// together and then all do it, to the same effect.
+struct OncePerDevice {
+  std::atomic<bool> done[64];
+};
+template <class F>
+inline cudaError_t once_per_device(OncePerDevice& once, F&& f) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < 64;
+  if (known && once.done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = f();
+  if (e == cudaSuccess && known) once.done[dev].store(true, std::memory_order_release);
+  return e;
+}
+template <class K>
+inline cudaError_t allow_shared(K kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 #ifdef __CUDACC__
 // Every kernel of the plan / encode / decode path but the first of a call is launched with programmatic stream serialization: it is

@@ -403,18 +403,18 @@ __global__ void k_noalloc_publish_status(int32_t* status_out) {
 // Device address of the scratch on the current device.  In host code the array's name is only a
 // handle for the runtime, so the address is asked for once per device and cached.
 static cudaError_t noalloc_scratch_address(void** out) {
-  static void* cached[64] = {};
+  static std::atomic<void*> cached[64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!cached[dev]) {
-    void* ptr = nullptr;
+  void* ptr = cached[dev].load(std::memory_order_acquire);
+  if (!ptr) {
     e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
-    cached[dev] = ptr;
+    cached[dev].store(ptr, std::memory_order_release);
   }
-  *out = cached[dev];
+  *out = ptr;
   return cudaSuccess;
 }
 

@@ -1406,17 +1406,12 @@ constexpr uint64_t kTuneRoomRows = 8 << 20;
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual) {
-  static bool attr_done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice once;
+  cudaError_t e = once_per_device(once, [] {
+    const cudaError_t e = allow_shared(k_select, kSelSmem);
+    return e != cudaSuccess ? e : allow_shared(k_sort_pass, sort_smem_bytes(CVLC_MAX_BATCH));
+  });
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem_bytes(CVLC_MAX_BATCH));
-    if (e != cudaSuccess) return e;
-    attr_done[dev] = true;
-  }
   const EncLayout L = enc_layout(shape.d, n, capacity);
   if (enc_lists_end(L) > L.off_buf_a) return cudaErrorInvalidValue;
   unsigned char* w = static_cast<unsigned char*>(ws);

@@ -1260,20 +1260,12 @@ constexpr size_t kFitSmem = 3 * 4096 * 8 + 4096 * 2;  // survival counts, the fi
 constexpr size_t kTuneSmem = (sizeof(PlanSolver) + 255) & ~(size_t)255;
 
 static cudaError_t plan_attributes() {
-  static bool attr_done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSub * CVLC_HIST_BINS * 4);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_plan_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFitSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_plan_tune, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTuneSmem);
-    if (e != cudaSuccess) return e;
-    attr_done[dev] = true;
-  }
-  return cudaSuccess;
+  static OncePerDevice once;
+  return once_per_device(once, [] {
+    cudaError_t e = allow_shared(k_hist, kHistSub * CVLC_HIST_BINS * 4);
+    if (e == cudaSuccess) e = allow_shared(k_plan_fit, kFitSmem);
+    return e != cudaSuccess ? e : allow_shared(k_plan_tune, kTuneSmem);
+  });
 }
 
 // the start of a planning call: the descriptors into the workspace, `bytes` from its start and `more` from `at` on zeroed

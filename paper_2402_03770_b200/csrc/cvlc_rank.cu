@@ -167,17 +167,12 @@ k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
 }
 
 cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
-  static bool attr_done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice once;
+  const cudaError_t e = once_per_device(once, [] {
+    const cudaError_t e = allow_shared(k_rank, sizeof(RankShared));
+    return e != cudaSuccess ? e : allow_shared(k_rank_rest, sizeof(RankShared));
+  });
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankShared));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_rank_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankShared));
-    if (e != cudaSuccess) return e;
-    attr_done[dev] = true;
-  }
   auto blocks = [](uint64_t tiles, uint64_t most) -> unsigned { return (unsigned)(tiles < most ? tiles : most); };
   launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * sms), kRankThreads, kRankSubs * 4, st, true,
                 batch, ws, L);

@@ -392,17 +392,12 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
 
 cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capacity,
                                  size_t stream_capacity, void* enc_ws, void* uf_ws, unsigned long long* sizes_out, cudaStream_t st) {
-  static bool attr_done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice once;
+  const cudaError_t e = once_per_device(once, [] {
+    const cudaError_t e = allow_shared(k_pack_unframed<false>, 200 * 1024);
+    return e != cudaSuccess ? e : allow_shared(k_pack_unframed<true>, 200 * 1024);
+  });
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-    e = cudaFuncSetAttribute(k_pack_unframed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_pack_unframed<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_done[dev] = true;
-  }
   const EncLayout L = enc_layout(shape.d, n, capacity);
   // the encoder has left the descriptors in its workspace
   const Batch batch{reinterpret_cast<const ClientDesc*>(static_cast<unsigned char*>(enc_ws) + L.off_desc), n};
@@ -733,8 +728,8 @@ cudaError_t launch_decode_unframed(const uint8_t* const* streams, const uint64_t
     if (e != cudaSuccess) return e;
   }
   const size_t prefix_bytes = ((size_t)n + 1) * 4;
-  if (prefix_bytes + sizeof(UfDecWarp) * kUfDecWarps > 47 * 1024) {  // hundreds of clients
-    const cudaError_t e = cudaFuncSetAttribute(k_decode_unframed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prefix_bytes);
+  if (prefix_bytes + sizeof(UfDecWarp) * kUfDecWarps > 47 * 1024) {  // hundreds of clients: the most of any call, another thread's too
+    const cudaError_t e = allow_shared(k_decode_unframed, ((size_t)CVLC_MAX_CLIENTS_PER_CALL + 1) * 4);
     if (e != cudaSuccess) return e;
   }
   launch_kernel(kKDecodeUnframed, k_decode_unframed, 4 * kNumSM, kUfDecThreads, prefix_bytes, st, true, streams, n, d, out, w);

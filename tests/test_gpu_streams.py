@@ -143,3 +143,42 @@ def test_capture_into_a_graph(kind):
         calls.load(which)
         graph.replay()
         calls.check(which)
+
+
+def test_calls_from_several_threads():
+    """Every thread on a stream and buffers of its own; no launch is missing from the count."""
+    import threading
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    kinds = ["client", "compress", "separate", "ec", "decode", "unframed", "decode_unframed", "compress"]
+    work = [Calls(kind) for kind in kinds]
+    each = []
+    for calls in work:
+        calls.load(0)
+        before = B.cvlc_launch_count()
+        calls.run()
+        each.append(B.cvlc_launch_count() - before)
+    torch.cuda.synchronize()
+    failed = []
+
+    def repeat(calls):
+        try:
+            torch.cuda.set_device(0)
+            with torch.cuda.stream(torch.cuda.Stream(calls.dev)):
+                for i in range(30):
+                    calls.load((i + 1) % 2)
+                    calls.run()
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:  # noqa: BLE001
+            failed.append((calls.kind, e))
+
+    before = B.cvlc_launch_count()
+    threads = [threading.Thread(target=repeat, args=(calls,)) for calls in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    assert B.cvlc_launch_count() - before == 30 * sum(each)
+    for calls in work:
+        calls.check(0)
