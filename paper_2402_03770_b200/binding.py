@@ -9,7 +9,8 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-from typing import List, Optional, Sequence
+import threading
+from typing import Dict, List, Optional, Sequence, Tuple
 
 import torch
 
@@ -536,9 +537,29 @@ def read_plan(plan: torch.Tensor) -> CvlcPlan:
     return CvlcPlan.from_buffer_copy(raw)
 
 
+_side_streams: Dict[Tuple[int, int], torch.cuda.Stream] = {}
+_side_lock = threading.Lock()
+
+
+def _side_stream(device: torch.device, stream: Optional[torch.cuda.Stream]) -> torch.cuda.Stream:
+    """The stream that runs the length tuning next to the work of `stream` (None: the current one).  One for every calling
+    stream, whose calls are in order anyway, not one for every encoder: torch hands out 32 in turn, and with more encoders the
+    tuning of one would queue behind the work of another.  They come from the pool of high priority, where few programs take
+    streams for other work; torch keeps them, so forgetting them all (after 64) costs nothing."""
+    index = torch.cuda.current_device() if device.index is None else device.index
+    key = (index, _stream_handle(stream))
+    side = _side_streams.get(key)
+    if side is None:
+        with _side_lock:
+            if len(_side_streams) >= 64:
+                _side_streams.clear()
+            side = _side_streams.setdefault(key, torch.cuda.Stream(index, priority=-1))
+    return side
+
+
 class ClientEncoder:
     """Owns the buffers one client's plan + encode needs; when `run` returns, `stream` is ordered after all its work (the
-    length tuning runs on a stream of the encoder's own, next to selection and ranking)."""
+    length tuning runs on a stream beside it, next to selection and ranking)."""
 
     def __init__(self, p: CvlcParams, device: torch.device):
         self.p = p
@@ -547,7 +568,7 @@ class ClientEncoder:
         self.plan_ws = alloc_bytes(cvlc_plan_workspace_bytes(p), device)
         self.enc_ws = alloc_bytes(cvlc_encode_workspace_bytes(p), device)
         self.out = alloc_bytes(cvlc_stream_bytes(p), device)
-        self._side = torch.cuda.Stream(device)
+        _side_stream(device, None)  # torch makes its streams before any capture
 
     def run(self, x: torch.Tensor, p: Optional[CvlcParams] = None, out: Optional[torch.Tensor] = None,
             stream: Optional[torch.cuda.Stream] = None, fixed_y: int = 0, use_plan_ws: bool = True) -> torch.Tensor:
@@ -555,7 +576,7 @@ class ClientEncoder:
         out = self.out if out is None else out
         if use_plan_ws:
             assert x.dtype == torch.float32 and x.numel() == p.d and out.dtype == torch.uint8
-            cvlc_compress_batch((x,), (p,), self.plan, (out,), self.plan_ws, self.enc_ws, 0, fixed_y, stream, self._side)
+            cvlc_compress_batch((x,), (p,), self.plan, (out,), self.plan_ws, self.enc_ws, 0, fixed_y, stream, _side_stream(self.device, stream))
             return out
         if fixed_y:
             cvlc_plan_fixed(x, p, fixed_y, self.plan, self.plan_ws, stream)

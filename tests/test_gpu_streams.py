@@ -182,3 +182,29 @@ def test_calls_from_several_threads():
     assert B.cvlc_launch_count() - before == 30 * sum(each)
     for calls in work:
         calls.check(0)
+
+
+def test_encoders_on_two_streams_do_not_wait_for_each_other():
+    """More encoders than torch has streams of a kind: those used on one stream finish while the other stream is held up."""
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    pd = params_dict(20_001, 12_000 * 4, seed=1)
+    x = np.random.default_rng(3).laplace(0, 1e-3, 20_001).astype(np.float32)
+    ref = O.encode(x, oracle_params(pd), O.plan(x, oracle_params(pd)))
+    dx = torch.from_numpy(x).to(dev)
+    encoders = [B.ClientEncoder(gpu_params(pd), dev) for _ in range(72)]
+    held, free = torch.cuda.Stream(dev), torch.cuda.Stream(dev)
+    for s in (held, free):
+        encoders[0].run(dx, stream=s)
+        s.synchronize()
+    with torch.cuda.stream(held):
+        torch.cuda._sleep(600_000_000)  # about 0.3 s
+        encoders[0].run(dx)
+    for e in encoders[1:]:
+        e.run(dx, stream=free)
+    free.synchronize()
+    assert not held.query()
+    held.synchronize()
+    for e in encoders:
+        assert e.status() == 0 and (e.out.cpu().numpy() == ref).all()
