@@ -89,9 +89,10 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   P.rows = (((d >> 2) + kRowUnits - 1) / kRowUnits + 15) & ~(uint64_t)15;
   if (P.rows == 0) P.rows = 16;
   P.total = P.rows * n;
-  // Three blocks per SM finish a small batch sooner (10 clients of 5 M coordinates: 44 instead of 47 us, 20 of 1.2 M: 26 instead of
-  // 29); a large one streams faster with two (100 of 11.2 M: 709 us instead of 729).
-  const uint64_t most = P.total <= (16u << 20) ? 3 * kNumSM : 2 * kNumSM;
+  // Three blocks per SM finish a small batch sooner (20 clients of 1.2 M coordinates: 26.6 instead of 28.2 us, 10 of 3 M 30.1 and 32.9, 10
+  // of 8 M 65.7 and 68.9); at 100 M coordinates the two are even, and a large one streams faster with two, which also leave the
+  // selection behind them more to find in the L2 (whole calls: 150 M 251 and 247 us, 280 M 421 and 394, 600 M 775 and 739).
+  const uint64_t most = P.total <= (8u << 20) ? 3 * kNumSM : 2 * kNumSM;
   uint64_t grid = (P.total + 255) / 256;
   if (grid > most) grid = most;
   P.grid = (uint32_t)grid;

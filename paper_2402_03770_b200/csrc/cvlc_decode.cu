@@ -315,11 +315,14 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
   // into the L2 right before its decode launch, by the zero fill or, when accumulating, by a prefetch: a
   // reduction that misses the L2 is a DRAM read-modify-write.
   // Reductions into a vector near the L2's size run at half the rate of a smaller one: a vector of one window above 20 Mi coordinates
-  // is better filled in two, if there are many clients' records (50 clients of 23.5 M coordinates: 351 -> 270 us; even at about
-  // 21 M: 30 clients of 22 M 200 -> 195, of 18 M 138 -> 163, of 13 M 97 -> 120).  Where several windows are needed anyway each
-  // of them costs a walk over all records, and smaller ones lose (20 clients of 1e8: 387 -> 488 us).
+  // is better filled in two, if there are many records (50 clients of 23.5 M coordinates at 1 bit: 351 -> 270 us; even at about
+  // 21 M: 30 clients of 22 M 200 -> 195, of 18 M 138 -> 163, of 13 M 97 -> 120).  How many there are only the device knows; by
+  // clients, one window and two, us, at 0.5 / 1 / 4 bits a coordinate: 23.5 M, 4 clients 39 and 40 / 51 and 56 / 133 and 114, 6
+  // clients 46 and 45 / 57 and 58 / 159 and 152, 8 clients 53 and 58 / 71 and 76 / 244 and 194; 25 M, 4 clients 41 and 42 / 53 and 57
+  // / 149 and 120, 6 clients 50 and 52 / 64 and 66 / 210 and 161.  Where several windows are needed anyway each of them costs a walk
+  // over all records, and smaller ones lose (20 clients of 1e8: 387 -> 488 us).
   uint64_t n_win = (d + kDecodeWindow - 1) / kDecodeWindow;
-  if (n_win == 1 && d > kDecodeWindow / 6 * 5 && n >= 8) n_win = 2;
+  if (n_win == 1 && d > kDecodeWindow / 6 * 5 && n >= 6) n_win = 2;
   const uint64_t win = (((d + n_win - 1) / n_win) + 1023) & ~(uint64_t)1023;
   auto fill_grid = [](uint64_t coords, uint64_t threads, uint64_t most) -> unsigned {
     const uint64_t want = (coords / 4 + threads - 1) / threads;

@@ -326,6 +326,7 @@ constexpr uint32_t kSelBuffer = 512;    // candidates in a warp's buffer: all of
 constexpr int kSelVec = 4;              // 128-bit loads per lane and step
 constexpr uint32_t kSelRows = 32;       // rows of a step
 constexpr uint32_t kSelDense = 96;      // a step with this many candidates takes each coordinate in turn, one with fewer only its candidates
+constexpr uint64_t kSelGiven = 2 << 20;  // rows of a batch (33 M coordinates) whose groups are all given out beforehand
 constexpr int kSelStages = 2;           // steps in shared memory: the current one and those on their way
 constexpr uint32_t kSelQueue = 256;     // rows a warp has found (ring)
 struct SelWarp {
@@ -392,14 +393,17 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   for (uint32_t i = lane; i < kRankCoarse; i += 32) sw.cnt[i] = 0;
   if (tid == 0) s_taken = 0;
   // Block b starts with client b n / grid; the first groups of a client go to the warps of the blocks that start with it, the rest
-  // by its counter.  A small batch would wait for that: there the warps have three quarters of the groups without asking (with few
-  // clients, whose blocks are as good as equally many, all).
+  // by its counter.  A small batch would wait for that: there the warps have three quarters of the groups without asking, and all
+  // of them with few clients, whose blocks are as good as equally many, and in the smallest batches, where the last of them are not
+  // worth a wait.  Whole calls with all and with three quarters, us: 4 clients of 3 M coordinates 113 and 121, 8 of 3 M 154 and 160;
+  // 10 of 0.3 / 1.2 / 3 M 65 and 69 / 100 and 105 / 174 and 176, 24 of 0.3 / 1.2 M 86 and 90 / 159 and 160; 12 / 16 of 3 M 205 and 201
+  // / 239 and 228, 40 of 1.2 M 235 and 226.
   const uint32_t home = (uint32_t)(((uint64_t)blockIdx.x * n) / gridDim.x);
   auto first_block = [&](uint32_t c) -> uint32_t { return (uint32_t)(((uint64_t)c * gridDim.x + n - 1) / n); };
   auto warps_of = [&](uint32_t c) -> uint32_t { return (first_block(c + 1) - first_block(c)) * (kSelThreads / 32); };
   auto rounds_of = [&](uint32_t warps) -> uint32_t {
     if (sg.count[0] + sg.count[1] || warps == 0) return 1;
-    const uint32_t most = n <= 8 ? (groups + warps - 1) / warps : groups / 4 * 3 / warps;
+    const uint32_t most = n <= 8 || part.total <= kSelGiven ? (groups + warps - 1) / warps : groups / 4 * 3 / warps;
     return most > 1 ? most : 1;
   };
   auto given = [&](uint32_t c) -> uint32_t { return warps_of(c) * rounds_of(warps_of(c)); };
@@ -1400,9 +1404,12 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
 
 // While the length tuning runs on another stream, one block per client, selection and ranking leave it its SMs: their blocks fill an
 // SM, those behind a tuning block start when that ends (after 25 to 80 us, 67 us into a selection of 120), and the kernel ends with
-// them.  Not for long selections, where blocks that start late still find work, nor for so many clients that too few SMs are left.
-constexpr uint32_t kTuneRoom = 24;
-constexpr uint64_t kTuneRoomRows = 8 << 20;
+// them.  Not for so many clients that too few SMs are left, nor for long selections, where blocks that start late still find work: the
+// SMs given away cost the clients times the length of the selection.  Whole calls with room and without, us: 24 clients of 0.3 M
+// coordinates 90 and 100, 32 of 0.3 / 1.2 / 3 M 98 and 111 / 195 and 203 / 385 and 390, 40 of 0.3 / 1.2 / 3 M 107 and 117 / 239 and 226
+// / 475 and 441; 10 of 13 / 20 / 40 M 319 and 346 / 434 and 467 / 816 and 820, 20 of 6 / 12 M 309 and 315 / 548 and 514.
+constexpr uint32_t kTuneRoom = 32;
+constexpr uint64_t kTuneRoomRows = 192 << 20;  // times clients
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual) {
@@ -1420,7 +1427,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
 
   const Partition part = make_partition(shape.d, n);
-  const unsigned sms = wait_before_pack && n <= kTuneRoom && part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
+  const unsigned sms = wait_before_pack && n <= kTuneRoom && n * part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
   if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st, overlap);
   else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st, overlap);
