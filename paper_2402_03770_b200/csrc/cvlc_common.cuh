@@ -146,6 +146,7 @@ struct EncHeader {
   uint32_t rank_tiles;      // largest per-client tile count of the final ranking
   uint32_t list_n[2], list_next[2];  // entries of the ranking's lists (of cells for a warp and for a block) and of them taken
   BigRound big[kBigRounds];
+  uint32_t own_n, own_next, own_done;  // large buckets that a block splits by itself, of them taken, finished
   uint32_t part_n, part_next;  // parts of large buckets to rank, and of them taken
   uint32_t sort_ticket[4];  // tile tickets of the digit passes
   uint32_t max_sort_tiles;  // largest per-client tile count of this batch
@@ -253,7 +254,7 @@ struct EncLayout {
   size_t off_sort_state;         // uint64[4][n * sort_tiles_max][512]
   // ranked by partition, in the place of the digit passes' states (see RankArgs):
   size_t off_list[2];            // cells left over for a warp and for a block
-  size_t off_big;                // buckets that a block cannot hold, per round
+  size_t off_big;                // buckets that a block cannot hold, per round, and those that one block splits
   size_t off_piece;              // pieces of them, per round
   size_t off_splitter, off_part_count, off_part_start;  // per bucket: the values its parts begin with, what they hold, where they begin
   size_t off_base;               // per piece and part: what earlier pieces have of the part
@@ -266,6 +267,8 @@ struct EncLayout {
 constexpr uint32_t kBigPart = 3072;   // candidates of a part, about
 constexpr uint32_t kBigParts = 1024;  // most parts of a bucket in one round
 constexpr uint32_t kBigPiece = 8192;  // candidates of a piece at least
+constexpr uint32_t kBigOwn = 32768;   // a bucket of up to this many is split by one block,
+constexpr int kBigOwnRow = kBigRounds;  // and stands in a row of its own behind those of the rounds
 constexpr uint32_t kBigSlot = 1024;   // candidates per entry of the tables of parts
 struct BigBucket {
   uint64_t pos;         // where it begins among all clients' candidates
@@ -309,7 +312,7 @@ static inline EncLayout enc_layout(uint64_t d, uint32_t n, uint64_t capacity) {
   L.off_list[0] = L.off_sort_state;
   L.off_list[1] = L.off_list[0] + align256((all / 49 + 1) * 16);
   L.off_big = L.off_list[1] + align256((all / 257 + all / 1024 + n + 1) * 16);
-  L.off_piece = L.off_big + align256(buckets * kBigRounds * sizeof(BigBucket));
+  L.off_piece = L.off_big + align256(buckets * (kBigRounds + 1) * sizeof(BigBucket));
   L.off_splitter = L.off_piece + align256((all / kBigPiece + buckets) * kBigRounds * 8);
   L.off_part_count = L.off_splitter + align256((all / kBigSlot + 1) * 8);
   L.off_part_start = L.off_part_count + align256((all / kBigSlot + 1) * 4);

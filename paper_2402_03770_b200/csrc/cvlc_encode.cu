@@ -130,7 +130,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     for (int p = 0; p < kSortPasses; ++p) hdr->sort_ticket[p] = 0;
     hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
     for (int r = 0; r < kBigRounds; ++r) hdr->big[r] = BigRound{};
-    hdr->part_n = hdr->part_next = 0;
+    hdr->own_n = hdr->own_next = hdr->own_done = hdr->part_n = hdr->part_next = 0;
     hdr->split_tiles = (s_most_split + kRankSplitTile - 1) / kRankSplitTile;
     // tiles small enough that the batch gives every SM several
     const uint64_t want = ((uint64_t)run * kSortTile + 4 * kNumSM - 1) / (4 * kNumSM);
@@ -364,9 +364,11 @@ __device__ __noinline__ void add_counts4_wide(float* p, uint4 v) {
 // a sub-bucket that a block of the ranking cannot hold
 __device__ __noinline__ void list_bucket(EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, const ClientRank& r, uint32_t sh,
                                          uint32_t bucket, uint32_t start, uint32_t m) {
-  atomicAdd(&hdr->big[0].slots, m / kBigSlot);
   const u64 lo = (u64)~r.keytop + ((u64)bucket << sh), end = lo + (1ull << sh);  // the last bucket may reach below key 0
-  reinterpret_cast<BigBucket*>(ws + L.off_big)[atomicAdd(&hdr->big[0].n, 1u)] =
+  const bool own = m <= kBigOwn;
+  if (!own) atomicAdd(&hdr->big[0].slots, m / kBigSlot);
+  const size_t row = own ? kBigOwnRow * ((size_t)L.n * L.capacity / kRankItems + 1) : 0;
+  reinterpret_cast<BigBucket*>(ws + L.off_big)[row + atomicAdd(own ? &hdr->own_n : &hdr->big[0].n, 1u)] =
       BigBucket{(u64)c * L.capacity + start, lo << 32, end >> 32 ? ~0ull : end << 32, ~0ull, m, big_parts(m), 0u, 0u};
 }
 

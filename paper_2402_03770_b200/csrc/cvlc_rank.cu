@@ -161,7 +161,7 @@ k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
-  if ((hdr->list_n[0] | hdr->list_n[1] | hdr->big[0].n) == 0) return;
+  if ((hdr->list_n[0] | hdr->list_n[1] | hdr->big[0].n | hdr->own_n) == 0) return;
   if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n);
   rank_lists<kRankThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, s_args);
 }

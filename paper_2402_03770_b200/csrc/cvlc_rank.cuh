@@ -569,12 +569,14 @@ __device__ __forceinline__ void find_tile(RankTile& T, const RankArgs& a) {
 // round's buckets (a bucket of more than kBigParts parts).  Values are distinct, so equal keys are split by their indices and no
 // distribution is special.  A step's items are drawn by ticket, and a block waits for the step before when no item of that is left: the
 // blocks it waits for are running.
-// A candidate is read three times and moved twice, whatever the bucket's size, and not moved where its part is never sent.  Steps in
-// this kernel, 2 blocks per SM: bound by the latencies of a piece (12 us for 8192 candidates, most of them the setting up) and of the
-// steps one behind the other (65 us for one bucket of 100,000).  The kernel's time for 4 clients of 50 M coordinates in 16 bits
-// (13.5 M candidates, buckets of 40,000): 335 us; 4 of 50 M on a grid of 24 steps per deviation: 339; one million equal keys in one
-// client of 11.2 M: 110; 10 of 5 M with 250,000 equal keys each: 115.  With every tile ranking its window of a bucket, reading all
-// of it, and digit passes over all candidates for buckets beyond 262,144: 1212, 2925, 308 and 1200.
+// Smaller ones are split by one block each, all steps at once (up to 8192 / 16384 / 32768 / 65536 candidates: 10 clients of 5 M
+// coordinates in 16 bits 111 / 72 / 73 / 72 us, one of 100 M with every seventh layer on a grid 321 / 300 / 292 / 378).
+// A candidate is read three times and moved twice, whatever the bucket's size, and not moved where its part is never sent.  Two
+// blocks per SM: bound by the latencies of a piece (12 us for 8192 candidates, most of them the setting up) and of the steps one
+// behind the other (68 us for one bucket of 100,000).  The kernel's time for 4 clients of 50 M coordinates in 16 bits (13.5 M
+// candidates, buckets of 40,000): 324 us; 4 of 50 M on a grid of 24 steps per deviation: 338; one million equal keys in one client of
+// 11.2 M: 108; 10 of 5 M with 250,000 equal keys each: 118.  With every tile ranking its window of a bucket, reading all of it, and
+// digit passes over all candidates for buckets beyond 262,144: 1212, 2925, 308 and 1200.
 
 __device__ __forceinline__ uint32_t big_parts(uint32_t m) { return m / kBigPart + 1 < kBigParts ? m / kBigPart + 1 : kBigParts; }
 // where a bucket's entries in the tables of parts begin: of its own candidates' slots
@@ -657,47 +659,12 @@ __device__ __forceinline__ void rank_keys(RankShared& s, const u64* src, uint32_
   else rank_with_cells<THREADS>(s, src, n, 0u, first_key - last_key, out, first_key);
 }
 
-// Step 1: the splitters of the round's buckets and their pieces.  A sample of 16 candidates for a part (1024 at least), one from every
-// equal stretch of the bucket at a scattered place of it, since neighbours lie there in the order of the update.  It is ranked where
-// the bucket's parts will lie (8192 of equal keys sorted in shared memory instead: 165 us).
-template <int THREADS>
-__device__ __noinline__ void big_sample(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
-  __shared__ uint32_t s_first;
-  BigRound& R = hdr->big[round];
-  const uint32_t piece_size = big_piece_size(R);
-  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.n);
-  while (true) {
-    const uint32_t i = block_takes(&R.next_sample);
-    if (i >= n) return;
-    const BigBucket b = big_bucket(a, round, i);
-    const u64* src = big_source(a, round, b.pos);
-    u64* sample = big_target(a, round, b.pos);
-    uint32_t samples = 1024;
-    while (samples < kRankItems && samples < 16 * b.parts) samples <<= 1;
-    for (uint32_t t = threadIdx.x; t < samples; t += THREADS) {
-      const uint32_t at = (uint32_t)((u64)t * b.m / samples), width = (uint32_t)((u64)(t + 1) * b.m / samples) - at;
-      sample[t] = src[at + (uint32_t)(((u64)(t * 2654435761u) * width) >> 32)];
-    }
-    __syncthreads();
-    rank_keys<THREADS>(s, sample, samples, ~(uint32_t)(b.from >> 32), ~(uint32_t)((b.to - 1) >> 32), sample);
-    const u64 slot = big_slot(b.pos);
-    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
-      if (p) a.splitter[slot + p - 1] = to_value(sample[(u64)p * samples / b.parts]);
-      a.part_count[slot + p] = 0;
-    }
-    const uint32_t pieces = (b.m + piece_size - 1) / piece_size;
-    if (threadIdx.x == 0) s_first = atomicAdd(&R.pieces, pieces);
-    __syncthreads();
-    for (uint32_t p = threadIdx.x; p < pieces; p += THREADS) a.piece[(size_t)round * a.piece_room + s_first + p] = (u64)i << 32 | p;
-    block_done(&R.done_sample);
-  }
-}
-
 // What a block needs to find a value's part, the number of splitters not above it: the bucket's splitters in s.items, and, where the
 // values between the first and the last of them are cut into equal cells, how many lie in the cells before each, in s.cell behind
 // the parts' counts.  Equal keys differ by their indices, which are spread about evenly: one cell, one splitter or two.  (A search
 // among all splitters, ten steps, took 1.6 times as long.)
 constexpr uint32_t kBigCells = 2048;
+static_assert(kBigRounds == 3, "the second round alone ends in the second buffer");
 struct BigSearch {
   u64 first, last;    // splitters (of a bucket with at least two parts)
   int shift;          // bits of a cell
@@ -767,6 +734,90 @@ __device__ __forceinline__ void big_piece(const RankShared& s, const BigSearch& 
   }
 }
 
+// Where the parts of bucket b, the i-th of the round, begin: their counts are in s.cell (at least kBigParts, zeros behind the last),
+// which then holds the starts.  The parts go to their lists.
+template <int THREADS>
+__device__ __forceinline__ void big_bounds(RankShared& s, EncHeader* hdr, const RankArgs& a, int round, uint32_t i, const BigBucket& b) {
+  const u64 slot = big_slot(b.pos);
+  for (uint32_t p = kBigParts + threadIdx.x; p < 2 * kBigParts; p += THREADS) s.cell[p] = 0u;
+  __syncthreads();
+  scan_cells<THREADS, 2 * kBigParts>(s.cell);
+  for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
+    const uint32_t start = s.cell[p], m = (p + 1 < b.parts ? s.cell[p + 1] : b.m) - start;
+    const bool sent = (b.pos + start) % a.capacity < a.limit;
+    a.part_start[slot + p] = start;
+    if (!sent && p && (b.pos + s.cell[p - 1]) % a.capacity < a.limit) a.big[(size_t)round * a.big_room + i].last = s.items[p - 1] - 1;
+    if (m == 0 || !sent) continue;
+    const u64 from = p ? s.items[p - 1] : b.from, to = p + 1 < b.parts ? s.items[p] : b.to;
+    if (m > kRankItems && round + 1 < kBigRounds) {
+      atomicAdd(&hdr->big[round + 1].slots, m / kBigSlot);
+      a.big[(size_t)(round + 1) * a.big_room + atomicAdd(&hdr->big[round + 1].n, 1u)] = BigBucket{b.pos + start, from, to, ~0ull, m, big_parts(m), 0u, 0u};
+    } else {
+      a.part[atomicAdd(&hdr->part_n, 1u)] = BigPart{b.pos + start, m, round == 1 ? 1u : 0u, ~(uint32_t)(from >> 32), ~(uint32_t)((to - 1) >> 32)};
+    }
+  }
+}
+
+// Step 1: the splitters of a bucket.  A sample of 16 candidates for a part (256 at least), one from every equal stretch of the bucket at
+// a scattered place of it, since neighbours lie there in the order of the update.  It is ranked where the bucket's parts will lie
+// (8192 of equal keys sorted in shared memory instead: 165 us).
+template <int THREADS>
+__device__ __forceinline__ void big_splitters(RankShared& s, const RankArgs& a, const BigBucket& b, const u64* src, u64* sample) {
+  uint32_t samples = 256;
+  while (samples < kRankItems && samples < 16 * b.parts) samples <<= 1;
+  for (uint32_t t = threadIdx.x; t < samples; t += THREADS) {
+    const uint32_t at = (uint32_t)((u64)t * b.m / samples), width = (uint32_t)((u64)(t + 1) * b.m / samples) - at;
+    sample[t] = src[at + (uint32_t)(((u64)(t * 2654435761u) * width) >> 32)];
+  }
+  __syncthreads();
+  rank_keys<THREADS>(s, sample, samples, ~(uint32_t)(b.from >> 32), ~(uint32_t)((b.to - 1) >> 32), sample);
+  const u64 slot = big_slot(b.pos);
+  for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
+    if (p) a.splitter[slot + p - 1] = to_value(sample[(u64)p * samples / b.parts]);
+    a.part_count[slot + p] = 0;
+  }
+}
+// ... of the round's buckets, and their pieces
+template <int THREADS>
+__device__ __noinline__ void big_sample(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
+  __shared__ uint32_t s_first;
+  BigRound& R = hdr->big[round];
+  const uint32_t piece_size = big_piece_size(R);
+  const uint32_t n = *reinterpret_cast<const volatile uint32_t*>(&R.n);
+  while (true) {
+    const uint32_t i = block_takes(&R.next_sample);
+    if (i >= n) return;
+    const BigBucket b = big_bucket(a, round, i);
+    big_splitters<THREADS>(s, a, b, big_source(a, round, b.pos), big_target(a, round, b.pos));
+    const uint32_t pieces = (b.m + piece_size - 1) / piece_size;
+    if (threadIdx.x == 0) s_first = atomicAdd(&R.pieces, pieces);
+    __syncthreads();
+    for (uint32_t p = threadIdx.x; p < pieces; p += THREADS) a.piece[(size_t)round * a.piece_room + s_first + p] = (u64)i << 32 | p;
+    block_done(&R.done_sample);
+  }
+}
+// Buckets of few pieces: all steps by one block, so that none of them waits for others
+template <int THREADS>
+__device__ __noinline__ void big_own(RankShared& s, EncHeader* hdr, const RankArgs& a) {
+  const uint32_t n = hdr->own_n;  // written by the selection alone
+  while (true) {
+    const uint32_t i = block_takes(&hdr->own_next);
+    if (i >= n) return;
+    const BigBucket b = big_bucket(a, kBigOwnRow, i);
+    const u64* src = big_source(a, 0, b.pos);
+    u64* dst = big_target(a, 0, b.pos);
+    big_splitters<THREADS>(s, a, b, src, dst);
+    __syncthreads();
+    const BigSearch h = big_prepare<THREADS>(s, a, b);
+    big_piece<THREADS>(s, h, b, src, 0, b.m, ~0ull, [&](uint32_t p, u64) { atomicAdd(&s.cell[p], 1u); });
+    __syncthreads();
+    big_bounds<THREADS>(s, hdr, a, kBigOwnRow, i, b);
+    __syncthreads();
+    big_piece<THREADS>(s, h, b, src, 0, b.m, big_bucket(a, kBigOwnRow, i).last, [&](uint32_t p, u64 v) { dst[atomicAdd(&s.cell[p], 1u)] = to_item(v); });
+    block_done(&hdr->own_done);
+  }
+}
+
 // Steps 2 and 3: the round's pieces counted; behind a bucket's last piece where its parts begin, and the parts to their lists
 template <int THREADS>
 __device__ __noinline__ void big_count(RankShared& s, EncHeader* hdr, const RankArgs& a, int round) {
@@ -792,23 +843,8 @@ __device__ __noinline__ void big_count(RankShared& s, EncHeader* hdr, const Rank
     __syncthreads();
     if (!s_last) continue;
     __threadfence();
-    for (uint32_t p = threadIdx.x; p < 2 * kBigParts; p += THREADS) s.cell[p] = p < b.parts ? __ldcg(a.part_count + slot + p) : 0u;
-    __syncthreads();
-    scan_cells<THREADS, 2 * kBigParts>(s.cell);
-    for (uint32_t p = threadIdx.x; p < b.parts; p += THREADS) {
-      const uint32_t start = s.cell[p], m = (p + 1 < b.parts ? s.cell[p + 1] : b.m) - start;
-      const bool sent = (b.pos + start) % a.capacity < a.limit;
-      a.part_start[slot + p] = start;
-      if (!sent && p && (b.pos + s.cell[p - 1]) % a.capacity < a.limit) a.big[(size_t)round * a.big_room + i].last = s.items[p - 1] - 1;
-      if (m == 0 || !sent) continue;
-      const u64 from = p ? s.items[p - 1] : b.from, to = p + 1 < b.parts ? s.items[p] : b.to;
-      if (m > kRankItems && round + 1 < kBigRounds) {
-        atomicAdd(&hdr->big[round + 1].slots, m / kBigSlot);
-        a.big[(size_t)(round + 1) * a.big_room + atomicAdd(&hdr->big[round + 1].n, 1u)] = BigBucket{b.pos + start, from, to, ~0ull, m, big_parts(m), 0u, 0u};
-      } else {
-        a.part[atomicAdd(&hdr->part_n, 1u)] = BigPart{b.pos + start, m, round & 1 ? 1u : 0u, ~(uint32_t)(from >> 32), ~(uint32_t)((to - 1) >> 32)};
-      }
-    }
+    for (uint32_t p = threadIdx.x; p < kBigParts; p += THREADS) s.cell[p] = p < b.parts ? __ldcg(a.part_count + slot + p) : 0u;
+    big_bounds<THREADS>(s, hdr, a, round, i, b);
     block_done(&R.done_bounds);
   }
 }
@@ -850,7 +886,7 @@ __device__ __noinline__ void big_rank(RankShared& s, EncHeader* hdr, const RankA
     const BigPart b{v->pos, v->n, v->in_b, v->first_key, v->last_key};
     const u64* src = (b.in_b ? a.buf_b : a.buf_a) + b.pos;
     u64* out = a.buf_a + b.pos;
-    if (b.n > kRankItems) {  // the samples of every round have missed: sorted where it lies
+    if (b.n > kRankItems) {  // the samples have missed: sorted where it lies
       for (uint32_t p = threadIdx.x; p < b.n; p += THREADS) out[p] = to_value(src[p]);
       __syncthreads();
       bitonic_sort(out, b.n, threadIdx.x, THREADS, [] { __syncthreads(); });
@@ -876,6 +912,7 @@ __device__ __noinline__ void rank_big(RankShared& s, EncHeader* hdr, const RankA
     big_place<THREADS>(s, hdr, a, round);
     if (!block_waits(&R.done_place, *reinterpret_cast<const volatile uint32_t*>(&R.pieces), &hdr->status)) return;
   }
+  if (!block_waits(&hdr->own_done, hdr->own_n, &hdr->status)) return;
   big_rank<THREADS>(s, hdr, a);
 }
 
@@ -912,8 +949,11 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
   __shared__ uint32_t s_entry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __syncthreads();  // the arguments are there
-  const bool big = hdr->big[0].n != 0;  // written by the selection alone
-  if (big) big_sample<THREADS>(s, hdr, a, 0);
+  const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the selection alone
+  if (big) {
+    big_sample<THREADS>(s, hdr, a, 0);
+    big_own<THREADS>(s, hdr, a);
+  }
   while (true) {
     __syncthreads();
     if (tid == 0) s_entry = atomicAdd(&hdr->list_next[1], 1u);
