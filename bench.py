@@ -39,11 +39,11 @@ FALLBACK_HBM_GBS = 6650.0
 # proportion to the clients); scaled to the clients of a launch, None for any other configuration, for fewer than
 # 32 clients per launch, and for a kernel that has changed since its capture.
 NCU_TRAFFIC_BYTES_PER_CLIENT = {
-    "k_hist": (1433.83e6 + 44.89e6) / 32,          # the update once, plus the rows' maxima
-    "k_select": (402.58e6 + 172.90e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
-    "k_rank_split": (203.49e6 + 155.95e6) / 32,
-    "k_rank": (203.13e6 + 158.17e6) / 32,
-    "k_pack": (177.98e6 + 55.82e6) / 32,
+    "k_hist": (1433.84e6 + 44.53e6) / 32,          # the update once, plus the rows' maxima
+    "k_select": (402.64e6 + 167.66e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
+    "k_rank_split": (203.46e6 + 154.20e6) / 32,
+    "k_rank": (203.13e6 + 156.04e6) / 32,
+    "k_pack": (177.98e6 + 54.06e6) / 32,
 }
 NOMINAL_HBM_GBS = 8000.0
 

@@ -233,7 +233,6 @@ struct PlanShared {
   uint32_t n[32];
   double beta, D, alpha, alpha_q;
   unsigned long long warp_tot[32];
-  unsigned long long carry;
   uint32_t warp_cnt[32];
   uint32_t n_points;
 };
@@ -1301,7 +1300,7 @@ static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape
   uint16_t* row_max = reinterpret_cast<uint16_t*>(w + plan_off_row_max(n));
   // header, histograms, flags and tuning keys start at zero; the rest is written in full by the kernels that follow
   const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), 0, 0, st);
-  // two resident blocks per SM share the concatenated updates evenly
+  // the resident blocks share the concatenated updates evenly
   launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape.d, part, hist, flags, row_max);
   if (hist_out) {
     // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
