@@ -485,7 +485,7 @@ def run_ours(args):
         "plan_of_client_0": {"k": int(plans[0].k), "R": int(plans[0].R), "n_candidates": int(plans[0].n_candidates), "alpha_q": plans[0].alpha_q,
                  "lengths": {str(y): int(plans[0].n_y[y]) for y in range(33) if plans[0].n_y[y]}},
         "phase_ms_per_step": {
-            "plan": sum(kernels[k]["ms_per_step"] for k in ("k_zero_words", "k_hist", "k_plan_fit", "k_plan_tune")
+            "plan": sum(kernels[k]["ms_per_step"] for k in ("k_zero_words", "k_hist", "k_plan_threshold", "k_plan_fit", "k_plan_tune")
                         if k in kernels),
             "encode": sum(kernels[k]["ms_per_step"] for k in ("k_encode_init", "k_select", "k_select_lookback", "k_rank_split",
                                                                 "k_rank", "k_rank_rest", "k_sort", "k_pack") if k in kernels),

@@ -120,6 +120,27 @@ int batch_shape(const cvlc_params* params, uint32_t i, uint32_t fixed_y, Shape* 
   return coeff_g(quant_Q(p.quantizer, S->cap[p.max_code_bits], p.max_code_bits), p.scale_B) > 0.0 ? CVLC_OK : CVLC_ERR_SCALE_TOO_SMALL;
 }
 
+// Records of a packet at the shortest candidate length: the shortest with g > 0 or, where the next one holds as many records, the
+// last of those (the planning kernels' list of candidates begins with it)
+uint32_t shortest_cap(const Shape& S, double B) {
+  uint32_t y = S.fixed_y;
+  if (y == 0) {
+    y = 1;
+    while (y < S.max_code_bits && !(coeff_g(quant_Q(S.quantizer, S.cap[y], y), B) > 0.0)) ++y;
+    while (y < S.max_code_bits && S.cap[y] <= S.cap[y + 1]) ++y;
+  }
+  return S.cap[y];
+}
+// the part of a client's descriptor that its parameters give; `before`: the client in front of it, or nullptr
+void describe(ClientDesc* desc, const ClientDesc* before, const Shape& S, const cvlc_params& p) {
+  desc->seed = p.seed;
+  desc->scale_B = p.scale_B;
+  desc->client_id = p.client_id;
+  desc->round = p.round;
+  desc->cap0 = before && before->scale_B == p.scale_B ? before->cap0 : shortest_cap(S, p.scale_B);
+  desc->pad = 0;
+}
+
 bool aligned(const void* p, size_t a) { return p && (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 size_t plan_ws_bytes_of(uint64_t d, uint32_t n) { return plan_ws_bytes(make_partition(d, n), n); }
@@ -207,10 +228,7 @@ int cvlc_plan_batch(const float* const* x_dev, const cvlc_params* params, uint32
     desc[i].x = x_dev[i];
     desc[i].plan = plans_dev + i;
     desc[i].stream = nullptr;
-    desc[i].seed = params[i].seed;
-    desc[i].scale_B = params[i].scale_B;
-    desc[i].client_id = params[i].client_id;
-    desc[i].round = params[i].round;
+    describe(desc + i, i ? desc + i - 1 : nullptr, S, params[i]);
   }
   if (!aligned(plans_dev, 8) || !aligned(ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
   if (ws_bytes < plan_ws_bytes_of(S.d, n)) return CVLC_ERR_WORKSPACE_TOO_SMALL;
@@ -249,10 +267,7 @@ int cvlc_plan_from_histogram_batch(const uint64_t* hist_dev, const cvlc_params* 
     if (rc != CVLC_OK) return rc;
     memset(&desc[i], 0, sizeof desc[i]);
     desc[i].plan = plans_dev + i;
-    desc[i].seed = params[i].seed;
-    desc[i].scale_B = params[i].scale_B;
-    desc[i].client_id = params[i].client_id;
-    desc[i].round = params[i].round;
+    describe(desc + i, i ? desc + i - 1 : nullptr, S, params[i]);
   }
   if (!aligned(hist_dev, 8) || !aligned(plans_dev, 8) || !aligned(ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
   if (ws_bytes < plan_ws_bytes_of(S.d, n)) return CVLC_ERR_WORKSPACE_TOO_SMALL;
@@ -332,10 +347,7 @@ static int encode_batch(const float* const* x_dev, const cvlc_params* params, ui
     desc[i].x = x_dev[i];
     desc[i].plan = const_cast<cvlc_plan_t*>(plans_dev) + i;
     desc[i].stream = streams_dev[i];
-    desc[i].seed = params[i].seed;
-    desc[i].scale_B = params[i].scale_B;
-    desc[i].client_id = params[i].client_id;
-    desc[i].round = params[i].round;
+    describe(desc + i, i ? desc + i - 1 : nullptr, S, params[i]);
   }
   if (!aligned(plans_dev, 8) || !aligned(ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
   if (plan_ws_dev && !aligned(plan_ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
@@ -423,10 +435,7 @@ int cvlc_encode_unframed_batch(const float* const* x_dev, const cvlc_params* par
     desc[i].x = x_dev[i];
     desc[i].plan = const_cast<cvlc_plan_t*>(plans_dev) + i;
     desc[i].stream = streams_dev[i];
-    desc[i].seed = params[i].seed;
-    desc[i].scale_B = params[i].scale_B;
-    desc[i].client_id = params[i].client_id;
-    desc[i].round = params[i].round;
+    describe(desc + i, i ? desc + i - 1 : nullptr, S, params[i]);
   }
   if (!aligned(plans_dev, 8) || !aligned(enc_ws_dev, 256) || !aligned(uf_ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
   if (plan_ws_dev && !aligned(plan_ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
@@ -502,10 +511,7 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
     desc[i].x = x_dev[i];
     desc[i].plan = plans_dev + i;
     desc[i].stream = streams_dev[i];
-    desc[i].seed = params[i].seed;
-    desc[i].scale_B = params[i].scale_B;
-    desc[i].client_id = params[i].client_id;
-    desc[i].round = params[i].round;
+    describe(desc + i, i ? desc + i - 1 : nullptr, S, params[i]);
   }
   if (!aligned(plans_dev, 8) || !aligned(plan_ws_dev, 256) || !aligned(enc_ws_dev, 256)) return CVLC_ERR_INVALID_ARG;
   if (plan_ws_bytes < plan_ws_bytes_of(S.d, n)) return CVLC_ERR_WORKSPACE_TOO_SMALL;
@@ -518,19 +524,19 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   const bool two = side_stream != nullptr && side_st != main_st;
   Shape Senc = S;
   Senc.fixed_y = 0;
-  if (launch_plan_front(desc, n, S, plan_ws_dev, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_plan_front(desc, n, S, plan_ws_dev, enc_front(enc_layout(S.d, n, cap), enc_ws_dev), main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
-    if (launch_plan_back(n, S, plan_ws_dev, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
+    if (launch_plan_back(n, S, plan_ws_dev, main_st, true, true) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
-  // the length tuning reads the histograms' fit only; selection and ranking do not need its result.  The lock keeps two
+  // exponent fit and length tuning read the histograms only; selection and ranking do not need their result.  The lock keeps two
   // threads from recording the device's events between each other's record and wait.
   static std::mutex order;
   std::lock_guard<std::mutex> hold(order);
   cudaEvent_t fork, join;
   if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;
-  if (launch_plan_back(n, S, plan_ws_dev, side_st, false) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_plan_back(n, S, plan_ws_dev, side_st, false, false) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(join, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
   return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
 }

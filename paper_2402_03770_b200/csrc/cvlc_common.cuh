@@ -39,6 +39,8 @@ struct ClientDesc {
   double scale_B;      // B of the scaling operation
   uint32_t client_id;  // Philox counter word 2
   uint32_t round;      // Philox counter word 3
+  uint32_t cap0;       // planning: records of a packet at the shortest candidate length
+  uint32_t pad;
 };
 
 constexpr int kSmallBatch = 4;
@@ -83,6 +85,7 @@ struct Partition {
   uint64_t chunk;     // rows per chunk of the histogram kernel
   uint32_t n_chunks;
   uint32_t grid;      // its blocks
+  uint32_t per_client;  // chunks of a client where they are cut from each client on its own; 0: from the concatenated rows
 };
 CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   Partition P;
@@ -98,6 +101,15 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   P.grid = (uint32_t)grid;
   // two chunks per block where that leaves each a megabyte and more: every chunk ends with a merge into a client's histogram
   // (with two of 64 KB and more 10 clients of 5 M coordinates take 53 us)
+  P.per_client = 0;
+  const uint64_t of_client = grid / n;
+  if (P.total <= (8u << 20) && of_client * n * 16 >= grid * 15) {
+    // a chunk then has one client: one merge per block, and the clients are finished by as many blocks (see finish_client)
+    P.chunk = ((P.rows + of_client - 1) / of_client + 15) & ~(uint64_t)15;
+    P.per_client = (uint32_t)((P.rows + P.chunk - 1) / P.chunk);
+    P.n_chunks = P.grid = P.per_client * n;
+    return P;
+  }
   const uint64_t n_chunks = P.total / (2 * grid) >= 16384 ? 2 * grid : grid;
   P.chunk = ((P.total + n_chunks - 1) / n_chunks + 15) & ~(uint64_t)15;
   P.n_chunks = (uint32_t)((P.total + P.chunk - 1) / P.chunk);
@@ -105,10 +117,11 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
 }
 
 // plan workspace:
-//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint64 tune_key[n][2] | ClientDesc[n]
-//   | uint32 bin_start[n][4096] | uint32 max_bin[n] | uint16 row_max[n][rows]
+//   [0] PlanWsHeader | [256] uint64 hist[n][4096] | uint32 nonfinite[n] | uint32 rows_done[n] | uint64 tune_key[n][2]
+//   | ClientDesc[n] | uint32 bin_start[n][4096] | uint32 max_bin[n] | uint16 row_max[n][rows]
+// rows_done: rows in the client's histogram, where the block that completes it works out the threshold and the bins' starts.
 // bin_start: candidates of the client in the bins above this one; max_bin: candidates in its fullest bin.
-// tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths;
+// tune_key = (bits of alpha_q, bits of scale_B): clients of a batch with equal keys have the same code lengths; in a large batch
 // the first of them runs the length tuning and writes the result to all.
 struct PlanWsHeader {
   int32_t status;   // byte 0
@@ -120,7 +133,8 @@ struct PlanWsHeader {
 constexpr uint32_t kPlanWsMagic = 0x53454743u;
 constexpr size_t kPlanWsHist = 256;
 CVLC_HD constexpr size_t plan_off_flags(uint32_t n) { return kPlanWsHist + (size_t)n * CVLC_HIST_BINS * 8; }
-CVLC_HD constexpr size_t plan_off_keys(uint32_t n) { return align256(plan_off_flags(n) + (size_t)n * 4); }
+CVLC_HD constexpr size_t plan_off_rows_done(uint32_t n) { return plan_off_flags(n) + (size_t)n * 4; }
+CVLC_HD constexpr size_t plan_off_keys(uint32_t n) { return align256(plan_off_rows_done(n) + (size_t)n * 4); }
 CVLC_HD constexpr size_t plan_off_desc(uint32_t n) { return align256(plan_off_keys(n) + (size_t)n * 16); }
 CVLC_HD constexpr size_t plan_off_bin_start(uint32_t n) { return align256(plan_off_desc(n) + (size_t)n * sizeof(ClientDesc)); }
 CVLC_HD constexpr size_t plan_off_max_bin(uint32_t n) { return align256(plan_off_bin_start(n) + (size_t)n * CVLC_HIST_BINS * 4); }
@@ -141,9 +155,9 @@ struct EncHeader {
   uint32_t limit;           // ranks from here on are never sent
   uint32_t select_ticket;   // tile tickets of the look-back selection
   uint32_t split_ticket, rank_ticket;  // tile tickets of the partition and of the final ranking
-  uint32_t split_tiles;     // largest per-client tile count among the clients that need the partition
-  uint32_t window;          // candidates per tile of the final ranking
-  uint32_t rank_tiles;      // largest per-client tile count of the final ranking
+  uint32_t most;            // candidates of the largest client, as far as they are ranked
+  uint32_t most_split;      // candidates of the largest client that needs the partition
+  uint32_t sort_tiles;      // all clients' tiles of kSortTile candidates
   uint32_t list_n[2], list_next[2];  // entries of the ranking's lists (of cells for a warp and for a block) and of them taken
   BigRound big[kBigRounds];
   uint32_t own_n, own_next, own_done;  // large buckets that a block splits by itself, of them taken, finished
@@ -338,7 +352,7 @@ CVLC_HD constexpr size_t dec_ws_bytes(uint32_t n) { return align256(dec_off_meta
 // ---- launch accounting and optional per-kernel timing ------------------------------
 
 enum KernelId {
-  kKZeroWords = 0, kKHist, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
+  kKZeroWords = 0, kKHist, kKPlanThreshold, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
   kKRankRest, kKSort, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
   kKPlanLiteral, kKEcAccumulate, kKPackUnframed, kKDecodeUnframed, kNumKernelIds
 };
@@ -411,12 +425,21 @@ __device__ __forceinline__ void pdl_enter() {
 
 // ---- launchers (one per translation unit) ---------------------------------------
 
-// Planning is launched in two parts.  The front (histogram, rows' maxima, exponent fit, selection threshold, the bins'
-// starts) is all the selection and ranking kernels need; the back (length tuning, copied to the clients that share a
-// tuning key) is only needed by the packing kernel, so it may run on another stream next to selection and ranking.
-cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
-// overlap: nothing but the planning front precedes it on the stream (no wait for an event)
-cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap);
+// What the planning front prepares for the encoder of the same call (ws = nullptr: nothing): its workspace's header, the clients'
+// shapes of the ranking, the counters of selection and partition at zero
+struct EncFront {
+  unsigned char* ws;
+  uint64_t capacity;
+  size_t off_rank, off_pass_mask, zero_end;
+};
+
+// Planning is launched in two parts.  The front (histogram, rows' maxima, selection threshold, the bins' starts) is all the
+// selection and ranking kernels need; the back (exponent fit and length tuning) is only needed by the packing kernel, so it may
+// run on another stream next to selection and ranking.
+cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st);
+constexpr uint32_t kTuneRoom = 32;  // clients whose tuning blocks selection and ranking leave an SM each (see launch_encode)
+// overlap: nothing but the planning front precedes it on the stream (no wait for an event); alone: nothing runs beside it
+cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st);
@@ -442,9 +465,12 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
 // the error-compensation memory (the input buffers are written: every sent coordinate loses what the parameter
 // server rebuilds for it); kPackNone = selection and ranking only (the unframed writer follows)
 constexpr int kPackFramed = 0, kPackResidual = 1, kPackNone = 2;
-// overlap: the planning of the same call precedes it on the stream
+// prepared: the planning front of the same call has prepared the workspace (see EncFront) and precedes it on the stream
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual);
+                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual);
+static inline EncFront enc_front(const EncLayout& L, void* ws) {
+  return EncFront{static_cast<unsigned char*>(ws), L.capacity, L.off_rank, L.off_pass_mask, L.off_sub_start};
+}
 cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st);
 // unframed stream (version 2)
 constexpr uint32_t kUfMaxRecords = 2048;  // records of a block (it is sorted and assembled in one warp's shared memory)
@@ -529,7 +555,8 @@ __device__ __forceinline__ uint32_t philox_coord(const PhiloxRoundKeys& rk, uint
   return c.x;
 }
 
-__device__ __forceinline__ uint32_t sort_keytop(const cvlc_plan_t* plan) { return ((plan->top_bin + 1u) << 19) - 1u; }
+__device__ __forceinline__ uint32_t sort_keytop(uint32_t top_bin) { return ((top_bin + 1u) << 19) - 1u; }
+__device__ __forceinline__ uint32_t sort_keytop(const cvlc_plan_t* plan) { return sort_keytop(plan->top_bin); }
 // candidates of a client in the coarse buckets before bucket i (bins from the top down)
 __device__ __forceinline__ uint32_t coarse_start(const ClientRank& r, const uint32_t* bin_start, uint32_t i) {
   return i < r.n_coarse ? bin_start[r.top_bin - (i << r.group)] : r.n;
@@ -538,6 +565,44 @@ __device__ __forceinline__ uint32_t coarse_start(const ClientRank& r, const uint
 __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
   // first error wins
   atomicCAS(status, 0, code);
+}
+
+__device__ __forceinline__ uint32_t sort_tiles_of(unsigned long long n_candidates, unsigned long long capacity) {
+  const unsigned long long nc = n_candidates < capacity ? n_candidates : capacity;
+  return (uint32_t)((nc + kSortTile - 1) / kSortTile);
+}
+
+// ranks from here on are never sent, whatever the lengths
+CVLC_HD inline uint32_t rank_limit(const Shape& shape) {
+  const unsigned long long most_sent = (unsigned long long)shape.R * shape.cap[1];
+  return most_sent < 0xFFFFFFFFull ? (uint32_t)most_sent : 0xFFFFFFFFu;
+}
+
+// a client's buckets from its plan's threshold and the tables beside it
+__device__ __forceinline__ ClientRank client_rank(uint32_t thresh_bin, uint32_t top_bin, unsigned long long n_candidates, uint32_t max_bin,
+                                                  unsigned long long capacity) {
+  ClientRank r;
+  const uint32_t top = top_bin < CVLC_HIST_BINS ? top_bin : CVLC_HIST_BINS - 1;
+  const uint32_t nb = thresh_bin <= top ? top - thresh_bin + 1 : 1;
+  rank_shape(nb, max_bin, &r);
+  r.n = (uint32_t)(n_candidates < capacity ? n_candidates : capacity);
+  r.keytop = sort_keytop(top_bin);
+  r.top_bin = top;
+  return r;
+}
+
+// a client's share of what the encoder's header says of the batch; by one thread, the header starts at zero
+__device__ __forceinline__ void add_client(EncHeader* hdr, const ClientRank& r, uint32_t limit, unsigned long long capacity) {
+  atomicMax(&hdr->most, r.n < limit ? r.n : limit);  // buckets from the limit on are not ranked
+  if (r.split) atomicMax(&hdr->most_split, r.n);
+  atomicAdd(&hdr->sort_tiles, sort_tiles_of(r.n, capacity));
+}
+// candidates per tile of the final ranking: small enough that the batch gives every SM several tiles
+__device__ __forceinline__ uint32_t rank_window(const EncHeader* hdr) {
+  const uint64_t want = ((uint64_t)hdr->sort_tiles * kSortTile + 4 * kNumSM - 1) / (4 * kNumSM);
+  uint32_t window = kRankWindow;
+  while (window > 1024 && window / 2 >= want) window >>= 1;
+  return window;
 }
 
 #endif  // __CUDACC__

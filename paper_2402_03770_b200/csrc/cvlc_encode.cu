@@ -13,14 +13,10 @@
 
 namespace cvlc {
 
-__device__ __forceinline__ uint32_t sort_tiles_of(unsigned long long n_candidates, unsigned long long capacity) {
-  const unsigned long long nc = n_candidates < capacity ? n_candidates : capacity;
-  return (uint32_t)((nc + kSortTile - 1) / kSortTile);
-}
-
 // ===================================================================================
 // K0  workspace reset, plan validation, sort-tile prefix over the clients
 // ===================================================================================
+// Where a plan comes from an earlier call; the planning front of cvlc_compress_batch does without (see EncFront).
 // The grid zeroes the per-client counters, digit histograms and look-back states; block 0
 // alone owns the 256-byte header and the sort-tile prefix (nobody else writes them).
 
@@ -33,8 +29,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
   __shared__ uint32_t s_most, s_most_split;  // candidates of the largest client / of the largest one that needs the partition
   __shared__ uint32_t s_tiles[CVLC_MAX_BATCH];  // sort tiles of every client
   const uint32_t n = batch.n;
-  const unsigned long long most_sent = (unsigned long long)shape.R * shape.cap[1];  // no plan sends more
-  const uint32_t limit = most_sent < 0xFFFFFFFFull ? (uint32_t)most_sent : 0xFFFFFFFFu;
+  const uint32_t limit = rank_limit(shape);
   pdl_enter();
   if (threadIdx.x == 0) {
     s_total = 0;
@@ -57,13 +52,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
       t += tiles;
       if (plan->top_bin + 1u - plan->thresh_bin > 256u) pass3 = 1;  // see top_digit_is_zero
       if (max_bin) {
-        ClientRank r;
-        const uint32_t top = plan->top_bin < CVLC_HIST_BINS ? plan->top_bin : CVLC_HIST_BINS - 1;
-        const uint32_t nb = plan->thresh_bin <= top ? top - plan->thresh_bin + 1 : 1;
-        rank_shape(nb, max_bin[c], &r);
-        r.n = (uint32_t)(plan->n_candidates < L.capacity ? plan->n_candidates : L.capacity);
-        r.keytop = sort_keytop(plan);
-        r.top_bin = top;
+        const ClientRank r = client_rank(plan->thresh_bin, plan->top_bin, plan->n_candidates, max_bin[c], L.capacity);
         atomicMax(&s_most, r.n < limit ? r.n : limit);  // buckets from the limit on are not ranked
         if (r.split) atomicMax(&s_most_split, r.n);
         if (blockIdx.x == 0) reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;
@@ -131,13 +120,9 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     hdr->list_n[0] = hdr->list_n[1] = hdr->list_next[0] = hdr->list_next[1] = 0;
     for (int r = 0; r < kBigRounds; ++r) hdr->big[r] = BigRound{};
     hdr->own_n = hdr->own_next = hdr->own_done = hdr->part_n = hdr->part_next = 0;
-    hdr->split_tiles = (s_most_split + kRankSplitTile - 1) / kRankSplitTile;
-    // tiles small enough that the batch gives every SM several
-    const uint64_t want = ((uint64_t)run * kSortTile + 4 * kNumSM - 1) / (4 * kNumSM);
-    uint32_t window = kRankWindow;
-    while (window > 1024 && window / 2 >= want) window >>= 1;
-    hdr->window = window;
-    hdr->rank_tiles = (s_most + window - 1) / window;
+    hdr->most = s_most;
+    hdr->most_split = s_most_split;
+    hdr->sort_tiles = run;
   }
   // ranked by partition: the result is in the first buffer (the digit passes write a mask of their own)
   if (plan_ws)
@@ -1378,12 +1363,12 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
 
 template <int CAP>
 static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, const unsigned char* plan_ws,
-                          unsigned char* w, cudaStream_t st, bool overlap) {
+                          unsigned char* w, cudaStream_t st) {
   BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
-  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, overlap, w, batch, shape, L, plan_ws);
+  launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, false, w, batch, shape, L, plan_ws);
 }
 
 template <int CAP>
@@ -1410,11 +1395,10 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
 // SMs given away cost the clients times the length of the selection.  Whole calls with room and without, us: 24 clients of 0.3 M
 // coordinates 90 and 100, 32 of 0.3 / 1.2 / 3 M 98 and 111 / 195 and 203 / 385 and 390, 40 of 0.3 / 1.2 / 3 M 107 and 117 / 239 and 226
 // / 475 and 441; 10 of 13 / 20 / 40 M 319 and 346 / 434 and 467 / 816 and 820, 20 of 6 / 12 M 309 and 315 / 548 and 514.
-constexpr uint32_t kTuneRoom = 32;
 constexpr uint64_t kTuneRoomRows = 192 << 20;  // times clients
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, bool overlap, cudaEvent_t wait_before_pack, int write_residual) {
+                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual) {
   static OncePerDevice once;
   cudaError_t e = once_per_device(once, [] {
     const cudaError_t e = allow_shared(k_select, kSelSmem);
@@ -1431,10 +1415,11 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const Partition part = make_partition(shape.d, n);
   const unsigned sms = wait_before_pack && n <= kTuneRoom && n * part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
-  if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st, overlap);
-  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st, overlap);
-  else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st, overlap);
-  const Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
+  Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
+  if (prepared) batch.c = reinterpret_cast<const ClientDesc*>(pws + plan_off_desc(n));
+  else if (n <= (uint32_t)kSmallBatch) launch_init_t<kSmallBatch>(clients, n, shape, L, pws, w, st);
+  else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st);
+  else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st);
   if (pws) {
     const uint64_t want = (uint64_t)select_groups(part, n).groups * n;
     const unsigned grid = (unsigned)(want < (uint64_t)sms ? want : sms);

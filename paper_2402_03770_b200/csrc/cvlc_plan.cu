@@ -12,117 +12,6 @@
 namespace cvlc {
 
 // ===================================================================================
-// K1  magnitude histogram: h[key >> 19], key = bits(|x|); HBM-bound, 4 bytes / coordinate
-// ===================================================================================
-
-constexpr int kHistThreads = kStreamThreads;
-constexpr int kHistSub = 2;  // shared sub-histograms per block (32 KB)
-
-// The clients' rows form one concatenated array that is cut into equal contiguous chunks, one or two
-// per block, so the load is even whatever the number of clients; a block that crosses a client
-// boundary merges its shared histogram into that client's global one and starts afresh.
-
-// counts the four magnitude keys of a float4; returns the largest of them
-__device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
-  const uint32_t k0 = __float_as_uint(a.x) & 0x7FFFFFFFu, k1 = __float_as_uint(a.y) & 0x7FFFFFFFu;
-  const uint32_t k2 = __float_as_uint(a.z) & 0x7FFFFFFFu, k3 = __float_as_uint(a.w) & 0x7FFFFFFFu;
-  atomicAdd(my + (k0 >> 19), 1u);
-  atomicAdd(my + (k1 >> 19), 1u);
-  atomicAdd(my + (k2 >> 19), 1u);
-  atomicAdd(my + (k3 >> 19), 1u);
-  const uint32_t m01 = k0 > k1 ? k0 : k1, m23 = k2 > k3 ? k2 : k3;
-  return m01 > m23 ? m01 : m23;
-}
-
-__global__ void __launch_bounds__(kHistThreads, 3)
-k_hist(const Batch batch, uint64_t d, const __grid_constant__ Partition part,
-       unsigned long long* __restrict__ hist_all, uint32_t* __restrict__ nonfinite_all, uint16_t* __restrict__ row_max_all) {
-  extern __shared__ uint32_t sh_hist[];  // [kHistSub][4096]
-  pdl_enter();
-  for (int i = threadIdx.x; i < kHistSub * CVLC_HIST_BINS; i += kHistThreads) sh_hist[i] = 0;
-  __syncthreads();
-  uint32_t* my = sh_hist + ((threadIdx.x >> 5) & (kHistSub - 1)) * CVLC_HIST_BINS;
-  const int lane = threadIdx.x & 31;
-
-  const uint64_t nvec = d >> 2;
-  for (uint32_t q = blockIdx.x; q < part.n_chunks; q += gridDim.x) {
-  uint64_t pos = (uint64_t)q * part.chunk;
-  const uint64_t end = (pos + part.chunk < part.total) ? pos + part.chunk : part.total;
-
-  while (pos < end) {
-    const uint64_t c = pos / part.rows;
-    const uint64_t seg_end = ((c + 1) * part.rows < end) ? (c + 1) * part.rows : end;
-    const uint64_t u0 = (pos - c * part.rows) * kRowUnits, u1 = (seg_end - c * part.rows) * kRowUnits;  // units of the client
-    const float* __restrict__ x = batch.c[c].x;
-    const float4* xv = reinterpret_cast<const float4*>(x);
-    const uint64_t v1 = (u1 < nvec) ? u1 : nvec;  // float4 units of this segment: [u0, v1)
-    uint16_t* __restrict__ row_max = row_max_all + c * part.rows;
-    static_assert(kRowUnits == 4, "a row is held by four neighbouring lanes");
-    uint32_t top = 0;
-    uint64_t v = u0 + threadIdx.x;
-    // four independent 128-bit loads in flight per thread; the loop condition is the same for the lanes of a warp
-    for (; (v - lane) + 31 + 3 * kHistThreads < v1; v += 4 * kHistThreads) {
-      float4 a[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = __ldg(xv + v + u * kHistThreads);
-      uint32_t m[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        m[u] = hist_add4(my, a[u]);
-        top = m[u] > top ? m[u] : top;
-      }
-      // The rows' maxima of the four loads, two bins to a word: the first exchange leaves an even lane with loads 0 and 1, an odd
-      // lane with 2 and 3, the second completes the rows; each lane then stores one of its row's four.
-      const uint32_t w01 = m[0] >> 19 | (m[1] >> 3 & 0xFFFF0000u), w23 = m[2] >> 19 | (m[3] >> 3 & 0xFFFF0000u);
-      uint32_t w = __vmaxu2(lane & 1 ? w23 : w01, __shfl_xor_sync(0xFFFFFFFFu, lane & 1 ? w01 : w23, 1));
-      w = __vmaxu2(w, __shfl_xor_sync(0xFFFFFFFFu, w, 2));
-      const uint32_t load = ((lane & 1) << 1) | (lane >> 1 & 1);
-      row_max[(v + load * kHistThreads) / kRowUnits] = (uint16_t)(lane & 2 ? w >> 16 : w);
-    }
-    for (; v - lane < v1; v += kHistThreads) {  // rows that may end inside the warp
-      const bool on = v < v1;
-      uint32_t m = on ? hist_add4(my, __ldg(xv + v)) : 0u;
-      top = m > top ? m : top;
-      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-      if (lane % kRowUnits == 0 && on) row_max[v / kRowUnits] = (uint16_t)(m >> 19);
-    }
-    // ragged tail of the client (d not a multiple of 4)
-    if (seg_end == (c + 1) * part.rows && threadIdx.x < (d & 3)) {
-      const uint32_t k0 = __float_as_uint(x[(nvec << 2) + threadIdx.x]) & 0x7FFFFFFFu;
-      top = k0 > top ? k0 : top;
-      atomicAdd(my + (k0 >> 19), 1u);
-    }
-    if (top >= 0x7F800000u) atomicOr(nonfinite_all + c, 1u);  // a key of exponent 255: Inf or NaN
-    __syncthreads();
-    unsigned long long* __restrict__ hist = hist_all + (size_t)c * CVLC_HIST_BINS;
-    for (int b = threadIdx.x; b < CVLC_HIST_BINS; b += kHistThreads) {
-      uint32_t cnt = 0;
-#pragma unroll
-      for (int sub = 0; sub < kHistSub; ++sub) {
-        cnt += sh_hist[sub * CVLC_HIST_BINS + b];
-        sh_hist[sub * CVLC_HIST_BINS + b] = 0;
-      }
-      if (cnt) atomicAdd(hist + b, (unsigned long long)cnt);
-    }
-    __syncthreads();
-    pos = seg_end;
-  }
-  }
-}
-
-// zeroes two ranges of the workspace and leaves the clients' descriptors in it
-template <int CAP>
-__global__ void __launch_bounds__(256)
-k_zero_words(const __grid_constant__ BatchDesc<CAP> batch, ClientDesc* desc, uint4* p, size_t n16, uint4* q, size_t m16) {
-  pdl_enter();
-  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t i = first; i < batch.n; i += stride) desc[i] = batch.c[i];
-  for (size_t i = first; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (size_t i = first; i < m16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// ===================================================================================
 // Series arithmetic of the planner
 // ===================================================================================
 
@@ -186,10 +75,12 @@ __device__ __forceinline__ double energy_E(uint64_t Z, double beta, double D) {
 }
 
 // ===================================================================================
-// K2  planner: per client a fit kernel (one CTA of 1024 threads) and a tuning kernel
+// K2  planner: threshold and bins' starts by the histogram's blocks, exponent fit and length tuning
 // ===================================================================================
 
-constexpr int kPlanThreads = 1024;  // the fit kernel: one thread per four histogram bins
+constexpr int kPlanThreads = 512;  // of the blocks that work on one client's histogram: that of the histogram, the fit's, the tuning's
+constexpr int kPlanBins = CVLC_HIST_BINS / kPlanThreads;
+constexpr size_t kSurvivalBytes = (CVLC_HIST_BINS + 4) * 4;  // survival counts in shared memory
 // The tuning kernel decides most atomic operations with one warp per operation or per trial split (see tune_fast below):
 // 16 warps are as many operations as a sweep over neighbouring lengths usually has, and a 17-way search.
 constexpr int kTuneThreads = 512;
@@ -231,10 +122,7 @@ struct PlanSolver {
 struct PlanShared {
   double Fv[32];
   uint32_t n[32];
-  double beta, D, alpha, alpha_q;
-  unsigned long long warp_tot[32];
-  uint32_t warp_cnt[32];
-  uint32_t n_points;
+  double D;
 };
 
 // candidate lengths of one client and their coefficients (Eq. (5)), built by warp 0
@@ -247,10 +135,15 @@ struct PlanTab {
   double QY[32];      // PQ error factor Q(Y[i]) = cap / (2^y - 1)^2
 };
 
-// candidate lengths: g(y) > 0 (the paper's B > (Q+1)/2) and not dominated; called by one full warp
-__device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, double B_in, int lane) {
+// Candidate lengths: g(y) > 0 (the paper's B > (Q+1)/2) and not dominated; called by one full warp, lane = length - 1.
+struct PlanLength {
+  unsigned member;      // bit y - 1: length y is a candidate
+  uint32_t cap, y_min;  // of this lane's length; shortest usable length
+  double g, Q;          // of this lane's length
+};
+__device__ __forceinline__ PlanLength plan_lengths(const Shape& shape, double B, int lane) {
+  PlanLength P;
   const uint32_t y = lane + 1;
-  const double B = B_in;
   const bool in_range = y <= shape.max_code_bits;
   const uint32_t cap_y = in_range ? shape.cap[y] : 0u;
   double Q;  // error factor of cap(y) values at y bits (Appendix, case study)
@@ -266,61 +159,422 @@ __device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, d
   }
   const double one_m = __dsub_rn(1.0, __ddiv_rn(1.0, B));
   const double g = __dsub_rn(1.0, __dadd_rn(__ddiv_rn(Q, __dmul_rn(B, B)), __dmul_rn(one_m, one_m)));
-  unsigned member;
-  uint32_t y_min;
   if (shape.fixed_y) {
-    y_min = shape.fixed_y;
-    member = 1u << (shape.fixed_y - 1);
+    P.y_min = shape.fixed_y;
+    P.member = 1u << (shape.fixed_y - 1);
   } else {
     const unsigned pos = __ballot_sync(kFull, in_range && g > 0.0);
-    y_min = pos ? (uint32_t)__ffs(pos) : 1u;  // the host has checked that one exists
+    P.y_min = pos ? (uint32_t)__ffs(pos) : 1u;  // the host has checked that one exists
     const uint32_t cap_next = __shfl_down_sync(kFull, cap_y, 1);
-    const bool keep = in_range && y >= y_min && (y == shape.max_code_bits || cap_y > cap_next);
-    member = __ballot_sync(kFull, keep);
+    const bool keep = in_range && y >= P.y_min && (y == shape.max_code_bits || cap_y > cap_next);
+    P.member = __ballot_sync(kFull, keep);
   }
-  if (member & (1u << lane)) {
-    const int i = __popc(member & ((1u << lane) - 1u));
-    T.Y[i] = y;
-    T.capY[i] = cap_y;
-    T.gY[i] = g;
-    T.QY[i] = Q;
+  P.cap = cap_y;
+  P.g = g;
+  P.Q = Q;
+  return P;
+}
+// zeroes two ranges of the workspace and leaves the clients' descriptors in it
+template <int CAP>
+__global__ void __launch_bounds__(256)
+k_zero_words(const __grid_constant__ BatchDesc<CAP> batch, ClientDesc* desc, uint4* p, size_t n16, uint4* q, size_t m16) {
+  pdl_enter();
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = first; i < batch.n; i += stride) desc[i] = batch.c[i];
+  for (size_t i = first; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = first; i < m16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// the table of one client's candidate lengths, by one full warp
+__device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, double B, int lane) {
+  const PlanLength P = plan_lengths(shape, B, lane);
+  if (P.member & (1u << lane)) {
+    const int i = __popc(P.member & ((1u << lane) - 1u));
+    T.Y[i] = lane + 1;
+    T.capY[i] = P.cap;
+    T.gY[i] = P.g;
+    T.QY[i] = P.Q;
   }
   if (lane == 0) {
     T.d = shape.d;
     T.s = shape.s;
     T.R = shape.R;
-    T.nY = (uint32_t)__popc(member);
-    T.y_min = y_min;
+    T.nY = (uint32_t)__popc(P.member);
+    T.y_min = P.y_min;
     T.fixed_y = shape.fixed_y;
   }
 }
 
-// K2a  per client: survival counts, exponent fit, the threshold bin of the selection and where each bin's candidates start.
-// Everything here depends on the histogram alone.  The number of transmitted coordinates k is not known before the
-// lengths are tuned, but it never exceeds k_sel = R * cap(shortest candidate length) (every packet at the shortest
-// code; with a fixed length, exactly R * cap(y)), so the selection keeps every coordinate down to the bin that holds
-// rank min(k_sel, d): a superset of the top k whose first k ranks are the top k.
-__global__ void __launch_bounds__(kPlanThreads, 1)
-k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __restrict__ nonfinite_all,
-           const Batch batch, const __grid_constant__ Shape shape,
-           unsigned char* ws, int have_rows) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned long long* Nsuf = reinterpret_cast<unsigned long long*>(smem_raw);  // [4096] survival counts
-  double* ptX = reinterpret_cast<double*>(smem_raw + 4096 * 8);                // fit points, ascending bin
-  double* ptY = ptX + 4096;
-  __shared__ PlanShared S;
-  __shared__ PlanTab T;
-  __shared__ uint32_t s_thresh_bin, s_top_bin, s_fullest;
-  int32_t* ws_status = reinterpret_cast<int32_t*>(ws);
-  pdl_enter();
-
-  // blockIdx.x = client
-  const unsigned long long* __restrict__ hist = hist_all + (size_t)blockIdx.x * CVLC_HIST_BINS;
-  const uint32_t nonfinite = nonfinite_all[blockIdx.x];
-  cvlc_plan_t* __restrict__ plan = batch.c[blockIdx.x].plan;
-
+// ---- what a client's histogram gives, by a block of kPlanThreads threads ------------------------
+// Survival counts N_j = #{bin >= j} into N[0 .. 4096] (they add up to d <= 2^31); ends with a barrier.
+__device__ __forceinline__ void survival_counts(const unsigned long long* hist, uint32_t* N) {
+  __shared__ uint32_t s_warp[kPlanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t h[kPlanBins];
+#pragma unroll
+  for (int i = 0; i < kPlanBins; i += 2) {
+    const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(hist) + (kPlanBins * tid + i) / 2);
+    h[i] = (uint32_t)v.x;
+    h[i + 1] = (uint32_t)v.y;
+  }
+  uint32_t sum = 0;
+#pragma unroll
+  for (int i = 0; i < kPlanBins; ++i) sum += h[i];
+  uint32_t incl = sum;  // from the top bin down: of this lane and those above
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t o = __shfl_down_sync(kFull, incl, off);
+    if (lane + off < 32) incl += o;
+  }
+  if (lane == 0) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t run = incl - sum + __reduce_add_sync(kFull, lane > warp && lane < kPlanThreads / 32 ? s_warp[lane] : 0u);
+#pragma unroll
+  for (int i = kPlanBins - 4; i >= 0; i -= 4) {
+    uint4 v;
+    v.w = run + h[i + 3];
+    v.z = v.w + h[i + 2];
+    v.y = v.z + h[i + 1];
+    v.x = v.y + h[i];
+    run = v.x;
+    reinterpret_cast<uint4*>(N)[(kPlanBins * tid + i) / 4] = v;
+  }
+  if (tid == 0) N[CVLC_HIST_BINS] = 0;
+  __syncthreads();
+}
 
+// The selection threshold.  The number of transmitted coordinates k is not known before the lengths are tuned, but it never exceeds
+// k_sel = R * cap(shortest candidate length) (every packet at the shortest code; with a fixed length, exactly R * cap(y)), so the
+// selection keeps every coordinate down to the bin that holds rank min(k_sel, d): a superset of the top k whose first k ranks are
+// the top k.  Written to the plan; where every candidate bin starts among the client's candidates (from the top bin down) to
+// bin_start (may be null).  Ends with a barrier.
+struct Threshold {
+  uint32_t bin, top, n, fullest;  // threshold's bin, highest bin, candidates, those in the fullest bin
+};
+__device__ __forceinline__ Threshold client_threshold(const uint32_t* N, const Shape& shape, uint32_t cap0, cvlc_plan_t* plan, uint32_t* bin_start) {
+  __shared__ Threshold s_t;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) s_t.fullest = 0;
+  const unsigned long long most = (unsigned long long)shape.R * cap0;
+  const uint32_t k_sel = (uint32_t)(most < shape.d ? most : shape.d);
+  __syncthreads();
+  const int first = kPlanBins * (tid & ~31);
+  if (N[first] > 0 && N[first + 32 * kPlanBins] < k_sel) {  // most warps' bins hold no candidates
+    uint32_t fullest = 0;
+#pragma unroll
+    for (int i = 0; i < kPlanBins; ++i) {
+      const int j = first + 32 * i + lane;
+      const uint32_t at = N[j], next = N[j + 1];  // from this bin on, in the bins above it
+      if (at > 0 && next < k_sel) {               // a candidate's bin
+        if (at >= k_sel) {
+          s_t.bin = (uint32_t)j;
+          s_t.n = at;
+        }
+        fullest = max(fullest, at - next);
+        if (next == 0) s_t.top = (uint32_t)j;
+        if (bin_start) bin_start[j] = next;
+      }
+    }
+    fullest = __reduce_max_sync(kFull, fullest);
+    if (lane == 0) atomicMax(&s_t.fullest, fullest);
+  }
+  __syncthreads();
+  const Threshold t = s_t;
+  if (tid == 0) {
+    plan->status = CVLC_OK;
+    plan->s = shape.s;
+    plan->R = shape.R;
+    plan->thresh_bin = t.bin;
+    plan->top_bin = t.top;
+    plan->n_candidates = t.n;
+  }
+  return t;
+}
+
+// The power law of Definition 1 (Algorithm 1, step 1): alpha and its quantised value, known to all threads.  Ends with a barrier.
+constexpr size_t kFitPoints = 4096;  // at most; shared memory: their coordinates and bins
+struct FitScratch {
+  double x[kFitPoints], y[kFitPoints];
+  uint16_t bin[kFitPoints];
+};
+__device__ __forceinline__ double2 client_fit(const uint32_t* N, FitScratch& F, const Shape& shape) {
+  __shared__ uint32_t s_warp[kPlanThreads / 32];
+  __shared__ double2 s_alpha;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (shape.fixed_y) return make_double2(-1.0, -1.0);
+  // ---- fit points: non-empty normal bins in the upper half of the ranks ----------
+  uint32_t flags = 0;
+  uint32_t at = N[kPlanBins * tid];
+#pragma unroll
+  for (int i = 0; i < kPlanBins; ++i) {
+    const int j = kPlanBins * tid + i;
+    const uint32_t next = N[j + 1];
+    if (j >= 16 && j <= 4079 && at > next && at <= shape.d / 2) flags |= 1u << i;
+    at = next;
+  }
+  const uint32_t cnt = __popc(flags);
+  uint32_t incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t o = __shfl_up_sync(kFull, incl, off);
+    if (lane >= off) incl += o;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  const uint32_t wt = lane < kPlanThreads / 32 ? s_warp[lane] : 0u;
+  const uint32_t np = __reduce_add_sync(kFull, wt);
+  uint32_t pos = __reduce_add_sync(kFull, lane < warp ? wt : 0u) + incl - cnt;
+  for (; flags; flags &= flags - 1) F.bin[pos++] = (uint16_t)(kPlanBins * tid + __ffs(flags) - 1);
+  __syncthreads();
+  // the logarithms, spread over the threads: those of a point in two neighbouring warps
+  for (uint32_t q = tid; q < 2 * ((np + 31) & ~31u); q += kPlanThreads) {
+    const uint32_t i = (q >> 6) * 32 + lane;
+    if (i >= np) continue;
+    const int j = F.bin[i];
+    const bool is_x = (q & 32) == 0;
+    const double l = series_log2(is_x ? (double)N[j] : __dadd_rn(1.0, (double)(j & 15) / 16.0));
+    if (is_x) F.x[i] = l;
+    else F.y[i] = __dadd_rn((double)((j >> 4) - 127), l);
+  }
+  __syncthreads();
+  // ---- least squares of log2|U{l}| on log2 l, sums in ascending bin order ----------
+  // four lanes, one sum each: X 1, Y 1, X X, X Y (a product with 1 is exact)
+  if (warp == 0) {
+    double acc = 0.0;
+    const double* A = (lane == 1) ? F.y : F.x;
+    const double* Bp = (lane == 3) ? F.y : F.x;
+    uint32_t i = 0;
+    for (; i + 8 <= np; i += 8) {
+      double t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t[u] = __dmul_rn(A[i + u], lane < 2 ? 1.0 : Bp[i + u]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, t[u]);
+    }
+    for (; i < np; ++i) acc = __dadd_rn(acc, __dmul_rn(A[i], lane < 2 ? 1.0 : Bp[i]));
+    const double n = (double)np;
+    const double Sx = __shfl_sync(kFull, acc, 0), Sy = __shfl_sync(kFull, acc, 1), Sxx = __shfl_sync(kFull, acc, 2), Sxy = __shfl_sync(kFull, acc, 3);
+    const double den = __dsub_rn(__dmul_rn(n, Sxx), __dmul_rn(Sx, Sx));
+    double a;
+    if (n < 2.0 || !(den > 0.0))
+      a = -1.0;
+    else
+      a = __ddiv_rn(__dsub_rn(__dmul_rn(n, Sxy), __dmul_rn(Sx, Sy)), den);
+    double aq = __dmul_rn(floor(__dadd_rn(__dmul_rn(a, 256.0), 0.5)), 1.0 / 256.0);
+    if (aq < -4.0) aq = -4.0;
+    if (aq > -1.0 / 256.0) aq = -1.0 / 256.0;
+    if (aq == -0.5) aq = -0.5 - 1.0 / 256.0;  // beta = 0 would make d^beta - 1 vanish
+    if (lane == 0) s_alpha = make_double2(a, aq);
+  }
+  __syncthreads();
+  return s_alpha;
+}
+
+// the plan's fields that the fit gives, by all threads
+__device__ __forceinline__ void write_fit(cvlc_plan_t* plan, double2 alpha, const PlanLength& P, const Shape& shape) {  // P: warp 0's
+  const int tid = threadIdx.x;
+  if (tid == 0) {
+    plan->y_min = P.y_min;
+    plan->n_lengths = (uint32_t)__popc(P.member);
+    plan->alpha = alpha.x;
+    plan->alpha_q = alpha.y;
+    plan->beta = __dadd_rn(__dmul_rn(2.0, alpha.y), 1.0);
+  }
+  if (tid <= CVLC_MAX_CODE_BITS) plan->cap[tid] = shape.cap[tid];
+}
+
+// What the last block of a client's histogram does: the client's threshold, the bins' starts and, for an encoder in the same call, its
+// buckets and its share of the workspace's header.
+__device__ __noinline__ void finish_client(uint32_t c, const Batch& batch, const Shape& shape, unsigned char* ws, const EncFront& enc, uint32_t* N) {
+  const int tid = threadIdx.x;
+  const uint32_t n = batch.n;
+  PlanWsHeader* hdr = reinterpret_cast<PlanWsHeader*>(ws);
+  EncHeader* eh = reinterpret_cast<EncHeader*>(enc.ws);
+  cvlc_plan_t* plan = batch.c[c].plan;
+  const uint32_t cap0 = batch.c[c].cap0;
+  const uint32_t nonfinite = __ldcg(reinterpret_cast<const uint32_t*>(ws + plan_off_flags(n)) + c);
+  survival_counts(reinterpret_cast<const unsigned long long*>(ws + kPlanWsHist) + (size_t)c * CVLC_HIST_BINS, N);
+  const Threshold t = client_threshold(N, shape, cap0, plan, reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS);
+  if (tid == 0) {
+    if (nonfinite) {
+      plan->status = CVLC_ERR_NONFINITE_INPUT;
+      set_status(&hdr->status, CVLC_ERR_NONFINITE_INPUT);
+    }
+    reinterpret_cast<uint32_t*>(ws + plan_off_max_bin(n))[c] = t.fullest;
+    if (c == 0) {
+      hdr->n = n;
+      hdr->d = shape.d;
+      hdr->magic = kPlanWsMagic;
+    }
+    if (enc.ws) {
+      if (nonfinite) set_status(&eh->status, CVLC_ERR_NONFINITE_INPUT);
+      else if (t.n > enc.capacity) set_status(&eh->status, CVLC_ERR_WORKSPACE_TOO_SMALL);
+      const uint32_t limit = rank_limit(shape);
+      const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.capacity);
+      reinterpret_cast<ClientRank*>(enc.ws + enc.off_rank)[c] = r;
+      reinterpret_cast<uint32_t*>(enc.ws + enc.off_pass_mask)[c] = (1u << kSortPasses) - 1u;  // ranked by partition: the result is in the first buffer
+      add_client(eh, r, limit, enc.capacity);
+      if (c == 0) eh->limit = limit;
+    }
+  }
+}
+
+// ===================================================================================
+// K1  magnitude histogram: h[key >> 19], key = bits(|x|); HBM-bound, 4 bytes / coordinate
+// ===================================================================================
+
+constexpr int kHistThreads = kStreamThreads;
+constexpr int kHistSub = 2;  // shared sub-histograms per block (32 KB)
+
+// The clients' rows form one concatenated array that is cut into equal contiguous chunks, one or two
+// per block, so the load is even whatever the number of clients; a block that crosses a client
+// boundary merges its shared histogram into that client's global one and starts afresh.
+
+// In small batches, whose blocks have one client each, the block that completes a client's histogram works out its threshold and
+// the bins' starts.  As kernels of their own, one block per client behind the exponent fit and one behind that for the encoder's
+// workspace, they stood between histogram and selection for 16 us; here it is 4 (20 clients of 1.2 M coordinates, whole call and
+// aggregation: 161 -> 150 us; 24 of 3 M 498 -> 487).  In large batches a block would have to finish up to four clients one after the
+// other at the end (100 clients of 11.2 M: 23 us): there a kernel of one block per client does it (k_plan_threshold).
+static_assert(kHistThreads == kPlanThreads && kSurvivalBytes <= kHistSub * CVLC_HIST_BINS * 4, "finish_client runs in the histogram's blocks");
+
+// An addition in front of which the block's writes before the last barrier are visible, and behind which those are that others
+// published in this way
+__device__ __forceinline__ uint32_t add_acq_rel(uint32_t* p, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
+
+// counts the four magnitude keys of a float4; returns the largest of them
+__device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
+  const uint32_t k0 = __float_as_uint(a.x) & 0x7FFFFFFFu, k1 = __float_as_uint(a.y) & 0x7FFFFFFFu;
+  const uint32_t k2 = __float_as_uint(a.z) & 0x7FFFFFFFu, k3 = __float_as_uint(a.w) & 0x7FFFFFFFu;
+  atomicAdd(my + (k0 >> 19), 1u);
+  atomicAdd(my + (k1 >> 19), 1u);
+  atomicAdd(my + (k2 >> 19), 1u);
+  atomicAdd(my + (k3 >> 19), 1u);
+  const uint32_t m01 = k0 > k1 ? k0 : k1, m23 = k2 > k3 ? k2 : k3;
+  return m01 > m23 ? m01 : m23;
+}
+
+__global__ void __launch_bounds__(kHistThreads, 3)
+k_hist(const Batch batch, const __grid_constant__ Shape shape, const __grid_constant__ Partition part, unsigned char* ws,
+       const __grid_constant__ EncFront enc, int finish) {
+  extern __shared__ __align__(16) uint32_t sh_hist[];  // [kHistSub][4096]
+  const uint64_t d = shape.d;
+  unsigned long long* hist_all = reinterpret_cast<unsigned long long*>(ws + kPlanWsHist);
+  uint32_t* nonfinite_all = reinterpret_cast<uint32_t*>(ws + plan_off_flags(batch.n));
+  uint16_t* row_max_all = reinterpret_cast<uint16_t*>(ws + plan_off_row_max(batch.n));
+  pdl_enter();
+  for (int i = threadIdx.x; i < kHistSub * CVLC_HIST_BINS; i += kHistThreads) sh_hist[i] = 0;
+  __syncthreads();
+  uint32_t* my = sh_hist + ((threadIdx.x >> 5) & (kHistSub - 1)) * CVLC_HIST_BINS;
+  const int lane = threadIdx.x & 31;
+
+  const uint64_t nvec = d >> 2;
+  for (uint32_t q = blockIdx.x; q < part.n_chunks; q += gridDim.x) {
+  uint64_t pos, end;
+  if (part.per_client) {
+    const uint32_t c = q / part.per_client;
+    pos = c * part.rows + (uint64_t)(q - c * part.per_client) * part.chunk;
+    end = (c + 1) * part.rows;
+  } else {
+    pos = (uint64_t)q * part.chunk;
+    end = part.total;
+  }
+  if (pos + part.chunk < end) end = pos + part.chunk;
+
+  while (pos < end) {
+    const uint64_t c = pos / part.rows;
+    const uint64_t seg_end = ((c + 1) * part.rows < end) ? (c + 1) * part.rows : end;
+    const uint64_t u0 = (pos - c * part.rows) * kRowUnits, u1 = (seg_end - c * part.rows) * kRowUnits;  // units of the client
+    const float* __restrict__ x = batch.c[c].x;
+    const float4* xv = reinterpret_cast<const float4*>(x);
+    const uint64_t v1 = (u1 < nvec) ? u1 : nvec;  // float4 units of this segment: [u0, v1)
+    uint16_t* __restrict__ row_max = row_max_all + c * part.rows;
+    static_assert(kRowUnits == 4, "a row is held by four neighbouring lanes");
+    uint32_t top = 0;
+    uint64_t v = u0 + threadIdx.x;
+    // four independent 128-bit loads in flight per thread; the loop condition is the same for the lanes of a warp
+    for (; (v - lane) + 31 + 3 * kHistThreads < v1; v += 4 * kHistThreads) {
+      float4 a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = __ldg(xv + v + u * kHistThreads);
+      uint32_t m[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        m[u] = hist_add4(my, a[u]);
+        top = m[u] > top ? m[u] : top;
+      }
+      // The rows' maxima of the four loads, two bins to a word: the first exchange leaves an even lane with loads 0 and 1, an odd
+      // lane with 2 and 3, the second completes the rows; each lane then stores one of its row's four.
+      const uint32_t w01 = m[0] >> 19 | (m[1] >> 3 & 0xFFFF0000u), w23 = m[2] >> 19 | (m[3] >> 3 & 0xFFFF0000u);
+      uint32_t w = __vmaxu2(lane & 1 ? w23 : w01, __shfl_xor_sync(0xFFFFFFFFu, lane & 1 ? w01 : w23, 1));
+      w = __vmaxu2(w, __shfl_xor_sync(0xFFFFFFFFu, w, 2));
+      const uint32_t load = ((lane & 1) << 1) | (lane >> 1 & 1);
+      row_max[(v + load * kHistThreads) / kRowUnits] = (uint16_t)(lane & 2 ? w >> 16 : w);
+    }
+    for (; v - lane < v1; v += kHistThreads) {  // rows that may end inside the warp
+      const bool on = v < v1;
+      uint32_t m = on ? hist_add4(my, __ldg(xv + v)) : 0u;
+      top = m > top ? m : top;
+      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+      m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+      if (lane % kRowUnits == 0 && on) row_max[v / kRowUnits] = (uint16_t)(m >> 19);
+    }
+    // ragged tail of the client (d not a multiple of 4)
+    if (seg_end == (c + 1) * part.rows && threadIdx.x < (d & 3)) {
+      const uint32_t k0 = __float_as_uint(x[(nvec << 2) + threadIdx.x]) & 0x7FFFFFFFu;
+      top = k0 > top ? k0 : top;
+      atomicAdd(my + (k0 >> 19), 1u);
+    }
+    if (top >= 0x7F800000u) atomicOr(nonfinite_all + c, 1u);  // a key of exponent 255: Inf or NaN
+    __syncthreads();
+    unsigned long long* __restrict__ hist = hist_all + (size_t)c * CVLC_HIST_BINS;
+    for (int b = threadIdx.x; b < CVLC_HIST_BINS; b += kHistThreads) {
+      uint32_t cnt = 0;
+#pragma unroll
+      for (int sub = 0; sub < kHistSub; ++sub) {
+        cnt += sh_hist[sub * CVLC_HIST_BINS + b];
+        sh_hist[sub * CVLC_HIST_BINS + b] = 0;
+      }
+      if (cnt) atomicAdd(hist + b, (unsigned long long)cnt);
+    }
+    __syncthreads();
+    pos = seg_end;
+  }
+  }
+  if (finish && part.per_client) {
+    __shared__ bool s_complete;
+    const uint32_t c = blockIdx.x / part.per_client, begin = (blockIdx.x - c * part.per_client) * (uint32_t)part.chunk;
+    const uint32_t left = (uint32_t)part.rows - begin, rows = left < (uint32_t)part.chunk ? left : (uint32_t)part.chunk;
+    uint32_t* rows_done = reinterpret_cast<uint32_t*>(ws + plan_off_rows_done(batch.n));
+    if (threadIdx.x == 0) s_complete = add_acq_rel(rows_done + c, rows) + rows == (uint32_t)part.rows;
+    __syncthreads();
+    if (s_complete) finish_client(c, batch, shape, ws, enc, sh_hist);
+  }
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_threshold(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws, const __grid_constant__ EncFront enc) {
+  __shared__ __align__(16) uint32_t N[kSurvivalBytes / 4];
+  pdl_enter();
+  finish_client(blockIdx.x, batch, shape, ws, enc, N);
+}
+
+// K2a  per client: exponent fit and tuning key, where the tuning is shared by clients of one key; for histograms from outside
+// (threshold = 1) also the threshold bin.
+__global__ void __launch_bounds__(kPlanThreads, 1)
+k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __restrict__ nonfinite_all, const Batch batch,
+           const __grid_constant__ Shape shape, unsigned char* ws, int threshold) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* N = reinterpret_cast<uint32_t*>(smem_raw);
+  pdl_enter();
+  const uint32_t c = blockIdx.x;
+  const uint32_t nonfinite = nonfinite_all[c];
+  cvlc_plan_t* plan = batch.c[c].plan;
+  int32_t* ws_status = reinterpret_cast<int32_t*>(ws);
+  const int tid = threadIdx.x, lane = tid & 31;
   if (nonfinite & 2u) {  // a histogram from outside whose counts do not add up to d (its tuning key stays zero: no tuning)
     if (tid == 0) {
       plan->status = CVLC_ERR_INVALID_ARG;
@@ -328,182 +582,26 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
     }
     return;
   }
-
-  if (warp == 0) build_plan_tab(T, shape, batch.c[blockIdx.x].scale_B, lane);
-  if (tid == 0) s_fullest = 0;
-  __syncthreads();
-
-  // ---- survival counts N_j = #{bin >= j} ------------------------------------------
-  unsigned long long h[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) h[i] = hist[4 * tid + i];
-  {
-    unsigned long long tot = h[0] + h[1] + h[2] + h[3];
-    // inclusive scan from the top bin down: reverse thread order
-    unsigned long long v = tot;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned long long o = __shfl_down_sync(kFull, v, off);
-      if (lane + off < 32) v += o;
-    }
-    if (lane == 0) S.warp_tot[warp] = v;
-    __syncthreads();
-    unsigned long long above = 0;
-    for (int w = warp + 1; w < 32; ++w) above += S.warp_tot[w];
-    const unsigned long long incl = v + above;  // sum over threads >= tid
-    unsigned long long run = incl - tot;        // sum over threads > tid
-#pragma unroll
-    for (int i = 3; i >= 0; --i) {
-      run += h[i];
-      Nsuf[4 * tid + i] = run;
-    }
-  }
-  __syncthreads();
-
-  if (T.fixed_y == 0) {
-    // ---- fit points: non-empty normal bins in the upper half of the ranks ----------
-    uint32_t flags = 0, cnt = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = 4 * tid + i;
-      const unsigned long long N = Nsuf[j];
-      const bool ok = (j >= 16) && (j <= 4079) && (h[i] > 0) && (N >= 1) && (N <= T.d / 2);
-      flags |= (ok ? 1u : 0u) << i;
-      cnt += ok;
-    }
-    uint32_t v = cnt;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t o = __shfl_up_sync(kFull, v, off);
-      if (lane >= off) v += o;
-    }
-    if (lane == 31) S.warp_cnt[warp] = v;
-    __syncthreads();
-    uint32_t below = 0;
-    for (int w = 0; w < warp; ++w) below += S.warp_cnt[w];
-    uint32_t pos = below + v - cnt;
-    if (tid == kPlanThreads - 1) S.n_points = below + v;
-    uint16_t* ptJ = reinterpret_cast<uint16_t*>(ptY + 4096);  // their bins: the logarithms are then spread over the threads
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (flags & (1u << i)) ptJ[pos++] = (uint16_t)(4 * tid + i);
-    __syncthreads();
-    const uint32_t np = S.n_points;
-    for (uint32_t q = tid; q < np; q += kPlanThreads) {
-      const int j = ptJ[q];
-      ptX[q] = series_log2((double)Nsuf[j]);
-      ptY[q] = __dadd_rn((double)((j >> 4) - 127), series_log2(__dadd_rn(1.0, (double)(j & 15) / 16.0)));
-    }
-    __syncthreads();
-    // ---- least squares of log2|U{l}| on log2 l, sums in ascending bin order ----------
-    // four lanes, one sum each: X 1, Y 1, X X, X Y (a product with 1 is exact)
-    if (warp == 0) {
-      double acc = 0.0;
-      const double* A = (lane == 1) ? ptY : ptX;
-      const double* Bp = (lane == 3) ? ptY : ptX;
-      uint32_t i = 0;
-      for (; i + 8 <= np; i += 8) {
-        double t[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = __dmul_rn(A[i + u], lane < 2 ? 1.0 : Bp[i + u]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, t[u]);
-      }
-      for (; i < np; ++i) acc = __dadd_rn(acc, __dmul_rn(A[i], lane < 2 ? 1.0 : Bp[i]));
-      const double n = (double)np;
-      const double Sx = __shfl_sync(kFull, acc, 0), Sy = __shfl_sync(kFull, acc, 1), Sxx = __shfl_sync(kFull, acc, 2), Sxy = __shfl_sync(kFull, acc, 3);
-      const double den = __dsub_rn(__dmul_rn(n, Sxx), __dmul_rn(Sx, Sx));
-      double a;
-      if (n < 2.0 || !(den > 0.0))
-        a = -1.0;
-      else
-        a = __ddiv_rn(__dsub_rn(__dmul_rn(n, Sxy), __dmul_rn(Sx, Sy)), den);
-      double aq = __dmul_rn(floor(__dadd_rn(__dmul_rn(a, 256.0), 0.5)), 1.0 / 256.0);
-      if (aq < -4.0) aq = -4.0;
-      if (aq > -1.0 / 256.0) aq = -1.0 / 256.0;
-      if (aq == -0.5) aq = -0.5 - 1.0 / 256.0;  // beta = 0 would make d^beta - 1 vanish
-      if (lane == 0) {
-        S.alpha = a;
-        S.alpha_q = aq;
-      }
-    }
-  } else if (tid == 0) {
-    S.alpha = -1.0;
-    S.alpha_q = -1.0;
-  }
-  __syncthreads();
-
-  // ---- selection threshold: the bin that holds rank min(k_sel, d) (1-based), how many coordinates sit in it
-  // or above, and the highest non-empty bin
-  unsigned long long k_sel = (unsigned long long)T.R * T.capY[0];
-  if (k_sel > T.d) k_sel = T.d;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int j = 4 * tid + i;
-    const unsigned long long N = Nsuf[j];
-    const unsigned long long Nn = (j == CVLC_HIST_BINS - 1) ? 0ull : Nsuf[j + 1];
-    if (N >= k_sel && Nn < k_sel) {
-      plan->thresh_bin = (uint32_t)j;
-      plan->n_candidates = N;
-      s_thresh_bin = (uint32_t)j;
-    }
-    if (N > 0 && Nn == 0) {
-      plan->top_bin = (uint32_t)j;
-      s_top_bin = (uint32_t)j;
+  const double B = batch.c[c].scale_B;
+  PlanLength P{};
+  if (tid < 32) P = plan_lengths(shape, B, lane);
+  survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
+  const double2 alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape);
+  write_fit(plan, alpha, P, shape);
+  if (threshold) {
+    client_threshold(N, shape, batch.c[c].cap0, plan, nullptr);
+    if (tid == 0 && nonfinite) {
+      plan->status = CVLC_ERR_NONFINITE_INPUT;
+      set_status(ws_status, CVLC_ERR_NONFINITE_INPUT);
     }
   }
   if (tid == 0) {
-    const double aq = S.alpha_q;
-    plan->status = nonfinite ? CVLC_ERR_NONFINITE_INPUT : CVLC_OK;
-    if (nonfinite) set_status(ws_status, CVLC_ERR_NONFINITE_INPUT);
-    plan->s = T.s;
-    plan->R = T.R;
-    plan->y_min = T.y_min;
-    plan->n_lengths = T.nY;
-    plan->k = 0;
-    plan->alpha = S.alpha;
-    plan->alpha_q = aq;
-    plan->beta = __dadd_rn(__dmul_rn(2.0, aq), 1.0);
-    plan->gamma = 0.0;
-    plan->B_next = 0.0;
     // clients with the same quantised exponent and the same scale get the same lengths
-    unsigned long long* key = reinterpret_cast<unsigned long long*>(ws + plan_off_keys(batch.n)) + 2 * (size_t)blockIdx.x;
-    key[0] = (unsigned long long)__double_as_longlong(aq);
-    key[1] = (unsigned long long)__double_as_longlong(batch.c[blockIdx.x].scale_B);
-  }
-  if (tid >= 64 && tid - 64 <= CVLC_MAX_CODE_BITS) {
-    plan->n_y[tid - 64] = 0;
-    plan->cap[tid - 64] = shape.cap[tid - 64];
-  }
-  __syncthreads();
-
-  // where every candidate bin starts among the client's candidates (from the top bin down) and the fullest of them: the
-  // selection's and the ranking's buckets.  A plan made from a histogram alone has no rows; its workspace header stays unmarked.
-  if (have_rows) {
-    uint32_t* bin_start = reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(batch.n)) + (size_t)blockIdx.x * CVLC_HIST_BINS;
-    uint32_t fullest = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = 4 * tid + i;
-      if (j < (int)s_thresh_bin || j > (int)s_top_bin) continue;
-      bin_start[j] = (j == CVLC_HIST_BINS - 1) ? 0u : (uint32_t)Nsuf[j + 1];
-      if ((uint32_t)h[i] > fullest) fullest = (uint32_t)h[i];
-    }
-    fullest = __reduce_max_sync(kFull, fullest);
-    if (lane == 0 && fullest) atomicMax(&s_fullest, fullest);
-    __syncthreads();
-    if (tid == 0) {
-      reinterpret_cast<uint32_t*>(ws + plan_off_max_bin(batch.n))[blockIdx.x] = s_fullest;
-      if (blockIdx.x == 0) {
-        PlanWsHeader* hdr = reinterpret_cast<PlanWsHeader*>(ws);
-        hdr->n = batch.n;
-        hdr->d = shape.d;
-        hdr->magic = kPlanWsMagic;
-      }
-    }
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(ws + plan_off_keys(batch.n)) + 2 * (size_t)c;
+    key[0] = (unsigned long long)__double_as_longlong(alpha.y);
+    key[1] = (unsigned long long)__double_as_longlong(B);
   }
 }
-
 
 // ---- atomic operations decided without the series arithmetic -----------------------------------
 // An atomic operation on the lengths i > j looks for the first split t with F(t + 1) <= F(t), F evaluated in the
@@ -596,10 +694,12 @@ __device__ __noinline__ int fast_sign64(double h, double at, double step, double
   diff *= inv_D;
   return diff > guard ? 1 : (diff < -guard ? -1 : 0);
 }
-// K2b  code-length tuning, one CTA per client; only the first client of every tuning key does the work
+// K2b  exponent fit and code-length tuning, one CTA per client.  Where every client has an SM to itself (hist given) it fits and
+// tunes for itself.  In larger batches, whose blocks take SMs from the selection beside them, the fit has been a kernel before and
+// only the first client of every tuning key does the work.
 __global__ void __launch_bounds__(kTuneThreads, 1)
-k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws) {
-  extern __shared__ unsigned char smem_raw[];
+k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws, const unsigned long long* __restrict__ hist_all) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PlanShared S;
   __shared__ PlanTab T;
   __shared__ FastShared FS;
@@ -611,14 +711,28 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_enter();
 
-  const unsigned long long key0 = keys[2 * (size_t)c], key1 = keys[2 * (size_t)c + 1];
-  if (key1 == 0ull) return;  // no key: the fit refused this client's histogram
-  if (tid == 0) s_leader = c;
-  __syncthreads();
-  for (uint32_t i = tid; i < c; i += kTuneThreads)
-    if (keys[2 * (size_t)i] == key0 && keys[2 * (size_t)i + 1] == key1) atomicMin(&s_leader, i);
-  __syncthreads();
-  if (s_leader != c) return;  // an earlier client of the batch tunes for this key and writes the result to all that share it
+  unsigned long long key0, key1;
+  if (hist_all) {
+    const double B = batch.c[c].scale_B;
+    PlanLength P{};
+    if (warp == 0) P = plan_lengths(shape, B, lane);
+    uint32_t* N = reinterpret_cast<uint32_t*>(smem_raw);
+    survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
+    const double2 alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape);
+    write_fit(batch.c[c].plan, alpha, P, shape);
+    key0 = (unsigned long long)__double_as_longlong(alpha.y);
+    key1 = (unsigned long long)__double_as_longlong(B);
+  } else {
+    key0 = keys[2 * (size_t)c];
+    key1 = keys[2 * (size_t)c + 1];
+    if (key1 == 0ull) return;  // no key: the fit refused this client's histogram
+    if (tid == 0) s_leader = c;
+    __syncthreads();
+    for (uint32_t i = tid; i < c; i += kTuneThreads)
+      if (keys[2 * (size_t)i] == key0 && keys[2 * (size_t)i + 1] == key1) atomicMin(&s_leader, i);
+    __syncthreads();
+    if (s_leader != c) return;  // an earlier client of the batch tunes for this key and writes the result to all that share it
+  }
 
   // side by side: the table of lengths, the powers of the single-length plans (lane = length - 1), the power of d
   const double beta = __dadd_rn(__dmul_rn(2.0, __longlong_as_double((long long)key0)), 1.0);
@@ -1237,8 +1351,8 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     if (o > Qmax) Qmax = o;
   }
   __syncthreads();
-  for (uint32_t i = c + warp; i < batch.n; i += kTuneWarps) {
-    if (keys[2 * (size_t)i] != key0 || keys[2 * (size_t)i + 1] != key1) continue;
+  for (uint32_t i = c + warp; i < (hist_all ? c + 1 : batch.n); i += kTuneWarps) {
+    if (i != c && (keys[2 * (size_t)i] != key0 || keys[2 * (size_t)i + 1] != key1)) continue;
     cvlc_plan_t* __restrict__ dst = batch.c[i].plan;
     dst->n_y[lane] = s_ny[lane];
     if (lane == 0) {
@@ -1254,9 +1368,8 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // launchers
 // ===================================================================================
 
-constexpr size_t kFitSmem = 3 * 4096 * 8 + 4096 * 2;  // survival counts, the fit points and their bins
-
-constexpr size_t kTuneSmem = (sizeof(PlanSolver) + 255) & ~(size_t)255;
+constexpr size_t kFitSmem = kSurvivalBytes + sizeof(FitScratch);
+constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) : kFitSmem;  // one after the other
 
 static cudaError_t plan_attributes() {
   static OncePerDevice once;
@@ -1270,73 +1383,76 @@ static cudaError_t plan_attributes() {
 // the start of a planning call: the descriptors into the workspace, `bytes` from its start and `more` from `at` on zeroed
 // (multiples of 256 bytes)
 template <int CAP>
-static void launch_zero_t(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t off_desc, size_t bytes, size_t at, size_t more, cudaStream_t st) {
+static void launch_zero_t(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t bytes, unsigned char* at, size_t more,
+                          cudaStream_t st) {
   BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
   const size_t want = (bytes + more) / 16 / 256 + 1;
   const unsigned grid = (unsigned)(want < (size_t)(4 * kNumSM) ? want : 4 * kNumSM);
-  launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, false, batch, reinterpret_cast<ClientDesc*>(w + off_desc),
-                reinterpret_cast<uint4*>(w), bytes / 16, reinterpret_cast<uint4*>(w + at), more / 16);
+  launch_kernel(kKZeroWords, k_zero_words<CAP>, grid, 256, 0, st, false, batch, reinterpret_cast<ClientDesc*>(w + plan_off_desc(n)),
+                reinterpret_cast<uint4*>(w), bytes / 16, reinterpret_cast<uint4*>(at), more / 16);
 }
-static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t bytes, size_t at, size_t more, cudaStream_t st) {
-  const size_t off_desc = plan_off_desc(n);
-  if (n <= (uint32_t)kSmallBatch) launch_zero_t<kSmallBatch>(clients, n, w, off_desc, bytes, at, more, st);
-  else if (n <= (uint32_t)kMediumBatch) launch_zero_t<kMediumBatch>(clients, n, w, off_desc, bytes, at, more, st);
-  else launch_zero_t<kLargeBatch>(clients, n, w, off_desc, bytes, at, more, st);
-  return Batch{reinterpret_cast<const ClientDesc*>(w + off_desc), n};
+static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w, size_t bytes, unsigned char* at, size_t more, cudaStream_t st) {
+  if (n <= (uint32_t)kSmallBatch) launch_zero_t<kSmallBatch>(clients, n, w, bytes, at, more, st);
+  else if (n <= (uint32_t)kMediumBatch) launch_zero_t<kMediumBatch>(clients, n, w, bytes, at, more, st);
+  else launch_zero_t<kLargeBatch>(clients, n, w, bytes, at, more, st);
+  return Batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
 }
 
-// histogram of every client, then (unless only the histograms are wanted) fit, threshold and the bins' tables
-static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
+// histogram of every client with (unless only the histograms are wanted) threshold and the bins' tables
+static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc,
                               unsigned long long* hist_out, cudaStream_t st) {
   cudaError_t e = plan_attributes();
   if (e != cudaSuccess) return e;
   unsigned char* w = static_cast<unsigned char*>(ws);
-  unsigned long long* hist = reinterpret_cast<unsigned long long*>(w + kPlanWsHist);
-  uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   const Partition part = make_partition(shape.d, n);
-  uint16_t* row_max = reinterpret_cast<uint16_t*>(w + plan_off_row_max(n));
-  // header, histograms, flags and tuning keys start at zero; the rest is written in full by the kernels that follow
-  const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), 0, 0, st);
+  // header, histograms, flags, counters and tuning keys start at zero (and so does the encoder's workspace up to what its selection
+  // writes in full); the rest is written in full by the kernels that follow
+  const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), enc.ws, enc.ws ? enc.zero_end : 0, st);
   // the resident blocks share the concatenated updates evenly
-  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape.d, part, hist, flags, row_max);
-  if (hist_out) {
-    // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
-    // header stays unmarked, so an encode call cannot take it for one that holds a plan's tables.
-    const cudaError_t e2 = cudaGetLastError();
-    if (e2 != cudaSuccess) return e2;
-    return cudaMemcpyAsync(hist_out, hist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
-  }
-  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 1);
-  return cudaGetLastError();
+  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape, part, w, enc, hist_out ? 0 : 1);
+  if (!hist_out && !part.per_client) launch_kernel(kKPlanThreshold, k_plan_threshold, n, kPlanThreads, 0, st, true, batch, shape, w, enc);
+  e = cudaGetLastError();
+  // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
+  // header stays unmarked, so an encode call cannot take it for one that holds a plan's tables.
+  if (e == cudaSuccess && hist_out) e = cudaMemcpyAsync(hist_out, w + kPlanWsHist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
+  return e;
 }
 
-static cudaError_t plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap) {
+// `alone`: nothing runs beside it, so that every client may have an SM
+static cudaError_t plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone) {
   unsigned char* w = static_cast<unsigned char*>(ws);
   const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
-  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w);
+  const unsigned long long* hist = reinterpret_cast<const unsigned long long*>(w + kPlanWsHist);
+  const bool own = n <= (alone ? (uint32_t)kNumSM : kTuneRoom);
+  if (!own) {
+    launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, overlap, hist, reinterpret_cast<const uint32_t*>(w + plan_off_flags(n)), batch,
+                  shape, w, 0);
+    overlap = true;
+  }
+  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w, own ? hist : nullptr);
   return cudaGetLastError();
 }
 
-cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  return plan_front(clients, n, shape, ws, nullptr, st);
+cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st) {
+  return plan_front(clients, n, shape, ws, enc, nullptr, st);
 }
 
-cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap) {
-  return plan_back(n, shape, ws, st, overlap);
+cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone) {
+  return plan_back(n, shape, ws, st, overlap, alone);
 }
 
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  const cudaError_t e = plan_front(clients, n, shape, ws, nullptr, st);
+  const cudaError_t e = plan_front(clients, n, shape, ws, EncFront{}, nullptr, st);
   if (e != cudaSuccess) return e;
-  return plan_back(n, shape, ws, st, true);
+  return plan_back(n, shape, ws, st, true, true);
 }
 
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st) {
-  return plan_front(clients, n, shape, ws, hist_out, st);
+  return plan_front(clients, n, shape, ws, EncFront{}, hist_out, st);
 }
 
 // Checks histograms that come from outside: flag bit 0 = a value of exponent 255 (Inf, NaN),
@@ -1374,12 +1490,11 @@ cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const S
   uint32_t* flags = reinterpret_cast<uint32_t*>(w + plan_off_flags(n));
   // status word, header and tuning keys start at zero: the header stays unmarked, so an encode call cannot take this
   // workspace for one that holds the rows' maxima
-  const Batch batch = launch_zero(clients, n, w, kPlanWsHist, plan_off_keys(n), plan_off_desc(n) - plan_off_keys(n), st);
+  const Batch batch = launch_zero(clients, n, w, kPlanWsHist, w + plan_off_keys(n), plan_off_desc(n) - plan_off_keys(n), st);
   launch_kernel(kKHistCheck, k_hist_check, n, 256, 0, st, true, hist, shape.d, flags);
-  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 0);
-  const cudaError_t e2 = cudaGetLastError();
-  if (e2 != cudaSuccess) return e2;
-  return plan_back(n, shape, ws, st, true);
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 1);
+  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, true, batch, shape, w, static_cast<const unsigned long long*>(nullptr));
+  return cudaGetLastError();
 }
 
 // ===================================================================================

@@ -35,7 +35,7 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
-  const uint32_t n = batch.n, tickets = hdr->split_tiles * n;
+  const uint32_t n = batch.n, tickets = (hdr->most_split + kRankSplitTile - 1) / kRankSplitTile * n;
   if (tickets == 0) return;
   const int tid = threadIdx.x;
   const ClientRank* rank = reinterpret_cast<const ClientRank*>(ws + L.off_rank);

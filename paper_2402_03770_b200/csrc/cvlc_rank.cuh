@@ -523,8 +523,8 @@ __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout
   a.big_room = (size_t)n * a.capacity / kRankItems + 1;
   a.piece_room = (size_t)n * a.capacity / kBigPiece + a.big_room;
   a.n = n;
-  a.tickets = hdr->rank_tiles * n;
-  a.window = hdr->window;
+  a.window = rank_window(hdr);
+  a.tickets = (hdr->most + a.window - 1) / a.window * n;
   a.limit = hdr->limit;
   return a;
 }
