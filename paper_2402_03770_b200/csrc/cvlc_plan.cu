@@ -81,8 +81,8 @@ __device__ __forceinline__ double energy_E(uint64_t Z, double beta, double D) {
 constexpr int kPlanThreads = 512;  // of the blocks that work on one client's histogram: that of the histogram, the fit's, the tuning's
 constexpr int kPlanBins = CVLC_HIST_BINS / kPlanThreads;
 constexpr size_t kSurvivalBytes = (CVLC_HIST_BINS + 4) * 4;  // survival counts in shared memory
-// The tuning kernel decides most atomic operations with one warp per operation or per trial split (see tune_fast below):
-// 16 warps are as many operations as a sweep over neighbouring lengths usually has, and a 17-way search.
+// The tuning kernel decides most atomic operations with four warps (see FastLane below); all of them fit the exponent and evaluate
+// what is left to the series arithmetic.
 constexpr int kTuneThreads = 512;
 constexpr int kTuneWarps = kTuneThreads / 32;
 constexpr int kPlanItems = 1024;
@@ -120,7 +120,6 @@ struct PlanSolver {
 };
 
 struct PlanShared {
-  double Fv[32];
   uint32_t n[32];
   double D;
 };
@@ -292,12 +291,15 @@ __device__ __forceinline__ Threshold client_threshold(const uint32_t* N, const S
 }
 
 // The power law of Definition 1 (Algorithm 1, step 1): alpha and its quantised value, known to all threads.  Ends with a barrier.
-constexpr size_t kFitPoints = 4096;  // at most; shared memory: their coordinates and bins
+constexpr size_t kFitPoints = 4096;  // at most, filled up with zeros to whole groups
+constexpr uint32_t kFitGroup = 16;
 struct FitScratch {
-  double x[kFitPoints], y[kFitPoints];
+  double sum_of[4][kFitPoints + 2 * kFitGroup];  // X, Y, X X, X Y of the points
   uint16_t bin[kFitPoints];
 };
-__device__ __forceinline__ double2 client_fit(const uint32_t* N, FitScratch& F, const Shape& shape) {
+// `meanwhile` is run by the warps but the first while that adds up.
+template <class Meanwhile>
+__device__ __forceinline__ double2 client_fit(const uint32_t* N, FitScratch& F, const Shape& shape, Meanwhile&& meanwhile) {
   __shared__ uint32_t s_warp[kPlanThreads / 32];
   __shared__ double2 s_alpha;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -333,25 +335,34 @@ __device__ __forceinline__ double2 client_fit(const uint32_t* N, FitScratch& F, 
     const int j = F.bin[i];
     const bool is_x = (q & 32) == 0;
     const double l = series_log2(is_x ? (double)N[j] : __dadd_rn(1.0, (double)(j & 15) / 16.0));
-    if (is_x) F.x[i] = l;
-    else F.y[i] = __dadd_rn((double)((j >> 4) - 127), l);
+    F.sum_of[is_x ? 0 : 1][i] = is_x ? l : __dadd_rn((double)((j >> 4) - 127), l);
   }
   __syncthreads();
-  // ---- least squares of log2|U{l}| on log2 l, sums in ascending bin order ----------
-  // four lanes, one sum each: X 1, Y 1, X X, X Y (a product with 1 is exact)
+  const uint32_t filled = (np + kFitGroup - 1) / kFitGroup * kFitGroup + kFitGroup;  // one group more: read ahead, not added
+  for (uint32_t i = tid; i < filled; i += kPlanThreads) {
+    const double X = i < np ? F.sum_of[0][i] : 0.0, Y = i < np ? F.sum_of[1][i] : 0.0;
+    if (i >= np) F.sum_of[0][i] = F.sum_of[1][i] = 0.0;
+    F.sum_of[2][i] = __dmul_rn(X, X);
+    F.sum_of[3][i] = __dmul_rn(X, Y);
+  }
+  __syncthreads();
+  // ---- least squares of log2|U{l}| on log2 l, sums in ascending bin order: four lanes, one sum each ----------
   if (warp == 0) {
     double acc = 0.0;
-    const double* A = (lane == 1) ? F.y : F.x;
-    const double* Bp = (lane == 3) ? F.y : F.x;
-    uint32_t i = 0;
-    for (; i + 8 <= np; i += 8) {
-      double t[8];
+    const double2* A = reinterpret_cast<const double2*>(F.sum_of[lane & 3]);
+    double2 t[kFitGroup / 2], next[kFitGroup / 2];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) t[u] = __dmul_rn(A[i + u], lane < 2 ? 1.0 : Bp[i + u]);
+    for (uint32_t u = 0; u < kFitGroup / 2; ++u) t[u] = A[u];
+    for (uint32_t i = kFitGroup; i < filled; i += kFitGroup) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, t[u]);
+      for (uint32_t u = 0; u < kFitGroup / 2; ++u) next[u] = A[i / 2 + u];
+#pragma unroll
+      for (uint32_t u = 0; u < kFitGroup / 2; ++u) {
+        acc = __dadd_rn(acc, t[u].x);
+        acc = __dadd_rn(acc, t[u].y);
+        t[u] = next[u];
+      }
     }
-    for (; i < np; ++i) acc = __dadd_rn(acc, __dmul_rn(A[i], lane < 2 ? 1.0 : Bp[i]));
     const double n = (double)np;
     const double Sx = __shfl_sync(kFull, acc, 0), Sy = __shfl_sync(kFull, acc, 1), Sxx = __shfl_sync(kFull, acc, 2), Sxy = __shfl_sync(kFull, acc, 3);
     const double den = __dsub_rn(__dmul_rn(n, Sxx), __dmul_rn(Sx, Sx));
@@ -365,17 +376,19 @@ __device__ __forceinline__ double2 client_fit(const uint32_t* N, FitScratch& F, 
     if (aq > -1.0 / 256.0) aq = -1.0 / 256.0;
     if (aq == -0.5) aq = -0.5 - 1.0 / 256.0;  // beta = 0 would make d^beta - 1 vanish
     if (lane == 0) s_alpha = make_double2(a, aq);
+  } else {
+    meanwhile();
   }
   __syncthreads();
   return s_alpha;
 }
 
 // the plan's fields that the fit gives, by all threads
-__device__ __forceinline__ void write_fit(cvlc_plan_t* plan, double2 alpha, const PlanLength& P, const Shape& shape) {  // P: warp 0's
+__device__ __forceinline__ void write_fit(cvlc_plan_t* plan, double2 alpha, const PlanTab& T, const Shape& shape) {
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    plan->y_min = P.y_min;
-    plan->n_lengths = (uint32_t)__popc(P.member);
+  if (tid == 32) {
+    plan->y_min = T.y_min;
+    plan->n_lengths = T.nY;
     plan->alpha = alpha.x;
     plan->alpha_q = alpha.y;
     plan->beta = __dadd_rn(__dmul_rn(2.0, alpha.y), 1.0);
@@ -583,11 +596,17 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
     return;
   }
   const double B = batch.c[c].scale_B;
-  PlanLength P{};
-  if (tid < 32) P = plan_lengths(shape, B, lane);
+  __shared__ PlanTab T;
   survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
-  const double2 alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape);
-  write_fit(plan, alpha, P, shape);
+  auto beside_fit = [&]() {
+    if (tid >= kPlanThreads - 32) build_plan_tab(T, shape, B, lane);
+  };
+  const double2 alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape, beside_fit);
+  if (shape.fixed_y) {
+    beside_fit();
+    __syncthreads();
+  }
+  write_fit(plan, alpha, T, shape);
   if (threshold) {
     client_threshold(N, shape, batch.c[c].cap0, plan, nullptr);
     if (tid == 0 && nonfinite) {
@@ -615,47 +634,69 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
 // roundings), the weights h_l add up to at most 1, the ordered sum of 32 terms adds 4e-15, twice: below
 // 3e-14 (1 + 1 / |D|); the guard is 7 times that.  Differences around an optimum are 1e-11 and more for the usual
 // budgets; an operation that meets a smaller one is left to the series arithmetic (steep power laws: most are).
-// Measured on one ResNet-18-sized client (15 moves, 22 + 13 rounds of checks, 27 of trial splits): the
-// kernel takes 53 us, 632 us with every difference in the series arithmetic; 11 instead of 45 us on a client of 100,000
-// coordinates.  What is left is instruction latency: about 60 steps of some 200 instructions and a barrier each.
+//
+// What is left is latency, about four cycles for every instruction of a lone warp, so the steps are few and short.  A packet moved
+// from length j to length i > j gives the covers of the lengths between them (and i) cap_i ranks and takes delta = cap_j - cap_i
+// from those up to j.  The latter is little next to their size a = W + 1, so that their part of the difference is four terms of a
+// Taylor series in delta, with coefficients that are prefix sums over the lengths of h / D a^(beta - k), the same for all pairs; the
+// former are worked out as they are.  Both directions of all neighbouring pairs are then one evaluation by one warp (lane = i), and
+// those of all pairs one per row (lane = j, a row per warp).  Where an operation on neighbours moves to follows from the condition
+// that the derivative vanishes, solved for a_i (the other covers hardly change); with the half step between difference and
+// derivative that is at most one packet from the answer.  The move is made, and the evaluation of the sweep's next operations
+// tells whether it was the right one.  Moves between other pairs (none after the neighbours are settled, in all the usual cases) are
+// left to the series arithmetic.
+// Measured, exponent fit and tuning together: one ResNet-18-sized client (12 moves, 23 evaluations of about 1200 cycles, a check of
+// all pairs of 3500) 68 -> 37 us, a client of 100,000 coordinates 25 -> 19, one of 300,000 of ten 30 -> 21, against an operation
+// per warp, 16 of them in step, and moves searched for by trial splits (35 steps of checks of 1400 cycles each, 27 of trials).
 constexpr double kTuneGuard = 0x1p-42;
 // Nearly every sign already shows in fp32, where the terms of a difference are worked out as
 // h / D a^beta ((1 + x)^beta - 1), x = step / a, without cancellation inside a term.  A term is good to 3e-6 of itself
 // (for |beta| <= 1; the argument of a^beta is split so that its rounding stays below 1e-7, see fast_power; the growth
-// factor where its logarithm leaves the series: 2.5e-6), the sum to 5e-7 of its largest term: a sum beyond
-// kTuneRel (1 + |beta|) of the terms' sizes has a certain sign, and the rest is looked at in fp64.
+// factor where its logarithm leaves the series: 2.5e-6), a sum of terms of one sign to 5e-7 more, the series' first term to 2e-6, its
+// remainder is bounded where it is used: a difference beyond kTuneRel (1 + |beta|) of its parts' sizes has a certain sign, and the
+// rest is looked at in fp64.
 constexpr float kTuneRel = 0x1p-17f;
+constexpr int kTuneTries = 8;  // corrections of a guess by one packet
 
-struct FastShared {  // one code and one pair per warp, in two buffers: a single barrier per step
-  int code[2][kTuneWarps];
-  int pair[2][kTuneWarps];
-};
-// every warp keeps a copy of the current counts, one candidate length per lane
+// the state of one warp: one candidate length per lane
 struct FastLane {
-  double h;         // weight of E(W) in F (0 beyond the last length)
-  float hD, u;      // h / D, h / D a^beta
-  uint32_t a;       // W + 1, W = ranks covered down to this lane's length
-  uint32_t n, cap;  // packets and records per packet of this lane's length
+  double h;                 // weight of E(W) in F (0 beyond the last length)
+  float hD, u, af, ra;      // h / D, h / D a^beta, a, 1 / a
+  uint32_t a;               // W + 1, W = ranks covered down to this lane's length
+  uint32_t n, cap;          // packets and records per packet of this lane's length
+  float M1, M2, M3, M4;     // prefix sums over the lengths up to this one of h / D a^(beta - k)
+};
+struct FastShared {
+  int4 result[2];           // of the operations on neighbours: cursor, whether something has moved, sweeps
+  uint4 lane_a[32], lane_b[32];  // a warp's state for the others: n, a, M1, M2; M3, M4
+  int key[kTuneWarps];      // first operation that is not known to stay, per warp
+  int code;
 };
 struct FastConst {
   double beta, inv_D, guard;
   float fbeta, frel, fguard;
+  float b1, b2, b3, b4;     // binomial coefficients of beta
+  float b51;                // size of the fifth against the first
 };
 
 __device__ __forceinline__ float fast_lg2(float v) {
   float r;
-  asm("lg2.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
   return r;
 }
 __device__ __forceinline__ float fast_ex2(float v) {
   float r;
-  asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float fast_rcp(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
   return r;
 }
 // a^beta, beta a multiple of 1/128 below 8 in size: beta times the exponent of a is exact, its whole part goes to the
 // result's exponent, and only a number below 5 is rounded before the exponential
-__device__ __forceinline__ float fast_power(uint32_t a, float beta) {
-  const float af = (float)a;
+__device__ __forceinline__ float fast_power(float af, float beta) {
   const uint32_t bits = __float_as_uint(af) - 0x3F3504F3u;        // mantissa into [sqrt(1/2), sqrt(2))
   const float e = (float)((int)bits >> 23);
   const float m = __uint_as_float((bits & 0x007FFFFFu) + 0x3F3504F3u);
@@ -664,35 +705,34 @@ __device__ __forceinline__ float fast_power(uint32_t a, float beta) {
   const float w = fmaxf(whole, -100.0f);                           // below 2^-100: nothing next to the guard
   return r * __uint_as_float((uint32_t)((int)w + 127) << 23);
 }
-// (b1 / b0)^beta - 1, step = b1 - b0
-__device__ __forceinline__ float fast_growth(uint32_t from, uint32_t to, int step, float beta) {
-  const float b0 = (float)from, b1 = (float)to;
-  const float s = __fdividef((float)step, b0 + b1), q = s * s;     // ln(b1 / b0) = 2 atanh(s)
+// (b1 / b0)^beta - 1, step = b1 - b0, r0 = 1 / b0
+__device__ __forceinline__ float fast_growth(float b0, float b1, float step, float r0, float beta) {
+  const float s = step * fast_rcp(b0 + b1), q = s * s;              // ln(b1 / b0) = 2 atanh(s)
   const float series = 2.0f * s * fmaf(q, fmaf(q, fmaf(q, 1.0f / 7, 1.0f / 5), 1.0f / 3), 1.0f);
-  const float ln = fabsf(s) <= 0.1f ? series : 0.693147181f * fast_lg2(__fdividef(b1, b0));
+  const float ln = fabsf(s) <= 0.1f ? series : 0.693147181f * fast_lg2(b1 * r0);
   const float z = beta * ln;
   const float e = z * fmaf(z, fmaf(z, fmaf(z, fmaf(z, fmaf(z, 1.0f / 720, 1.0f / 120), 1.0f / 24), 1.0f / 6), 0.5f), 1.0f);
   return fabsf(z) < 0.25f ? e : fast_ex2(1.44269504f * z) - 1.0f;
 }
-// the terms' sum and the sum of their sizes, to 2^-21 of the largest term (fixed point relative to it)
-__device__ __forceinline__ void fast_sum(float term, float& sum, float& size) {
-  const uint32_t top = __reduce_max_sync(kFull, __float_as_uint(term) & 0x7F800000u);  // exponent field of the largest term
-  const uint32_t e = top >> 23;
-  const bool in_range = e > 32u && e < 220u;
-  const float up = in_range ? __uint_as_float((127u + 25u + 127u - e) << 23) : 0.0f;   // 2^(25 - exponent)
-  const float down = in_range ? __uint_as_float((e - 25u) << 23) : 0.0f;
-  const int v = __float2int_rn(term * up);                                             // below 2^26: no sum leaves 32 bits
-  sum = (float)__reduce_add_sync(kFull, v) * down;
-  size = (float)__reduce_add_sync(kFull, (uint32_t)(v < 0 ? -v : v)) * down;
-}
 
-// sign of F(t + 1) - F(t) from fp64 powers; 0: too close to tell
-__device__ __noinline__ int fast_sign64(double h, double at, double step, double beta, double inv_D, double guard) {
-  double diff = h * (exp2(beta * log2(at + step)) - exp2(beta * log2(at)));
+// Signs of F(t + 1) - F(t) and F(t) - F(t - 1) from fp64 powers, by a whole warp; 0: too close to tell.  `on` / `back`: whether there
+// is such a split; at = covers plus one at t, step = what they gain for a packet
+__device__ __noinline__ int2 fast_signs64(double h, double at, double step, bool on, bool back, double beta, double inv_D, double guard) {
+  double p[3];
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    const double a = k == 0 ? at : (k == 1 ? at + step : at - step);
+    p[k] = (k == 1 && !on) || (k == 2 && !back) ? 0.0 : exp2(beta * log2(a));
+  }
+  double up = h * (p[1] - p[0]), down = h * (p[0] - p[2]);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) diff += __shfl_xor_sync(kFull, diff, off);
-  diff *= inv_D;
-  return diff > guard ? 1 : (diff < -guard ? -1 : 0);
+  for (int off = 16; off > 0; off >>= 1) {
+    up += __shfl_xor_sync(kFull, up, off);
+    down += __shfl_xor_sync(kFull, down, off);
+  }
+  up *= inv_D;
+  down *= inv_D;
+  return make_int2(up > guard ? 1 : (up < -guard ? -1 : 0), down > guard ? 1 : (down < -guard ? -1 : 0));
 }
 // K2b  exponent fit and code-length tuning, one CTA per client.  Where every client has an SM to itself (hist given) it fits and
 // tunes for itself.  In larger batches, whose blocks take SMs from the selection beside them, the fit has been a kernel before and
@@ -712,14 +752,19 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   pdl_enter();
 
   unsigned long long key0, key1;
+  cvlc_plan_t* const my_plan = batch.c[c].plan;
+  // beside the fit: the table of lengths; the logarithms of the single-length plans' covers (lane = length - 1) and of d
+  auto beside_fit = [&]() {
+    if (warp == kTuneWarps - 1) build_plan_tab(T, shape, batch.c[c].scale_B, lane);
+    if (warp == 1) s_single[lane] = series_log2((double)((uint64_t)shape.R * shape.cap[lane + 1] + 1));
+    if (tid == 64) S.D = series_log2((double)shape.d);
+  };
+  double2 alpha = make_double2(0.0, 0.0);
   if (hist_all) {
     const double B = batch.c[c].scale_B;
-    PlanLength P{};
-    if (warp == 0) P = plan_lengths(shape, B, lane);
     uint32_t* N = reinterpret_cast<uint32_t*>(smem_raw);
     survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
-    const double2 alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape);
-    write_fit(batch.c[c].plan, alpha, P, shape);
+    alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape, beside_fit);
     key0 = (unsigned long long)__double_as_longlong(alpha.y);
     key1 = (unsigned long long)__double_as_longlong(B);
   } else {
@@ -734,11 +779,13 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     if (s_leader != c) return;  // an earlier client of the batch tunes for this key and writes the result to all that share it
   }
 
-  // side by side: the table of lengths, the powers of the single-length plans (lane = length - 1), the power of d
   const double beta = __dadd_rn(__dmul_rn(2.0, __longlong_as_double((long long)key0)), 1.0);
-  if (warp == 0) build_plan_tab(T, shape, batch.c[c].scale_B, lane);
-  if (warp == 1) s_single[lane] = series_powr((double)((uint64_t)shape.R * shape.cap[lane + 1] + 1), beta);
-  if (tid == 64) S.D = __dsub_rn(series_powr((double)shape.d, beta), 1.0);
+  if (!hist_all || shape.fixed_y) {  // a fixed length has no fit to stand beside
+    beside_fit();
+    __syncthreads();
+  }
+  if (warp == 1) s_single[lane] = series_exp2(__dmul_rn(beta, s_single[lane]));
+  if (tid == 64) S.D = __dsub_rn(series_exp2(__dmul_rn(beta, S.D)), 1.0);
   if (warp == 3) S.n[lane] = 0;
   __syncthreads();
   const double D = S.D;
@@ -756,8 +803,8 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   // full evaluation, on a fraction of the lanes.
   PlanSolver& Q = *reinterpret_cast<PlanSolver*>(smem_raw);
 
-  auto refresh_state = [&]() {  // all threads; ends with a barrier
-    if (warp == 0) {
+  auto refresh_warp = [&]() {  // by one warp
+    {
       const uint32_t my_n = (lane < nY) ? S.n[lane] : 0u;
       uint64_t W = (uint64_t)my_n * my_cap;
 #pragma unroll
@@ -789,6 +836,9 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
         Q.Eab[32] = 0.0;
       }
     }
+  };
+  auto refresh_state = [&]() {  // all threads; ends with a barrier
+    if (warp == 0) refresh_warp();
     __syncthreads();
   };
 
@@ -798,24 +848,19 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     refresh_state();
   } else {
     // ---- equal packets: best admissible single-length plan, ties to the longer code ----
-    if (tid < nY) {
-      const uint64_t W = (uint64_t)T.R * T.capY[tid];
+    if (warp == 0) {
+      const uint64_t W = (uint64_t)T.R * my_cap;
       // one term: F = 0 + g * (E - 0), E = (power - 1) / D
-      S.Fv[tid] = (W > T.d) ? -CUDART_INF : __dmul_rn(T.gY[tid], __ddiv_rn(__dsub_rn(s_single[T.Y[tid] - 1], 1.0), D));
-    }
-    __syncthreads();
-    if (tid == 0) {
-      int best = -1;
-      double bestF = -CUDART_INF;
-      for (int i = 0; i < nY; ++i) {
-        const double F = S.Fv[i];
-        if (F == -CUDART_INF) continue;
-        if (best < 0 || F >= bestF) {
-          best = i;
-          bestF = F;
-        }
+      const bool on = lane < nY && W <= T.d;
+      const double F = on ? __dmul_rn(T.gY[lane], __ddiv_rn(__dsub_rn(s_single[T.Y[lane] - 1], 1.0), D)) : -CUDART_INF;
+      double most = F;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const double o = __shfl_xor_sync(kFull, most, off);
+        if (o > most) most = o;
       }
-      S.n[best < 0 ? 0 : best] = T.R;  // the host has checked that a plan is admissible
+      const unsigned best = __ballot_sync(kFull, on && F == most);
+      if (lane == (best ? 31 - __clz(best) : 0)) S.n[lane] = T.R;  // the host has checked that a plan is admissible
     }
     __syncthreads();
 
@@ -849,13 +894,41 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     fc.fbeta = (float)beta;
     fc.frel = kTuneRel * (1.0f + fabsf(fc.fbeta));
     fc.fguard = (float)fc.guard * 1.0001f;
-    FastLane fl;
+    fc.b1 = fc.fbeta;
+    fc.b2 = fc.b1 * (fc.fbeta - 1.0f) * 0.5f;
+    fc.b3 = fc.b2 * (fc.fbeta - 2.0f) * (1.0f / 3);
+    fc.b4 = fc.b3 * (fc.fbeta - 3.0f) * 0.25f;
+    fc.b51 = fabsf((fc.fbeta - 1.0f) * (fc.fbeta - 2.0f) * (fc.fbeta - 3.0f) * (fc.fbeta - 4.0f)) * (1.001f / 120);
+    FastLane fl;  // warp 0's throughout, the others' while all pairs are looked at
     fl.cap = my_cap;
     fl.h = (lane < nY) ? T.gY[lane] - (lane ? T.gY[lane - 1] : 0.0) : 0.0;
     fl.hD = (float)(fl.h * fc.inv_D);
     bool stale = true;  // the bookkeeping of the series arithmetic is behind the counts
-    int buf = 0;
-    auto load_counts = [&]() {  // the counts of S.n into every warp's copy
+    int turns = 0;
+    auto set_cover = [&]() {  // what follows from a
+      fl.af = (float)fl.a;
+      fl.ra = fast_rcp(fl.af);
+      fl.u = fl.hD * fast_power(fl.af, fc.fbeta);
+    };
+    auto set_sums = [&]() {
+      float M1 = fl.u * fl.ra, M2 = M1 * fl.ra, M3 = M2 * fl.ra, M4 = M3 * fl.ra;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const float o1 = __shfl_up_sync(kFull, M1, off), o2 = __shfl_up_sync(kFull, M2, off);
+        const float o3 = __shfl_up_sync(kFull, M3, off), o4 = __shfl_up_sync(kFull, M4, off);
+        if (lane >= off) {
+          M1 += o1;
+          M2 += o2;
+          M3 += o3;
+          M4 += o4;
+        }
+      }
+      fl.M1 = M1;
+      fl.M2 = M2;
+      fl.M3 = M3;
+      fl.M4 = M4;
+    };
+    auto load_counts = [&]() {  // the counts of S.n into the warp's copy
       fl.n = S.n[lane];
       uint32_t W = fl.n * my_cap;  // at most d in all
 #pragma unroll
@@ -864,156 +937,206 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
         if (lane + off < 32) W += o;
       }
       fl.a = W + 1u;
-      fl.u = fl.hD * fast_power(fl.a, fc.fbeta);
+      set_cover();
     };
     // ranks that this lane's cover W gains for every packet moved from length j to length i > j
     auto cover_step = [&](int i, int j) -> int {
       const int ci = (int)__shfl_sync(kFull, fl.cap, i), cj = (int)__shfl_sync(kFull, fl.cap, j);
       return lane > i ? 0 : (lane > j ? ci : ci - cj);
     };
-    // One step of every warp's search: all warps learn all codes.  Returns this lane's (lane < kTuneWarps) code.
-    auto exchange = [&](int code, int pair) -> int {
-      if (lane == 0) {
-        FS.code[buf][warp] = code;
-        FS.pair[buf][warp] = pair;
-      }
-      __syncthreads();
-      const int got = lane < kTuneWarps ? FS.code[buf][lane] : 0;
-      buf ^= 1;
-      return got;
+    // What an operation does by its two differences, rise = sign of F(t + 1) - F(t) and came = sign of F(t) - F(t - 1): 0 stays,
+    // 1 more packets of the longer code, 2 fewer, 3 too close to tell
+    auto op_code = [](int rise, int came) -> int { return (rise < 0 && came > 0) ? 0 : rise > 0 ? 1 : came < 0 ? 2 : 3; };
+    // The same for this lane's pair of ni and nj packets: gu, gd = what the lengths between contribute if a packet is moved to the
+    // longer code and back; S1 .. S4 the sums over those up to j, x = delta / a_j the largest relative step among them, whose fifth
+    // term bounds the series' remainder
+    auto lane_code = [&](float gu, float gd, float delta, float S1, float S2, float S3, float S4, float x, uint32_t ni, uint32_t nj) -> int {
+      const float d2 = delta * delta;
+      const float t1 = fc.b1 * delta * S1, odd = fmaf(fc.b3 * d2 * delta, S3, t1), even = d2 * fmaf(fc.b4 * d2, S4, fc.b2 * S2);
+      const float up = gu + (even - odd), back = gd + (even + odd);
+      const float size = fabsf(t1), left = size * fc.b51 * (x * x) * (x * x);
+      const float away = fast_ex2((fc.fbeta - 5.0f) * fast_lg2(1.0f - x));  // the remainder's growth towards smaller a
+      const float up_err = fmaf(fc.frel, fabsf(gu) + size, fmaf(left, away, fc.fguard));
+      const float back_err = fmaf(fc.frel, fabsf(gd) + size, left + fc.fguard);
+      int rise = (x < 0.5f && fabsf(up) > up_err) ? (up > 0.0f ? 1 : -1) : 0;
+      int came = (x < 0.5f && fabsf(back) > back_err) ? (back > 0.0f ? -1 : 1) : 0;
+      if (nj == 0) rise = -1;
+      if (ni == 0) came = 1;
+      return op_code(rise, came);
     };
-    // Walks the sweep from the cursor (ci, cj) on; ends with ci = 0 behind its last operation, or with the cursor on an
-    // operation that only the series arithmetic can decide.
-    auto fast_sweep = [&](int phase, int& ci, int& cj, int& moved) {
-      while (ci >= 1) {
-        // operations left in every row i = lane: pairs (i, j) that share packets, rows and columns descending
-        const unsigned used = __ballot_sync(kFull, fl.n > 0);
-        const int jmax = (lane == ci) ? cj : lane - 1;
-        const unsigned below = (jmax >= 0) ? used & (kFull >> (31 - jmax)) : 0u;
-        int cnt = 0;
-        if (lane <= ci && jmax >= 0) {
-          if (phase == 0) cnt = (fl.n > 0 || ((used >> jmax) & 1u)) ? 1 : 0;
-          else cnt = (fl.n > 0) ? jmax + 1 : __popc(below);
+    // the same in fp64, by a whole warp
+    auto exact_code = [&](int i, int j) -> int {
+      const uint32_t ni = __shfl_sync(kFull, fl.n, i), nj = __shfl_sync(kFull, fl.n, j);
+      const int step = cover_step(i, j);
+      const int2 sign = fast_signs64(fl.h, (double)fl.a, (double)step, nj != 0, ni != 0, fc.beta, fc.inv_D, fc.guard);
+      return op_code(nj == 0 ? -1 : sign.x, ni == 0 ? 1 : sign.y);
+    };
+    // moves length i's packets from the pair (i, i - 1) of X packets to t
+    auto put_split = [&](int i, uint32_t ni, uint32_t X, uint32_t t) {
+      const int step = cover_step(i, i - 1);
+      if (lane == i) fl.n = t;
+      if (lane == i - 1) fl.n = X - t;
+      fl.a += (t - ni) * (uint32_t)step;
+      set_cover();
+    };
+    // Walks a sweep over neighbours from the pair (ci, ci - 1) on, by one warp; ends with ci = 0 behind its last operation, or with ci
+    // on one that only the series arithmetic can decide.
+    auto fast_sweep = [&](int& ci, int& moved) {
+      int i = 0;                            // the operation whose move is still to be confirmed (0: none)
+      uint32_t old = 0, X = 0, t = 0, lo = 0, hi = 0;
+      int tries = 0;
+      while (true) {
+        set_sums();
+        // lane i: the pair (i, i - 1)
+        int mine;
+        {
+          const float S1 = __shfl_up_sync(kFull, fl.M1, 1), S2 = __shfl_up_sync(kFull, fl.M2, 1), S3 = __shfl_up_sync(kFull, fl.M3, 1), S4 = __shfl_up_sync(kFull, fl.M4, 1);
+          const uint32_t nj = __shfl_up_sync(kFull, fl.n, 1), capj = __shfl_up_sync(kFull, fl.cap, 1);
+          const float raj = __shfl_up_sync(kFull, fl.ra, 1);
+          const float give = (float)fl.cap, delta = (float)capj - give;
+          const float gu = fl.u * fast_growth(fl.af, fl.af + give, give, fl.ra, fc.fbeta);
+          const float gd = fl.n > 0 ? fl.u * fast_growth(fl.af, (float)(fl.a - fl.cap), -give, fl.ra, fc.fbeta) : 0.0f;
+          mine = lane_code(gu, gd, delta, S1, S2, S3, S4, delta * raj, fl.n, nj);
+          if (lane == 0 || (fl.n | nj) == 0) mine = 0;
         }
-        int first = 0;  // operations in the rows above
-        if (phase == 0) {
-          first = __popc(__ballot_sync(kFull, cnt != 0) & ~(kFull >> (31 - lane)));
-        } else {
-          first = cnt;
-#pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_down_sync(kFull, first, off);
-            if (lane + off < 32) first += o;
-          }
-          first -= cnt;
-        }
-        const int total = __shfl_sync(kFull, first + cnt, 0);
-        int code = 0, i = 0, j = 0;
-        for (int base = 0; base < total && code == 0; base += kTuneWarps) {
-          // ---- one operation per warp: does the current split stay?
-          const int q = base + warp;
-          int mine = 0;
-          if (q < total) {
-            i = __ffs(__ballot_sync(kFull, q >= first && q < first + cnt)) - 1;
-            const int o = q - __shfl_sync(kFull, first, i);
-            const int top = __shfl_sync(kFull, jmax, i);
-            const uint32_t ni = __shfl_sync(kFull, fl.n, i);
-            if (phase == 0 || ni > 0) {
-              j = top - o;
-            } else {  // the o-th used length below, from the longest on
-              const unsigned m = __shfl_sync(kFull, below, i);
-              j = __ffs(__ballot_sync(kFull, ((m >> lane) & 1u) && __popc(m & ~(kFull >> (31 - lane))) == o)) - 1;
+        if (i) {  // was the move the right one?
+          int code = __shfl_sync(kFull, mine, i);
+          if (code == 3) code = exact_code(i, i - 1);
+          const uint32_t next = code == 1 ? t + 1 : t - 1;
+          if (code) {
+            if (code == 3 || ++tries > kTuneTries || next - lo > hi - lo) {  // back to where it was
+              put_split(i, t, X, old);
+              ci = i;
+              return;
             }
-            const uint32_t nj = __shfl_sync(kFull, fl.n, j);
-            const int step = cover_step(i, j);
-            // forward from the current split, and forward to it from one packet less (a side without packets: no trial)
-            const uint32_t ahead = nj > 0 ? fl.a + (uint32_t)step : fl.a, back = ni > 0 ? fl.a - (uint32_t)step : fl.a;
-            float u, d, u_size, d_size;
-            fast_sum(fl.u * fast_growth(fl.a, ahead, nj > 0 ? step : 0, fc.fbeta), u, u_size);
-            fast_sum(-fl.u * fast_growth(fl.a, back, ni > 0 ? -step : 0, fc.fbeta), d, d_size);
-            int su = fabsf(u) > fc.frel * u_size + fc.fguard ? (u > 0.0f ? 1 : -1) : 0;
-            int sd = fabsf(d) > fc.frel * d_size + fc.fguard ? (d > 0.0f ? 1 : -1) : 0;
-            if (nj == 0) su = -1;
-            if (ni == 0) sd = 1;
-            if (su == 0) su = fast_sign64(fl.h, (double)fl.a, (double)step, fc.beta, fc.inv_D, fc.guard);
-            if (sd == 0) sd = fast_sign64(fl.h, (double)back, (double)step, fc.beta, fc.inv_D, fc.guard);
-            mine = (su < 0 && sd > 0) ? 0 : (su > 0) ? 1 : (sd < 0) ? 2 : 3;
+            put_split(i, t, X, next);
+            t = next;
+            continue;
           }
-          const int parity = buf;
-          const int got = exchange(mine, (i << 8) | j);
-          const unsigned hit = __ballot_sync(kFull, got != 0);
-          if (hit) {  // the first operation of the sweep that moves, or may
-            const int w = __ffs(hit) - 1;
-            code = __shfl_sync(kFull, got, w);
-            i = FS.pair[parity][w] >> 8;
-            j = FS.pair[parity][w] & 0xFF;
-          }
+          moved = 1;
+          ci = i - 1;
+          i = 0;
+        }
+        int code = 0;
+        for (unsigned flagged = __ballot_sync(kFull, mine != 0 && lane <= ci); flagged && code == 0;) {  // in the order of the sweep
+          i = 31 - __clz(flagged);
+          flagged ^= 1u << i;
+          code = __shfl_sync(kFull, mine, i);
+          if (code == 3) code = exact_code(i, i - 1);
         }
         if (code == 0) {
           ci = 0;
           return;
         }
         ci = i;
-        cj = j;
         if (code == 3) return;
-        // ---- where to: one trial split per warp, first at distances 1, 2, 4, ..., then evenly spread over the bracket
-        const uint32_t ni = __shfl_sync(kFull, fl.n, i), nj = __shfl_sync(kFull, fl.n, j);
-        const int step = cover_step(i, j);
-        uint32_t lo = (code == 1) ? ni + 1 : 0u, hi = (code == 1) ? ni + nj : ni - 1;  // the answer lies in [lo, hi]
-        bool spread = false;
-        while (lo < hi) {
-          const uint32_t span = hi - lo;
-          uint32_t t = hi;  // hi: no trial
-          if (!spread && span > (uint32_t)kTuneWarps) {
-            const uint32_t away = 1u << warp;
-            if (away <= span) t = (code == 1) ? lo + away - 1 : hi - away;
-          } else if (span <= (uint32_t)kTuneWarps) {
-            if ((uint32_t)warp < span) t = lo + warp;
-          } else {
-            t = lo + (uint32_t)(((uint64_t)span * (warp + 1)) / (kTuneWarps + 1));
+        old = __shfl_sync(kFull, fl.n, i);
+        X = old + __shfl_sync(kFull, fl.n, i - 1);
+        lo = (code == 1) ? old + 1 : 0u;  // the answer lies in [lo, hi]
+        hi = (code == 1) ? X : old - 1;
+        {
+          const float give = (float)__shfl_sync(kFull, fl.cap, i), delta = (float)__shfl_sync(kFull, fl.cap, i - 1) - give;
+          const float S1 = __shfl_sync(kFull, fl.M1, i - 1), S2 = __shfl_sync(kFull, fl.M2, i - 1), ai = __shfl_sync(kFull, fl.af, i);
+          const float inv_give = fast_rcp(give), per = fast_rcp(fc.fbeta - 1.0f);
+          const float base = fast_lg2(delta * S1 * fast_rcp(__shfl_sync(kFull, fl.hD, i) * give));
+          const float drift = (1.0f - fc.fbeta) * delta * S2 * fast_rcp(S1);
+          float by = 0.0f;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {  // delta S1(t) = h_i / D cap_i a_i(t)^(beta - 1)
+            const float a_new = fast_ex2(per * (base + fast_lg2(fmaxf(fmaf(drift, by, 1.0f), 1e-3f))));
+            by = fminf(fmaxf((a_new - ai) * inv_give, -(float)old), (float)(X - old));
           }
-          int mine = -1;
-          if (t < hi) {
-            const uint32_t at = fl.a + (t - ni) * (uint32_t)step;
-            float sum, size;
-            fast_sum(fl.hD * fast_power(at, fc.fbeta) * fast_growth(at, at + (uint32_t)step, step, fc.fbeta), sum, size);
-            mine = fabsf(sum) > fc.frel * size + fc.fguard ? (sum > 0.0f ? 1 : -1) : 0;
-            if (mine == 0) mine = fast_sign64(fl.h, (double)at, (double)step, fc.beta, fc.inv_D, fc.guard);
-          }
-          const int parity = buf;
-          const int got = exchange(mine, (int)t);
-          const int got_t = lane < kTuneWarps ? FS.pair[parity][lane] : (int)hi;
-          if (__any_sync(kFull, lane < kTuneWarps && got == 0)) return;  // too close to tell
-          // F still rises at the trials below the answer and no longer at those from it on
-          const uint32_t rises = __reduce_max_sync(kFull, (lane < kTuneWarps && got > 0) ? (uint32_t)got_t + 1 : lo);
-          const uint32_t falls = __reduce_min_sync(kFull, (lane < kTuneWarps && got < 0) ? (uint32_t)got_t : hi);
-          lo = rises;
-          hi = falls < hi ? falls : hi;
-          spread = true;
+          t = (uint32_t)fminf(fmaxf(ceilf((float)old + by - 0.5f), (float)lo), (float)hi);
+          t = t < lo ? lo : (t > hi ? hi : t);
         }
-        if (lane == i) fl.n = lo;
-        if (lane == j) fl.n = ni + nj - lo;
-        fl.a += (lo - ni) * (uint32_t)step;
-        fl.u = fl.hD * fast_power(fl.a, fc.fbeta);
-        stale = true;
-        moved = 1;
-        next_pair(phase, ci, cj);
+        tries = 0;
+        put_split(i, old, X, t);
       }
     };
-    if (fast) load_counts();
-    for (int round = 0; round < 64; ++round) {
-      int movedB = 0;
-      for (int phase = 0; phase < 2; ++phase) {  // 0: neighbouring lengths until quiet; 1: every pair once
-        const int max_sweeps = (phase == 0) ? 256 : 1;
-        for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-          int moved = 0;
-          int ci = nY - 1, cj = nY - 2;  // cursor of the sweep
-          while (ci >= 1) {
-            if (fast) {
-              fast_sweep(phase, ci, cj, moved);
-              if (ci < 1) break;
-              if (stale && warp == 0) S.n[lane] = fl.n;
+    // the neighbours' sweeps until one of them is quiet (ci = 0), or up to an operation for the series arithmetic; by warp 0
+    auto fast_neighbours = [&](int& ci, int& moved, int& sweep) {
+      while (true) {
+        fast_sweep(ci, moved);
+        if (ci >= 1) break;
+        if (!moved || ++sweep == 256) break;
+        moved = 0;
+        ci = nY - 1;
+      }
+      S.n[lane] = fl.n;
+    };
+    // All pairs from the cursor on, by all warps: leaves the cursor on the first operation that moves or that fp64 cannot tell, or
+    // ci = 0.  Warp 0's state is the current one; the last warp meanwhile brings the series' bookkeeping up to date.
+    auto fast_all_pairs = [&](int& ci, int& cj) {
+      if (warp == 0) {
+        set_sums();
+        FS.lane_a[lane] = make_uint4(fl.n, fl.a, __float_as_uint(fl.M1), __float_as_uint(fl.M2));
+        FS.lane_b[lane] = make_uint4(__float_as_uint(fl.M3), __float_as_uint(fl.M4), __float_as_uint(fl.u), 0u);
+      }
+      __syncthreads();
+      if (warp != 0) {
+        const uint4 v = FS.lane_a[lane], w = FS.lane_b[lane];
+        fl.n = v.x;
+        fl.a = v.y;
+        fl.M1 = __uint_as_float(v.z);
+        fl.M2 = __uint_as_float(v.w);
+        fl.M3 = __uint_as_float(w.x);
+        fl.M4 = __uint_as_float(w.y);
+        fl.u = __uint_as_float(w.z);
+        fl.af = (float)fl.a;
+        fl.ra = fast_rcp(fl.af);
+      }
+      const unsigned used = __ballot_sync(kFull, fl.n > 0);
+      while (ci >= 1) {
+        int key = 0;
+        if (warp == kTuneWarps - 1) {
+          if (stale) refresh_warp();
+        } else {
+          for (int row = ci - warp; row >= 1 && key == 0; row -= kTuneWarps - 1) {  // a row i per warp, lane j: the pairs (i, j)
+            const uint32_t ni = __shfl_sync(kFull, fl.n, row);
+            if (ni == 0 && (used & ((1u << row) - 1u)) == 0) continue;
+            const uint32_t cap_i = __shfl_sync(kFull, fl.cap, row);
+            const float give = (float)cap_i;
+            float gu = lane <= row ? fl.u * fast_growth(fl.af, fl.af + give, give, fl.ra, fc.fbeta) : 0.0f, gd = 0.0f;
+            if (ni > 0 && lane <= row) gd = fl.u * fast_growth(fl.af, (float)(fl.a - cap_i), -give, fl.ra, fc.fbeta);
+            // summed from the row's length down to the one above this lane's
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+              const float o1 = __shfl_down_sync(kFull, gu, off), o2 = __shfl_down_sync(kFull, gd, off);
+              if (lane + off < 32) {
+                gu += o1;
+                gd += o2;
+              }
             }
+            gu = __shfl_down_sync(kFull, gu, 1);
+            gd = __shfl_down_sync(kFull, gd, 1);
+            const float delta = (float)fl.cap - give;
+            int mine = lane_code(gu, gd, delta, fl.M1, fl.M2, fl.M3, fl.M4, delta * fl.ra, ni, fl.n);
+            if (lane >= row || (row == ci && lane > cj) || (ni | fl.n) == 0) mine = 0;
+            const unsigned flagged = __ballot_sync(kFull, mine != 0);
+            if (flagged) {
+              const int col = 31 - __clz(flagged);
+              key = (row << 16) | (col << 8) | __shfl_sync(kFull, mine, col);
+            }
+          }
+        }
+        if (lane == 0) FS.key[warp] = key;
+        __syncthreads();
+        stale = false;
+        key = __reduce_max_sync(kFull, lane < kTuneWarps ? FS.key[lane] : 0);
+        ci = key >> 16;
+        cj = (key >> 8) & 0xFF;
+        if ((key & 0xFF) != 3) return;
+        if (warp == 0) {
+          const int code = exact_code(ci, cj);
+          if (lane == 0) FS.code = code;
+        }
+        __syncthreads();
+        if (FS.code != 0) return;
+        next_pair(1, ci, cj);
+      }
+    };
+    // One batch of operations from the cursor on in the series arithmetic (see above), by all warps
+    auto series_batch = [&](int phase, int& ci, int& cj, int& moved) {
             if (stale) {
               __syncthreads();
               refresh_state();
@@ -1125,7 +1248,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
               cj = bj;
               if (n_ops == 0) {  // the rest of the sweep had nothing to split
                 __syncthreads();  // the collection's scratch is reset by the next one
-                continue;
+                return;
               }
             }
             __syncthreads();
@@ -1320,40 +1443,71 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
             if (Q.moved) {
               moved = 1;
               refresh_state();
-              if (fast) load_counts();
+              if (fast && warp == 0) load_counts();
             } else {
               __syncthreads();
             }
+    };
+    if (fast && warp == 0) load_counts();
+    for (int round = 0; round < 64; ++round) {
+      // neighbouring lengths until quiet
+      int ci = nY - 1, cj = nY - 2, moved = 0;  // cursor of the sweep
+      for (int sweep = 0; ci >= 1 || sweep == 0;) {
+        if (fast) {
+          if (warp == 0) {
+            fast_neighbours(ci, moved, sweep);
+            if (lane == 0) FS.result[turns & 1] = make_int4(ci, moved, sweep, 0);
           }
-          if (phase == 1) movedB = moved;
-          if (!moved) break;
+          __syncthreads();
+          const int4 r = FS.result[turns++ & 1];
+          ci = r.x;
+          cj = ci - 1;
+          moved = r.y;
+          sweep = r.z;
+          stale = true;
+          if (ci < 1) break;
+        }
+        series_batch(0, ci, cj, moved);
+        if (ci < 1) {
+          if (!moved || ++sweep == 256) break;
+          moved = 0;
+          ci = nY - 1;
+          cj = nY - 2;
         }
       }
-      if (!movedB) break;
+      // every pair once
+      ci = nY - 1;
+      cj = nY - 2;
+      moved = 0;
+      while (ci >= 1) {
+        if (fast) fast_all_pairs(ci, cj);
+        if (ci >= 1) series_batch(1, ci, cj, moved);
+      }
+      if (!moved) break;
     }
     if (stale) {
-      if (fast && warp == 0) S.n[lane] = fl.n;
       __syncthreads();
       refresh_state();
     }
   }
 
   // ---- outputs, to this client and to the later ones that share its tuning key -------------------
+  if (hist_all) write_fit(my_plan, alpha, T, shape);
   if (tid <= CVLC_MAX_CODE_BITS) s_ny[tid] = 0;
   __syncthreads();
   if (tid < nY) s_ny[T.Y[tid]] = S.n[tid];
-  unsigned long long k = (lane < nY) ? (unsigned long long)S.n[lane] * my_cap : 0ull;
-  double Qmax = (lane < nY && S.n[lane] > 0) ? T.QY[lane] : 0.0;
+  const uint32_t my_n = lane < nY ? S.n[lane] : 0u;
+  const unsigned long long k = __reduce_add_sync(kFull, my_n * my_cap);  // at most d
+  double Qmax = my_n > 0 ? T.QY[lane] : 0.0;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    k += __shfl_xor_sync(kFull, k, off);
     const double o = __shfl_xor_sync(kFull, Qmax, off);
     if (o > Qmax) Qmax = o;
   }
   __syncthreads();
   for (uint32_t i = c + warp; i < (hist_all ? c + 1 : batch.n); i += kTuneWarps) {
     if (i != c && (keys[2 * (size_t)i] != key0 || keys[2 * (size_t)i + 1] != key1)) continue;
-    cvlc_plan_t* __restrict__ dst = batch.c[i].plan;
+    cvlc_plan_t* __restrict__ dst = i == c ? my_plan : batch.c[i].plan;
     dst->n_y[lane] = s_ny[lane];
     if (lane == 0) {
       dst->n_y[CVLC_MAX_CODE_BITS] = s_ny[CVLC_MAX_CODE_BITS];
