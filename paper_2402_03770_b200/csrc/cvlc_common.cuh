@@ -200,6 +200,8 @@ struct ClientRank {
   uint32_t split;      // 1: coarse buckets are partitioned into sub-buckets
   uint32_t top_bin;
   uint32_t wide;       // 1: sub-buckets are counted in whole numbers, their counts may be beyond fp32's
+  uint32_t thresh_bin; // lowest bin of the candidates: the plan's or, where k is known, the one that holds rank k
+  uint32_t pad[3];
 };
 // The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates.  As few
 // sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that a block
@@ -578,7 +580,7 @@ CVLC_HD inline uint32_t rank_limit(const Shape& shape) {
   return most_sent < 0xFFFFFFFFull ? (uint32_t)most_sent : 0xFFFFFFFFu;
 }
 
-// a client's buckets from its plan's threshold and the tables beside it
+// a client's buckets from its threshold, the candidates from there on, and what the fullest bin holds
 __device__ __forceinline__ ClientRank client_rank(uint32_t thresh_bin, uint32_t top_bin, unsigned long long n_candidates, uint32_t max_bin,
                                                   unsigned long long capacity) {
   ClientRank r;
@@ -588,6 +590,7 @@ __device__ __forceinline__ ClientRank client_rank(uint32_t thresh_bin, uint32_t 
   r.n = (uint32_t)(n_candidates < capacity ? n_candidates : capacity);
   r.keytop = sort_keytop(top_bin);
   r.top_bin = top;
+  r.thresh_bin = thresh_bin;
   return r;
 }
 

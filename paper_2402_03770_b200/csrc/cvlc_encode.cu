@@ -20,6 +20,29 @@ namespace cvlc {
 // The grid zeroes the per-client counters, digit histograms and look-back states; block 0
 // alone owns the 256-byte header and the sort-tile prefix (nobody else writes them).
 
+// The bin that holds rank k and how many candidates there are from it on.  The plan's threshold was set before the lengths were tuned, for
+// the most that could be sent; where the plan is complete, a tenth of its candidates are known not to be (8 clients of 1.2 M coordinates in
+// the unframed format: 198 -> 192 us).  bin_start falls from bin to bin; eight places of the range are looked at together.
+__device__ __forceinline__ uint2 sent_from(const cvlc_plan_t* plan, const uint32_t* __restrict__ bin_start) {
+  const unsigned long long k = plan->k;
+  const uint32_t thresh = plan->thresh_bin, n = (uint32_t)plan->n_candidates;
+  if (k == 0 || k > n || thresh > plan->top_bin || plan->top_bin >= CVLC_HIST_BINS) return make_uint2(thresh, n);
+  uint32_t lo = thresh, hi = plan->top_bin;  // the first bin with fewer than k candidates above it lies in [lo, hi]: none lies above the top
+  while (lo < hi) {
+    const uint32_t step = (hi - lo + 8) / 9;
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = bin_start[min(lo + i * step, hi)];
+    uint32_t below = 0;  // places with k candidates or more above them
+#pragma unroll
+    for (int i = 0; i < 8; ++i) below += v[i] >= k ? 1u : 0u;
+    const uint32_t new_hi = below < 8 ? min(lo + below * step, hi) : hi;
+    if (below) lo = min(lo + (below - 1) * step, hi) + 1;
+    hi = new_hi;
+  }
+  return make_uint2(lo, lo > thresh ? bin_start[lo - 1] : n);
+}
+
 template <int CAP>
 __global__ void __launch_bounds__(256)
 k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape,
@@ -51,11 +74,12 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
       s_tiles[c] = tiles;
       t += tiles;
       if (plan->top_bin + 1u - plan->thresh_bin > 256u) pass3 = 1;  // see top_digit_is_zero
-      if (max_bin) {
-        const ClientRank r = client_rank(plan->thresh_bin, plan->top_bin, plan->n_candidates, max_bin[c], L.capacity);
+      if (max_bin && blockIdx.x == 0) {
+        const uint2 from = sent_from(plan, reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS);
+        const ClientRank r = client_rank(from.x, plan->top_bin, from.y, max_bin[c], L.capacity);
         atomicMax(&s_most, r.n < limit ? r.n : limit);  // buckets from the limit on are not ranked
         if (r.split) atomicMax(&s_most_split, r.n);
-        if (blockIdx.x == 0) reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;
+        reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;
       }
     }
     if (t) atomicAdd(&s_total, t);
@@ -419,7 +443,7 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     const float* __restrict__ x = batch.c[c].x;
     const float4* __restrict__ xv = reinterpret_cast<const float4*>(x);
     const uint16_t* __restrict__ row_max = reinterpret_cast<const uint16_t*>(plan_ws + plan_off_row_max(n)) + (size_t)c * rows;
-    const uint32_t thresh_bin = batch.c[c].plan->thresh_bin, thresh = thresh_bin << 19, keytop = r.keytop;
+    const uint32_t thresh_bin = r.thresh_bin, thresh = thresh_bin << 19, keytop = r.keytop;
     const float below_thresh = thresh ? __uint_as_float(thresh - 1u) : -1.0f;       // key >= thresh <=> |x| > below_thresh
     const uint32_t sh_coarse = 19 + r.group, sh_sub = sh_coarse - r.sub_bits;
     unsigned long long* __restrict__ out = reinterpret_cast<unsigned long long*>(ws + L.off_buf_a) + (size_t)c * L.capacity;
