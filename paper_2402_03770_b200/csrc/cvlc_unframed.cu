@@ -533,20 +533,26 @@ constexpr int kUfDecThreads = 128;
 constexpr int kUfDecWarps = kUfDecThreads / 32;
 constexpr uint32_t kUfStage = 288;    // words of a block staged at a time
 constexpr uint32_t kUfChunk = 512;    // records whose starts are found before the warp takes them apart
+constexpr uint32_t kUfSteps = 16;     // records that are followed between two looks at what was met
 struct UfDecWarp {
-  alignas(16) uint8_t len[kUfStage * 32];  // length of a record that starts at this bit of the stage
-  uint32_t bits[kUfStage + 4];             // the block's words from the current stage on (four words of zeros behind them)
-  uint16_t start[kUfChunk];                // first bit of every record
+  alignas(16) uint8_t len[kUfStage * 32 + 256];  // length of a record that starts at this bit of the stage; zeros behind it
+  uint32_t bits[kUfStage + 4];                   // the block's words from the current stage on (four words of zeros behind them)
+  uint16_t start[kUfChunk + kUfSteps];           // first bit of every record, and the one behind the last
 };
 
 // One warp per block.  The unary parts make finding the records sequential; to keep the chain short, the lanes first work out how
-// long a record would be from every bit of a staged piece on, and one lane then only adds lengths up.  The warp then takes 32 records at a time apart, sums their differences by a scan, dequantizes and
-// accumulates.  8 clients of 1.2 M coordinates at 2 bits (1600 blocks): 59 us; 105 us with the records taken apart by lane 0 out of
-// shared memory, 188 us out of global memory.
+// long a record would be from every bit of a staged piece on (four bits by one multiplication from a table of their 16 patterns), and
+// one lane then only adds lengths up: a load from shared memory and an addition per record, with a look every 16 records at whether the
+// piece has ended or a unary part was too long for the table (updates with layers that send nothing have some; they are counted out word by
+// word).  The warp then takes 32 records at a time apart, sums their differences by a scan, dequantizes and accumulates.
+// 8 clients of 1.2 M coordinates at 2 bits (1600 blocks of about 400 records): 57 us with the checks in the chain (117 cycles a record) and
+// a new piece behind every long unary part, 24 us here.  (Four warps per block, each following a quarter of the piece from 64 entries at once:
+// 86 us; only a lone client gains by it.)
 __global__ void __launch_bounds__(kUfDecThreads)
 k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64_t d, float* __restrict__ out, unsigned char* ws) {
   extern __shared__ uint32_t s_dec[];  // [n + 1] block prefix
   __shared__ UfDecWarp s_warp[kUfDecWarps];
+  __shared__ uint2 s_nibble[16];  // of four bits: ones from each bit on (a byte each), and whether they go on above the fourth
   __shared__ int s_err;
   pdl_enter();
   int32_t* status = reinterpret_cast<int32_t*>(ws + kDecWsStatus);
@@ -554,10 +560,20 @@ k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64
   const uint32_t* prefix = reinterpret_cast<const uint32_t*>(ws + dec_off_prefix(n));
   if (threadIdx.x == 0) s_err = *reinterpret_cast<const volatile int32_t*>(status);
   for (uint32_t i = threadIdx.x; i <= n; i += kUfDecThreads) s_dec[i] = prefix[i];
+  if (threadIdx.x < 16) {
+    uint2 v = make_uint2(0u, 0u);
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t ones = (uint32_t)__ffs((int)~(threadIdx.x >> e)) - 1u;  // at most 4 - e
+      v.x |= ones << (8 * e);
+      v.y |= (ones == 4u - e ? 1u : 0u) << (8 * e);
+    }
+    s_nibble[threadIdx.x] = v;
+  }
   __syncthreads();
   if (s_err != 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   UfDecWarp& sw = s_warp[warp];
+  for (uint32_t i = lane; i < 64; i += 32) reinterpret_cast<uint32_t*>(sw.len + kUfStage * 32)[i] = 0u;
   const uint32_t total = s_dec[n];
   const uint32_t warps_total = gridDim.x * kUfDecWarps;
   for (uint32_t g = blockIdx.x * kUfDecWarps + warp; g < total; g += warps_total) {
@@ -618,41 +634,64 @@ k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64
       __syncwarp();
       const unsigned long long base = w0 << 5;
       const uint32_t first = (uint32_t)(pos - base);
-      const uint32_t last = (uint32_t)(total_bits - base < kUfStage * 32ull ? total_bits - base : kUfStage * 32ull);
-      uint32_t count = 0, p = first;
+      const uint32_t last = (uint32_t)(next > base ? (next - base < kUfStage * 32ull ? next - base : kUfStage * 32ull) : 0ull);  // the piece's end
       // The length of a record that started at any bit of the stage (128 and more: its unary part leaves the next word), every
-      // lane a word of bits at a time, from the top bit down; then one lane follows the lengths from record to record.
-      for (uint32_t i = lane; i < kUfStage; i += 32) {
+      // lane a word of bits at a time, from the top bits down; then one lane follows the lengths from record to record.
+      for (uint32_t i = lane; 32 * i < last; i += 32) {
         const uint32_t x0 = sw.bits[i], x1 = sw.bits[i + 1];
         uint32_t run = x1 == 0xFFFFFFFFu ? 128u : (uint32_t)__ffs((int)~x1) - 1u;
         uint32_t packed[8];
 #pragma unroll
         for (int q = 7; q >= 0; --q) {
-          uint32_t v = 0;
-#pragma unroll
-          for (int e = 3; e >= 0; --e) {
-            run = ((x0 >> (4 * q + e)) & 1u) ? run + 1u : 0u;
-            v |= (run + tail_bits) << (8 * e);
-          }
-          packed[q] = v;
+          const uint2 v = s_nibble[(x0 >> (4 * q)) & 15u];
+          const uint32_t runs = v.y * run + v.x;
+          run = runs & 0xFFu;
+          packed[q] = runs + tail_bits * 0x01010101u;
         }
         uint4* len4 = reinterpret_cast<uint4*>(sw.len) + 2 * i;
         len4[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
         len4[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
       }
       __syncwarp();
+      const uint32_t want = P - done < kUfChunk ? P - done : kUfChunk;
+      uint32_t found = 0;  // starts written down, and the one behind them
       if (lane == 0) {
-        const uint32_t want = P - done < kUfChunk ? P - done : kUfChunk;
-        for (; count < want; ++count) {
-          const uint32_t len = p < last ? sw.len[p] : 255u;
-          if (len >= 128u || p + len > last) break;  // not whole inside the stage (or the stream)
-          sw.start[count] = (uint16_t)p;
-          p += len;
+        uint32_t p = first;
+        while (found < want && p < last) {
+          const uint32_t from = p;
+          uint32_t seen = 0;
+#pragma unroll
+          for (uint32_t u = 0; u < kUfSteps; ++u) {
+            const uint32_t l = sw.len[p];
+            sw.start[found + u] = (uint16_t)p;
+            seen |= l;
+            p += l;
+          }
+          found += kUfSteps;
+          if (seen < 128u) continue;
+          found -= kUfSteps;  // once more, up to the long one
+          p = from;
+          while (sw.len[p] < 128u) {
+            sw.start[found++] = (uint16_t)p;
+            p += sw.len[p];
+          }
+          if (p >= last) break;
+          uint32_t w = p >> 5, ones = ~sw.bits[w] >> (p & 31u);
+          uint32_t zero = p + (ones ? (uint32_t)__ffs((int)ones) - 1u : 32u - (p & 31u));  // where its unary part ends
+          while (ones == 0 && zero < last) {
+            ones = ~sw.bits[++w];
+            zero += ones ? (uint32_t)__ffs((int)ones) - 1u : 32u;
+          }
+          if (zero + tail_bits > last || found >= want) break;  // not whole in the piece: the next one begins with it
+          sw.start[found++] = (uint16_t)p;
+          p = zero + tail_bits;
         }
+        sw.start[found] = (uint16_t)p;
       }
-      count = __shfl_sync(kFull, count, 0);
-      p = __shfl_sync(kFull, p, 0);
+      found = __shfl_sync(kFull, found, 0);
       __syncwarp();
+      // a record that is whole inside the piece
+      auto whole = [&](uint32_t j) -> bool { return j < found && sw.start[j] < last && sw.start[j + 1] <= last; };
       auto accumulate = [&](uint32_t pid, uint32_t code) {
         float v;
         if (qsgd) {
@@ -663,7 +702,7 @@ k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64
         }
         atomicAdd(out + pid, cf * v);
       };
-      if (count == 0) {
+      if (!whole(0)) {
         // a record longer than a stage (the unary parts of a block add up to less than two bits per record, so only a malformed
         // or extremely sparse block has one): walked in global memory, by all lanes alike
         unsigned long long q = pos, quo = 0;
@@ -684,13 +723,15 @@ k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64
         done += 1;
         continue;
       }
-      for (uint32_t j0 = 0; j0 < count; j0 += 32) {
-        const bool on = j0 + lane < count;
+      uint32_t count = 0;
+      for (uint32_t j0 = 0; j0 < want; j0 += 32) {
+        const unsigned there = __ballot_sync(kFull, j0 + lane < want && whole(j0 + lane));
+        const uint32_t here = there == kFull ? 32u : (uint32_t)__ffs((int)~there) - 1u;  // up to the first that is not
+        const bool on = (uint32_t)lane < here;
         unsigned long long gap = 0;  // this record's distance from the first place behind the one before it, plus one
         uint32_t code = 0;
         if (on) {
-          const uint32_t begin = sw.start[j0 + lane];
-          const uint32_t end = (j0 + lane + 1 < count) ? sw.start[j0 + lane + 1] : p;
+          const uint32_t begin = sw.start[j0 + lane], end = sw.start[j0 + lane + 1];
           const uint32_t q = end - tail_bits + 1;  // behind the unary part and its stop bit
           const uint32_t w = q >> 5, sh = q & 31u;
           const uint32_t x0 = sw.bits[w], x1 = sw.bits[w + 1], x2 = sw.bits[w + 2];
@@ -709,9 +750,11 @@ k_decode_unframed(const uint8_t* const* __restrict__ streams, uint32_t n, uint64
         if (bad) break;
         if (on) accumulate((uint32_t)pid, code);
         prev += __shfl_sync(kFull, incl, 31);
+        count += here;
+        if (here < 32) break;
       }
       if (bad) break;
-      pos = base + p;
+      pos = base + sw.start[count];
       done += count;
     }
     if ((bad || pos != next) && lane == 0) set_status(status, CVLC_ERR_BAD_STREAM);

@@ -163,3 +163,43 @@ def test_unframed_refusals(env):
     from gpu_util import gpu_decode_aggregate
     status, _ = gpu_decode_aggregate([u], w, 20_000)                                     # the framed decoder refuses it
     assert status == B.CVLC_ERR_BAD_STREAM
+
+
+@pytest.mark.parametrize("quantizer", [0, 1])
+@pytest.mark.parametrize("d,pb,R,shape", [(4_000_000, 12000, 3, "ends"), (4_000_000, 12000, 3, "steps"), (1_000_000, 2048, 4, "ends"), (300_000, 36000, 2, "steps"),
+                                          (70_000, 36000, 2, "dense"), (40, 256, 1, "dense")])
+def test_unframed_decoder_meets_long_and_short_unary_parts(env, d, pb, R, shape, quantizer):
+    """unary parts of no bits, around a word's and a table entry's length and of hundreds of bits (positions in two heaps, or at steps
+    of growing width), blocks of more and of less than a staged piece"""
+    torch, B = env
+    rng = np.random.default_rng(d + pb)
+    x = (rng.laplace(0, 1e-6, d)).astype(np.float32)
+    m = min(d // 2, 3 * R * pb // 24)
+    if shape == "ends":
+        at = np.r_[0:m // 2, d - (m - m // 2):d]
+    elif shape == "steps":
+        at = np.unique(np.minimum(np.cumsum(np.r_[np.ones(m - 64, dtype=np.int64), np.geomspace(2, d // 8, 64).astype(np.int64)]), d - 1))
+    else:
+        at = np.arange(d)
+    x[at] += (rng.choice([-1.0, 1.0], at.size) * rng.uniform(1.0, 2.0, at.size)).astype(np.float32)
+    pd = params_dict(d, R * pb, packet_bits=pb, seed=5, quantizer=quantizer)
+    po = oracle_params(pd)
+    ref = O.encode_unframed(x, po, O.plan(x, po))
+    status, got, _, _ = gpu_unframed(torch, B, [x], [pd])
+    assert status == 0 and np.array_equal(got[0], ref)
+    w = np.ones(1, dtype=np.float32)
+    status, out = gpu_decode_unframed(torch, B, [ref], w, d)
+    assert status == 0
+    assert_aggregate_close(out, O.decode_aggregate_unframed([ref], w, d))
+    # a bit of the body the other way round: a length or a position is wrong, mostly to be seen from the directory
+    for bit in rng.integers(8 * (336 + 8 * R) + 64, 8 * ref.size - 64, 12):
+        bent = ref.copy()
+        bent[bit // 8] ^= np.uint8(1 << (bit % 8))
+        status, out = gpu_decode_unframed(torch, B, [bent], w, d)
+        try:
+            want = O.decode_aggregate_unframed([bent], w, d)
+        except Exception:
+            assert status == B.CVLC_ERR_BAD_STREAM
+        else:
+            assert status == 0
+            assert_aggregate_close(out, want)
