@@ -229,6 +229,7 @@ CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
 // the batch; a small batch is spread over all warps.
 constexpr int kSelThreads = 608;
 constexpr uint32_t kSelPiece = 128;  // rows whose maxima a warp loads at once (64 bits per lane)
+constexpr uint32_t kSelRun = 16;     // neighbouring rows of a small group: their maxima are a sector of 32 bytes
 struct SelectGroups {
   uint32_t pieces[2], count[2];  // large and middle groups: pieces in one, how many
   uint32_t small, groups;        // rows of a small group; all groups

@@ -397,6 +397,12 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   const uint32_t rows = (uint32_t)part.rows, held_rows = ((uint32_t)(d >> 2) + kRowUnits - 1) / kRowUnits;  // with coordinates
   const SelectGroups sg = select_groups(part, n);
   const uint32_t groups = sg.groups;
+  // A group's rows are spread over all that the groups of its size share, in runs of kSelRun (small groups) or pieces (larger ones), so
+  // that all of them meet a layer that holds most of a client's candidates, where neighbouring rows made a group dense or empty: 24
+  // clients of 3 M coordinates, blocks done after 69 to 119 us -> 69 to 95, whole calls 477 -> 449 us (4 bits), 321 -> 310 (QSGD, 2
+  // bits); one of 11.2 M 94 -> 90; 100 of 11.2 M 3080 -> 3040.  (Runs in the larger groups too: 3054, and 50 of 23.5 M 2440 -> 2460.)
+  const uint32_t small_row = (sg.count[0] * sg.pieces[0] + sg.count[1] * sg.pieces[1]) * kSelPiece, runs = (rows - small_row) / kSelRun;
+  const uint32_t small_groups = groups - sg.count[0] - sg.count[1], last_group = (runs - 1) % small_groups;
   const uint32_t nvec = (uint32_t)(d >> 2);
   uint32_t* group_next = reinterpret_cast<uint32_t*>(ws + L.off_group_next);
   uint32_t* group_done = reinterpret_cast<uint32_t*>(ws + L.off_group_done);
@@ -517,25 +523,28 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     }
     if (lane == 0 && rounds == 0) group2 = dynamic + atomicAdd(group_next + c, 1u);
     struct Piece {
-      uint32_t row, end;  // [row, end): none left where row = end
-      uint2 maxima;       // lane l: rows row + 4 l .. row + 4 l + 3
+      uint32_t row;  // lane: its four rows begin here; beyond the client's rows: none
+      bool any, last;  // a piece at all; the one that holds the client's last rows
+      uint2 maxima;  // of the lane's rows
     };
     auto next_piece = [&]() -> Piece {
-      Piece p{0u, 0u, make_uint2(0u, 0u)};
-      if (group >= groups) return p;
-      uint32_t pieces = 1;
-      if (group < sg.count[0]) {
+      Piece p{rows, group < groups, false, make_uint2(0u, 0u)};
+      if (!p.any) return p;
+      uint32_t pieces = 1, g = group;
+      if (g < sg.count[0]) {
         pieces = sg.pieces[0];
-        p.row = (group * pieces + piece) * kSelPiece;
-      } else if (group < sg.count[0] + sg.count[1]) {
+        p.row = (piece * sg.count[0] + g) * kSelPiece + 4 * (uint32_t)lane;
+      } else if ((g -= sg.count[0]) < sg.count[1]) {
         pieces = sg.pieces[1];
-        p.row = (sg.count[0] * sg.pieces[0] + (group - sg.count[0]) * pieces + piece) * kSelPiece;
+        p.row = (sg.count[0] * sg.pieces[0] + piece * sg.count[1] + g) * kSelPiece + 4 * (uint32_t)lane;
       } else {
-        p.row = (sg.count[0] * sg.pieces[0] + sg.count[1] * sg.pieces[1]) * kSelPiece + (group - sg.count[0] - sg.count[1]) * sg.small;
+        g -= sg.count[1];
+        const uint32_t run = (uint32_t)lane / (kSelRun / 4) * small_groups + g;
+        if (4 * (uint32_t)lane < sg.small) p.row = small_row + run * kSelRun + 4 * ((uint32_t)lane % (kSelRun / 4));
+        p.last = g == last_group;
       }
-      p.end = p.row + (group < sg.count[0] + sg.count[1] ? kSelPiece : sg.small);
       ++piece;
-      if (p.row + 4 * (uint32_t)lane < (p.end < rows ? p.end : rows)) p.maxima = __ldg(reinterpret_cast<const uint2*>(row_max + p.row) + lane);
+      if (p.row < rows) p.maxima = __ldg(reinterpret_cast<const uint2*>(row_max + p.row));
       if (piece == pieces) {
         ++taken;
         piece = 0;
@@ -556,11 +565,11 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     // and its loads (lane l reads 4 l .. 4 l + 3) are then both free of bank conflicts.
     const uint32_t stage0 = (uint32_t)__cvta_generic_to_shared(sw.stage[0]);
     auto request = [&](uint32_t& my_row) -> uint32_t {  // asks for the next rows that hold a candidate; returns how many there are
-      while (tail - head < kSelRows && now.row < now.end) {
+      while (tail - head < kSelRows && now.any) {
         const Piece p = now;
         now = then;
         then = next_piece();
-        if (p.end >= rows && lane < (int)(d & 3)) {  // the client's ragged tail goes with its last piece: straight to its buckets
+        if (p.last && lane < (int)(d & 3)) {  // the client's ragged tail goes with its last piece: straight to its buckets
           const uint32_t b = __float_as_uint(x[(uint64_t)nvec * 4 + lane]), key = b & 0x7FFFFFFFu;
           if (key >= thresh) {
             if (key > keytop) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
@@ -572,13 +581,12 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
         }
         // bins are 12 bits: the top bit of a half survives the subtraction where the row's bin reaches the threshold's
         uint32_t h01 = (p.maxima.x | 0x80008000u) - thresh_bin * 0x10001u, h23 = (p.maxima.y | 0x80008000u) - thresh_bin * 0x10001u;
-        const uint32_t row = p.row + 4 * (uint32_t)lane;
-        if (p.end - p.row < kSelPiece || p.end >= held_rows) {  // not every lane has rows
-          const uint32_t end = p.end < held_rows ? p.end : held_rows;
-          h01 &= (row < end ? 0x8000u : 0u) | (row + 1 < end ? 0x80000000u : 0u);
-          h23 &= (row + 2 < end ? 0x8000u : 0u) | (row + 3 < end ? 0x80000000u : 0u);
-          ragged |= p.end >= held_rows;
+        const uint32_t row = p.row;
+        if (row + 4 > held_rows) {  // not all of the lane's rows are there
+          h01 &= (row < held_rows ? 0x8000u : 0u) | (row + 1 < held_rows ? 0x80000000u : 0u);
+          h23 &= (row + 2 < held_rows ? 0x8000u : 0u) | (row + 3 < held_rows ? 0x80000000u : 0u);
         }
+        ragged |= p.last;
         if (!__any_sync(kFull, ((h01 | h23) & 0x80008000u) != 0)) continue;
         auto list = [&](bool hit, uint32_t which) {
           const unsigned hits = __ballot_sync(kFull, hit);
@@ -694,52 +702,61 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
     __syncthreads();
     if (s_client == groups) {
       __threadfence();
+      // A thread has sixteen sub-buckets: their counts and the check of the coarse ones are read side by side, and one scan does.  A
+      // client's end takes 2.7 us of 8192 sub-buckets (two rounds of eight, read behind the check: 6.5).
+      constexpr uint32_t kMine = 16;
+      static_assert(kSelThreads * kMine >= kRankSubs && kRankSubs % kMine == 0, "one scan");
+      const uint32_t n_sub = r.split ? r.n_coarse << r.sub_bits : 0u, i0 = (uint32_t)tid * kMine;
+      uint4 v4[kMine / 4];
+      if (i0 < n_sub) {
+        const uint4* count = reinterpret_cast<const uint4*>(ws + L.off_sub_count) + ((size_t)c * kRankSubs + i0) / 4;
+#pragma unroll
+        for (uint32_t e = 0; e < kMine / 4; ++e) v4[e] = __ldcg(count + e);
+      } else {
+#pragma unroll
+        for (uint32_t e = 0; e < kMine / 4; ++e) v4[e] = make_uint4(0u, 0u, 0u, 0u);
+      }
       // the update must be the one the plan was made from
       for (uint32_t i = tid; i < r.n_coarse; i += kSelThreads) {
         const uint32_t end = i + 1 < r.n_coarse ? s_start[i + 1] : r.n;
         if (__ldcg(fill + i) != end - s_start[i]) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
       }
       if (r.split) {
-        const uint32_t n_sub = r.n_coarse << r.sub_bits;
-        const float* count = reinterpret_cast<const float*>(ws + L.off_sub_count) + (size_t)c * kRankSubs;
         uint32_t* start = reinterpret_cast<uint32_t*>(ws + L.off_sub_start) + (size_t)c * (kRankSubs + 64);
         uint32_t* next = reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs;
-        constexpr uint32_t kMine = 8;
-        uint32_t carry = 0;
-        for (uint32_t base = 0; base < n_sub; base += kSelThreads * kMine) {
-          const uint32_t i0 = base + (uint32_t)tid * kMine;
-          uint32_t v[kMine], sum = 0;
+        uint32_t v[kMine], sum = 0;
 #pragma unroll
-          for (uint32_t e = 0; e < kMine; ++e) v[e] = (i0 + e < n_sub) ? (r.wide ? __float_as_uint(__ldcg(count + i0 + e)) : (uint32_t)__ldcg(count + i0 + e)) : 0u;
-#pragma unroll
-          for (uint32_t e = 0; e < kMine; ++e) sum += v[e];
-          uint32_t incl = sum;
-#pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t o = __shfl_up_sync(kFull, incl, off);
-            if (lane >= off) incl += o;
-          }
-          if (lane == 31) s_scan[warp] = incl;
-          __syncthreads();
-          uint32_t run = carry + incl - sum, all = 0;
-          for (int w = 0; w < kSelThreads / 32; ++w) {
-            const uint32_t t = s_scan[w];
-            if (w < warp) run += t;
-            all += t;
-          }
-#pragma unroll
-          for (uint32_t e = 0; e < kMine; ++e) {
-            if (i0 + e < n_sub) {
-              start[i0 + e] = run;
-              next[i0 + e] = run;
-              if (v[e] > kRankItems && run < hdr->limit && run + v[e] <= r.n) list_bucket(hdr, ws, L, c, r, sh_sub, i0 + e, run, v[e]);
-            }
-            run += v[e];
-          }
-          carry += all;
-          __syncthreads();
+        for (uint32_t e = 0; e < kMine; ++e) {
+          const uint32_t w = e % 4 == 0 ? v4[e / 4].x : e % 4 == 1 ? v4[e / 4].y : e % 4 == 2 ? v4[e / 4].z : v4[e / 4].w;
+          v[e] = r.wide ? w : (uint32_t)__uint_as_float(w);
+          sum += v[e];
         }
-        if (tid == 0) start[n_sub] = carry;
+        const uint32_t incl = warp_inclusive(sum);
+        if (lane == 31) s_scan[warp] = incl;
+        __syncthreads();
+        const uint32_t of_warp = lane < kSelThreads / 32 ? s_scan[lane] : 0u;
+        const uint32_t all = __reduce_add_sync(kFull, of_warp);
+        uint32_t run = __reduce_add_sync(kFull, lane < warp ? of_warp : 0u) + incl - sum;
+        if (i0 < n_sub) {  // behind the last sub-bucket there are none: the total
+#pragma unroll
+          for (uint32_t e = 0; e < kMine; e += 4) {
+            uint4 at;
+            at.x = run;
+            at.y = at.x + v[e];
+            at.z = at.y + v[e + 1];
+            at.w = at.z + v[e + 2];
+            run = at.w + v[e + 3];
+            reinterpret_cast<uint4*>(start + i0)[e / 4] = at;
+            reinterpret_cast<uint4*>(next + i0)[e / 4] = at;
+            if (max(max(v[e], v[e + 1]), max(v[e + 2], v[e + 3])) > kRankItems) {
+              const uint32_t from[4] = {at.x, at.y, at.z, at.w};
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u)
+                if (v[e + u] > kRankItems && from[u] < hdr->limit && from[u] + v[e + u] <= r.n) list_bucket(hdr, ws, L, c, r, sh_sub, i0 + e + u, from[u], v[e + u]);
+            }
+          }
+        }
+        if (tid == 0 && n_sub % kMine == 0) start[n_sub] = all;  // else among the above
       }
     }
     __syncthreads();
