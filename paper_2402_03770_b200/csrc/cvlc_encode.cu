@@ -1147,33 +1147,54 @@ k_sort_pass(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
 // ===================================================================================
 // K5  per-packet centroid distribution (PQ: min/max; QSGD: l2-norm), stochastic quantization, bit packing
 // ===================================================================================
-// One warp works through kPackGroup consecutive packets of one client, without block-wide barriers.  Packet r
-// (longest codes first) holds ranks [Z, Z + cap(y_r)).  The packet is assembled in the warp's shared-memory
-// buffer: every record ORs its bits into the (at most three) 32-bit words it touches, then the words go out with
-// consecutive addresses.  The ranked pairs are read twice from global memory (statistics, then quantization);
-// the second read hits in cache.  A lane quantizes about twelve records of a packet: twelve independent Philox
-// chains in flight.
+// One warp works through kPackGroup consecutive packets of one client, without block-wide barriers; where a batch has so few packets
+// that most of the chip would stand idle, the block's four warps share one.  Packet r (longest codes first) holds ranks
+// [Z, Z + cap(y_r)).  The packet is assembled in a shared-memory buffer: every record ORs its bits into the (at most three) 32-bit
+// words it touches, then the words go out with consecutive addresses.  The ranked pairs are read twice from global memory
+// (statistics, then quantization); the second read hits in cache.  A lane of a warp alone quantizes about twelve records of a packet
+// one after the other, one of four warps three.
 
 constexpr int kPackThreads = 128;
 constexpr int kPackWarps = kPackThreads / 32;
 constexpr int kPackGroup = 1;  // packets per warp (more of them amortise the length table but lengthen the tail)
+// Packets of a batch up to which a block works on one, about those that are resident at a time (9 blocks per SM).  Kernel with a warp
+// and with the block for a packet, us, one / 24 clients: 500 packets 16.5 and 12.1 / 14.5 and 12.3, 1000 16.2 and 12.2 / 15.9 and
+// 13.4, 1500 17.4 and 14.4 / 16.3 and 16.2, 2000 18.2 and 16.1 / 16.8 and 18.0, 3000 20.3 and 20.3 / 19.4 and 22.2.  With QSGD, whose
+// norm is one lane's chain in both, 500 16.3 and 12.9 / 17.3 and 13.9, 1000 16.2 and 14.1 / 20.1 and 16.0, 1500 18.2 and 18.3 / 21.2 and
+// 20.4, 2000 18.5 and 20.2 / 22.4 and 22.4.
+constexpr uint64_t kTeamPackets = 13 * kNumSM, kTeamPacketsQsgd = 9 * kNumSM;
 
-template <int CAP, bool QSGD>
+template <int CAP, bool QSGD, int TEAM>
 __global__ void __launch_bounds__(kPackThreads)
 k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Shape shape, unsigned char* ws,
        const __grid_constant__ EncLayout L, uint32_t warp_bytes, int write_residual) {
-  extern __shared__ __align__(16) unsigned char s_pack[];  // per warp: packet words; QSGD: then cap(1) squares
+  [[maybe_unused]] __shared__ float s_team[2][TEAM];
+  extern __shared__ __align__(16) unsigned char s_pack[];  // per packet at work: packet words; QSGD: then cap(1) squares
+  static_assert(TEAM == 1 || TEAM == kPackWarps, "a warp or the block for a packet");
+  constexpr uint32_t STEP = TEAM * 32;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t at = TEAM == 1 ? lane : tid;  // thread of the packet's
+  auto sync = [] {
+    if constexpr (TEAM == 1) __syncwarp();
+    else __syncthreads();
+  };
   const uint32_t c = blockIdx.y;
   const ClientDesc& cd = batch.c[c];
   const cvlc_plan_t* __restrict__ plan = cd.plan;
+  // packet -> its code length and first rank: lane l holds length 32 - l (longest first), below with the
+  // inclusive sums of packets and of records up to and including that length
+  const uint32_t yl = CVLC_MAX_CODE_BITS - lane;
+  const uint32_t ny = plan->n_y[yl];
+  const uint32_t capl = plan->cap[yl];
+  const unsigned long long plan_k = plan->k, plan_candidates = plan->n_candidates;
+  const uint32_t mask = reinterpret_cast<const uint32_t*>(ws + L.off_pass_mask)[c];
+  if (block_sees_error(&hdr->status)) return;  // looked at behind the others' requests
   const uint32_t s = shape.s;
   const uint32_t H = shape.header_bits;
   const uint32_t n_words = shape.packet_bits / 32;
-  unsigned char* s_mine = s_pack + (size_t)warp * warp_bytes;
+  unsigned char* s_mine = s_pack + (TEAM == 1 ? (size_t)warp * warp_bytes : 0);
   uint32_t* words = reinterpret_cast<uint32_t*>(s_mine);
   uint32_t* stream_words = reinterpret_cast<uint32_t*>(cd.stream);
   // error compensation: the encoder's input is memory + update and becomes the new memory, i.e. every sent
@@ -1181,16 +1202,10 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
   float* __restrict__ residual = write_residual ? const_cast<float*>(cd.x) : nullptr;
   const PhiloxRoundKeys rk = philox_round_keys(cd.seed);
 
-  const uint32_t mask = reinterpret_cast<const uint32_t*>(ws + L.off_pass_mask)[c];
   const int flips = __popc(~mask & ((1u << kSortPasses) - 1u));
   const unsigned long long* __restrict__ sorted =
       reinterpret_cast<const unsigned long long*>(ws + ((flips & 1) ? L.off_buf_b : L.off_buf_a)) + (size_t)c * L.capacity;
 
-  // packet -> its code length and first rank: lane l holds length 32 - l (longest first) with the
-  // inclusive sums of packets and of records up to and including that length
-  const uint32_t yl = CVLC_MAX_CODE_BITS - lane;
-  const uint32_t ny = plan->n_y[yl];
-  const uint32_t capl = plan->cap[yl];
   const unsigned long long nz = (unsigned long long)ny * capl;
   uint32_t cum = ny;
   unsigned long long zc = nz;
@@ -1209,7 +1224,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     const uint32_t tot_packets = __shfl_sync(kFull, cum, 31);
     const unsigned long long tot_records = __shfl_sync(kFull, zc, 31);
     const bool qsgd_one_bit = QSGD && __shfl_sync(kFull, ny, 31) != 0;  // a one-bit QSGD code holds no level
-    if (tot_packets != shape.R || tot_records != plan->k || tot_records == 0 || tot_records > plan->n_candidates ||
+    if (tot_packets != shape.R || tot_records != plan_k || tot_records == 0 || tot_records > plan_candidates ||
         tot_records > (unsigned long long)shape.R * shape.cap[1] || qsgd_one_bit) {
       if (blockIdx.x == 0 && tid == 0) set_status(&hdr->status, CVLC_ERR_PLAN_MISMATCH);
       return;
@@ -1217,7 +1232,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
   }
 
   for (int g = 0; g < kPackGroup; ++g) {
-    const uint32_t r = (blockIdx.x * kPackWarps + warp) * kPackGroup + g;
+    const uint32_t r = (TEAM == 1 ? blockIdx.x * kPackWarps + warp : blockIdx.x) * kPackGroup + g;
     if (r >= shape.R) break;
     const unsigned hit = __ballot_sync(kFull, r < cum);
     if (hit == 0) break;
@@ -1225,8 +1240,8 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     const uint32_t y = CVLC_MAX_CODE_BITS - (uint32_t)src_lane;
     const unsigned long long Z = __shfl_sync(kFull, (zc - nz) + (unsigned long long)(r - (cum - ny)) * capl, src_lane);
     const uint32_t P = __shfl_sync(kFull, capl, src_lane);
-    for (uint32_t w = lane; w < n_words; w += 32) words[w] = 0u;
-    __syncwarp();
+    for (uint32_t w = at; w < n_words; w += STEP) words[w] = 0u;
+    sync();
     const uint32_t wd = s + y;
     const unsigned long long* __restrict__ seg = sorted + Z;
     float lo, hi;  // the header's two centroid fields
@@ -1253,15 +1268,21 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     if constexpr (QSGD) {
       // ---- QSGD: |x| against the packet's l2-norm; code = sign bit above a level of s_q = 2^(y-1) - 1 steps ----
       double* sqv = reinterpret_cast<double*>(s_mine + (((size_t)n_words * 4 + 8 + 15) & ~(size_t)15));
-      for (uint32_t j = lane; j < P; j += 32) {
+      for (uint32_t j = at; j < P; j += STEP) {
         const double a = (double)__uint_as_float((uint32_t)(seg[j] >> 32));
         sqv[j] = __dmul_rn(a, a);  // exact: 24 x 24 bits
       }
-      __syncwarp();
+      sync();
       // the norm is defined with the squares added in rank order in double: one lane walks the chain
       float norm = 0.0f;
-      if (lane == 0) norm = qsgd_norm_of_squares(sqv, P);
-      norm = __shfl_sync(kFull, norm, 0);
+      if (at == 0) norm = qsgd_norm_of_squares(sqv, P);
+      if constexpr (TEAM == 1) {
+        norm = __shfl_sync(kFull, norm, 0);
+      } else {
+        if (at == 0) s_team[0][0] = norm;
+        __syncthreads();
+        norm = s_team[0][0];
+      }
       lo = norm;
       hi = 0.0f;
       const uint32_t sq = (uint32_t)((1ull << (y - 1)) - 1ull);  // y >= 2: checked with the plan
@@ -1269,7 +1290,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
       const double dn = (double)norm;
       const double scale = (norm > 0.0f) ? __ddiv_rn(sqd, dn) : 0.0;
       const float fscale = fast_scale(scale, y - 1);
-      for (uint32_t j = lane; j < P; j += 32) {
+      for (uint32_t j = at; j < P; j += STEP) {
         const unsigned long long pair = seg[j];
         const uint32_t key = (uint32_t)(pair >> 32);
         const uint32_t pid = (uint32_t)pair & 0x7FFFFFFFu;
@@ -1291,7 +1312,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     } else {
       // ---- PQ: minimum / maximum of the packet's signed values (its centroid distribution) ----
       float vmin = CUDART_INF_F, vmax = -CUDART_INF_F;
-      for (uint32_t j = lane; j < P; j += 32) {
+      for (uint32_t j = at; j < P; j += STEP) {
         const unsigned long long pair = seg[j];
         const uint32_t key = (uint32_t)(pair >> 32);
         const uint32_t b = key ? (key | ((uint32_t)pair & 0x80000000u)) : 0u;  // -0 is stored as +0
@@ -1303,6 +1324,18 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
       for (int off = 16; off > 0; off >>= 1) {
         vmin = fminf(vmin, __shfl_xor_sync(kFull, vmin, off));
         vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, off));
+      }
+      if constexpr (TEAM > 1) {
+        if (lane == 0) {
+          s_team[0][warp] = vmin;
+          s_team[1][warp] = vmax;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < TEAM; ++w) {
+          vmin = fminf(vmin, s_team[0][w]);
+          vmax = fmaxf(vmax, s_team[1][w]);
+        }
       }
       lo = vmin;
       hi = vmax;
@@ -1318,11 +1351,11 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
       if (plain) {
         // the usual case, without a branch but for the rounding fp32 cannot tell; the next record is requested ahead
         const float fL = (float)Lc;
-        unsigned long long next = (uint32_t)lane < P ? seg[lane] : 0ull;
-        uint32_t bitpos = H + (uint32_t)lane * wd;
-        for (uint32_t j = lane; j < P; j += 32, bitpos += 32 * wd) {
+        unsigned long long next = at < P ? seg[at] : 0ull;
+        uint32_t bitpos = H + at * wd;
+        for (uint32_t j = at; j < P; j += STEP, bitpos += STEP * wd) {
           const unsigned long long pair = next;
-          if (j + 32 < P) next = seg[j + 32];
+          if (j + STEP < P) next = seg[j + STEP];
           const uint32_t key = (uint32_t)(pair >> 32), pid = (uint32_t)pair & 0x7FFFFFFFu;
           const float v = __uint_as_float(key | ((uint32_t)pair & 0x80000000u));
           const uint32_t word = philox_coord(rk, cd.client_id, cd.round, pid);
@@ -1340,7 +1373,7 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
           }
         }
       }
-      for (uint32_t j = plain ? P : lane; j < P; j += 32) {
+      for (uint32_t j = plain ? P : at; j < P; j += STEP) {
         const unsigned long long pair = seg[j];
         const uint32_t key = (uint32_t)(pair >> 32);
         const uint32_t pid = (uint32_t)pair & 0x7FFFFFFFu;
@@ -1359,16 +1392,16 @@ k_pack(const __grid_constant__ BatchDesc<CAP> batch, const __grid_constant__ Sha
     }  // PQ
 
     // packet header {s, y, lo, hi} in bits 0..79 (bits 80..H-1 stay zero)
-    if (lane == 0) {
+    if (at == 0) {
       const uint32_t blo = __float_as_uint(lo), bhi = __float_as_uint(hi);
       atomicOr(words + 0, s | (y << 8) | (blo << 16));
       atomicOr(words + 1, (blo >> 16) | (bhi << 16));
       atomicOr(words + 2, bhi >> 16);
     }
-    __syncwarp();
+    sync();
     uint32_t* pkt = stream_words + CVLC_STREAM_HEADER_BYTES / 4 + (size_t)r * n_words;
-    for (uint32_t w = lane; w < n_words; w += 32) pkt[w] = words[w];
-    __syncwarp();  // the word buffer is reused by the next packet
+    for (uint32_t w = at; w < n_words; w += STEP) pkt[w] = words[w];
+    sync();  // the word buffer is reused by the next packet
   }
 
   // global header (64 bytes), written once per client
@@ -1416,8 +1449,10 @@ template <int CAP>
 static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, unsigned char* w, size_t warp_bytes,
                                  int write_residual, cudaStream_t st, bool overlap) {
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
-  auto kernel = qsgd ? k_pack<CAP, true> : k_pack<CAP, false>;
-  if (warp_bytes * kPackWarps > 48 * 1024) {  // large packets only
+  const bool team = (uint64_t)shape.R * n <= (qsgd ? kTeamPacketsQsgd : kTeamPackets);
+  auto kernel = team ? (qsgd ? k_pack<CAP, true, kPackWarps> : k_pack<CAP, false, kPackWarps>) : (qsgd ? k_pack<CAP, true, 1> : k_pack<CAP, false, 1>);
+  const uint32_t at_work = team ? 1 : kPackWarps;  // packets of a block
+  if (warp_bytes * at_work > 48 * 1024) {  // large packets only
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
   }
@@ -1425,8 +1460,8 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
   batch.n = n;
   batch.pad = 0;
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
-  const unsigned grid = (shape.R + kPackWarps * kPackGroup - 1) / (kPackWarps * kPackGroup);
-  launch_kernel(kKPack, kernel, dim3(grid, n), kPackThreads, warp_bytes * kPackWarps, st, overlap, batch, shape, w, L, (uint32_t)warp_bytes, write_residual);
+  const unsigned grid = (shape.R + at_work * kPackGroup - 1) / (at_work * kPackGroup);
+  launch_kernel(kKPack, kernel, dim3(grid, n), kPackThreads, warp_bytes * at_work, st, overlap, batch, shape, w, L, (uint32_t)warp_bytes, write_residual);
   return cudaGetLastError();
 }
 
