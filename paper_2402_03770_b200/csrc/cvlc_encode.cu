@@ -146,7 +146,6 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
     hdr->own_n = hdr->own_next = hdr->own_done = hdr->part_n = hdr->part_next = 0;
     hdr->most = s_most;
     hdr->most_split = s_most_split;
-    hdr->sort_tiles = run;
   }
   // ranked by partition: the result is in the first buffer (the digit passes write a mask of their own)
   if (plan_ws)

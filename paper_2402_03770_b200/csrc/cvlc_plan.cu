@@ -426,7 +426,7 @@ __device__ __noinline__ void finish_client(uint32_t c, const Batch& batch, const
       const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.capacity);
       reinterpret_cast<ClientRank*>(enc.ws + enc.off_rank)[c] = r;
       reinterpret_cast<uint32_t*>(enc.ws + enc.off_pass_mask)[c] = (1u << kSortPasses) - 1u;  // ranked by partition: the result is in the first buffer
-      add_client(eh, r, limit, enc.capacity);
+      add_client(eh, r, limit);
       if (c == 0) eh->limit = limit;
     }
   }

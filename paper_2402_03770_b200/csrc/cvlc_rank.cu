@@ -114,7 +114,7 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
 // a grid: 784 -> 303 (and 143).  Half as many cells, or blocks of 256 threads with half the window, are within 5 %; twice the cells cost
 // 20 % (clearing and scanning them), keeping an item's place from the counting 10 % (the atomic then returns a value).
 __global__ void __launch_bounds__(kRankThreads, 2)
-k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all) {
+k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, uint32_t blocks) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   RankShared& s = *reinterpret_cast<RankShared*>(s_raw);
   __shared__ RankTile s_tile[2];
@@ -124,7 +124,7 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x;
   if (tid == 0) {
-    s_args = rank_args(ws, L, bin_start_all, hdr, batch.n);
+    s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks);
     s_tile[0].ticket = atomicAdd(&hdr->rank_ticket, 1u);
   }
   __syncthreads();
@@ -155,14 +155,14 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
 
 // What the ranking has left over (see rank_lists)
 __global__ void __launch_bounds__(kRankThreads, 2)
-k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all) {
+k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, uint32_t blocks) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   __shared__ RankArgs s_args;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   if ((hdr->list_n[0] | hdr->list_n[1] | hdr->big[0].n | hdr->own_n) == 0) return;
-  if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n);
+  if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks);
   rank_lists<kRankThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, s_args);
 }
 
@@ -177,9 +177,10 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
   launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * sms), kRankThreads, kRankSubs * 4, st, true,
                 batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
-  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start);
+  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start,
+                2 * sms);
   launch_kernel(kKRankRest, k_rank_rest, blocks((L.capacity + kRankItems - 1) / kRankItems * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true,
-                batch, ws, L, bin_start);
+                batch, ws, L, bin_start, 2 * sms);
   return cudaGetLastError();
 }
 

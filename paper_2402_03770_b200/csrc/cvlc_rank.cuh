@@ -503,7 +503,8 @@ struct RankArgs {
   size_t capacity, big_room, piece_room;  // the latter two per round
   uint32_t n, tickets, window, limit;
 };
-__device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout& L, const uint32_t* bin_start, const EncHeader* hdr, uint32_t n) {
+__device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout& L, const uint32_t* bin_start, const EncHeader* hdr, uint32_t n,
+                                              uint32_t blocks) {
   RankArgs a;
   a.rank = reinterpret_cast<const ClientRank*>(ws + L.off_rank);
   a.sub_start = reinterpret_cast<const uint32_t*>(ws + L.off_sub_start);
@@ -523,7 +524,7 @@ __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout
   a.big_room = (size_t)n * a.capacity / kRankItems + 1;
   a.piece_room = (size_t)n * a.capacity / kBigPiece + a.big_room;
   a.n = n;
-  a.window = rank_window(hdr);
+  a.window = rank_window(hdr->most, n, blocks);
   a.tickets = (hdr->most + a.window - 1) / a.window * n;
   a.limit = hdr->limit;
   return a;
