@@ -475,7 +475,7 @@ static inline EncFront enc_front(const EncLayout& L, void* ws) {
 }
 cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st);
 // unframed stream (version 2)
-constexpr uint32_t kUfMaxRecords = 2048;  // records of a block (it is sorted and assembled in one warp's shared memory)
+constexpr uint32_t kUfMaxRecords = 2048;  // records of a block (they are sorted and assembled in shared memory)
 constexpr size_t kUfTables = 64, kUfTotalBits = 64 + 264, kUfDirectory = 64 + 264 + 8;
 CVLC_HD constexpr size_t uf_head_bytes(uint32_t R) { return kUfDirectory + (size_t)R * 8; }
 CVLC_HD constexpr size_t uf_off_ticket() { return 256; }

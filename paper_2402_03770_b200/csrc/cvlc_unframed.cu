@@ -63,32 +63,41 @@ __device__ __forceinline__ void or_ones(uint32_t* img, uint32_t pos, uint32_t co
   }
 }
 
-// One warp writes one block.  Blocks are handed out by a per-client ticket, so every earlier block of the client is
-// being written or done when a warp looks back for its bit offset.
+// One thread block writes one block of records.  They are handed out by a per-client ticket, so every earlier one of the client is
+// being written or done when a thread block looks back for its bit offset.  A block of records takes 13 KB of shared memory (1500-byte
+// packets): with a warp each, four to a thread block, an SM held 16 warps, and the kernel was the chain of one.  Between events, us: 8 clients of
+// 1.2 M coordinates at 2 bits 38.0 -> 29.1, one of 0.75 M at 0.8 29.2 -> 17.8, 60 of 0.3 M at 1 48.3 -> 27.5, 20 of 11.2 M at 2 428 ->
+// 378.  For twelve on an SM (40 registers) a few words are spilled; with nine it is 35.4, 17.2, 33.6 and 443, with sixteen 31.2, 18.9,
+// 32.8 and 364.
 template <bool QSGD>
-__global__ void __launch_bounds__(kUfThreads)
+__global__ void __launch_bounds__(kUfThreads, 12)
 k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned char* enc_ws,
                 const __grid_constant__ EncLayout L, unsigned char* uf_ws, uint32_t P_max, uint32_t img_words,
-                uint32_t warp_bytes, unsigned long long* __restrict__ sizes_out) {
+                unsigned long long* __restrict__ sizes_out) {
   extern __shared__ __align__(16) unsigned char s_uf[];
   __shared__ int s_err;
+  __shared__ uint32_t s_ticket, s_low[kUfWarps], s_high[kUfWarps], s_full[kUfWarps], s_sum[kUfWarps], s_len[2][kUfWarps];
+  __shared__ float s_lo[kUfWarps], s_hi[kUfWarps];
+  __shared__ unsigned long long s_run;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(enc_ws);
-  if (threadIdx.x == 0) s_err = *reinterpret_cast<const volatile int32_t*>(&hdr->status);
+  const uint32_t c = blockIdx.y;
+  if (threadIdx.x == 0) {
+    s_err = *reinterpret_cast<const volatile int32_t*>(&hdr->status);
+    s_ticket = atomicAdd(reinterpret_cast<uint32_t*>(uf_ws + uf_off_ticket()) + c, 1u);
+  }
   __syncthreads();
   if (s_err != 0) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t c = blockIdx.y;
+  const uint32_t tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
   const ClientDesc cd = batch.c[c];
   const cvlc_plan_t* __restrict__ plan = cd.plan;
   const uint32_t R = shape.R;
-  unsigned char* s_mine = s_uf + (size_t)warp * warp_bytes;
-  unsigned long long* rec = reinterpret_cast<unsigned long long*>(s_mine);  // [P_max] position << 32 | value bits
+  unsigned long long* rec = reinterpret_cast<unsigned long long*>(s_uf);     // [P_max] position << 32 | value bits
   unsigned long long* by_cell = rec + P_max;                                // [P_max] the records by their cells
   double* sqv = reinterpret_cast<double*>(by_cell);                         // QSGD: before that the squares of the values
   uint32_t* cell = reinterpret_cast<uint32_t*>(by_cell + P_max);            // [kUfCells]
   uint32_t* img = cell + kUfCells;                                          // [img_words + 2] the block's bits
-  uint32_t* ticket = reinterpret_cast<uint32_t*>(uf_ws + uf_off_ticket());
   unsigned long long* state = reinterpret_cast<unsigned long long*>(uf_ws + uf_off_state(batch.n)) + (size_t)c * R;
   uint32_t* stream_words = reinterpret_cast<uint32_t*>(cd.stream);
   uint32_t* body = stream_words + uf_head_bytes(R) / 4;
@@ -125,10 +134,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     }
   }
 
-  uint32_t r = 0;
-  if (lane == 0) r = atomicAdd(ticket + c, 1u);
-  r = __shfl_sync(kFull, r, 0);
-  if (r >= R) return;
+  const uint32_t r = s_ticket;  // below R: the client has R thread blocks
   const unsigned hit = __ballot_sync(kFull, r < cum);
   const int src_lane = __ffs(hit) - 1;
   const uint32_t y = CVLC_MAX_CODE_BITS - (uint32_t)src_lane;
@@ -141,7 +147,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
   // ---- the block's records and its centroid distribution (over the records in rank order, as for a packet)
   float vmin = CUDART_INF_F, vmax = -CUDART_INF_F;
   uint32_t pmin = 0xFFFFFFFFu, pmax = 0u;
-  for (uint32_t j = lane; j < P; j += 32) {
+  for (uint32_t j = tid; j < P; j += kUfThreads) {
     const unsigned long long pair = seg[j];
     const uint32_t key = (uint32_t)(pair >> 32), pid = (uint32_t)pair & 0x7FFFFFFFu;
     const uint32_t b = key ? (key | ((uint32_t)pair & 0x80000000u)) : 0u;  // -0 is stored as +0
@@ -159,64 +165,82 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
   }
   pmin = __reduce_min_sync(kFull, pmin);
   pmax = __reduce_max_sync(kFull, pmax);
-#pragma unroll
-  for (uint32_t i = 0; i < kUfCells / 32; ++i) cell[i * 32 + lane] = 0u;
-  for (uint32_t w = lane; w < img_words + 2; w += 32) img[w] = 0u;
-  __syncwarp();
-  float lo, hi;
-  if constexpr (QSGD) {
-    float norm = 0.0f;
-    if (lane == 0) norm = qsgd_norm_of_squares(sqv, P);
-    lo = __shfl_sync(kFull, norm, 0);
-    hi = 0.0f;
-  } else {
+  if constexpr (!QSGD) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       vmin = fminf(vmin, __shfl_xor_sync(kFull, vmin, off));
       vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, off));
     }
+  }
+  if (lane == 0) {
+    s_low[warp] = pmin;
+    s_high[warp] = pmax;
+    s_lo[warp] = vmin;
+    s_hi[warp] = vmax;
+  }
+  for (uint32_t i = tid; i < kUfCells; i += kUfThreads) cell[i] = 0u;
+  for (uint32_t w = tid; w < img_words + 2; w += kUfThreads) img[w] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kUfWarps; ++w) {
+    pmin = min(pmin, s_low[w]);
+    pmax = max(pmax, s_high[w]);
+  }
+  float lo, hi;
+  if constexpr (QSGD) {
+    if (tid == 0) s_lo[0] = qsgd_norm_of_squares(sqv, P);
+    __syncthreads();
+    lo = s_lo[0];
+    hi = 0.0f;
+  } else {
     lo = vmin;
     hi = vmax;
+#pragma unroll
+    for (int w = 0; w < kUfWarps; ++w) {
+      lo = fminf(lo, s_lo[w]);
+      hi = fmaxf(hi, s_hi[w]);
+    }
   }
 
   // ---- ascending position: the records are spread over kUfCells equal ranges of the block's positions, a few in each, and
   // compared with the others of their cell.  Where the positions crowd into few cells, a bitonic network sorts them instead.
   const uint32_t csh = (pmax - pmin) < kUfCells ? 0u : 32u - __clz(pmax - pmin) - kUfCellBits;  // (pmax - pmin) >> csh < kUfCells
-  __syncwarp();
-  for (uint32_t j = lane; j < P; j += 32) atomicAdd(cell + (((uint32_t)(rec[j] >> 32) - pmin) >> csh), 1u);
-  __syncwarp();
-  uint32_t fullest = 0;
+  for (uint32_t j = tid; j < P; j += kUfThreads) atomicAdd(cell + (((uint32_t)(rec[j] >> 32) - pmin) >> csh), 1u);
+  __syncthreads();
+  uint32_t fullest;
   {
-    constexpr uint32_t kMine = kUfCells / 32;
-    uint32_t v[kMine], sum = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < kMine; ++i) {
-      v[i] = cell[kMine * lane + i];
-      sum += v[i];
-      fullest = v[i] > fullest ? v[i] : fullest;
-    }
+    static_assert(kUfCells == 4 * kUfThreads, "four cells a thread");
+    uint4* mine = reinterpret_cast<uint4*>(cell) + tid;
+    const uint4 v = *mine;
+    const uint32_t sum = v.x + v.y + v.z + v.w;
+    fullest = __reduce_max_sync(kFull, max(max(v.x, v.y), max(v.z, v.w)));
     uint32_t run = sum;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const uint32_t o = __shfl_up_sync(kFull, run, off);
       if (lane >= off) run += o;
     }
+    if (lane == 31) {
+      s_sum[warp] = run;
+      s_full[warp] = fullest;
+    }
+    __syncthreads();
     run -= sum;
 #pragma unroll
-    for (uint32_t i = 0; i < kMine; ++i) {
-      cell[kMine * lane + i] = run;
-      run += v[i];
+    for (int w = 0; w < kUfWarps; ++w) {
+      if (w < warp) run += s_sum[w];
+      fullest = max(fullest, s_full[w]);
     }
-    fullest = __reduce_max_sync(kFull, fullest);
+    *mine = make_uint4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
   }
-  __syncwarp();
+  __syncthreads();
   if (fullest <= 64) {
-    for (uint32_t j = lane; j < P; j += 32) {
+    for (uint32_t j = tid; j < P; j += kUfThreads) {
       const unsigned long long e = rec[j];
       by_cell[atomicAdd(cell + (((uint32_t)(e >> 32) - pmin) >> csh), 1u)] = e;
     }
-    __syncwarp();
-    for (uint32_t j = lane; j < P; j += 32) {
+    __syncthreads();
+    for (uint32_t j = tid; j < P; j += kUfThreads) {
       const unsigned long long e = by_cell[j];
       const uint32_t k = ((uint32_t)(e >> 32) - pmin) >> csh;
       const uint32_t q0 = k ? cell[k - 1] : 0u, q1 = cell[k];  // the places have advanced to the cells' ends
@@ -224,7 +248,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       for (uint32_t q = q0; q < q1; ++q) rank += by_cell[q] < e ? 1u : 0u;
       rec[rank] = e;
     }
-    __syncwarp();
+    __syncthreads();
   } else {
     // comparators that all point the same way: places behind the last record need none
     uint32_t size = 2;
@@ -232,7 +256,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     for (uint32_t k = 2; k <= size; k <<= 1) {
       for (uint32_t jj = k >> 1; jj > 0; jj >>= 1) {
         const uint32_t flip = (jj == k >> 1) ? k - 1 : jj;  // first step of a merge: against the mirror image
-        for (uint32_t t = lane; t < size / 2; t += 32) {
+        for (uint32_t t = tid; t < size / 2; t += kUfThreads) {
           const uint32_t i = ((t & ~(jj - 1)) << 1) | (t & (jj - 1)), p = i ^ flip;
           if (p < P) {
             const unsigned long long x = rec[i], z = rec[p];
@@ -242,17 +266,17 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
             }
           }
         }
-        __syncwarp();
+        __syncthreads();
       }
     }
   }
 
-  // ---- records, 32 at a time: code, length, offset by a warp scan, bits OR-ed into the block's image
-  if (lane == 0) {
+  // ---- records, one a thread at a time: code, length, offset by a scan, bits OR-ed into the block's image
+  if (tid == 0) {
     img[0] = __float_as_uint(lo);
     img[1] = __float_as_uint(hi);
   }
-  __syncwarp();
+  __syncthreads();
   const double Lc = (double)((1ull << y) - 1ull);
   const double dlo = (double)lo;
   const double den = __dsub_rn((double)hi, dlo);
@@ -262,8 +286,8 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
   const double q_scale = (QSGD && lo > 0.0f) ? __ddiv_rn(sqd, dn) : 0.0;
   const float fscale = QSGD ? fast_scale(q_scale, y - 1) : fast_scale(pq_scale, y);
   uint32_t carry = 64;
-  for (uint32_t base = 0; base < P; base += 32) {
-    const uint32_t j = base + lane;
+  for (uint32_t base = 0; base < P; base += kUfThreads) {
+    const uint32_t j = base + tid;
     const bool valid = j < P;
     uint32_t len = 0, quo = 0;
     unsigned long long tail = 0;
@@ -295,20 +319,27 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       const uint32_t o = __shfl_up_sync(kFull, incl, off);
       if (lane >= off) incl += o;
     }
+    uint32_t* sums = s_len[(base / kUfThreads) & 1];  // the last but one's have been read: a barrier lies between
+    if (lane == 31) sums[warp] = incl;
+    __syncthreads();
     if (valid) {
-      const uint32_t pos = carry + incl - len;
+      uint32_t pos = carry + incl - len;
+#pragma unroll
+      for (int w = 0; w < kUfWarps; ++w)
+        if (w < warp) pos += sums[w];
       or_ones(img, pos, quo);
       or_bits(img, pos + quo, tail);
     }
-    carry += __shfl_sync(kFull, incl, 31);
+#pragma unroll
+    for (int w = 0; w < kUfWarps; ++w) carry += sums[w];
   }
-  __syncwarp();
+  __syncthreads();
   const uint32_t block_bits = carry;
 
-  // ---- bit offset of the block: decoupled look-back over the client's earlier blocks, 32 at a time
-  if (lane == 0) st_relaxed(state + r, (r == 0 ? kFlagPrefix : kFlagAgg) | block_bits);
+  // ---- bit offset of the block: decoupled look-back over the client's earlier blocks, 32 at a time, by one warp
+  if (tid == 0) st_relaxed(state + r, (r == 0 ? kFlagPrefix : kFlagAgg) | block_bits);
   unsigned long long run = 0;
-  if (r > 0) {
+  if (r > 0 && warp == 0) {
     long long top = (long long)r - 1;
     while (true) {
       const long long idx = top - lane;
@@ -326,15 +357,20 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       if (is_prefix) break;
       top -= 32;
     }
-    if (lane == 0) st_relaxed(state + r, kFlagPrefix | (run + block_bits));
+    if (lane == 0) {
+      st_relaxed(state + r, kFlagPrefix | (run + block_bits));
+      s_run = run;
+    }
   }
+  __syncthreads();
+  if (r > 0) run = s_run;
 
   // ---- the image goes out shifted to its bit offset; the first and the last word are shared with the neighbours
   {
     const uint32_t shift = (uint32_t)(run & 31ull);
     const size_t w0 = (size_t)(run >> 5);
     const uint32_t n_out = (shift + block_bits + 31) >> 5;
-    for (uint32_t ow = lane; ow < n_out; ow += 32) {
+    for (uint32_t ow = tid; ow < n_out; ow += kUfThreads) {
       uint32_t v = img[ow] << shift;  // img has two zero words behind its last used one
       if (shift && ow) v |= img[ow - 1] >> (32 - shift);
       if (ow == 0 || ow == n_out - 1) {
@@ -343,7 +379,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
         body[w0 + ow] = v;
       }
     }
-    if (lane == 0) {
+    if (tid == 0) {
       unsigned long long* dir = reinterpret_cast<unsigned long long*>(cd.stream + kUfDirectory);
       dir[r] = run;
       if (r == R - 1) {
@@ -354,8 +390,8 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     }
   }
 
-  // ---- stream header and the tables of lengths, by the warp that wrote block 0
-  if (r == 0) {
+  // ---- stream header and the tables of lengths, by the thread block that wrote block 0
+  if (r == 0 && warp == 0) {
     if (lane < 16) {
       uint32_t v = 0;
       const unsigned long long Bbits = (unsigned long long)__double_as_longlong(cd.scale_B);
@@ -412,12 +448,11 @@ cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capaci
     if (b > bits) bits = b;
   }
   const uint32_t img_words = (uint32_t)((bits + 31) / 32);
-  const size_t warp_bytes = (size_t)P_max * 16 + ((((size_t)img_words + 2 + kUfCells) * 4 + 15) & ~(size_t)15);
+  const size_t block_bytes = (size_t)P_max * 16 + ((((size_t)img_words + 2 + kUfCells) * 4 + 15) & ~(size_t)15);
   launch_kernel(kKZeroWords, k_uf_clear, 4 * kNumSM, 256, 0, st, true, batch, stream_capacity / 16, static_cast<unsigned char*>(uf_ws),
                 uf_ws_bytes(n, shape.R) / 4);
-  const unsigned grid = (shape.R + kUfWarps - 1) / kUfWarps;
-  launch_kernel(kKPackUnframed, qsgd ? k_pack_unframed<true> : k_pack_unframed<false>, dim3(grid, n), kUfThreads, warp_bytes * kUfWarps, st, true,
-                batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), P_max, img_words, (uint32_t)warp_bytes, sizes_out);
+  launch_kernel(kKPackUnframed, qsgd ? k_pack_unframed<true> : k_pack_unframed<false>, dim3(shape.R, n), kUfThreads, block_bytes, st, true,
+                batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), P_max, img_words, sizes_out);
   return cudaGetLastError();
 }
 

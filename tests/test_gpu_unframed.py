@@ -203,3 +203,26 @@ def test_unframed_decoder_meets_long_and_short_unary_parts(env, d, pb, R, shape,
         else:
             assert status == 0
             assert_aggregate_close(out, want)
+
+
+@pytest.mark.parametrize("quantizer", [0, 1])
+@pytest.mark.parametrize("crowded", [False, True])
+@pytest.mark.parametrize("records", [1, 31, 33, 127, 129, 511, 513, 1_750])
+def test_blocks_around_the_threads_that_share_them(env, records, crowded, quantizer):
+    """records per block at the edges of a warp, a thread block and its cells; positions spread or nearly all in one cell"""
+    torch, B = env
+    d, y, R = 70_000, 4, 5
+    pb = (80 + 21 * records + 31) // 32 * 32                  # 17 bits of position and 4 of code in a packet
+    pd = params_dict(d, R * pb, packet_bits=pb, quantizer=quantizer, seed=records, max_code_bits=8,
+                     scale_B=1e3)
+    po = oracle_params(pd)
+    plan = O.plan_fixed(po, y)
+    rng = np.random.default_rng(records + crowded)
+    x = rng.standard_normal(d) * 1e-6
+    at = np.arange(plan.k) + 900 if crowded else rng.permutation(d)[:plan.k]
+    x[at] = rng.standard_normal(plan.k) + 3.0
+    x[d - 1] = 10.0                                           # one record far from the others
+    x = x.astype(np.float32)
+    ref = O.encode_unframed(x, po, plan)
+    status, got, _, _ = gpu_unframed(torch, B, [x], [pd], fixed_y=y)
+    assert status == 0 and got[0].size == ref.size and (got[0] == ref).all()
