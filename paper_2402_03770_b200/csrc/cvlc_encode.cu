@@ -381,8 +381,8 @@ __device__ __noinline__ void list_bucket(EncHeader* hdr, unsigned char* ws, cons
 }
 
 __global__ void __launch_bounds__(kSelThreads, 1)
-k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, const unsigned char* __restrict__ plan_ws, unsigned char* ws,
-         const __grid_constant__ EncLayout L) {
+k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, const __grid_constant__ SelectGroups sg,
+         const unsigned char* __restrict__ plan_ws, unsigned char* ws, const __grid_constant__ EncLayout L) {
   extern __shared__ __align__(16) unsigned char s_sel[];
   SelWarp& sw = reinterpret_cast<SelWarp*>(s_sel)[threadIdx.x >> 5];
   uint32_t* s_start = reinterpret_cast<uint32_t*>(s_sel + (kSelThreads / 32) * sizeof(SelWarp));  // [kRankCoarse] starts of the client's buckets
@@ -390,11 +390,13 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   __shared__ uint32_t s_client, s_taken, s_scan[kSelThreads / 32];
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
-  if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t i = tid; i < kRankSubs / 4; i += kSelThreads) reinterpret_cast<uint4*>(s_sub)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (uint32_t i = lane; i < kRankCoarse; i += 32) sw.cnt[i] = 0;
+  if (tid == 0) s_taken = 0;
+  if (block_sees_error(&hdr->status)) return;
   const uint32_t n = batch.n;
   const uint32_t rows = (uint32_t)part.rows, held_rows = ((uint32_t)(d >> 2) + kRowUnits - 1) / kRowUnits;  // with coordinates
-  const SelectGroups sg = select_groups(part, n);
   const uint32_t groups = sg.groups;
   // A group's rows are spread over all that the groups of its size share, in runs of kSelRun (small groups) or pieces (larger ones), so
   // that all of them meet a layer that holds most of a client's candidates, where neighbouring rows made a group dense or empty: 24
@@ -405,17 +407,14 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
   const uint32_t nvec = (uint32_t)(d >> 2);
   uint32_t* group_next = reinterpret_cast<uint32_t*>(ws + L.off_group_next);
   uint32_t* group_done = reinterpret_cast<uint32_t*>(ws + L.off_group_done);
-  for (uint32_t i = tid; i < kRankSubs; i += kSelThreads) s_sub[i] = 0;
-  for (uint32_t i = lane; i < kRankCoarse; i += 32) sw.cnt[i] = 0;
-  if (tid == 0) s_taken = 0;
   // Block b starts with client b n / grid; the first groups of a client go to the warps of the blocks that start with it, the rest
   // by its counter.  A small batch would wait for that: there the warps have three quarters of the groups without asking, and all
   // of them with few clients, whose blocks are as good as equally many, and in the smallest batches, where the last of them are not
   // worth a wait.  Whole calls with all and with three quarters, us: 4 clients of 3 M coordinates 113 and 121, 8 of 3 M 154 and 160;
   // 10 of 0.3 / 1.2 / 3 M 65 and 69 / 100 and 105 / 174 and 176, 24 of 0.3 / 1.2 M 86 and 90 / 159 and 160; 12 / 16 of 3 M 205 and 201
   // / 239 and 228, 40 of 1.2 M 235 and 226.
-  const uint32_t home = (uint32_t)(((uint64_t)blockIdx.x * n) / gridDim.x);
-  auto first_block = [&](uint32_t c) -> uint32_t { return (uint32_t)(((uint64_t)c * gridDim.x + n - 1) / n); };
+  const uint32_t home = blockIdx.x * n / gridDim.x;
+  auto first_block = [&](uint32_t c) -> uint32_t { return (c * gridDim.x + n - 1) / n; };
   auto warps_of = [&](uint32_t c) -> uint32_t { return (first_block(c + 1) - first_block(c)) * (kSelThreads / 32); };
   auto rounds_of = [&](uint32_t warps) -> uint32_t {
     if (sg.count[0] + sg.count[1] || warps == 0) return 1;
@@ -1496,9 +1495,10 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   else if (n <= (uint32_t)kMediumBatch) launch_init_t<kMediumBatch>(clients, n, shape, L, pws, w, st);
   else launch_init_t<kLargeBatch>(clients, n, shape, L, pws, w, st);
   if (pws) {
-    const uint64_t want = (uint64_t)select_groups(part, n).groups * n;
+    const SelectGroups sg = select_groups(part, n);  // here: its divisions in every warp took a microsecond
+    const uint64_t want = (uint64_t)sg.groups * n;
     const unsigned grid = (unsigned)(want < (uint64_t)sms ? want : sms);
-    launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, pws, w, L);
+    launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, sg, pws, w, L);
     e = launch_rank(batch, L, pws, w, sms, st);
     if (e != cudaSuccess) return e;
   } else {

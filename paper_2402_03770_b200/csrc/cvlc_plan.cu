@@ -498,7 +498,7 @@ k_hist(const Batch batch, const __grid_constant__ Shape shape, const __grid_cons
   if (pos + part.chunk < end) end = pos + part.chunk;
 
   while (pos < end) {
-    const uint64_t c = pos / part.rows;
+    const uint64_t c = part.per_client ? q / part.per_client : pos / part.rows;
     const uint64_t seg_end = ((c + 1) * part.rows < end) ? (c + 1) * part.rows : end;
     const uint64_t u0 = (pos - c * part.rows) * kRowUnits, u1 = (seg_end - c * part.rows) * kRowUnits;  // units of the client
     const float* __restrict__ x = batch.c[c].x;
