@@ -495,7 +495,6 @@ cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capaci
 cudaError_t launch_decode_unframed(const uint8_t* const* streams, const uint64_t* stream_bytes, const float* weights,
                                    uint32_t n, double weight_total, uint64_t d, uint32_t s, float* out, int accumulate,
                                    void* ws, cudaStream_t st);
-cudaError_t launch_fill_zero(float* out, uint64_t d, cudaStream_t st);
 cudaError_t launch_selftest_wait(unsigned long long* word, int32_t* status, uint32_t max_polls, cudaStream_t st);
 cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_bytes, const float* weights,
                           uint32_t n, double weight_total, uint64_t d, uint32_t s, float* out, int accumulate,
@@ -608,6 +607,20 @@ __device__ __forceinline__ uint32_t rank_window(uint32_t most, uint32_t n, uint3
   const uint32_t tiles = (least * n + blocks - 1) / blocks * blocks / n;  // below 2^29: at most 2^19 tiles of at most 512 clients
   const uint32_t window = tiles ? (most + tiles - 1) / tiles : 0u;
   return window > 1024 ? window : 1024;
+}
+
+// thread `first` of `stride` writes its share of d zeros
+__device__ __forceinline__ void zero_fill(float* __restrict__ out, uint64_t d, uint64_t first, uint64_t stride) {
+  const uint64_t nvec = d >> 2;
+  float4* ov = reinterpret_cast<float4*>(out);
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (uint64_t v = first; v < nvec; v += stride) ov[v] = z;
+  if (first < (d & 3)) out[(nvec << 2) + first] = 0.f;
+}
+// blocks of `threads` for it, `most` at the most
+inline unsigned fill_grid(uint64_t coords, uint64_t threads, uint64_t most) {
+  const uint64_t want = (coords / 4 + threads - 1) / threads;
+  return (unsigned)(want < most ? (want ? want : 1) : most);
 }
 
 #endif  // __CUDACC__

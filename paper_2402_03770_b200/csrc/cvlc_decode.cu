@@ -12,15 +12,6 @@ constexpr int kDecodeThreads = 256;
 constexpr uint32_t kDecStageWords = 512;  // packets up to 2 KB are staged in shared memory
 constexpr uint64_t kDecodeWindow = 24ull << 20;  // coordinates of the accumulator filled per decode launch (96 MB: inside the L2)
 
-// thread `first` of `stride` writes its share of d zeros
-__device__ __forceinline__ void zero_fill(float* __restrict__ out, uint64_t d, uint64_t first, uint64_t stride) {
-  const uint64_t nvec = d >> 2;
-  float4* ov = reinterpret_cast<float4*>(out);
-  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (uint64_t v = first; v < nvec; v += stride) ov[v] = z;
-  if (first < (d & 3)) out[(nvec << 2) + first] = 0.f;
-}
-
 struct StreamHead {
   uint32_t magic, ver_q_s, d_lo, d_hi, R, packet_bits, header_bits, client_id, seed_lo, seed_hi, round, zero, B_lo, B_hi, k_lo, k_hi;
 };
@@ -324,10 +315,6 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
   uint64_t n_win = (d + kDecodeWindow - 1) / kDecodeWindow;
   if (n_win == 1 && d > kDecodeWindow / 6 * 5 && n >= 6) n_win = 2;
   const uint64_t win = (((d + n_win - 1) / n_win) + 1023) & ~(uint64_t)1023;
-  auto fill_grid = [](uint64_t coords, uint64_t threads, uint64_t most) -> unsigned {
-    const uint64_t want = (coords / 4 + threads - 1) / threads;
-    return (unsigned)(want < most ? (want ? want : 1) : most);
-  };
   const uint64_t first = win < d ? win : d;
   const uint64_t zero_d = accumulate ? 0 : first;
   launch_kernel(kKDecodePrepare, k_decode_prepare, 1 + (accumulate ? 0 : fill_grid(first, kPrepThreads, 2 * kNumSM)), kPrepThreads, 0, st, false,
@@ -342,13 +329,6 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
     }
     launch_kernel(kKDecode, k_decode, 8 * kNumSM, kDecodeThreads, ((size_t)n + 1) * 4, st, true, streams, n, d, s, out, w, lo, hi);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fill_zero(float* out, uint64_t d, cudaStream_t st) {
-  const uint64_t want = (d / 4 + 255) / 256;
-  const int grid = (int)(want < (uint64_t)(8 * kNumSM) ? (want ? want : 1) : 8 * kNumSM);
-  launch_kernel(kKFillZero, k_fill_zero, grid, 256, 0, st, true, out, d);
   return cudaGetLastError();
 }
 

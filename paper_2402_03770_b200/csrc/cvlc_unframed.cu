@@ -462,10 +462,12 @@ cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capaci
 
 constexpr int kUfPrepThreads = 1024;
 
-// validates the headers and tables, derives the per-client coefficients and the prefix of block counts
+// validates the headers and tables, derives the per-client coefficients and the prefix of block counts (block 0); meanwhile the other
+// blocks write the accumulator's zeros, which depend on nothing
 __global__ void __launch_bounds__(kUfPrepThreads)
 k_uf_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* __restrict__ stream_bytes,
-                    const float* __restrict__ weights, uint32_t n, double weight_total, uint64_t d, uint32_t s, unsigned char* ws) {
+                    const float* __restrict__ weights, uint32_t n, double weight_total, uint64_t d, uint32_t s, unsigned char* ws,
+                    float* __restrict__ zero_out) {
   __shared__ double s_part[kUfPrepThreads / 32];
   __shared__ uint32_t s_cnt[kUfPrepThreads / 32];
   __shared__ double s_W;
@@ -475,6 +477,10 @@ k_uf_decode_prepare(const uint8_t* const* __restrict__ streams, const uint64_t* 
   uint32_t* prefix = reinterpret_cast<uint32_t*>(ws + dec_off_prefix(n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_enter();
+  if (blockIdx.x > 0) {
+    zero_fill(zero_out, d, (uint64_t)(blockIdx.x - 1) * kUfPrepThreads + tid, (uint64_t)(gridDim.x - 1) * kUfPrepThreads);
+    return;
+  }
   if (tid == 0) {
     *status = 0;
     s_carry = 0;
@@ -800,11 +806,8 @@ cudaError_t launch_decode_unframed(const uint8_t* const* streams, const uint64_t
                                    uint32_t n, double weight_total, uint64_t d, uint32_t s, float* out, int accumulate,
                                    void* ws, cudaStream_t st) {
   unsigned char* w = static_cast<unsigned char*>(ws);
-  launch_kernel(kKDecodePrepare, k_uf_decode_prepare, 1, kUfPrepThreads, 0, st, false, streams, stream_bytes, weights, n, weight_total, d, s, w);
-  if (!accumulate) {
-    const cudaError_t e = launch_fill_zero(out, d, st);
-    if (e != cudaSuccess) return e;
-  }
+  launch_kernel(kKDecodePrepare, k_uf_decode_prepare, 1 + (accumulate ? 0 : fill_grid(d, kUfPrepThreads, 2 * kNumSM)), kUfPrepThreads, 0, st, false,
+                streams, stream_bytes, weights, n, weight_total, d, s, w, out);
   const size_t prefix_bytes = ((size_t)n + 1) * 4;
   if (prefix_bytes + sizeof(UfDecWarp) * kUfDecWarps > 47 * 1024) {  // hundreds of clients: the most of any call, another thread's too
     const cudaError_t e = allow_shared(k_decode_unframed, ((size_t)CVLC_MAX_CLIENTS_PER_CALL + 1) * 4);
