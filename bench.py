@@ -39,11 +39,11 @@ FALLBACK_HBM_GBS = 6650.0
 # proportion to the clients); scaled to the clients of a launch, None for any other configuration, for fewer than
 # 32 clients per launch, and for a kernel that has changed since its capture.
 NCU_TRAFFIC_BYTES_PER_CLIENT = {
-    "k_hist": (1433.84e6 + 44.53e6) / 32,          # the update once, plus the rows' maxima
-    "k_select": (402.64e6 + 167.66e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
-    "k_rank_split": (203.46e6 + 154.20e6) / 32,
-    "k_rank": (203.13e6 + 156.04e6) / 32,
-    "k_pack": (177.98e6 + 54.06e6) / 32,
+    "k_hist": (1433.86e6 + 45.05e6) / 32,          # the update once, plus the rows' maxima
+    "k_select": (402.01e6 + 168.91e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
+    "k_rank_split": (203.41e6 + 153.67e6) / 32,
+    "k_rank": (203.13e6 + 155.47e6) / 32,
+    "k_pack": (177.99e6 + 53.81e6) / 32,
 }
 NOMINAL_HBM_GBS = 8000.0
 
@@ -405,10 +405,12 @@ def run_ours(args):
     plans = [enc.read_plan(i) for enc in encoders for i in range(enc.n)]
     stream_bytes = B.cvlc_stream_bytes(params[0])
     n_groups = len(groups)
-    sum_cand = float(sum(p.n_candidates for p in plans))
     sum_k = float(sum(p.k for p in plans))
+    # Large batches are tuned before they are selected from, and then the selection begins at the bin that holds rank k, so the plans'
+    # n_candidates are more than what is moved: counted are those that are sent
+    sum_cand = sum_k
     # the partition moves the candidates of clients with a bucket of more than 4096 (here: on average)
-    split_bytes = float(sum(16.0 * p.n_candidates for p in plans if p.n_candidates > 4096 * min(256, p.top_bin + 1 - p.thresh_bin)))
+    split_bytes = float(sum(16.0 * p.k for p in plans if p.k > 4096 * min(256, p.top_bin + 1 - p.thresh_bin)))
     alg_bytes_per_step = {   # algorithmic bytes all launches of one step move
         "k_hist": 4.0 * d * n_clients,
         "k_select": 4.0 * d * n_clients + 8.0 * sum_cand,

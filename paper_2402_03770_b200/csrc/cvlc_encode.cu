@@ -324,8 +324,8 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
 // buffer.  When that is full the warp counts its candidates per coarse bucket, reserves room in every bucket with one global
 // addition and puts the candidates there; they are also counted per sub-bucket where the client needs the partition.  The block
 // that completes a client turns those counts into offsets.
-// Bound by instruction issue (0.55 per scheduler and cycle).  100 clients of 11.2 M coordinates, 7 % candidates: 680 us; 50 of
-// 23.5 M, 3.5 %: 587; 10 of 100 M, 1 %: 229.  The copies go past the L1 (cp.async.cg): with loads into registers the warps were
+// Bound by instruction issue (0.60 per scheduler and cycle).  100 clients of 11.2 M coordinates, 6 % candidates: 568 us; 50 of
+// 23.5 M, 3.5 %: 610; 10 of 100 M, 1 %: 210.  The copies go past the L1 (cp.async.cg): with loads into registers the warps were
 // bound by the L1 lines that shared memory leaves for loads in flight (832, 943 and 377 us), and more warps made it worse; asking
 // the L2 for 64 bytes instead of the 128 that it fetches by default takes 344 instead of 512 MB from DRAM for 8 of the second.
 // (One buffer per block, emptied by all its warps together, left them waiting for one another: 860 us for the first.)
