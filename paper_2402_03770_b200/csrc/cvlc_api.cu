@@ -148,7 +148,7 @@ size_t plan_ws_bytes_of(uint64_t d, uint32_t n) { return plan_ws_bytes(make_part
 // the packing kernel assembles one packet per warp, four warps per block, in shared memory (QSGD: each next to the
 // squares of the packet's values): four of them must fit
 bool pack_fits(const Shape& S) {
-  return 4 * ((size_t)S.packet_bits / 8 + 16 + (S.quantizer == CVLC_QUANT_QSGD ? (size_t)S.cap[1] * 8 : 0)) <= 200 * 1024;
+  return 4 * ((size_t)S.packet_bits / 8 + 16 + (S.quantizer == CVLC_QUANT_QSGD ? (size_t)S.cap[1] * 8 : 0)) <= kPackSharedMax;
 }
 
 }  // namespace

@@ -471,6 +471,7 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
 // the error-compensation memory (the input buffers are written: every sent coordinate loses what the parameter
 // server rebuilds for it); kPackNone = selection and ranking only (the unframed writer follows)
 constexpr int kPackFramed = 0, kPackResidual = 1, kPackNone = 2;
+constexpr size_t kPackSharedMax = 200 * 1024;  // shared memory of four packets at work, at most
 // prepared: the planning front of the same call has prepared the workspace (see EncFront) and precedes it on the stream
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual);

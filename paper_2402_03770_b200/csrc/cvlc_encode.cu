@@ -1443,6 +1443,16 @@ static void launch_init_t(const ClientDesc* clients, uint32_t n, const Shape& sh
   launch_kernel(kKEncodeInit, k_encode_init<CAP>, 2 * kNumSM, 256, 0, st, false, w, batch, shape, L, plan_ws);
 }
 
+// What the largest packets take is allowed to every form of the kernel beforehand.  (Asked for where a launch has more than 48 KB of its
+// own, that line would have to count the kernel's static shared memory too.)
+template <int CAP>
+static cudaError_t pack_attributes() {
+  cudaError_t e = allow_shared(k_pack<CAP, false, 1>, kPackSharedMax);
+  if (e == cudaSuccess) e = allow_shared(k_pack<CAP, false, kPackWarps>, kPackSharedMax);
+  if (e == cudaSuccess) e = allow_shared(k_pack<CAP, true, 1>, kPackSharedMax);
+  return e != cudaSuccess ? e : allow_shared(k_pack<CAP, true, kPackWarps>, kPackSharedMax);
+}
+
 template <int CAP>
 static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, unsigned char* w, size_t warp_bytes,
                                  int write_residual, cudaStream_t st, bool overlap) {
@@ -1450,10 +1460,6 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
   const bool team = (uint64_t)shape.R * n <= (qsgd ? kTeamPacketsQsgd : kTeamPackets);
   auto kernel = team ? (qsgd ? k_pack<CAP, true, kPackWarps> : k_pack<CAP, false, kPackWarps>) : (qsgd ? k_pack<CAP, true, 1> : k_pack<CAP, false, 1>);
   const uint32_t at_work = team ? 1 : kPackWarps;  // packets of a block
-  if (warp_bytes * at_work > 48 * 1024) {  // large packets only
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-  }
   BatchDesc<CAP> batch;
   batch.n = n;
   batch.pad = 0;
@@ -1475,8 +1481,11 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
                           const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual) {
   static OncePerDevice once;
   cudaError_t e = once_per_device(once, [] {
-    const cudaError_t e = allow_shared(k_select, kSelSmem);
-    return e != cudaSuccess ? e : allow_shared(k_sort_pass, sort_smem_bytes(CVLC_MAX_BATCH));
+    cudaError_t e = allow_shared(k_select, kSelSmem);
+    if (e == cudaSuccess) e = allow_shared(k_sort_pass, sort_smem_bytes(CVLC_MAX_BATCH));
+    if (e == cudaSuccess) e = pack_attributes<kSmallBatch>();
+    if (e == cudaSuccess) e = pack_attributes<kMediumBatch>();
+    return e != cudaSuccess ? e : pack_attributes<kLargeBatch>();
   });
   if (e != cudaSuccess) return e;
   const EncLayout L = enc_layout(shape.d, n, capacity);
