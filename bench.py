@@ -405,12 +405,10 @@ def run_ours(args):
     plans = [enc.read_plan(i) for enc in encoders for i in range(enc.n)]
     stream_bytes = B.cvlc_stream_bytes(params[0])
     n_groups = len(groups)
+    sum_cand = float(sum(p.n_candidates for p in plans))
     sum_k = float(sum(p.k for p in plans))
-    # Large batches are tuned before they are selected from, and then the selection begins at the bin that holds rank k, so the plans'
-    # n_candidates are more than what is moved: counted are those that are sent
-    sum_cand = sum_k
     # the partition moves the candidates of clients with a bucket of more than 4096 (here: on average)
-    split_bytes = float(sum(16.0 * p.k for p in plans if p.k > 4096 * min(256, p.top_bin + 1 - p.thresh_bin)))
+    split_bytes = float(sum(16.0 * p.n_candidates for p in plans if p.n_candidates > 4096 * min(256, p.top_bin + 1 - p.thresh_bin)))
     alg_bytes_per_step = {   # algorithmic bytes all launches of one step move
         "k_hist": 4.0 * d * n_clients,
         "k_select": 4.0 * d * n_clients + 8.0 * sum_cand,

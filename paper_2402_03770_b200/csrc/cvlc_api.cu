@@ -477,13 +477,6 @@ int cvlc_ec_accumulate_batch(float* const* memory_dev, const float* const* updat
                                                                                                                   : CVLC_ERR_CUDA;
 }
 
-// Coordinates of a batch from which on the lengths are tuned before the selection instead of beside it: a tenth of the candidates then
-// need not be selected and ranked (see sent_from), at the price of the tuning's 25 to 80 us (some clients need the series arithmetic).
-// Whole rounds with the tuning first and beside, us: 100 clients of 11.2 M coordinates at 2 bits 3064 and 3107, at 1 bit 2052 and 2076, 50
-// of 23.5 M 2446 and 2482, 10 of 100 M 1271 and 1304; 20 of 23.5 M 1059 and 1068, 50 of 11.2 M 1660 and 1640, 30 of 11.2 M 1058 and 1053,
-// 10 of 11.2 M 463 and 439, 24 of 3 M at 4 bits 488 and 477.
-constexpr uint64_t kTuneFirst = 800000000;
-
 // Two events per device order the two streams of cvlc_compress_batch (created on first use, kept until exit).
 static cudaError_t compress_events(cudaEvent_t* fork, cudaEvent_t* join) {
   static cudaEvent_t ev[64][2];
@@ -531,17 +524,16 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   const bool two = side_stream != nullptr && side_st != main_st;
   Shape Senc = S;
   Senc.fixed_y = 0;
-  if (S.d * n >= kTuneFirst) {
-    if (launch_plan(desc, n, S, plan_ws_dev, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
-    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, false, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
-  }
   if (launch_plan_front(desc, n, S, plan_ws_dev, enc_front(enc_layout(S.d, n, cap), enc_ws_dev), main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
     if (launch_plan_back(n, S, plan_ws_dev, main_st, true, true) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
-  // exponent fit and length tuning read the histograms only; selection and ranking do not need their result.  The lock keeps two
-  // threads from recording the device's events between each other's record and wait.
+  // Exponent fit and length tuning read the histograms only; selection and ranking do not need their result.  (With the tuning first, a
+  // tenth of the candidates need not be selected and ranked: 100 clients of 11.2 M coordinates 2564 instead of 2640 us for layers of
+  // different scales, 2961 instead of 2935 for one normal distribution; but the tuning takes 25 us to 3 ms, and then in front of the
+  // selection: magnitudes that fall as rank^-1 3294 instead of 2945 us, as rank^-1.3 4622 instead of 3898.)  The lock keeps two threads from
+  // recording the device's events between each other's record and wait.
   static std::mutex order;
   std::lock_guard<std::mutex> hold(order);
   cudaEvent_t fork, join;
