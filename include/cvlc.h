@@ -323,7 +323,9 @@ int cvlc_decode_aggregate_unframed(const uint8_t* const* streams_dev, const uint
  * update to the packets.  Selection and ranking need the histogram but not the tuned lengths (they work on
  * the candidates down to an upper bound of k, see cvlc_plan_t::thresh_bin), so with a second stream the
  * length tuning (Algorithm 1 steps 2-14, a latency-bound computation that leaves the memory system idle)
- * runs on side_stream next to them and is joined right before the packets are assembled.
+ * runs next to them, one of the two on side_stream, and is joined right before the packets are assembled.
+ * (Which one is a matter of the batch's size: the tuning, or, where the selection would keep every SM to
+ * itself, selection and ranking.)
  *  plan_ws_dev / enc_ws_dev   workspaces sized by cvlc_plan_batch_workspace_bytes and
  *                             cvlc_encode_batch_workspace_bytes (with the same max_candidates)
  *  side_stream                a second stream of the same device, or NULL / the same stream: everything

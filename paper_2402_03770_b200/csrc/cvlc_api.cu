@@ -356,7 +356,7 @@ static int encode_batch(const float* const* x_dev, const cvlc_params* params, ui
   if (ws_bytes < enc_layout(S.d, n, cap).total) return CVLC_ERR_WORKSPACE_TOO_SMALL;
   if (!pack_fits(S)) return CVLC_ERR_INVALID_ARG;
   if (S.R > 0x7FFFFFFFu || n > 65535) return CVLC_ERR_INVALID_ARG;
-  return launch_encode(desc, n, S, cap, plan_ws_dev, ws_dev, static_cast<cudaStream_t>(cuda_stream), false, nullptr, write_residual) ==
+  return launch_encode(desc, n, S, cap, plan_ws_dev, ws_dev, static_cast<cudaStream_t>(cuda_stream), false, false, nullptr, write_residual) ==
                  cudaSuccess
              ? CVLC_OK
              : CVLC_ERR_CUDA;
@@ -445,7 +445,7 @@ int cvlc_encode_unframed_batch(const float* const* x_dev, const cvlc_params* par
   if (enc_ws_bytes < enc_layout(S.d, n, cap).total || uf_ws_bytes_given < uf_ws_bytes(n, S.R)) return CVLC_ERR_WORKSPACE_TOO_SMALL;
   if (S.R > 0x7FFFFFFFu || n > 65535) return CVLC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (launch_encode(desc, n, S, cap, plan_ws_dev, enc_ws_dev, st, false, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_encode(desc, n, S, cap, plan_ws_dev, enc_ws_dev, st, false, false, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
   return launch_pack_unframed(n, S, cap, stream_capacity, enc_ws_dev, uf_ws_dev,
                               reinterpret_cast<unsigned long long*>(stream_bytes_dev), st) == cudaSuccess
              ? CVLC_OK
@@ -524,24 +524,33 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   const bool two = side_stream != nullptr && side_st != main_st;
   Shape Senc = S;
   Senc.fixed_y = 0;
-  if (launch_plan_front(desc, n, S, plan_ws_dev, enc_front(enc_layout(S.d, n, cap), enc_ws_dev), main_st) != cudaSuccess) return CVLC_ERR_CUDA;
+  const TunePlace place = two ? tune_place(S.d, n) : kTuneAlone;
+  if (launch_plan_front(desc, n, S, plan_ws_dev, enc_front(enc_layout(S.d, n, cap), enc_ws_dev), place, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
-    if (launch_plan_back(n, S, plan_ws_dev, main_st, true, true) != cudaSuccess) return CVLC_ERR_CUDA;
-    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+    if (launch_plan_back(n, S, plan_ws_dev, place, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
+    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, false, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
   // Exponent fit and length tuning read the histograms only; selection and ranking do not need their result.  (With the tuning first, a
   // tenth of the candidates need not be selected and ranked: 100 clients of 11.2 M coordinates 2564 instead of 2640 us for layers of
   // different scales, 2961 instead of 2935 for one normal distribution; but the tuning takes 25 us to 3 ms, and then in front of the
-  // selection: magnitudes that fall as rank^-1 3294 instead of 2945 us, as rank^-1.3 4622 instead of 3898.)  The lock keeps two threads from
+  // selection: magnitudes that fall as rank^-1 3294 instead of 2945 us, as rank^-1.3 4622 instead of 3093.)  The lock keeps two threads from
   // recording the device's events between each other's record and wait.
   static std::mutex order;
   std::lock_guard<std::mutex> hold(order);
   cudaEvent_t fork, join;
   if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;
-  if (launch_plan_back(n, S, plan_ws_dev, side_st, false, false) != cudaSuccess) return CVLC_ERR_CUDA;
-  if (cudaEventRecord(join, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
-  return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+  if (place != kTuneAhead) {
+    if (launch_plan_back(n, S, plan_ws_dev, place, side_st, false) != cudaSuccess) return CVLC_ERR_CUDA;
+    if (cudaEventRecord(join, side_st) != cudaSuccess) return CVLC_ERR_CUDA;
+    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, false, join, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+  }
+  // The tuning directly behind the planning front, selection and ranking on the other stream, behind an event: so the tuning's blocks are on
+  // their SMs first.  (A selection that follows the front on its own stream is there before any kernel of another stream.)
+  if (launch_plan_back(n, S, plan_ws_dev, place, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, side_st, true, true, nullptr, kPackNone) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (cudaEventRecord(join, side_st) != cudaSuccess || cudaStreamWaitEvent(main_st, join, 0) != cudaSuccess) return CVLC_ERR_CUDA;
+  return launch_pack(desc, n, Senc, cap, enc_ws_dev, main_st, false, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
 }
 
 int cvlc_encode(const float* x_dev, const cvlc_params* p, const cvlc_plan_t* plan_dev, const void* plan_ws_dev,

@@ -439,13 +439,36 @@ struct EncFront {
   size_t off_rank, off_pass_mask, zero_end;
 };
 
+// Where the length tuning runs, one block per client that tunes.  Beside selection and ranking, whose blocks fill an SM each, its place
+// matters:
+//  - They leave it its SMs where the clients are few and the selection short: blocks behind a tuning block would start when that ends
+//    (after 25 to 80 us, 67 us into a selection of 120), and the kernel ends with them.  Not for long selections, where blocks that start
+//    late still find work: the SMs given away cost the clients times the length of the selection.  Whole calls with room and without, us:
+//    24 clients of 0.3 M coordinates 90 and 100, 32 of 0.3 / 1.2 / 3 M 98 and 111 / 195 and 203 / 385 and 390, 40 of 0.3 / 1.2 / 3 M 107
+//    and 117 / 239 and 226 / 475 and 441; 10 of 13 / 20 / 40 M 319 and 346 / 434 and 467 / 816 and 820, 20 of 6 / 12 M 309 and 315 / 548
+//    and 514.
+//  - Else it must be ahead of the selection to find an SM before that ends.  That costs the selection's start: the exponent fit of more
+//    than kTuneRoom clients comes first (10 us), then an event.  Behind the selection a tuning of a few hundred us, which steep power
+//    laws need, ends behind the ranking.  Whole calls ahead and behind, us, for one normal distribution / for magnitudes that fall as
+//    rank^-1.3: 10 clients of 40 M 566 and 567 / 1537 and 1672, 20 of 12 M 534 and 526 / 1627 and 1751, 100 of 11.2 M 2937 and 2928 / 3093 and
+//    3904, 60 of 3 M 438 and 430 / 621 and 731; but 40 of 1.2 M 212 and 192 / 435 and 486, 100 of 0.3 M 124 and 105 / 132 and 131 (rank^-1.8:
+//    404 and 446), 33 of 0.3 M 72 and 61 / 80 and 83 (382 and 393).  So short selections with more clients than there is room for, which
+//    is a loss of up to a tenth for steep laws, and one of up to a sixth avoided for all others, have it behind.
+enum TunePlace { kTuneAlone, kTuneRoomLeft, kTuneAhead, kTuneBehind };
+constexpr uint32_t kTuneRoom = 32;
+constexpr uint64_t kTuneRoomRows = 192 << 20;  // times clients
+constexpr uint64_t kShortSelectRows = 8 << 20;
+inline TunePlace tune_place(uint64_t d, uint32_t n) {
+  const uint64_t rows = make_partition(d, n).total;
+  if (n <= kTuneRoom && n * rows <= kTuneRoomRows) return kTuneRoomLeft;
+  return n <= kTuneRoom || rows > kShortSelectRows ? kTuneAhead : kTuneBehind;
+}
 // Planning is launched in two parts.  The front (histogram, rows' maxima, selection threshold, the bins' starts) is all the
-// selection and ranking kernels need; the back (exponent fit and length tuning) is only needed by the packing kernel, so it may
-// run on another stream next to selection and ranking.
-cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st);
-constexpr uint32_t kTuneRoom = 32;  // clients whose tuning blocks selection and ranking leave an SM each (see launch_encode)
-// overlap: nothing but the planning front precedes it on the stream (no wait for an event); alone: nothing runs beside it
-cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone);
+// selection and ranking kernels need; the back (exponent fit, unless it is done ahead of the selection, and length tuning) is only needed by
+// the packing kernel, so it may run on another stream than they do.
+cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, TunePlace place, cudaStream_t st);
+// overlap: nothing but the front precedes the back on its stream (no wait for an event)
+cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st);
@@ -469,12 +492,17 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into
 // the error-compensation memory (the input buffers are written: every sent coordinate loses what the parameter
-// server rebuilds for it); kPackNone = selection and ranking only (the unframed writer follows)
+// server rebuilds for it); kPackNone = selection and ranking only (launch_pack or the unframed writer follows)
 constexpr int kPackFramed = 0, kPackResidual = 1, kPackNone = 2;
 constexpr size_t kPackSharedMax = 200 * 1024;  // shared memory of four packets at work, at most
-// prepared: the planning front of the same call has prepared the workspace (see EncFront) and precedes it on the stream
+// prepared: the planning front of the same call has prepared the workspace (see EncFront) and precedes it on the stream; behind_wait:
+// and a wait for another stream's event lies between
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual);
+                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, bool behind_wait, cudaEvent_t wait_before_pack,
+                          int write_residual);
+// the packing alone, behind selection and ranking; overlap: they directly precede it on the stream
+cudaError_t launch_pack(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity, void* ws, cudaStream_t st, bool overlap,
+                        int write_residual);
 static inline EncFront enc_front(const EncLayout& L, void* ws) {
   return EncFront{static_cast<unsigned char*>(ws), L.capacity, L.off_rank, L.off_pass_mask, L.off_sub_start};
 }

@@ -1469,16 +1469,20 @@ static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Sh
   return cudaGetLastError();
 }
 
-// While the length tuning runs on another stream, one block per client, selection and ranking leave it its SMs: their blocks fill an
-// SM, those behind a tuning block start when that ends (after 25 to 80 us, 67 us into a selection of 120), and the kernel ends with
-// them.  Not for so many clients that too few SMs are left, nor for long selections, where blocks that start late still find work: the
-// SMs given away cost the clients times the length of the selection.  Whole calls with room and without, us: 24 clients of 0.3 M
-// coordinates 90 and 100, 32 of 0.3 / 1.2 / 3 M 98 and 111 / 195 and 203 / 385 and 390, 40 of 0.3 / 1.2 / 3 M 107 and 117 / 239 and 226
-// / 475 and 441; 10 of 13 / 20 / 40 M 319 and 346 / 434 and 467 / 816 and 820, 20 of 6 / 12 M 309 and 315 / 548 and 514.
-constexpr uint64_t kTuneRoomRows = 192 << 20;  // times clients
+cudaError_t launch_pack(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity, void* ws, cudaStream_t st, bool overlap,
+                        int write_residual) {
+  const EncLayout L = enc_layout(shape.d, n, capacity);
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  // packet words and two more; QSGD: and the squares of a packet's values
+  const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 8 + 15) & ~(size_t)15) + (shape.quantizer == CVLC_QUANT_QSGD ? (size_t)shape.cap[1] * 8 : 0);
+  if (n <= (uint32_t)kSmallBatch) return launch_pack_t<kSmallBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+  if (n <= (uint32_t)kMediumBatch) return launch_pack_t<kMediumBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+  return launch_pack_t<kLargeBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, overlap);
+}
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
-                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, cudaEvent_t wait_before_pack, int write_residual) {
+                          const void* plan_ws, void* ws, cudaStream_t st, bool prepared, bool behind_wait, cudaEvent_t wait_before_pack,
+                          int write_residual) {
   static OncePerDevice once;
   cudaError_t e = once_per_device(once, [] {
     cudaError_t e = allow_shared(k_select, kSelSmem);
@@ -1491,12 +1495,8 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const EncLayout L = enc_layout(shape.d, n, capacity);
   if (enc_lists_end(L) > L.off_buf_a) return cudaErrorInvalidValue;
   unsigned char* w = static_cast<unsigned char*>(ws);
-  const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
-  // packet words and two more; QSGD: and the squares of a packet's values
-  const size_t pack_warp = (((size_t)shape.packet_bits / 8 + 8 + 15) & ~(size_t)15) + (qsgd ? (size_t)shape.cap[1] * 8 : 0);
-
   const Partition part = make_partition(shape.d, n);
-  const unsigned sms = wait_before_pack && n <= kTuneRoom && n * part.total <= kTuneRoomRows ? kNumSM - n : kNumSM;
+  const unsigned sms = wait_before_pack && tune_place(shape.d, n) == kTuneRoomLeft ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);
   Batch batch{reinterpret_cast<const ClientDesc*>(w + L.off_desc), n};
   if (prepared) batch.c = reinterpret_cast<const ClientDesc*>(pws + plan_off_desc(n));
@@ -1507,7 +1507,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     const SelectGroups sg = select_groups(part, n);  // here: its divisions in every warp took a microsecond
     const uint64_t want = (uint64_t)sg.groups * n;
     const unsigned grid = (unsigned)(want < (uint64_t)sms ? want : sms);
-    launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, true, batch, shape.d, part, sg, pws, w, L);
+    launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, !behind_wait, batch, shape.d, part, sg, pws, w, L);
     e = launch_rank(batch, L, pws, w, sms, st);
     if (e != cudaSuccess) return e;
   } else {
@@ -1525,11 +1525,8 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     const cudaError_t ew = cudaStreamWaitEvent(st, wait_before_pack, 0);
     if (ew != cudaSuccess) return ew;
   }
-  if (write_residual == kPackNone) return cudaGetLastError();  // the caller writes the ranked records in a format of its own
-  const bool pack_overlap = wait_before_pack == nullptr;
-  if (n <= (uint32_t)kSmallBatch) return launch_pack_t<kSmallBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
-  if (n <= (uint32_t)kMediumBatch) return launch_pack_t<kMediumBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
-  return launch_pack_t<kLargeBatch>(clients, n, shape, L, w, pack_warp, write_residual, st, pack_overlap);
+  if (write_residual == kPackNone) return cudaGetLastError();  // the caller goes on from the ranked records
+  return launch_pack(clients, n, shape, capacity, ws, st, wait_before_pack == nullptr, write_residual);
 }
 
 // memory <- memory + update in fp32, for every client of a batch (the first step of a round with error compensation)

@@ -575,11 +575,15 @@ k_plan_threshold(const Batch batch, const __grid_constant__ Shape shape, unsigne
   finish_client(blockIdx.x, batch, shape, ws, enc, N);
 }
 
-// K2a  per client: exponent fit and tuning key, where the tuning is shared by clients of one key; for histograms from outside
-// (threshold = 1) also the threshold bin.
+// K2a  per client: exponent fit and tuning key, where the tuning is shared by clients of one key.  What the threshold bin comes from:
+enum FitThreshold {
+  kThresholdThere,    // the histogram's last blocks have worked it out
+  kThresholdFinish,   // finish_client, here
+  kThresholdOutside,  // a histogram from outside: the bin alone
+};
 __global__ void __launch_bounds__(kPlanThreads, 1)
 k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __restrict__ nonfinite_all, const Batch batch,
-           const __grid_constant__ Shape shape, unsigned char* ws, int threshold) {
+           const __grid_constant__ Shape shape, unsigned char* ws, const __grid_constant__ EncFront enc, FitThreshold threshold) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* N = reinterpret_cast<uint32_t*>(smem_raw);
   pdl_enter();
@@ -597,7 +601,8 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
   }
   const double B = batch.c[c].scale_B;
   __shared__ PlanTab T;
-  survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
+  if (threshold == kThresholdFinish) finish_client(c, batch, shape, ws, enc, N);
+  else survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
   auto beside_fit = [&]() {
     if (tid >= kPlanThreads - 32) build_plan_tab(T, shape, B, lane);
   };
@@ -607,7 +612,7 @@ k_plan_fit(const unsigned long long* __restrict__ hist_all, const uint32_t* __re
     __syncthreads();
   }
   write_fit(plan, alpha, T, shape);
-  if (threshold) {
+  if (threshold == kThresholdOutside) {
     client_threshold(N, shape, batch.c[c].cap0, plan, nullptr);
     if (tid == 0 && nonfinite) {
       plan->status = CVLC_ERR_NONFINITE_INPUT;
@@ -1555,58 +1560,66 @@ static Batch launch_zero(const ClientDesc* clients, uint32_t n, unsigned char* w
   return Batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
 }
 
-// histogram of every client with (unless only the histograms are wanted) threshold and the bins' tables
-static cudaError_t plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc,
-                              unsigned long long* hist_out, cudaStream_t st) {
-  cudaError_t e = plan_attributes();
-  if (e != cudaSuccess) return e;
-  unsigned char* w = static_cast<unsigned char*>(ws);
-  const Partition part = make_partition(shape.d, n);
-  // header, histograms, flags, counters and tuning keys start at zero (and so does the encoder's workspace up to what its selection
-  // writes in full); the rest is written in full by the kernels that follow
-  const Batch batch = launch_zero(clients, n, w, plan_off_desc(n), enc.ws, enc.ws ? enc.zero_end : 0, st);
-  // the resident blocks share the concatenated updates evenly
-  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, batch, shape, part, w, enc, hist_out ? 0 : 1);
-  if (!hist_out && !part.per_client) launch_kernel(kKPlanThreshold, k_plan_threshold, n, kPlanThreads, 0, st, true, batch, shape, w, enc);
-  e = cudaGetLastError();
-  // the histograms alone: what a client sends when the parameter server plans for it.  The workspace
-  // header stays unmarked, so an encode call cannot take it for one that holds a plan's tables.
-  if (e == cudaSuccess && hist_out) e = cudaMemcpyAsync(hist_out, w + kPlanWsHist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
-  return e;
+// Whether every client has an SM for its tuning and then fits and tunes for itself, or one tunes for all that share a key
+static bool own_tuning(uint32_t n, TunePlace place) { return n <= (place == kTuneAlone ? (uint32_t)kNumSM : kTuneRoom); }
+
+static void launch_fit(const Batch& batch, const Shape& shape, unsigned char* w, const EncFront& enc, FitThreshold threshold, cudaStream_t st, bool overlap) {
+  launch_kernel(kKPlanFit, k_plan_fit, batch.n, kPlanThreads, kFitSmem, st, overlap, reinterpret_cast<const unsigned long long*>(w + kPlanWsHist),
+                reinterpret_cast<const uint32_t*>(w + plan_off_flags(batch.n)), batch, shape, w, enc, threshold);
 }
 
-// `alone`: nothing runs beside it, so that every client may have an SM
-static cudaError_t plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone) {
-  unsigned char* w = static_cast<unsigned char*>(ws);
-  const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
-  const unsigned long long* hist = reinterpret_cast<const unsigned long long*>(w + kPlanWsHist);
-  const bool own = n <= (alone ? (uint32_t)kNumSM : kTuneRoom);
-  if (!own) {
-    launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, overlap, hist, reinterpret_cast<const uint32_t*>(w + plan_off_flags(n)), batch,
-                  shape, w, 0);
-    overlap = true;
-  }
-  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w, own ? hist : nullptr);
+// histogram of every client
+static cudaError_t launch_hist(const ClientDesc* clients, uint32_t n, const Shape& shape, unsigned char* w, const Partition& part, const EncFront& enc,
+                               bool finish, Batch* batch, cudaStream_t st) {
+  const cudaError_t e = plan_attributes();
+  if (e != cudaSuccess) return e;
+  // header, histograms, flags, counters and tuning keys start at zero (and so does the encoder's workspace up to what its selection
+  // writes in full); the rest is written in full by the kernels that follow
+  *batch = launch_zero(clients, n, w, plan_off_desc(n), enc.ws, enc.ws ? enc.zero_end : 0, st);
+  // the resident blocks share the concatenated updates evenly
+  launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, *batch, shape, part, w, enc, finish ? 1 : 0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st) {
-  return plan_front(clients, n, shape, ws, enc, nullptr, st);
+cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, TunePlace place, cudaStream_t st) {
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  const Partition part = make_partition(shape.d, n);
+  Batch batch;
+  const cudaError_t e = launch_hist(clients, n, shape, w, part, enc, true, &batch, st);
+  if (e != cudaSuccess) return e;
+  if (place != kTuneBehind && !own_tuning(n, place))
+    launch_fit(batch, shape, w, enc, part.per_client ? kThresholdThere : kThresholdFinish, st, true);
+  else if (!part.per_client)
+    launch_kernel(kKPlanThreshold, k_plan_threshold, n, kPlanThreads, 0, st, true, batch, shape, w, enc);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, cudaStream_t st, bool overlap, bool alone) {
-  return plan_back(n, shape, ws, st, overlap, alone);
+cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap) {
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  const Batch batch{reinterpret_cast<const ClientDesc*>(w + plan_off_desc(n)), n};
+  const bool own = own_tuning(n, place);
+  if (place == kTuneBehind && !own) {
+    launch_fit(batch, shape, w, EncFront{}, kThresholdThere, st, overlap);
+    overlap = true;
+  }
+  launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, overlap, batch, shape, w,
+                own ? reinterpret_cast<const unsigned long long*>(w + kPlanWsHist) : nullptr);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st) {
-  const cudaError_t e = plan_front(clients, n, shape, ws, EncFront{}, nullptr, st);
-  if (e != cudaSuccess) return e;
-  return plan_back(n, shape, ws, st, true, true);
+  const cudaError_t e = launch_plan_front(clients, n, shape, ws, EncFront{}, kTuneAlone, st);
+  return e != cudaSuccess ? e : launch_plan_back(n, shape, ws, kTuneAlone, st, true);
 }
 
+// The histograms alone: what a client sends when the parameter server plans for it.  The workspace header stays unmarked, so an
+// encode call cannot take it for one that holds a plan's tables.
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st) {
-  return plan_front(clients, n, shape, ws, EncFront{}, hist_out, st);
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  Batch batch;
+  const cudaError_t e = launch_hist(clients, n, shape, w, make_partition(shape.d, n), EncFront{}, false, &batch, st);
+  return e != cudaSuccess ? e : cudaMemcpyAsync(hist_out, w + kPlanWsHist, (size_t)n * CVLC_HIST_BINS * 8, cudaMemcpyDeviceToDevice, st);
 }
 
 // Checks histograms that come from outside: flag bit 0 = a value of exponent 255 (Inf, NaN),
@@ -1646,7 +1659,7 @@ cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const S
   // workspace for one that holds the rows' maxima
   const Batch batch = launch_zero(clients, n, w, kPlanWsHist, w + plan_off_keys(n), plan_off_desc(n) - plan_off_keys(n), st);
   launch_kernel(kKHistCheck, k_hist_check, n, 256, 0, st, true, hist, shape.d, flags);
-  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, 1);
+  launch_kernel(kKPlanFit, k_plan_fit, n, kPlanThreads, kFitSmem, st, true, hist, flags, batch, shape, w, EncFront{}, kThresholdOutside);
   launch_kernel(kKPlanTune, k_plan_tune, n, kTuneThreads, kTuneSmem, st, true, batch, shape, w, static_cast<const unsigned long long*>(nullptr));
   return cudaGetLastError();
 }
