@@ -204,13 +204,14 @@ struct ClientRank {
 };
 // The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates.  As few
 // sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that a block
-// meets costs the selection a global addition); up to 2048 of a client four times as many, since they often lie at one end of it: error
-// compensation leaves the memories crowded below the threshold, in buckets that no block holds (10 clients of 5 M / 1 M coordinates in a
-// later round, ranking and what is left over, us between events: 75 -> 19 / 85 -> 38), and even tiles are ranked sooner (20 of 1.2 M,
-// whole call with aggregation, 143 -> 140; batches that fill the chip unchanged).  No distribution is excluded: sub-buckets that a
-// block cannot hold are split by their own values (see rank_big), zeros among them where more coordinates are sent than are not zero.
-// (Digit passes for a batch with such a client, as phases of one kernel, took it from 844 to 1110 us for one of 11.2 M coordinates,
-// 97 % zeros, and from 1636 to 3100 for 10 of 5 M, 95 % zeros.)
+// meets costs the selection a global addition); up to 512 of a client four times as many, since they often lie at one end of it: error
+// compensation leaves the memories crowded below the threshold, in buckets that no block holds (10 clients of 5 M coordinates in a
+// later round 283 -> 256 us), and even tiles are ranked sooner (20 of 1.2 M 121 -> 119, 10 of 1.2 M 78 -> 75, 100 of 1.2 M 423 -> 415).  Not for
+// clients with more, whose partition then writes its 4096 candidates at a time to places of two each: with up to 1024 300 of 3 M take
+// 2549 us instead of 2498, with up to 2048 2632 (partition 392 us instead of 264), and 100 of 11.2 M in layers of different scales 2610
+// instead of 2558.  No distribution is excluded: sub-buckets that a block cannot hold are split by their own values (see rank_big),
+// zeros among them where more coordinates are sent than are not zero.  (Digit passes for a batch with such a client, as phases of one
+// kernel, took it from 844 to 1110 us for one of 11.2 M coordinates, 97 % zeros, and from 1636 to 3100 for 10 of 5 M, 95 % zeros.)
 CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
   uint32_t g = 0;
   while (((nb - 1) >> g) + 1 > kRankCoarse) ++g;
@@ -220,7 +221,7 @@ CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
   r->split = fullest > kRankBucket ? 1u : 0u;
   uint32_t k = 0;
   while ((fullest >> k) > kRankItems - kRankWindow && (r->n_coarse << (k + 1)) <= kRankSubs && k < 16) ++k;
-  for (int more = 0; r->split && more < 2 && (r->n_coarse << (k + 1)) <= 2048 && k < 16; ++more) ++k;
+  for (int more = 0; r->split && more < 2 && (r->n_coarse << (k + 1)) <= 512 && k < 16; ++more) ++k;
   r->sub_bits = k;
   r->wide = fullest >= (1u << 24) ? 1u : 0u;
 }
