@@ -26,6 +26,7 @@ namespace cvlc {
 
 constexpr int kUfThreads = 128;
 constexpr int kUfWarps = kUfThreads / 32;
+constexpr size_t kUfSharedMax = 200 * 1024;
 constexpr uint32_t kUfCellBits = 9, kUfCells = 1u << kUfCellBits;  // position ranges a block's records are sorted by
 
 // every byte of the output buffers starts at zero: block boundaries share words (they are OR-ed in) and the
@@ -63,37 +64,54 @@ __device__ __forceinline__ void or_ones(uint32_t* img, uint32_t pos, uint32_t co
   }
 }
 
-// One thread block writes one block of records.  They are handed out by a per-client ticket, so every earlier one of the client is
-// being written or done when a thread block looks back for its bit offset.  A block of records takes 13 KB of shared memory (1500-byte
-// packets): with a warp each, four to a thread block, an SM held 16 warps, and the kernel was the chain of one.  Between events, us: 8 clients of
-// 1.2 M coordinates at 2 bits 38.0 -> 29.1, one of 0.75 M at 0.8 29.2 -> 17.8, 60 of 0.3 M at 1 48.3 -> 27.5, 20 of 11.2 M at 2 428 ->
-// 378.  For twelve on an SM (40 registers) a few words are spilled; with nine it is 35.4, 17.2, 33.6 and 443, with sixteen 31.2, 18.9,
-// 32.8 and 364.
-template <bool QSGD>
-__global__ void __launch_bounds__(kUfThreads, 12)
+// A thread block writes one block of records, or each of its four warps writes one.  They are handed out by a per-client ticket, so every
+// earlier one of the client is being written or done when a team looks back for its bit offset.  A block of records takes 13 KB of shared
+// memory (1500-byte packets): with a warp each an SM holds 16 warps, and the kernel is the chain of one; a thread block each finishes
+// sooner wherever all of them are resident at a time.  Short ones are over before four warps' barriers pay: there many warps do it.
+// Between events, a warp and a thread block each, us: 8 clients of 1.2 M coordinates at 2 bits in packets of 1500 / 1000 / 512 / 128 / 24 bytes
+// 37 and 31 / 34 and 36 / 36 and 50 / 76 and 130 / 320 and 614; one client of 0.3 M 31 and 18 / 27 and 18 / 21 and 17 / 23 and 19 / 25 and
+// 31; 4 of 0.6 M in packets of 512 / 376 / 256 bytes (1171, 1595, 2343 blocks) 25 and 22 / 25 and 22 / 28 and 30.  For twelve thread blocks on
+// an SM (40 registers) a few words are spilled; with nine 8 clients of 1.2 M take 35.4 instead of 29.1, with sixteen 31.2.
+constexpr uint64_t kUfTeamBlocks = 12 * kNumSM;   // blocks of records up to which all are resident, a thread block each
+constexpr uint32_t kUfTeamRecords = 16;           // of a block, at least
+constexpr size_t kUfTeamBytes = 11 * 1024;        // shared memory of one from which on an SM holds fewer than 20 warps
+inline bool uf_team(uint64_t blocks, uint32_t records, size_t bytes) {
+  return (blocks <= kUfTeamBlocks && records >= kUfTeamRecords) || bytes > kUfTeamBytes;
+}
+
+template <bool QSGD, int TEAM>
+__global__ void __launch_bounds__(kUfThreads, TEAM == 1 ? 8 : 12)
 k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned char* enc_ws,
-                const __grid_constant__ EncLayout L, unsigned char* uf_ws, uint32_t P_max, uint32_t img_words,
+                const __grid_constant__ EncLayout L, unsigned char* uf_ws, uint32_t P_max, uint32_t img_words, uint32_t team_bytes,
                 unsigned long long* __restrict__ sizes_out) {
-  extern __shared__ __align__(16) unsigned char s_uf[];
+  extern __shared__ __align__(16) unsigned char s_uf[];  // per block of records
   __shared__ int s_err;
-  __shared__ uint32_t s_ticket, s_low[kUfWarps], s_high[kUfWarps], s_full[kUfWarps], s_sum[kUfWarps], s_len[2][kUfWarps];
-  __shared__ float s_lo[kUfWarps], s_hi[kUfWarps];
-  __shared__ unsigned long long s_run;
+  // across the warps of a team
+  [[maybe_unused]] __shared__ uint32_t s_ticket, s_low[TEAM], s_high[TEAM], s_full[TEAM], s_sum[TEAM], s_len[2][TEAM];
+  [[maybe_unused]] __shared__ float s_lo[TEAM], s_hi[TEAM];
+  [[maybe_unused]] __shared__ unsigned long long s_run;
+  static_assert(TEAM == 1 || TEAM == kUfWarps, "a warp or the thread block for a block of records");
+  constexpr uint32_t STEP = TEAM * 32;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(enc_ws);
   const uint32_t c = blockIdx.y;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tid = TEAM == 1 ? (uint32_t)lane : threadIdx.x;  // thread of the team
+  auto sync = [] {
+    if constexpr (TEAM == 1) __syncwarp();
+    else __syncthreads();
+  };
+  uint32_t* ticket = reinterpret_cast<uint32_t*>(uf_ws + uf_off_ticket()) + c;
   if (threadIdx.x == 0) {
     s_err = *reinterpret_cast<const volatile int32_t*>(&hdr->status);
-    s_ticket = atomicAdd(reinterpret_cast<uint32_t*>(uf_ws + uf_off_ticket()) + c, 1u);
+    if (TEAM > 1) s_ticket = atomicAdd(ticket, 1u);
   }
   __syncthreads();
   if (s_err != 0) return;
-  const uint32_t tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
   const ClientDesc cd = batch.c[c];
   const cvlc_plan_t* __restrict__ plan = cd.plan;
   const uint32_t R = shape.R;
-  unsigned long long* rec = reinterpret_cast<unsigned long long*>(s_uf);     // [P_max] position << 32 | value bits
+  unsigned long long* rec = reinterpret_cast<unsigned long long*>(s_uf + (TEAM == 1 ? (size_t)warp * team_bytes : 0));  // [P_max] position << 32 | value bits
   unsigned long long* by_cell = rec + P_max;                                // [P_max] the records by their cells
   double* sqv = reinterpret_cast<double*>(by_cell);                         // QSGD: before that the squares of the values
   uint32_t* cell = reinterpret_cast<uint32_t*>(by_cell + P_max);            // [kUfCells]
@@ -134,7 +152,15 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     }
   }
 
-  const uint32_t r = s_ticket;  // below R: the client has R thread blocks
+  uint32_t r;
+  if constexpr (TEAM == 1) {
+    r = 0;
+    if (lane == 0) r = atomicAdd(ticket, 1u);
+    r = __shfl_sync(kFull, r, 0);
+    if (r >= R) return;
+  } else {
+    r = s_ticket;  // below R: the client has R thread blocks
+  }
   const unsigned hit = __ballot_sync(kFull, r < cum);
   const int src_lane = __ffs(hit) - 1;
   const uint32_t y = CVLC_MAX_CODE_BITS - (uint32_t)src_lane;
@@ -147,7 +173,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
   // ---- the block's records and its centroid distribution (over the records in rank order, as for a packet)
   float vmin = CUDART_INF_F, vmax = -CUDART_INF_F;
   uint32_t pmin = 0xFFFFFFFFu, pmax = 0u;
-  for (uint32_t j = tid; j < P; j += kUfThreads) {
+  for (uint32_t j = tid; j < P; j += STEP) {
     const unsigned long long pair = seg[j];
     const uint32_t key = (uint32_t)(pair >> 32), pid = (uint32_t)pair & 0x7FFFFFFFu;
     const uint32_t b = key ? (key | ((uint32_t)pair & 0x80000000u)) : 0u;  // -0 is stored as +0
@@ -172,75 +198,100 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, off));
     }
   }
-  if (lane == 0) {
+  if (TEAM > 1 && lane == 0) {
     s_low[warp] = pmin;
     s_high[warp] = pmax;
     s_lo[warp] = vmin;
     s_hi[warp] = vmax;
   }
-  for (uint32_t i = tid; i < kUfCells; i += kUfThreads) cell[i] = 0u;
-  for (uint32_t w = tid; w < img_words + 2; w += kUfThreads) img[w] = 0u;
-  __syncthreads();
+  for (uint32_t i = tid; i < kUfCells; i += STEP) cell[i] = 0u;
+  for (uint32_t w = tid; w < img_words + 2; w += STEP) img[w] = 0u;
+  sync();
+  if constexpr (TEAM > 1) {
 #pragma unroll
-  for (int w = 0; w < kUfWarps; ++w) {
-    pmin = min(pmin, s_low[w]);
-    pmax = max(pmax, s_high[w]);
+    for (int w = 0; w < TEAM; ++w) {
+      pmin = min(pmin, s_low[w]);
+      pmax = max(pmax, s_high[w]);
+    }
   }
   float lo, hi;
   if constexpr (QSGD) {
-    if (tid == 0) s_lo[0] = qsgd_norm_of_squares(sqv, P);
-    __syncthreads();
-    lo = s_lo[0];
+    lo = 0.0f;
+    if (tid == 0) lo = qsgd_norm_of_squares(sqv, P);
+    if constexpr (TEAM == 1) {
+      lo = __shfl_sync(kFull, lo, 0);
+    } else {
+      if (tid == 0) s_lo[0] = lo;
+      sync();
+      lo = s_lo[0];
+    }
     hi = 0.0f;
   } else {
     lo = vmin;
     hi = vmax;
+    if constexpr (TEAM > 1) {
 #pragma unroll
-    for (int w = 0; w < kUfWarps; ++w) {
-      lo = fminf(lo, s_lo[w]);
-      hi = fmaxf(hi, s_hi[w]);
+      for (int w = 0; w < TEAM; ++w) {
+        lo = fminf(lo, s_lo[w]);
+        hi = fmaxf(hi, s_hi[w]);
+      }
     }
   }
 
   // ---- ascending position: the records are spread over kUfCells equal ranges of the block's positions, a few in each, and
   // compared with the others of their cell.  Where the positions crowd into few cells, a bitonic network sorts them instead.
   const uint32_t csh = (pmax - pmin) < kUfCells ? 0u : 32u - __clz(pmax - pmin) - kUfCellBits;  // (pmax - pmin) >> csh < kUfCells
-  for (uint32_t j = tid; j < P; j += kUfThreads) atomicAdd(cell + (((uint32_t)(rec[j] >> 32) - pmin) >> csh), 1u);
-  __syncthreads();
+  for (uint32_t j = tid; j < P; j += STEP) atomicAdd(cell + (((uint32_t)(rec[j] >> 32) - pmin) >> csh), 1u);
+  sync();
   uint32_t fullest;
   {
-    static_assert(kUfCells == 4 * kUfThreads, "four cells a thread");
-    uint4* mine = reinterpret_cast<uint4*>(cell) + tid;
-    const uint4 v = *mine;
-    const uint32_t sum = v.x + v.y + v.z + v.w;
-    fullest = __reduce_max_sync(kFull, max(max(v.x, v.y), max(v.z, v.w)));
+    constexpr uint32_t kMine = kUfCells / STEP / 4;  // a thread's cells, by fours
+    uint4* mine = reinterpret_cast<uint4*>(cell) + tid * kMine;
+    uint4 v[kMine];
+    uint32_t sum = 0;
+    fullest = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < kMine; ++i) {
+      v[i] = mine[i];
+      sum += v[i].x + v[i].y + v[i].z + v[i].w;
+      fullest = max(fullest, max(max(v[i].x, v[i].y), max(v[i].z, v[i].w)));
+    }
+    fullest = __reduce_max_sync(kFull, fullest);
     uint32_t run = sum;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const uint32_t o = __shfl_up_sync(kFull, run, off);
       if (lane >= off) run += o;
     }
-    if (lane == 31) {
-      s_sum[warp] = run;
-      s_full[warp] = fullest;
+    if constexpr (TEAM > 1) {
+      if (lane == 31) {
+        s_sum[warp] = run;
+        s_full[warp] = fullest;
+      }
+      sync();
     }
-    __syncthreads();
     run -= sum;
+    if constexpr (TEAM > 1) {
 #pragma unroll
-    for (int w = 0; w < kUfWarps; ++w) {
-      if (w < warp) run += s_sum[w];
-      fullest = max(fullest, s_full[w]);
+      for (int w = 0; w < TEAM; ++w) {
+        if (w < warp) run += s_sum[w];
+        fullest = max(fullest, s_full[w]);
+      }
     }
-    *mine = make_uint4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
+#pragma unroll
+    for (uint32_t i = 0; i < kMine; ++i) {
+      mine[i] = make_uint4(run, run + v[i].x, run + v[i].x + v[i].y, run + v[i].x + v[i].y + v[i].z);
+      run += v[i].x + v[i].y + v[i].z + v[i].w;
+    }
   }
-  __syncthreads();
+  sync();
   if (fullest <= 64) {
-    for (uint32_t j = tid; j < P; j += kUfThreads) {
+    for (uint32_t j = tid; j < P; j += STEP) {
       const unsigned long long e = rec[j];
       by_cell[atomicAdd(cell + (((uint32_t)(e >> 32) - pmin) >> csh), 1u)] = e;
     }
-    __syncthreads();
-    for (uint32_t j = tid; j < P; j += kUfThreads) {
+    sync();
+    for (uint32_t j = tid; j < P; j += STEP) {
       const unsigned long long e = by_cell[j];
       const uint32_t k = ((uint32_t)(e >> 32) - pmin) >> csh;
       const uint32_t q0 = k ? cell[k - 1] : 0u, q1 = cell[k];  // the places have advanced to the cells' ends
@@ -248,7 +299,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       for (uint32_t q = q0; q < q1; ++q) rank += by_cell[q] < e ? 1u : 0u;
       rec[rank] = e;
     }
-    __syncthreads();
+    sync();
   } else {
     // comparators that all point the same way: places behind the last record need none
     uint32_t size = 2;
@@ -256,7 +307,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     for (uint32_t k = 2; k <= size; k <<= 1) {
       for (uint32_t jj = k >> 1; jj > 0; jj >>= 1) {
         const uint32_t flip = (jj == k >> 1) ? k - 1 : jj;  // first step of a merge: against the mirror image
-        for (uint32_t t = tid; t < size / 2; t += kUfThreads) {
+        for (uint32_t t = tid; t < size / 2; t += STEP) {
           const uint32_t i = ((t & ~(jj - 1)) << 1) | (t & (jj - 1)), p = i ^ flip;
           if (p < P) {
             const unsigned long long x = rec[i], z = rec[p];
@@ -266,7 +317,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
             }
           }
         }
-        __syncthreads();
+        sync();
       }
     }
   }
@@ -276,7 +327,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     img[0] = __float_as_uint(lo);
     img[1] = __float_as_uint(hi);
   }
-  __syncthreads();
+  sync();
   const double Lc = (double)((1ull << y) - 1ull);
   const double dlo = (double)lo;
   const double den = __dsub_rn((double)hi, dlo);
@@ -286,7 +337,7 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
   const double q_scale = (QSGD && lo > 0.0f) ? __ddiv_rn(sqd, dn) : 0.0;
   const float fscale = QSGD ? fast_scale(q_scale, y - 1) : fast_scale(pq_scale, y);
   uint32_t carry = 64;
-  for (uint32_t base = 0; base < P; base += kUfThreads) {
+  for (uint32_t base = 0; base < P; base += STEP) {
     const uint32_t j = base + tid;
     const bool valid = j < P;
     uint32_t len = 0, quo = 0;
@@ -319,27 +370,31 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
       const uint32_t o = __shfl_up_sync(kFull, incl, off);
       if (lane >= off) incl += o;
     }
-    uint32_t* sums = s_len[(base / kUfThreads) & 1];  // the last but one's have been read: a barrier lies between
-    if (lane == 31) sums[warp] = incl;
-    __syncthreads();
-    if (valid) {
-      uint32_t pos = carry + incl - len;
+    uint32_t pos = carry + incl - len;
+    if constexpr (TEAM == 1) {
+      carry += __shfl_sync(kFull, incl, 31);
+    } else {
+      uint32_t* sums = s_len[(base / STEP) & 1];  // the last but one's have been read: a barrier lies between
+      if (lane == 31) sums[warp] = incl;
+      sync();
 #pragma unroll
-      for (int w = 0; w < kUfWarps; ++w)
+      for (int w = 0; w < TEAM; ++w) {
         if (w < warp) pos += sums[w];
+        carry += sums[w];
+      }
+    }
+    if (valid) {
       or_ones(img, pos, quo);
       or_bits(img, pos + quo, tail);
     }
-#pragma unroll
-    for (int w = 0; w < kUfWarps; ++w) carry += sums[w];
   }
-  __syncthreads();
+  sync();
   const uint32_t block_bits = carry;
 
   // ---- bit offset of the block: decoupled look-back over the client's earlier blocks, 32 at a time, by one warp
   if (tid == 0) st_relaxed(state + r, (r == 0 ? kFlagPrefix : kFlagAgg) | block_bits);
   unsigned long long run = 0;
-  if (r > 0 && warp == 0) {
+  if (r > 0 && (TEAM == 1 || warp == 0)) {
     long long top = (long long)r - 1;
     while (true) {
       const long long idx = top - lane;
@@ -359,18 +414,20 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     }
     if (lane == 0) {
       st_relaxed(state + r, kFlagPrefix | (run + block_bits));
-      s_run = run;
+      if (TEAM > 1) s_run = run;
     }
   }
-  __syncthreads();
-  if (r > 0) run = s_run;
+  if constexpr (TEAM > 1) {
+    sync();
+    if (r > 0) run = s_run;
+  }
 
   // ---- the image goes out shifted to its bit offset; the first and the last word are shared with the neighbours
   {
     const uint32_t shift = (uint32_t)(run & 31ull);
     const size_t w0 = (size_t)(run >> 5);
     const uint32_t n_out = (shift + block_bits + 31) >> 5;
-    for (uint32_t ow = tid; ow < n_out; ow += kUfThreads) {
+    for (uint32_t ow = tid; ow < n_out; ow += STEP) {
       uint32_t v = img[ow] << shift;  // img has two zero words behind its last used one
       if (shift && ow) v |= img[ow - 1] >> (32 - shift);
       if (ow == 0 || ow == n_out - 1) {
@@ -390,8 +447,8 @@ k_pack_unframed(const Batch batch, const __grid_constant__ Shape shape, unsigned
     }
   }
 
-  // ---- stream header and the tables of lengths, by the thread block that wrote block 0
-  if (r == 0 && warp == 0) {
+  // ---- stream header and the tables of lengths, by the first warp of the team that wrote block 0
+  if (r == 0 && (TEAM == 1 || warp == 0)) {
     if (lane < 16) {
       uint32_t v = 0;
       const unsigned long long Bbits = (unsigned long long)__double_as_longlong(cd.scale_B);
@@ -430,8 +487,10 @@ cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capaci
                                  size_t stream_capacity, void* enc_ws, void* uf_ws, unsigned long long* sizes_out, cudaStream_t st) {
   static OncePerDevice once;
   const cudaError_t e = once_per_device(once, [] {
-    const cudaError_t e = allow_shared(k_pack_unframed<false>, 200 * 1024);
-    return e != cudaSuccess ? e : allow_shared(k_pack_unframed<true>, 200 * 1024);
+    cudaError_t e = allow_shared(k_pack_unframed<false, 1>, kUfSharedMax);
+    if (e == cudaSuccess) e = allow_shared(k_pack_unframed<true, 1>, kUfSharedMax);
+    if (e == cudaSuccess) e = allow_shared(k_pack_unframed<false, kUfWarps>, kUfSharedMax);
+    return e != cudaSuccess ? e : allow_shared(k_pack_unframed<true, kUfWarps>, kUfSharedMax);
   });
   if (e != cudaSuccess) return e;
   const EncLayout L = enc_layout(shape.d, n, capacity);
@@ -451,8 +510,12 @@ cudaError_t launch_pack_unframed(uint32_t n, const Shape& shape, uint64_t capaci
   const size_t block_bytes = (size_t)P_max * 16 + ((((size_t)img_words + 2 + kUfCells) * 4 + 15) & ~(size_t)15);
   launch_kernel(kKZeroWords, k_uf_clear, 4 * kNumSM, 256, 0, st, true, batch, stream_capacity / 16, static_cast<unsigned char*>(uf_ws),
                 uf_ws_bytes(n, shape.R) / 4);
-  launch_kernel(kKPackUnframed, qsgd ? k_pack_unframed<true> : k_pack_unframed<false>, dim3(shape.R, n), kUfThreads, block_bytes, st, true,
-                batch, shape, static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), P_max, img_words, sizes_out);
+  const bool team = uf_team((uint64_t)shape.R * n, P_max, block_bytes);
+  auto kernel = team ? (qsgd ? k_pack_unframed<true, kUfWarps> : k_pack_unframed<false, kUfWarps>)
+                     : (qsgd ? k_pack_unframed<true, 1> : k_pack_unframed<false, 1>);
+  const uint32_t at_work = team ? 1 : kUfWarps;  // blocks of records of a thread block
+  launch_kernel(kKPackUnframed, kernel, dim3((shape.R + at_work - 1) / at_work, n), kUfThreads, block_bytes * at_work, st, true, batch, shape,
+                static_cast<unsigned char*>(enc_ws), L, static_cast<unsigned char*>(uf_ws), P_max, img_words, (uint32_t)block_bytes, sizes_out);
   return cudaGetLastError();
 }
 
