@@ -1155,12 +1155,15 @@ k_sort_pass(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
 constexpr int kPackThreads = 128;
 constexpr int kPackWarps = kPackThreads / 32;
 constexpr int kPackGroup = 1;  // packets per warp (more of them amortise the length table but lengthen the tail)
-// Packets of a batch up to which a block works on one, about those that are resident at a time (9 blocks per SM).  Kernel with a warp
-// and with the block for a packet, us, one / 24 clients: 500 packets 16.5 and 12.1 / 14.5 and 12.3, 1000 16.2 and 12.2 / 15.9 and
-// 13.4, 1500 17.4 and 14.4 / 16.3 and 16.2, 2000 18.2 and 16.1 / 16.8 and 18.0, 3000 20.3 and 20.3 / 19.4 and 22.2.  With QSGD, whose
-// norm is one lane's chain in both, 500 16.3 and 12.9 / 17.3 and 13.9, 1000 16.2 and 14.1 / 20.1 and 16.0, 1500 18.2 and 18.3 / 21.2 and
-// 20.4, 2000 18.5 and 20.2 / 22.4 and 22.4.
-constexpr uint64_t kTeamPackets = 13 * kNumSM, kTeamPacketsQsgd = 9 * kNumSM;
+// A block works on a packet where all of them are resident at a time (9 blocks per SM) and have records for its threads; with packets of
+// 4.5 KB and more up to a half beyond that.  Block minus warp for a packet, whole encoding calls of one client, us, at 200 / 600 / 1000 /
+// 1332 / 1500 / 1924 packets of 1500 bytes -1.8 / -0.8 / -0.1 / 0 / +1.2 / +2.1 (QSGD, whose norm is one lane's chain in both: -2.1 / -3.6
+// / -2.0 / -1.4 / +2.7 / +1.9), of 752 bytes -0.7 / -0.9 / -0.2 / -1.1 / +2.0 / +2.1, of 256 bytes 0 / +0.1 / +0.4 / +0.8 / +2.0 / +2.1 (QSGD
+// -0.8 / -0.3 / -0.6 / -0.9 / +1.9 / +2.0), of 32 bytes -0.2 / +0.8 / +0.2 / +0.1 / +2.1 / +2.1; at 1332 / 1700 / 1924 / 2300 packets of 3000
+// bytes -1.1 / +0.9 / +0.3 / +0.1, of 4500 -7.2 / +0.1 / -3.8 / -1.4 (8 clients -6.3 / -4.9 / -5.1 / -3.5).
+inline bool pack_team(uint64_t packets, bool qsgd, uint32_t records, size_t packet_bytes) {
+  return records >= (qsgd ? 48u : 128u) && packets <= (!qsgd && packet_bytes >= 4500 ? 13u : 9u) * (uint64_t)kNumSM;
+}
 
 template <int CAP, bool QSGD, int TEAM>
 __global__ void __launch_bounds__(kPackThreads)
@@ -1457,7 +1460,7 @@ template <int CAP>
 static cudaError_t launch_pack_t(const ClientDesc* clients, uint32_t n, const Shape& shape, const EncLayout& L, unsigned char* w, size_t warp_bytes,
                                  int write_residual, cudaStream_t st, bool overlap) {
   const bool qsgd = shape.quantizer == CVLC_QUANT_QSGD;
-  const bool team = (uint64_t)shape.R * n <= (qsgd ? kTeamPacketsQsgd : kTeamPackets);
+  const bool team = pack_team((uint64_t)shape.R * n, qsgd, shape.cap[1], shape.packet_bits / 8);
   auto kernel = team ? (qsgd ? k_pack<CAP, true, kPackWarps> : k_pack<CAP, false, kPackWarps>) : (qsgd ? k_pack<CAP, true, 1> : k_pack<CAP, false, 1>);
   const uint32_t at_work = team ? 1 : kPackWarps;  // packets of a block
   BatchDesc<CAP> batch;

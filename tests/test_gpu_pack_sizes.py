@@ -1,5 +1,6 @@
-"""GPU parity of few large packets whose assembly takes just below or above 48 KB of shared memory, what a kernel gets unasked (its
-static part counted).  Every size is the first call of a process of its own: what an earlier call has asked for stays allowed."""
+"""GPU parity of the packing over packet sizes.  Few large packets whose assembly takes just below or above 48 KB of shared memory, what a
+kernel gets unasked (its static part counted): every size is the first call of a process of its own, since what an earlier call has
+asked for stays allowed.  And sizes at the lines between a block and a warp for a packet."""
 import multiprocessing as mp
 
 import numpy as np
@@ -45,3 +46,20 @@ def test_first_call_with_large_packets(quantizer, packet_bytes):
     finally:
         p.join(timeout=60)
     assert got == (0, True)
+
+
+SMS = 148
+
+
+@pytest.mark.parametrize("quantizer,packet_bits,R,d", [
+    (0, 1_824, 3, 8_000), (0, 1_888, 3, 8_000), (1, 736, 3, 8_000), (1, 768, 3, 8_000),              # 124 to 135, 46 to 49 records
+    (0, 2_080, 9 * SMS, 200_003), (0, 2_528, 9 * SMS, 200_003), (0, 2_528, 9 * SMS + 1, 200_003),    # few and enough records
+    (0, 35_968, 9 * SMS + 1, 6_000_001), (0, 36_000, 9 * SMS + 1, 6_000_001),                        # 4496 and 4500 bytes
+    (0, 36_000, 13 * SMS, 6_000_001), (0, 36_000, 13 * SMS + 1, 6_000_001)])
+def test_block_or_warp_for_a_packet(quantizer, packet_bits, R, d):
+    from gpu_util import gpu_plan_encode
+    x = np.random.default_rng(packet_bits + R).laplace(0, 1e-3, d).astype(np.float32)
+    pd = params_dict(d, R * packet_bits, packet_bits=packet_bits, quantizer=quantizer, seed=4)
+    status, _, out = gpu_plan_encode(x, pd)
+    assert status == 0
+    assert np.array_equal(out, oracle_plan_encode(x, pd)[1])
