@@ -32,3 +32,24 @@ def test_a_dense_layer_anywhere(d, n, layer):
     assert enc.status() == B.CVLC_OK
     for x, pd, out in list(zip(xs, pds, outs))[:2]:
         assert np.array_equal(out.cpu().numpy(), oracle_plan_encode(x, pd)[1])
+
+
+@pytest.mark.parametrize("d,n,bits", [(11_800_003, 32, 1.0), (100_000_003, 10, 0.25)])
+def test_groups_of_three_sizes(d, n, bits):
+    """367 M coordinates and more in at most 32 clients: groups of many pieces, of a quarter as many and of single pieces, spread over a
+    client each (8 and 2 pieces of 128 rows, or 21 and 5).  The clients are the same one, so that the oracle runs once."""
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal(d, dtype=np.float32)
+    for q in range(16):  # layers of different scales, so that rows differ in how many candidates they hold
+        x[q * d // 16:(q + 1) * d // 16] *= np.float32(10.0 ** -rng.uniform(0, 2))
+    pd = params_dict(d, int(bits * d), seed=n)
+    most = 3 * (int(bits * d) // 12_000) * ((12_000 - 80) // (int(d - 1).bit_length() + 1))
+    dev = torch.device("cuda:0")
+    enc = B.BatchEncoder([gpu_params(pd)] * n, dev, max_candidates=most)
+    outs = enc.compress([torch.from_numpy(x).to(dev)] * n, side_stream=torch.cuda.Stream(dev))
+    assert enc.status() == B.CVLC_OK
+    stream = torch.from_numpy(oracle_plan_encode(x, pd)[1]).to(dev)
+    for out in outs:
+        assert torch.equal(out, stream)
