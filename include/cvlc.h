@@ -230,7 +230,9 @@ int cvlc_plan_literal(const cvlc_params* p, double alpha_q, uint32_t n_k, uint32
  * = Philox4x32-10 of the coordinate index) and packs (position ID, centroid ID) pairs
  * behind the packet header (Fig. 2).
  * stream_dev (16-byte aligned) receives cvlc_stream_bytes(p) bytes.
- * plan_dev must come from cvlc_plan / cvlc_plan_fixed on the same x_dev and params.
+ * plan_dev must come from cvlc_plan / cvlc_plan_fixed on the same x_dev and params.  Another update
+ * is reported (PLAN_MISMATCH) where the counts of its candidates differ; with the plan's workspace those
+ * are the coordinates from the histogram bin of rank k on, and what differs below it is not sent either way.
  * plan_ws_dev: the workspace that call used, untouched since (it holds where the candidates
  * of every histogram bin start, so that the selection can put them into value buckets, and the
  * bin of the largest key of every 16 coordinates, so that only those that hold a candidate are

@@ -99,8 +99,6 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
   uint64_t grid = (P.total + 255) / 256;
   if (grid > most) grid = most;
   P.grid = (uint32_t)grid;
-  // two chunks per block where that leaves each a megabyte and more: every chunk ends with a merge into a client's histogram
-  // (with two of 64 KB and more 10 clients of 5 M coordinates take 53 us)
   P.per_client = 0;
   const uint64_t of_client = grid / n;
   if (P.total <= (8u << 20) && of_client * n * 16 >= grid * 15) {
@@ -110,6 +108,8 @@ CVLC_HD inline Partition make_partition(uint64_t d, uint32_t n) {
     P.n_chunks = P.grid = P.per_client * n;
     return P;
   }
+  // two chunks per block where that leaves each a megabyte and more: every chunk ends with a merge into a client's histogram
+  // (with two of 64 KB and more 10 clients of 5 M coordinates take 53 us)
   const uint64_t n_chunks = P.total / (2 * grid) >= 16384 ? 2 * grid : grid;
   P.chunk = ((P.total + n_chunks - 1) / n_chunks + 15) & ~(uint64_t)15;
   P.n_chunks = (uint32_t)((P.total + P.chunk - 1) / P.chunk);

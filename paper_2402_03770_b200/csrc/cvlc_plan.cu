@@ -1,6 +1,6 @@
-// Planning kernels: magnitude histogram (Algorithm 1, step 1), the exponent fit of Definition 1 with the
-// selection threshold, and the code-length tuning by atomic operations on Eq. (5) (Algorithm 1 steps 2-14),
-// one CTA per client, run once per distinct (exponent, scale) of a batch.
+// Planning kernels: magnitude histogram (Algorithm 1, step 1) with the selection threshold, the exponent fit of
+// Definition 1, and the code-length tuning by atomic operations on Eq. (5) (Algorithm 1 steps 2-14), one CTA per
+// client or, in larger batches, per distinct (exponent, scale).
 //
 // The planner's floating point is IEEE binary64 with every multiply and add
 // rounded separately (the *_rn intrinsics keep the compiler from contracting
@@ -81,8 +81,8 @@ __device__ __forceinline__ double energy_E(uint64_t Z, double beta, double D) {
 constexpr int kPlanThreads = 512;  // of the blocks that work on one client's histogram: that of the histogram, the fit's, the tuning's
 constexpr int kPlanBins = CVLC_HIST_BINS / kPlanThreads;
 constexpr size_t kSurvivalBytes = (CVLC_HIST_BINS + 4) * 4;  // survival counts in shared memory
-// The tuning kernel decides most atomic operations with four warps (see FastLane below); all of them fit the exponent and evaluate
-// what is left to the series arithmetic.
+// The tuning kernel settles neighbouring lengths with one warp and looks at all pairs with all but one (see FastLane below); all of its
+// warps fit the exponent and evaluate what is left to the series arithmetic.
 constexpr int kTuneThreads = 512;
 constexpr int kTuneWarps = kTuneThreads / 32;
 constexpr int kPlanItems = 1024;
@@ -101,7 +101,6 @@ struct PlanOp {                   // one atomic operation of a batch
   unsigned char slot_lane[32];    // those lengths, longest first
 };
 struct PlanSolver {
-  double Ecur[32];                // E(W_l) of the current counts
   double Fpre[33];                // running sum of F after length l (index 32: nothing yet)
   double Eab[33];                 // energy of the nearest used length at or above l
   unsigned long long Wc[32];      // ranks covered by lengths >= l, current counts
@@ -124,7 +123,7 @@ struct PlanShared {
   double D;
 };
 
-// candidate lengths of one client and their coefficients (Eq. (5)), built by warp 0
+// candidate lengths of one client and their coefficients (Eq. (5)): g(y) > 0 (the paper's B > (Q+1)/2) and not dominated
 struct PlanTab {
   uint64_t d;
   uint32_t s, R, nY, y_min, fixed_y;
@@ -134,14 +133,8 @@ struct PlanTab {
   double QY[32];      // PQ error factor Q(Y[i]) = cap / (2^y - 1)^2
 };
 
-// Candidate lengths: g(y) > 0 (the paper's B > (Q+1)/2) and not dominated; called by one full warp, lane = length - 1.
-struct PlanLength {
-  unsigned member;      // bit y - 1: length y is a candidate
-  uint32_t cap, y_min;  // of this lane's length; shortest usable length
-  double g, Q;          // of this lane's length
-};
-__device__ __forceinline__ PlanLength plan_lengths(const Shape& shape, double B, int lane) {
-  PlanLength P;
+// by one full warp, lane = length - 1
+__device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, double B, int lane) {
   const uint32_t y = lane + 1;
   const bool in_range = y <= shape.max_code_bits;
   const uint32_t cap_y = in_range ? shape.cap[y] : 0u;
@@ -158,20 +151,33 @@ __device__ __forceinline__ PlanLength plan_lengths(const Shape& shape, double B,
   }
   const double one_m = __dsub_rn(1.0, __ddiv_rn(1.0, B));
   const double g = __dsub_rn(1.0, __dadd_rn(__ddiv_rn(Q, __dmul_rn(B, B)), __dmul_rn(one_m, one_m)));
+  unsigned member;  // bit y - 1: length y is a candidate
+  uint32_t y_min;
   if (shape.fixed_y) {
-    P.y_min = shape.fixed_y;
-    P.member = 1u << (shape.fixed_y - 1);
+    y_min = shape.fixed_y;
+    member = 1u << (shape.fixed_y - 1);
   } else {
     const unsigned pos = __ballot_sync(kFull, in_range && g > 0.0);
-    P.y_min = pos ? (uint32_t)__ffs(pos) : 1u;  // the host has checked that one exists
+    y_min = pos ? (uint32_t)__ffs(pos) : 1u;  // the host has checked that one exists
     const uint32_t cap_next = __shfl_down_sync(kFull, cap_y, 1);
-    const bool keep = in_range && y >= P.y_min && (y == shape.max_code_bits || cap_y > cap_next);
-    P.member = __ballot_sync(kFull, keep);
+    const bool keep = in_range && y >= y_min && (y == shape.max_code_bits || cap_y > cap_next);
+    member = __ballot_sync(kFull, keep);
   }
-  P.cap = cap_y;
-  P.g = g;
-  P.Q = Q;
-  return P;
+  if (member & (1u << lane)) {
+    const int i = __popc(member & ((1u << lane) - 1u));
+    T.Y[i] = y;
+    T.capY[i] = cap_y;
+    T.gY[i] = g;
+    T.QY[i] = Q;
+  }
+  if (lane == 0) {
+    T.d = shape.d;
+    T.s = shape.s;
+    T.R = shape.R;
+    T.nY = (uint32_t)__popc(member);
+    T.y_min = y_min;
+    T.fixed_y = shape.fixed_y;
+  }
 }
 // zeroes two ranges of the workspace and leaves the clients' descriptors in it
 template <int CAP>
@@ -182,26 +188,6 @@ k_zero_words(const __grid_constant__ BatchDesc<CAP> batch, ClientDesc* desc, uin
   for (size_t i = first; i < batch.n; i += stride) desc[i] = batch.c[i];
   for (size_t i = first; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
   for (size_t i = first; i < m16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// the table of one client's candidate lengths, by one full warp
-__device__ __forceinline__ void build_plan_tab(PlanTab& T, const Shape& shape, double B, int lane) {
-  const PlanLength P = plan_lengths(shape, B, lane);
-  if (P.member & (1u << lane)) {
-    const int i = __popc(P.member & ((1u << lane) - 1u));
-    T.Y[i] = lane + 1;
-    T.capY[i] = P.cap;
-    T.gY[i] = P.g;
-    T.QY[i] = P.Q;
-  }
-  if (lane == 0) {
-    T.d = shape.d;
-    T.s = shape.s;
-    T.R = shape.R;
-    T.nY = (uint32_t)__popc(P.member);
-    T.y_min = P.y_min;
-    T.fixed_y = shape.fixed_y;
-  }
 }
 
 // ---- what a client's histogram gives, by a block of kPlanThreads threads ------------------------
@@ -800,46 +786,43 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   // ---- objective bookkeeping -----------------------------------------------------------
   // F(n) = 1 - gamma of Eq. (5) is a running sum over the used lengths, longest first:
   // F += g_l * (E(W_l) - E(W_prev)), W_l = ranks covered down to and including length l.
-  // For the current counts the kernel keeps, per candidate index l: the energy E(W_l)
-  // (Q.Ecur), the running sum after length l (Q.Fpre) and the energy of the nearest used
-  // length at or above l (Q.Eab).  An atomic operation on the lengths i > j leaves everything
-  // above i untouched, so a trial split only needs E for the used lengths at or below i and
-  // continues the running sum from Q.Fpre[i + 1]: the same operations in the same order as a
-  // full evaluation, on a fraction of the lanes.
+  // For the current counts the kernel keeps, per candidate index l: the running sum after
+  // length l (Q.Fpre) and the energy of the nearest used length at or above l (Q.Eab).  An
+  // atomic operation on the lengths i > j leaves everything above i untouched, so a trial split
+  // only needs E for the used lengths at or below i and continues the running sum from
+  // Q.Fpre[i + 1]: the same operations in the same order as a full evaluation, on a fraction of
+  // the lanes.
   PlanSolver& Q = *reinterpret_cast<PlanSolver*>(smem_raw);
 
   auto refresh_warp = [&]() {  // by one warp
-    {
-      const uint32_t my_n = (lane < nY) ? S.n[lane] : 0u;
-      uint64_t W = (uint64_t)my_n * my_cap;
+    const uint32_t my_n = (lane < nY) ? S.n[lane] : 0u;
+    uint64_t W = (uint64_t)my_n * my_cap;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint64_t o = __shfl_down_sync(kFull, W, off);
-        if (lane + off < 32) W += o;
-      }
-      const double E = (my_n > 0) ? energy_E(W, beta, D) : 0.0;
-      const unsigned used = __ballot_sync(kFull, my_n > 0);
-      // the terms side by side, their sum in the order of the lengths
-      const unsigned above = lane < 31 ? used & (kFull << (lane + 1)) : 0u;
-      const double Eup = __shfl_sync(kFull, E, above ? __ffs(above) - 1 : 0);
-      const double Eprev = above ? Eup : 0.0;
-      const double term = (my_n > 0) ? __dmul_rn(T.gY[lane], __dsub_rn(E, Eprev)) : 0.0;
-      double F = 0.0, Fmine = 0.0;
-      for (unsigned rest = used; rest;) {
-        const int l = 31 - __clz(rest);
-        rest ^= 1u << l;
-        F = __dadd_rn(F, __shfl_sync(kFull, term, l));
-        if (lane <= l) Fmine = F;
-      }
-      Q.Ecur[lane] = E;
-      Q.Wc[lane] = W;
-      Q.Fpre[lane] = Fmine;
-      Q.Eab[lane] = (my_n > 0) ? E : Eprev;
-      if (lane == 0) {
-        Q.used = used;
-        Q.Fpre[32] = 0.0;
-        Q.Eab[32] = 0.0;
-      }
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint64_t o = __shfl_down_sync(kFull, W, off);
+      if (lane + off < 32) W += o;
+    }
+    const double E = (my_n > 0) ? energy_E(W, beta, D) : 0.0;
+    const unsigned used = __ballot_sync(kFull, my_n > 0);
+    // the terms side by side, their sum in the order of the lengths
+    const unsigned above = lane < 31 ? used & (kFull << (lane + 1)) : 0u;
+    const double Eup = __shfl_sync(kFull, E, above ? __ffs(above) - 1 : 0);
+    const double Eprev = above ? Eup : 0.0;
+    const double term = (my_n > 0) ? __dmul_rn(T.gY[lane], __dsub_rn(E, Eprev)) : 0.0;
+    double F = 0.0, Fmine = 0.0;
+    for (unsigned rest = used; rest;) {
+      const int l = 31 - __clz(rest);
+      rest ^= 1u << l;
+      F = __dadd_rn(F, __shfl_sync(kFull, term, l));
+      if (lane <= l) Fmine = F;
+    }
+    Q.Wc[lane] = W;
+    Q.Fpre[lane] = Fmine;
+    Q.Eab[lane] = (my_n > 0) ? E : Eprev;
+    if (lane == 0) {
+      Q.used = used;
+      Q.Fpre[32] = 0.0;
+      Q.Eab[32] = 0.0;
     }
   };
   auto refresh_state = [&]() {  // all threads; ends with a barrier
