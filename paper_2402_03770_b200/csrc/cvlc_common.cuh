@@ -190,6 +190,7 @@ constexpr uint32_t kRankItems = 8192;      // candidates a block of the final ra
 constexpr uint32_t kRankBucket = 4096;     // largest coarse bucket that is ranked without a partition
 constexpr uint32_t kRankWindow = 4096;     // candidates of a tile of the final ranking
 constexpr uint32_t kRankSplitTile = 4096;  // candidates of a tile of the partition
+constexpr uint64_t kRankOneRound = 2ull * kNumSM * kRankSplitTile;  // candidates of a batch up to which a block of the partition has one tile
 struct ClientRank {
   uint32_t n;          // candidates
   uint32_t keytop;     // largest key of the top bin
@@ -202,17 +203,19 @@ struct ClientRank {
   uint32_t thresh_bin; // lowest bin of the candidates: the plan's or, where k is known, the one that holds rank k
   uint32_t pad[3];
 };
-// The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates.  As few
-// sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that a block
-// meets costs the selection a global addition); up to 512 of a client four times as many, since they often lie at one end of it: error
-// compensation leaves the memories crowded below the threshold, in buckets that no block holds (10 clients of 5 M coordinates in a
-// later round 283 -> 256 us), and even tiles are ranked sooner (20 of 1.2 M 121 -> 119, 10 of 1.2 M 78 -> 75, 100 of 1.2 M 423 -> 415).  Not for
-// clients with more, whose partition then writes its 4096 candidates at a time to places of two each: with up to 1024 300 of 3 M take
-// 2549 us instead of 2498, with up to 2048 2632 (partition 392 us instead of 264), and 100 of 11.2 M in layers of different scales 2610
-// instead of 2558.  No distribution is excluded: sub-buckets that a block cannot hold are split by their own values (see rank_big),
-// zeros among them where more coordinates are sent than are not zero.  (Digit passes for a batch with such a client, as phases of one
-// kernel, took it from 844 to 1110 us for one of 11.2 M coordinates, 97 % zeros, and from 1636 to 3100 for 10 of 5 M, 95 % zeros.)
-CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
+// The buckets of a client with nb bins between threshold and top, the fullest of them holding max_bin candidates, in a batch of `all`
+// candidates.  As few sub-buckets as let a window and one of them fit a block if a bin's candidates spread evenly over it (every one that
+// a block meets costs the selection a global addition); four times as many while a client then has at most 512, or 2048 where the
+// partition's blocks have one tile each, since they often lie at one end of it: error compensation leaves the memories crowded below the
+// threshold, in buckets that no block holds (10 clients of 5 M coordinates, up to 512 / 2048, us: 40th round 234 / 233, 150th 261 / 239,
+// 400th 278 / 252), and even tiles are ranked sooner (as few as fit / up to 512: 20 of 1.2 M 121 / 119, 100 of 1.2 M 423 / 415).  Not up to
+// 2048 beyond that: a partition that fills the chip then writes its 4096 candidates at a time to places of two each (512 / 2048: 300 of 3 M
+// 2133 / 2184, 24 of 3 M at 4 bits 400 / 407, 20 of 1.2 M 115.1 / 116.1; only 40 of 5 M with error compensation, 400th round, gain,
+// 842 / 811).  Nor in the smallest batches, whose selection and partition are the additions' latency (one of 1.2 M 47.9 / 49.0).  No
+// distribution is excluded: sub-buckets that a block cannot hold are split by their own values (see rank_big), zeros among them where more
+// coordinates are sent than are not zero.  (Digit passes for a batch with such a client, as phases of one kernel, took it from 844 to
+// 1110 us for one of 11.2 M coordinates, 97 % zeros, and from 1636 to 3100 for 10 of 5 M, 95 % zeros.)
+CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, uint64_t all, ClientRank* r) {
   uint32_t g = 0;
   while (((nb - 1) >> g) + 1 > kRankCoarse) ++g;
   r->group = g;
@@ -221,7 +224,8 @@ CVLC_HD inline void rank_shape(uint32_t nb, uint32_t max_bin, ClientRank* r) {
   r->split = fullest > kRankBucket ? 1u : 0u;
   uint32_t k = 0;
   while ((fullest >> k) > kRankItems - kRankWindow && (r->n_coarse << (k + 1)) <= kRankSubs && k < 16) ++k;
-  for (int more = 0; r->split && more < 2 && (r->n_coarse << (k + 1)) <= 512 && k < 16; ++more) ++k;
+  const uint32_t most = all <= kRankOneRound && all > kRankOneRound / 4 ? 2048 : 512;
+  for (int more = 0; r->split && more < 2 && (r->n_coarse << (k + 1)) <= most && k < 16; ++more) ++k;
   r->sub_bits = k;
   r->wide = fullest >= (1u << 24) ? 1u : 0u;
 }
@@ -615,12 +619,12 @@ CVLC_HD inline uint32_t rank_limit(const Shape& shape) {
 
 // a client's buckets from its threshold, the candidates from there on, and what the fullest bin holds
 __device__ __forceinline__ ClientRank client_rank(uint32_t thresh_bin, uint32_t top_bin, unsigned long long n_candidates, uint32_t max_bin,
-                                                  unsigned long long capacity) {
+                                                  unsigned long long capacity, uint32_t n) {
   ClientRank r;
   const uint32_t top = top_bin < CVLC_HIST_BINS ? top_bin : CVLC_HIST_BINS - 1;
   const uint32_t nb = thresh_bin <= top ? top - thresh_bin + 1 : 1;
-  rank_shape(nb, max_bin, &r);
   r.n = (uint32_t)(n_candidates < capacity ? n_candidates : capacity);
+  rank_shape(nb, max_bin, (uint64_t)r.n * n, &r);
   r.keytop = sort_keytop(top_bin);
   r.top_bin = top;
   r.thresh_bin = thresh_bin;

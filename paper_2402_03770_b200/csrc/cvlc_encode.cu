@@ -76,7 +76,7 @@ k_encode_init(unsigned char* ws, const __grid_constant__ BatchDesc<CAP> batch, c
       if (plan->top_bin + 1u - plan->thresh_bin > 256u) pass3 = 1;  // see top_digit_is_zero
       if (max_bin && blockIdx.x == 0) {
         const uint2 from = sent_from(plan, reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS);
-        const ClientRank r = client_rank(from.x, plan->top_bin, from.y, max_bin[c], L.capacity);
+        const ClientRank r = client_rank(from.x, plan->top_bin, from.y, max_bin[c], L.capacity, n);
         atomicMax(&s_most, r.n < limit ? r.n : limit);  // buckets from the limit on are not ranked
         if (r.split) atomicMax(&s_most_split, r.n);
         reinterpret_cast<ClientRank*>(ws + L.off_rank)[c] = r;

@@ -409,7 +409,7 @@ __device__ __noinline__ void finish_client(uint32_t c, const Batch& batch, const
       if (nonfinite) set_status(&eh->status, CVLC_ERR_NONFINITE_INPUT);
       else if (t.n > enc.capacity) set_status(&eh->status, CVLC_ERR_WORKSPACE_TOO_SMALL);
       const uint32_t limit = rank_limit(shape);
-      const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.capacity);
+      const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.capacity, n);
       reinterpret_cast<ClientRank*>(enc.ws + enc.off_rank)[c] = r;
       reinterpret_cast<uint32_t*>(enc.ws + enc.off_pass_mask)[c] = (1u << kSortPasses) - 1u;  // ranked by partition: the result is in the first buffer
       add_client(eh, r, limit);
