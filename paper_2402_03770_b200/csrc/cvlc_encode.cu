@@ -324,8 +324,8 @@ k_select_lookback(const Batch batch, uint64_t d, unsigned char* ws, const __grid
 // buffer.  When that is full the warp counts its candidates per coarse bucket, reserves room in every bucket with one global
 // addition and puts the candidates there; they are also counted per sub-bucket where the client needs the partition.  The block
 // that completes a client turns those counts into offsets.
-// Bound by instruction issue (0.60 per scheduler and cycle).  100 clients of 11.2 M coordinates, 6 % candidates: 568 us; 50 of
-// 23.5 M, 3.5 %: 610; 10 of 100 M, 1 %: 210.  The copies go past the L1 (cp.async.cg): with loads into registers the warps were
+// Bound by instruction issue (0.60 per scheduler and cycle).  100 clients of 11.2 M coordinates, 7 % candidates: 622 us (from the bin
+// of rank k on, 6 %: 568); 50 of 23.5 M, 3.5 %: 610; 10 of 100 M, 1 %: 210.  The copies go past the L1 (cp.async.cg): with loads into registers the warps were
 // bound by the L1 lines that shared memory leaves for loads in flight (832, 943 and 377 us), and more warps made it worse; asking
 // the L2 for 64 bytes instead of the 128 that it fetches by default takes 344 instead of 512 MB from DRAM for 8 of the second.
 // (One buffer per block, emptied by all its warps together, left them waiting for one another: 860 us for the first.)
@@ -1160,7 +1160,9 @@ constexpr int kPackGroup = 1;  // packets per warp (more of them amortise the le
 // 1332 / 1500 / 1924 packets of 1500 bytes -1.8 / -0.8 / -0.1 / 0 / +1.2 / +2.1 (QSGD, whose norm is one lane's chain in both: -2.1 / -3.6
 // / -2.0 / -1.4 / +2.7 / +1.9), of 752 bytes -0.7 / -0.9 / -0.2 / -1.1 / +2.0 / +2.1, of 256 bytes 0 / +0.1 / +0.4 / +0.8 / +2.0 / +2.1 (QSGD
 // -0.8 / -0.3 / -0.6 / -0.9 / +1.9 / +2.0), of 32 bytes -0.2 / +0.8 / +0.2 / +0.1 / +2.1 / +2.1; at 1332 / 1700 / 1924 / 2300 packets of 3000
-// bytes -1.1 / +0.9 / +0.3 / +0.1, of 4500 -7.2 / +0.1 / -3.8 / -1.4 (8 clients -6.3 / -4.9 / -5.1 / -3.5).
+// bytes -1.1 / +0.9 / +0.3 / +0.1, of 4500 -7.2 / +0.1 / -3.8 / -1.4 (8 clients -6.3 / -4.9 / -5.1 / -3.5).  Between the two lines it
+// also depends on the values: 1340 to 1920 packets of 1500 bytes, one and four clients, +1 to +7 for one Laplace distribution, -3.5 to 0 for
+// layers of different scales; 8 and 24 clients -1.6 to +3.
 inline bool pack_team(uint64_t packets, bool qsgd, uint32_t records, size_t packet_bytes) {
   return records >= (qsgd ? 48u : 128u) && packets <= (!qsgd && packet_bytes >= 4500 ? 13u : 9u) * (uint64_t)kNumSM;
 }

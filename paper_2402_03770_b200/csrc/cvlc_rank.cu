@@ -110,7 +110,7 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
 // Tiles of buckets (RankTile), drawn by ticket; the next tile's buckets are searched for by two warps while the others compare.
 // No calls and no per-client state in registers: 62 of them and no spills (with the crowded cells ranked here, 80 bytes of
 // spills and waiting warps).  Bound by instruction issue, about 100 instructions per warp of candidates, and by a tile's barriers.
-// 79 M candidates of 100 clients: 750 -> 555 us (and 38 for what is left over, see k_rank_rest), the 70 M that are sent 502; 41 M of
+// 79 M candidates of 100 clients: 750 -> 549 us (and 38 for what is left over, see k_rank_rest), the 70 M that are sent 502; 41 M of
 // 50, every seventh layer on a grid: 784 -> 303 (and 143).  Half as many cells, or blocks of 256 threads with half the window, are
 // within 5 %; twice the cells cost 20 % (clearing and scanning them), keeping an item's place from the counting 10 % (the atomic then
 // returns a value).

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 def gpu_batch_encode(workload, clients, d, bpc, max_candidates, torch, B, quantizer=0, one_call=True):
-    """one_call: cvlc_compress_batch with the length tuning on a side stream (what the benchmark times); otherwise
+    """one_call: cvlc_compress_batch with a side stream (what the benchmark times); otherwise
     cvlc_plan_batch followed by cvlc_encode_batch"""
     w = W.WORKLOADS[workload]
     dev = torch.device("cuda:0")
@@ -92,8 +92,8 @@ def test_resnet18_budget_sweep_two_clients(env, bpc):
 
 
 def test_resnet18_all_100_clients_as_benchmarked(env):
-    """the benchmark's step: plan + encode of 100 clients at 2 bits per coordinate in one call, the length tuning on
-    a side stream, with the benchmark's reduced candidate workspace, then one decode-aggregate with sample-count
+    """the benchmark's step: plan + encode of 100 clients at 2 bits per coordinate in one call, selection and ranking
+    on a side stream beside the length tuning, with the benchmark's reduced candidate workspace, then one decode-aggregate with sample-count
     weights"""
     torch, B = env
     w = W.WORKLOADS["resnet18"]
