@@ -513,7 +513,7 @@ def cvlc_profile_reset() -> None:
     _check(lib().cvlc_profile_reset(), "cvlc_profile_reset")
 
 
-KERNEL_NAMES = ["k_zero_words", "k_hist", "k_plan_threshold", "k_plan_fit", "k_plan_tune", "k_encode_init", "k_select",
+KERNEL_NAMES = ["k_zero_words", "k_client", "k_hist", "k_plan_threshold", "k_plan_fit", "k_plan_tune", "k_encode_init", "k_select",
                 "k_select_lookback", "k_rank_split", "k_rank", "k_rank_rest", "k_sort", "k_pack", "k_decode_prepare", "k_fill_zero",
                 "k_prefetch_l2", "k_decode", "k_noalloc_publish_status", "k_selftest", "k_hist_check", "k_apply", "k_plan_literal", "k_ec_accumulate", "k_pack_unframed", "k_decode_unframed"]
 

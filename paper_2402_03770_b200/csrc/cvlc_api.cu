@@ -524,8 +524,13 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   const bool two = side_stream != nullptr && side_st != main_st;
   Shape Senc = S;
   Senc.fixed_y = 0;
+  const EncFront front{static_cast<unsigned char*>(enc_ws_dev), enc_layout(S.d, n, cap)};
+  if (by_clusters(S, n, desc[0].cap0)) {  // the second stream has nothing to do: the tuning is in the same kernel
+    if (launch_clients(desc, n, S, plan_ws_dev, front, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
+    return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, false, nullptr, kPackFramed, true) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
+  }
   const TunePlace place = two ? tune_place(S.d, n) : kTuneAlone;
-  if (launch_plan_front(desc, n, S, plan_ws_dev, enc_front(enc_layout(S.d, n, cap), enc_ws_dev), place, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
+  if (launch_plan_front(desc, n, S, plan_ws_dev, front, place, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
   if (!two) {
     if (launch_plan_back(n, S, plan_ws_dev, place, main_st, true) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, false, nullptr, kPackFramed) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;

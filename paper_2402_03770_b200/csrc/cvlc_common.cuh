@@ -363,7 +363,7 @@ CVLC_HD constexpr size_t dec_ws_bytes(uint32_t n) { return align256(dec_off_meta
 // ---- launch accounting and optional per-kernel timing ------------------------------
 
 enum KernelId {
-  kKZeroWords = 0, kKHist, kKPlanThreshold, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
+  kKZeroWords = 0, kKClient, kKHist, kKPlanThreshold, kKPlanFit, kKPlanTune, kKEncodeInit, kKSelect, kKSelectLookback, kKRankSplit, kKRank,
   kKRankRest, kKSort, kKPack, kKDecodePrepare, kKFillZero, kKPrefetchL2, kKDecode, kKNoallocStatus, kKSelftest, kKHistCheck, kKApply,
   kKPlanLiteral, kKEcAccumulate, kKPackUnframed, kKDecodeUnframed, kNumKernelIds
 };
@@ -440,8 +440,7 @@ __device__ __forceinline__ void pdl_enter() {
 // shapes of the ranking, the counters of selection and partition at zero
 struct EncFront {
   unsigned char* ws;
-  uint64_t capacity;
-  size_t off_rank, off_pass_mask, zero_end;
+  EncLayout L;
 };
 
 // Where the length tuning runs, one block per client that tunes.  Beside selection and ranking, whose blocks fill an SM each, its place
@@ -475,6 +474,18 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
 // overlap: nothing but the front precedes the back on its stream (no wait for an event)
 cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
+// Few small clients: planning, selection and ranking by a cluster of blocks per client (see k_client).  All clusters run at a time, a
+// block of eight for each eighth of the coordinates, which it keeps in shared memory; few candidates, so that the seven that rank have one
+// tile each.
+constexpr int kClusterBlocks = 8;
+constexpr uint32_t kClusterUnits = 10240;  // float4 units that a block keeps
+constexpr uint32_t kClusterClients = 15;   // clusters of eight blocks, an SM each, that run at a time (cudaOccupancyMaxActiveClusters)
+constexpr uint64_t kClusterCandidates = 32768;
+inline bool by_clusters(const Shape& shape, uint32_t n, uint32_t cap0) {
+  return n <= kClusterClients && make_partition(shape.d, n).rows <= (uint64_t)kClusterBlocks * (kClusterUnits / kRowUnits) &&
+         (uint64_t)shape.R * cap0 <= kClusterCandidates;
+}
+cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st);
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,
                              unsigned long long* hist_out, cudaStream_t st);
 cudaError_t launch_plan_from_hist(const ClientDesc* clients, uint32_t n, const Shape& shape,
@@ -493,6 +504,8 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
 // ranking by partition (after the selection)
 cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
+// its last kernel alone: the large buckets that are on the lists
+cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into
@@ -500,17 +513,15 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
 // server rebuilds for it); kPackNone = selection and ranking only (launch_pack or the unframed writer follows)
 constexpr int kPackFramed = 0, kPackResidual = 1, kPackNone = 2;
 constexpr size_t kPackSharedMax = 200 * 1024;  // shared memory of four packets at work, at most
+// ranked: planned, selected and ranked by launch_clients on the same stream
 // prepared: the planning front of the same call has prepared the workspace (see EncFront) and precedes it on the stream; behind_wait:
 // and a wait for another stream's event lies between
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, bool prepared, bool behind_wait, cudaEvent_t wait_before_pack,
-                          int write_residual);
+                          int write_residual, bool ranked = false);
 // the packing alone, behind selection and ranking; overlap: they directly precede it on the stream
 cudaError_t launch_pack(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity, void* ws, cudaStream_t st, bool overlap,
                         int write_residual);
-static inline EncFront enc_front(const EncLayout& L, void* ws) {
-  return EncFront{static_cast<unsigned char*>(ws), L.capacity, L.off_rank, L.off_pass_mask, L.off_sub_start};
-}
 cudaError_t launch_ec_accumulate(float* const* memory, const float* const* update, uint32_t n, uint64_t d, cudaStream_t st);
 // unframed stream (version 2)
 constexpr uint32_t kUfMaxRecords = 2048;  // records of a block (they are sorted and assembled in shared memory)

@@ -369,17 +369,6 @@ __device__ __noinline__ void add_counts4_wide(float* p, uint4 v) {
   if (v.w) atomicAdd(whole + 3, v.w);
 }
 
-// a sub-bucket that a block of the ranking cannot hold
-__device__ __noinline__ void list_bucket(EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, const ClientRank& r, uint32_t sh,
-                                         uint32_t bucket, uint32_t start, uint32_t m) {
-  const u64 lo = (u64)~r.keytop + ((u64)bucket << sh), end = lo + (1ull << sh);  // the last bucket may reach below key 0
-  const bool own = m <= kBigOwn;
-  if (!own) atomicAdd(&hdr->big[0].slots, m / kBigSlot);
-  const size_t row = own ? kBigOwnRow * ((size_t)L.n * L.capacity / kRankItems + 1) : 0;
-  reinterpret_cast<BigBucket*>(ws + L.off_big)[row + atomicAdd(own ? &hdr->own_n : &hdr->big[0].n, 1u)] =
-      BigBucket{(u64)c * L.capacity + start, lo << 32, end >> 32 ? ~0ull : end << 32, ~0ull, m, big_parts(m), 0u, 0u};
-}
-
 __global__ void __launch_bounds__(kSelThreads, 1)
 k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, const __grid_constant__ SelectGroups sg,
          const unsigned char* __restrict__ plan_ws, unsigned char* ws, const __grid_constant__ EncLayout L) {
@@ -750,7 +739,7 @@ k_select(const Batch batch, uint64_t d, const __grid_constant__ Partition part, 
               const uint32_t from[4] = {at.x, at.y, at.z, at.w};
 #pragma unroll
               for (uint32_t u = 0; u < 4; ++u)
-                if (v[e + u] > kRankItems && from[u] < hdr->limit && from[u] + v[e + u] <= r.n) list_bucket(hdr, ws, L, c, r, sh_sub, i0 + e + u, from[u], v[e + u]);
+                if (v[e + u] > kRankItems && from[u] < hdr->limit && from[u] + v[e + u] <= r.n) list_bucket(hdr, ws, L, c, keytop, (u64)(i0 + e + u) << sh_sub, (u64)(i0 + e + u + 1) << sh_sub, from[u], v[e + u]);
             }
           }
         }
@@ -1487,7 +1476,7 @@ cudaError_t launch_pack(const ClientDesc* clients, uint32_t n, const Shape& shap
 
 cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& shape, uint64_t capacity,
                           const void* plan_ws, void* ws, cudaStream_t st, bool prepared, bool behind_wait, cudaEvent_t wait_before_pack,
-                          int write_residual) {
+                          int write_residual, bool ranked) {
   static OncePerDevice once;
   cudaError_t e = once_per_device(once, [] {
     cudaError_t e = allow_shared(k_select, kSelSmem);
@@ -1500,6 +1489,10 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   const EncLayout L = enc_layout(shape.d, n, capacity);
   if (enc_lists_end(L) > L.off_buf_a) return cudaErrorInvalidValue;
   unsigned char* w = static_cast<unsigned char*>(ws);
+  if (ranked) {
+    e = launch_rank_rest(Batch{nullptr, n}, L, static_cast<const unsigned char*>(plan_ws), w, kNumSM, st);
+    return e != cudaSuccess ? e : launch_pack(clients, n, shape, capacity, ws, st, true, write_residual);
+  }
   const Partition part = make_partition(shape.d, n);
   const unsigned sms = wait_before_pack && tune_place(shape.d, n) == kTuneRoomLeft ? kNumSM - n : kNumSM;
   const unsigned char* pws = static_cast<const unsigned char*>(plan_ws);

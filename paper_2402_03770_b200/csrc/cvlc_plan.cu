@@ -5,9 +5,11 @@
 // The planner's floating point is IEEE binary64 with every multiply and add
 // rounded separately (the *_rn intrinsics keep the compiler from contracting
 // them), in a fixed order, so that its decisions do not depend on the machine.
+#include <cooperative_groups.h>
 #include <string.h>
 
 #include "cvlc_common.cuh"
+#include "cvlc_rank.cuh"
 
 namespace cvlc {
 
@@ -192,16 +194,10 @@ k_zero_words(const __grid_constant__ BatchDesc<CAP> batch, ClientDesc* desc, uin
 
 // ---- what a client's histogram gives, by a block of kPlanThreads threads ------------------------
 // Survival counts N_j = #{bin >= j} into N[0 .. 4096] (they add up to d <= 2^31); ends with a barrier.
-__device__ __forceinline__ void survival_counts(const unsigned long long* hist, uint32_t* N) {
+// h: the thread's kPlanBins bins.
+__device__ __forceinline__ void survival_of(const uint32_t (&h)[kPlanBins], uint32_t* N) {
   __shared__ uint32_t s_warp[kPlanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t h[kPlanBins];
-#pragma unroll
-  for (int i = 0; i < kPlanBins; i += 2) {
-    const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(hist) + (kPlanBins * tid + i) / 2);
-    h[i] = (uint32_t)v.x;
-    h[i + 1] = (uint32_t)v.y;
-  }
   uint32_t sum = 0;
 #pragma unroll
   for (int i = 0; i < kPlanBins; ++i) sum += h[i];
@@ -227,11 +223,21 @@ __device__ __forceinline__ void survival_counts(const unsigned long long* hist, 
   if (tid == 0) N[CVLC_HIST_BINS] = 0;
   __syncthreads();
 }
+__device__ __forceinline__ void survival_counts(const unsigned long long* hist, uint32_t* N) {
+  uint32_t h[kPlanBins];
+#pragma unroll
+  for (int i = 0; i < kPlanBins; i += 2) {
+    const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(hist) + (kPlanBins * threadIdx.x + i) / 2);
+    h[i] = (uint32_t)v.x;
+    h[i + 1] = (uint32_t)v.y;
+  }
+  survival_of(h, N);
+}
 
 // The selection threshold.  The number of transmitted coordinates k is not known before the lengths are tuned, but it never exceeds
 // k_sel = R * cap(shortest candidate length) (every packet at the shortest code; with a fixed length, exactly R * cap(y)), so the
 // selection keeps every coordinate down to the bin that holds rank min(k_sel, d): a superset of the top k whose first k ranks are
-// the top k.  Written to the plan; where every candidate bin starts among the client's candidates (from the top bin down) to
+// the top k.  Written to the plan (may be null); where every candidate bin starts among the client's candidates (from the top bin down) to
 // bin_start (may be null).  Ends with a barrier.
 struct Threshold {
   uint32_t bin, top, n, fullest;  // threshold's bin, highest bin, candidates, those in the fullest bin
@@ -265,7 +271,7 @@ __device__ __forceinline__ Threshold client_threshold(const uint32_t* N, const S
   }
   __syncthreads();
   const Threshold t = s_t;
-  if (tid == 0) {
+  if (tid == 0 && plan) {
     plan->status = CVLC_OK;
     plan->s = shape.s;
     plan->R = shape.R;
@@ -382,40 +388,42 @@ __device__ __forceinline__ void write_fit(cvlc_plan_t* plan, double2 alpha, cons
   if (tid <= CVLC_MAX_CODE_BITS) plan->cap[tid] = shape.cap[tid];
 }
 
-// What the last block of a client's histogram does: the client's threshold, the bins' starts and, for an encoder in the same call, its
-// buckets and its share of the workspace's header.
-__device__ __noinline__ void finish_client(uint32_t c, const Batch& batch, const Shape& shape, unsigned char* ws, const EncFront& enc, uint32_t* N) {
-  const int tid = threadIdx.x;
-  const uint32_t n = batch.n;
+// What is known with a client's threshold, by one thread: the headers and, for an encoder in the same call, the client's buckets
+__device__ __forceinline__ void write_client(uint32_t c, uint32_t n, cvlc_plan_t* plan, const Threshold& t, uint32_t nonfinite, const Shape& shape,
+                                             unsigned char* ws, const EncFront& enc) {
   PlanWsHeader* hdr = reinterpret_cast<PlanWsHeader*>(ws);
   EncHeader* eh = reinterpret_cast<EncHeader*>(enc.ws);
+  if (nonfinite) {
+    plan->status = CVLC_ERR_NONFINITE_INPUT;
+    set_status(&hdr->status, CVLC_ERR_NONFINITE_INPUT);
+  }
+  reinterpret_cast<uint32_t*>(ws + plan_off_max_bin(n))[c] = t.fullest;
+  if (c == 0) {
+    hdr->n = n;
+    hdr->d = shape.d;
+    hdr->magic = kPlanWsMagic;
+  }
+  if (enc.ws) {
+    if (nonfinite) set_status(&eh->status, CVLC_ERR_NONFINITE_INPUT);
+    else if (t.n > enc.L.capacity) set_status(&eh->status, CVLC_ERR_WORKSPACE_TOO_SMALL);
+    const uint32_t limit = rank_limit(shape);
+    const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.L.capacity, n);
+    reinterpret_cast<ClientRank*>(enc.ws + enc.L.off_rank)[c] = r;
+    reinterpret_cast<uint32_t*>(enc.ws + enc.L.off_pass_mask)[c] = (1u << kSortPasses) - 1u;  // ranked by partition: the result is in the first buffer
+    add_client(eh, r, limit);
+    if (c == 0) eh->limit = limit;
+  }
+}
+
+// What the last block of a client's histogram does: the client's threshold, the bins' starts and the above
+__device__ __noinline__ void finish_client(uint32_t c, const Batch& batch, const Shape& shape, unsigned char* ws, const EncFront& enc, uint32_t* N) {
+  const uint32_t n = batch.n;
   cvlc_plan_t* plan = batch.c[c].plan;
   const uint32_t cap0 = batch.c[c].cap0;
   const uint32_t nonfinite = __ldcg(reinterpret_cast<const uint32_t*>(ws + plan_off_flags(n)) + c);
   survival_counts(reinterpret_cast<const unsigned long long*>(ws + kPlanWsHist) + (size_t)c * CVLC_HIST_BINS, N);
   const Threshold t = client_threshold(N, shape, cap0, plan, reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS);
-  if (tid == 0) {
-    if (nonfinite) {
-      plan->status = CVLC_ERR_NONFINITE_INPUT;
-      set_status(&hdr->status, CVLC_ERR_NONFINITE_INPUT);
-    }
-    reinterpret_cast<uint32_t*>(ws + plan_off_max_bin(n))[c] = t.fullest;
-    if (c == 0) {
-      hdr->n = n;
-      hdr->d = shape.d;
-      hdr->magic = kPlanWsMagic;
-    }
-    if (enc.ws) {
-      if (nonfinite) set_status(&eh->status, CVLC_ERR_NONFINITE_INPUT);
-      else if (t.n > enc.capacity) set_status(&eh->status, CVLC_ERR_WORKSPACE_TOO_SMALL);
-      const uint32_t limit = rank_limit(shape);
-      const ClientRank r = client_rank(t.bin, t.top, t.n, t.fullest, enc.capacity, n);
-      reinterpret_cast<ClientRank*>(enc.ws + enc.off_rank)[c] = r;
-      reinterpret_cast<uint32_t*>(enc.ws + enc.off_pass_mask)[c] = (1u << kSortPasses) - 1u;  // ranked by partition: the result is in the first buffer
-      add_client(eh, r, limit);
-      if (c == 0) eh->limit = limit;
-    }
-  }
+  if (threadIdx.x == 0) write_client(c, n, plan, t, nonfinite, shape, ws, enc);
 }
 
 // ===================================================================================
@@ -725,22 +733,19 @@ __device__ __noinline__ int2 fast_signs64(double h, double at, double step, bool
   down *= inv_D;
   return make_int2(up > guard ? 1 : (up < -guard ? -1 : 0), down > guard ? 1 : (down < -guard ? -1 : 0));
 }
-// K2b  exponent fit and code-length tuning, one CTA per client.  Where every client has an SM to itself (hist given) it fits and
+// K2b  exponent fit and code-length tuning, one CTA per client.  Where every client has an SM to itself (hist or survival counts given) it fits and
 // tunes for itself.  In larger batches, whose blocks take SMs from the selection beside them, the fit has been a kernel before and
 // only the first client of every tuning key does the work.
-__global__ void __launch_bounds__(kTuneThreads, 1)
-k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws, const unsigned long long* __restrict__ hist_all) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+__device__ __forceinline__ void tune_client(uint32_t c, const Batch& batch, const Shape& shape, unsigned char* ws,
+                                            const unsigned long long* __restrict__ hist_all, const uint32_t* survival, unsigned char* smem_raw) {
   __shared__ PlanShared S;
   __shared__ PlanTab T;
   __shared__ FastShared FS;
   __shared__ uint32_t s_leader;
   __shared__ uint32_t s_ny[CVLC_MAX_CODE_BITS + 1];
   __shared__ double s_single[CVLC_MAX_CODE_BITS];
-  const uint32_t c = blockIdx.x;
   const unsigned long long* keys = reinterpret_cast<const unsigned long long*>(ws + plan_off_keys(batch.n));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  pdl_enter();
 
   unsigned long long key0, key1;
   cvlc_plan_t* const my_plan = batch.c[c].plan;
@@ -751,10 +756,14 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     if (tid == 64) S.D = series_log2((double)shape.d);
   };
   double2 alpha = make_double2(0.0, 0.0);
-  if (hist_all) {
+  const bool own = hist_all || survival;
+  if (own) {
     const double B = batch.c[c].scale_B;
-    uint32_t* N = reinterpret_cast<uint32_t*>(smem_raw);
-    survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, N);
+    const uint32_t* N = survival;
+    if (!survival) {
+      survival_counts(hist_all + (size_t)c * CVLC_HIST_BINS, reinterpret_cast<uint32_t*>(smem_raw));
+      N = reinterpret_cast<const uint32_t*>(smem_raw);
+    }
     alpha = client_fit(N, *reinterpret_cast<FitScratch*>(smem_raw + kSurvivalBytes), shape, beside_fit);
     key0 = (unsigned long long)__double_as_longlong(alpha.y);
     key1 = (unsigned long long)__double_as_longlong(B);
@@ -771,7 +780,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   }
 
   const double beta = __dadd_rn(__dmul_rn(2.0, __longlong_as_double((long long)key0)), 1.0);
-  if (!hist_all || shape.fixed_y) {  // a fixed length has no fit to stand beside
+  if (!own || shape.fixed_y) {  // a fixed length has no fit to stand beside
     beside_fit();
     __syncthreads();
   }
@@ -1480,7 +1489,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   }
 
   // ---- outputs, to this client and to the later ones that share its tuning key -------------------
-  if (hist_all) write_fit(my_plan, alpha, T, shape);
+  if (own) write_fit(my_plan, alpha, T, shape);
   if (tid <= CVLC_MAX_CODE_BITS) s_ny[tid] = 0;
   __syncthreads();
   if (tid < nY) s_ny[T.Y[tid]] = S.n[tid];
@@ -1493,7 +1502,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
     if (o > Qmax) Qmax = o;
   }
   __syncthreads();
-  for (uint32_t i = c + warp; i < (hist_all ? c + 1 : batch.n); i += kTuneWarps) {
+  for (uint32_t i = c + warp; i < (own ? c + 1 : batch.n); i += kTuneWarps) {
     if (i != c && (keys[2 * (size_t)i] != key0 || keys[2 * (size_t)i + 1] != key1)) continue;
     cvlc_plan_t* __restrict__ dst = i == c ? my_plan : batch.c[i].plan;
     dst->n_y[lane] = s_ny[lane];
@@ -1506,18 +1515,213 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
   }
 }
 
+__global__ void __launch_bounds__(kTuneThreads, 1)
+k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned char* ws, const unsigned long long* __restrict__ hist_all) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_enter();
+  tune_client(blockIdx.x, batch, shape, ws, hist_all, nullptr, smem_raw);
+}
+
+// ===================================================================================
+// K1-K4 of few small clients: a cluster of blocks per client
+// ===================================================================================
+// Every block keeps its eighth of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's shared
+// memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
+// knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a second
+// barrier the first seven blocks rank a seventh each, in whole bins, while the last one fits the exponent and tunes the lengths.  Bins that a block
+// cannot hold (equal values) are left to k_rank_rest.
+// Bound by latencies: of 19 us for one client of 100,000 coordinates and 26 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
+// of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
+// events) the steps took 30 and 39; whole calls 36.9 -> 26.7 us, 56.7 -> 45.5 with the aggregation.
+
+struct ClusterShared {
+  uint32_t own[CVLC_HIST_BINS + 4];  // the block's counts; then the client's survival counts
+  uint32_t total[CVLC_HIST_BINS];    // the client's
+  uint32_t place[CVLC_HIST_BINS];    // those of the blocks before it; then next places
+};
+constexpr size_t kFitSmem = kSurvivalBytes + sizeof(FitScratch);
+constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) : kFitSmem;  // one after the other
+constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 16;
+static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
+              kClusterSmem <= 216 * 1024, "shared memory");
+
+// FIRST: the call's only kernel before packing (one client): it clears the headers
+template <bool FIRST>
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kPlanThreads, 1)
+k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_constant__ Shape shape, uint32_t rows, unsigned char* ws,
+         const __grid_constant__ EncFront enc) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  ClusterShared& S = *reinterpret_cast<ClusterShared*>(smem_raw);
+  unsigned char* rest = smem_raw + sizeof(ClusterShared);
+  float4* data = reinterpret_cast<float4*>(rest);
+  __shared__ int s_bin[2];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t c = blockIdx.x / kClusterBlocks, q = blockIdx.x % kClusterBlocks, n = batch.n;
+  for (int i = tid; i < CVLC_HIST_BINS; i += kPlanThreads) S.own[i] = 0;
+  __syncthreads();
+  pdl_enter();
+  const ClientDesc& cd = batch.c[c];
+  if (q == 0) {
+    if (tid == 0) reinterpret_cast<ClientDesc*>(ws + plan_off_desc(n))[c] = cd;
+    if (FIRST) {
+      if (tid < 64) reinterpret_cast<uint32_t*>(ws)[tid] = 0;
+      else if (tid < 128) reinterpret_cast<uint32_t*>(enc.ws)[tid - 64] = 0;
+    }
+    if (tid == 128) reinterpret_cast<uint32_t*>(ws + plan_off_flags(n))[c] = 0;
+  }
+  // ---- the block's rows: kept, counted, their maxima written
+  const float* __restrict__ x = cd.x;
+  const float4* xv = reinterpret_cast<const float4*>(x);
+  const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + kClusterBlocks - 1) / kClusterBlocks * kRowUnits;
+  const uint32_t u0 = min(q * slice, nvec), units = min(u0 + slice, nvec) - u0;
+  uint16_t* __restrict__ row_max = reinterpret_cast<uint16_t*>(ws + plan_off_row_max(n)) + (size_t)c * rows;
+  uint32_t top = 0, tail = 0;
+  const bool has_tail = q == kClusterBlocks - 1 && tid < (int)(shape.d & 3);
+  if (has_tail) tail = __float_as_uint(x[4 * (size_t)nvec + tid]);
+  constexpr int kLoads = 8;
+  for (uint32_t i0 = 0; i0 < units; i0 += kLoads * kPlanThreads) {
+    float4 a[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u)
+      if (i0 + u * kPlanThreads + tid < units) a[u] = __ldg(xv + u0 + i0 + u * kPlanThreads + tid);
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const uint32_t i = i0 + u * kPlanThreads + tid;
+      if (i0 + u * kPlanThreads < units) {
+        const bool on = i < units;
+        uint32_t m = 0;
+        if (on) {
+          data[i] = a[u];
+          m = hist_add4(S.own, a[u]);
+        }
+        top = max(top, m);
+        m = max(m, __shfl_xor_sync(kFull, m, 1));
+        m = max(m, __shfl_xor_sync(kFull, m, 2));
+        if (lane % kRowUnits == 0 && on) row_max[(u0 + i) / kRowUnits] = (uint16_t)(m >> 19);
+      }
+    }
+  }
+  if (has_tail) {
+    top = max(top, tail & 0x7FFFFFFFu);
+    atomicAdd(S.own + ((tail & 0x7FFFFFFFu) >> 19), 1u);
+  }
+  cluster.sync();
+  // ---- the client's counts, and those of the blocks before each, by 512 bins a block
+  uint32_t* flag = reinterpret_cast<uint32_t*>(ws + plan_off_flags(n)) + c;
+  if (top >= 0x7F800000u) atomicOr(flag, 1u);  // a key of exponent 255: Inf or NaN
+  {
+    static_assert(kClusterBlocks * kPlanThreads == CVLC_HIST_BINS, "a bin for every thread");
+    const uint32_t b = q * kPlanThreads + tid;
+    uint32_t v[kClusterBlocks], run = 0;
+#pragma unroll
+    for (int r = 0; r < kClusterBlocks; ++r) v[r] = cluster.map_shared_rank(S.own, r)[b];
+#pragma unroll
+    for (int r = 0; r < kClusterBlocks; ++r) {
+      cluster.map_shared_rank(S.place, r)[b] = run;
+      run += v[r];
+    }
+#pragma unroll
+    for (int r = 0; r < kClusterBlocks; ++r) cluster.map_shared_rank(S.total, r)[b] = run;
+    (reinterpret_cast<unsigned long long*>(ws + kPlanWsHist) + (size_t)c * CVLC_HIST_BINS)[b] = run;
+  }
+  cluster.sync();
+  const uint32_t nonfinite = __ldcg(flag);
+  uint32_t* N = S.own;
+  {
+    uint32_t h[kPlanBins];
+#pragma unroll
+    for (int i = 0; i < kPlanBins; i += 4) {
+      const uint4 v = reinterpret_cast<const uint4*>(S.total)[(kPlanBins * tid + i) / 4];
+      h[i] = v.x;
+      h[i + 1] = v.y;
+      h[i + 2] = v.z;
+      h[i + 3] = v.w;
+    }
+    survival_of(h, N);
+  }
+  const Threshold t = client_threshold(N, shape, cd.cap0, q == 0 ? cd.plan : nullptr,
+                                       q == 0 ? reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS : nullptr);
+  if (q == 0 && tid == 0) write_client(c, n, cd.plan, t, nonfinite, shape, ws, enc);
+  const EncLayout& L = enc.L;
+  const bool go = !nonfinite && t.n <= L.capacity;
+  unsigned long long* by_bin = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_b) + (size_t)c * L.capacity;
+  // ---- the candidates to their bins
+  if (go) {
+    for (uint32_t b = t.bin + tid; b <= t.top; b += kPlanThreads) S.place[b] += N[b + 1];
+    __syncthreads();
+    const uint32_t thresh = t.bin << 19;
+    auto put = [&](uint32_t b, uint32_t index) {
+      const uint32_t key = b & 0x7FFFFFFFu;
+      if (key >= thresh) by_bin[atomicAdd(S.place + (key >> 19), 1u)] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | index);
+    };
+#pragma unroll 4
+    for (uint32_t i = tid; i < units; i += kPlanThreads) {
+      const float4 a = data[i];
+      const uint32_t at = 4 * (u0 + i);
+      put(__float_as_uint(a.x), at);
+      put(__float_as_uint(a.y), at + 1);
+      put(__float_as_uint(a.z), at + 2);
+      put(__float_as_uint(a.w), at + 3);
+    }
+    if (has_tail) put(tail, 4 * nvec + tid);
+  }
+  if (q == kClusterBlocks - 1) {
+    __syncthreads();  // the kept rows have been read
+    cg::cluster_group::arrival_token token = cluster.barrier_arrive();
+    const Batch all{reinterpret_cast<const ClientDesc*>(ws + plan_off_desc(n)), n};
+    tune_client(c, all, shape, ws, nullptr, N, rest);
+    cluster.barrier_wait(std::move(token));
+    return;
+  }
+  cluster.sync();
+  if (!go) return;
+  // ---- the bins whose candidates begin in the block's share of the ranks
+  const uint32_t limit = rank_limit(shape), ranked = min(t.n, limit);
+  const uint32_t share = (ranked + kClusterBlocks - 2) / (kClusterBlocks - 1);
+  if (tid < 2) s_bin[tid] = (int)t.bin - 1;
+  __syncthreads();
+  for (uint32_t b = t.bin + tid; b <= t.top; b += kPlanThreads) {
+#pragma unroll
+    for (int end = 0; end < 2; ++end) {
+      const uint32_t first = (q + end) * share;
+      if (N[b + 1] >= first && (b == t.top || N[b + 2] < first)) s_bin[end] = (int)b;
+    }
+  }
+  __syncthreads();
+  const int last = s_bin[1];
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_a) + (size_t)c * L.capacity;
+  const uint32_t keytop = sort_keytop(t.top);
+  for (int hi = s_bin[0]; hi > last;) {  // bins (lo, hi], as many as a block holds
+    const uint32_t at = N[hi + 1];
+    if (at >= ranked) break;
+    int lo = last;
+    if (N[last + 1] - at > kRankItems)
+      for (lo = hi - 1; lo > last && N[lo] - at <= kRankItems; --lo) {
+      }
+    const uint32_t m = N[lo + 1] - at;
+    const u64 inv = (u64)((int)t.top - hi) << 19, end = (u64)((int)t.top - lo) << 19;
+    if (m > kRankItems) {
+      if (tid == 0) list_bucket(reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, inv, end, at, m);
+    } else if (m) {
+      rank_with_cells<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), out + at, keytop);
+    }
+    hi = lo;
+  }
+}
+
 // ===================================================================================
 // launchers
 // ===================================================================================
-
-constexpr size_t kFitSmem = kSurvivalBytes + sizeof(FitScratch);
-constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) : kFitSmem;  // one after the other
 
 static cudaError_t plan_attributes() {
   static OncePerDevice once;
   return once_per_device(once, [] {
     cudaError_t e = allow_shared(k_hist, kHistSub * CVLC_HIST_BINS * 4);
     if (e == cudaSuccess) e = allow_shared(k_plan_fit, kFitSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<false>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<true>, kClusterSmem);
     return e != cudaSuccess ? e : allow_shared(k_plan_tune, kTuneSmem);
   });
 }
@@ -1558,7 +1762,7 @@ static cudaError_t launch_hist(const ClientDesc* clients, uint32_t n, const Shap
   if (e != cudaSuccess) return e;
   // header, histograms, flags, counters and tuning keys start at zero (and so does the encoder's workspace up to what its selection
   // writes in full); the rest is written in full by the kernels that follow
-  *batch = launch_zero(clients, n, w, plan_off_desc(n), enc.ws, enc.ws ? enc.zero_end : 0, st);
+  *batch = launch_zero(clients, n, w, plan_off_desc(n), enc.ws, enc.ws ? enc.L.off_sub_start : 0, st);
   // the resident blocks share the concatenated updates evenly
   launch_kernel(kKHist, k_hist, part.grid, kHistThreads, kHistSub * CVLC_HIST_BINS * 4, st, true, *batch, shape, part, w, enc, finish ? 1 : 0);
   return cudaGetLastError();
@@ -1574,6 +1778,20 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
     launch_fit(batch, shape, w, enc, part.per_client ? kThresholdThere : kThresholdFinish, st, true);
   else if (!part.per_client)
     launch_kernel(kKPlanThreshold, k_plan_threshold, n, kPlanThreads, 0, st, true, batch, shape, w, enc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st) {
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  const cudaError_t e = plan_attributes();
+  if (e != cudaSuccess) return e;
+  BatchDesc<kMediumBatch> batch;
+  batch.n = n;
+  batch.pad = 0;
+  memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
+  const uint32_t rows = (uint32_t)make_partition(shape.d, n).rows;
+  if (n > 1) launch_zero(clients, n, w, 256, enc.ws, 256, st);
+  launch_kernel(kKClient, n > 1 ? k_client<false> : k_client<true>, kClusterBlocks * n, kPlanThreads, kClusterSmem, st, n > 1, batch, shape, rows, w, enc);
   return cudaGetLastError();
 }
 

@@ -167,22 +167,32 @@ k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
   rank_lists<kRankThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, s_args);
 }
 
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
+static cudaError_t rank_attributes() {
   static OncePerDevice once;
-  const cudaError_t e = once_per_device(once, [] {
+  return once_per_device(once, [] {
     const cudaError_t e = allow_shared(k_rank, sizeof(RankShared));
     return e != cudaSuccess ? e : allow_shared(k_rank_rest, sizeof(RankShared));
   });
+}
+static unsigned blocks(uint64_t tiles, uint64_t most) { return (unsigned)(tiles < most ? tiles : most); }
+
+cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
+  const cudaError_t e = rank_attributes();
   if (e != cudaSuccess) return e;
-  auto blocks = [](uint64_t tiles, uint64_t most) -> unsigned { return (unsigned)(tiles < most ? tiles : most); };
+  launch_kernel(kKRankRest, k_rank_rest, blocks((L.capacity + kRankItems - 1) / kRankItems * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true,
+                batch, ws, L, reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n)), 2 * sms);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
+  const cudaError_t e = rank_attributes();
+  if (e != cudaSuccess) return e;
   launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * sms), kRankThreads, kRankSubs * 4, st, true,
                 batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
   launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start,
                 2 * sms);
-  launch_kernel(kKRankRest, k_rank_rest, blocks((L.capacity + kRankItems - 1) / kRankItems * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true,
-                batch, ws, L, bin_start, 2 * sms);
-  return cudaGetLastError();
+  return launch_rank_rest(batch, L, plan_ws, ws, sms, st);
 }
 
 }  // namespace cvlc

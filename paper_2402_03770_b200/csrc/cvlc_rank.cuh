@@ -585,6 +585,17 @@ __device__ __forceinline__ u64 big_slot(u64 pos) { return (pos + kBigSlot - 1) /
 static_assert(kRankItems / kBigSlot - 1 > kRankItems / kBigPart + 1 && kBigPart > 2 * kBigSlot, "a bucket has a slot for every part");
 static_assert(kBigParts <= kRankItems / 8 && 2 * kBigParts <= kCells, "splitters and counts in shared memory, eight samples for a part");
 
+// a bucket that a block of the ranking cannot hold: its sort keys lie in [lo, end)
+static __device__ __noinline__ void list_bucket(EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop, u64 lo, u64 end,
+                                                uint32_t start, uint32_t m) {
+  const u64 from = (u64)~keytop + lo, to = (u64)~keytop + end;  // the last bucket may reach below key 0
+  const bool own = m <= kBigOwn;
+  if (!own) atomicAdd(&hdr->big[0].slots, m / kBigSlot);
+  const size_t row = own ? kBigOwnRow * ((size_t)L.n * L.capacity / kRankItems + 1) : 0;
+  reinterpret_cast<BigBucket*>(ws + L.off_big)[row + atomicAdd(own ? &hdr->own_n : &hdr->big[0].n, 1u)] =
+      BigBucket{(u64)c * L.capacity + start, from << 32, to >> 32 ? ~0ull : to << 32, ~0ull, m, big_parts(m), 0u, 0u};
+}
+
 // Waits (bounded) until *done reaches `want`.  False: the wait ran out.  By the whole block.
 __device__ __forceinline__ bool block_waits(const uint32_t* done, uint32_t want, int32_t* status) {
   __shared__ int s_ok;

@@ -1,0 +1,112 @@
+"""GPU parity of cvlc_compress_batch where a cluster of blocks per client plans, selects and ranks: at most 15 clients of up to 327,683
+coordinates.  Sizes around its limits and its blocks' slices (rows of 16 coordinates, an eighth each, a ragged tail in the last block),
+and updates whose candidates crowd into bins that a block cannot hold."""
+import numpy as np
+import pytest
+
+from gpu_util import gpu_params, oracle_plan_encode, params_dict
+
+pytestmark = pytest.mark.gpu
+
+
+def update(kind, d, rng):
+    x = rng.standard_normal(d)
+    if kind == "layers":
+        x *= np.repeat(10.0 ** rng.uniform(-3, 0, 9), d // 9 + 1)[:d]
+    elif kind == "equal":  # more equal magnitudes than a block holds, most of them sent
+        x = np.where(rng.random(d) < 0.15, np.sign(x) * 3.0, x)
+    elif kind == "grid":
+        x = np.round(x * 8.0) / 8.0
+    elif kind == "zeros":  # fewer that are not zero than are sent
+        x[rng.random(d) < 0.999] = 0.0
+    elif kind == "signs":
+        x = np.sign(x)
+    elif kind == "front":  # all candidates in the first block's slice
+        x[d // 12:] *= 1e-6
+    return x.astype(np.float32)
+
+
+def check(xs, pds, side, fixed_y=0, checked=3):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    before = B.cvlc_launch_count("k_client")
+    outs = enc.compress([torch.from_numpy(x).to(dev) for x in xs], side_stream=torch.cuda.Stream(dev) if side else None, fixed_y=fixed_y)
+    assert enc.status() == B.CVLC_OK
+    for i in list(range(len(xs)))[-checked:]:
+        want = oracle_plan_encode(xs[i], pds[i], fixed_y)
+        assert enc.read_plan(i).k == want[0]["k"]
+        assert np.array_equal(outs[i].cpu().numpy(), want[1]), i
+    return B.cvlc_launch_count("k_client") - before
+
+
+@pytest.mark.parametrize("d,n", [(2, 1), (5, 2), (127, 1), (129, 3), (2_047, 15), (40_961, 5), (100_003, 1), (300_000, 3), (327_680, 2), (327_683, 1)])
+@pytest.mark.parametrize("side", [False, True])
+def test_sizes(d, n, side):
+    rng = np.random.default_rng(d)
+    packet_bits = 128 if d < 1_000 else 1024 if d < 100_000 else 12_000
+    pds = [params_dict(d, max(packet_bits, d // 2), packet_bits=packet_bits, seed=c, client_id=c, quantizer=c % 2 if n == 1 else 0) for c in range(n)]
+    assert check([update("layers", d, rng) for _ in range(n)], pds, side) == 1
+
+
+def test_limits():
+    rng = np.random.default_rng(0)
+    for d, n, bits in [(327_684, 1, 0.5), (4_000, 16, 0.5), (300_000, 1, 4.0)]:  # coordinates, clients, candidates: the kernels of their own
+        pds = [params_dict(d, int(bits * d), seed=c, packet_bits=1024) for c in range(n)]
+        assert check([update("normal", d, rng) for _ in range(n)], pds, True, checked=2) == 0
+
+
+@pytest.mark.parametrize("kind", ["normal", "equal", "grid", "zeros", "signs", "front"])
+@pytest.mark.parametrize("quantizer", [0, 1])
+def test_distributions(kind, quantizer):
+    rng = np.random.default_rng(3)
+    d, n = 200_003, 4
+    pds = [params_dict(d, 2 * d, seed=c, client_id=c, quantizer=quantizer) for c in range(n)]
+    check([update(kind if c % 2 == 0 else "layers", d, rng) for c in range(n)], pds, True, checked=2)
+
+
+def test_fixed_length():
+    rng = np.random.default_rng(4)
+    check([update("layers", 150_001, rng)], [params_dict(150_001, 150_001)], False, fixed_y=5)
+
+
+def test_errors():
+    """Inf in one client; a workspace for fewer candidates than there are: reported, and the buffers serve the next call"""
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(5)
+    d, n = 50_001, 3
+    pds = [params_dict(d, d, seed=c) for c in range(n)]
+    xs = [torch.from_numpy(update("normal", d, rng)).to(dev) for _ in range(n)]
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    bad = xs[1].clone()
+    bad[d - 1] = float("inf")
+    enc.compress([xs[0], bad, xs[2]])
+    assert enc.status() == B.CVLC_ERR_NONFINITE_INPUT
+    outs = enc.compress(xs)
+    assert enc.status() == B.CVLC_OK
+    assert np.array_equal(outs[2].cpu().numpy(), oracle_plan_encode(xs[2].cpu().numpy(), pds[2])[1])
+    small = B.BatchEncoder([gpu_params(pd) for pd in pds], dev, max_candidates=256)
+    small.compress(xs)
+    assert small.status() == B.CVLC_ERR_WORKSPACE_TOO_SMALL
+
+
+def test_plan_workspace_serves_the_encoder():
+    """the plan's tables that a compress call leaves are those of a plan call"""
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(6)
+    d, n = 120_005, 2
+    pds = [params_dict(d, d, seed=c) for c in range(n)]
+    xs = [torch.from_numpy(update("layers", d, rng)).to(dev) for _ in range(n)]
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    want = [o.clone() for o in enc.compress(xs)]
+    for o in enc.outs:
+        o.zero_()
+    got = enc.encode(xs)
+    assert enc.status() == B.CVLC_OK
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
