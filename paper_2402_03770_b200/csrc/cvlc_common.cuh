@@ -188,7 +188,9 @@ constexpr uint32_t kRankCoarse = 256;      // coarse buckets of a client
 constexpr uint32_t kRankSubs = 8192;       // sub-buckets of a client
 constexpr uint32_t kRankItems = 8192;      // candidates a block of the final ranking holds
 constexpr uint32_t kRankBucket = 4096;     // largest coarse bucket that is ranked without a partition
-constexpr uint32_t kRankWindow = 4096;     // candidates of a tile of the final ranking
+// Candidates of a tile of the final ranking, but for its last bucket, where an SM has two or three blocks
+constexpr uint32_t kRankWindow = 4096, kRankWindow3 = 3072;
+constexpr uint32_t kRankTile3 = kRankWindow3 + kRankBucket;  // with the last bucket: what one of three holds
 constexpr uint32_t kRankSplitTile = 4096;  // candidates of a tile of the partition
 constexpr uint64_t kRankOneRound = 2ull * kNumSM * kRankSplitTile;  // candidates of a batch up to which a block of the partition has one tile
 struct ClientRank {
@@ -502,10 +504,10 @@ cudaError_t launch_plan_literal(const cvlc_params& p, double alpha_q, uint32_t s
                                 unsigned long long k_lo, unsigned long long k_hi, double P_min, double P_max, double tol,
                                 cvlc_literal_plan_t* out, double* P_star, void* ws, cudaStream_t st);
 cudaError_t launch_apply(float* model, const float* agg, uint64_t d, const void* dec_ws, cudaStream_t st);
-// ranking by partition (after the selection)
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
+// ranking by partition (after the selection); most: candidates of a client that can be sent
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, uint64_t most, cudaStream_t st);
 // its last kernel alone: the large buckets that are on the lists
-cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st);
+cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, bool three, cudaStream_t st);
 // wait_before_pack: an event the stream waits for right before the packing kernel (the length tuning on
 // another stream), or nullptr
 // write_residual: kPackFramed = packets only; kPackResidual = the packing kernel also turns the encoder's input into
@@ -651,8 +653,8 @@ __device__ __forceinline__ void add_client(EncHeader* hdr, const ClientRank& r, 
 // tiles of at most kRankWindow allow.  With powers of two, at least four tiles an SM, some blocks had a tile more than the others:
 // one client of 11.2 M coordinates (2048 in 1.4 rounds, now 2800 in one) 18.0 -> 15.6 us between events, 8 of 1.2 M 17.3 -> 14.8, one
 // of 52 M, with what is left over, 73 -> 48.
-__device__ __forceinline__ uint32_t rank_window(uint32_t most, uint32_t n, uint32_t blocks) {
-  const uint32_t least = (most + kRankWindow - 1) / kRankWindow;  // tiles of the largest client
+__device__ __forceinline__ uint32_t rank_window(uint32_t most, uint32_t n, uint32_t blocks, uint32_t largest) {
+  const uint32_t least = (most + largest - 1) / largest;  // tiles of the largest client
   const uint32_t tiles = (least * n + blocks - 1) / blocks * blocks / n;  // below 2^29: at most 2^19 tiles of at most 512 clients
   const uint32_t window = tiles ? (most + tiles - 1) / tiles : 0u;
   return window > 1024 ? window : 1024;

@@ -1490,7 +1490,7 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
   if (enc_lists_end(L) > L.off_buf_a) return cudaErrorInvalidValue;
   unsigned char* w = static_cast<unsigned char*>(ws);
   if (ranked) {
-    e = launch_rank_rest(Batch{nullptr, n}, L, static_cast<const unsigned char*>(plan_ws), w, kNumSM, st);
+    e = launch_rank_rest(Batch{nullptr, n}, L, static_cast<const unsigned char*>(plan_ws), w, kNumSM, false, st);
     return e != cudaSuccess ? e : launch_pack(clients, n, shape, capacity, ws, st, true, write_residual);
   }
   const Partition part = make_partition(shape.d, n);
@@ -1506,7 +1506,8 @@ cudaError_t launch_encode(const ClientDesc* clients, uint32_t n, const Shape& sh
     const uint64_t want = (uint64_t)sg.groups * n;
     const unsigned grid = (unsigned)(want < (uint64_t)sms ? want : sms);
     launch_kernel(kKSelect, k_select, grid, kSelThreads, kSelSmem, st, !behind_wait, batch, shape.d, part, sg, pws, w, L);
-    e = launch_rank(batch, L, pws, w, sms, st);
+    const uint64_t most = (uint64_t)shape.R * shape.cap[1];
+    e = launch_rank(batch, L, pws, w, sms, most < shape.d ? most : shape.d, st);
     if (e != cudaSuccess) return e;
   } else {
     const uint64_t want = select_tiles_of(shape.d) * n;

@@ -20,15 +20,20 @@ __device__ __forceinline__ uint32_t inv_of(u64 item, uint32_t keytop) { return k
 // partition of the coarse buckets into sub-buckets
 // ===================================================================================
 // Tiles of kSplitTile consecutive candidates, held in registers.  A tile spans few coarse buckets, so its sub-buckets are a
-// short range of counters: count, reserve each sub-bucket's room with one global atomic, place.  The next tile's candidates are
-// requested before the current one is placed.  16 bytes per candidate; the stores are scattered 8 bytes at a time and merge in
-// the L2.
+// short range of counters: count, reserve each sub-bucket's room with one global atomic, place.  16 bytes per
+// candidate; the stores are scattered 8 bytes at a time and merge in the L2.
 
 constexpr int kSplitItems = 8;  // per thread
 constexpr uint32_t kSplitTile = kRankThreads * kSplitItems;
 static_assert(kSplitTile == kRankSplitTile, "tiles of the partition");
+constexpr uint64_t kRankThree = 4 << 20;  // candidates of a batch, about, from which three blocks per SM are better than two
 
-__global__ void __launch_bounds__(kRankThreads, 2)
+// THREE: three blocks per SM, the next tile asked into the L2 alone; else two, with the next tile's candidates on their way to registers.
+// Three are better where the blocks have many tiles (two / three, us: 79 M candidates of 100 clients 321 / 296, 14 M of 24 46 / 40, 7 M
+// of 24 24.7 / 21.5, 41 M of 50 178 / 172, 9 M of 10, about even: 54 / 55), two where they have one or two and its latency is all there is
+// (2 M of 20 10.8 / 11.2, 0.9 M of one 8.1 / 10.0, 0.4 M of 10 7.9 / 9.4).
+template <bool THREE>
+__global__ void __launch_bounds__(kRankThreads, THREE ? 3 : 2)
 k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L) {
   extern __shared__ uint32_t s_at[];  // [kRankSubs] counts, then next places
   __shared__ uint32_t s_next;
@@ -53,9 +58,10 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
   if (tid == 0) s_next = atomicAdd(&hdr->split_ticket, 1u);
   __syncthreads();
   uint32_t t = s_next;
-  request(t);
+  if (!THREE) request(t);
   while (t < tickets) {
     __syncthreads();  // everyone has read the ticket
+    if (THREE) request(t);
     if (tid == 0) s_next = atomicAdd(&hdr->split_ticket, 1u);
     const uint32_t tile = t / n, c = t - tile * n;
     const ClientRank r = rank[c];
@@ -80,6 +86,10 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
     }
     __syncthreads();
     const uint32_t next = s_next;
+    if (THREE && next < tickets) {  // a request per 128 bytes
+      const uint32_t tile2 = next / n, c2 = next - tile2 * n, i = tile2 * kSplitTile + tid * 16;
+      if (tid < kSplitTile / 16 && i < rank[c2].n) asm volatile("prefetch.global.L2 [%0];" ::"l"(buf_a + (size_t)c2 * L.capacity + i));
+    }
     uint32_t* room = reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs + s0;
     for (uint32_t i = tid; i < ns; i += kRankThreads) {
       const uint32_t v = s_at[i];
@@ -89,7 +99,7 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
     u64 cur[kSplitItems];
 #pragma unroll
     for (int u = 0; u < kSplitItems; ++u) cur[u] = it[u];
-    request(next);
+    if (!THREE) request(next);
     u64* __restrict__ dst = reinterpret_cast<u64*>(ws + L.off_buf_b) + (size_t)c * L.capacity;
 #pragma unroll
     for (int u = 0; u < kSplitItems; ++u) {
@@ -108,16 +118,20 @@ k_rank_split(const Batch batch, unsigned char* ws, const __grid_constant__ EncLa
 // ===================================================================================
 
 // Tiles of buckets (RankTile), drawn by ticket; the next tile's buckets are searched for by two warps while the others compare.
-// No calls and no per-client state in registers: 62 of them and no spills (with the crowded cells ranked here, 80 bytes of
-// spills and waiting warps).  Bound by instruction issue, about 100 instructions per warp of candidates, and by a tile's barriers.
-// 79 M candidates of 100 clients: 750 -> 549 us (and 38 for what is left over, see k_rank_rest), the 70 M that are sent 502; 41 M of
-// 50, every seventh layer on a grid: 784 -> 303 (and 143).  Half as many cells, or blocks of 256 threads with half the window, are
-// within 5 %; twice the cells cost 20 % (clearing and scanning them), keeping an item's place from the counting 10 % (the atomic then
-// returns a value).
-__global__ void __launch_bounds__(kRankThreads, 2)
+// THREE: three blocks per SM, each with three quarters of the window.
+// No calls and no per-client state in registers: 62 of them and no spills, 40 with THREE (with the crowded cells ranked here, 80 bytes of
+// spills and waiting warps).  Bound by a tile's barriers and the latency of shared memory (two blocks issue 0.44 per scheduler and cycle), about
+// 100 instructions per warp of candidates.  Two blocks and three, us: 79 M candidates of 100 clients 551 / 528 (and 41 for what is left over, see
+// k_rank_rest), 41 M of 50, every seventh layer on a grid, 301 / 285 (and 113), 14 M of 24 92 / 86, 17 M of 20 in two calls 148 / 135; but whole
+// calls of 5 clients of 600,000 coordinates 56.7 / 58.3, one of 11.2 M 87 / 88.  Half as many cells, or blocks of 256 threads with half the
+// window, are within 5 %; twice the cells cost 20 % (clearing and scanning them), keeping an item's place from the counting 10 % (the atomic
+// then returns a value); the next tile's candidates requested before the comparing: no gain, 2 us lost by 43,000 of ten clients.
+template <bool THREE>
+__global__ void __launch_bounds__(kRankThreads, THREE ? 3 : 2)
 k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, uint32_t blocks) {
   extern __shared__ __align__(16) unsigned char s_raw[];
-  RankShared& s = *reinterpret_cast<RankShared*>(s_raw);
+  typedef RankSharedOf<THREE ? kRankTile3 : kRankItems> Shared;
+  Shared& s = *reinterpret_cast<Shared*>(s_raw);
   __shared__ RankTile s_tile[2];
   __shared__ RankArgs s_args;
   pdl_enter();
@@ -125,7 +139,7 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
   if (block_sees_error(&hdr->status)) return;
   const int tid = threadIdx.x;
   if (tid == 0) {
-    s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks);
+    s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks, THREE ? kRankWindow3 : kRankWindow);
     s_tile[0].ticket = atomicAdd(&hdr->rank_ticket, 1u);
   }
   __syncthreads();
@@ -136,11 +150,11 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
     if (T.ticket >= s_args.tickets) return;
     if (tid == 0) s_tile[slot ^ 1u].ticket = atomicAdd(&hdr->rank_ticket, 1u);
     const uint32_t at = T.start[0], m = T.start[1] - at;
-    const bool large = m > kRankItems;
+    const bool large = m > (THREE ? kRankTile3 : kRankItems);
     auto leave = [&](uint32_t list, u64 what, uint32_t items) { s_args.list[list][atomicAdd(&hdr->list_n[list], 1u)] = make_ulonglong2(what, items); };
     if (!large && m != 0) {
       const uint32_t sh = T.sh, base = T.bucket[0] << sh;
-      rank_buckets<kRankThreads>(s, T.from + at, m, base, (uint32_t)(((u64)T.bucket[1] << sh) - ((u64)T.bucket[0] << sh) - 1), T.into + at, T.keytop,
+      rank_buckets<kRankThreads, THREE ? 6 : 8>(s, T.from + at, m, base, (uint32_t)(((u64)T.bucket[1] << sh) - ((u64)T.bucket[0] << sh) - 1), T.into + at, T.keytop,
                                  [&](u64* where, uint32_t items) { leave(items > kWarpCell ? 1u : 0u, (u64)(where - s_args.buf_a), items); },
                                  [&]() {  // behind a barrier that follows the ticket
                                    if (tid < 64) find_tile(s_tile[slot ^ 1u], s_args);
@@ -156,43 +170,46 @@ k_rank(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L
 
 // What the ranking has left over (see rank_lists)
 __global__ void __launch_bounds__(kRankThreads, 2)
-k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, uint32_t blocks) {
+k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLayout L, const uint32_t* __restrict__ bin_start_all, uint32_t blocks,
+            uint32_t window) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   __shared__ RankArgs s_args;
   pdl_enter();
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   if (block_sees_error(&hdr->status)) return;
   if ((hdr->list_n[0] | hdr->list_n[1] | hdr->big[0].n | hdr->own_n) == 0) return;
-  if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks);
+  if (threadIdx.x == 0) s_args = rank_args(ws, L, bin_start_all, hdr, batch.n, blocks, window);
   rank_lists<kRankThreads>(*reinterpret_cast<RankShared*>(s_raw), hdr, s_args);
 }
 
 static cudaError_t rank_attributes() {
   static OncePerDevice once;
   return once_per_device(once, [] {
-    const cudaError_t e = allow_shared(k_rank, sizeof(RankShared));
+    cudaError_t e = allow_shared(k_rank<false>, sizeof(RankShared));
+    if (e == cudaSuccess) e = allow_shared(k_rank<true>, sizeof(RankSharedOf<kRankTile3>));
     return e != cudaSuccess ? e : allow_shared(k_rank_rest, sizeof(RankShared));
   });
 }
 static unsigned blocks(uint64_t tiles, uint64_t most) { return (unsigned)(tiles < most ? tiles : most); }
 
-cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
+cudaError_t launch_rank_rest(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, bool three, cudaStream_t st) {
   const cudaError_t e = rank_attributes();
   if (e != cudaSuccess) return e;
   launch_kernel(kKRankRest, k_rank_rest, blocks((L.capacity + kRankItems - 1) / kRankItems * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true,
-                batch, ws, L, reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n)), 2 * sms);
+                batch, ws, L, reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n)), (three ? 3 : 2) * sms, three ? kRankWindow3 : kRankWindow);
   return cudaGetLastError();
 }
 
-cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, cudaStream_t st) {
+cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* plan_ws, unsigned char* ws, unsigned sms, uint64_t most, cudaStream_t st) {
   const cudaError_t e = rank_attributes();
   if (e != cudaSuccess) return e;
-  launch_kernel(kKRankSplit, k_rank_split, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, 2 * sms), kRankThreads, kRankSubs * 4, st, true,
-                batch, ws, L);
+  const bool three = most * L.n >= kRankThree;
+  launch_kernel(kKRankSplit, three ? k_rank_split<true> : k_rank_split<false>, blocks((L.capacity + kSplitTile - 1) / kSplitTile * L.n, (three ? 3 : 2) * sms),
+                kRankThreads, kRankSubs * 4, st, true, batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
-  launch_kernel(kKRank, k_rank, blocks((L.capacity + 1023) / 1024 * L.n, 2 * sms), kRankThreads, sizeof(RankShared), st, true, batch, ws, L, bin_start,
-                2 * sms);
-  return launch_rank_rest(batch, L, plan_ws, ws, sms, st);
+  launch_kernel(kKRank, three ? k_rank<true> : k_rank<false>, blocks((L.capacity + 1023) / 1024 * L.n, (three ? 3 : 2) * sms), kRankThreads,
+                three ? sizeof(RankSharedOf<kRankTile3>) : sizeof(RankShared), st, true, batch, ws, L, bin_start, (three ? 3 : 2) * sms);
+  return launch_rank_rest(batch, L, plan_ws, ws, sms, three, st);
 }
 
 }  // namespace cvlc

@@ -21,11 +21,13 @@ __device__ __forceinline__ bool block_sees_error(const int32_t* status) {
   return s_err != 0;
 }
 
-struct RankShared {
-  u64 items[kRankItems + 2];  // values (see to_value): all distinct, ordered like the ranks
+template <uint32_t ITEMS>
+struct RankSharedOf {
+  u64 items[ITEMS + 2];       // values (see to_value): all distinct, ordered like the ranks
   uint32_t zero[4];           // cell[-1] = 0: where the first cell starts
   uint32_t cell[kCells];      // counts, then starts, then (after placing) ends of the cells
 };
+typedef RankSharedOf<kRankItems> RankShared;
 
 // A candidate as a value to rank: the key's complement in the high word, index << 1 | sign in the low word.
 __device__ __forceinline__ u64 to_value(u64 item) {
@@ -427,15 +429,14 @@ __device__ __noinline__ void rank_cell(RankShared& s, const u64* at, uint32_t n,
 // Ranks m <= kRankItems items whose inv lies in [base, base + span]: spread over kCells equal ranges of inv, about one item per
 // cell, then compared with the others of their cell.  Cells of more than kCompareAll items are left to `later`, their items in any
 // order in their place.  `meanwhile` is run once all threads have passed a barrier.
-template <int THREADS, class Later, class Meanwhile>
-__device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+template <int THREADS, int HOLD = 8, class Shared, class Later, class Meanwhile>
+__device__ __forceinline__ void rank_buckets(Shared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
                                              Later&& later, Meanwhile&& meanwhile) {
   const int tid = threadIdx.x;
-  // the first kHold candidates of a thread stay in registers between counting and placing
-  constexpr int kHold = 8;
-  u64 it[kHold];
+  // the first HOLD candidates of a thread stay in registers between counting and placing
+  u64 it[HOLD];
 #pragma unroll
-  for (int u = 0; u < kHold; ++u)
+  for (int u = 0; u < HOLD; ++u)
     if ((uint32_t)tid + u * THREADS < m) it[u] = src[tid + u * THREADS];
   {
     uint4* cells = reinterpret_cast<uint4*>(s.zero);
@@ -449,16 +450,16 @@ __device__ __forceinline__ void rank_buckets(RankShared& s, const u64* src, uint
     return k < kCells ? k : kCells - 1;
   };
 #pragma unroll
-  for (int u = 0; u < kHold; ++u)
+  for (int u = 0; u < HOLD; ++u)
     if ((uint32_t)tid + u * THREADS < m) atomicAdd(&s.cell[cell_of_key((uint32_t)(it[u] >> 32))], 1u);
-  for (uint32_t i = tid + kHold * THREADS; i < m; i += THREADS) atomicAdd(&s.cell[cell_of_key((uint32_t)(src[i] >> 32))], 1u);
+  for (uint32_t i = tid + HOLD * THREADS; i < m; i += THREADS) atomicAdd(&s.cell[cell_of_key((uint32_t)(src[i] >> 32))], 1u);
   __syncthreads();
   scan_cells<THREADS>(s.cell);
   auto put = [&](u64 item) { s.items[atomicAdd(&s.cell[cell_of_key((uint32_t)(item >> 32))], 1u)] = to_value(item); };
 #pragma unroll
-  for (int u = 0; u < kHold; ++u)
+  for (int u = 0; u < HOLD; ++u)
     if ((uint32_t)tid + u * THREADS < m) put(it[u]);
-  for (uint32_t i = tid + kHold * THREADS; i < m; i += THREADS) put(src[i]);
+  for (uint32_t i = tid + HOLD * THREADS; i < m; i += THREADS) put(src[i]);
   __syncthreads();
   meanwhile();
   for (uint32_t p = tid; p < m; p += THREADS) {
@@ -504,7 +505,7 @@ struct RankArgs {
   uint32_t n, tickets, window, limit;
 };
 __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout& L, const uint32_t* bin_start, const EncHeader* hdr, uint32_t n,
-                                              uint32_t blocks) {
+                                              uint32_t blocks, uint32_t window) {
   RankArgs a;
   a.rank = reinterpret_cast<const ClientRank*>(ws + L.off_rank);
   a.sub_start = reinterpret_cast<const uint32_t*>(ws + L.off_sub_start);
@@ -524,7 +525,7 @@ __device__ __forceinline__ RankArgs rank_args(unsigned char* ws, const EncLayout
   a.big_room = (size_t)n * a.capacity / kRankItems + 1;
   a.piece_room = (size_t)n * a.capacity / kBigPiece + a.big_room;
   a.n = n;
-  a.window = rank_window(hdr->most, n, blocks);
+  a.window = rank_window(hdr->most, n, blocks, window);
   a.tickets = (hdr->most + a.window - 1) / a.window * n;
   a.limit = hdr->limit;
   return a;
