@@ -476,16 +476,22 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
 // overlap: nothing but the front precedes the back on its stream (no wait for an event)
 cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
-// Few small clients: planning, selection and ranking by a cluster of blocks per client (see k_client).  All clusters run at a time, a
-// block of eight for each eighth of the coordinates, which it keeps in shared memory; few candidates, so that the seven that rank have one
-// tile each.
-constexpr int kClusterBlocks = 8;
+// Few small clients: planning, selection and ranking by a cluster of blocks per client (see k_client).  All clusters run at a time, every block
+// keeps its share of the coordinates in shared memory; few candidates, so that the blocks that rank have one tile each.
 constexpr uint32_t kClusterUnits = 10240;  // float4 units that a block keeps
-constexpr uint32_t kClusterClients = 15;   // clusters of eight blocks, an SM each, that run at a time (cudaOccupancyMaxActiveClusters)
 constexpr uint64_t kClusterCandidates = 32768;
+// Blocks of a client's cluster; 0: too many clients or coordinates.  Clusters that run at a time, a block on an SM
+// (cudaOccupancyMaxActiveClusters): 15 of eight blocks, 7 of sixteen.  Sixteen exchange more counts, eight read longer; whole calls with the
+// aggregation, eight and sixteen, us: one client of 100,000 coordinates 39.0 and 40.6, of 200,000 41.0 and 41.0, of 320,000 44.1 and 42.7, seven
+// of 320,000 47.2 and 45.1.  Beyond that the kernels of their own and sixteen: one of 340,000 47.8 and 42.9, three of 450,000 54.3 and 47.2, seven
+// of 650,000 57.5 and 49.7.
+inline uint32_t cluster_blocks(uint64_t rows, uint32_t n) {
+  const uint64_t of_block = kClusterUnits / kRowUnits;
+  if (n <= 7 && rows > 6 * of_block && rows <= 16 * of_block) return 16;
+  return n <= 15 && rows <= 8 * of_block ? 8 : 0;
+}
 inline bool by_clusters(const Shape& shape, uint32_t n, uint32_t cap0) {
-  return n <= kClusterClients && make_partition(shape.d, n).rows <= (uint64_t)kClusterBlocks * (kClusterUnits / kRowUnits) &&
-         (uint64_t)shape.R * cap0 <= kClusterCandidates;
+  return cluster_blocks(make_partition(shape.d, n).rows, n) != 0 && (uint64_t)shape.R * cap0 <= kClusterCandidates;
 }
 cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st);
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,

@@ -1525,10 +1525,10 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // ===================================================================================
 // K1-K4 of few small clients: a cluster of blocks per client
 // ===================================================================================
-// Every block keeps its eighth of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's shared
+// Every block keeps its share of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's shared
 // memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
 // knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a second
-// barrier the first seven blocks rank a seventh each, in whole bins, while the last one fits the exponent and tunes the lengths.  Bins that a block
+// barrier all blocks but the last rank a share each, in whole bins, while that one fits the exponent and tunes the lengths.  Bins that a block
 // cannot hold (equal values) are left to k_rank_rest.
 // Bound by latencies: of 19 us for one client of 100,000 coordinates and 26 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
 // of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
@@ -1546,8 +1546,8 @@ static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (
               kClusterSmem <= 216 * 1024, "shared memory");
 
 // FIRST: the call's only kernel before packing (one client): it clears the headers
-template <bool FIRST>
-__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kPlanThreads, 1)
+template <int CL, bool FIRST>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kPlanThreads, 1)
 k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_constant__ Shape shape, uint32_t rows, unsigned char* ws,
          const __grid_constant__ EncFront enc) {
   namespace cg = cooperative_groups;
@@ -1558,7 +1558,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   __shared__ int s_bin[2];
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31;
-  const uint32_t c = blockIdx.x / kClusterBlocks, q = blockIdx.x % kClusterBlocks, n = batch.n;
+  const uint32_t c = blockIdx.x / CL, q = blockIdx.x % CL, n = batch.n;
   for (int i = tid; i < CVLC_HIST_BINS; i += kPlanThreads) S.own[i] = 0;
   __syncthreads();
   pdl_enter();
@@ -1574,11 +1574,11 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   // ---- the block's rows: kept, counted, their maxima written
   const float* __restrict__ x = cd.x;
   const float4* xv = reinterpret_cast<const float4*>(x);
-  const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + kClusterBlocks - 1) / kClusterBlocks * kRowUnits;
+  const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + CL - 1) / CL * kRowUnits;
   const uint32_t u0 = min(q * slice, nvec), units = min(u0 + slice, nvec) - u0;
   uint16_t* __restrict__ row_max = reinterpret_cast<uint16_t*>(ws + plan_off_row_max(n)) + (size_t)c * rows;
   uint32_t top = 0, tail = 0;
-  const bool has_tail = q == kClusterBlocks - 1 && tid < (int)(shape.d & 3);
+  const bool has_tail = q == CL - 1 && tid < (int)(shape.d & 3);
   if (has_tail) tail = __float_as_uint(x[4 * (size_t)nvec + tid]);
   constexpr int kLoads = 8;
   for (uint32_t i0 = 0; i0 < units; i0 += kLoads * kPlanThreads) {
@@ -1608,22 +1608,20 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
     atomicAdd(S.own + ((tail & 0x7FFFFFFFu) >> 19), 1u);
   }
   cluster.sync();
-  // ---- the client's counts, and those of the blocks before each, by 512 bins a block
+  // ---- the client's counts, and those of the blocks before each, a share of the bins by every block
   uint32_t* flag = reinterpret_cast<uint32_t*>(ws + plan_off_flags(n)) + c;
   if (top >= 0x7F800000u) atomicOr(flag, 1u);  // a key of exponent 255: Inf or NaN
-  {
-    static_assert(kClusterBlocks * kPlanThreads == CVLC_HIST_BINS, "a bin for every thread");
-    const uint32_t b = q * kPlanThreads + tid;
-    uint32_t v[kClusterBlocks], run = 0;
+  for (uint32_t b = q * kPlanThreads + tid; b < CVLC_HIST_BINS; b += CL * kPlanThreads) {
+    uint32_t v[CL], run = 0;
 #pragma unroll
-    for (int r = 0; r < kClusterBlocks; ++r) v[r] = cluster.map_shared_rank(S.own, r)[b];
+    for (int r = 0; r < CL; ++r) v[r] = cluster.map_shared_rank(S.own, r)[b];
 #pragma unroll
-    for (int r = 0; r < kClusterBlocks; ++r) {
+    for (int r = 0; r < CL; ++r) {
       cluster.map_shared_rank(S.place, r)[b] = run;
       run += v[r];
     }
 #pragma unroll
-    for (int r = 0; r < kClusterBlocks; ++r) cluster.map_shared_rank(S.total, r)[b] = run;
+    for (int r = 0; r < CL; ++r) cluster.map_shared_rank(S.total, r)[b] = run;
     (reinterpret_cast<unsigned long long*>(ws + kPlanWsHist) + (size_t)c * CVLC_HIST_BINS)[b] = run;
   }
   cluster.sync();
@@ -1667,7 +1665,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
     }
     if (has_tail) put(tail, 4 * nvec + tid);
   }
-  if (q == kClusterBlocks - 1) {
+  if (q == CL - 1) {
     __syncthreads();  // the kept rows have been read
     cg::cluster_group::arrival_token token = cluster.barrier_arrive();
     const Batch all{reinterpret_cast<const ClientDesc*>(ws + plan_off_desc(n)), n};
@@ -1679,7 +1677,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   if (!go) return;
   // ---- the bins whose candidates begin in the block's share of the ranks
   const uint32_t limit = rank_limit(shape), ranked = min(t.n, limit);
-  const uint32_t share = (ranked + kClusterBlocks - 2) / (kClusterBlocks - 1);
+  const uint32_t share = (ranked + CL - 2) / (CL - 1);
   if (tid < 2) s_bin[tid] = (int)t.bin - 1;
   __syncthreads();
   for (uint32_t b = t.bin + tid; b <= t.top; b += kPlanThreads) {
@@ -1720,8 +1718,12 @@ static cudaError_t plan_attributes() {
   return once_per_device(once, [] {
     cudaError_t e = allow_shared(k_hist, kHistSub * CVLC_HIST_BINS * 4);
     if (e == cudaSuccess) e = allow_shared(k_plan_fit, kFitSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<false>, kClusterSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<true>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<8, false>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<8, true>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<16, false>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<16, true>, kClusterSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_client<16, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_client<16, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e != cudaSuccess ? e : allow_shared(k_plan_tune, kTuneSmem);
   });
 }
@@ -1791,7 +1793,9 @@ cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& s
   memcpy(batch.c, clients, (size_t)n * sizeof(ClientDesc));
   const uint32_t rows = (uint32_t)make_partition(shape.d, n).rows;
   if (n > 1) launch_zero(clients, n, w, 256, enc.ws, 256, st);
-  launch_kernel(kKClient, n > 1 ? k_client<false> : k_client<true>, kClusterBlocks * n, kPlanThreads, kClusterSmem, st, n > 1, batch, shape, rows, w, enc);
+  const uint32_t blocks = cluster_blocks(rows, n);
+  auto kernel = blocks == 16 ? (n > 1 ? k_client<16, false> : k_client<16, true>) : (n > 1 ? k_client<8, false> : k_client<8, true>);
+  launch_kernel(kKClient, kernel, blocks * n, kPlanThreads, kClusterSmem, st, n > 1, batch, shape, rows, w, enc);
   return cudaGetLastError();
 }
 

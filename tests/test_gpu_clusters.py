@@ -1,6 +1,6 @@
 """GPU parity of cvlc_compress_batch where a cluster of blocks per client plans, selects and ranks: at most 15 clients of up to 327,683
-coordinates.  Sizes around its limits and its blocks' slices (rows of 16 coordinates, an eighth each, a ragged tail in the last block),
-and updates whose candidates crowd into bins that a block cannot hold."""
+coordinates (eight blocks), at most 7 of 245,764 to 655,363 (sixteen).  Sizes around its limits and its blocks' slices (rows of 16
+coordinates, an eighth or a sixteenth each, a ragged tail in the last block), and updates whose candidates crowd into bins that a block cannot hold."""
 import numpy as np
 import pytest
 
@@ -41,7 +41,8 @@ def check(xs, pds, side, fixed_y=0, checked=3):
     return B.cvlc_launch_count("k_client") - before
 
 
-@pytest.mark.parametrize("d,n", [(2, 1), (5, 2), (127, 1), (129, 3), (2_047, 15), (40_961, 5), (100_003, 1), (300_000, 3), (327_680, 2), (327_683, 1)])
+@pytest.mark.parametrize("d,n", [(2, 1), (5, 2), (127, 1), (129, 3), (2_047, 15), (40_961, 5), (100_003, 1), (300_000, 3), (245_763, 7), (245_764, 7), (327_680, 8), (327_683, 1),
+                                 (400_001, 3), (655_363, 7)])
 @pytest.mark.parametrize("side", [False, True])
 def test_sizes(d, n, side):
     rng = np.random.default_rng(d)
@@ -52,7 +53,7 @@ def test_sizes(d, n, side):
 
 def test_limits():
     rng = np.random.default_rng(0)
-    for d, n, bits in [(327_684, 1, 0.5), (4_000, 16, 0.5), (300_000, 1, 4.0)]:  # coordinates, clients, candidates: the kernels of their own
+    for d, n, bits in [(327_684, 8, 0.3), (655_364, 1, 0.3), (4_000, 16, 0.5), (300_000, 1, 4.0)]:  # coordinates, clients, candidates: the kernels of their own
         pds = [params_dict(d, int(bits * d), seed=c, packet_bits=1024) for c in range(n)]
         assert check([update("normal", d, rng) for _ in range(n)], pds, True, checked=2) == 0
 
