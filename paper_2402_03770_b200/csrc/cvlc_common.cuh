@@ -477,9 +477,11 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
 cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
 // Few small clients: planning, selection and ranking by a cluster of blocks per client (see k_client).  All clusters run at a time, every block
-// keeps its share of the coordinates in shared memory; few candidates, so that the blocks that rank have one tile each.
+// keeps its share of the coordinates in shared memory, and no more candidates than a block ranks in two tiles.  From 32,768 candidates on, the
+// kernels of their own and this, us: 1 / 7 / 12 clients of 320,000 coordinates at 4 / 4 / 2.8 bits 51 and 44 / 61 and 50 / 67 and 59, 12 of 240,000 at
+// 4 bits 66 and 57, 3 of 600,000 at 3 bits 63 and 52, 1 / 7 of 655,000 at 4 / 3 bits 58 and 55 / 73 and 66.
 constexpr uint32_t kClusterUnits = 10240;  // float4 units that a block keeps
-constexpr uint64_t kClusterCandidates = 32768;
+constexpr uint64_t kClusterCandidates = 65536;
 // Blocks of a client's cluster; 0: too many clients or coordinates.  Clusters that run at a time, a block on an SM
 // (cudaOccupancyMaxActiveClusters): 15 of eight blocks, 7 of sixteen.  Sixteen exchange more counts, eight read longer; whole calls with the
 // aggregation, eight and sixteen, us: one client of 100,000 coordinates 39.0 and 40.6, of 200,000 41.0 and 41.0, of 320,000 44.1 and 42.7, seven

@@ -464,6 +464,10 @@ __device__ __forceinline__ uint32_t hist_add4(uint32_t* my, const float4 a) {
   return m01 > m23 ? m01 : m23;
 }
 
+__device__ __forceinline__ uint32_t largest_key(const float4& a) {
+  return max(max(__float_as_uint(a.x) & 0x7FFFFFFFu, __float_as_uint(a.y) & 0x7FFFFFFFu), max(__float_as_uint(a.z) & 0x7FFFFFFFu, __float_as_uint(a.w) & 0x7FFFFFFFu));
+}
+
 __global__ void __launch_bounds__(kHistThreads, 3)
 k_hist(const Batch batch, const __grid_constant__ Shape shape, const __grid_constant__ Partition part, unsigned char* ws,
        const __grid_constant__ EncFront enc, int finish) {
@@ -1528,8 +1532,9 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // Every block keeps its share of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's shared
 // memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
 // knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a second
-// barrier all blocks but the last rank a share each, in whole bins, while that one fits the exponent and tunes the lengths.  Bins that a block
-// cannot hold (equal values) are left to k_rank_rest.
+// barrier all blocks but the last rank a share each, in whole bins, while that one fits the exponent and tunes the lengths.  Bins of more
+// than a block holds are cut again (see rank_large_bin); cells of more than 256 equal or nearly equal keys are left to k_rank_rest, whose blocks work
+// them off side by side.
 // Bound by latencies: of 19 us for one client of 100,000 coordinates and 26 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
 // of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
 // events) the steps took 30 and 39; whole calls 36.9 -> 26.7 us, 56.7 -> 45.5 with the aggregation.
@@ -1544,6 +1549,79 @@ constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) 
 constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 16;
 static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
               kClusterSmem <= 216 * 1024, "shared memory");
+
+// A bin of a few more candidates than a block holds, by one block: cut into 64 equal ranges of its keys, which are ranked as many as fit at a time.
+// A bin of more, as equal values fill it, or with a range of too many, is left to k_rank_rest.
+constexpr uint32_t kBinRanges = 64, kBinRangeBits = 13, kBinCut = 2 * kRankItems;
+static_assert(kBinRanges << kBinRangeBits == 1u << 19, "a bin");
+__device__ __noinline__ void rank_large_bin(RankShared& s, EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop, u64 inv,
+                                            const u64* src, u64* out, uint32_t at, uint32_t m) {
+  __shared__ uint32_t s_start[kBinRanges + 1], s_next[kBinRanges];
+  const int tid = threadIdx.x;
+  auto range_of = [](u64 item) -> uint32_t { return (~(uint32_t)(item >> 32) & 0x7FFFFu) >> kBinRangeBits; };
+  if (tid < (int)kBinRanges) s_next[tid] = 0;
+  __syncthreads();
+  for_items<kPlanThreads>(src, m, [&](uint32_t, u64 item) { atomicAdd(s_next + range_of(item), 1u); });
+  __syncthreads();
+  uint32_t most = 0;
+  for (uint32_t r = 0; r < kBinRanges; ++r) most = max(most, s_next[r]);
+  if (tid == 0) {
+    uint32_t run = 0;
+    for (uint32_t r = 0; r < kBinRanges; ++r) {
+      s_start[r] = run;
+      run += s_next[r];
+    }
+    s_start[kBinRanges] = run;
+  }
+  __syncthreads();
+  if (most > kRankItems) {
+    if (tid == 0) list_bucket(hdr, ws, L, c, keytop, inv, inv + (1u << 19), at, m);
+    return;
+  }
+  if (tid < (int)kBinRanges) s_next[tid] = s_start[tid];
+  __syncthreads();
+  for_items<kPlanThreads>(src, m, [&](uint32_t, u64 item) { out[atomicAdd(s_next + range_of(item), 1u)] = item; });
+  __syncthreads();
+  for (uint32_t lo = 0; lo < kBinRanges;) {
+    uint32_t hi = lo + 1;
+    while (hi < kBinRanges && s_start[hi + 1] - s_start[lo] <= kRankItems) ++hi;
+    const uint32_t first = s_start[lo], n = s_start[hi] - first;
+    if (n)
+      rank_and_leave<kPlanThreads>(s, out + first, n, (uint32_t)inv + (lo << kBinRangeBits), ((hi - lo) << kBinRangeBits) - 1, out + first, keytop, hdr,
+                                   reinterpret_cast<ulonglong2*>(ws + L.off_list[1]), reinterpret_cast<const u64*>(ws + L.off_buf_a));
+    lo = hi;
+  }
+}
+
+// A block's candidates to their places where one bin holds a good part of all coordinates, as the threshold's does with zeros or one magnitude among the
+// candidates: a warp takes the places in that bin together, its counter would give them out one after the other.
+__device__ __noinline__ void put_crowded(uint32_t* place, uint32_t bin, const float4* data, uint32_t units, uint32_t u0, unsigned long long* by_bin) {
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t i0 = 0; i0 < units; i0 += kPlanThreads) {
+    const uint32_t i = i0 + threadIdx.x;
+    const bool on = i < units;
+    const float4 a = on ? data[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t v[4] = {__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(a.z), __float_as_uint(a.w)};
+    uint32_t together = 0, before = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned in = __ballot_sync(kFull, on && (v[j] & 0x7FFFFFFFu) >> 19 == bin);
+      together += __popc(in);
+      before += __popc(in & ((1u << lane) - 1u));
+    }
+    uint32_t at = 0;
+    if (lane == 0 && together) at = atomicAdd(place + bin, together);
+    at = __shfl_sync(kFull, at, 0) + before;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t key = v[j] & 0x7FFFFFFFu, b = key >> 19;
+      if (on && b >= bin) {
+        const uint32_t to = b == bin ? at++ : atomicAdd(place + b, 1u);
+        by_bin[to] = ((unsigned long long)key << 32) | (unsigned long long)((v[j] & 0x80000000u) | (4 * (u0 + i) + j));
+      }
+    }
+  }
+}
 
 // FIRST: the call's only kernel before packing (one client): it clears the headers
 template <int CL, bool FIRST>
@@ -1577,7 +1655,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + CL - 1) / CL * kRowUnits;
   const uint32_t u0 = min(q * slice, nvec), units = min(u0 + slice, nvec) - u0;
   uint16_t* __restrict__ row_max = reinterpret_cast<uint16_t*>(ws + plan_off_row_max(n)) + (size_t)c * rows;
-  uint32_t top = 0, tail = 0;
+  uint32_t top = 0, tail = 0, zeros = 0;
   const bool has_tail = q == CL - 1 && tid < (int)(shape.d & 3);
   if (has_tail) tail = __float_as_uint(x[4 * (size_t)nvec + tid]);
   constexpr int kLoads = 8;
@@ -1594,7 +1672,9 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
         uint32_t m = 0;
         if (on) {
           data[i] = a[u];
-          m = hist_add4(S.own, a[u]);
+          m = largest_key(a[u]);
+          if (m == 0) zeros += 4;  // a counter takes one addition a cycle
+          else hist_add4(S.own, a[u]);
         }
         top = max(top, m);
         m = max(m, __shfl_xor_sync(kFull, m, 1));
@@ -1603,6 +1683,8 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       }
     }
   }
+  zeros = __reduce_add_sync(kFull, zeros);
+  if (lane == 0 && zeros) atomicAdd(S.own, zeros);
   if (has_tail) {
     top = max(top, tail & 0x7FFFFFFFu);
     atomicAdd(S.own + ((tail & 0x7FFFFFFFu) >> 19), 1u);
@@ -1654,14 +1736,18 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       const uint32_t key = b & 0x7FFFFFFFu;
       if (key >= thresh) by_bin[atomicAdd(S.place + (key >> 19), 1u)] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | index);
     };
+    if (t.fullest > shape.d / 16) {
+      put_crowded(S.place, t.bin, data, units, u0, by_bin);
+    } else {
 #pragma unroll 4
-    for (uint32_t i = tid; i < units; i += kPlanThreads) {
-      const float4 a = data[i];
-      const uint32_t at = 4 * (u0 + i);
-      put(__float_as_uint(a.x), at);
-      put(__float_as_uint(a.y), at + 1);
-      put(__float_as_uint(a.z), at + 2);
-      put(__float_as_uint(a.w), at + 3);
+      for (uint32_t i = tid; i < units; i += kPlanThreads) {
+        const float4 a = data[i];
+        const uint32_t at = 4 * (u0 + i);
+        put(__float_as_uint(a.x), at);
+        put(__float_as_uint(a.y), at + 1);
+        put(__float_as_uint(a.z), at + 2);
+        put(__float_as_uint(a.w), at + 3);
+      }
     }
     if (has_tail) put(tail, 4 * nvec + tid);
   }
@@ -1700,10 +1786,14 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       }
     const uint32_t m = N[lo + 1] - at;
     const u64 inv = (u64)((int)t.top - hi) << 19, end = (u64)((int)t.top - lo) << 19;
-    if (m > kRankItems) {
+    if (m > kBinCut) {
       if (tid == 0) list_bucket(reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, inv, end, at, m);
+    } else if (m > kRankItems) {
+      rank_large_bin(*reinterpret_cast<RankShared*>(rest), reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, inv, by_bin + at, out + at, at, m);
     } else if (m) {
-      rank_with_cells<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), out + at, keytop);
+      rank_and_leave<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), out + at, keytop,
+                                   reinterpret_cast<EncHeader*>(enc.ws), reinterpret_cast<ulonglong2*>(enc.ws + L.off_list[1]),
+                                   reinterpret_cast<const u64*>(enc.ws + L.off_buf_a));
     }
     hi = lo;
   }

@@ -650,19 +650,50 @@ __device__ __forceinline__ BigBucket big_bucket(const RankArgs& a, int round, ui
 __device__ __forceinline__ const u64* big_source(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_a : a.buf_b) + pos; }
 __device__ __forceinline__ u64* big_target(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_b : a.buf_a) + pos; }
 
-// Ranks m <= kRankItems items in [base, base + span] of inv, with the cells of equal keys among them; by the whole block
+// A cell of up to kWarpCell items, by one warp of the block
 template <int THREADS>
-__device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop) {
+__device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32_t m) {
+  static_assert(kWarpCell * (THREADS / 32) <= kRankItems, "room for every warp's cell");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  u64* mine = s.items + warp * kWarpCell;
+  for (uint32_t i = lane; i < m; i += 32) mine[i] = to_value(at[i]);
+  __syncwarp();
+  if (!rank_equal_by_warp<THREADS>(s.cell + warp * kWarpCells, mine, m, at)) {
+    bitonic_sort(mine, m, lane, 32, [] { __syncwarp(); });
+    for (uint32_t i = lane; i < m; i += 32) at[i] = to_item(mine[i]);
+    __syncwarp();
+  }
+}
+
+// Ranks m <= kRankItems items in [base, base + span] of inv, with the cells of equal keys among them; by the whole block.  large(where, items) for
+// those that a warp cannot rank
+template <int THREADS, class Large>
+__device__ __forceinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+                                                Large&& large) {
   __shared__ uint32_t s_n, s_big[kRankItems / kCompareAll];
   if (threadIdx.x == 0) s_n = 0;
   rank_buckets<THREADS>(s, src, m, base, span, out, keytop,
                         [&](u64* where, uint32_t items) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
   const uint32_t n_big = s_n;
-  for (uint32_t g = 0; g < n_big; ++g) {
-    u64* at = out + (s_big[g] & 0xFFFFu);
-    rank_cell<THREADS>(s, at, s_big[g] >> 16, at);
-  }
+  for (uint32_t g = threadIdx.x >> 5; g < n_big; g += THREADS / 32)
+    if (s_big[g] >> 16 <= kWarpCell) rank_cell_by_warp<THREADS>(s, out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
   __syncthreads();
+  for (uint32_t g = 0; g < n_big; ++g)
+    if (s_big[g] >> 16 > kWarpCell) large(out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
+  __syncthreads();
+}
+// ... by the block, one after the other
+template <int THREADS>
+__device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop) {
+  rank_with_cells<THREADS>(s, src, m, base, span, out, keytop, [&](u64* at, uint32_t items) { rank_cell<THREADS>(s, at, items, at); });
+}
+// ... by k_rank_rest, by all its blocks
+template <int THREADS>
+__device__ __noinline__ void rank_and_leave(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+                                            EncHeader* hdr, ulonglong2* list, const u64* buf_a) {
+  rank_with_cells<THREADS>(s, src, m, base, span, out, keytop, [&](u64* at, uint32_t items) {
+    if (threadIdx.x == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(at - buf_a), items);
+  });
 }
 
 // Ranks n <= kRankItems items whose keys lie between two, the larger one first; by the whole block
@@ -960,7 +991,7 @@ template <int THREADS>
 __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const RankArgs& a) {
   __shared__ RankTile s_tile;
   __shared__ uint32_t s_entry;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   __syncthreads();  // the arguments are there
   const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the selection alone
   if (big) {
@@ -986,23 +1017,13 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
     }
   }
   __syncthreads();
-  static_assert(kWarpCell * (THREADS / 32) <= kRankItems, "room for every warp's cell");
-  u64* mine = s.items + warp * kWarpCell;
   while (true) {
     uint32_t g = 0;
     if (lane == 0) g = atomicAdd(&hdr->list_next[0], 1u);
     g = __shfl_sync(kFull, g, 0);
     if (g >= hdr->list_n[0]) break;
     const ulonglong2 e = a.list[0][g];
-    const uint32_t m = (uint32_t)e.y;
-    u64* at = a.buf_a + e.x;
-    for (uint32_t i = lane; i < m; i += 32) mine[i] = to_value(at[i]);
-    __syncwarp();
-    if (!rank_equal_by_warp<THREADS>(s.cell + warp * kWarpCells, mine, m, at)) {
-      bitonic_sort(mine, m, lane, 32, [] { __syncwarp(); });
-      for (uint32_t i = lane; i < m; i += 32) at[i] = to_item(mine[i]);
-      __syncwarp();
-    }
+    rank_cell_by_warp<THREADS>(s, a.buf_a + e.x, (uint32_t)e.y);
   }
   if (!big) return;
   __syncthreads();

@@ -21,6 +21,10 @@ def update(kind, d, rng):
         x[rng.random(d) < 0.999] = 0.0
     elif kind == "signs":
         x = np.sign(x)
+    elif kind == "narrow":  # all candidates in one bin of the histogram, a few thousand in each range of it
+        x = np.where(rng.random(d) < 0.12, np.sign(x) * rng.uniform(1.0, 1.04, d), x * 1e-3)
+    elif kind == "steps":  # ... and on eight values of it
+        x = np.where(rng.random(d) < 0.12, np.sign(x) * (1.0 + rng.integers(0, 8, d) / 256.0), x * 1e-3)
     elif kind == "front":  # all candidates in the first block's slice
         x[d // 12:] *= 1e-6
     return x.astype(np.float32)
@@ -53,17 +57,17 @@ def test_sizes(d, n, side):
 
 def test_limits():
     rng = np.random.default_rng(0)
-    for d, n, bits in [(327_684, 8, 0.3), (655_364, 1, 0.3), (4_000, 16, 0.5), (300_000, 1, 4.0)]:  # coordinates, clients, candidates: the kernels of their own
+    for d, n, bits in [(327_684, 8, 0.3), (655_364, 1, 0.3), (4_000, 16, 0.5), (655_000, 1, 5.0)]:  # coordinates, clients, candidates: the kernels of their own
         pds = [params_dict(d, int(bits * d), seed=c, packet_bits=1024) for c in range(n)]
         assert check([update("normal", d, rng) for _ in range(n)], pds, True, checked=2) == 0
 
 
-@pytest.mark.parametrize("kind", ["normal", "equal", "grid", "zeros", "signs", "front"])
+@pytest.mark.parametrize("kind", ["normal", "equal", "grid", "zeros", "signs", "front", "narrow", "steps"])
 @pytest.mark.parametrize("quantizer", [0, 1])
-def test_distributions(kind, quantizer):
+@pytest.mark.parametrize("d,n,bits", [(200_003, 4, 2.0), (327_001, 3, 4.0), (600_001, 2, 4.0)])
+def test_distributions(kind, quantizer, d, n, bits):
     rng = np.random.default_rng(3)
-    d, n = 200_003, 4
-    pds = [params_dict(d, 2 * d, seed=c, client_id=c, quantizer=quantizer) for c in range(n)]
+    pds = [params_dict(d, int(bits * d), seed=c, client_id=c, quantizer=quantizer) for c in range(n)]
     check([update(kind if c % 2 == 0 else "layers", d, rng) for c in range(n)], pds, True, checked=2)
 
 
