@@ -327,7 +327,8 @@ int cvlc_decode_aggregate_unframed(const uint8_t* const* streams_dev, const uint
  * length tuning (Algorithm 1 steps 2-14, a latency-bound computation that leaves the memory system idle)
  * runs next to them, one of the two on side_stream, and is joined right before the packets are assembled.
  * (Which one is a matter of the batch's size: the tuning, or, where the selection would keep every SM to
- * itself, selection and ranking.)
+ * itself, selection and ranking.  A few small clients are planned, selected and ranked by one kernel;
+ * side_stream is then not used.)
  *  plan_ws_dev / enc_ws_dev   workspaces sized by cvlc_plan_batch_workspace_bytes and
  *                             cvlc_encode_batch_workspace_bytes (with the same max_candidates)
  *  side_stream                a second stream of the same device, or NULL / the same stream: everything

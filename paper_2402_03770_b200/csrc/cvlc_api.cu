@@ -477,6 +477,7 @@ int cvlc_ec_accumulate_batch(float* const* memory_dev, const float* const* updat
                                                                                                                   : CVLC_ERR_CUDA;
 }
 
+static std::mutex compress_order;  // see cvlc_compress_batch
 // Two events per device order the two streams of cvlc_compress_batch (created on first use, kept until exit).
 static cudaError_t compress_events(cudaEvent_t* fork, cudaEvent_t* join) {
   static cudaEvent_t ev[64][2];
@@ -526,6 +527,11 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   Senc.fixed_y = 0;
   const EncFront front{static_cast<unsigned char*>(enc_ws_dev), enc_layout(S.d, n, cap)};
   if (by_clusters(S, n, desc[0].cap0)) {  // the second stream has nothing to do: the tuning is in the same kernel
+    if (two) {  // made by the first call with two streams, whatever its clients, for those that follow it in a stream capture
+      std::lock_guard<std::mutex> hold(compress_order);
+      cudaEvent_t fork, join;
+      if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
+    }
     if (launch_clients(desc, n, S, plan_ws_dev, front, main_st) != cudaSuccess) return CVLC_ERR_CUDA;
     return launch_encode(desc, n, Senc, cap, plan_ws_dev, enc_ws_dev, main_st, true, false, nullptr, kPackFramed, true) == cudaSuccess ? CVLC_OK : CVLC_ERR_CUDA;
   }
@@ -540,8 +546,7 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   // different scales, 2961 instead of 2935 for one normal distribution; but the tuning takes 25 us to 3 ms, and then in front of the
   // selection: magnitudes that fall as rank^-1 3294 instead of 2945 us, as rank^-1.3 4622 instead of 3093.)  The lock keeps two threads from
   // recording the device's events between each other's record and wait.
-  static std::mutex order;
-  std::lock_guard<std::mutex> hold(order);
+  std::lock_guard<std::mutex> hold(compress_order);
   cudaEvent_t fork, join;
   if (compress_events(&fork, &join) != cudaSuccess) return CVLC_ERR_CUDA;
   if (cudaEventRecord(fork, main_st) != cudaSuccess || cudaStreamWaitEvent(side_st, fork, 0) != cudaSuccess) return CVLC_ERR_CUDA;

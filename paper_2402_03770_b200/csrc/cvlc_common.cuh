@@ -658,7 +658,7 @@ __device__ __forceinline__ void add_client(EncHeader* hdr, const ClientRank& r, 
   if (r.split) atomicMax(&hdr->most_split, r.n);
 }
 // Candidates per tile of the final ranking: as many as make the tiles of all clients whole rounds of the blocks, as few rounds as
-// tiles of at most kRankWindow allow.  With powers of two, at least four tiles an SM, some blocks had a tile more than the others:
+// tiles of at most `largest` allow.  With powers of two, at least four tiles an SM, some blocks had a tile more than the others:
 // one client of 11.2 M coordinates (2048 in 1.4 rounds, now 2800 in one) 18.0 -> 15.6 us between events, 8 of 1.2 M 17.3 -> 14.8, one
 // of 52 M, with what is left over, 73 -> 48.
 __device__ __forceinline__ uint32_t rank_window(uint32_t most, uint32_t n, uint32_t blocks, uint32_t largest) {
