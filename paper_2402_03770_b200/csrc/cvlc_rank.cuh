@@ -665,35 +665,42 @@ __device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32
   }
 }
 
-// Ranks m <= kRankItems items in [base, base + span] of inv, with the cells of equal keys among them; by the whole block.  large(where, items) for
-// those that a warp cannot rank
-template <int THREADS, class Large>
-__device__ __forceinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
-                                                Large&& large) {
-  __shared__ uint32_t s_n, s_big[kRankItems / kCompareAll];
+// Ranks m <= kRankItems items in [base, base + span] of inv, but for the cells of more than kCompareAll items, whose places and items go to
+// `cells`; returns how many.  By the whole block.
+template <int THREADS>
+__device__ __forceinline__ uint32_t rank_but_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+                                                   uint32_t (&cells)[kRankItems / kCompareAll]) {
+  __shared__ uint32_t s_n;
   if (threadIdx.x == 0) s_n = 0;
   rank_buckets<THREADS>(s, src, m, base, span, out, keytop,
-                        [&](u64* where, uint32_t items) { s_big[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
-  const uint32_t n_big = s_n;
-  for (uint32_t g = threadIdx.x >> 5; g < n_big; g += THREADS / 32)
-    if (s_big[g] >> 16 <= kWarpCell) rank_cell_by_warp<THREADS>(s, out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
-  __syncthreads();
-  for (uint32_t g = 0; g < n_big; ++g)
-    if (s_big[g] >> 16 > kWarpCell) large(out + (s_big[g] & 0xFFFFu), s_big[g] >> 16);
-  __syncthreads();
+                        [&](u64* where, uint32_t items) { cells[atomicAdd(&s_n, 1u)] = (uint32_t)(where - out) | items << 16; }, [] {});
+  return s_n;
 }
-// ... by the block, one after the other
+// ... with those cells, by the block one after the other.  (Those of up to 256 by its warps side by side, as in clusters: one client of 11.2 M
+// coordinates in 255 steps 163.5 -> 167.6 us, on a grid of 24 steps per deviation 163.8 -> 169.7, one of 5 M 122.0 -> 126.5.)
 template <int THREADS>
 __device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop) {
-  rank_with_cells<THREADS>(s, src, m, base, span, out, keytop, [&](u64* at, uint32_t items) { rank_cell<THREADS>(s, at, items, at); });
+  __shared__ uint32_t s_cell[kRankItems / kCompareAll];
+  const uint32_t n = rank_but_cells<THREADS>(s, src, m, base, span, out, keytop, s_cell);
+  for (uint32_t g = 0; g < n; ++g) {
+    u64* at = out + (s_cell[g] & 0xFFFFu);
+    rank_cell<THREADS>(s, at, s_cell[g] >> 16, at);
+  }
+  __syncthreads();
 }
-// ... by k_rank_rest, by all its blocks
+// ... by its warps; those that a warp cannot rank by k_rank_rest, by all its blocks
 template <int THREADS>
 __device__ __noinline__ void rank_and_leave(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
                                             EncHeader* hdr, ulonglong2* list, const u64* buf_a) {
-  rank_with_cells<THREADS>(s, src, m, base, span, out, keytop, [&](u64* at, uint32_t items) {
-    if (threadIdx.x == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(at - buf_a), items);
-  });
+  __shared__ uint32_t s_cell[kRankItems / kCompareAll];
+  const uint32_t n = rank_but_cells<THREADS>(s, src, m, base, span, out, keytop, s_cell);
+  for (uint32_t g = threadIdx.x >> 5; g < n; g += THREADS / 32) {
+    u64* at = out + (s_cell[g] & 0xFFFFu);
+    const uint32_t items = s_cell[g] >> 16;
+    if (items <= kWarpCell) rank_cell_by_warp<THREADS>(s, at, items);
+    else if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(at - buf_a), items);
+  }
+  __syncthreads();
 }
 
 // Ranks n <= kRankItems items whose keys lie between two, the larger one first; by the whole block
