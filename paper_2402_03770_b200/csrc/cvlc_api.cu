@@ -526,7 +526,9 @@ int cvlc_compress_batch(const float* const* x_dev, const cvlc_params* params, ui
   Shape Senc = S;
   Senc.fixed_y = 0;
   const EncFront front{static_cast<unsigned char*>(enc_ws_dev), enc_layout(S.d, n, cap)};
-  if (by_clusters(S, n, desc[0].cap0)) {  // the second stream has nothing to do: the tuning is in the same kernel
+  uint32_t cap0 = 0;  // the clients' scales may differ, and with them how much each may send
+  for (uint32_t i = 0; i < n; ++i) cap0 = desc[i].cap0 > cap0 ? desc[i].cap0 : cap0;
+  if (by_clusters(S, n, cap0)) {  // the second stream has nothing to do: the tuning is in the same kernel
     if (two) {  // made by the first call with two streams, whatever its clients, for those that follow it in a stream capture
       std::lock_guard<std::mutex> hold(compress_order);
       cudaEvent_t fork, join;

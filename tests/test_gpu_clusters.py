@@ -62,6 +62,21 @@ def test_limits():
         assert check([update("normal", d, rng) for _ in range(n)], pds, True, checked=2) == 0
 
 
+@pytest.mark.parametrize("side", [False, True])
+def test_the_limit_holds_for_every_client(side):
+    """Clients whose scales differ may send different numbers of records: the call takes clusters only if all of them may send up to
+    65,536, whichever stands first."""
+    d = 320_001
+    rng = np.random.default_rng(7)
+    xs = [update("layers", d, rng) for _ in range(3)]
+    # 130 packets; shortest lengths of 5 bits (130 * 496 records) and of 2 (130 * 567, beyond the limit)
+    few, many = (params_dict(d, 130 * 12_000, seed=c, scale_B=scale) for c, scale in ((1, None), (2, 100.0)))
+    assert check(xs, [few] * 3, side) == 1
+    assert check(xs, [many] * 3, side) == 0
+    assert check(xs, [few, many, few], side) == 0
+    assert check(xs, [many, few, few], side) == 0
+
+
 @pytest.mark.parametrize("kind", ["normal", "equal", "grid", "zeros", "signs", "front", "narrow", "steps"])
 @pytest.mark.parametrize("quantizer", [0, 1])
 @pytest.mark.parametrize("d,n,bits", [(200_003, 4, 2.0), (327_001, 3, 4.0), (600_001, 2, 4.0)])
