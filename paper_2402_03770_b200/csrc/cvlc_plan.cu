@@ -1533,7 +1533,7 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
 // knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a second
 // barrier all blocks but the last rank a share each, in whole bins, while that one fits the exponent and tunes the lengths.  Bins of more
-// than a block holds are cut again (see rank_large_bin); cells of more than 256 equal or nearly equal keys are left to k_rank_rest, whose blocks work
+// than a block holds are cut again (see cut_bins); cells of more than 256 equal or nearly equal keys are left to k_rank_rest, whose blocks work
 // them off side by side.
 // Bound by latencies: of 19 us for one client of 100,000 coordinates and 26 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
 // of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
@@ -1550,74 +1550,273 @@ constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 
 static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
               kClusterSmem <= 216 * 1024, "shared memory");
 
-// A bin of a few more candidates than a block holds, by one block: cut into 64 equal ranges of its keys, which are ranked as many as fit at a time.
-// A bin of more, as equal values fill it, or with a range of too many, is left to k_rank_rest.
-constexpr uint32_t kBinRanges = 64, kBinRangeBits = 13, kBinCut = 2 * kRankItems;
-static_assert(kBinRanges << kBinRangeBits == 1u << 19, "a bin");
-__device__ __noinline__ void rank_large_bin(RankShared& s, EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop, u64 inv,
-                                            const u64* src, u64* out, uint32_t at, uint32_t m) {
-  __shared__ uint32_t s_start[kBinRanges + 1], s_next[kBinRanges];
-  const int tid = threadIdx.x;
-  auto range_of = [](u64 item) -> uint32_t { return (~(uint32_t)(item >> 32) & 0x7FFFFu) >> kBinRangeBits; };
-  if (tid < (int)kBinRanges) s_next[tid] = 0;
-  __syncthreads();
-  for_items<kPlanThreads>(src, m, [&](uint32_t, u64 item) { atomicAdd(s_next + range_of(item), 1u); });
-  __syncthreads();
-  uint32_t most = 0;
-  for (uint32_t r = 0; r < kBinRanges; ++r) most = max(most, s_next[r]);
-  if (tid == 0) {
-    uint32_t run = 0;
-    for (uint32_t r = 0; r < kBinRanges; ++r) {
-      s_start[r] = run;
-      run += s_next[r];
-    }
-    s_start[kBinRanges] = run;
-  }
-  __syncthreads();
-  if (most > kRankItems) {
-    if (tid == 0) list_bucket(hdr, ws, L, c, keytop, inv, inv + (1u << 19), at, m);
-    return;
-  }
-  if (tid < (int)kBinRanges) s_next[tid] = s_start[tid];
-  __syncthreads();
-  for_items<kPlanThreads>(src, m, [&](uint32_t, u64 item) { out[atomicAdd(s_next + range_of(item), 1u)] = item; });
-  __syncthreads();
-  for (uint32_t lo = 0; lo < kBinRanges;) {
-    uint32_t hi = lo + 1;
-    while (hi < kBinRanges && s_start[hi + 1] - s_start[lo] <= kRankItems) ++hi;
-    const uint32_t first = s_start[lo], n = s_start[hi] - first;
-    if (n)
-      rank_and_leave<kPlanThreads>(s, out + first, n, (uint32_t)inv + (lo << kBinRangeBits), ((hi - lo) << kBinRangeBits) - 1, out + first, keytop, hdr,
-                                   reinterpret_cast<ulonglong2*>(ws + L.off_list[1]), reinterpret_cast<const u64*>(ws + L.off_buf_a));
-    lo = hi;
+// One more in counters of a table for each of the lanes' values that is on: what was in them before.  One addition where all of the warp's go to
+// one counter (which takes one a cycle), or all of a lane's.
+template <int V>
+__device__ __forceinline__ void add_all(uint32_t* table, const bool (&on)[V], const uint32_t (&i)[V], uint32_t (&at)[V]) {
+  bool all = true;
+#pragma unroll
+  for (int u = 0; u < V; ++u) all = all && on[u] && i[u] == i[0];
+  const uint32_t lane = threadIdx.x & 31, first = __shfl_sync(kFull, i[0], 0);
+  if (__all_sync(kFull, all && i[0] == first)) {
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(table + first, 32u * V);
+    at[0] = __shfl_sync(kFull, base, 0) + lane;
+#pragma unroll
+    for (uint32_t u = 1; u < V; ++u) at[u] = at[0] + 32 * u;
+  } else if (all) {
+    at[0] = atomicAdd(table + i[0], (uint32_t)V);
+#pragma unroll
+    for (uint32_t u = 1; u < V; ++u) at[u] = at[0] + u;
+  } else {
+#pragma unroll
+    for (int u = 0; u < V; ++u) at[u] = on[u] ? atomicAdd(table + i[u], 1u) : 0u;
   }
 }
 
-// A block's candidates to their places where one bin holds a good part of all coordinates, as the threshold's does with zeros or one magnitude among the
-// candidates: a warp takes the places in that bin together, its counter would give them out one after the other.
-__device__ __noinline__ void put_crowded(uint32_t* place, uint32_t bin, const float4* data, uint32_t units, uint32_t u0, unsigned long long* by_bin) {
-  const uint32_t lane = threadIdx.x & 31;
+// A block's candidates to their places where a bin holds many
+__device__ __noinline__ void put_crowded(uint32_t* place, uint32_t thresh_bin, const float4* data, uint32_t units, uint32_t u0, unsigned long long* by_bin) {
   for (uint32_t i0 = 0; i0 < units; i0 += kPlanThreads) {
     const uint32_t i = i0 + threadIdx.x;
-    const bool on = i < units;
-    const float4 a = on ? data[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 a = i < units ? data[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t v[4] = {__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(a.z), __float_as_uint(a.w)};
-    uint32_t together = 0, before = 0;
+    uint32_t bin[4], at[4];
+    bool on[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const unsigned in = __ballot_sync(kFull, on && (v[j] & 0x7FFFFFFFu) >> 19 == bin);
-      together += __popc(in);
-      before += __popc(in & ((1u << lane) - 1u));
+    for (int u = 0; u < 4; ++u) {
+      bin[u] = (v[u] & 0x7FFFFFFFu) >> 19;
+      on[u] = i < units && bin[u] >= thresh_bin;
     }
-    uint32_t at = 0;
-    if (lane == 0 && together) at = atomicAdd(place + bin, together);
-    at = __shfl_sync(kFull, at, 0) + before;
+    add_all(place, on, bin, at);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t key = v[j] & 0x7FFFFFFFu, b = key >> 19;
-      if (on && b >= bin) {
-        const uint32_t to = b == bin ? at++ : atomicAdd(place + b, 1u);
-        by_bin[to] = ((unsigned long long)key << 32) | (unsigned long long)((v[j] & 0x80000000u) | (4 * (u0 + i) + j));
+    for (uint32_t u = 0; u < 4; ++u)
+      if (on[u]) by_bin[at[u]] = ((unsigned long long)(v[u] & 0x7FFFFFFFu) << 32) | (unsigned long long)((v[u] & 0x80000000u) | (4 * (u0 + i) + u));
+  }
+}
+
+// ---- bins of more candidates than a block ranks: values crowded in a bin, repeated ones, zeros --------------------------------
+// Cut by all ranking blocks of the cluster, beside the tuning: every block counts a share of such a bin's candidates by the next nine bits of (key,
+// index), the counts are added up in global memory, and the candidates go to the places of their parts.  Parts that are still too large
+// are cut again; after the third cut a part is what 4096 neighbouring coordinates have of one key.
+// A cut is a chain of latencies: reading, counting and moving 1 to 5 us each, two waits of the blocks for one another 1.5 each.  Left to k_rank_rest, as large
+// buckets of other batches are, such bins came behind the tuning and took 45 to 120 us there.  Whole calls, as kernels of their own / left to
+// k_rank_rest / cut, us: 36,000 candidates spread over one bin, ten clients of 300,000 coordinates 57 / 107 / 47; on eight values 74 / 125 / 65;
+// signs only, one of 600,000 107 / 120 / 78, ten of 300,000 183 / 142 / 80; 5 % of one magnitude, one of 600,000 104 / 106 / 64; 98 % zeros, one of
+// 320,000 101 / 101 / 91.  But one client of 600,000 in 16 bits (fp16, 59,500 records) 59 / 84 / 68: 15 blocks rank where 296 did.
+constexpr uint32_t kCutParts = 512, kCutRanges = 8, kCuts = 3, kCutTable = kCutRanges * kCutParts;
+static_assert(kCutParts == kPlanThreads && kCutParts == 16 * 32 && kCutTable <= CVLC_HIST_BINS && kCutRanges <= kPlanThreads / 32, "one part per thread");
+static_assert((kRankItems + 1) * kCutRanges > kClusterCandidates, "room for all ranges that begin with a rank that may be sent");
+static_assert(2 * kCutTable <= kRankSubs, "the tables' place");
+static_assert(16 * 4 * kClusterUnits + 3 < 1u << 20, "bits of an index");
+struct Cut {
+  uint32_t n;                   // ranges that are cut
+  uint32_t prefix[kCutRanges];  // their bits of (key's complement, index), those that follow say the part
+  uint32_t start[kCutRanges], size[kCutRanges];
+  uint32_t part[kCutRanges];    // their parts of the cut before (of the first cut: bins)
+  bool in_a;                    // their candidates lie in the first buffer and go to the second
+};
+__device__ __forceinline__ uint32_t cut_part(u64 item, uint32_t cut) {
+  const uint32_t inv_key = ~(uint32_t)(item >> 32);
+  return cut == 0 ? (inv_key >> 10) & 511u : cut == 1 ? (inv_key >> 1) & 511u : (inv_key & 1u) << 8 | ((uint32_t)item & 0x7FFFFFFFu) >> 12;
+}
+// keytop - key where part `part` of range r begins
+__device__ __forceinline__ uint32_t cut_inv(const Cut& C, uint32_t cut, uint32_t r, uint32_t part, uint32_t keytop) {
+  const uint32_t inv_key = cut == 2 ? (C.prefix[r] << 1) + (part >> 8) : ((C.prefix[r] << 9) + part) << (cut == 0 ? 10 : 1);
+  return inv_key - (0x7FFFFFFFu - keytop);
+}
+// what the parts of a cut hold, and the ranks that they begin with; the first are zero when the cutting begins
+__device__ __forceinline__ uint32_t* cut_totals(unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t cut) {
+  return cut < 2 ? reinterpret_cast<uint32_t*>(ws + L.off_sub_start) + (size_t)c * (kRankSubs + 64) + cut * kCutTable
+                 : reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs;
+}
+__device__ __forceinline__ uint32_t* cut_starts(unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t cut) {
+  return cut < 2 ? reinterpret_cast<uint32_t*>(ws + L.off_sub_count) + (size_t)c * kRankSubs + cut * kCutTable
+                 : reinterpret_cast<uint32_t*>(ws + L.off_sub_pos) + (size_t)c * kRankSubs + kCutTable;
+}
+// the ranking blocks' turns behind one another
+__device__ __forceinline__ uint32_t* cut_turns(unsigned char* ws, const EncLayout& L, uint32_t c) { return reinterpret_cast<uint32_t*>(ws + L.off_group_done) + c; }
+
+// f(items, which of them are there), kCutHold of src[lo .. hi) a thread at a time, by whole warps
+constexpr int kCutHold = 8;
+template <class F>
+__device__ __forceinline__ void by_eights(const u64* src, uint32_t lo, uint32_t hi, F&& f) {
+  for (uint32_t i0 = lo; i0 < hi; i0 += kCutHold * kPlanThreads) {
+    const uint32_t first = i0 + kCutHold * (threadIdx.x & ~31u) + (threadIdx.x & 31u);  // a warp's are neighbours
+    u64 v[kCutHold];
+    bool on[kCutHold];
+#pragma unroll
+    for (uint32_t u = 0; u < kCutHold; ++u) {
+      on[u] = first + 32 * u < hi;
+      v[u] = on[u] ? __ldcg(src + first + 32 * u) : 0ull;
+    }
+    f(v, on);
+  }
+}
+
+// By the ranking blocks of the cluster, q of `blocks`; N: the client's survival counts; table: of kCutTable counters.  False: a wait has run out.
+__device__ __noinline__ bool cut_bins(uint32_t* table, const uint32_t* N, Cut* cuts, const Threshold& t, uint32_t limit, unsigned char* ws, const EncLayout& L,
+                                      uint32_t c, uint32_t q, uint32_t blocks, u64* buf_a, u64* buf_b) {
+  __shared__ uint32_t s_found[kCutRanges][kCutRanges][3], s_n[kCutRanges];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int32_t* status = &reinterpret_cast<EncHeader*>(ws)->status;
+  uint32_t* turns = cut_turns(ws, L, c);
+  uint32_t turn = 0;
+  if (warp == 0) {
+    uint32_t n = 0;
+    for (int b0 = (int)t.top; b0 >= (int)t.bin; b0 -= 32) {
+      const int b = b0 - lane;
+      const uint32_t m = b >= (int)t.bin ? N[b] - N[b + 1] : 0u;
+      const unsigned large = __ballot_sync(kFull, m > kRankItems);
+      const uint32_t at = n + __popc(large & ((1u << lane) - 1u));
+      if (m > kRankItems && at < kCutRanges) {
+        cuts[0].prefix[at] = 4095u - (uint32_t)b;
+        cuts[0].start[at] = N[b + 1];
+        cuts[0].size[at] = m;
+        cuts[0].part[at] = (uint32_t)b;
+      }
+      n += __popc(large);
+    }
+    if (lane == 0) {
+      cuts[0].n = min(n, kCutRanges);
+      cuts[0].in_a = false;
+    }
+  }
+  for (uint32_t cut = 0; cut < kCuts; ++cut) {
+    const Cut& C = cuts[cut];
+    __syncthreads();
+    const uint32_t n = C.n;
+    if (n == 0) break;
+    for (uint32_t i = tid; i < n * kCutParts; i += kPlanThreads) table[i] = 0;
+    __syncthreads();
+    const u64* src = C.in_a ? buf_a : buf_b;
+    u64* dst = C.in_a ? buf_b : buf_a;
+    uint32_t* totals = cut_totals(ws, L, c, cut);
+    // f(items, which there are, their entries of the table, their places) of the block's share of the ranges
+    auto share = [&](auto&& f) {
+      for (uint32_t r = 0; r < n; ++r) {
+        const uint32_t m = C.size[r];
+        by_eights(src + C.start[r], m * q / blocks, m * (q + 1) / blocks, [&](const u64 (&v)[kCutHold], bool (&on)[kCutHold]) {
+          uint32_t e[kCutHold], at[kCutHold];
+#pragma unroll
+          for (int u = 0; u < kCutHold; ++u) e[u] = r * kCutParts + cut_part(v[u], cut);
+          f(v, on, e, at);
+        });
+      }
+    };
+    share([&](const u64 (&)[kCutHold], bool (&on)[kCutHold], const uint32_t (&e)[kCutHold], uint32_t (&at)[kCutHold]) { add_all(table, on, e, at); });
+    __syncthreads();
+    for (uint32_t i = tid; i < n * kCutParts; i += kPlanThreads) table[i] = table[i] ? atomicAdd(totals + i, table[i]) : 0u;
+    block_done(turns);
+    if (!block_waits(turns, ++turn * blocks, status)) return false;
+    if (warp < (int)n) {  // a warp per range, a lane for 16 parts
+      uint32_t v[16], sum = 0;
+#pragma unroll
+      for (int i = 0; i < 16; i += 4) {
+        const uint4 w = __ldcg(reinterpret_cast<const uint4*>(totals + warp * kCutParts + lane * 16 + i));
+        v[i] = w.x;
+        v[i + 1] = w.y;
+        v[i + 2] = w.z;
+        v[i + 3] = w.w;
+        sum += w.x + w.y + w.z + w.w;
+      }
+      uint32_t at = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_up_sync(kFull, at, off);
+        if (lane >= off) at += o;
+      }
+      at += C.start[warp] - sum;
+      uint32_t found = 0;
+      uint32_t* starts = cut_starts(ws, L, c, cut) + warp * kCutParts + lane * 16;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const uint32_t part = lane * 16 + i;
+        const bool again = v[i] > kRankItems && at < limit && cut + 1 < kCuts;
+        const unsigned all = __ballot_sync(kFull, again);
+        const uint32_t k = found + __popc(all & ((1u << lane) - 1u));
+        if (again && k < kCutRanges) {
+          s_found[warp][k][0] = part;
+          s_found[warp][k][1] = at;
+          s_found[warp][k][2] = v[i];
+        }
+        found += __popc(all);
+        uint32_t* mine = table + warp * kCutParts + part;
+        *mine = at < limit ? *mine + at : 0x80000000u;  // not moved where it is never sent
+        if (q == 0) starts[i] = at;
+        at += v[i];
+      }
+      if (lane == 0) s_n[warp] = min(found, kCutRanges);
+    }
+    __syncthreads();
+    if (tid == 0 && cut + 1 < kCuts) {
+      Cut& next = cuts[cut + 1];
+      uint32_t m = 0;
+      bool whole = true;  // a range is one part
+      for (uint32_t r = 0; r < n; ++r) {
+        whole = whole && s_n[r] == 1 && s_found[r][0][2] == C.size[r] && m < kCutRanges;
+        for (uint32_t k = 0; k < s_n[r] && m < kCutRanges; ++k, ++m) {
+          next.prefix[m] = C.prefix[r] << 9 | s_found[r][k][0];
+          next.start[m] = s_found[r][k][1];
+          next.size[m] = s_found[r][k][2];
+          next.part[m] = r * kCutParts + s_found[r][k][0];
+        }
+      }
+      next.n = m;
+      next.in_a = whole ? C.in_a : !C.in_a;
+    }
+    __syncthreads();
+    if (cut + 1 < kCuts && cuts[cut + 1].in_a == C.in_a) continue;  // they stay where they are
+    share([&](const u64 (&v)[kCutHold], bool (&on)[kCutHold], const uint32_t (&e)[kCutHold], uint32_t (&at)[kCutHold]) {
+#pragma unroll
+      for (int u = 0; u < kCutHold; ++u) on[u] = on[u] && table[e[u]] < 0x80000000u;
+      add_all(table, on, e, at);
+#pragma unroll
+      for (int u = 0; u < kCutHold; ++u)
+        if (on[u]) dst[at[u]] = v[u];
+    });
+    block_done(turns);
+    if (!block_waits(turns, ++turn * blocks, status)) return false;
+  }
+  return true;
+}
+
+// The parts whose candidates begin with the ranks [first, end), as many of a range as a block holds at a time; by the whole block
+__device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop,
+                                        u64* buf_a, u64* buf_b, uint32_t first, uint32_t end) {
+  __shared__ uint32_t s_start[kCutParts + 1];
+  const uint32_t tid = threadIdx.x;
+  for (uint32_t cut = 0; cut < kCuts && cuts[cut].n; ++cut) {
+    const Cut& C = cuts[cut];
+    const u64* src = C.in_a ? buf_b : buf_a;
+    for (uint32_t r = 0; r < C.n; ++r) {
+      if (C.start[r] >= end || C.start[r] + C.size[r] <= first) continue;
+      __syncthreads();
+      s_start[tid] = __ldcg(cut_starts(ws, L, c, cut) + r * kCutParts + tid);
+      if (tid == 0) s_start[kCutParts] = C.start[r] + C.size[r];
+      __syncthreads();
+      uint32_t i = __syncthreads_count(s_start[tid] < first);
+      while (i < kCutParts && s_start[i] < end) {
+        uint32_t stop = cut == 2 && i < kCutParts / 2 ? kCutParts / 2 : kCutParts;  // (one key at a time)
+        if (cut + 1 < kCuts)  // those that have been cut again lie between
+          for (uint32_t k = 0; k < cuts[cut + 1].n; ++k) {
+            const uint32_t part = cuts[cut + 1].part[k] - r * kCutParts;
+            if (part >= i && part < stop) stop = part;
+          }
+        if (stop == i) {
+          ++i;
+          continue;
+        }
+        const uint32_t at = s_start[i];
+        const uint32_t fit = __syncthreads_count(tid >= i && tid < stop && s_start[tid] < end && s_start[tid + 1] - at <= kRankItems);
+        const uint32_t behind = i + fit, m = s_start[behind] - at;  // one at least: what does not fit has been cut again
+        const uint32_t inv = cut_inv(C, cut, r, i, keytop), inv_end = cut_inv(C, cut, r, behind, keytop);
+        if (m && cut == 2) {
+          rank_cell<kPlanThreads>(s, src + at, m, buf_a + at);
+        } else if (m) {
+          rank_and_leave<kPlanThreads>(s, src + at, m, inv, inv_end - inv - 1, buf_a + at, keytop, hdr, reinterpret_cast<ulonglong2*>(ws + L.off_list[1]),
+                                       reinterpret_cast<const u64*>(ws + L.off_buf_a));
+        }
+        i = behind;
       }
     }
   }
@@ -1634,6 +1833,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   unsigned char* rest = smem_raw + sizeof(ClusterShared);
   float4* data = reinterpret_cast<float4*>(rest);
   __shared__ int s_bin[2];
+  __shared__ Cut s_cut[kCuts];
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t c = blockIdx.x / CL, q = blockIdx.x % CL, n = batch.n;
@@ -1725,7 +1925,8 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
                                        q == 0 ? reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS : nullptr);
   if (q == 0 && tid == 0) write_client(c, n, cd.plan, t, nonfinite, shape, ws, enc);
   const EncLayout& L = enc.L;
-  const bool go = !nonfinite && t.n <= L.capacity;
+  const bool go = !nonfinite && t.n <= L.capacity, crowded = t.fullest > kRankItems;
+  const uint32_t limit = shape.R * cd.cap0;  // ranks from here on are not sent (see by_clusters)
   unsigned long long* by_bin = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_b) + (size_t)c * L.capacity;
   // ---- the candidates to their bins
   if (go) {
@@ -1736,8 +1937,10 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       const uint32_t key = b & 0x7FFFFFFFu;
       if (key >= thresh) by_bin[atomicAdd(S.place + (key >> 19), 1u)] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | index);
     };
-    if (t.fullest > shape.d / 16) {
+    if (crowded) {
       put_crowded(S.place, t.bin, data, units, u0, by_bin);
+      for (uint32_t i = q * kPlanThreads + tid; i < kCuts * kCutTable; i += CL * kPlanThreads) cut_totals(enc.ws, L, c, i / kCutTable)[i % kCutTable] = 0;
+      if (q == 0 && tid == 0) *cut_turns(enc.ws, L, c) = 0;
     } else {
 #pragma unroll 4
       for (uint32_t i = tid; i < units; i += kPlanThreads) {
@@ -1762,7 +1965,9 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   cluster.sync();
   if (!go) return;
   // ---- the bins whose candidates begin in the block's share of the ranks
-  const uint32_t limit = rank_limit(shape), ranked = min(t.n, limit);
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_a) + (size_t)c * L.capacity;
+  if (crowded && !cut_bins(S.total, N, s_cut, t, limit, enc.ws, L, c, q, CL - 1, out, by_bin)) return;
+  const uint32_t ranked = min(t.n, limit);
   const uint32_t share = (ranked + CL - 2) / (CL - 1);
   if (tid < 2) s_bin[tid] = (int)t.bin - 1;
   __syncthreads();
@@ -1775,7 +1980,6 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   }
   __syncthreads();
   const int last = s_bin[1];
-  unsigned long long* out = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_a) + (size_t)c * L.capacity;
   const uint32_t keytop = sort_keytop(t.top);
   for (int hi = s_bin[0]; hi > last;) {  // bins (lo, hi], as many as a block holds
     const uint32_t at = N[hi + 1];
@@ -1792,17 +1996,16 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
     }
     const uint32_t m = N[lo + 1] - at;
     const u64 inv = (u64)((int)t.top - hi) << 19, end = (u64)((int)t.top - lo) << 19;
-    if (m > kBinCut) {
-      if (tid == 0) list_bucket(reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, inv, end, at, m);
-    } else if (m > kRankItems) {
-      rank_large_bin(*reinterpret_cast<RankShared*>(rest), reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, inv, by_bin + at, out + at, at, m);
-    } else if (m) {
+    if (m && m <= kRankItems) {  // else it is one bin, which has been cut
       rank_and_leave<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), out + at, keytop,
                                    reinterpret_cast<EncHeader*>(enc.ws), reinterpret_cast<ulonglong2*>(enc.ws + L.off_list[1]),
                                    reinterpret_cast<const u64*>(enc.ws + L.off_buf_a));
     }
     hi = lo;
   }
+  if (crowded)
+    rank_parts(*reinterpret_cast<RankShared*>(rest), s_cut, reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, out, by_bin, q * share,
+               min((q + 1) * share, ranked));
 }
 
 // ===================================================================================

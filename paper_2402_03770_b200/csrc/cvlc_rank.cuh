@@ -650,19 +650,23 @@ __device__ __forceinline__ BigBucket big_bucket(const RankArgs& a, int round, ui
 __device__ __forceinline__ const u64* big_source(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_a : a.buf_b) + pos; }
 __device__ __forceinline__ u64* big_target(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_b : a.buf_a) + pos; }
 
-// A cell of up to kWarpCell items, by one warp of the block
+// A cell of up to kWarpCell items, whose values are `mine`, by one warp of the block
 template <int THREADS>
-__device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32_t m) {
-  static_assert(kWarpCell * (THREADS / 32) <= kRankItems, "room for every warp's cell");
+__device__ __forceinline__ void rank_values_by_warp(RankShared& s, u64* mine, uint32_t m, u64* at) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  u64* mine = s.items + warp * kWarpCell;
-  for (uint32_t i = lane; i < m; i += 32) mine[i] = to_value(at[i]);
-  __syncwarp();
   if (!rank_equal_by_warp<THREADS>(s.cell + warp * kWarpCells, mine, m, at)) {
     bitonic_sort(mine, m, lane, 32, [] { __syncwarp(); });
     for (uint32_t i = lane; i < m; i += 32) at[i] = to_item(mine[i]);
     __syncwarp();
   }
+}
+template <int THREADS>
+__device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32_t m) {
+  static_assert(kWarpCell * (THREADS / 32) <= kRankItems, "room for every warp's cell");
+  u64* mine = s.items + (threadIdx.x >> 5) * kWarpCell;
+  for (uint32_t i = threadIdx.x & 31; i < m; i += 32) mine[i] = to_value(at[i]);
+  __syncwarp();
+  rank_values_by_warp<THREADS>(s, mine, m, at);
 }
 
 // Ranks m <= kRankItems items in [base, base + span] of inv, but for the cells of more than kCompareAll items, whose places and items go to
@@ -697,7 +701,7 @@ __device__ __noinline__ void rank_and_leave(RankShared& s, const u64* src, uint3
   for (uint32_t g = threadIdx.x >> 5; g < n; g += THREADS / 32) {
     u64* at = out + (s_cell[g] & 0xFFFFu);
     const uint32_t items = s_cell[g] >> 16;
-    if (items <= kWarpCell) rank_cell_by_warp<THREADS>(s, at, items);
+    if (items <= kWarpCell) rank_values_by_warp<THREADS>(s, s.items + (s_cell[g] & 0xFFFFu), items, at);
     else if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(at - buf_a), items);
   }
   __syncthreads();

@@ -79,16 +79,57 @@ def test_the_limit_holds_for_every_client(side):
 
 @pytest.mark.parametrize("kind", ["normal", "equal", "grid", "zeros", "signs", "front", "narrow", "steps"])
 @pytest.mark.parametrize("quantizer", [0, 1])
-@pytest.mark.parametrize("d,n,bits", [(200_003, 4, 2.0), (327_001, 3, 4.0), (600_001, 2, 4.0)])
+@pytest.mark.parametrize("d,n,bits", [(200_003, 4, 2.0), (327_001, 3, 4.0), (600_001, 2, 2.5)])
 def test_distributions(kind, quantizer, d, n, bits):
     rng = np.random.default_rng(3)
     pds = [params_dict(d, int(bits * d), seed=c, client_id=c, quantizer=quantizer) for c in range(n)]
-    check([update(kind if c % 2 == 0 else "layers", d, rng) for c in range(n)], pds, True, checked=2)
+    assert check([update(kind if c % 2 == 0 else "layers", d, rng) for c in range(n)], pds, True, checked=2) == 1
+
+
+def in_one_bin(m, values, d, rng):
+    """m coordinates at scattered places whose keys are 1.0 and the next `values` ones, as evenly as can be; the others a thousand times smaller"""
+    x = rng.standard_normal(d).astype(np.float32) * np.float32(1e-3)
+    low = rng.permutation(1 << 19)[:m] if values == 1 << 19 else np.arange(m) % values
+    at = rng.permutation(d)[:m]
+    x[at] = (0x3F800000 + low.astype(np.uint32)).astype(np.uint32).view(np.float32) * np.where(rng.random(m) < 0.5, -1.0, 1.0).astype(np.float32)
+    return x
+
+
+# all different: one cut, where a bin has more than 8192; 512 neighbouring keys: parts of one cut that are cut again; two and one: by coordinates
+@pytest.mark.parametrize("values", [1 << 19, 512, 2, 1])
+@pytest.mark.parametrize("m", [8_192, 8_193, 12_000, 16_384, 16_385, 33_000])
+@pytest.mark.parametrize("d,n", [(200_003, 2), (600_001, 1)])
+def test_bins_that_a_block_does_not_hold(values, m, d, n):
+    """what is sent ends inside the bin and behind it"""
+    rng = np.random.default_rng(m + values)
+    xs = [in_one_bin(m, values, d, rng) for _ in range(n)]
+    for sent in (m * 3 // 5, min(64_000, m + 9_000)):
+        pds = [params_dict(d, 12_000 * (sent // 530 + 1), seed=c, client_id=c) for c in range(n)]
+        assert check(xs, pds, True) == 1
+
+
+def test_as_many_bins_as_can_be_too_large():
+    """Seven bins of 8193 and more, one after the other and with others between, and one that is sent in part; a bin with seven such parts;
+    values next to one another where every cut leaves some too large"""
+    rng = np.random.default_rng(8)
+    d = 640_003
+    pd = params_dict(d, 12_000 * 137, seed=1)  # 65,212 records
+    x = rng.standard_normal(d).astype(np.float32) * np.float32(1e-4)
+    at = rng.permutation(d)[:80_000]
+    x[at] = (1.0 + (np.arange(80_000) // 8_200) / 16 + rng.random(80_000) / 17).astype(np.float32)
+    assert check([x], [pd], True) == 1
+    x[at] = (2.0 ** (np.arange(80_000) // 8_200) + rng.random(80_000) / 17).astype(np.float32)
+    assert check([x], [pd], False) == 1
+    x[at] = (0x3F800000 + (np.arange(80_000) // 8_200 * 2048).astype(np.uint32) + rng.integers(0, 512, 80_000).astype(np.uint32)).astype(np.uint32).view(np.float32)
+    assert check([x], [pd], True) == 1
+    x[at] = (0x3F800000 + (np.arange(80_000) // 20_000 * 1023).astype(np.uint32)).astype(np.uint32).view(np.float32)
+    assert check([x], [pd], True) == 1
 
 
 def test_fixed_length():
     rng = np.random.default_rng(4)
-    check([update("layers", 150_001, rng)], [params_dict(150_001, 150_001)], False, fixed_y=5)
+    assert check([update("layers", 150_001, rng)], [params_dict(150_001, 150_001)], False, fixed_y=5) == 1
+    assert check([in_one_bin(20_000, 3, 150_001, rng)], [params_dict(150_001, 360_000)], False, fixed_y=5) == 1
 
 
 def test_errors():
