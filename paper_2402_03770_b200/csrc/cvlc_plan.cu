@@ -1529,13 +1529,16 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // ===================================================================================
 // K1-K4 of few small clients: a cluster of blocks per client
 // ===================================================================================
-// Every block keeps its share of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's shared
-// memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
-// knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a second
-// barrier all blocks but the last rank a share each, in whole bins, while that one fits the exponent and tunes the lengths.  Bins of more
+// Every block but the last keeps its share of the update in shared memory and counts its bins.  The counts are exchanged through the cluster's
+// shared memory: every block then has the client's histogram and, for each bin, how many of its values are in the blocks before it, so that it
+// knows the place of each of its candidates by bin, without an addition in global memory.  They go there (the L2), and behind a third
+// barrier those blocks rank a share each, in whole bins, while the last one, which needs the histogram alone, has been fitting the exponent and
+// tuning the lengths.  (With a share of the update for that one too the tuning began 3 to 5 us later: one client of 100,000 coordinates whose
+// magnitudes fall as rank^-1.3 38.6 -> 37.0 us, ten of 300,000 at 0.4 bits 45.3 -> 41.3, a normal distribution 34.5 -> 31.0; one of 600,000 at 2.5
+// bits, where the ranking is what the cluster ends with, 37.1 -> 37.4.)  A share may be more than a block keeps; the rest is read again.  Bins of more
 // than a block holds are cut again (see cut_bins); cells of more than 256 equal or nearly equal keys are left to k_rank_rest, whose blocks work
 // them off side by side.
-// Bound by latencies: of 19 us for one client of 100,000 coordinates and 26 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
+// Bound by latencies: of 17 us for one client of 100,000 coordinates and 22 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
 // of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
 // events) the steps took 30 and 39; whole calls 36.9 -> 26.7 us, 56.7 -> 45.5 with the aggregation.
 
@@ -1852,11 +1855,11 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   // ---- the block's rows: kept, counted, their maxima written
   const float* __restrict__ x = cd.x;
   const float4* xv = reinterpret_cast<const float4*>(x);
-  const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + CL - 1) / CL * kRowUnits;
-  const uint32_t u0 = min(q * slice, nvec), units = min(u0 + slice, nvec) - u0;
+  const uint32_t nvec = (uint32_t)(shape.d >> 2), slice = (rows + CL - 2) / (CL - 1) * kRowUnits;
+  const uint32_t u0 = min(q * slice, nvec), units = q < CL - 1 ? min(u0 + slice, nvec) - u0 : 0u;
   uint16_t* __restrict__ row_max = reinterpret_cast<uint16_t*>(ws + plan_off_row_max(n)) + (size_t)c * rows;
   uint32_t top = 0, tail = 0, zeros = 0;
-  const bool has_tail = q == CL - 1 && tid < (int)(shape.d & 3);
+  const bool has_tail = q == CL - 2 && tid < (int)(shape.d & 3);
   if (has_tail) tail = __float_as_uint(x[4 * (size_t)nvec + tid]);
   constexpr int kLoads = 8;
   for (uint32_t i0 = 0; i0 < units; i0 += kLoads * kPlanThreads) {
@@ -1871,7 +1874,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
         const bool on = i < units;
         uint32_t m = 0;
         if (on) {
-          data[i] = a[u];
+          if (i < kClusterUnits) data[i] = a[u];
           m = largest_key(a[u]);
           if (m == 0) zeros += 4;  // a counter takes one addition a cycle
           else hist_add4(S.own, a[u]);
@@ -1929,7 +1932,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   const uint32_t limit = shape.R * cd.cap0;  // ranks from here on are not sent (see by_clusters)
   unsigned long long* by_bin = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_b) + (size_t)c * L.capacity;
   // ---- the candidates to their bins
-  if (go) {
+  if (go && q < CL - 1) {
     for (uint32_t b = t.bin + tid; b <= t.top; b += kPlanThreads) S.place[b] += N[b + 1];
     __syncthreads();
     const uint32_t thresh = t.bin << 19;
@@ -1937,36 +1940,33 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       const uint32_t key = b & 0x7FFFFFFFu;
       if (key >= thresh) by_bin[atomicAdd(S.place + (key >> 19), 1u)] = ((unsigned long long)key << 32) | (unsigned long long)((b & 0x80000000u) | index);
     };
+    auto put4 = [&](const float4 a, uint32_t at) {  // (by value: one load, ahead of the additions)
+      put(__float_as_uint(a.x), at);
+      put(__float_as_uint(a.y), at + 1);
+      put(__float_as_uint(a.z), at + 2);
+      put(__float_as_uint(a.w), at + 3);
+    };
+    const uint32_t kept = min(units, kClusterUnits);
     if (crowded) {
-      put_crowded(S.place, t.bin, data, units, u0, by_bin);
-      for (uint32_t i = q * kPlanThreads + tid; i < kCuts * kCutTable; i += CL * kPlanThreads) cut_totals(enc.ws, L, c, i / kCutTable)[i % kCutTable] = 0;
+      put_crowded(S.place, t.bin, data, kept, u0, by_bin);
+      put_crowded(S.place, t.bin, xv + u0 + kept, units - kept, u0 + kept, by_bin);
+      for (uint32_t i = q * kPlanThreads + tid; i < kCuts * kCutTable; i += (CL - 1) * kPlanThreads) cut_totals(enc.ws, L, c, i / kCutTable)[i % kCutTable] = 0;
       if (q == 0 && tid == 0) *cut_turns(enc.ws, L, c) = 0;
     } else {
+      for (uint32_t i = kept + tid; i < units; i += kPlanThreads) put4(__ldg(xv + u0 + i), 4 * (u0 + i));
 #pragma unroll 4
-      for (uint32_t i = tid; i < units; i += kPlanThreads) {
-        const float4 a = data[i];
-        const uint32_t at = 4 * (u0 + i);
-        put(__float_as_uint(a.x), at);
-        put(__float_as_uint(a.y), at + 1);
-        put(__float_as_uint(a.z), at + 2);
-        put(__float_as_uint(a.w), at + 3);
-      }
+      for (uint32_t i = tid; i < kept; i += kPlanThreads) put4(data[i], 4 * (u0 + i));
     }
     if (has_tail) put(tail, 4 * nvec + tid);
   }
+  cg::cluster_group::arrival_token token = cluster.barrier_arrive();
   if (q == CL - 1) {
-    __syncthreads();  // the kept rows have been read
-    cg::cluster_group::arrival_token token = cluster.barrier_arrive();
     const Batch all{reinterpret_cast<const ClientDesc*>(ws + plan_off_desc(n)), n};
     tune_client(c, all, shape, ws, nullptr, N, rest);
     cluster.barrier_wait(std::move(token));
     return;
   }
-  cluster.sync();
-  if (!go) return;
   // ---- the bins whose candidates begin in the block's share of the ranks
-  unsigned long long* out = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_a) + (size_t)c * L.capacity;
-  if (crowded && !cut_bins(S.total, N, s_cut, t, limit, enc.ws, L, c, q, CL - 1, out, by_bin)) return;
   const uint32_t ranked = min(t.n, limit);
   const uint32_t share = (ranked + CL - 2) / (CL - 1);
   if (tid < 2) s_bin[tid] = (int)t.bin - 1;
@@ -1980,6 +1980,10 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   }
   __syncthreads();
   const int last = s_bin[1];
+  cluster.barrier_wait(std::move(token));
+  if (!go) return;
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_a) + (size_t)c * L.capacity;
+  if (crowded && !cut_bins(S.total, N, s_cut, t, limit, enc.ws, L, c, q, CL - 1, out, by_bin)) return;
   const uint32_t keytop = sort_keytop(t.top);
   for (int hi = s_bin[0]; hi > last;) {  // bins (lo, hi], as many as a block holds
     const uint32_t at = N[hi + 1];
