@@ -10,13 +10,16 @@ namespace cvlc {
 constexpr int kPrepThreads = 1024;
 constexpr int kDecodeThreads = 256;
 // Blocks of a decode: five run at a time on an SM.  How many packets there are only the device knows; by coordinates and clients, at 2 bits a
-// coordinate, a packet or two for every warp, but 8 to 32 blocks per SM.  With 8 for all the second round of blocks left the chip half empty at
-// the end; blocks without a packet cost small batches (1 x 50 M in three windows 11 us with 32).  8, 20, 32 and 48 per SM, us: 100 clients of 11.2 M
-// coordinates at 2 bits 380, 372, 356 and 357, at 1 bit 200, 192, 194 and 195, 50 of 23.5 M 276, 260, 263 and 255, 30 of 18 M 131 to 136 each, 24 of
-// 3 M at 4 bits 59 each, 20 of 1.2 M 18.6, 18.6, 18.6 and 20.6.
-inline unsigned decode_blocks(uint64_t d, uint32_t n) {
-  const uint64_t want = d * n / 48000;
-  return (unsigned)(want < 8 * kNumSM ? 8 * kNumSM : want < 32 * kNumSM ? want : 32 * kNumSM);
+// coordinate and 1500 bytes a packet, a packet or two for every warp of all windows together, in whole rounds of the resident blocks, but 8 to 32 per
+// SM.  With 8 for all the second round left the chip half empty at the end; blocks without a packet are paid for in every window (1 x 50 M in
+// three windows 11 us with 32).  8, 20, 32 and 48 per SM, us: 100 clients of 11.2 M coordinates at 2 bits 380, 372, 356 and 357, at 1 bit 200, 192, 194 and
+// 195, 50 of 23.5 M 276, 260, 263 and 255, 30 of 18 M 131 to 136 each, 24 of 3 M at 4 bits 59 each, 20 of 1.2 M 18.6, 18.6, 18.6 and 20.6.  8 for all, a
+// packet or two for every warp of each window, and this, us: 8 clients of 30 M at 0.2 bits (4000 packets, two windows) 43.2, 45.0 and 43.2, 6 of 25 M at 2
+// bits (two windows) 94.6, 92.4 and 89.9; half as many blocks in one window 100 of 3 M at 2 bits 116, 107 and 112.
+constexpr uint64_t kDecodeResident = 5 * kNumSM;
+inline unsigned decode_blocks(uint64_t d, uint32_t n, uint64_t windows) {
+  const uint64_t want = d * n / (48000 * windows);
+  return (unsigned)(want < 2 * kDecodeResident ? 8 * kNumSM : want < 32 * kNumSM ? want / kDecodeResident * kDecodeResident : 32 * kNumSM);
 }
 constexpr uint32_t kDecStageWords = 512;  // packets up to 2 KB are staged in shared memory
 constexpr uint64_t kDecodeWindow = 24ull << 20;  // coordinates of the accumulator filled per decode launch (96 MB: inside the L2)
@@ -336,7 +339,7 @@ cudaError_t launch_decode(const uint8_t* const* streams, const uint64_t* stream_
     } else if (n_win > 1) {
       launch_kernel(kKPrefetchL2, k_prefetch_l2, grid, 256, 0, st, true, out + lo, hi - lo);
     }
-    launch_kernel(kKDecode, k_decode, decode_blocks(d, n), kDecodeThreads, ((size_t)n + 1) * 4, st, true, streams, n, d, s, out, w, lo, hi);
+    launch_kernel(kKDecode, k_decode, decode_blocks(d, n, n_win), kDecodeThreads, ((size_t)n + 1) * 4, st, true, streams, n, d, s, out, w, lo, hi);
   }
   return cudaGetLastError();
 }
