@@ -89,8 +89,12 @@ def gpu_plan_encode(x: np.ndarray, pd: dict, fixed_y: int = 0, device: str = "cu
         out = enc.compress([xd], side_stream=side, fixed_y=fixed_y)[0]
     else:
         enc = B.ClientEncoder(p, dev)
-        enc.out.fill_(0xAB)
-        out = enc.run(xd, fixed_y=fixed_y, use_plan_ws=use_plan_ws)
+        out = enc.out.fill_(0xAB)
+        if fixed_y:
+            B.cvlc_plan_fixed(xd, p, fixed_y, enc.plan, enc.plan_ws)
+        else:
+            B.cvlc_plan(xd, p, enc.plan, enc.plan_ws)
+        B.cvlc_encode(xd, p, enc.plan, out, enc.enc_ws, plan_ws=enc.plan_ws if use_plan_ws else None)
     status = enc.status()
     plan = B.read_plan(enc.plan)
     st = out.cpu().numpy().copy()

@@ -1,6 +1,6 @@
 """GPU parity of cvlc_compress_batch where a cluster of blocks per client plans, selects and ranks: at most 15 clients of up to 327,683
-coordinates (eight blocks), at most 7 of 245,764 to 655,363 (sixteen).  Sizes around its limits and its blocks' slices (rows of 16
-coordinates, an eighth or a sixteenth each, a ragged tail in the last block), and updates whose candidates crowd into bins that a block cannot hold."""
+coordinates (eight blocks), at most 7 of 245,764 to 655,363 (sixteen).  Sizes around its limits, its blocks' shares (rows of 16
+coordinates, a seventh or a fifteenth each, a ragged tail with the last) and what a block keeps of one (40,960 coordinates), and updates whose candidates crowd into bins that a block cannot hold."""
 import numpy as np
 import pytest
 
@@ -46,7 +46,8 @@ def check(xs, pds, side, fixed_y=0, checked=3):
 
 
 @pytest.mark.parametrize("d,n", [(2, 1), (5, 2), (127, 1), (129, 3), (2_047, 15), (40_961, 5), (100_003, 1), (300_000, 3), (245_763, 7), (245_764, 7), (327_680, 8), (327_683, 1),
-                                 (400_001, 3), (655_363, 7)])
+                                 (400_001, 3), (655_363, 7),
+                                 (286_720, 8), (286_833, 9), (614_400, 1), (614_465, 1)])
 @pytest.mark.parametrize("side", [False, True])
 def test_sizes(d, n, side):
     rng = np.random.default_rng(d)
@@ -144,6 +145,7 @@ def test_errors():
     enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
     bad = xs[1].clone()
     bad[d - 1] = float("inf")
+    before = B.cvlc_launch_count("k_client")
     enc.compress([xs[0], bad, xs[2]])
     assert enc.status() == B.CVLC_ERR_NONFINITE_INPUT
     outs = enc.compress(xs)
@@ -152,6 +154,10 @@ def test_errors():
     small = B.BatchEncoder([gpu_params(pd) for pd in pds], dev, max_candidates=256)
     small.compress(xs)
     assert small.status() == B.CVLC_ERR_WORKSPACE_TOO_SMALL
+    crowded = [torch.from_numpy(update("signs", d, rng)).to(dev)] * n  # bins that would be cut
+    small.compress(crowded)
+    assert small.status() == B.CVLC_ERR_WORKSPACE_TOO_SMALL
+    assert B.cvlc_launch_count("k_client") == before + 4
 
 
 def test_plan_workspace_serves_the_encoder():
@@ -164,7 +170,9 @@ def test_plan_workspace_serves_the_encoder():
     pds = [params_dict(d, d, seed=c) for c in range(n)]
     xs = [torch.from_numpy(update("layers", d, rng)).to(dev) for _ in range(n)]
     enc = B.BatchEncoder([gpu_params(pd) for pd in pds], dev)
+    before = B.cvlc_launch_count("k_client")
     want = [o.clone() for o in enc.compress(xs)]
+    assert B.cvlc_launch_count("k_client") == before + 1
     for o in enc.outs:
         o.zero_()
     got = enc.encode(xs)

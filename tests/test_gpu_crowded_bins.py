@@ -1,5 +1,5 @@
 """GPU parity of the ranking where the candidates crowd at one end of few histogram bins, as the memories of error compensation do
-below the threshold after some rounds."""
+below the threshold after some rounds: by separate calls, and by cvlc_compress_batch, which ranks the smaller two by clusters."""
 import numpy as np
 import pytest
 

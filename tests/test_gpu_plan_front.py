@@ -1,6 +1,7 @@
 """GPU parity of the planning front over the ways a batch can be cut: chunks of one client each, whose last block finishes the
 client, or chunks of the concatenated clients; exponent fit and tuning per client or shared by clients of one key; with and without a
-side stream.  Sizes at the edges of rows (16 coordinates) and chunks (256 rows); clients with different scales, so that their
+side stream.  Up to fifteen such small clients are planned by clusters in these calls, so the planning call is checked as well, and
+sixteen clients of the same sizes.  Sizes at the edges of rows (16 coordinates) and chunks (256 rows); clients with different scales, so that their
 shortest lengths differ."""
 import numpy as np
 import pytest
@@ -35,8 +36,16 @@ def run_batch(xs, pds, side):
     return status, plans, [o.cpu().numpy() for o in outs]
 
 
+def plan_batch(xs, pds):
+    import torch
+    from paper_2402_03770_b200 import binding as B
+    enc = B.BatchEncoder([gpu_params(pd) for pd in pds], torch.device("cuda:0"))
+    enc.plan([torch.from_numpy(x).to("cuda:0") for x in xs])
+    return [enc.read_plan(i) for i in range(len(xs))]
+
+
 @pytest.mark.parametrize("d,n", [(200, 1), (255, 5), (4095, 1), (4096, 3), (4097, 1), (8193, 2), (20_000, 11), (3_000, 33), (2_000, 148),
-                                 (1_500, 149), (400, 400), (100_003, 3)])
+                                 (1_500, 149), (400, 400), (100_003, 3), (200, 16), (255, 17), (4095, 16), (4096, 18), (4097, 16), (8193, 17), (700_003, 1)])
 def test_every_cut_gives_the_oracles_plan_and_stream(d, n):
     xs, pds = make_batch(d, n, seed=d + n)
     refs = [oracle_plan_encode(x, pd) for x, pd in zip(xs, pds)]
@@ -46,9 +55,11 @@ def test_every_cut_gives_the_oracles_plan_and_stream(d, n):
         for (fields, stream), plan, out in zip(refs, plans, outs):
             assert_plan_equal(plan, fields)
             assert np.array_equal(out, stream)
+    for (fields, _), plan in zip(refs, plan_batch(xs, pds)):
+        assert_plan_equal(plan, fields)
 
 
-@pytest.mark.parametrize("n,bad", [(1, 0), (4, 3), (40, 17), (149, 148)])
+@pytest.mark.parametrize("n,bad", [(1, 0), (4, 3), (16, 9), (40, 17), (149, 148)])
 def test_non_finite_client_stops_the_batch_and_keeps_the_others_plans(n, bad):
     xs, pds = make_batch(1_777, n, seed=n)
     xs[bad][1_776] = np.inf
@@ -60,3 +71,4 @@ def test_non_finite_client_stops_the_batch_and_keeps_the_others_plans(n, bad):
                 assert plan.status == O.ORC_ERR_NONFINITE_INPUT
             else:
                 assert_plan_equal(plan, oracle_plan_encode(xs[c], pds[c])[0])
+    assert [plan.status for plan in plan_batch(xs, pds)] == [O.ORC_ERR_NONFINITE_INPUT if c == bad else O.ORC_OK for c in range(n)]

@@ -1,5 +1,6 @@
 """GPU parity of the ranking over the sizes of its tiles: candidates that make one round of the blocks or a little more, from the
-smallest tile (1024) to the largest (4096), one client and several of different sizes; the window is whatever makes whole rounds."""
+smallest tile (1024) to the largest (4096), one client and several of different sizes; the window is whatever makes whole rounds.  (One client of
+one packet is ranked by a cluster, sixteen are not.)"""
 import numpy as np
 import pytest
 
@@ -8,7 +9,7 @@ from gpu_util import gpu_params, oracle_plan_encode, params_dict
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,R", [(1, 1), (1, 620), (1, 700), (1, 1_500), (1, 2_400), (1, 2_700), (3, 260), (20, 41)])
+@pytest.mark.parametrize("n,R", [(1, 1), (16, 1), (1, 620), (1, 700), (1, 1_500), (1, 2_400), (1, 2_700), (3, 260), (20, 41)])
 @pytest.mark.parametrize("side", [False, True])
 def test_tiles_of_any_size(n, R, side):
     import torch

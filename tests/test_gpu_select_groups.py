@@ -1,5 +1,6 @@
 """GPU parity of the selection over the ways its groups of rows are cut: runs of 16 rows (256 coordinates) spread over a client, in
-groups of two runs in small batches and of eight in larger ones, the client's last rows and its ragged tail among them.  Nearly all
+groups of two runs in small batches and of eight in larger ones, the client's last rows and its ragged tail among them.  (Up to fifteen
+small clients are selected by clusters; sixteen of the same sizes, and 700,003 coordinates, are not.)  Nearly all
 candidates lie in one layer, at the front, in the middle or at the end; few or many sub-buckets are summed up at a client's end."""
 import numpy as np
 import pytest
@@ -10,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,n", [(17, 1), (255, 2), (256, 1), (257, 1), (511, 3), (513, 1), (4_096, 1), (36_867, 1), (40_960, 12),
-                                 (360_000, 16), (5_762_049, 1), (5_800_003, 2)])
+                                 (360_000, 16), (5_762_049, 1), (5_800_003, 2), (17, 16), (255, 17), (256, 16), (257, 16), (511, 18), (513, 16),
+                                 (4_096, 16), (36_867, 16), (40_960, 17), (700_003, 1)])
 @pytest.mark.parametrize("layer", ["front", "middle", "end"])
 def test_a_dense_layer_anywhere(d, n, layer):
     import torch

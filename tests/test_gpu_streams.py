@@ -9,6 +9,7 @@ from gpu_util import assert_aggregate_close, gpu_params, oracle_params, params_d
 pytestmark = pytest.mark.gpu
 
 D, N = 200_003, 3
+FORKED = 700_003  # coordinates of clients that cvlc_compress_batch does not give to clusters: the length tuning runs on the side stream
 KINDS = ["client", "compress", "separate", "ec", "decode", "unframed", "decode_unframed"]
 
 
@@ -16,10 +17,10 @@ class Calls:
     """Buffers of N clients.  `load` puts one of two sets of inputs in place, `run` makes the calls of a kind on the current stream,
     `check` compares what they left with the oracle's for a set of inputs."""
 
-    def __init__(self, kind):
+    def __init__(self, kind, D=D):
         import torch
         from paper_2402_03770_b200 import binding as B
-        self.torch, self.B, self.kind = torch, B, kind
+        self.torch, self.B, self.kind, self.D = torch, B, kind, D
         self.dev = dev = torch.device("cuda:0")
         rng = np.random.default_rng(len(kind))
         self.pds = [params_dict(D, 2 * D, seed=11 + c, client_id=c) for c in range(N)]
@@ -82,7 +83,7 @@ class Calls:
             B.cvlc_encode_unframed_batch(self.xs, self.params, enc.plans, self.bytes_out, self.sizes, enc.enc_ws, self.uf_ws, 0,
                                          plan_ws=enc.plan_ws)
         else:
-            B.cvlc_decode_aggregate_unframed(self.agg.ptrs, self.agg.sizes, self.agg.weights, N, 0.0, D, self.out, False, self.agg.ws)
+            B.cvlc_decode_aggregate_unframed(self.agg.ptrs, self.agg.sizes, self.agg.weights, N, 0.0, self.D, self.out, False, self.agg.ws)
 
     def check(self, which):
         self.torch.cuda.synchronize()
@@ -104,10 +105,13 @@ class Calls:
                 assert (self.memories[c].cpu().numpy() == O.ec_residual(self.updates[which][c], ref)).all()
 
 
-@pytest.mark.parametrize("kind", KINDS)
-def test_inputs_behind_an_event_wait(kind):
+SIZES = [(kind, D) for kind in KINDS] + [("client", FORKED), ("compress", FORKED)]
+
+
+@pytest.mark.parametrize("kind,d", SIZES)
+def test_inputs_behind_an_event_wait(kind, d):
     """The stream holds a finished call on other inputs, then a wait for the stream that is still making the right ones."""
-    calls = Calls(kind)
+    calls = Calls(kind, d)
     torch = calls.torch
     work, maker, made = torch.cuda.Stream(calls.dev), torch.cuda.Stream(calls.dev), torch.cuda.Event()
     with torch.cuda.stream(work):
@@ -126,10 +130,10 @@ def test_inputs_behind_an_event_wait(kind):
         calls.check(which)
 
 
-@pytest.mark.parametrize("kind", KINDS)
-def test_capture_into_a_graph(kind):
-    """One capture, replayed for two sets of inputs; the length tuning's fork is captured with it."""
-    calls = Calls(kind)
+@pytest.mark.parametrize("kind,d", SIZES)
+def test_capture_into_a_graph(kind, d):
+    """One capture, replayed for two sets of inputs; with the larger clients the length tuning's fork is captured with it."""
+    calls = Calls(kind, d)
     torch = calls.torch
     warm = torch.cuda.Stream(calls.dev)
     with torch.cuda.stream(warm):  # attributes are set and modules loaded before the capture
@@ -145,13 +149,48 @@ def test_capture_into_a_graph(kind):
         calls.check(which)
 
 
+def test_capture_behind_a_call_by_clusters():
+    """In a process of its own: a two-stream call of a small client, which forks nothing, is enough for one that does to be captured."""
+    import os
+    import subprocess
+    import sys
+    code = """if 1:
+        import numpy as np, torch
+        from gpu_util import gpu_params, oracle_plan_encode, params_dict
+        from paper_2402_03770_b200 import binding as B
+        dev = torch.device("cuda:0")
+        side, ready = torch.cuda.Stream(dev), []
+        for d in (20_001, 700_003):
+            x = np.random.default_rng(d).laplace(0, 1e-3, d).astype(np.float32)
+            pd = params_dict(d, d)
+            ready.append((B.BatchEncoder([gpu_params(pd)], dev), torch.from_numpy(x).to(dev), oracle_plan_encode(x, pd)[1]))
+        ready[1][0].run([ready[1][1]])  # its kernels' attributes, without a second stream
+        ready[1][0].compress([ready[1][1]])
+        ready[0][0].compress([ready[0][1]], side_stream=side)
+        torch.cuda.synchronize()
+        assert B.cvlc_launch_count("k_client") == 1
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            ready[1][0].compress([ready[1][1]], side_stream=side)
+        ready[1][0].outs[0].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for enc, _, stream in ready:
+            assert enc.status() == 0 and np.array_equal(enc.outs[0].cpu().numpy(), stream)
+        """
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here)] + os.environ.get("PYTHONPATH", "").split(os.pathsep)))
+    done = subprocess.run([sys.executable, "-c", code], env=env, timeout=120, capture_output=True, text=True)
+    assert done.returncode == 0, done.stderr
+
+
 def test_calls_from_several_threads():
-    """Every thread on a stream and buffers of its own; no launch is missing from the count."""
+    """Every thread on a stream and buffers of its own; no launch is missing from the count.  Four of them share the device's two events."""
     import threading
     import torch
     from paper_2402_03770_b200 import binding as B
     kinds = ["client", "compress", "separate", "ec", "decode", "unframed", "decode_unframed", "compress"]
-    work = [Calls(kind) for kind in kinds]
+    work = [Calls(kind) for kind in kinds] + [Calls(kind, FORKED) for kind in ("client", "compress", "compress", "client")]
     each = []
     for calls in work:
         calls.load(0)

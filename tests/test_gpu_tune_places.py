@@ -1,4 +1,4 @@
-"""GPU parity of cvlc_compress_batch over where the length tuning runs: beside a selection that leaves it SMs, behind a short selection of
+"""GPU parity of cvlc_compress_batch over where the length tuning runs: in the clusters of few small clients, beside a selection that leaves it SMs, behind a short selection of
 many clients, ahead of a long one with the clients tuned each for itself or together, and on one stream.  Every second client's magnitudes
 fall as a steep power law, whose tuning takes longer than its selection; both quantizers, fixed lengths, a client that is not finite
 and a workspace for too few candidates."""
@@ -10,7 +10,8 @@ from gpu_util import assert_plan_equal, gpu_params, oracle_plan_encode, params_d
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(100_003, 3),     # room left
+SHAPES = [(100_003, 3),     # clusters, which tune in the same kernel
+          (700_003, 3),     # room left
           (40_000, 33),     # behind
           (4_200_001, 33),  # ahead, one tuning per key, the threshold by the fit's kernel
           (3_150_001, 32),  # ahead, a tuning per client, the threshold by a kernel of its own
