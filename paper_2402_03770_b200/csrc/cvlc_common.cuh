@@ -492,8 +492,10 @@ inline uint32_t cluster_blocks(uint64_t rows, uint32_t n) {
   if (n <= 7 && rows > 6 * of_block && rows <= 16 * of_block) return 16;
   return n <= 15 && rows <= 8 * of_block ? 8 : 0;
 }
+bool clusters_run(uint32_t blocks);  // on the current device: a part of a GPU may have too few SMs side by side
 inline bool by_clusters(const Shape& shape, uint32_t n, uint32_t cap0) {  // cap0: the largest of the clients'
-  return cluster_blocks(make_partition(shape.d, n).rows, n) != 0 && (uint64_t)shape.R * cap0 <= kClusterCandidates;
+  const uint32_t blocks = cluster_blocks(make_partition(shape.d, n).rows, n);
+  return blocks != 0 && (uint64_t)shape.R * cap0 <= kClusterCandidates && clusters_run(blocks);
 }
 cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st);
 cudaError_t launch_histogram(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws,

@@ -2086,6 +2086,25 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
   return cudaGetLastError();
 }
 
+// Asked once per device.  The shared memory of a block has to be allowed before.
+bool clusters_run(uint32_t blocks) {
+  static std::atomic<int> known[64][2];  // 1: they do, 2: they don't
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || plan_attributes() != cudaSuccess) return false;
+  std::atomic<int>& answer = known[dev][blocks == 16];
+  if (answer.load(std::memory_order_acquire) == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = blocks;
+    cfg.blockDim = kPlanThreads;
+    cfg.dynamicSmemBytes = kClusterSmem;
+    int n = 0;
+    const cudaError_t e = blocks == 16 ? cudaOccupancyMaxActiveClusters(&n, k_client<16, true>, &cfg) : cudaOccupancyMaxActiveClusters(&n, k_client<8, true>, &cfg);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // it is no launch's
+    answer.store(e == cudaSuccess && n > 0 ? 1 : 2, std::memory_order_release);
+  }
+  return answer.load(std::memory_order_acquire) == 1;
+}
+
 cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, const EncFront& enc, cudaStream_t st) {
   unsigned char* w = static_cast<unsigned char*>(ws);
   const cudaError_t e = plan_attributes();
