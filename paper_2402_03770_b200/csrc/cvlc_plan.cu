@@ -1825,10 +1825,10 @@ __device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, EncHeade
   }
 }
 
-// FIRST: the call's only kernel before packing (one client): it clears the headers
-template <int CL, bool FIRST>
+// first: the call's first kernel (one client): it clears the headers
+template <int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kPlanThreads, 1)
-k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_constant__ Shape shape, uint32_t rows, unsigned char* ws,
+k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_constant__ Shape shape, uint32_t rows, int first, unsigned char* ws,
          const __grid_constant__ EncFront enc) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1846,7 +1846,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
   const ClientDesc& cd = batch.c[c];
   if (q == 0) {
     if (tid == 0) reinterpret_cast<ClientDesc*>(ws + plan_off_desc(n))[c] = cd;
-    if (FIRST) {
+    if (first) {
       if (tid < 64) reinterpret_cast<uint32_t*>(ws)[tid] = 0;
       else if (tid < 128) reinterpret_cast<uint32_t*>(enc.ws)[tid - 64] = 0;
     }
@@ -2021,12 +2021,9 @@ static cudaError_t plan_attributes() {
   return once_per_device(once, [] {
     cudaError_t e = allow_shared(k_hist, kHistSub * CVLC_HIST_BINS * 4);
     if (e == cudaSuccess) e = allow_shared(k_plan_fit, kFitSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<8, false>, kClusterSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<8, true>, kClusterSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<16, false>, kClusterSmem);
-    if (e == cudaSuccess) e = allow_shared(k_client<16, true>, kClusterSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_client<16, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_client<16, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = allow_shared(k_client<8>, kClusterSmem);
+    if (e == cudaSuccess) e = allow_shared(k_client<16>, kClusterSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_client<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e != cudaSuccess ? e : allow_shared(k_plan_tune, kTuneSmem);
   });
 }
@@ -2098,7 +2095,7 @@ bool clusters_run(uint32_t blocks) {
     cfg.blockDim = kPlanThreads;
     cfg.dynamicSmemBytes = kClusterSmem;
     int n = 0;
-    const cudaError_t e = blocks == 16 ? cudaOccupancyMaxActiveClusters(&n, k_client<16, true>, &cfg) : cudaOccupancyMaxActiveClusters(&n, k_client<8, true>, &cfg);
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, blocks == 16 ? k_client<16> : k_client<8>, &cfg);
     if (e != cudaSuccess) (void)cudaGetLastError();  // it is no launch's
     answer.store(e == cudaSuccess && n > 0 ? 1 : 2, std::memory_order_release);
   }
@@ -2116,8 +2113,7 @@ cudaError_t launch_clients(const ClientDesc* clients, uint32_t n, const Shape& s
   const uint32_t rows = (uint32_t)make_partition(shape.d, n).rows;
   if (n > 1) launch_zero(clients, n, w, 256, enc.ws, 256, st);
   const uint32_t blocks = cluster_blocks(rows, n);
-  auto kernel = blocks == 16 ? (n > 1 ? k_client<16, false> : k_client<16, true>) : (n > 1 ? k_client<8, false> : k_client<8, true>);
-  launch_kernel(kKClient, kernel, blocks * n, kPlanThreads, kClusterSmem, st, n > 1, batch, shape, rows, w, enc);
+  launch_kernel(kKClient, blocks == 16 ? k_client<16> : k_client<8>, blocks * n, kPlanThreads, kClusterSmem, st, n > 1, batch, shape, rows, n > 1 ? 0 : 1, w, enc);
   return cudaGetLastError();
 }
 
