@@ -1550,7 +1550,12 @@ struct ClusterShared {
 constexpr size_t kFitSmem = kSurvivalBytes + sizeof(FitScratch);
 constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) : kFitSmem;  // one after the other
 constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 16;
-static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
+// Candidates of a bin that one block ranks; a bin of more is cut.  The fullest bin of a spread-out update has about an eighth of the candidates, 0.131 of a
+// normal distribution.  With 8192, as in the other ranking kernels, it was cut from 62,400 records on: one client of 655,000 coordinates at 2.4 bits
+// 49.4 us, 47.0 as kernels of their own, 39.1 with a block for such a bin; seven of them 54.0, 59.1 and 43.3.
+constexpr uint32_t kClusterItems = 9216;
+typedef RankSharedOf<kClusterItems> ClusterRank;
+static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(ClusterRank) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
               kClusterSmem <= 216 * 1024, "shared memory");
 
 // One more in counters of a table for each of the lanes' values that is on: what was in them before.  One addition where all of the warp's go to
@@ -1669,9 +1674,9 @@ __device__ __noinline__ bool cut_bins(uint32_t* table, const uint32_t* N, Cut* c
     for (int b0 = (int)t.top; b0 >= (int)t.bin; b0 -= 32) {
       const int b = b0 - lane;
       const uint32_t m = b >= (int)t.bin ? N[b] - N[b + 1] : 0u;
-      const unsigned large = __ballot_sync(kFull, m > kRankItems);
+      const unsigned large = __ballot_sync(kFull, m > kClusterItems);
       const uint32_t at = n + __popc(large & ((1u << lane) - 1u));
-      if (m > kRankItems && at < kCutRanges) {
+      if (m > kClusterItems && at < kCutRanges) {
         cuts[0].prefix[at] = 4095u - (uint32_t)b;
         cuts[0].start[at] = N[b + 1];
         cuts[0].size[at] = m;
@@ -1784,7 +1789,7 @@ __device__ __noinline__ bool cut_bins(uint32_t* table, const uint32_t* N, Cut* c
 }
 
 // The parts whose candidates begin with the ranks [first, end), as many of a range as a block holds at a time; by the whole block
-__device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, EncHeader* hdr, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop,
+__device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, unsigned char* ws, const EncLayout& L, uint32_t c, uint32_t keytop,
                                         u64* buf_a, u64* buf_b, uint32_t first, uint32_t end) {
   __shared__ uint32_t s_start[kCutParts + 1];
   const uint32_t tid = threadIdx.x;
@@ -1816,8 +1821,7 @@ __device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, EncHeade
         if (m && cut == 2) {
           rank_cell<kPlanThreads>(s, src + at, m, buf_a + at);
         } else if (m) {
-          rank_and_leave<kPlanThreads>(s, src + at, m, inv, inv_end - inv - 1, buf_a + at, keytop, hdr, reinterpret_cast<ulonglong2*>(ws + L.off_list[1]),
-                                       reinterpret_cast<const u64*>(ws + L.off_buf_a));
+          rank_and_leave<kPlanThreads>(reinterpret_cast<ClusterRank&>(s), src + at, m, inv, inv_end - inv - 1, keytop, ws, L, c, at);
         }
         i = behind;
       }
@@ -1928,7 +1932,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
                                        q == 0 ? reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS : nullptr);
   if (q == 0 && tid == 0) write_client(c, n, cd.plan, t, nonfinite, shape, ws, enc);
   const EncLayout& L = enc.L;
-  const bool go = !nonfinite && t.n <= L.capacity, crowded = t.fullest > kRankItems;
+  const bool go = !nonfinite && t.n <= L.capacity, crowded = t.fullest > kClusterItems;
   const uint32_t limit = shape.R * cd.cap0;  // ranks from here on are not sent (see by_clusters)
   unsigned long long* by_bin = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_b) + (size_t)c * L.capacity;
   // ---- the candidates to their bins
@@ -2000,15 +2004,12 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
     }
     const uint32_t m = N[lo + 1] - at;
     const u64 inv = (u64)((int)t.top - hi) << 19, end = (u64)((int)t.top - lo) << 19;
-    if (m && m <= kRankItems) {  // else it is one bin, which has been cut
-      rank_and_leave<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), out + at, keytop,
-                                   reinterpret_cast<EncHeader*>(enc.ws), reinterpret_cast<ulonglong2*>(enc.ws + L.off_list[1]),
-                                   reinterpret_cast<const u64*>(enc.ws + L.off_buf_a));
-    }
+    if (m && m <= kClusterItems)  // else it is one bin, which has been cut
+      rank_and_leave<kPlanThreads>(*reinterpret_cast<ClusterRank*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), keytop, enc.ws, L, c, at);
     hi = lo;
   }
   if (crowded)
-    rank_parts(*reinterpret_cast<RankShared*>(rest), s_cut, reinterpret_cast<EncHeader*>(enc.ws), enc.ws, L, c, keytop, out, by_bin, q * share,
+    rank_parts(*reinterpret_cast<RankShared*>(rest), s_cut, enc.ws, L, c, keytop, out, by_bin, q * share,
                min((q + 1) * share, ranked));
 }
 

@@ -650,11 +650,11 @@ __device__ __forceinline__ BigBucket big_bucket(const RankArgs& a, int round, ui
 __device__ __forceinline__ const u64* big_source(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_a : a.buf_b) + pos; }
 __device__ __forceinline__ u64* big_target(const RankArgs& a, int round, u64 pos) { return (round & 1 ? a.buf_b : a.buf_a) + pos; }
 
-// A cell of up to kWarpCell items, whose values are `mine`, by one warp of the block
+// A cell of up to kWarpCell items, whose values are `mine`, by one warp of the block; cell: kWarpCells counters of its own
 template <int THREADS>
-__device__ __forceinline__ void rank_values_by_warp(RankShared& s, u64* mine, uint32_t m, u64* at) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (!rank_equal_by_warp<THREADS>(s.cell + warp * kWarpCells, mine, m, at)) {
+__device__ __forceinline__ void rank_values_by_warp(uint32_t* cell, u64* mine, uint32_t m, u64* at) {
+  const int lane = threadIdx.x & 31;
+  if (!rank_equal_by_warp<THREADS>(cell, mine, m, at)) {
     bitonic_sort(mine, m, lane, 32, [] { __syncwarp(); });
     for (uint32_t i = lane; i < m; i += 32) at[i] = to_item(mine[i]);
     __syncwarp();
@@ -666,14 +666,15 @@ __device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32
   u64* mine = s.items + (threadIdx.x >> 5) * kWarpCell;
   for (uint32_t i = threadIdx.x & 31; i < m; i += 32) mine[i] = to_value(at[i]);
   __syncwarp();
-  rank_values_by_warp<THREADS>(s, mine, m, at);
+  rank_values_by_warp<THREADS>(s.cell + (threadIdx.x >> 5) * kWarpCells, mine, m, at);
 }
 
-// Ranks m <= kRankItems items in [base, base + span] of inv, but for the cells of more than kCompareAll items, whose places and items go to
+// Ranks m items, as many as Shared holds at most, in [base, base + span] of inv, but for the cells of more than kCompareAll, whose places and items go to
 // `cells`; returns how many.  By the whole block.
-template <int THREADS>
-__device__ __forceinline__ uint32_t rank_but_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
-                                                   uint32_t (&cells)[kRankItems / kCompareAll]) {
+template <int THREADS, class Shared, uint32_t CELLS>
+__device__ __forceinline__ uint32_t rank_but_cells(Shared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+                                                   uint32_t (&cells)[CELLS]) {
+  static_assert(CELLS * kCompareAll + CELLS > sizeof(s.items) / 8 - 2, "room for all");
   __shared__ uint32_t s_n;
   if (threadIdx.x == 0) s_n = 0;
   rank_buckets<THREADS>(s, src, m, base, span, out, keytop,
@@ -692,17 +693,28 @@ __device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint
   }
   __syncthreads();
 }
-// ... by its warps; those that a warp cannot rank by k_rank_rest, by all its blocks
-template <int THREADS>
-__device__ __noinline__ void rank_and_leave(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
-                                            EncHeader* hdr, ulonglong2* list, const u64* buf_a) {
-  __shared__ uint32_t s_cell[kRankItems / kCompareAll];
+// ... by its warps; those that a warp cannot rank by k_rank_rest, by all its blocks.  The items are client c's from rank `start` on; they come from either
+// buffer and go to the first.
+template <int THREADS, class Shared>
+__device__ __noinline__ void rank_and_leave(Shared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, uint32_t keytop, unsigned char* ws,
+                                            const EncLayout& L, uint32_t c, uint32_t start) {
+  __shared__ uint32_t s_cell[sizeof(s.items) / 8 / kCompareAll];
+  EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
+  u64* buf_a = reinterpret_cast<u64*>(ws + L.off_buf_a);
+  u64* out = buf_a + (size_t)c * L.capacity + start;
+  ulonglong2* list = reinterpret_cast<ulonglong2*>(ws + L.off_list[1]);
   const uint32_t n = rank_but_cells<THREADS>(s, src, m, base, span, out, keytop, s_cell);
   for (uint32_t g = threadIdx.x >> 5; g < n; g += THREADS / 32) {
-    u64* at = out + (s_cell[g] & 0xFFFFu);
-    const uint32_t items = s_cell[g] >> 16;
-    if (items <= kWarpCell) rank_values_by_warp<THREADS>(s, s.items + (s_cell[g] & 0xFFFFu), items, at);
-    else if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(at - buf_a), items);
+    const uint32_t first = s_cell[g] & 0xFFFFu, items = s_cell[g] >> 16;
+    if (items <= kWarpCell) {
+      rank_values_by_warp<THREADS>(s.cell + (threadIdx.x >> 5) * kWarpCells, s.items + first, items, out + first);
+    } else if (items <= kRankItems) {
+      if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(out + first - buf_a), items);
+    } else {  // more than a block of that kernel holds: a large bucket, from the second buffer
+      u64* from = reinterpret_cast<u64*>(ws + L.off_buf_b) + (size_t)c * L.capacity + start + first;
+      for (uint32_t i = threadIdx.x & 31; i < items; i += 32) from[i] = out[first + i];
+      if ((threadIdx.x & 31) == 0) list_bucket(hdr, ws, L, c, keytop, base, (u64)base + span + 1, start + first, items);
+    }
   }
   __syncthreads();
 }

@@ -96,9 +96,9 @@ def in_one_bin(m, values, d, rng):
     return x
 
 
-# all different: one cut, where a bin has more than 8192; 512 neighbouring keys: parts of one cut that are cut again; two and one: by coordinates
+# all different: one cut, where a bin has more than 9216 (a cell of it more than 8192: split behind the clusters); 512 neighbouring keys: parts of one cut that are cut again; two and one: by coordinates
 @pytest.mark.parametrize("values", [1 << 19, 512, 2, 1])
-@pytest.mark.parametrize("m", [8_192, 8_193, 12_000, 16_384, 16_385, 33_000])
+@pytest.mark.parametrize("m", [8_192, 8_193, 9_216, 9_217, 12_000, 16_384, 16_385, 33_000])
 @pytest.mark.parametrize("d,n", [(200_003, 2), (600_001, 1)])
 def test_bins_that_a_block_does_not_hold(values, m, d, n):
     """what is sent ends inside the bin and behind it"""
