@@ -1550,6 +1550,9 @@ struct ClusterShared {
 constexpr size_t kFitSmem = kSurvivalBytes + sizeof(FitScratch);
 constexpr size_t kTuneSmem = sizeof(PlanSolver) > kFitSmem ? sizeof(PlanSolver) : kFitSmem;  // one after the other
 constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 16;
+// Units of a share beyond those that a block keeps, for each of its threads: a share is a seventh or a fifteenth of what eight or sixteen blocks keep
+constexpr uint32_t kClusterOver = 3;
+static_assert(kClusterOver * kPlanThreads >= kClusterUnits / 7 + kRowUnits, "a share");
 // Candidates of a bin that one block ranks; a bin of more is cut.  The fullest bin of a spread-out update has about an eighth of the candidates, 0.131 of a
 // normal distribution.  With 8192, as in the other ranking kernels, it was cut from 62,400 records on: one client of 655,000 coordinates at 2.4 bits
 // 49.4 us, 47.0 as kernels of their own, 39.1 with a block for such a bin; seven of them 54.0, 59.1 and 43.3.
@@ -1957,9 +1960,15 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
       for (uint32_t i = q * kPlanThreads + tid; i < kCuts * kCutTable; i += (CL - 1) * kPlanThreads) cut_totals(enc.ws, L, c, i / kCutTable)[i % kCutTable] = 0;
       if (q == 0 && tid == 0) *cut_turns(enc.ws, L, c) = 0;
     } else {
-      for (uint32_t i = kept + tid; i < units; i += kPlanThreads) put4(__ldg(xv + u0 + i), 4 * (u0 + i));
+      float4 over[kClusterOver];  // on their way while the others go
+#pragma unroll
+      for (uint32_t u = 0; u < kClusterOver; ++u)
+        if (kept + u * kPlanThreads + tid < units) over[u] = __ldg(xv + u0 + kept + u * kPlanThreads + tid);
 #pragma unroll 4
       for (uint32_t i = tid; i < kept; i += kPlanThreads) put4(data[i], 4 * (u0 + i));
+#pragma unroll
+      for (uint32_t u = 0; u < kClusterOver; ++u)
+        if (kept + u * kPlanThreads + tid < units) put4(over[u], 4 * (u0 + kept + u * kPlanThreads + tid));
     }
     if (has_tail) put(tail, 4 * nvec + tid);
   }
