@@ -41,6 +41,8 @@ FALLBACK_HBM_GBS = 6650.0
 NCU_TRAFFIC_BYTES_PER_CLIENT = {
     "k_hist": (1433.86e6 + 45.05e6) / 32,          # the update once, plus the rows' maxima
     "k_select": (402.01e6 + 168.91e6) / 32,        # the rows that hold candidates (a quarter of the update), plus the candidates
+    "k_rank_split": (203.82e6 + 157.72e6) / 32,    # three blocks per SM, as batches of 32 clients and more have
+    "k_rank": (203.13e6 + 157.69e6) / 32,
     "k_pack": (177.99e6 + 53.81e6) / 32,
 }
 NOMINAL_HBM_GBS = 8000.0

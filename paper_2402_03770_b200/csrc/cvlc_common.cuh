@@ -477,16 +477,17 @@ cudaError_t launch_plan_front(const ClientDesc* clients, uint32_t n, const Shape
 cudaError_t launch_plan_back(uint32_t n, const Shape& shape, void* ws, TunePlace place, cudaStream_t st, bool overlap);
 cudaError_t launch_plan(const ClientDesc* clients, uint32_t n, const Shape& shape, void* ws, cudaStream_t st);
 // Few small clients: planning, selection and ranking by a cluster of blocks per client (see k_client).  All clusters run at a time, every block
-// keeps its share of the coordinates in shared memory, and no more candidates than a block ranks in two tiles.  From 32,768 candidates on, the
-// kernels of their own and this, us: 1 / 7 / 12 clients of 320,000 coordinates at 4 / 4 / 2.8 bits 51 and 44 / 61 and 50 / 67 and 59, 12 of 240,000 at
-// 4 bits 66 and 57, 3 of 600,000 at 3 bits 63 and 52, 1 / 7 of 655,000 at 4 / 3 bits 58 and 55 / 73 and 66.
-constexpr uint32_t kClusterUnits = 10240;  // float4 units that a block keeps
+// keeps most of its share of the coordinates in shared memory, and there is room for all bins that can be too large for a block (see kCutRanges).  The
+// kernels of their own and this, close to the limit of 65,536 records, us: 1 / 7 clients of 320,000 coordinates at 4 bits (52,600 records) 44 and 31 / 54
+// and 35, 12 of 320,000 at 2.8 (36,700) 58 and 41, 12 of 240,000 at 4 (41,400) 58 and 43, 3 of 600,000 at 2.7 (64,300) 51 and 40, 1 / 7 of 655,000 at 2.4
+// (62,400) 48 and 39 / 59 and 43.
+constexpr uint32_t kClusterUnits = 10240;  // float4 units that a block keeps at most
 constexpr uint64_t kClusterCandidates = 65536;
 // Blocks of a client's cluster; 0: too many clients or coordinates.  Clusters that run at a time, a block on an SM
-// (cudaOccupancyMaxActiveClusters): 15 of eight blocks, 7 of sixteen.  Sixteen exchange more counts, eight read longer; whole calls with the
-// aggregation, eight and sixteen, us: one client of 100,000 coordinates 39.0 and 40.6, of 200,000 41.0 and 41.0, of 320,000 44.1 and 42.7, seven
-// of 320,000 47.2 and 45.1.  Beyond that the kernels of their own and sixteen: one of 340,000 47.8 and 42.9, three of 450,000 54.3 and 47.2, seven
-// of 650,000 57.5 and 49.7.
+// (cudaOccupancyMaxActiveClusters): 15 of eight blocks, 7 of sixteen.  Sixteen exchange more counts, eight read and rank longer; calls at 1 bit a
+// coordinate, eight and sixteen, us: one client of 100,000 coordinates 26.8 each, of 200,000 27.3 and 27.6, of 240,000 28.9 and 28.4, of 320,000 30.9 and
+// 28.9, seven of 200,000 29.0 and 31.0, of 240,000 31.0 each, of 320,000 33.1 and 31.0; at 4 bits one of 320,000 41.2 and 30.9.  Beyond that the kernels of
+// their own and sixteen: one of 340,000 43.5 and 28.9, three of 450,000 47.7 and 34.4, seven of 650,000 52.7 and 41.3.
 inline uint32_t cluster_blocks(uint64_t rows, uint32_t n) {
   const uint64_t of_block = kClusterUnits / kRowUnits;
   if (n <= 7 && rows > 6 * of_block && rows <= 16 * of_block) return 16;
@@ -665,7 +666,7 @@ __device__ __forceinline__ void add_client(EncHeader* hdr, const ClientRank& r, 
 // of 52 M, with what is left over, 73 -> 48.
 __device__ __forceinline__ uint32_t rank_window(uint32_t most, uint32_t n, uint32_t blocks, uint32_t largest) {
   const uint32_t least = (most + largest - 1) / largest;  // tiles of the largest client
-  const uint32_t tiles = (least * n + blocks - 1) / blocks * blocks / n;  // below 2^29: at most 2^19 tiles of at most 512 clients
+  const uint32_t tiles = (least * n + blocks - 1) / blocks * blocks / n;  // below 2^29: at most 699,051 tiles (of 3072) of at most 512 clients
   const uint32_t window = tiles ? (most + tiles - 1) / tiles : 0u;
   return window > 1024 ? window : 1024;
 }

@@ -1538,9 +1538,9 @@ k_plan_tune(const Batch batch, const __grid_constant__ Shape shape, unsigned cha
 // bits, where the ranking is what the cluster ends with, 37.1 -> 37.4.)  A share may be more than a block keeps; the rest is read again.  Bins of more
 // than a block holds are cut again (see cut_bins); cells of more than 256 equal or nearly equal keys are left to k_rank_rest, whose blocks work
 // them off side by side.
-// Bound by latencies: of 17 us for one client of 100,000 coordinates and 22 for ten of 300,000 the tuning takes the last 11 to 13.  As kernels
+// Bound by latencies: of 17 us for one client of 100,000 coordinates and 20 for ten of 300,000 the tuning takes the last 10.  As kernels
 // of their own (zeros, histogram, selection, partition, ranking, what that leaves over, and the tuning on another stream between two
-// events) the steps took 30 and 39; whole calls 36.9 -> 26.7 us, 56.7 -> 45.5 with the aggregation.
+// events) the steps took 30 and 39; whole calls 36.9 -> 26.5 us, 56.7 -> 45.2 with the aggregation.
 
 struct ClusterShared {
   uint32_t own[CVLC_HIST_BINS + 4];  // the block's counts; then the client's survival counts

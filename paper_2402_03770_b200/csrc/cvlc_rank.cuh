@@ -866,7 +866,7 @@ __device__ __noinline__ void big_sample(RankShared& s, EncHeader* hdr, const Ran
 // Buckets of few pieces: all steps by one block, so that none of them waits for others
 template <int THREADS>
 __device__ __noinline__ void big_own(RankShared& s, EncHeader* hdr, const RankArgs& a) {
-  const uint32_t n = hdr->own_n;  // written by the selection alone
+  const uint32_t n = hdr->own_n;  // written by the kernels in front alone
   while (true) {
     const uint32_t i = block_takes(&hdr->own_next);
     if (i >= n) return;
@@ -1016,7 +1016,7 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
   __shared__ uint32_t s_entry;
   const int tid = threadIdx.x, lane = tid & 31;
   __syncthreads();  // the arguments are there
-  const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the selection alone
+  const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the kernels in front alone: the selection, the clusters
   if (big) {
     big_sample<THREADS>(s, hdr, a, 0);
     big_own<THREADS>(s, hdr, a);
