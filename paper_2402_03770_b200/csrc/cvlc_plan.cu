@@ -1553,12 +1553,7 @@ constexpr size_t kClusterSmem = sizeof(ClusterShared) + (size_t)kClusterUnits * 
 // Units of a share beyond those that a block keeps, for each of its threads: a share is a seventh or a fifteenth of what eight or sixteen blocks keep
 constexpr uint32_t kClusterOver = 3;
 static_assert(kClusterOver * kPlanThreads >= kClusterUnits / 7 + kRowUnits, "a share");
-// Candidates of a bin that one block ranks; a bin of more is cut.  The fullest bin of a spread-out update has about an eighth of the candidates, 0.131 of a
-// normal distribution.  With 8192, as in the other ranking kernels, it was cut from 62,400 records on: one client of 655,000 coordinates at 2.4 bits
-// 49.4 us, 47.0 as kernels of their own, 39.1 with a block for such a bin; seven of them 54.0, 59.1 and 43.3.
-constexpr uint32_t kClusterItems = 9216;
-typedef RankSharedOf<kClusterItems> ClusterRank;
-static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(ClusterRank) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
+static_assert(kTuneSmem <= (size_t)kClusterUnits * 16 && sizeof(RankShared) <= (size_t)kClusterUnits * 16 && sizeof(ClusterShared) % 16 == 0 &&
               kClusterSmem <= 216 * 1024, "shared memory");
 
 // One more in counters of a table for each of the lanes' values that is on: what was in them before.  One addition where all of the warp's go to
@@ -1677,9 +1672,9 @@ __device__ __noinline__ bool cut_bins(uint32_t* table, const uint32_t* N, Cut* c
     for (int b0 = (int)t.top; b0 >= (int)t.bin; b0 -= 32) {
       const int b = b0 - lane;
       const uint32_t m = b >= (int)t.bin ? N[b] - N[b + 1] : 0u;
-      const unsigned large = __ballot_sync(kFull, m > kClusterItems);
+      const unsigned large = __ballot_sync(kFull, m > kRankHold);
       const uint32_t at = n + __popc(large & ((1u << lane) - 1u));
-      if (m > kClusterItems && at < kCutRanges) {
+      if (m > kRankHold && at < kCutRanges) {
         cuts[0].prefix[at] = 4095u - (uint32_t)b;
         cuts[0].start[at] = N[b + 1];
         cuts[0].size[at] = m;
@@ -1824,7 +1819,7 @@ __device__ __noinline__ void rank_parts(RankShared& s, const Cut* cuts, unsigned
         if (m && cut == 2) {
           rank_cell<kPlanThreads>(s, src + at, m, buf_a + at);
         } else if (m) {
-          rank_and_leave<kPlanThreads>(reinterpret_cast<ClusterRank&>(s), src + at, m, inv, inv_end - inv - 1, keytop, ws, L, c, at);
+          rank_and_leave<kPlanThreads>(s, src + at, m, inv, inv_end - inv - 1, keytop, ws, L, c, at);
         }
         i = behind;
       }
@@ -1935,7 +1930,7 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
                                        q == 0 ? reinterpret_cast<uint32_t*>(ws + plan_off_bin_start(n)) + (size_t)c * CVLC_HIST_BINS : nullptr);
   if (q == 0 && tid == 0) write_client(c, n, cd.plan, t, nonfinite, shape, ws, enc);
   const EncLayout& L = enc.L;
-  const bool go = !nonfinite && t.n <= L.capacity, crowded = t.fullest > kClusterItems;
+  const bool go = !nonfinite && t.n <= L.capacity, crowded = t.fullest > kRankHold;
   const uint32_t limit = shape.R * cd.cap0;  // ranks from here on are not sent (see by_clusters)
   unsigned long long* by_bin = reinterpret_cast<unsigned long long*>(enc.ws + L.off_buf_b) + (size_t)c * L.capacity;
   // ---- the candidates to their bins
@@ -2013,8 +2008,8 @@ k_client(const __grid_constant__ BatchDesc<kMediumBatch> batch, const __grid_con
     }
     const uint32_t m = N[lo + 1] - at;
     const u64 inv = (u64)((int)t.top - hi) << 19, end = (u64)((int)t.top - lo) << 19;
-    if (m && m <= kClusterItems)  // else it is one bin, which has been cut
-      rank_and_leave<kPlanThreads>(*reinterpret_cast<ClusterRank*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), keytop, enc.ws, L, c, at);
+    if (m && m <= kRankHold)  // else it is one bin, which has been cut
+      rank_and_leave<kPlanThreads>(*reinterpret_cast<RankShared*>(rest), by_bin + at, m, (uint32_t)inv, (uint32_t)(end - inv - 1), keytop, enc.ws, L, c, at);
     hi = lo;
   }
   if (crowded)

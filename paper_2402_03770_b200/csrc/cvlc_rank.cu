@@ -185,7 +185,7 @@ k_rank_rest(const Batch batch, unsigned char* ws, const __grid_constant__ EncLay
 static cudaError_t rank_attributes() {
   static OncePerDevice once;
   return once_per_device(once, [] {
-    cudaError_t e = allow_shared(k_rank<false>, sizeof(RankShared));
+    cudaError_t e = allow_shared(k_rank<false>, sizeof(RankSharedOf<kRankItems>));
     if (e == cudaSuccess) e = allow_shared(k_rank<true>, sizeof(RankSharedOf<kRankTile3>));
     return e != cudaSuccess ? e : allow_shared(k_rank_rest, sizeof(RankShared));
   });
@@ -208,7 +208,7 @@ cudaError_t launch_rank(Batch batch, const EncLayout& L, const unsigned char* pl
                 kRankThreads, kRankSubs * 4, st, true, batch, ws, L);
   const uint32_t* bin_start = reinterpret_cast<const uint32_t*>(plan_ws + plan_off_bin_start(L.n));
   launch_kernel(kKRank, three ? k_rank<true> : k_rank<false>, blocks((L.capacity + 1023) / 1024 * L.n, (three ? 3 : 2) * sms), kRankThreads,
-                three ? sizeof(RankSharedOf<kRankTile3>) : sizeof(RankShared), st, true, batch, ws, L, bin_start, (three ? 3 : 2) * sms);
+                three ? sizeof(RankSharedOf<kRankTile3>) : sizeof(RankSharedOf<kRankItems>), st, true, batch, ws, L, bin_start, (three ? 3 : 2) * sms);
   return launch_rank_rest(batch, L, plan_ws, ws, sms, three, st);
 }
 

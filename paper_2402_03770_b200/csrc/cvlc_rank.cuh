@@ -27,7 +27,12 @@ struct RankSharedOf {
   uint32_t zero[4];           // cell[-1] = 0: where the first cell starts
   uint32_t cell[kCells];      // counts, then starts, then (after placing) ends of the cells
 };
-typedef RankSharedOf<kRankItems> RankShared;
+// What a block of the clusters ranks at most, and one of k_rank_rest of equal keys that they leave: a bin of kRankItems and some more.  The fullest bin
+// of a spread-out update has about an eighth of the candidates, 0.131 of a normal distribution.  With 8192 in clusters, too, it was cut from 62,400
+// records on: one client of 655,000 coordinates at 2.4 bits 49.4 us, 47.0 as kernels of their own, 39.1 with a block for such a bin; seven of them
+// 54.0, 59.1 and 43.3.
+constexpr uint32_t kRankHold = 9216;
+typedef RankSharedOf<kRankHold> RankShared;
 
 // A candidate as a value to rank: the key's complement in the high word, index << 1 | sign in the low word.
 __device__ __forceinline__ u64 to_value(u64 item) {
@@ -185,7 +190,7 @@ __device__ __forceinline__ void rank_other(Others& o, uint32_t i, uint32_t key, 
   out[rank] = to_item(v);
 }
 
-// Ranks items[0 .. n), n <= kRankItems, and writes them out; by the whole block.  False, and nothing done, if too many keys differ or
+// Ranks items[0 .. n), n <= kRankHold, and writes them out; by the whole block.  False, and nothing done, if too many keys differ or
 // a range has too many items.
 template <int THREADS, uint32_t BITS>
 __device__ __noinline__ bool rank_equal(RankShared& s, u64* items, uint32_t n, u64* __restrict__ out) {
@@ -348,7 +353,7 @@ __device__ __forceinline__ bool rank_equal_by_warp(uint32_t* cell, u64* items, u
   return true;
 }
 
-// Ranks the n <= kRankItems items of a cell of many keys and writes them out (in their place, too); by the whole block.  They are
+// Ranks the n <= kRankHold items of a cell of many keys and writes them out (in their place, too); by the whole block.  They are
 // spread over equal ranges of (key, index) between the least and the largest of each.  False, and nothing done, if a range has too many.
 template <int THREADS>
 __device__ __noinline__ bool rank_spread(RankShared& s, const u64* at, uint32_t n, u64* out) {
@@ -409,7 +414,7 @@ __device__ __noinline__ bool rank_spread(RankShared& s, const u64* at, uint32_t 
   return true;
 }
 
-// Ranks n <= kRankItems items, most of them of one key or nearly equal, and writes them out (in their place, too); by the whole block
+// Ranks n <= kRankHold items, most of them of one key or nearly equal, and writes them out (in their place, too); by the whole block
 template <int THREADS>
 __device__ __noinline__ void rank_cell(RankShared& s, const u64* at, uint32_t n, u64* out) {
   for (int attempt = 0; attempt < 3; ++attempt) {
@@ -669,12 +674,11 @@ __device__ __forceinline__ void rank_cell_by_warp(RankShared& s, u64* at, uint32
   rank_values_by_warp<THREADS>(s.cell + (threadIdx.x >> 5) * kWarpCells, mine, m, at);
 }
 
-// Ranks m items, as many as Shared holds at most, in [base, base + span] of inv, but for the cells of more than kCompareAll, whose places and items go to
-// `cells`; returns how many.  By the whole block.
-template <int THREADS, class Shared, uint32_t CELLS>
-__device__ __forceinline__ uint32_t rank_but_cells(Shared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
-                                                   uint32_t (&cells)[CELLS]) {
-  static_assert(CELLS * kCompareAll + CELLS > sizeof(s.items) / 8 - 2, "room for all");
+// Ranks m <= kRankHold items in [base, base + span] of inv, but for the cells of more than kCompareAll, whose places and items go to `cells`; returns
+// how many.  By the whole block.
+template <int THREADS>
+__device__ __forceinline__ uint32_t rank_but_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop,
+                                                   uint32_t (&cells)[kRankHold / kCompareAll]) {
   __shared__ uint32_t s_n;
   if (threadIdx.x == 0) s_n = 0;
   rank_buckets<THREADS>(s, src, m, base, span, out, keytop,
@@ -685,7 +689,7 @@ __device__ __forceinline__ uint32_t rank_but_cells(Shared& s, const u64* src, ui
 // coordinates in 255 steps 163.5 -> 167.6 us, on a grid of 24 steps per deviation 163.8 -> 169.7, one of 5 M 122.0 -> 126.5.)
 template <int THREADS>
 __device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, u64* out, uint32_t keytop) {
-  __shared__ uint32_t s_cell[kRankItems / kCompareAll];
+  __shared__ uint32_t s_cell[kRankHold / kCompareAll];
   const uint32_t n = rank_but_cells<THREADS>(s, src, m, base, span, out, keytop, s_cell);
   for (uint32_t g = 0; g < n; ++g) {
     u64* at = out + (s_cell[g] & 0xFFFFu);
@@ -695,10 +699,10 @@ __device__ __noinline__ void rank_with_cells(RankShared& s, const u64* src, uint
 }
 // ... by its warps; those that a warp cannot rank by k_rank_rest, by all its blocks.  The items are client c's from rank `start` on; they come from either
 // buffer and go to the first.
-template <int THREADS, class Shared>
-__device__ __noinline__ void rank_and_leave(Shared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, uint32_t keytop, unsigned char* ws,
+template <int THREADS>
+__device__ __noinline__ void rank_and_leave(RankShared& s, const u64* src, uint32_t m, uint32_t base, uint32_t span, uint32_t keytop, unsigned char* ws,
                                             const EncLayout& L, uint32_t c, uint32_t start) {
-  __shared__ uint32_t s_cell[sizeof(s.items) / 8 / kCompareAll];
+  __shared__ uint32_t s_cell[kRankHold / kCompareAll];
   EncHeader* hdr = reinterpret_cast<EncHeader*>(ws);
   u64* buf_a = reinterpret_cast<u64*>(ws + L.off_buf_a);
   u64* out = buf_a + (size_t)c * L.capacity + start;
@@ -706,15 +710,8 @@ __device__ __noinline__ void rank_and_leave(Shared& s, const u64* src, uint32_t 
   const uint32_t n = rank_but_cells<THREADS>(s, src, m, base, span, out, keytop, s_cell);
   for (uint32_t g = threadIdx.x >> 5; g < n; g += THREADS / 32) {
     const uint32_t first = s_cell[g] & 0xFFFFu, items = s_cell[g] >> 16;
-    if (items <= kWarpCell) {
-      rank_values_by_warp<THREADS>(s.cell + (threadIdx.x >> 5) * kWarpCells, s.items + first, items, out + first);
-    } else if (items <= kRankItems) {
-      if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(out + first - buf_a), items);
-    } else {  // more than a block of that kernel holds: a large bucket, from the second buffer
-      u64* from = reinterpret_cast<u64*>(ws + L.off_buf_b) + (size_t)c * L.capacity + start + first;
-      for (uint32_t i = threadIdx.x & 31; i < items; i += 32) from[i] = out[first + i];
-      if ((threadIdx.x & 31) == 0) list_bucket(hdr, ws, L, c, keytop, base, (u64)base + span + 1, start + first, items);
-    }
+    if (items <= kWarpCell) rank_values_by_warp<THREADS>(s.cell + (threadIdx.x >> 5) * kWarpCells, s.items + first, items, out + first);
+    else if ((threadIdx.x & 31) == 0) list[atomicAdd(&hdr->list_n[1], 1u)] = make_ulonglong2((u64)(out + first - buf_a), items);
   }
   __syncthreads();
 }
@@ -866,7 +863,7 @@ __device__ __noinline__ void big_sample(RankShared& s, EncHeader* hdr, const Ran
 // Buckets of few pieces: all steps by one block, so that none of them waits for others
 template <int THREADS>
 __device__ __noinline__ void big_own(RankShared& s, EncHeader* hdr, const RankArgs& a) {
-  const uint32_t n = hdr->own_n;  // written by the kernels in front alone
+  const uint32_t n = hdr->own_n;  // written by the selection alone
   while (true) {
     const uint32_t i = block_takes(&hdr->own_next);
     if (i >= n) return;
@@ -1016,7 +1013,7 @@ __device__ __noinline__ void rank_lists(RankShared& s, EncHeader* hdr, const Ran
   __shared__ uint32_t s_entry;
   const int tid = threadIdx.x, lane = tid & 31;
   __syncthreads();  // the arguments are there
-  const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the kernels in front alone: the selection, the clusters
+  const bool big = (hdr->big[0].n | hdr->own_n) != 0;  // written by the selection alone
   if (big) {
     big_sample<THREADS>(s, hdr, a, 0);
     big_own<THREADS>(s, hdr, a);

@@ -96,7 +96,7 @@ def in_one_bin(m, values, d, rng):
     return x
 
 
-# all different: one cut, where a bin has more than 9216 (a cell of it more than 8192: split behind the clusters); 512 neighbouring keys: parts of one cut that are cut again; two and one: by coordinates
+# all different: one cut, where a bin has more than 9216 (up to that many of one key are left to k_rank_rest); 512 neighbouring keys: parts of one cut that are cut again; two and one: by coordinates
 @pytest.mark.parametrize("values", [1 << 19, 512, 2, 1])
 @pytest.mark.parametrize("m", [8_192, 8_193, 9_216, 9_217, 12_000, 16_384, 16_385, 33_000])
 @pytest.mark.parametrize("d,n", [(200_003, 2), (600_001, 1)])
