@@ -1606,9 +1606,9 @@ __device__ __noinline__ void put_crowded(uint32_t* place, uint32_t thresh_bin, c
 // are cut again; after the third cut a part is what 4096 neighbouring coordinates have of one key.
 // A cut is a chain of latencies: reading, counting and moving 1 to 5 us each, two waits of the blocks for one another 1.5 each.  Left to k_rank_rest, as large
 // buckets of other batches are, such bins came behind the tuning and took 45 to 120 us there.  Whole calls, as kernels of their own / left to
-// k_rank_rest / cut, us: 36,000 candidates spread over one bin, ten clients of 300,000 coordinates 57 / 107 / 47; on eight values 74 / 125 / 65;
-// signs only, one of 600,000 107 / 120 / 78, ten of 300,000 183 / 142 / 80; 5 % of one magnitude, one of 600,000 104 / 106 / 64; 98 % zeros, one of
-// 320,000 101 / 101 / 91.  But one client of 600,000 in 16 bits (fp16, 59,500 records) 59 / 84 / 68: 15 blocks rank where 296 did.
+// k_rank_rest / cut, us: 36,000 candidates spread over one bin, ten clients of 300,000 coordinates 57 / 107 / 47; on eight values 74 / 125 / 66;
+// signs only, one of 600,000 107 / 120 / 79, ten of 300,000 181 / 143 / 81; 5 % of one magnitude, one of 600,000 104 / 106 / 65; 98 % zeros, one of
+// 320,000 101 / 101 / 91.  But one client of 600,000 in 16 bits (fp16, 59,500 records) 59 / 84 / 67: 15 blocks rank where 296 did.
 constexpr uint32_t kCutParts = 512, kCutRanges = 8, kCuts = 3, kCutTable = kCutRanges * kCutParts;
 static_assert(kCutParts == kPlanThreads && kCutParts == 16 * 32 && kCutTable <= CVLC_HIST_BINS && kCutRanges <= kPlanThreads / 32, "one part per thread");
 static_assert((kRankItems + 1) * kCutRanges > kClusterCandidates, "room for all ranges that begin with a rank that may be sent");
